@@ -20,6 +20,7 @@
 #include "pac_gemm.cuh"
 #include "pac_quant.cuh"
 #include "pac_tbody.cuh"
+#include "pac_sgemm.cuh"
 
 using namespace pac;
 
@@ -60,6 +61,7 @@ struct Scratch {
     bf16* wdT = nullptr;           // [L][2][d][r] bf16 hi/lo shadow of W_down
     float* lm_part = nullptr;      // [slices][...] partial sums of the LM path's two skinny products (dW_up, da_L)
     float* dw_part = nullptr;      // split partials of dW_down
+    float* dw_spart = nullptr;     // row-slice partials of dW_down on the plain path
     unsigned* gates = nullptr;     // [M][r] ReLU gates of all layers, one word per element (chain-in-epilogue forward)
     float* pool_part = nullptr;    // [B][s_chunks * 4][r] token sums of a_L per 32-token group (chain-in-epilogue forward)
     float* prodW = nullptr;        // [r][C] W_up W_head of the current parameters (stand-alone head kernels)
@@ -77,6 +79,11 @@ struct TBody {
     // work buffers of the backward pass
     float *da = nullptr, *dx1 = nullptr, *dn = nullptr, *dqkv = nullptr, *dpre = nullptr, *dtmp = nullptr;
     long long sMr = 0, sMf = 0, sP = 0, sM = 0;      // per-layer strides of the stacks
+};
+    TbPack pk{};
+    TbStacks st{};
+    float *packed = nullptr, *wg_part = nullptr;     // weights laid out for the ring [L][..]; row slices of the weight products
+    int wg_slices = 1;
 };
 
 // A cache that lives in host memory (Section V-B, storage cost analysis: the cache is kept on
@@ -193,6 +200,7 @@ struct pac_ctx {
     bool lm_tensor = false;
     bool lm_skinny_tensor = false; // the three products around W_up also run on the tensor cores
     int sms = 0;                   // multiprocessors of the device
+    int dw_simt_max = 1;           // row slices sc.dw_spart has room for on the plain path
     bool lm_ce_stream = false;     // LM cross-entropy as a register-resident stream over the logits (V <= 32768, V % 4 == 0)
     HostCache hc;                  // out-of-core mode (pac_cache_register_host)
     TBody tb;                      // transformer-body adapters (plain fp32 kernels)
@@ -348,17 +356,50 @@ pac_status stage_ids(pac_ctx* c, const int* ids, int B, const char* who) {
 // ---------------------------------------------------------------------------
 // Forward: u_l for every layer, the chain, and the head.  ids are on the device.
 // ---------------------------------------------------------------------------
+// out[z] = rows(z) W[z] in fp32.  Tile widths follow N (a 64-wide tile of N = 16 would multiply 48 columns of zeros);
+// few 64-row tiles: 32-row tiles, so that the same work spreads over twice the CTAs.
+template <class AL>
+pac_status sgemm_rows(pac_ctx* c, int M, int N, int K, int Z, const AL& A, const SgRows& W, float* out, long long zstride) {
+    auto grid = [&](int bm, int bn) { return dim3(cdiv(N, bn), cdiv(M, bm), (unsigned)Z); };
+    cudaStream_t st = c->stream;
+    if (N <= 16) sgemm_rows_kernel<32, 16, 2, 2><<<grid(32, 16), 128, 0, st>>>(M, N, K, A, W, out, zstride);
+    else if (N <= 32 || (N > 64 && N <= 96)) sgemm_rows_kernel<64, 32, 4, 4><<<grid(64, 32), 128, 0, st>>>(M, N, K, A, W, out, zstride);
+    else if ((long long)cdiv(N, 64) * cdiv(M, 64) * Z < c->sms) sgemm_rows_kernel<32, 64, 4, 4><<<grid(32, 64), 128, 0, st>>>(M, N, K, A, W, out, zstride);
+    else sgemm_rows_kernel<64, 64, 8, 4><<<grid(64, 64), 128, 0, st>>>(M, N, K, A, W, out, zstride);
+    LAUNCH_CHECK(c);
+    return PAC_OK;
+}
+
+// Tile of the A^T B products whose output is N wide.
+void tn_tile(int N, int* bi, int* bj) { *bi = 64; *bj = N <= 16 ? 16 : (N <= 32 || (N > 64 && N <= 96)) ? 32 : 64; }
+
+// The jobs' products over M rows for all Z layers, `slices` row slices (partial sums part_stride apart when more than one).
+template <class AL>
+pac_status sgemm_tn(pac_ctx* c, const TnJobs<AL>& J, int M, int Z, int slices, float* out, long long zstride, long long part_stride) {
+    const int m_slice = (int)cdiv(cdiv(M, slices), TN_KR) * TN_KR;
+    dim3 grid((unsigned)J.first[J.n], (unsigned)Z, (unsigned)slices);
+    cudaStream_t st = c->stream;
+    if (J.tile_j == 16) sgemm_tn_kernel<64, 16, 4, 2><<<grid, 128, 0, st>>>(J, M, m_slice, out, zstride, part_stride);
+    else if (J.tile_j == 32) sgemm_tn_kernel<64, 32, 4, 4><<<grid, 128, 0, st>>>(J, M, m_slice, out, zstride, part_stride);
+    else sgemm_tn_kernel<64, 64, 8, 4><<<grid, 128, 0, st>>>(J, M, m_slice, out, zstride, part_stride);
+    LAUNCH_CHECK(c);
+    return PAC_OK;
+}
+
+SgRows sg_rows(const float* base, long long zstride, int ld) {
+    return SgRows{base, zstride, ld, ((uintptr_t)base & 15) == 0 && zstride % 4 == 0 && ld % 4 == 0};
+}
+template <typename T>
+SgCacheRows<T> sg_cache_rows(const pac_ctx* c, const int* d_ids) {
+    const Dims& dm = c->dm;
+    return SgCacheRows<T>{(const T*)c->cache, d_ids, dm.N, dm.L, dm.S, dm.d, dm.d % 4 == 0};
+}
+
 template <typename T>
 pac_status down_projection_simt(pac_ctx* c, const int* d_ids, int B) {
     const Dims& dm = c->dm;
-    const int M = B * dm.S;
-    CacheRows<T> A{(const T*)c->cache, d_ids, dm.N, dm.L, dm.S, dm.d, 0};
-    MatB_RowMajor Bm{{c->params + c->lay.w_down, (long long)dm.d * dm.r, dm.r}};
-    StoreRowMajor E{c->sc.u, (long long)c->max_rows * dm.r, dm.r};
-    dim3 grid(cdiv(dm.r, SG_BN), cdiv(M, SG_BM), dm.L);
-    gemm_simt<<<grid, 256, 0, c->stream>>>(M, dm.r, dm.d, A, Bm, E);
-    LAUNCH_CHECK(c);
-    return PAC_OK;
+    return sgemm_rows(c, B * dm.S, dm.r, dm.d, dm.L, sg_cache_rows<T>(c, d_ids), sg_rows(c->params + c->lay.w_down, (long long)dm.d * dm.r, dm.r),
+                      c->sc.u, (long long)c->max_rows * dm.r);
 }
 
 pac_status forward(pac_ctx* c, const int* d_ids, int B, bool train, float* d_logits_out) {
@@ -444,15 +485,25 @@ pac_status forward(pac_ctx* c, const int* d_ids, int B, bool train, float* d_log
     return PAC_OK;
 }
 
-template <typename T>
-pac_status dw_down_simt(pac_ctx* c, const int* d_ids, int B) {
+// Row slices of the plain path's dW_down (partial sums in sc.dw_spart when more than one).
+int dw_simt_slices(const pac_ctx* c, int B) {
     const Dims& dm = c->dm;
-    const int M = B * dm.S;
-    CacheRowsT<T> A{(const T*)c->cache, d_ids, dm.N, dm.L, dm.S, dm.d};
-    MatB_RowMajor Bm{{c->sc.du, (long long)c->max_rows * dm.r, dm.r}};
-    StoreRowMajor E{c->grads + c->lay.w_down, (long long)dm.d * dm.r, dm.r};
-    dim3 grid(cdiv(dm.r, SG_BN), cdiv(dm.d, SG_BM), dm.L);
-    gemm_simt<<<grid, 256, 0, c->stream>>>(dm.d, dm.r, M, A, Bm, E);
+    int bi, bj;
+    tn_tile(dm.r, &bi, &bj);
+    return c->sc.dw_spart ? tn_slices((long long)dm.L * cdiv(dm.d, bi) * cdiv(dm.r, bj), B * dm.S, c->sms, c->dw_simt_max) : 1;
+}
+
+template <typename T>
+pac_status dw_down_simt(pac_ctx* c, const int* d_ids, int B, bool reduce_splits) {
+    const Dims& dm = c->dm;
+    TnJobs<SgCacheRows<T>> J;
+    tn_tile(dm.r, &J.tile_i, &J.tile_j);
+    J.add(sg_cache_rows<T>(c, d_ids), dm.d, sg_rows(c->sc.du, (long long)c->max_rows * dm.r, dm.r), dm.r, 0);
+    const int slices = dw_simt_slices(c, B);
+    const long long ne = (long long)dm.L * dm.d * dm.r;
+    pac_status st = sgemm_tn(c, J, B * dm.S, dm.L, slices, slices > 1 ? c->sc.dw_spart : c->grads + c->lay.w_down, (long long)dm.d * dm.r, ne);
+    if (st != PAC_OK || slices == 1 || !reduce_splits) return st;
+    reduce_splits_kernel<<<cdiv(ne / 4, 256), 256, 0, c->stream>>>(c->sc.dw_spart, slices, ne, c->grads + c->lay.w_down);
     LAUNCH_CHECK(c);
     return PAC_OK;
 }
@@ -501,23 +552,19 @@ pac_status backward(pac_ctx* c, const int* d_ids, int B, float* d_loss) {
             return (int)std::max<long long>(1, s);
         };
         // dW_up = a_L^T dy
-        dim3 g2(cdiv(dm.d, SG_BN), cdiv(dm.r, SG_BM), 1);
-        MatA_ColMajor At{{aL, 0, dm.r}};
-        MatB_RowMajor Bd{{sc.dy, 0, dm.d}};
-        const int s2 = k_slices((long long)g2.x * g2.y, M, (long long)dm.r * dm.d);
-        if (s2 > 1) {
-            const int k_slice = (int)cdiv(cdiv(M, s2), SG_BK) * SG_BK;
-            g2.z = cdiv(M, k_slice);
-            gemm_simt_ksplit<<<g2, 256, 0, c->stream>>>(dm.r, dm.d, M, k_slice, At, Bd, sc.lm_part);
-            LAUNCH_CHECK(c);
+        {
+            TnJobs<SgRows> J;
+            tn_tile(dm.d, &J.tile_i, &J.tile_j);
+            J.add(sg_rows(aL, 0, dm.r), dm.r, sg_rows(sc.dy, 0, dm.d), dm.d, 0);
             const long long ne = (long long)dm.r * dm.d;
-            reduce_splits_kernel<<<cdiv(ne / 4, 256), 256, 0, c->stream>>>(sc.lm_part, (int)g2.z, ne, c->grads + c->lay.w_up);
-            c->launches++;
-        } else {
-            StoreRowMajor Eu{c->grads + c->lay.w_up, 0, dm.d};
-            gemm_simt<<<g2, 256, 0, c->stream>>>(dm.r, dm.d, M, At, Bd, Eu);
+            const int sl = sc.lm_part && ne % 4 == 0 ? tn_slices(J.first[1], M, c->sms, LM_MAX_K_SLICES) : 1;
+            pac_status ts = sgemm_tn(c, J, M, 1, sl, sl > 1 ? sc.lm_part : c->grads + c->lay.w_up, 0, ne);
+            if (ts != PAC_OK) return ts;
+            if (sl > 1) {
+                sum_slices_kernel<<<cdiv(ne / 4, 256), 256, 0, c->stream>>>(sc.lm_part, sl, ne, c->grads + c->lay.w_up);
+                LAUNCH_CHECK(c);
+            }
         }
-        LAUNCH_CHECK(c);
         // da_L = dy W_up^T: on the tensor cores when the bf16 copy of dy exists (da_L only feeds du, which is
         // rounded to bf16 anyway).  dW_up above stays in fp32 FMA: with a_L and dy rounded to bf16 its error,
         // amplified by Adam, took the parameters after ten steps past the 1e-2 bound (1.1e-2 measured).
@@ -732,7 +779,7 @@ pac_status dw_down(pac_ctx* c, const int* d_ids, int B, bool reduce_splits) {
                             c->step_early_ids && !c->step_host_ids);       // ids no kernel in flight writes
         if (st != PAC_OK) return fail(c, st, "tensor-core dW_down launch failed: %s", tensor_last_error());
     } else {
-        st = c->dtype == PAC_F32 ? dw_down_simt<float>(c, d_ids, B) : dw_down_simt<bf16>(c, d_ids, B);
+        st = c->dtype == PAC_F32 ? dw_down_simt<float>(c, d_ids, B, reduce_splits) : dw_down_simt<bf16>(c, d_ids, B, reduce_splits);
         if (st != PAC_OK) return st;
     }
     time_mark(c, 2, true);
@@ -863,8 +910,8 @@ pac_status finalize_enqueue(pac_ctx* c, const int* d_ids, int B, float* d_loss, 
     Scratch& sc = c->sc;
     FinalizeParams f{};
     f.lay = c->lay; f.B = B; f.d = dm.d; f.r = dm.r; f.C = dm.C; f.L = dm.L;
-    f.dw_part = sc.dw_part;
-    f.splits = use_tensor(c) ? tensor_splits(c->tplan, B) : 1;
+    f.dw_part = use_tensor(c) ? sc.dw_part : sc.dw_spart;
+    f.splits = use_tensor(c) ? tensor_splits(c->tplan, B) : dw_simt_slices(c, B);
     f.dw_elems = (long long)dm.L * dm.d * dm.r;
     f.lam_part = sc.lam_part; f.lam_blocks = B * cls_cluster_size(c, B);
     f.pooled_a = sc.pooled_a; f.dlogits = sc.dlogits; f.loss_b = sc.loss_b;
@@ -958,7 +1005,7 @@ void free_all(pac_ctx* c) {
     Scratch& s = c->sc;
     if (c->hc.on) s.hbar = nullptr;            // points into a staging slot, freed below
     void* ptrs[] = {s.ids, s.u, s.a, s.du, s.du16, s.lam_part, s.loss, s.hbar, s.pooled_a, s.pooled_y, s.logits,
-                    s.dlogits, s.loss_b, s.gvec, s.daL, s.y, s.lm_logits, s.dy, s.y16, s.dlog16, s.aL16, s.wup16, s.dy16, s.wdT, s.lm_part, s.dw_part, s.gates, s.pool_part, s.prodW, c->tb.buf, c->params, c->grads,
+                    s.dlogits, s.loss_b, s.gvec, s.daL, s.y, s.lm_logits, s.dy, s.y16, s.dlog16, s.aL16, s.wup16, s.dy16, s.wdT, s.lm_part, s.dw_part, s.dw_spart, s.gates, s.pool_part, s.prodW, c->tb.buf, c->params, c->grads,
                     c->m, c->v, c->status, c->d_perm, c->d_losses, c->d_stamps};
     for (void* p : ptrs)
         if (p) cudaFree(p);
@@ -1285,7 +1332,14 @@ pac_status pac_adapter_init(pac_ctx* c, const pac_adapter_cfg* cfg, unsigned lon
             c->lm_skinny_tensor = g1 == PAC_OK && g2 == PAC_OK;
         }
     }
-    if (st == PAC_OK && !use_tensor(c)) A(dmalloc(c, &s.du, Mr * dm.L));    // the plain path keeps du in fp32
+    if (st == PAC_OK && !use_tensor(c)) {
+        A(dmalloc(c, &s.du, Mr * dm.L));    // the plain path keeps du in fp32
+        const long long ne = (long long)dm.L * dm.d * dm.r;
+        int bi, bj;
+        tn_tile(dm.r, &bi, &bj);
+        c->dw_simt_max = ne % 4 == 0 ? tn_slices((long long)dm.L * cdiv(dm.d, bi) * cdiv(dm.r, bj), c->max_rows, c->sms, 8) : 1;
+        if (c->dw_simt_max > 1) A(dmalloc(c, &s.dw_spart, ne * c->dw_simt_max));
+    }
     if (st == PAC_OK && c->tb.on) {
         TBody& t = c->tb;
         const long long Mx = c->max_rows;
