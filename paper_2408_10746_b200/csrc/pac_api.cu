@@ -21,6 +21,7 @@
 #include "pac_quant.cuh"
 #include "pac_tbody.cuh"
 #include "pac_sgemm.cuh"
+#include "pac_tbody_fused.cuh"
 
 using namespace pac;
 
@@ -79,7 +80,9 @@ struct TBody {
     // work buffers of the backward pass
     float *da = nullptr, *dx1 = nullptr, *dn = nullptr, *dqkv = nullptr, *dpre = nullptr, *dtmp = nullptr;
     long long sMr = 0, sMf = 0, sP = 0, sM = 0;      // per-layer strides of the stacks
-};
+    // one launch per layer boundary (pac_tbody_fused.cuh) when the widths fit its shared memory; x, xhat1, n1, qkv, o,
+    // xhat2, n2, P, rstd1, rstd2 above are its stacks too, the rest of the kernels above are then not used
+    TbPlan plan{};
     TbPack pk{};
     TbStacks st{};
     float *packed = nullptr, *wg_part = nullptr;     // weights laid out for the ring [L][..]; row slices of the weight products
@@ -622,6 +625,83 @@ pac_status tb_gemm(pac_ctx* c, int M, int N, int K, int Z, const AF& A, const BF
 }
 #define TB_OK(call) do { pac_status s_ = (call); if (s_ != PAC_OK) return s_; } while (0)
 
+// Launches of pac_tbody_fused.cuh: what every layer boundary has in common.
+TbLayerParams tb_params(pac_ctx* c, int B, bool train) {
+    TBody& t = c->tb;
+    TbLayerParams p{};
+    p.B = B; p.S = c->dm.S; p.r = c->dm.r; p.f = t.f; p.H = t.H; p.train = train ? 1 : 0;
+    p.s = t.st;
+    p.u = c->sc.u; p.u_stride = (long long)c->max_rows * c->dm.r; p.du = c->sc.du;
+    p.lam = c->params + c->lay.lam; p.daL = c->sc.daL;
+    return p;
+}
+
+pac_status tb_fused_forward(pac_ctx* c, int B, bool train) {
+    TBody& t = c->tb;
+    const TbPack& pk = t.pk;
+    const BodyLayout& bl = t.bl;
+    const int L = c->dm.L;
+    for (int i = 0; i <= L; ++i) {
+        TbLayerParams p = tb_params(c, B, train);
+        p.tail = i - 1; p.head = i < L ? i : -1;
+        if (p.tail >= 0) {
+            const float *w = t.packed + p.tail * pk.per_layer, *v = c->params + c->lay.body + p.tail * bl.per_layer;
+            for (int m = 0; m < 3; ++m) p.mats[m] = pk.mat(w, m);
+            p.g2 = v + bl.g2; p.b2 = v + bl.b2; p.c1 = v + bl.c1; p.c2 = v + bl.c2;
+        }
+        if (p.head >= 0) {
+            const float* v = c->params + c->lay.body + p.head * bl.per_layer;
+            p.mats[3] = pk.mat(t.packed + p.head * pk.per_layer, 3);
+            p.g1 = v + bl.g1; p.b1 = v + bl.b1;
+        }
+        cudaError_t e = tb_layer_launch(t.plan, p, false, c->stream);
+        c->launches++;
+        if (e != cudaSuccess) return fail(c, PAC_ERR_CUDA, "transformer-body forward launch failed: %s", cudaGetErrorString(e));
+    }
+    return PAC_OK;
+}
+
+pac_status tb_fused_backward(pac_ctx* c, int B) {
+    TBody& t = c->tb;
+    const TbPack& pk = t.pk;
+    const BodyLayout& bl = t.bl;
+    const TbStacks& s = t.st;
+    const int L = c->dm.L, r = c->dm.r, f = t.f, M = B * c->dm.S;
+    for (int l = L - 1; l >= -1; --l) {
+        TbLayerParams p = tb_params(c, B, true);
+        p.tail = l + 1 < L ? l + 1 : -1; p.head = l;
+        if (p.tail >= 0) {
+            p.mats[0] = pk.mat(t.packed + p.tail * pk.per_layer, 4);
+            p.g1 = c->params + c->lay.body + p.tail * bl.per_layer + bl.g1;
+        }
+        if (p.head >= 0) {
+            const float* w = t.packed + p.head * pk.per_layer;
+            for (int m = 1; m < 4; ++m) p.mats[m] = pk.mat(w, 4 + m);
+            p.g2 = c->params + c->lay.body + p.head * bl.per_layer + bl.g2;
+        }
+        cudaError_t e = tb_layer_launch(t.plan, p, true, c->stream);
+        c->launches++;
+        if (e != cudaSuccess) return fail(c, PAC_ERR_CUDA, "transformer-body backward launch failed: %s", cudaGetErrorString(e));
+    }
+    float* gbody = c->grads + c->lay.body;
+    tb_reduce_parts_kernel<<<dim3(cdiv(s.part_w, 32), (unsigned)L), 256, 0, c->stream>>>(s.part, tb_ctas(B, c->dm.S), s.part_w, r, f, bl, gbody, c->grads + c->lay.lam);
+    LAUNCH_CHECK(c);
+    // dW = A^T B over all rows, all six products of all layers at once
+    const long long rr = (long long)r * r, rf = (long long)r * f, per = 4 * rr + 2 * rf;
+    TnJobs<SgRows> J;
+    tn_tile(r, &J.tile_i, &J.tile_j);
+    for (int k = 0; k < 3; ++k) J.add(sg_rows(s.n1, s.sMr, r), r, sg_rows(s.dqkv + k * s.sMr, 3 * s.sMr, r), r, k * rr);
+    J.add(sg_rows(s.o, s.sMr, r), r, sg_rows(s.dx1, s.sMr, r), r, 3 * rr);
+    J.add(sg_rows(s.n2, s.sMr, r), r, sg_rows(s.dpre, s.sMf, f), f, 4 * rr);
+    J.add(sg_rows(s.hid, s.sMf, f), f, sg_rows(s.da, s.sMr, r), r, 4 * rr + rf);
+    const int slices = tn_slices((long long)J.first[J.n] * L, M, c->sms, t.wg_slices);
+    pac_status st = sgemm_tn(c, J, M, L, slices, t.wg_part, per, per * L);
+    if (st != PAC_OK) return st;
+    tb_reduce_slices_kernel<<<dim3(cdiv(per, 256), (unsigned)L), 256, 0, c->stream>>>(t.wg_part, slices, per * L, per, bl, gbody);
+    LAUNCH_CHECK(c);
+    return PAC_OK;
+}
+
 pac_status tb_forward(pac_ctx* c, const int* d_ids, int B, bool train, float* d_logits_out) {
     const Dims& dm = c->dm;
     TBody& t = c->tb;
@@ -630,10 +710,15 @@ pac_status tb_forward(pac_ctx* c, const int* d_ids, int B, bool train, float* d_
     const int M = B * dm.S, r = dm.r, f = t.f;
     const long long n = (long long)M * r, stride = (long long)c->max_rows * r;
     cudaStream_t st = c->stream;
+    if (t.plan.ok) {
+        tb_pack_kernel<<<dim3(cdiv(t.pk.per_layer, 1024), (unsigned)dm.L), 256, 0, st>>>(c->params + c->lay.body, bl.per_layer, bl, t.pk, t.packed);
+        LAUNCH_CHECK(c);
+    }
     TB_OK(down_projection(c, d_ids, B));
     const float* lam = c->params + c->lay.lam;
     const unsigned rows_grid = cdiv(M, 8), heads_grid = cdiv((long long)B * t.H * dm.S, 128);
-    for (int l = 0; l < dm.L; ++l) {
+    if (t.plan.ok) TB_OK(tb_fused_forward(c, B, train));
+    for (int l = 0; l < dm.L && !t.plan.ok; ++l) {
         const float* w = c->params + c->lay.body + (long long)l * bl.per_layer;
         float *x = t.x + l * t.sMr, *xhat1 = t.xhat1 + l * t.sMr, *n1 = t.n1 + l * t.sMr, *qkv = t.qkv + 3 * l * t.sMr,
               *o = t.o + l * t.sMr, *x1 = t.x1 + l * t.sMr, *xhat2 = t.xhat2 + l * t.sMr, *n2 = t.n2 + l * t.sMr,
@@ -679,6 +764,10 @@ pac_status tb_backward(pac_ctx* c, const int* d_ids, int B, float* d_loss) {
         cls_grads_kernel<<<cdiv(ne, 256), 256, 0, st>>>(sc.pooled_a, sc.gvec, sc.pooled_y, sc.dlogits, sc.loss_b, B, dm.d, r, dm.C,
                                                         c->grads + c->lay.w_up, c->grads + c->lay.w_head, c->grads + c->lay.b_head, d_loss);
         LAUNCH_CHECK(c);
+    }
+    if (t.plan.ok) {
+        TB_OK(tb_fused_backward(c, B));
+        return dw_down(c, d_ids, B, true);
     }
     tb_expand_kernel<<<cdiv(n, 256), 256, 0, st>>>(sc.daL, dm.S, r, n, t.da);
     LAUNCH_CHECK(c);
@@ -1344,6 +1433,30 @@ pac_status pac_adapter_init(pac_ctx* c, const pac_adapter_cfg* cfg, unsigned lon
         TBody& t = c->tb;
         const long long Mx = c->max_rows;
         t.sMr = Mx * dm.r; t.sMf = Mx * t.f; t.sP = (long long)cfg->max_batch * t.H * dm.S * dm.S; t.sM = Mx;
+        int max_smem = 0;
+        CU_OK(c, cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device));
+        t.plan = tb_plan(dm.S, dm.r, t.f, t.H, max_smem);
+        if (t.plan.ok) {
+            TbStacks& k = t.st;
+            t.pk = TbPack::make(dm.r, t.f);
+            k.sMr = (t.sMr + 3) & ~3LL; k.sMf = (t.sMf + 3) & ~3LL; k.sP = t.sP; k.sM = t.sM;
+            k.part_w = 5 * dm.r + t.f + 1;
+            const long long ctas = tb_ctas(cfg->max_batch, dm.S);
+            const long long per = 4LL * dm.r * dm.r + 2LL * dm.r * t.f;
+            t.wg_slices = 8;
+            const long long parts[] = {
+                k.sMr * dm.L, k.sMr * dm.L, k.sMr * dm.L, 3 * k.sMr * dm.L, k.sMr * dm.L, k.sMr * dm.L, k.sMr * dm.L,
+                k.sMf * dm.L, k.sP * dm.L, k.sM * dm.L, k.sM * dm.L, k.sMr * dm.L, k.sMr * dm.L, 3 * k.sMr * dm.L, k.sMf * dm.L,
+                k.sMr, k.sMr, k.sP, k.sP, ctas * k.part_w * dm.L, t.pk.per_layer * dm.L, per * dm.L * t.wg_slices};
+            float** const where[] = {&k.x, &k.xhat1, &k.n1, &k.qkv, &k.o, &k.xhat2, &k.n2, &k.hid, &k.P, &k.rstd1, &k.rstd2, &k.da,
+                                     &k.dx1, &k.dqkv, &k.dpre, &k.dob[0], &k.dob[1], &k.dS[0], &k.dS[1], &k.part, &t.packed, &t.wg_part};
+            long long total = 0;
+            for (long long q : parts) total += (q + 3) & ~3LL;
+            A(dmalloc(c, &t.buf, total));
+            float* q = t.buf;
+            for (size_t i = 0; i < sizeof(parts) / sizeof(parts[0]); ++i) { *where[i] = q; q += (parts[i] + 3) & ~3LL; }
+            k.a = s.a;
+        } else {
         const long long per_layer = 10 * t.sMr + t.sMf + t.sP + 2 * t.sM;     // x xhat1 n1 qkv(3) o x1 xhat2 n2 | pre | P | rstd1 rstd2
         const long long work = 7 * t.sMr + t.sMf;                             // da dx1 dn dqkv(3) dtmp | dpre
         A(dmalloc(c, &t.buf, per_layer * dm.L + work));
@@ -1355,6 +1468,7 @@ pac_status pac_adapter_init(pac_ctx* c, const pac_adapter_cfg* cfg, unsigned lon
             t.pre = take(t.sMf * dm.L); t.P = take(t.sP * dm.L); t.rstd1 = take(t.sM * dm.L); t.rstd2 = take(t.sM * dm.L);
             t.da = take(t.sMr); t.dx1 = take(t.sMr); t.dn = take(t.sMr); t.dqkv = take(3 * t.sMr); t.dtmp = take(t.sMr);
             t.dpre = take(t.sMf);
+        }
         }
     }
     if (st != PAC_OK) return st;
