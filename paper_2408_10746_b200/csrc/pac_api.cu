@@ -37,7 +37,7 @@ struct Scratch {
     float* u = nullptr;            // [L][M][r] down-projections
     float* a = nullptr;            // [L][M][r] adapter states
     float* du = nullptr;           // [L][M][r] fp32 (plain path)
-    bf16* du16 = nullptr;          // [L][M][r] bf16 (tensor path)
+    bf16* du16 = nullptr;          // [L][M][r] bf16 (tensor path), or three terms of du, [L][3][M][r]
     float* lam_part = nullptr;     // [L][blocks]
     float* loss = nullptr;         // [1]
     // classifier head
@@ -59,7 +59,7 @@ struct Scratch {
     bf16* wup16 = nullptr;
     bf16* dy16 = nullptr;
     // tensor path
-    bf16* wdT = nullptr;           // [L][2][d][r] bf16 hi/lo shadow of W_down
+    bf16* wdT = nullptr;           // bf16 terms of W_down, [L][2 or 3][d][r]
     float* lm_part = nullptr;      // [slices][...] partial sums of the LM path's two skinny products (dW_up, da_L)
     float* dw_part = nullptr;      // split partials of dW_down
     float* dw_spart = nullptr;     // row-slice partials of dW_down on the plain path
@@ -189,6 +189,7 @@ struct pac_ctx {
     unsigned long long* d_stamps = nullptr;
     size_t stamps_used[2] = {0, 0};
     bool tensor_ok = false;
+    bool exact_ok = false;         // the two cache passes run on the tensor cores at fp32 precision (three bf16 terms per fp32 operand)
     long long launches = 0;
     TensorPlan tplan{};
     MidPlan mplan{};               // fused classifier-head kernel (when the shape allows)
@@ -258,6 +259,7 @@ pac_status dmalloc(pac_ctx* c, T** p, long long n) {
 }
 
 bool use_tensor(const pac_ctx* c) { return c->tensor_ok && !c->force_simt; }
+WdShadow wd_shadow(const pac_ctx* c) { return WdShadow{c->sc.wdT, c->exact_ok ? 3 : 2}; }
 pac_status adam_enqueue(pac_ctx* c, const pac_adamw* hp);
 pac_status down_projection(pac_ctx* c, const int* d_ids, int B);
 pac_status dw_down(pac_ctx* c, const int* d_ids, int B, bool reduce_splits);
@@ -405,12 +407,55 @@ pac_status down_projection_simt(pac_ctx* c, const int* d_ids, int B) {
                       c->sc.u, (long long)c->max_rows * dm.r);
 }
 
+pac_status head_matrix_enqueue(pac_ctx* c);
+pac_status finalize_enqueue(pac_ctx* c, const int* d_ids, int B, float* d_loss, const pac_adamw* hp);
+pac_status adam_body_enqueue(pac_ctx* c, const pac_adamw* hp);
+
+// Classifier heads outside the fused kernels: few classes take plain_head_kernel and the finalisation kernel, whose W_down blocks
+// move four elements at a time; otherwise the kernels that form the d-wide vectors.
+bool plain_head_ok(const pac_ctx* c, int B) {
+    const Dims& dm = c->dm;
+    return c->cfg.head == PAC_HEAD_MEANPOOL_CLS && dm.C <= MID_MAX_C && 9 * dm.r + dm.C + 32 <= 12000 && ((long long)dm.L * dm.d * dm.r) % 4 == 0 &&
+           (2LL * B + dm.r + dm.C) * FIN_KB * 4 <= 48 * 1024;
+}
+pac_status plain_head(pac_ctx* c, const int* d_ids, int B, bool train, const float* aL, float* d_logits_out) {
+    const Dims& dm = c->dm;
+    Scratch& sc = c->sc;
+    float* lg = train ? sc.logits : d_logits_out;
+    if (plain_head_ok(c, B)) {
+        const size_t smem = sizeof(float) * (9 * dm.r + dm.C + 32);
+        plain_head_kernel<<<B, 256, smem, c->stream>>>(aL, sc.hbar, d_ids, dm.N, c->labels, sc.prodW, c->params + c->lay.w_head, c->params + c->lay.b_head, B,
+                                                       dm.S, dm.d, dm.r, dm.C, train ? 1 : 0, sc.pooled_a, lg, sc.loss_b, sc.dlogits, sc.daL, c->status);
+        LAUNCH_CHECK(c);
+        return PAC_OK;
+    }
+    pool_tokens_kernel<<<B, 128, 0, c->stream>>>(aL, sc.pooled_a, dm.S, dm.r);
+    LAUNCH_CHECK(c);
+    const size_t smem = sizeof(float) * (dm.d + dm.C + 32);
+    cls_head_kernel<<<B, 256, smem, c->stream>>>(sc.hbar, d_ids, dm.N, c->labels, sc.pooled_a, c->params + c->lay.w_up,
+                                                 c->params + c->lay.w_head, c->params + c->lay.b_head, B, dm.S, dm.d, dm.r, dm.C,
+                                                 train ? 1 : 0, sc.pooled_y, lg, sc.loss_b, sc.dlogits, sc.gvec, sc.daL, c->status);
+    LAUNCH_CHECK(c);
+    return PAC_OK;
+}
+pac_status plain_head_grads(pac_ctx* c, int B, float* d_loss) {
+    const Dims& dm = c->dm;
+    Scratch& sc = c->sc;
+    const long long n = (long long)dm.r * dm.d + (long long)dm.d * dm.C + dm.C + 1;
+    cls_grads_kernel<<<cdiv(n, 256), 256, 0, c->stream>>>(sc.pooled_a, sc.gvec, sc.pooled_y, sc.dlogits, sc.loss_b, B, dm.d, dm.r, dm.C,
+                                                          c->grads + c->lay.w_up, c->grads + c->lay.w_head, c->grads + c->lay.b_head, d_loss);
+    LAUNCH_CHECK(c);
+    return PAC_OK;
+}
+
 pac_status forward(pac_ctx* c, const int* d_ids, int B, bool train, float* d_logits_out) {
     const Dims& dm = c->dm;
     const int M = B * dm.S;
     const long long n = (long long)M * dm.r, stride = (long long)c->max_rows * dm.r;
     Scratch& sc = c->sc;
-    pac_status st = down_projection(c, d_ids, B);
+    pac_status st = PAC_OK;
+    if (plain_head_ok(c, B) && (st = head_matrix_enqueue(c)) != PAC_OK) return st;
+    st = down_projection(c, d_ids, B);
     if (st != PAC_OK) return st;
     const float* lam = c->params + c->lay.lam;
     if (c->cfg.act == PAC_ACT_RELU)
@@ -421,15 +466,7 @@ pac_status forward(pac_ctx* c, const int* d_ids, int B, bool train, float* d_log
     const float* aL = sc.a + (long long)(dm.L - 1) * stride;
     const float* W_up = c->params + c->lay.w_up;
     if (c->cfg.head == PAC_HEAD_MEANPOOL_CLS) {
-        pool_tokens_kernel<<<B, 128, 0, c->stream>>>(aL, sc.pooled_a, dm.S, dm.r);
-        LAUNCH_CHECK(c);
-        size_t smem = sizeof(float) * (dm.d + dm.C + 32);
-        cls_head_kernel<<<B, 256, smem, c->stream>>>(sc.hbar, d_ids, dm.N, c->labels, sc.pooled_a, W_up,
-                                                     c->params + c->lay.w_head, c->params + c->lay.b_head, B, dm.S,
-                                                     dm.d, dm.r, dm.C, train ? 1 : 0, sc.pooled_y,
-                                                     train ? sc.logits : d_logits_out, sc.loss_b, sc.dlogits,
-                                                     sc.gvec, sc.daL, c->status);
-        LAUNCH_CHECK(c);
+        if ((st = plain_head(c, d_ids, B, train, aL, d_logits_out)) != PAC_OK) return st;
     } else {
         // y = h_L + a_L W_up
         dim3 g1(cdiv(dm.d, SG_BN), cdiv(M, SG_BM), 1);
@@ -512,7 +549,7 @@ pac_status dw_down_simt(pac_ctx* c, const int* d_ids, int B, bool reduce_splits)
 }
 
 // Backward through the adapters only, after forward(train=true).  d_loss receives the mean loss.
-pac_status backward(pac_ctx* c, const int* d_ids, int B, float* d_loss) {
+pac_status backward(pac_ctx* c, const int* d_ids, int B, float* d_loss, const pac_adamw* hp, bool* updated) {
     const Dims& dm = c->dm;
     const int M = B * dm.S;
     const long long n = (long long)M * dm.r, stride = (long long)c->max_rows * dm.r;
@@ -521,11 +558,10 @@ pac_status backward(pac_ctx* c, const int* d_ids, int B, float* d_loss) {
     const float* W_up = c->params + c->lay.w_up;
     int per_sample;
     if (c->cfg.head == PAC_HEAD_MEANPOOL_CLS) {
-        long long n = (long long)dm.r * dm.d + (long long)dm.d * dm.C + dm.C + 1;
-        cls_grads_kernel<<<cdiv(n, 256), 256, 0, c->stream>>>(sc.pooled_a, sc.gvec, sc.pooled_y, sc.dlogits, sc.loss_b,
-                                                              B, dm.d, dm.r, dm.C, c->grads + c->lay.w_up,
-                                                              c->grads + c->lay.w_head, c->grads + c->lay.b_head, d_loss);
-        LAUNCH_CHECK(c);
+        if (!plain_head_ok(c, B)) {
+            pac_status hs = plain_head_grads(c, B, d_loss);
+            if (hs != PAC_OK) return hs;
+        }
         per_sample = 1;
     } else {
         mean_kernel<<<1, 1024, 0, c->stream>>>(sc.loss_b, M, d_loss);
@@ -608,8 +644,16 @@ pac_status backward(pac_ctx* c, const int* d_ids, int B, float* d_loss) {
     }
 #undef CHAIN_BWD
     LAUNCH_CHECK(c);
-    reduce_rows_kernel<<<dm.L, 256, 0, c->stream>>>(sc.lam_part, (int)blocks, c->grads + c->lay.lam);
-    LAUNCH_CHECK(c);
+    if (!plain_head_ok(c, B)) {
+        reduce_rows_kernel<<<dm.L, 256, 0, c->stream>>>(sc.lam_part, (int)blocks, c->grads + c->lay.lam);
+        LAUNCH_CHECK(c);
+    }
+    if (plain_head_ok(c, B)) {
+        pac_status ds = dw_down(c, d_ids, B, false);
+        if (ds != PAC_OK) return ds;
+        *updated = true;
+        return finalize_enqueue(c, d_ids, B, d_loss, hp);
+    }
     return dw_down(c, d_ids, B, true);
 }
 
@@ -631,7 +675,7 @@ TbLayerParams tb_params(pac_ctx* c, int B, bool train) {
     TbLayerParams p{};
     p.B = B; p.S = c->dm.S; p.r = c->dm.r; p.f = t.f; p.H = t.H; p.train = train ? 1 : 0;
     p.s = t.st;
-    p.u = c->sc.u; p.u_stride = (long long)c->max_rows * c->dm.r; p.du = c->sc.du;
+    p.u = c->sc.u; p.u_stride = (long long)c->max_rows * c->dm.r; p.du = c->sc.du; p.du3 = c->exact_ok ? c->sc.du16 : nullptr;
     p.lam = c->params + c->lay.lam; p.daL = c->sc.daL;
     return p;
 }
@@ -714,6 +758,7 @@ pac_status tb_forward(pac_ctx* c, const int* d_ids, int B, bool train, float* d_
         tb_pack_kernel<<<dim3(cdiv(t.pk.per_layer, 1024), (unsigned)dm.L), 256, 0, st>>>(c->params + c->lay.body, bl.per_layer, bl, t.pk, t.packed);
         LAUNCH_CHECK(c);
     }
+    if (plain_head_ok(c, B)) TB_OK(head_matrix_enqueue(c));
     TB_OK(down_projection(c, d_ids, B));
     const float* lam = c->params + c->lay.lam;
     const unsigned rows_grid = cdiv(M, 8), heads_grid = cdiv((long long)B * t.H * dm.S, 128);
@@ -739,19 +784,19 @@ pac_status tb_forward(pac_ctx* c, const int* d_ids, int B, bool train, float* d_
         TB_OK(tb_gemm(c, M, r, f, 1, MatA_ReluRowMajor{pre, f}, MatB_RowMajor{{w + bl.w2, 0, r}}, StoreAddBias{a, x1, w + bl.c2, r}));
     }
     // head: the same kernels as the point-wise plain path
-    const float* aL = sc.a + (long long)(dm.L - 1) * stride;
-    pool_tokens_kernel<<<B, 128, 0, st>>>(aL, sc.pooled_a, dm.S, r);
-    LAUNCH_CHECK(c);
-    const size_t smem = sizeof(float) * (dm.d + dm.C + 32);
-    cls_head_kernel<<<B, 256, smem, st>>>(sc.hbar, d_ids, dm.N, c->labels, sc.pooled_a, c->params + c->lay.w_up,
-                                          c->params + c->lay.w_head, c->params + c->lay.b_head, B, dm.S, dm.d, r, dm.C,
-                                          train ? 1 : 0, sc.pooled_y, train ? sc.logits : d_logits_out, sc.loss_b, sc.dlogits,
-                                          sc.gvec, sc.daL, c->status);
-    LAUNCH_CHECK(c);
-    return PAC_OK;
+    return plain_head(c, d_ids, B, train, sc.a + (long long)(dm.L - 1) * stride, d_logits_out);
 }
 
-pac_status tb_backward(pac_ctx* c, const int* d_ids, int B, float* d_loss) {
+// dW_down, the head's gradients and, with hp, the update: the finalisation kernel for everything up to the head, adamw_body_kernel
+// for the layers' bodies.
+pac_status tb_finish(pac_ctx* c, const int* d_ids, int B, float* d_loss, const pac_adamw* hp, bool fin) {
+    TB_OK(dw_down(c, d_ids, B, !fin));
+    if (!fin) return hp ? adam_enqueue(c, hp) : PAC_OK;
+    TB_OK(finalize_enqueue(c, d_ids, B, d_loss, hp));
+    return hp ? adam_body_enqueue(c, hp) : PAC_OK;
+}
+
+pac_status tb_backward(pac_ctx* c, const int* d_ids, int B, float* d_loss, const pac_adamw* hp) {
     const Dims& dm = c->dm;
     TBody& t = c->tb;
     const BodyLayout& bl = t.bl;
@@ -759,15 +804,11 @@ pac_status tb_backward(pac_ctx* c, const int* d_ids, int B, float* d_loss) {
     const int M = B * dm.S, r = dm.r, f = t.f;
     const long long n = (long long)M * r, stride = (long long)c->max_rows * r;
     cudaStream_t st = c->stream;
-    {
-        const long long ne = (long long)r * dm.d + (long long)dm.d * dm.C + dm.C + 1;
-        cls_grads_kernel<<<cdiv(ne, 256), 256, 0, st>>>(sc.pooled_a, sc.gvec, sc.pooled_y, sc.dlogits, sc.loss_b, B, dm.d, r, dm.C,
-                                                        c->grads + c->lay.w_up, c->grads + c->lay.w_head, c->grads + c->lay.b_head, d_loss);
-        LAUNCH_CHECK(c);
-    }
+    const bool fin = plain_head_ok(c, B);
+    if (!fin) TB_OK(plain_head_grads(c, B, d_loss));
     if (t.plan.ok) {
         TB_OK(tb_fused_backward(c, B));
-        return dw_down(c, d_ids, B, true);
+        return tb_finish(c, d_ids, B, d_loss, hp, fin);
     }
     tb_expand_kernel<<<cdiv(n, 256), 256, 0, st>>>(sc.daL, dm.S, r, n, t.da);
     LAUNCH_CHECK(c);
@@ -821,7 +862,7 @@ pac_status tb_backward(pac_ctx* c, const int* d_ids, int B, float* d_loss) {
                                               sc.du + l * stride, da, c->grads + c->lay.lam);
         LAUNCH_CHECK(c);
     }
-    return dw_down(c, d_ids, B, true);
+    return tb_finish(c, d_ids, B, d_loss, hp, fin);
 }
 #undef TB_OK
 
@@ -848,7 +889,7 @@ int cls_cluster_size(const pac_ctx* c, int B) {
 pac_status down_projection(pac_ctx* c, const int* d_ids, int B) {
     pac_status st;
     time_mark(c, 0, false);
-    if (use_tensor(c)) {
+    if (use_tensor(c) || c->exact_ok) {
         st = tensor_down_projection(c->tplan, c->stream, d_ids, B, c->sc.u, c->status, &c->launches, next_stamp(c, 0));
         if (st != PAC_OK) return fail(c, st, "tensor-core down-projection launch failed: %s", tensor_last_error());
     } else {
@@ -862,7 +903,7 @@ pac_status down_projection(pac_ctx* c, const int* d_ids, int B) {
 pac_status dw_down(pac_ctx* c, const int* d_ids, int B, bool reduce_splits) {
     pac_status st;
     time_mark(c, 2, false);
-    if (use_tensor(c)) {
+    if (use_tensor(c) || c->exact_ok) {
         st = tensor_dw_down(c->tplan, c->stream, d_ids, B, c->sc.du16, c->grads + c->lay.w_down, c->sc.dw_part,
                             reduce_splits, c->status, &c->launches, next_stamp(c, 1),
                             c->step_early_ids && !c->step_host_ids);       // ids no kernel in flight writes
@@ -999,10 +1040,13 @@ pac_status finalize_enqueue(pac_ctx* c, const int* d_ids, int B, float* d_loss, 
     Scratch& sc = c->sc;
     FinalizeParams f{};
     f.lay = c->lay; f.B = B; f.d = dm.d; f.r = dm.r; f.C = dm.C; f.L = dm.L;
-    f.dw_part = use_tensor(c) ? sc.dw_part : sc.dw_spart;
-    f.splits = use_tensor(c) ? tensor_splits(c->tplan, B) : dw_simt_slices(c, B);
+    const bool tens = use_tensor(c) || c->exact_ok;
+    f.dw_part = tens ? sc.dw_part : sc.dw_spart;
+    f.splits = tens ? tensor_splits(c->tplan, B) : dw_simt_slices(c, B);
     f.dw_elems = (long long)dm.L * dm.d * dm.r;
-    f.lam_part = sc.lam_part; f.lam_blocks = B * cls_cluster_size(c, B);
+    // per-CTA partial sums of dlambda: the fused head kernels', or the plain reverse chain's; transformer bodies: done
+    f.lam_part = c->tb.on ? nullptr : sc.lam_part;
+    f.lam_blocks = use_fused_cls(c) ? B * cls_cluster_size(c, B) : (int)cdiv((long long)B * dm.S * dm.r, 256);
     f.pooled_a = sc.pooled_a; f.dlogits = sc.dlogits; f.loss_b = sc.loss_b;
     f.hbar = sc.hbar; f.ids = d_ids; f.N = dm.N; f.params_in = c->params;
     f.grads = c->grads; f.loss_out = d_loss;
@@ -1011,7 +1055,7 @@ pac_status finalize_enqueue(pac_ctx* c, const int* d_ids, int B, float* d_loss, 
         c->step += 1;
         f.params = c->params; f.m = c->m; f.v = c->v; f.hp = *hp;
         bias_corrections(hp, c->step, &f.bc1, &f.bc2);
-        f.wdT = sc.wdT;
+        f.wdT = wd_shadow(c);
         f.grad_scale = c->grad_scale;
     }
     f.wd_blocks = (int)cdiv(c->lay.lam / 4, 256);
@@ -1044,8 +1088,7 @@ pac_status train_enqueue(pac_ctx* c, const int* d_ids, int B, float* d_loss, con
     pac_status st;
     if (c->tb.on) {
         if ((st = tb_forward(c, d_ids, B, true, nullptr)) != PAC_OK) return st;
-        if ((st = tb_backward(c, d_ids, B, d_loss)) != PAC_OK) return st;
-        return hp ? adam_enqueue(c, hp) : PAC_OK;
+        return tb_backward(c, d_ids, B, d_loss, hp);
     }
     if (use_fused_cls(c)) {
         if ((st = cls_forward_enqueue(c, d_ids, B, true, nullptr)) != PAC_OK) return st;
@@ -1057,8 +1100,20 @@ pac_status train_enqueue(pac_ctx* c, const int* d_ids, int B, float* d_loss, con
         return st;
     }
     if ((st = forward(c, d_ids, B, true, nullptr)) != PAC_OK) return st;
-    if ((st = backward(c, d_ids, B, d_loss)) != PAC_OK) return st;
-    if (hp) return adam_enqueue(c, hp);
+    bool updated = false;
+    if ((st = backward(c, d_ids, B, d_loss, hp, &updated)) != PAC_OK) return st;
+    if (hp && !updated) return adam_enqueue(c, hp);
+    return PAC_OK;
+}
+
+// The transformer bodies' share of the update (step number as set by the update before it).
+pac_status adam_body_enqueue(pac_ctx* c, const pac_adamw* hp) {
+    float bc1, bc2;
+    bias_corrections(hp, c->step, &bc1, &bc2);
+    const int per = (int)c->tb.bl.per_layer;
+    adamw_body_kernel<<<dim3(cdiv(per, 256), (unsigned)c->dm.L), 256, 0, c->stream>>>(c->params + c->lay.body, c->grads + c->lay.body, c->m + c->lay.body,
+                                                                                    c->v + c->lay.body, per, c->tb.bl, *hp, bc1, bc2, c->status, c->grad_scale);
+    LAUNCH_CHECK(c);
     return PAC_OK;
 }
 
@@ -1067,11 +1122,12 @@ pac_status adam_enqueue(pac_ctx* c, const pac_adamw* hp) {
     float bc1, bc2;
     bias_corrections(hp, c->step, &bc1, &bc2);
     const int wd_blocks = (c->lay.lam % 4 == 0) ? (int)cdiv(c->lay.lam / 4, 256) : 0;
-    const unsigned rest = cdiv(c->lay.total - (wd_blocks ? c->lay.lam : 0), 256);
-    adamw_kernel<<<wd_blocks + rest, 256, 0, c->stream>>>(c->params, c->grads, c->m, c->v, c->lay.total, c->lay, *hp, bc1, bc2,
-                                                          c->sc.wdT, c->dm.d, c->dm.r, wd_blocks, c->status, c->grad_scale);
+    const long long total = c->tb.on ? c->lay.body : c->lay.total;
+    const unsigned rest = cdiv(total - (wd_blocks ? c->lay.lam : 0), 256);
+    adamw_kernel<<<wd_blocks + rest, 256, 0, c->stream>>>(c->params, c->grads, c->m, c->v, total, c->lay, *hp, bc1, bc2,
+                                                          wd_shadow(c), c->dm.d, c->dm.r, wd_blocks, c->status, c->grad_scale);
     LAUNCH_CHECK(c);
-    return PAC_OK;
+    return c->tb.on ? adam_body_enqueue(c, hp) : PAC_OK;
 }
 
 pac_status check_hp(pac_ctx* c, const pac_adamw* hp) {
@@ -1085,7 +1141,7 @@ pac_status check_hp(pac_ctx* c, const pac_adamw* hp) {
 pac_status refresh_shadow(pac_ctx* c) {
     if (!c->sc.wdT) return PAC_OK;
     long long n = (long long)c->dm.L * c->dm.d * c->dm.r;
-    shadow_wdown_kernel<<<cdiv(n, 256), 256, 0, c->stream>>>(c->params, c->sc.wdT, c->dm.L, c->dm.d, c->dm.r);
+    shadow_wdown_kernel<<<cdiv(n, 256), 256, 0, c->stream>>>(c->params, wd_shadow(c), c->dm.L, c->dm.d, c->dm.r);
     LAUNCH_CHECK(c);
     return PAC_OK;
 }
@@ -1471,11 +1527,27 @@ pac_status pac_adapter_init(pac_ctx* c, const pac_adapter_cfg* cfg, unsigned lon
         }
         }
     }
+    // transformer bodies on a bf16 cache: the cache passes alone, at the precision of the fp32 kernels around them
+    c->exact_ok = false;
+    if (st == PAC_OK && c->dtype == PAC_BF16 && tensor_shape_supported(dm) && c->tb.plan.ok && !c->force_simt) {
+        A(dmalloc(c, &s.wdT, (long long)dm.L * 3 * dm.r * dm.d));
+        A(dmalloc(c, &s.du16, 3 * Mr * dm.L));
+        long long part_floats = 0;
+        if (st == PAC_OK) {
+            pac_status ts = tensor_plan_create(c->tplan, c->device, (const bf16*)c->cache, dm, cfg->max_batch, s.wdT, s.du16, &part_floats, true);
+            if (ts == PAC_OK) {
+                A(dmalloc(c, &s.dw_part, part_floats));
+                c->exact_ok = st == PAC_OK;
+            } else if (ts != PAC_ERR_UNSUPPORTED) {
+                st = fail(c, ts, "tensor path set-up failed: %s", tensor_last_error());
+            }
+        }
+    }
     if (st != PAC_OK) return st;
     CU_OK(c, cudaMemsetAsync(s.u, 0, sizeof(float) * Mr * dm.L, c->stream));
     CU_OK(c, cudaMemsetAsync(s.a, 0, sizeof(float) * Mr * dm.L, c->stream));
     if (s.du) CU_OK(c, cudaMemsetAsync(s.du, 0, sizeof(float) * Mr * dm.L, c->stream));
-    if (s.du16) CU_OK(c, cudaMemsetAsync(s.du16, 0, sizeof(bf16) * Mr * dm.L, c->stream));
+    if (s.du16) CU_OK(c, cudaMemsetAsync(s.du16, 0, sizeof(bf16) * Mr * dm.L * (c->exact_ok ? 3 : 1), c->stream));
     CU_OK(c, cudaMemsetAsync(c->grads, 0, sizeof(float) * c->lay.total, c->stream));
     CU_OK(c, cudaMemsetAsync(c->m, 0, sizeof(float) * c->lay.total, c->stream));
     CU_OK(c, cudaMemsetAsync(c->v, 0, sizeof(float) * c->lay.total, c->stream));

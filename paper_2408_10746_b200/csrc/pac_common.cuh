@@ -53,6 +53,19 @@ inline cudaError_t smem_opt_in(const void* kernel, size_t bytes) {
     return e;
 }
 
+// bf16 terms of W_down for the tensor-core products, [L][terms][d][r] in the master's order: term 0 = bf16(W), term 1 = bf16(W -
+// term 0), ...; two terms carry about 16 mantissa bits, three the fp32 value exactly.
+struct WdShadow {
+    bf16* p; int terms;
+    __device__ __forceinline__ void put(long long l, long long dr, long long rem, float x) const {
+        for (int t = 0; t < terms; ++t) {
+            const bf16 v = __float2bfloat16(x);
+            p[(l * terms + t) * dr + rem] = v;
+            x -= __bfloat162float(v);
+        }
+    }
+};
+
 struct Dims {
     long long N;   // samples in the cache
     int L, S, d;   // layers, tokens, hidden width

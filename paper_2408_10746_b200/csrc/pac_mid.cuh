@@ -172,6 +172,73 @@ __global__ void __launch_bounds__(256) head_matrix_kernel(const float* __restric
     if (lane == 0) prodW[e] = acc;
 }
 
+// Classifier head of the plain path, one CTA per sample: token mean of a_L, logits from the C-vectors (the head's matrix
+// product prodW = W_up W_head stands in for the d-wide ones), loss, dlogits and da_L / S.  What the parameters' gradients
+// need of the d-wide vectors the finalisation kernel rebuilds.  (The kernel that formed mean_s y and g per sample
+// read W_up twice per sample: 93 us at T5-Base widths against 9.)
+// Dynamic shared memory: 9 r + C + 32 floats.
+__global__ void __launch_bounds__(256) plain_head_kernel(const float* __restrict__ aL, const float* __restrict__ hbar, const int* __restrict__ ids,
+                                                         long long N, const int* __restrict__ labels, const float* __restrict__ prodW,
+                                                         const float* __restrict__ W_head, const float* __restrict__ b_head, int B, int S, int d, int r,
+                                                         int C, int train, float* __restrict__ pooled_a, float* __restrict__ logits_out,
+                                                         float* __restrict__ loss_b, float* __restrict__ dlogits, float* __restrict__ daL, unsigned* status) {
+    extern __shared__ float hsm[];
+    float *pa = hsm, *part = pa + r, *lg = part + 8 * r, *red = lg + C;
+    const int b = blockIdx.x, t = threadIdx.x, warp = t >> 5, lane = t & 31;
+    const long long id = safe_id(ids, b, N, t == 0 ? status : nullptr);
+    for (int c = lane; c < r; c += 32) {
+        const float* col = aL + (long long)b * S * r + c;
+        float acc = 0.f;
+#pragma unroll 8
+        for (int s = warp; s < S; s += 8) acc += __ldg(col + (long long)s * r);
+        part[warp * r + c] = acc;
+    }
+    __syncthreads();
+    for (int c = t; c < r; c += 256) {
+        float acc = 0.f;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) acc += part[w * r + c];
+        pa[c] = acc / (float)S;
+        if (train) pooled_a[(long long)b * r + c] = pa[c];
+    }
+    __syncthreads();
+    for (int c = 0; c < C; ++c) {
+        float acc = 0.f;
+#pragma unroll 4
+        for (int k = t; k < d; k += 256) acc = fmaf(__ldg(hbar + id * d + k), __ldg(W_head + (long long)k * C + c), acc);
+        for (int j = t; j < r; j += 256) acc = fmaf(pa[j], __ldg(prodW + j * C + c), acc);
+        acc = warp_sum(acc);
+        if (lane == 0) red[warp] = acc;
+        __syncthreads();
+        if (t == 0) {
+            float v = 0.f;
+#pragma unroll
+            for (int w = 0; w < 8; ++w) v += red[w];
+            lg[c] = v + b_head[c];
+        }
+        __syncthreads();
+    }
+    for (int c = t; c < C; c += 256) logits_out[(long long)b * C + c] = lg[c];
+    if (!train) return;
+    float mx = -INFINITY, se = 0.f;
+    for (int c = 0; c < C; ++c) mx = fmaxf(mx, lg[c]);
+    for (int c = 0; c < C; ++c) se += expf(lg[c] - mx);
+    const int label = labels[id];
+    if (t == 0) loss_b[b] = mx + logf(se) - lg[label];
+    __syncthreads();
+    for (int c = t; c < C; c += 256) {
+        const float g = (expf(lg[c] - mx) / se - (c == label ? 1.f : 0.f)) / (float)B;
+        lg[c] = g;
+        dlogits[(long long)b * C + c] = g;
+    }
+    __syncthreads();
+    for (int j = t; j < r; j += 256) {
+        float acc = 0.f;
+        for (int c = 0; c < C; ++c) acc = fmaf(__ldg(prodW + j * C + c), lg[c], acc);
+        daL[(long long)b * r + j] = acc / (float)S;
+    }
+}
+
 // After a cluster-wide barrier behind mid_head_products: the sum over the cluster, in rank order.  The
 // last row also takes the classifier bias, so the head needs no global load of its own later on.
 __device__ __forceinline__ void mid_sum_products(const MidParams& p, const MidShared& h, cg::cluster_group& cluster, int t, int nthr) {
@@ -618,7 +685,7 @@ struct FinalizeParams {
     ParamLayout lay;
     int B, d, r, C, L;
     const float* dw_part; int splits; long long dw_elems;     // splits <= 1: W_down gradient already in grads
-    const float* lam_part; int lam_blocks;
+    const float* lam_part; int lam_blocks;                   // null: the lambda gradients are already in grads
     const float *pooled_a, *dlogits, *loss_b;                // per-sample vectors the forward half left: mean_s a_L, dlogits, loss
     const float* hbar; const int* ids; long long N;          // token mean of the last cached layer, per cache sample; the batch's ids
     const float* params_in;                                  // the parameters the forward half used (W_up, W_head are read)
@@ -630,7 +697,7 @@ struct FinalizeParams {
     float *params, *m, *v;
     pac_adamw hp; float bc1, bc2;
     float grad_scale;                                        // factor on every gradient entering the fused update
-    bf16* wdT;                                               // [L][2][d][r] bf16 hi/lo shadow of W_down (may be null)
+    WdShadow wdT;                                            // bf16 terms of W_down (p may be null)
     // Ids of the NEXT step (pac_train_step_async): if the host has already published them in its page-locked
     // ring (tag == next_seq), block 0 copies them to device memory, off every kernel's critical path.
     const int* next_host_ids; const unsigned* next_host_tag; unsigned next_seq; int next_n;
@@ -685,11 +752,15 @@ __global__ void __launch_bounds__(256, 5) finalize_cls_kernel(FinalizeParams f) 
         const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
         if (dead && f.adam && threadIdx.x == 0) atomicAdd(&f.status[ST_SKIPPED_STEPS], 1u);
         for (int l = warp; l < f.L && !dead; l += nw) {
+            const long long i = lay.lam + l;
             float acc = 0.f;
-            for (int k = lane; k < f.lam_blocks; k += 32) acc += f.lam_part[(long long)l * f.lam_blocks + k];
-            acc = warp_sum(acc);
+            if (f.lam_part) {
+                for (int k = lane; k < f.lam_blocks; k += 32) acc += f.lam_part[(long long)l * f.lam_blocks + k];
+                acc = warp_sum(acc);
+            } else {
+                acc = f.grads[i];
+            }
             if (lane == 0) {
-                const long long i = lay.lam + l;
                 f.grads[i] = acc;
                 if (f.adam) adamw_element(f.params, f.m, f.v, i, acc * f.grad_scale, f.lay, f.hp, f.bc1, f.bc2, f.wdT, f.d, f.r);
             }

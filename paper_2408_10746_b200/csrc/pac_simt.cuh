@@ -459,7 +459,7 @@ __global__ void mean_kernel(const float* __restrict__ x, int n, float* __restric
 // ---------------------------------------------------------------------------
 // Fused AdamW over the flat parameter vector (decoupled decay on the weight matrices
 // only).  bc1 = 1-beta1^t, bc2 = 1-beta2^t (bias corrections, computed on the host in double).  Also refreshes the bf16
-// hi/lo shadow of W_down ([L][2][d][r]) that the tensor-core path multiplies with.
+// terms of W_down that the tensor-core path multiplies with.
 // ---------------------------------------------------------------------------
 // One element of the update, shared by every kernel that applies AdamW so that fused and
 // separate updates are bit-identical.
@@ -477,18 +477,16 @@ __device__ __forceinline__ float adamw_math(float th, float& mi, float& vi, floa
 
 __device__ __forceinline__ void adamw_element(float* __restrict__ p, float* __restrict__ m, float* __restrict__ v,
                                               long long i, float gi, const ParamLayout& lay, const pac_adamw& hp,
-                                              float bc1, float bc2, bf16* __restrict__ wdT, int d, int r) {
+                                              float bc1, float bc2, WdShadow wdT, int d, int r) {
     const bool decays = lay.decays(i);
     float mi = m[i], vi = v[i];
     const float th = adamw_math(p[i], mi, vi, gi, decays, hp, bc1, bc2);
     m[i] = mi;
     v[i] = vi;
     p[i] = th;
-    if (wdT && i < lay.lam) {
-        const long long dr = (long long)d * r, l = i / dr, rem = i - l * dr;
-        const bf16 hi = __float2bfloat16(th);
-        wdT[(l * 2 + 0) * dr + rem] = hi;
-        wdT[(l * 2 + 1) * dr + rem] = __float2bfloat16(th - __bfloat162float(hi));
+    if (wdT.p && i < lay.lam) {
+        const long long dr = (long long)d * r, l = i / dr;
+        wdT.put(l, dr, i - l * dr, th);
     }
 }
 
@@ -497,16 +495,16 @@ __device__ __forceinline__ void adamw_element(float* __restrict__ p, float* __re
 // The same with the old parameter and moments already in registers (a caller may fetch them early).
 __device__ __forceinline__ void adamw_w_down4_loaded(float* __restrict__ p, float* __restrict__ m, float* __restrict__ v,
                                                      long long i, float4 p4, float4 m4, float4 v4, float4 g4, const pac_adamw& hp,
-                                                     float bc1, float bc2, bf16* __restrict__ wdT, int d, int r);
+                                                     float bc1, float bc2, WdShadow wdT, int d, int r);
 __device__ __forceinline__ void adamw_w_down4(float* __restrict__ p, float* __restrict__ m, float* __restrict__ v,
                                               long long i, float4 g4, const pac_adamw& hp, float bc1, float bc2,
-                                              bf16* __restrict__ wdT, int d, int r) {
+                                              WdShadow wdT, int d, int r) {
     const float4 p4 = *reinterpret_cast<float4*>(p + i), m4 = *reinterpret_cast<float4*>(m + i), v4 = *reinterpret_cast<float4*>(v + i);
     adamw_w_down4_loaded(p, m, v, i, p4, m4, v4, g4, hp, bc1, bc2, wdT, d, r);
 }
 __device__ __forceinline__ void adamw_w_down4_loaded(float* __restrict__ p, float* __restrict__ m, float* __restrict__ v,
                                                      long long i, float4 p4, float4 m4, float4 v4, float4 g4, const pac_adamw& hp,
-                                                     float bc1, float bc2, bf16* __restrict__ wdT, int d, int r) {
+                                                     float bc1, float bc2, WdShadow wdT, int d, int r) {
     p4.x = adamw_math(p4.x, m4.x, v4.x, g4.x, true, hp, bc1, bc2);
     p4.y = adamw_math(p4.y, m4.y, v4.y, g4.y, true, hp, bc1, bc2);
     p4.z = adamw_math(p4.z, m4.z, v4.z, g4.z, true, hp, bc1, bc2);
@@ -514,17 +512,18 @@ __device__ __forceinline__ void adamw_w_down4_loaded(float* __restrict__ p, floa
     *reinterpret_cast<float4*>(p + i) = p4;
     *reinterpret_cast<float4*>(m + i) = m4;
     *reinterpret_cast<float4*>(v + i) = v4;
-    if (wdT) {
+    if (wdT.p) {
         const long long dr = (long long)d * r, l = i / dr, rem = i - l * dr;
-        const float th[4] = {p4.x, p4.y, p4.z, p4.w};
-        bf16 hi[4], lo[4];
+        float th[4] = {p4.x, p4.y, p4.z, p4.w};
+        for (int t = 0; t < wdT.terms; ++t) {
+            bf16 v[4];
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            hi[e] = __float2bfloat16(th[e]);
-            lo[e] = __float2bfloat16(th[e] - __bfloat162float(hi[e]));
+            for (int e = 0; e < 4; ++e) {
+                v[e] = __float2bfloat16(th[e]);
+                th[e] -= __bfloat162float(v[e]);
+            }
+            *reinterpret_cast<uint2*>(wdT.p + (l * wdT.terms + t) * dr + rem) = *reinterpret_cast<const uint2*>(v);
         }
-        *reinterpret_cast<uint2*>(wdT + (l * 2 + 0) * dr + rem) = *reinterpret_cast<const uint2*>(hi);
-        *reinterpret_cast<uint2*>(wdT + (l * 2 + 1) * dr + rem) = *reinterpret_cast<const uint2*>(lo);
     }
 }
 
@@ -534,7 +533,7 @@ __device__ __forceinline__ void adamw_w_down4_loaded(float* __restrict__ p, floa
 // when the gradient buffer holds the SUM over data-parallel ranks); the buffer itself is not changed.
 __global__ void adamw_kernel(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m,
                              float* __restrict__ v, long long n, ParamLayout lay, pac_adamw hp, float bc1,
-                             float bc2, bf16* __restrict__ wdT, int d, int r, int wd_blocks, unsigned* status,
+                             float bc2, WdShadow wdT, int d, int r, int wd_blocks, unsigned* status,
                              float grad_scale) {
     // gradients computed after a bounded wait ran out are not trustworthy: leave the state alone
     if (status_timed_out(status)) {
@@ -555,15 +554,12 @@ __global__ void adamw_kernel(float* __restrict__ p, const float* __restrict__ g,
     adamw_element(p, m, v, i, g[i] * grad_scale, lay, hp, bc1, bc2, wdT, d, r);
 }
 
-// bf16 hi/lo shadow of W_down from the fp32 master, same [d][r] order:
-// wdT[l][0][k][j] = bf16(W_down[l][k][j]), wdT[l][1][k][j] = bf16(W_down[l][k][j] - hi).
-__global__ void shadow_wdown_kernel(const float* __restrict__ w, bf16* __restrict__ wdT, int L, int d, int r) {
+// The bf16 terms of W_down from the fp32 master.
+__global__ void shadow_wdown_kernel(const float* __restrict__ w, WdShadow wdT, int L, int d, int r) {
     long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= (long long)L * d * r) return;
-    long long l = i / ((long long)d * r), rem = i - l * (long long)d * r;
-    const bf16 hi = __float2bfloat16(w[i]);
-    wdT[(l * 2 + 0) * (long long)d * r + rem] = hi;
-    wdT[(l * 2 + 1) * (long long)d * r + rem] = __float2bfloat16(w[i] - __bfloat162float(hi));
+    const long long dr = (long long)d * r, l = i / dr;
+    wdT.put(l, dr, i - l * dr, w[i]);
 }
 
 }  // namespace pac

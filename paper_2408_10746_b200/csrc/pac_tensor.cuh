@@ -308,7 +308,8 @@ struct FwdParams {
     int stages;
     int tmem_cols;                         // power of two >= 2 * r_pad
     int acc_stride;                        // column offset of the second accumulator
-    int wide_n;                            // 1: hi and lo blocks form one N = 128*r_blocks MMA, summed in the epilogue
+    int terms;                             // bf16 terms of W_down: 2 (hi + lo), or 3 (the fp32 value exactly)
+    int wide_n;                            // 1: the terms' blocks form one N = 64 * terms * r_blocks MMA, summed in the epilogue
     float* u; long long layer_stride;      // u[l][m][j], layer_stride = max_rows * r
     unsigned* status;
     unsigned long long* stamp;             // optional stream-phase timestamps (see stamp_begin)
@@ -319,7 +320,7 @@ struct FwdParams {
 // straight from the cache.  B tile: 64 rows of W_down^l in its natural [d][r] order (an
 // MN-major operand), split into two bf16 terms (hi = bf16(W), lo = bf16(W - hi); shadow
 // [L][2][d][r]); both products accumulate into the same fp32 accumulator, so the weights
-// enter with about 16 mantissa bits.  (With bf16-rounded weights alone the ReLU masks of about one element in a
+// enter with about 16 mantissa bits, or with a third term exactly.  (With bf16-rounded weights alone the ReLU masks of about one element in a
 // thousand flip, which alone costs ~3% relative error in dW_down and dlambda.)
 // Persistent CTAs walk tiles (layer, sample, token chunk); accumulators are double-buffered
 // in TMEM so the epilogue of one tile overlaps the loads and MMAs of the next.
@@ -331,7 +332,7 @@ down_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_cache, const __grid_c
     const int r_pad = (p.r + 7) & ~7;
     const int r_blocks = (p.r + 63) >> 6;
     const uint32_t a_bytes = FWD_ROWS * KC * 2, b_box = KC * 128;            // one [64 k][64 columns of r] box
-    const uint32_t b_bytes = (uint32_t)r_blocks * 2 * b_box;                 // [r block][hi|lo][64 k][128 B]
+    const uint32_t rb_bytes = (uint32_t)p.terms * b_box, b_bytes = (uint32_t)r_blocks * rb_bytes;      // [r block][term][64 k][128 B]
     const uint32_t b_off = a_bytes, stage_bytes = a_bytes + b_bytes;
     __shared__ __align__(8) unsigned long long bars[2 * 16 + 4];
     __shared__ uint32_t tmem_base_sh;
@@ -381,7 +382,7 @@ down_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_cache, const __grid_c
                     mbar_expect_tx(full, a_bytes + b_bytes);
                     tma_load_4d_hint(dst, &map_cache, full, kc * KC, sc * FWD_ROWS, l, id, pol);
                     for (int rb = 0; rb < r_blocks; ++rb)
-                        tma_load_4d(dst + b_off + rb * 2 * b_box, &map_w, full, rb * 64, kc * KC, 0, l);
+                        tma_load_4d(dst + b_off + rb * rb_bytes, &map_w, full, rb * 64, kc * KC, 0, l);
                 }
                 __syncwarp();
                 dst += stage_bytes;
@@ -389,14 +390,14 @@ down_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_cache, const __grid_c
             }
         }
     } else if (warp == 1) {
-        // wide_n: the hi and lo blocks lie next to each other along N ([r block][hi|lo] in 64-column
-        // blocks), so one MMA of N = 128 * r_blocks yields u_hi | u_lo side by side in TMEM
-        const uint32_t idesc = p.wide_n ? instr_desc_bf16(FWD_ROWS, 128 * r_blocks, 0, 1) : instr_desc_bf16(FWD_ROWS, r_pad, 0, 1);
+        // wide_n: the terms' blocks lie next to each other along N ([r block][term] in 64-column
+        // blocks), so one MMA of N = 64 * terms * r_blocks yields the terms' sums side by side in TMEM
+        const uint32_t idesc = p.wide_n ? instr_desc_bf16(FWD_ROWS, 64 * p.terms * r_blocks, 0, 1) : instr_desc_bf16(FWD_ROWS, r_pad, 0, 1);
         // descriptors of a stage's first 16-wide K step (start-address field in 16-byte units); later steps
         // only move the start address: +32 B per step in the K-major A tile, +2048 B (16 rows) in B
         const uint32_t ring0 = smem_u32(smem);
         const uint64_t a_desc0 = smem_desc_sw128(ring0, 16, 1024), bw_desc0 = smem_desc_sw128(ring0 + b_off, b_box, 1024);
-        const uint64_t bh_desc0 = smem_desc_sw128(ring0 + b_off, 2 * b_box, 1024), bl_desc0 = smem_desc_sw128(ring0 + b_off + b_box, 2 * b_box, 1024);
+        const uint64_t bh_desc0 = smem_desc_sw128(ring0 + b_off, rb_bytes, 1024), term_step = (uint64_t)(b_box >> 4);
         const uint64_t desc_step = (uint64_t)(stage_bytes >> 4);
         uint64_t doff = 0;
         uint32_t s = 0, ph = 0, tile_n = 0;
@@ -410,7 +411,7 @@ down_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_cache, const __grid_c
             for (int kc = 0; kc < p.k_chunks; ++kc) {
                 if (!mbar_wait_uniform(full0 + 8 * s, ph, abort_flag, p.status)) { ok = false; break; }
                 tc_fence_after();
-                const uint64_t ad0 = a_desc0 + doff, bh0 = bh_desc0 + doff, bl0 = bl_desc0 + doff;
+                const uint64_t ad0 = a_desc0 + doff, bh0 = bh_desc0 + doff;
                 if (elect_one()) {
                     if (p.wide_n) {
                         const uint64_t bw0 = bw_desc0 + doff;
@@ -421,7 +422,8 @@ down_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_cache, const __grid_c
 #pragma unroll
                         for (int k = 0; k < KC / 16; ++k) {
                             umma_bf16(d_tmem, ad0 + (uint64_t)(k * 2), bh0 + (uint64_t)(k * 128), idesc, (kc | k) ? 1u : 0u);
-                            umma_bf16(d_tmem, ad0 + (uint64_t)(k * 2), bl0 + (uint64_t)(k * 128), idesc, 1u);
+                            umma_bf16(d_tmem, ad0 + (uint64_t)(k * 2), bh0 + term_step + (uint64_t)(k * 128), idesc, 1u);
+                            if (p.terms == 3) umma_bf16(d_tmem, ad0 + (uint64_t)(k * 2), bh0 + 2 * term_step + (uint64_t)(k * 128), idesc, 1u);
                         }
                     }
                     umma_commit(empty0 + 8 * s);          // frees the smem slot once these MMAs are done
@@ -451,12 +453,19 @@ down_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_cache, const __grid_c
             for (int c0 = 0; c0 < p.r; c0 += 16) {
                 float v[16];
                 if (p.wide_n) {
-                    // column c of u: hi part at TMEM column (c/64)*128 + c%64, lo part 64 columns further
+                    // column c of u: first term at TMEM column (c/64)*64*terms + c%64, the next 64 columns further
                     float w[16];
-                    const uint32_t col = (uint32_t)((c0 >> 6) * 128 + (c0 & 63));
+                    const uint32_t col = (uint32_t)((c0 >> 6) * 64 * p.terms + (c0 & 63));
                     tmem_ld16(taddr + col, v);
                     tmem_ld16(taddr + col + 64, w);
                     tmem_ld_wait();
+                    if (p.terms == 3) {
+                        float x[16];
+                        tmem_ld16(taddr + col + 128, x);
+                        tmem_ld_wait();
+#pragma unroll
+                        for (int c = 0; c < 16; ++c) w[c] += x[c];
+                    }
 #pragma unroll
                     for (int c = 0; c < 16; ++c) v[c] += w[c];
                 } else {
@@ -490,6 +499,7 @@ struct BwdParams {
     int chunks;                            // 128-column blocks of h per CTA (accumulators in TMEM)
     int splits;                            // row splits J: partial sums per output
     int r_blocks;                          // ceil(r / 64)
+    int terms;                             // bf16 terms of du: 1, or 3 (the fp32 value exactly); term t of layer l at l * terms + t of the du map
     int stages;
     int tmem_cols;
     int early_ids;                         // 1: no kernel ahead of this one in the stream writes the ids
@@ -510,7 +520,7 @@ dw_down_tc_kernel(const __grid_constant__ CUtensorMap map_cache, const __grid_co
     unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     const int r_pad = (p.r + 15) & ~15;
     const uint32_t box_bytes = BWD_KR * 128;                       // one [64 tokens][64 columns] box
-    const uint32_t a_bytes = (uint32_t)p.chunks * 2 * box_bytes, b_bytes = (uint32_t)p.r_blocks * box_bytes;
+    const uint32_t a_bytes = (uint32_t)p.chunks * 2 * box_bytes, b_bytes = (uint32_t)(p.r_blocks * p.terms) * box_bytes;
     const uint32_t stage_bytes = a_bytes + b_bytes;
     __shared__ __align__(8) unsigned long long bars[2 * 16 + 2];
     __shared__ uint32_t tmem_base_sh;
@@ -578,16 +588,16 @@ dw_down_tc_kernel(const __grid_constant__ CUtensorMap map_cache, const __grid_co
                 // first ring: the h tiles are already on their way
                 --pre;
                 if (elect_one())
-                    for (int q = 0; q < p.r_blocks; ++q)
-                        tma_load_3d(dst + a_bytes + q * box_bytes, &map_du, full, q * 64, b * p.S + sc * BWD_KR, l);
+                    for (int q = 0; q < p.r_blocks * p.terms; ++q)
+                        tma_load_3d(dst + a_bytes + q * box_bytes, &map_du, full, (q % p.r_blocks) * 64, b * p.S + sc * BWD_KR, l * p.terms + q / p.r_blocks);
             } else {
                 if (!mbar_wait_uniform(empty0 + 8 * s, eph, abort_flag, p.status)) break;
                 if (elect_one()) {
                     mbar_expect_tx(full, stage_bytes);
                     for (int q = 0; q < 2 * p.chunks; ++q)
                         tma_load_4d_hint(dst + q * box_bytes, &map_cache, full, col0 + q * 64, sc * BWD_KR, l, id, pol);
-                    for (int q = 0; q < p.r_blocks; ++q)
-                        tma_load_3d(dst + a_bytes + q * box_bytes, &map_du, full, q * 64, b * p.S + sc * BWD_KR, l);
+                    for (int q = 0; q < p.r_blocks * p.terms; ++q)
+                        tma_load_3d(dst + a_bytes + q * box_bytes, &map_du, full, (q % p.r_blocks) * 64, b * p.S + sc * BWD_KR, l * p.terms + q / p.r_blocks);
                 }
             }
             __syncwarp();
@@ -603,7 +613,7 @@ dw_down_tc_kernel(const __grid_constant__ CUtensorMap map_cache, const __grid_co
         // descriptors of a stage's first K step (start-address field in 16-byte units)
         const uint32_t ring0 = smem_u32(smem);
         const uint64_t a_desc0 = smem_desc_sw128(ring0, box_bytes, 1024), b_desc0 = smem_desc_sw128(ring0 + a_bytes, box_bytes, 1024);
-        const uint64_t desc_step = (uint64_t)(stage_bytes >> 4), a_chunk = (uint64_t)((2 * box_bytes) >> 4);
+        const uint64_t desc_step = (uint64_t)(stage_bytes >> 4), a_chunk = (uint64_t)((2 * box_bytes) >> 4), term_step = (uint64_t)((p.r_blocks * box_bytes) >> 4);
         uint64_t doff = 0;
         uint32_t s = 0, ph = 0, first = 0;                         // first: 0 until the first K step has been issued
         bool ok = true;
@@ -616,9 +626,10 @@ dw_down_tc_kernel(const __grid_constant__ CUtensorMap map_cache, const __grid_co
                 // the result of the one before it would have to wait for that one to finish
 #pragma unroll
                 for (int k = 0; k < BWD_KR / 16; ++k)          // 16 tokens = 2048 B further along K in both operands
-                    for (int c = 0; c < p.chunks; ++c)
-                        umma_bf16(tmem_base + (uint32_t)(c * r_pad), ad0 + (uint64_t)c * a_chunk + (uint64_t)(k * 128),
-                                  bd0 + (uint64_t)(k * 128), idesc, (first | (uint32_t)k) ? 1u : 0u);
+                    for (int t = 0; t < p.terms; ++t)
+                        for (int c = 0; c < p.chunks; ++c)
+                            umma_bf16(tmem_base + (uint32_t)(c * r_pad), ad0 + (uint64_t)c * a_chunk + (uint64_t)(k * 128),
+                                      bd0 + (uint64_t)t * term_step + (uint64_t)(k * 128), idesc, (first | (uint32_t)k | (uint32_t)t) ? 1u : 0u);
                 umma_commit(empty0 + 8 * s);
             }
             __syncwarp();
@@ -753,10 +764,11 @@ inline bool make_map(CUtensorMap* map, const void* base, int rank, const cuuint6
 
 inline int pow2_at_least(int x) { int p = 32; while (p < x) p <<= 1; return p; }
 
-// wdT: [L][2][d][r] bf16 hi/lo shadow of W_down; du16: [L][max_rows][r] bf16.  *part_floats receives the
+// wdT: [L][2][d][r] bf16 hi/lo shadow of W_down; du16: [L][max_rows][r] bf16; exact: three terms of either ([L][3][d][r],
+// [L][3][max_rows][r]), whose sum is the fp32 value, so the products are those of fp32 operands.  *part_floats receives the
 // size of the split-partial buffer dW needs (0 when no split is used).
 inline pac_status tensor_plan_create(TensorPlan& tp, int device, const bf16* cache, const Dims& dm, int max_batch,
-                                     const bf16* wdT, const bf16* du16, long long* part_floats) {
+                                     const bf16* wdT, const bf16* du16, long long* part_floats, bool exact = false) {
     tp.ready = false;
     tp.dm = dm;
     tp.max_batch = max_batch;
@@ -767,6 +779,7 @@ inline pac_status tensor_plan_create(TensorPlan& tp, int device, const bf16* cac
     const int max_smem = (int)prop.sharedMemPerBlockOptin;
     const long long max_rows = (long long)max_batch * dm.S;
     const int r_pad = (dm.r + 15) & ~15;
+    const int wt = exact ? 3 : 2, dt = exact ? 3 : 1;        // bf16 terms of W_down and du
 
     // ---- tensor maps ----
     {
@@ -777,13 +790,13 @@ inline pac_status tensor_plan_create(TensorPlan& tp, int device, const bf16* cac
         if (!make_map(&tp.map_cache_bwd, cache, 4, dims, str, box_b)) return PAC_ERR_UNSUPPORTED;
     }
     {
-        cuuint64_t dims[4] = {(cuuint64_t)dm.r, (cuuint64_t)dm.d, 2, (cuuint64_t)dm.L};
-        cuuint64_t str[3] = {(cuuint64_t)dm.r * 2, (cuuint64_t)dm.r * dm.d * 2, (cuuint64_t)2 * dm.r * dm.d * 2};
-        cuuint32_t box[4] = {64, KC, 2, 1};
+        cuuint64_t dims[4] = {(cuuint64_t)dm.r, (cuuint64_t)dm.d, (cuuint64_t)wt, (cuuint64_t)dm.L};
+        cuuint64_t str[3] = {(cuuint64_t)dm.r * 2, (cuuint64_t)dm.r * dm.d * 2, (cuuint64_t)wt * dm.r * dm.d * 2};
+        cuuint32_t box[4] = {64, KC, (cuuint32_t)wt, 1};
         if (!make_map(&tp.map_w, wdT, 4, dims, str, box)) return PAC_ERR_UNSUPPORTED;
     }
     {
-        cuuint64_t dims[3] = {(cuuint64_t)dm.r, (cuuint64_t)max_rows, (cuuint64_t)dm.L};
+        cuuint64_t dims[3] = {(cuuint64_t)dm.r, (cuuint64_t)max_rows, (cuuint64_t)dm.L * dt};
         cuuint64_t str[2] = {(cuuint64_t)dm.r * 2, (cuuint64_t)max_rows * dm.r * 2};
         cuuint32_t box[3] = {KC, BWD_KR, 1};
         if (!make_map(&tp.map_du, du16, 3, dims, str, box)) return PAC_ERR_UNSUPPORTED;
@@ -794,11 +807,12 @@ inline pac_status tensor_plan_create(TensorPlan& tp, int device, const bf16* cac
     f.N = dm.N; f.L = dm.L; f.S = dm.S; f.d = dm.d; f.r = dm.r;
     f.s_chunks = (dm.S + FWD_ROWS - 1) / FWD_ROWS;
     f.k_chunks = (dm.d + KC - 1) / KC;
-    f.wide_n = dm.r <= 128 ? 1 : 0;          // N = 128 * r_blocks must stay within 256
-    f.tmem_cols = pow2_at_least(2 * (f.wide_n ? 128 * ((dm.r + 63) / 64) : r_pad));
+    f.terms = wt;
+    f.wide_n = 64 * wt * ((dm.r + 63) / 64) <= 256 ? 1 : 0;
+    f.tmem_cols = pow2_at_least(2 * (f.wide_n ? 64 * wt * ((dm.r + 63) / 64) : r_pad));
     f.acc_stride = f.tmem_cols / 2;
     {
-        const int stage = FWD_ROWS * KC * 2 + ((dm.r + 63) / 64) * 2 * KC * 128;
+        const int stage = FWD_ROWS * KC * 2 + ((dm.r + 63) / 64) * wt * KC * 128;
         int st = (max_smem - 2048) / stage;
         if (st > 16) st = 16;
         if (st < 2) { tensor_err() = "not enough shared memory for the forward pipeline"; return PAC_ERR_UNSUPPORTED; }
@@ -812,11 +826,12 @@ inline pac_status tensor_plan_create(TensorPlan& tp, int device, const bf16* cac
     b.N = dm.N; b.L = dm.L; b.S = dm.S; b.d = dm.d; b.r = dm.r;
     b.s_chunks = (dm.S + BWD_KR - 1) / BWD_KR;
     b.r_blocks = (dm.r + 63) / 64;
+    b.terms = dt;
     b.chunks = (dm.d >= 256 && 2 * r_pad <= 512) ? 2 : 1;
     b.d_groups = (dm.d + 128 * b.chunks - 1) / (128 * b.chunks);
     b.tmem_cols = pow2_at_least(b.chunks * r_pad);
     {
-        const int stage = (b.chunks * 2 + b.r_blocks) * BWD_KR * 128;
+        const int stage = (b.chunks * 2 + b.r_blocks * dt) * BWD_KR * 128;
         int st = (max_smem - 2048) / stage;
         if (st > 16) st = 16;
         if (st < 2) { tensor_err() = "not enough shared memory for the backward pipeline"; return PAC_ERR_UNSUPPORTED; }
