@@ -2157,19 +2157,24 @@ extern "C" pac_status pac_quantize_absmax(int device, void* cuda_stream, const f
     if (cudaSetDevice(device) != cudaSuccess) return PAC_ERR_CUDA;
     cudaStream_t st = (cudaStream_t)cuda_stream;
     const long long n_blocks = (n + block - 1) / block;
-    const bool vec = (n % 4 == 0) && (((uintptr_t)dev_x & 15) == 0) && (((uintptr_t)dev_q & 3) == 0);
-    if (vec && (block == 16 || block == 32 || block == 64 || block == 128)) {
-        const long long n4 = n / 4, want = (n4 + 255) / 256;
+    const bool al32 = ((uintptr_t)dev_x & 31) == 0 && ((uintptr_t)dev_q & 15) == 0, al16 = ((uintptr_t)dev_x & 15) == 0 && ((uintptr_t)dev_q & 3) == 0;
+    // widest form that the block's length and the pointers' alignment allow: 16 values per lane, a CTA per block, 4 values per lane
+    if (al32 && block >= 16 && block <= 512 && (block & (block - 1)) == 0) {
+        const long long want = ((n + 15) / 16 + 255) / 256;
         const unsigned grid = (unsigned)(want < 148LL * 32 ? want : 148LL * 32);
-        quantize_absmax_subwarp_kernel<<<grid, 256, 0, st>>>((const float4*)dev_x, n4, block / 4, (char4*)dev_q, dev_c);
-    } else if (vec && block % 1024 == 0 && block <= 4096 && n_blocks <= 0x7fffffffLL) {
-        const long long n4 = n / 4;
+        int lanes_log2 = 0;
+        while ((16 << lanes_log2) < block) ++lanes_log2;
+        quantize_absmax_subwarp_kernel<<<grid, 256, 0, st>>>(dev_x, n, lanes_log2, dev_q, dev_c);
+    } else if (al16 && block % 1024 == 0 && block <= 4096 && n_blocks <= 0x7fffffffLL) {
         switch (block / 1024) {
-            case 1: quantize_absmax_cta_reg_kernel<1><<<(unsigned)n_blocks, 256, 0, st>>>((const float4*)dev_x, n4, (char4*)dev_q, dev_c); break;
-            case 2: quantize_absmax_cta_reg_kernel<2><<<(unsigned)n_blocks, 256, 0, st>>>((const float4*)dev_x, n4, (char4*)dev_q, dev_c); break;
-            case 3: quantize_absmax_cta_reg_kernel<3><<<(unsigned)n_blocks, 256, 0, st>>>((const float4*)dev_x, n4, (char4*)dev_q, dev_c); break;
-            default: quantize_absmax_cta_reg_kernel<4><<<(unsigned)n_blocks, 256, 0, st>>>((const float4*)dev_x, n4, (char4*)dev_q, dev_c); break;
+            case 1: quantize_absmax_cta_reg_kernel<1><<<(unsigned)n_blocks, 256, 0, st>>>(dev_x, n, dev_q, dev_c); break;
+            case 2: quantize_absmax_cta_reg_kernel<2><<<(unsigned)n_blocks, 256, 0, st>>>(dev_x, n, dev_q, dev_c); break;
+            case 3: quantize_absmax_cta_reg_kernel<3><<<(unsigned)n_blocks, 256, 0, st>>>(dev_x, n, dev_q, dev_c); break;
+            default: quantize_absmax_cta_reg_kernel<4><<<(unsigned)n_blocks, 256, 0, st>>>(dev_x, n, dev_q, dev_c); break;
         }
+    } else if (al16 && block % 4 == 0 && block <= 1024) {
+        const long long warps = n_blocks < 148LL * 64 ? n_blocks : 148LL * 64;
+        quantize_absmax_warp4_kernel<<<(unsigned)((warps + 7) / 8), 256, 0, st>>>(dev_x, n, block, n_blocks, dev_q, dev_c);
     } else if (block <= QUANT_WARP_MAX) {
         const long long warps = n_blocks < 148LL * 64 ? n_blocks : 148LL * 64;      // up to 8 CTAs of 8 warps per SM
         quantize_absmax_warp_kernel<<<(unsigned)((warps + 7) / 8), 256, 0, st>>>(dev_x, n, block, n_blocks, dev_q, dev_c);
@@ -2184,10 +2189,17 @@ extern "C" pac_status pac_dequantize_absmax(int device, void* cuda_stream, const
                                             long long n, int block, float* dev_out) {
     if (!dev_q || !dev_c || !dev_out || n < 1 || block < 1) return PAC_ERR_INVALID_ARG;
     if (cudaSetDevice(device) != cudaSuccess) return PAC_ERR_CUDA;
-    if (n % 4 == 0 && block % 4 == 0 && ((uintptr_t)dev_q & 3) == 0 && ((uintptr_t)dev_out & 15) == 0) {
-        const long long n4 = n / 4, want = (n4 + 1023) / 1024;
+    if (block % 16 == 0 && ((uintptr_t)dev_q & 15) == 0 && ((uintptr_t)dev_out & 31) == 0) {
+        const int b16 = block / 16;
+        int shift = -1;
+        if ((b16 & (b16 - 1)) == 0) for (shift = 0; (1 << shift) < b16; ++shift) {}
+        const long long want = ((n + 15) / 16 + 255) / 256;
         const unsigned grid = (unsigned)(want < 148LL * 32 ? want : 148LL * 32);
-        dequantize_absmax_vec_kernel<<<grid, 256, 0, (cudaStream_t)cuda_stream>>>((const char4*)dev_q, dev_c, n4, block / 4, (float4*)dev_out);
+        dequantize_absmax_16_kernel<<<grid, 256, 0, (cudaStream_t)cuda_stream>>>(dev_q, dev_c, n, b16, shift, dev_out);
+    } else if (block % 4 == 0 && ((uintptr_t)dev_q & 3) == 0 && ((uintptr_t)dev_out & 15) == 0) {
+        const long long want = (n / 4 + 1023) / 1024;
+        const unsigned grid = (unsigned)(want < 148LL * 32 ? (want > 0 ? want : 1) : 148LL * 32);
+        dequantize_absmax_vec_kernel<<<grid, 256, 0, (cudaStream_t)cuda_stream>>>(dev_q, dev_c, n, block / 4, dev_out);
     } else {
         const long long want = (n + 255) / 256;
         const unsigned grid = (unsigned)(want < 148LL * 16 ? want : 148LL * 16);
