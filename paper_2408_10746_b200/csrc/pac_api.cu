@@ -193,7 +193,8 @@ struct pac_ctx {
     long long launches = 0;
     TensorPlan tplan{};
     MidPlan mplan{};               // fused classifier-head kernel (when the shape allows)
-    FusedFwdPlan fplan{};          // down-projections + classifier-head kernel in one launch (short sequences)
+    // down-projections + classifier-head kernel in one launch (short sequences): one geometry per useful cluster size
+    std::vector<FusedFwdPlan> fplans;
     MidPlan pplan{};               // head / reverse-chain kernel behind the chain-in-epilogue forward
     bool chain_ok = false;         // the chain-in-epilogue forward can take this shape
     int chain_pair_stages = 0;     // > 0: its CTA-pair form can too, with this many stages
@@ -868,12 +869,18 @@ pac_status tb_backward(pac_ctx* c, const int* d_ids, int B, float* d_loss, const
 
 bool use_fused_cls(const pac_ctx* c) { return c->cfg.head == PAC_HEAD_MEANPOOL_CLS && c->mplan.ok; }
 // The one-launch forward pays off when all of the batch's clusters run at the same time (its GEMM
-// and chain phases do not overlap across waves); larger batches keep the two separate kernels.
-bool use_fused_fwd(const pac_ctx* c, int B) {
-    if (!use_fused_cls(c) || !use_tensor(c) || !c->fplan.ok) return false;
-    if ((c->forward_mode == 4 || c->forward_mode == 5) && c->chain_ok) return false;
-    return c->forward_mode == 3 || B <= c->fplan.max_clusters;
+// and chain phases do not overlap across waves); larger batches keep the two separate kernels.  Among the cluster
+// sizes that fit so, the one with the fewest layers per CTA (the stream's length; then the smallest): at S = 30, B = 20,
+// L = 12 clusters of 6 instead of 2, step 56.6 -> 39.7 us.
+const FusedFwdPlan* fused_plan(const pac_ctx* c, int B) {
+    if (!use_fused_cls(c) || !use_tensor(c) || c->fplans.empty()) return nullptr;
+    if ((c->forward_mode == 4 || c->forward_mode == 5) && c->chain_ok) return nullptr;
+    const FusedFwdPlan* best = nullptr;
+    for (const FusedFwdPlan& pl : c->fplans)                       // ascending cluster size, descending layers per CTA
+        if (B <= pl.max_clusters) best = &pl;
+    return best ? best : c->forward_mode == 3 ? &c->fplans.front() : nullptr;
 }
+bool use_fused_fwd(const pac_ctx* c, int B) { return fused_plan(c, B) != nullptr; }
 // Chain-in-epilogue forward: one CTA per 128-token tile walks all layers, so it needs enough tiles to fill
 // the device (long sequences or large batches); the one-launch cluster forward keeps the short shapes.
 bool use_chain_fwd(const pac_ctx* c, int B) {
@@ -883,7 +890,7 @@ bool use_chain_fwd(const pac_ctx* c, int B) {
     return 2 * B * c->tplan.fp.s_chunks >= c->sms;
 }
 int cls_cluster_size(const pac_ctx* c, int B) {
-    return use_chain_fwd(c, B) ? c->pplan.G : use_fused_fwd(c, B) ? c->fplan.mp.G : c->mplan.G;
+    return use_chain_fwd(c, B) ? c->pplan.G : use_fused_fwd(c, B) ? fused_plan(c, B)->mp.G : c->mplan.G;
 }
 
 pac_status down_projection(pac_ctx* c, const int* d_ids, int B) {
@@ -960,7 +967,7 @@ pac_status mid_enqueue(pac_ctx* c, const int* d_ids, int B, bool train, float* d
 
 // Down-projections, chain, head, loss and reverse chain of a batch in one cluster launch.
 pac_status fused_fwd_enqueue(pac_ctx* c, const int* d_ids, int B, bool train, float* d_logits_out) {
-    const FusedFwdPlan& pl = c->fplan;
+    const FusedFwdPlan& pl = *fused_plan(c, B);
     FusedFwdParams fp{};
     fp.mid = mid_params(c, pl.mp, d_ids, B, train, d_logits_out);
     fp.mid.layers_per_cta = pl.layers_per_cta;
@@ -1352,14 +1359,18 @@ pac_status pac_adapter_init(pac_ctx* c, const pac_adapter_cfg* cfg, unsigned lon
     c->chain_blocks_max = (int)cdiv(Mr, 256);
     c->mplan = (cls && !c->tb.on) ? mid_plan(dm) : MidPlan{};
     if (c->mplan.ok && cfg->max_batch * 8 > c->chain_blocks_max) c->chain_blocks_max = cfg->max_batch * 8;     // clusters of up to 8
-    FusedFwdPlan fwd_plan{};
+    c->fplans.clear();
     if (c->mplan.ok && c->dtype == PAC_BF16 && tensor_shape_supported(dm) && !c->force_simt && c->forward_mode != 2) {
         int max_smem = 0;
         CU_OK(c, cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device));
-        fwd_plan = fused_fwd_plan(dm, max_smem);
-        if (fwd_plan.ok && cfg->max_batch * fwd_plan.mp.G > c->chain_blocks_max) c->chain_blocks_max = cfg->max_batch * fwd_plan.mp.G;
+        for (int G = 1; G <= FUSED_MAX_G; ++G) {
+            FusedFwdPlan pl = fused_fwd_plan(dm, max_smem, G);
+            if (!pl.ok || (!c->fplans.empty() && c->fplans.back().layers_per_cta == pl.layers_per_cta)) continue;
+            c->fplans.push_back(pl);
+            if (cfg->max_batch * G > c->chain_blocks_max) c->chain_blocks_max = cfg->max_batch * G;
+        }
     }
-    c->fplan = FusedFwdPlan{};
+    const bool fused_shape = !c->fplans.empty();
     Scratch& s = c->sc;
     pac_status st = PAC_OK;
     auto A = [&](pac_status x) { if (st == PAC_OK) st = x; };
@@ -1408,7 +1419,7 @@ pac_status pac_adapter_init(pac_ctx* c, const pac_adapter_cfg* cfg, unsigned lon
     }
     if (st == PAC_OK && cudaMallocHost((void**)&c->h_ids, sizeof(int) * STAGE_SLOTS * cfg->max_batch) != cudaSuccess)
         st = fail(c, PAC_ERR_NOMEM, "pinned id staging allocation failed");
-    if (st == PAC_OK && fwd_plan.ok) {
+    if (st == PAC_OK && fused_shape) {
         // id ring of pac_train_step_async (only the one-launch forward reads ids from host memory)
         if (cudaMallocHost((void**)&c->zc_ids, sizeof(int) * ZC_SLOTS * cfg->max_batch) != cudaSuccess ||
             cudaMallocHost((void**)&c->zc_tags, sizeof(unsigned) * ZC_SLOTS) != cudaSuccess ||
@@ -1457,9 +1468,13 @@ pac_status pac_adapter_init(pac_ctx* c, const pac_adapter_cfg* cfg, unsigned lon
                     }
                 }
                 c->tensor_ok = (st == PAC_OK);
-                if (c->tensor_ok && fwd_plan.ok) {
-                    fwd_plan.max_clusters = fused_fwd_max_clusters(fwd_plan, cfg->act);
-                    if (fwd_plan.max_clusters > 0) c->fplan = fwd_plan;
+                if (c->tensor_ok) {
+                    std::vector<FusedFwdPlan> fit;
+                    for (FusedFwdPlan& pl : c->fplans) {
+                        pl.max_clusters = fused_fwd_max_clusters(pl, cfg->act);
+                        if (pl.max_clusters > 0) fit.push_back(pl);
+                    }
+                    c->fplans = fit;
                 }
             } else if (ts != PAC_ERR_UNSUPPORTED) {
                 st = fail(c, ts, "tensor path set-up failed: %s", tensor_last_error());

@@ -283,8 +283,8 @@ fwd_cluster_kernel(const __grid_constant__ CUtensorMap map_cache, const __grid_c
     mid_body<ACT, bf16, 1, STATE_SMEM>(p, cluster, state, h, true, id, n_land, land_bar, abort_flag);
 }
 
-// Launch geometry: smallest cluster that gives one 4-column group per thread, at most FUSED_MAX_LPC
-// layers per CTA and fits shared memory.
+// Launch geometry for clusters of G CTAs: one 4-column group per thread, at most FUSED_MAX_LPC layers per CTA, as many
+// stages as fit shared memory.
 struct FusedFwdPlan {
     bool ok = false;
     MidPlan mp;
@@ -294,14 +294,15 @@ struct FusedFwdPlan {
     int n_land = 0;                // top layers handed over through shared memory
 };
 
-inline FusedFwdPlan fused_fwd_plan(const Dims& dm, int max_smem) {
+constexpr int FUSED_MAX_G = 16;     // clusters above 8 CTAs need the kernel's opt-in
+inline FusedFwdPlan fused_fwd_plan(const Dims& dm, int max_smem, int G) {
     FusedFwdPlan fp;
     if (dm.S > FWD_ROWS || dm.r > 64 || dm.r % 16 != 0 || dm.d % 8 != 0 || dm.d < 64 || dm.C > MID_MAX_C || dm.L > MID_MAX_L) return fp;
     const size_t stage = FWD_ROWS * KC * 2 + 2 * KC * 128;
-    for (int G = 1; G <= 8; G *= 2) {
+    {
         const int Sg = (dm.S + G - 1) / G, dg = (dm.d + G - 1) / G, lpc = (dm.L + G - 1) / G;
         const long long need = (long long)Sg * (dm.r / 4);
-        if (need > 512 || lpc > FUSED_MAX_LPC) continue;
+        if (need > 512 || lpc > FUSED_MAX_LPC) return fp;
         int th = (int)((need + 31) / 32 * 32);
         if (th < 256) th = 256;                                  // producer, MMA, prefetch and drain warps
         int scratch;
@@ -312,11 +313,11 @@ inline FusedFwdPlan fused_fwd_plan(const Dims& dm, int max_smem) {
         const size_t budget = (size_t)max_smem - 2048;
         {
             const size_t mid_bytes = floats * sizeof(float);
-            if (mid_bytes + state > budget) continue;
+            if (mid_bytes + state > budget) return fp;
             // Without a hand-over the stage ring and the chain state share one region, head vectors behind it.
             int st = (int)((budget - mid_bytes) / stage);
             if (st > 16) st = 16;
-            if (st < 3) continue;
+            if (st < 3) return fp;
             size_t region = (size_t)st * stage;
             if (region < state) region = (state + 1023) & ~(size_t)1023;
             fp.state_offset = 0;
@@ -353,7 +354,8 @@ inline FusedFwdPlan fused_fwd_plan(const Dims& dm, int max_smem) {
 // How many of the plan's clusters can be resident at once (0 when the query fails).
 template <int ACT>
 inline int fused_fwd_max_clusters_act(const FusedFwdPlan& pl) {
-    if (smem_opt_in((const void*)fwd_cluster_kernel<ACT>, pl.smem) != cudaSuccess) {
+    if (smem_opt_in((const void*)fwd_cluster_kernel<ACT>, pl.smem) != cudaSuccess ||
+        (pl.mp.G > 8 && cudaFuncSetAttribute((const void*)fwd_cluster_kernel<ACT>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)) {
         cudaGetLastError();
         return 0;
     }
