@@ -2,12 +2,11 @@
 // cache, fused into one kernel, and the gradient finalisation (+ AdamW) fused into another.
 //
 // mid_cls_kernel: one thread-block cluster per batch sample.  From the down-projections
-// u_l it runs the lambda-merge / adapter-body chain (Section IV-A) for all layers keeping
-// what the reverse pass needs (u_l - a_{l-1} in shared memory, the ReLU masks in registers), pools a_L over
+// u_l it runs the lambda-merge / adapter-body chain (Section IV-A) for all layers, pools a_L over
 // the sample's tokens through distributed shared memory, evaluates head, loss and their
-// gradients for the sample, and walks the chain backwards to emit du_l (bf16 or fp32) and
-// per-block partial sums of dlambda_l.  Nothing but u is read and nothing but du and a few
-// per-sample vectors is written.
+// gradients for the sample.  On the tensor-core path that is all: one gate byte per element and da_L
+// per sample are what the second pass over the cache builds du_l from (see MidParams).  On the plain path
+// it walks the chain backwards to emit du_l (fp32) and per-block partial sums of dlambda_l.
 //
 // All cross-thread sums use a fixed order, so results are bit-reproducible.
 #pragma once
@@ -39,8 +38,7 @@ struct MidParams {
     // memory (valid when *pref_tag == pref_seq); otherwise the ids are fetched across the host link
     const int* pref_ids; const unsigned* pref_tag; unsigned pref_seq;
     int* ids_copy;              // one-kernel forward: device copy of the batch's (clamped) ids for the later kernels, or null
-    // STATE_PARKED: what the down-projection kernel's epilogue left behind
-    const unsigned* gates;      // [max_rows][r] bit l = gate of layer l
+    // STATE_POOLED: what the down-projection kernel's epilogue left behind
     const float* pool_part;     // [B][n_pool_parts][r] token sums of a_L per token group
     int n_pool_parts;
     const float* u; long long lstride;
@@ -52,12 +50,17 @@ struct MidParams {
     float* lam_part;            // [L][B*G]
     float* logits_out;          // [B][C] (train: scratch copy; eval: caller's buffer)
     unsigned* status;
+    // What the second pass needs of the reverse chain (tensor-core path).  da_L is the same vector for every token of a sample and a
+    // gate multiplies by exactly 1 or 0, so dz_l[t][j] = cprod_l * (gates l .. L of (t, j) all open ? da_L[j] : 0) with
+    // cprod_l = prod_{l' > l} (1 - lambda_l'): one byte per element and one vector per sample describe it for all layers.
+    uint8_t* tc;                // [max_rows][r]: 1 + the highest layer whose gate is closed (0: none)
+    bf16* da16; long long da_stride;      // [2][max_batch][r]: da_L in two bf16 terms
+    float* coef;                // [L]: lambda_l cprod_l, the factor of dW_down^l
     const float* prodW;         // optional [r][C]: W_up W_head, formed once per step by head_matrix_kernel (else per CTA)
 };
 
 constexpr int MID_MAX_C = 32;
 constexpr size_t MID_SMEM_BUDGET = 220 * 1024;    // dynamic shared memory the fused kernel may use
-constexpr int MID_RING = 4;       // layers of parked state in flight per thread in the reverse pass of long sequences
 constexpr int MID_MAX_L = 32;     // ReLU masks of all layers live in one 32-bit word per element
 
 __device__ __forceinline__ void cp_async_4(void* smem_dst, const void* gsrc) {
@@ -81,14 +84,12 @@ __device__ __forceinline__ int state_swizzle(int s_local, int groups_per_tok) {
     return s_local & m;
 }
 
-// Where the per-layer chain state (u_l on the way in, u_l - a_{l-1} for the reverse pass) lives.
+// Where u_l comes from.
 enum {
     STATE_SMEM = 0,      // this CTA's shared memory, prefetched from the global u buffer with cp.async
-    STATE_DU = 1,        // u read from global memory; u_l - a_{l-1} parked, in du's type, in the du slot
-                         // that the reverse pass overwrites with du_l once it has consumed it
-    STATE_PARKED = 2     // the forward chain already ran in the down-projection kernel's epilogue: u_l - a_{l-1} is
-                         // parked in the du slots, the gates of all layers are one word per element in global
-                         // memory, and the token sums of a_L come as per-group partial sums
+    STATE_GLOBAL = 1,    // the global u buffer, a few layers in flight per thread
+    STATE_POOLED = 2     // nowhere: the forward chain ran in the down-projection kernel's epilogue, which left token sums of
+                         // a_L per token group and the gates
 };
 
 // The small per-CTA vectors of the head computation, carved from one shared-memory region.
@@ -284,8 +285,9 @@ __device__ __forceinline__ void mid_body(const MidParams& p, cg::cluster_group& 
         base[g] = ((long long)b * p.S + s) * r + j4[g];
         ts[g] = t ^ state_swizzle(s_local[g], groups_per_tok);
     }
+    constexpr bool GATES = sizeof(DU) == 2;              // tensor-core path: gates and da_L go out instead of du (see MidParams)
     DU* du = reinterpret_cast<DU*>(p.du);
-    // layer l of group g: read u, park / fetch the reverse-pass state
+    // layer l of group g: read u, keep / fetch the reverse-pass state (fp32 du only)
     auto load_u = [&](int l, int g) -> float4 {
         if constexpr (STATE == STATE_SMEM) return u_s[((size_t)l * GPT + g) * nt + ts[g]];
         else return *reinterpret_cast<const float4*>(p.u + (long long)l * p.lstride + base[g]);
@@ -293,12 +295,6 @@ __device__ __forceinline__ void mid_body(const MidParams& p, cg::cluster_group& 
     auto store_w = [&](int l, int g, const float* wv) {
         if constexpr (STATE == STATE_SMEM) {
             u_s[((size_t)l * GPT + g) * nt + ts[g]] = make_float4(wv[0], wv[1], wv[2], wv[3]);
-        } else if constexpr (sizeof(DU) == 2) {
-            __nv_bfloat162 lo = __floats2bfloat162_rn(wv[0], wv[1]), hi = __floats2bfloat162_rn(wv[2], wv[3]);
-            uint2 pk;
-            pk.x = *reinterpret_cast<unsigned*>(&lo);
-            pk.y = *reinterpret_cast<unsigned*>(&hi);
-            *reinterpret_cast<uint2*>(du + (long long)l * p.lstride + base[g]) = pk;
         } else {
             *reinterpret_cast<float4*>(du + (long long)l * p.lstride + base[g]) = make_float4(wv[0], wv[1], wv[2], wv[3]);
         }
@@ -306,11 +302,6 @@ __device__ __forceinline__ void mid_body(const MidParams& p, cg::cluster_group& 
     auto load_w = [&](int l, int g) -> float4 {
         if constexpr (STATE == STATE_SMEM) {
             return u_s[((size_t)l * GPT + g) * nt + ts[g]];
-        } else if constexpr (sizeof(DU) == 2) {
-            const uint2 pk = *reinterpret_cast<const uint2*>(du + (long long)l * p.lstride + base[g]);
-            const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&pk.x));
-            const float2 c = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&pk.y));
-            return make_float4(a.x, a.y, c.x, c.y);
         } else {
             return *reinterpret_cast<const float4*>(du + (long long)l * p.lstride + base[g]);
         }
@@ -340,23 +331,16 @@ __device__ __forceinline__ void mid_body(const MidParams& p, cg::cluster_group& 
     // masks stay in registers (bit l of mask[g][e]).  Layers are taken four at a time so that the
     // loads of a batch are in flight together; the outer loops stay rolled (every CTA runs this
     // code once, so small code beats unrolled code).
-    unsigned mask[GPT][4];
+    unsigned mask[GPT][4];                               // fp32 du: bit l = gate of layer l open; gates: 1 + highest closed layer
     float ap[GPT][4];
     bool landed = false;
     // column sums of a_L straight from registers when a warp holds whole tokens (one group per thread, 4, 8 or 16 groups per token)
-    const bool shuffle_sums = GPT == 1 && STATE != STATE_PARKED && groups_per_tok <= 32 && (32 % groups_per_tok) == 0;
+    const bool shuffle_sums = GPT == 1 && STATE != STATE_POOLED && groups_per_tok <= 32 && (32 % groups_per_tok) == 0;
 #pragma unroll
     for (int g = 0; g < GPT; ++g) {
 #pragma unroll
         for (int e = 0; e < 4; ++e) { mask[g][e] = 0u; ap[g][e] = 0.f; }      // a_0 = 0
-        if constexpr (STATE == STATE_PARKED) {
-            // the chain ran in the down-projection kernel's epilogue: only the gate words are fetched
-            if (live[g] && ACT == PAC_ACT_RELU && p.train) {
-                const uint4 gw = *reinterpret_cast<const uint4*>(p.gates + base[g]);
-                mask[g][0] = gw.x; mask[g][1] = gw.y; mask[g][2] = gw.z; mask[g][3] = gw.w;
-            }
-            continue;
-        }
+        if constexpr (STATE == STATE_POOLED) continue;       // the chain ran in the down-projection kernel's epilogue
         if (live[g]) {
 #pragma unroll 1
             for (int l0 = 0; l0 < L; l0 += 4) {
@@ -378,19 +362,22 @@ __device__ __forceinline__ void mid_body(const MidParams& p, cg::cluster_group& 
 #pragma unroll
                         for (int e = 0; e < 4; ++e) {
                             const float z = lm * uv[e] + (1.f - lm) * ap[g][e];
-                            wv[e] = uv[e] - ap[g][e];
+                            if constexpr (!GATES) wv[e] = uv[e] - ap[g][e];
                             if (ACT == PAC_ACT_RELU) {
                                 const bool on = z > 0.f;
-                                mask[g][e] |= (on ? 1u : 0u) << l;
+                                if constexpr (GATES) mask[g][e] = on ? mask[g][e] : (unsigned)(l + 1);
+                                else mask[g][e] |= (on ? 1u : 0u) << l;
                                 ap[g][e] = on ? z : 0.f;
                             } else {
                                 ap[g][e] = z;
                             }
                         }
-                        store_w(l, g, wv);
+                        if constexpr (!GATES) store_w(l, g, wv);
                     }
                 }
             }
+            if constexpr (GATES)
+                if (p.train) *reinterpret_cast<uint32_t*>(p.tc + base[g]) = mask[g][0] | (mask[g][1] << 8) | (mask[g][2] << 16) | (mask[g][3] << 24);
         }
         if (!shuffle_sums && s_local[g] < p.Sg) {
 #pragma unroll
@@ -417,7 +404,7 @@ __device__ __forceinline__ void mid_body(const MidParams& p, cg::cluster_group& 
         int parts = 1;
         if (shuffle_sums) {
             parts = nwarps;
-        } else if constexpr (STATE == STATE_PARKED) {
+        } else if constexpr (STATE == STATE_POOLED) {
             // token-group sums from the down-projection kernel; CTA q of the cluster takes groups q, q + G, ...
             if (t < r) {
                 float acc = 0.f;
@@ -481,7 +468,16 @@ __device__ __forceinline__ void mid_body(const MidParams& p, cg::cluster_group& 
             for (int j = lane; j < r; j += 32) {
                 float acc = 0.f;
                 for (int c = 0; c < C; ++c) acc = fmaf(prod[j * C + c], lg[c], acc);
-                daL[j] = acc / (float)p.S;                // da_L, the same for every token of the sample
+                const float v = acc / (float)p.S;         // da_L, the same for every token of the sample
+                if constexpr (GATES) {
+                    if (q == 0) {
+                        const bf16 hi = __float2bfloat16(v);
+                        p.da16[(long long)b * r + j] = hi;
+                        p.da16[p.da_stride + (long long)b * r + j] = __float2bfloat16(v - __bfloat162float(hi));
+                    }
+                } else {
+                    daL[j] = v;
+                }
             }
         }
     } else if (warp == 1 && q == 0 && p.train) {
@@ -490,13 +486,19 @@ __device__ __forceinline__ void mid_body(const MidParams& p, cg::cluster_group& 
             for (int g = 0; g < p.G; ++g) acc += cluster.map_shared_rank(colsum, g)[j];
             p.pooled_a[(long long)b * r + j] = acc / (float)p.S;      // mean_s a_L
         }
+    } else if (GATES && warp == 2 && blockIdx.x == 0 && p.train) {
+        for (int l = lane; l < L; l += 32) p.coef[l] = lam_s[l] * cprod[l];
     }
     // That was this CTA's last access to a peer's shared memory: say so now and wait, at the very end, only
     // for the peers to have said the same (a CTA must not exit while a peer may still read its memory).
     cluster.barrier_arrive();
+    if constexpr (GATES) {
+        cluster.barrier_wait();                           // peers may still be reading this CTA's shared memory
+        return;
+    } else {
     __syncthreads();
     if (!p.train) {
-        cluster.barrier_wait();                           // peers may still be reading this CTA's shared memory
+        cluster.barrier_wait();
         return;
     }
 
@@ -530,90 +532,9 @@ __device__ __forceinline__ void mid_body(const MidParams& p, cg::cluster_group& 
             part = fmaf(dz, wv[e], part);
             dv[e] = lm * dz;                                   // du_l
         }
-        if constexpr (sizeof(DU) == 2) {
-            __nv_bfloat162 lo = __floats2bfloat162_rn(dv[0], dv[1]), hi = __floats2bfloat162_rn(dv[2], dv[3]);
-            uint2 pk;
-            pk.x = *reinterpret_cast<unsigned*>(&lo);
-            pk.y = *reinterpret_cast<unsigned*>(&hi);
-            *reinterpret_cast<uint2*>(dst) = pk;
-        } else {
-            *reinterpret_cast<float4*>(dst) = make_float4(dv[0], dv[1], dv[2], dv[3]);
-        }
+        *reinterpret_cast<float4*>(dst) = make_float4(dv[0], dv[1], dv[2], dv[3]);
     };
-    if constexpr (STATE == STATE_PARKED) {
-        // Long sequences: the reverse pass is a pure stream over the parked state.  It is fetched through a
-        // ring of MID_RING layers in shared memory (cp.async, each thread reads back only what it requested),
-        // so that GPT * MID_RING loads per thread are in flight without holding registers.
-        uint2* ring = reinterpret_cast<uint2*>(u_s);
-        // Running pointers instead of per-layer index arithmetic: src[g] walks the parked rows MID_RING layers
-        // ahead of dst[g] (the same slots of the du buffer), slot walks the ring.
-        DU* dst[GPT];
-        const DU* src[GPT];
-#pragma unroll
-        for (int g = 0; g < GPT; ++g) { dst[g] = du + (long long)(L - 1) * p.lstride + base[g]; src[g] = dst[g]; }
-        uint2* const ring_t = ring + t;
-        const size_t slot_stride = (size_t)GPT * nt;
-        int slot = 0;                                            // ring slot of the layer consumed next
-        for (int i = 0; i < MID_RING; ++i) {
-            if (L - 1 - i >= 0) {
-#pragma unroll
-                for (int g = 0; g < GPT; ++g) {
-                    if (live[g]) cp_async_8(ring_t + (size_t)i * slot_stride + (size_t)g * nt, src[g]);
-                    src[g] -= p.lstride;
-                }
-            }
-            cp_async_commit();
-        }
-        // the launch geometry of this mode gives every group of a thread the same four columns, so the
-        // per-layer coefficients are formed once per thread and layer
-#pragma unroll 1
-        for (int l = L - 1; l >= 0; --l) {
-            cp_async_wait_group<MID_RING - 1>();
-            float part = 0.f;
-            const float cp = cprod[l], lm = lam_s[l];          // read once per layer (the stores below could alias them)
-            float dzc[4], duc[4];
-#pragma unroll
-            for (int e = 0; e < 4; ++e) { dzc[e] = daLr[0][e] * cp; duc[e] = lm * dzc[e]; }
-            uint2* const rp = ring_t + (size_t)slot * slot_stride;
-            uint2 x[GPT];
-#pragma unroll
-            for (int g = 0; g < GPT; ++g)
-                if (live[g]) x[g] = rp[(size_t)g * nt];
-#pragma unroll
-            for (int g = 0; g < GPT; ++g) {
-                if (live[g]) {
-                    const float2 a2 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&x[g].x));
-                    const float2 c2 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&x[g].y));
-                    const float wv[4] = {a2.x, a2.y, c2.x, c2.y};
-                    float dv[4];
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        const bool open = l > top_closed[g][e];
-                        part = fmaf(open ? dzc[e] : 0.f, wv[e], part);
-                        dv[e] = open ? duc[e] : 0.f;
-                    }
-                    __nv_bfloat162 lo = __floats2bfloat162_rn(dv[0], dv[1]), hi = __floats2bfloat162_rn(dv[2], dv[3]);
-                    uint2 pk;
-                    pk.x = *reinterpret_cast<unsigned*>(&lo);
-                    pk.y = *reinterpret_cast<unsigned*>(&hi);
-                    *reinterpret_cast<uint2*>(dst[g]) = pk;
-                }
-                dst[g] -= p.lstride;
-            }
-            // the slot just consumed takes the layer MID_RING further down
-            if (l - MID_RING >= 0) {
-#pragma unroll
-                for (int g = 0; g < GPT; ++g) {
-                    if (live[g]) cp_async_8(rp + (size_t)g * nt, src[g]);
-                    src[g] -= p.lstride;
-                }
-            }
-            cp_async_commit();
-            if (++slot == MID_RING) slot = 0;
-            part = warp_sum(part);
-            if (lane == 0) lred[warp * LT + l] = part;
-        }
-    } else {
+    {
         // layers per batch: about four state loads in flight per thread whatever the number of groups it owns
         constexpr int LB = GPT >= 4 ? 1 : 4 / GPT;
         DU* dstp[GPT];                                        // running pointers into du, one layer down per step
@@ -658,6 +579,7 @@ __device__ __forceinline__ void mid_body(const MidParams& p, cg::cluster_group& 
         p.lam_part[(long long)t * (p.B * p.G) + blockIdx.x] = acc;
     }
     cluster.barrier_wait();                               // keep shared memory alive until every peer has read it
+    }
 }
 
 // The stand-alone kernel: u comes from the global buffer written by the down-projection kernel.
@@ -667,10 +589,10 @@ __global__ void __launch_bounds__(512, STATE == STATE_SMEM ? 1 : 2) mid_cls_kern
     extern __shared__ float4 sm4[];
     float4* u_s = sm4;                           // [L][GPT][nt] each thread's own u values, later u_l - a_{l-1}
     float* sm = reinterpret_cast<float*>(sm4 + (STATE == STATE_SMEM ? (size_t)p.L * GPT * blockDim.x
-                                               : STATE == STATE_PARKED ? (size_t)MID_RING * GPT * blockDim.x / 2 : 0));
+                                               : 0));
     const MidShared h = mid_carve(sm, p);
     pdl_trigger();
-    pdl_wait();             // u (or the parked chain state) comes from the kernel before this one
+    pdl_wait();             // u (or the token sums) comes from the kernel before this one
     mid_body<ACT, DU, GPT, STATE>(p, cluster, u_s, h, false);
 }
 
@@ -880,7 +802,7 @@ __global__ void __launch_bounds__(256, 5) finalize_cls_kernel(FinalizeParams f) 
 struct MidPlan {
     bool ok = false;
     int G = 1, Sg = 0, dg = 0, threads = 0, scratch = 0;
-    int gpt = 1, smem_state = 1;      // 4-column groups per thread; chain state in shared memory or parked in the du buffer
+    int gpt = 1, smem_state = 1;      // 4-column groups per thread; u through shared memory, or from global memory as it is used
     int aL_floats = 0;                // a_L tile in shared memory (0: the chain ran in the down-projection kernel)
     size_t smem = 0;
 };
@@ -916,7 +838,7 @@ inline MidPlan mid_plan(const Dims& dm) {
         mp.ok = true;
         return mp;
     }
-    // otherwise: 8 CTAs per sample, up to 4 groups per thread, state parked in the du buffer
+    // otherwise: 8 CTAs per sample, up to 4 groups per thread, u read from global memory
     {
         const int G = 8, Sg = (dm.S + G - 1) / G, dg = (dm.d + G - 1) / G;
         const long long need = (long long)Sg * (dm.r / 4);
@@ -934,31 +856,16 @@ inline MidPlan mid_plan(const Dims& dm) {
     return mp;
 }
 
-// Geometry for the parked mode: the chain state never needs shared memory, so the smallest cluster with at
-// most four 4-column groups per thread serves (fewer, fuller CTAs than the plan above).
-inline MidPlan mid_plan_parked(const Dims& dm) {
+// Geometry behind a kernel that already ran the chain: only the head is left, one CTA per sample.
+inline MidPlan mid_plan_pooled(const Dims& dm) {
     MidPlan mp;
-    if (dm.r % 4 != 0 || dm.C > MID_MAX_C || dm.L > MID_MAX_L) return mp;
-    for (int G = 1; G <= 8; G *= 2) {
-        const int Sg = (dm.S + G - 1) / G, dg = (dm.d + G - 1) / G;
-        const long long need = (long long)Sg * (dm.r / 4);
-        if (need > 4 * 512) continue;
-        const int gpt = need <= 512 ? 1 : need <= 1024 ? 2 : 4;
-        // every group of a thread must land on the same four columns: threads a multiple of the groups per token
-        const int gtok = dm.r / 4;
-        int unit = 32;
-        while (unit % gtok != 0) unit += 32;                    // lcm(32, r/4)
-        int th = (int)(((need + gpt - 1) / gpt + unit - 1) / unit * unit);
-        if (th < 128) th = (128 + unit - 1) / unit * unit;
-        if (th > 512) continue;
-        int scratch;
-        const size_t floats = mid_base_floats(dm, Sg, dg, th, &scratch, false) + (size_t)MID_RING * gpt * th * 2;    // + the state ring (8 bytes per slot)
-        if (floats > 110 * 1024 / sizeof(float)) continue;                // two CTAs per SM
-        mp.G = G; mp.Sg = Sg; mp.dg = dg; mp.threads = th; mp.scratch = scratch; mp.gpt = gpt; mp.smem_state = 0;
-        mp.smem = sizeof(float) * floats;
-        mp.ok = true;
-        return mp;
-    }
+    if (dm.r % 4 != 0 || dm.r > 256 || dm.C > MID_MAX_C || dm.L > MID_MAX_L) return mp;
+    int scratch;
+    const size_t floats = mid_base_floats(dm, dm.S, dm.d, 256, &scratch, false);
+    if (floats > MID_SMEM_BUDGET / sizeof(float)) return mp;
+    mp.G = 1; mp.Sg = dm.S; mp.dg = dm.d; mp.threads = 256; mp.scratch = scratch; mp.gpt = 1; mp.smem_state = 0;
+    mp.smem = sizeof(float) * floats;
+    mp.ok = true;
     return mp;
 }
 
@@ -989,29 +896,23 @@ template <int ACT, typename DU>
 inline cudaError_t mid_launch_shape(const MidPlan& mp, const MidParams& p, cudaStream_t stream) {
     if (mp.smem_state) return mid_launch_one<ACT, DU, 1, STATE_SMEM>(mp, p, stream);
     switch (mp.gpt) {
-        case 1: return mid_launch_one<ACT, DU, 1, STATE_DU>(mp, p, stream);
-        case 2: return mid_launch_one<ACT, DU, 2, STATE_DU>(mp, p, stream);
-        default: return mid_launch_one<ACT, DU, 4, STATE_DU>(mp, p, stream);
+        case 1: return mid_launch_one<ACT, DU, 1, STATE_GLOBAL>(mp, p, stream);
+        case 2: return mid_launch_one<ACT, DU, 2, STATE_GLOBAL>(mp, p, stream);
+        default: return mid_launch_one<ACT, DU, 4, STATE_GLOBAL>(mp, p, stream);
     }
 }
 
-// The same kernel behind a down-projection kernel that already ran the forward chain (bf16 state parked in du).
-template <int ACT>
-inline cudaError_t mid_launch_parked_act(const MidPlan& mp, const MidParams& p, cudaStream_t stream) {
-    switch (mp.gpt) {
-        case 1: return mid_launch_one<ACT, bf16, 1, STATE_PARKED>(mp, p, stream);
-        case 2: return mid_launch_one<ACT, bf16, 2, STATE_PARKED>(mp, p, stream);
-        default: return mid_launch_one<ACT, bf16, 4, STATE_PARKED>(mp, p, stream);
-    }
-}
-inline cudaError_t mid_launch_parked(const MidPlan& mp, const MidParams& p, int act, cudaStream_t stream) {
-    return act == PAC_ACT_RELU ? mid_launch_parked_act<PAC_ACT_RELU>(mp, p, stream) : mid_launch_parked_act<PAC_ACT_IDENTITY>(mp, p, stream);
+// The same kernel behind a down-projection kernel that already ran the forward chain.
+inline cudaError_t mid_launch_pooled(const MidPlan& mp, const MidParams& p, int act, cudaStream_t stream) {
+    return act == PAC_ACT_RELU ? mid_launch_one<PAC_ACT_RELU, bf16, 1, STATE_POOLED>(mp, p, stream)
+                               : mid_launch_one<PAC_ACT_IDENTITY, bf16, 1, STATE_POOLED>(mp, p, stream);
 }
 
-inline cudaError_t mid_launch(const MidPlan& mp, const MidParams& p, int act, bool du_bf16, cudaStream_t stream) {
+// gates: the tensor-core path's form (see MidParams), else du in fp32.
+inline cudaError_t mid_launch(const MidPlan& mp, const MidParams& p, int act, bool gates, cudaStream_t stream) {
     if (act == PAC_ACT_RELU)
-        return du_bf16 ? mid_launch_shape<PAC_ACT_RELU, bf16>(mp, p, stream) : mid_launch_shape<PAC_ACT_RELU, float>(mp, p, stream);
-    return du_bf16 ? mid_launch_shape<PAC_ACT_IDENTITY, bf16>(mp, p, stream) : mid_launch_shape<PAC_ACT_IDENTITY, float>(mp, p, stream);
+        return gates ? mid_launch_shape<PAC_ACT_RELU, bf16>(mp, p, stream) : mid_launch_shape<PAC_ACT_RELU, float>(mp, p, stream);
+    return gates ? mid_launch_shape<PAC_ACT_IDENTITY, bf16>(mp, p, stream) : mid_launch_shape<PAC_ACT_IDENTITY, float>(mp, p, stream);
 }
 
 }  // namespace pac
