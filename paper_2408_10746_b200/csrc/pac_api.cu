@@ -37,7 +37,7 @@ struct Scratch {
     float* u = nullptr;            // [L][M][r] down-projections
     float* a = nullptr;            // [L][M][r] adapter states
     float* du = nullptr;           // [L][M][r] fp32 (plain path)
-    bf16* du16 = nullptr;          // [L][M][r] bf16 (tensor path), or three terms of du, [L][3][M][r]
+    bf16* du16 = nullptr;          // three terms of du, [L][3][M][r] (transformer bodies on a bf16 cache)
     float* lam_part = nullptr;     // [L][blocks]
     float* loss = nullptr;         // [1]
     // classifier head
@@ -63,7 +63,11 @@ struct Scratch {
     float* lm_part = nullptr;      // [slices][...] partial sums of the LM path's two skinny products (dW_up, da_L)
     float* dw_part = nullptr;      // split partials of dW_down
     float* dw_spart = nullptr;     // row-slice partials of dW_down on the plain path
-    unsigned* gates = nullptr;     // [M][r] ReLU gates of all layers, one word per element (chain-in-epilogue forward)
+    // what the second pass over the cache builds du from (tensor-core path, see MidParams)
+    uint8_t* tc = nullptr;         // [M][r] 1 + highest closed layer
+    bf16* da16 = nullptr;          // [2][max_batch][r] (classifier) or [2][M][r] (LM): da_L in two terms
+    float* coef = nullptr;         // [L] lambda_l prod_{l' > l} (1 - lambda_l')
+    float* dot_part = nullptr;     // [L][d groups][splits] shares of <D_l, W_down^l>
     float* pool_part = nullptr;    // [B][s_chunks * 4][r] token sums of a_L per 32-token group (chain-in-epilogue forward)
     float* prodW = nullptr;        // [r][C] W_up W_head of the current parameters (stand-alone head kernels)
 };
@@ -195,7 +199,7 @@ struct pac_ctx {
     MidPlan mplan{};               // fused classifier-head kernel (when the shape allows)
     // down-projections + classifier-head kernel in one launch (short sequences): one geometry per useful cluster size
     std::vector<FusedFwdPlan> fplans;
-    MidPlan pplan{};               // head / reverse-chain kernel behind the chain-in-epilogue forward
+    MidPlan pplan{};               // head kernel behind the chain-in-epilogue forward
     bool chain_ok = false;         // the chain-in-epilogue forward can take this shape
     int chain_pair_stages = 0;     // > 0: its CTA-pair form can too, with this many stages
     int forward_mode = 0;          // 0: automatic, 2: down-projections and head phase as two plain launches, 3: one-launch
@@ -416,7 +420,7 @@ pac_status adam_body_enqueue(pac_ctx* c, const pac_adamw* hp);
 // move four elements at a time; otherwise the kernels that form the d-wide vectors.
 bool plain_head_ok(const pac_ctx* c, int B) {
     const Dims& dm = c->dm;
-    return c->cfg.head == PAC_HEAD_MEANPOOL_CLS && dm.C <= MID_MAX_C && 9 * dm.r + dm.C + 32 <= 12000 && ((long long)dm.L * dm.d * dm.r) % 4 == 0 &&
+    return c->cfg.head == PAC_HEAD_MEANPOOL_CLS && dm.C <= MID_MAX_C && (!use_tensor(c) || dm.L <= MID_MAX_L) && 9 * dm.r + dm.C + 32 <= 12000 && ((long long)dm.L * dm.d * dm.r) % 4 == 0 &&
            (2LL * B + dm.r + dm.C) * FIN_KB * 4 <= 48 * 1024;
 }
 pac_status plain_head(pac_ctx* c, const int* d_ids, int B, bool train, const float* aL, float* d_logits_out) {
@@ -459,12 +463,13 @@ pac_status forward(pac_ctx* c, const int* d_ids, int B, bool train, float* d_log
     st = down_projection(c, d_ids, B);
     if (st != PAC_OK) return st;
     const float* lam = c->params + c->lay.lam;
-    if (c->cfg.act == PAC_ACT_RELU)
-        chain_fwd_kernel<PAC_ACT_RELU><<<cdiv(n, 256), 256, 0, c->stream>>>(sc.u, sc.a, lam, dm.L, n, stride);
+    float* aL = sc.a + (long long)(dm.L - 1) * stride;
+    const bool relu = c->cfg.act == PAC_ACT_RELU;
+    if (use_tensor(c))
+        (relu ? chain_gate_kernel<PAC_ACT_RELU> : chain_gate_kernel<PAC_ACT_IDENTITY>)<<<cdiv(n / 4, 256), 256, 0, c->stream>>>(sc.u, aL, sc.tc, lam, dm.L, n, stride, sc.coef);
     else
-        chain_fwd_kernel<PAC_ACT_IDENTITY><<<cdiv(n, 256), 256, 0, c->stream>>>(sc.u, sc.a, lam, dm.L, n, stride);
+        (relu ? chain_fwd_kernel<PAC_ACT_RELU> : chain_fwd_kernel<PAC_ACT_IDENTITY>)<<<cdiv(n, 256), 256, 0, c->stream>>>(sc.u, sc.a, lam, dm.L, n, stride);
     LAUNCH_CHECK(c);
-    const float* aL = sc.a + (long long)(dm.L - 1) * stride;
     const float* W_up = c->params + c->lay.w_up;
     if (c->cfg.head == PAC_HEAD_MEANPOOL_CLS) {
         if ((st = plain_head(c, d_ids, B, train, aL, d_logits_out)) != PAC_OK) return st;
@@ -632,17 +637,30 @@ pac_status backward(pac_ctx* c, const int* d_ids, int B, float* d_loss, const pa
         }
         per_sample = 0;
     }
+    if (use_tensor(c)) {
+        // the second pass builds du from the gates and da_L: per sample (classifier) or per token (LM)
+        const int nd = (per_sample ? B : M) * dm.r;
+        split_terms_kernel<<<cdiv(nd, 256), 256, 0, c->stream>>>(sc.daL, nd, (long long)(per_sample ? c->cfg.max_batch : c->max_rows) * dm.r, sc.da16);
+        LAUNCH_CHECK(c);
+        pac_status ds = dw_down(c, d_ids, B, false);
+        if (ds != PAC_OK) return ds;
+        if (plain_head_ok(c, B)) {
+            *updated = true;
+            return finalize_enqueue(c, d_ids, B, d_loss, hp);
+        }
+        const long long ne = (long long)dm.L * dm.d * dm.r;
+        const int J = tensor_splits(c->tplan, B);
+        gated_grads_kernel<<<cdiv(ne / 4, 256) + 1, 256, 0, c->stream>>>(sc.dw_part, J, ne, dm.d * dm.r, dm.L, c->params + c->lay.lam, sc.coef, sc.dot_part,
+                                                                       c->tplan.bp.d_groups * J, c->grads + c->lay.w_down, c->grads + c->lay.lam);
+        LAUNCH_CHECK(c);
+        return PAC_OK;
+    }
     const float* lam = c->params + c->lay.lam;
     const unsigned blocks = cdiv(n, 256);
-    const bool tens = use_tensor(c);
-#define CHAIN_BWD(ACT, DUT, DUP)                                                                              \
-    chain_bwd_kernel<ACT, DUT><<<blocks, 256, 0, c->stream>>>(sc.u, sc.a, lam, sc.daL, per_sample, dm.S, dm.r, \
-                                                              dm.L, n, stride, DUP, sc.lam_part)
-    if (c->cfg.act == PAC_ACT_RELU) {
-        if (tens) CHAIN_BWD(PAC_ACT_RELU, bf16, sc.du16); else CHAIN_BWD(PAC_ACT_RELU, float, sc.du);
-    } else {
-        if (tens) CHAIN_BWD(PAC_ACT_IDENTITY, bf16, sc.du16); else CHAIN_BWD(PAC_ACT_IDENTITY, float, sc.du);
-    }
+#define CHAIN_BWD(ACT)                                                                                        \
+    chain_bwd_kernel<ACT, float><<<blocks, 256, 0, c->stream>>>(sc.u, sc.a, lam, sc.daL, per_sample, dm.S, dm.r, \
+                                                                dm.L, n, stride, sc.du, sc.lam_part)
+    if (c->cfg.act == PAC_ACT_RELU) CHAIN_BWD(PAC_ACT_RELU); else CHAIN_BWD(PAC_ACT_IDENTITY);
 #undef CHAIN_BWD
     LAUNCH_CHECK(c);
     if (!plain_head_ok(c, B)) {
@@ -911,9 +929,15 @@ pac_status dw_down(pac_ctx* c, const int* d_ids, int B, bool reduce_splits) {
     pac_status st;
     time_mark(c, 2, false);
     if (use_tensor(c) || c->exact_ok) {
+        const Dims& dm = c->dm;
+        DuGen gen{};
+        const bool lm = c->cfg.head == PAC_HEAD_FROZEN_LM;
+        gen.tc = c->sc.tc; gen.da = c->sc.da16; gen.da_term = (long long)(lm ? c->max_rows : c->cfg.max_batch) * dm.r;
+        gen.da_sample = lm ? (long long)dm.S * dm.r : dm.r; gen.da_token = lm ? dm.r : 0;
+        gen.w = c->params + c->lay.w_down; gen.dot_part = c->sc.dot_part;
         st = tensor_dw_down(c->tplan, c->stream, d_ids, B, c->sc.du16, c->grads + c->lay.w_down, c->sc.dw_part,
                             reduce_splits, c->status, &c->launches, next_stamp(c, 1),
-                            c->step_early_ids && !c->step_host_ids);       // ids no kernel in flight writes
+                            c->step_early_ids && !c->step_host_ids, &gen);       // ids no kernel in flight writes
         if (st != PAC_OK) return fail(c, st, "tensor-core dW_down launch failed: %s", tensor_last_error());
     } else {
         st = c->dtype == PAC_F32 ? dw_down_simt<float>(c, d_ids, B, reduce_splits) : dw_down_simt<bf16>(c, d_ids, B, reduce_splits);
@@ -934,7 +958,8 @@ MidParams mid_params(pac_ctx* c, const MidPlan& mp, const int* d_ids, int B, boo
     p.u = sc.u; p.lstride = (long long)c->max_rows * dm.r;
     p.lam = c->params + c->lay.lam; p.W_up = c->params + c->lay.w_up;
     p.W_head = c->params + c->lay.w_head; p.b_head = c->params + c->lay.b_head; p.hbar = sc.hbar;
-    p.du = use_tensor(c) ? (void*)sc.du16 : (void*)sc.du;
+    p.du = sc.du;
+    p.tc = sc.tc; p.da16 = sc.da16; p.da_stride = (long long)c->cfg.max_batch * dm.r; p.coef = sc.coef;
     p.pooled_a = sc.pooled_a; p.dlogits = sc.dlogits;
     p.loss_b = sc.loss_b; p.lam_part = sc.lam_part; p.logits_out = train ? sc.logits : d_logits_out;
     p.status = c->status;
@@ -987,7 +1012,7 @@ pac_status fused_fwd_enqueue(pac_ctx* c, const int* d_ids, int B, bool train, fl
     return PAC_OK;
 }
 
-// Down-projections with the chain in their epilogue, then head / loss / reverse chain from the parked state.
+// Down-projections with the chain in their epilogue, then head and loss from its token sums.
 pac_status chain_fwd_enqueue(pac_ctx* c, const int* d_ids, int B, bool train, float* d_logits_out) {
     const Dims& dm = c->dm;
     ChainFwdParams cp{};
@@ -995,8 +1020,7 @@ pac_status chain_fwd_enqueue(pac_ctx* c, const int* d_ids, int B, bool train, fl
     cp.s_chunks = c->tplan.fp.s_chunks; cp.k_chunks = c->tplan.fp.k_chunks; cp.stages = c->tplan.fp.stages;
     cp.train = train ? 1 : 0;
     cp.lam = c->params + c->lay.lam;
-    cp.parked = c->sc.du16; cp.layer_stride = (long long)c->max_rows * dm.r;
-    cp.gates = c->sc.gates; cp.pool_part = c->sc.pool_part;
+    cp.tc = c->sc.tc; cp.pool_part = c->sc.pool_part;
     cp.status = c->status; cp.stamp = next_stamp(c, 0);
     pac_status hs = head_matrix_enqueue(c);
     if (hs != PAC_OK) return hs;
@@ -1009,10 +1033,10 @@ pac_status chain_fwd_enqueue(pac_ctx* c, const int* d_ids, int B, bool train, fl
     time_mark(c, 0, true);
     if (e != cudaSuccess) return fail(c, PAC_ERR_CUDA, "chain-in-epilogue forward launch failed: %s", cudaGetErrorString(e));
     MidParams p = mid_params(c, c->pplan, d_ids, B, train, d_logits_out);
-    p.gates = c->sc.gates; p.pool_part = c->sc.pool_part; p.n_pool_parts = cp.s_chunks * CF_POOL_PARTS;
+    p.pool_part = c->sc.pool_part; p.n_pool_parts = cp.s_chunks * CF_POOL_PARTS;
     p.prodW = c->sc.prodW;
     time_mark(c, 1, false);
-    e = mid_launch_parked(c->pplan, p, c->cfg.act, c->stream);
+    e = mid_launch_pooled(c->pplan, p, c->cfg.act, c->stream);
     c->launches++;
     time_mark(c, 1, true);
     if (e != cudaSuccess) return fail(c, PAC_ERR_CUDA, "head kernel launch failed: %s", cudaGetErrorString(e));
@@ -1050,6 +1074,8 @@ pac_status finalize_enqueue(pac_ctx* c, const int* d_ids, int B, float* d_loss, 
     const bool tens = use_tensor(c) || c->exact_ok;
     f.dw_part = tens ? sc.dw_part : sc.dw_spart;
     f.splits = tens ? tensor_splits(c->tplan, B) : dw_simt_slices(c, B);
+    if (use_tensor(c)) { f.coef = sc.coef; f.dot_part = sc.dot_part; f.dot_n = c->tplan.bp.d_groups * f.splits; }
+    else if (f.splits <= 1) f.splits = 0;                // already in the gradient buffer
     f.dw_elems = (long long)dm.L * dm.d * dm.r;
     // per-CTA partial sums of dlambda: the fused head kernels', or the plain reverse chain's; transformer bodies: done
     f.lam_part = c->tb.on ? nullptr : sc.lam_part;
@@ -1157,7 +1183,7 @@ void free_all(pac_ctx* c) {
     Scratch& s = c->sc;
     if (c->hc.on) s.hbar = nullptr;            // points into a staging slot, freed below
     void* ptrs[] = {s.ids, s.u, s.a, s.du, s.du16, s.lam_part, s.loss, s.hbar, s.pooled_a, s.pooled_y, s.logits,
-                    s.dlogits, s.loss_b, s.gvec, s.daL, s.y, s.lm_logits, s.dy, s.y16, s.dlog16, s.aL16, s.wup16, s.dy16, s.wdT, s.lm_part, s.dw_part, s.dw_spart, s.gates, s.pool_part, s.prodW, c->tb.buf, c->params, c->grads,
+                    s.dlogits, s.loss_b, s.gvec, s.daL, s.y, s.lm_logits, s.dy, s.y16, s.dlog16, s.aL16, s.wup16, s.dy16, s.wdT, s.lm_part, s.dw_part, s.dw_spart, s.tc, s.da16, s.coef, s.dot_part, s.pool_part, s.prodW, c->tb.buf, c->params, c->grads,
                     c->m, c->v, c->status, c->d_perm, c->d_losses, c->d_stamps};
     for (void* p : ptrs)
         if (p) cudaFree(p);
@@ -1439,24 +1465,25 @@ pac_status pac_adapter_init(pac_ctx* c, const pac_adapter_cfg* cfg, unsigned lon
     c->tensor_ok = false;
     if (st == PAC_OK && c->dtype == PAC_BF16 && tensor_shape_supported(dm) && !c->tb.on) {
         A(dmalloc(c, &s.wdT, (long long)dm.L * 2 * dm.r * dm.d));
-        A(dmalloc(c, &s.du16, Mr * dm.L));
+        A(dmalloc(c, &s.tc, Mr)); A(dmalloc(c, &s.coef, dm.L));
+        A(dmalloc(c, &s.da16, 2LL * (cls ? (long long)cfg->max_batch * dm.r : Mr)));
         long long part_floats = 0;
         if (st == PAC_OK) {
             pac_status ts = tensor_plan_create(c->tplan, c->device, (const bf16*)c->cache, dm, cfg->max_batch, s.wdT,
-                                               s.du16, &part_floats);
+                                               nullptr, &part_floats, false, !cls);
             if (ts == PAC_OK && c->hc.on) {
                 // one set of tensor maps per staging slot
                 c->hc.tplan[0] = c->tplan;
                 long long pf2 = 0;
-                ts = tensor_plan_create(c->hc.tplan[1], c->device, (const bf16*)c->hc.stage[1], dm, cfg->max_batch, s.wdT, s.du16, &pf2);
+                ts = tensor_plan_create(c->hc.tplan[1], c->device, (const bf16*)c->hc.stage[1], dm, cfg->max_batch, s.wdT, nullptr, &pf2, false, !cls);
             }
             if (ts == PAC_OK) {
                 A(dmalloc(c, &s.dw_part, part_floats));
+                A(dmalloc(c, &s.dot_part, (long long)dm.L * c->tplan.bp.d_groups * c->tplan.bp.splits));
                 c->chain_ok = false;
                 if (st == PAC_OK && cls && c->mplan.ok && chain_fwd_supported(dm) && c->tplan.fp.wide_n) {
-                    c->pplan = mid_plan_parked(dm);
+                    c->pplan = mid_plan_pooled(dm);
                     if (c->pplan.ok) {
-                        A(dmalloc(c, &s.gates, Mr));
                         A(dmalloc(c, &s.pool_part, (long long)cfg->max_batch * c->tplan.fp.s_chunks * CF_POOL_PARTS * dm.r));
                         c->chain_ok = (st == PAC_OK);
                         int max_smem = 0;

@@ -606,7 +606,10 @@ __global__ void __launch_bounds__(512, STATE == STATE_SMEM ? 1 : 2) mid_cls_kern
 struct FinalizeParams {
     ParamLayout lay;
     int B, d, r, C, L;
-    const float* dw_part; int splits; long long dw_elems;     // splits <= 1: W_down gradient already in grads
+    const float* dw_part; int splits; long long dw_elems;     // splits < 1: W_down gradient already in grads
+    // Tensor-core path: dw_part holds D_l = h_l^T (open_l daL) (see MidParams), dW_down^l = coef[l] D_l, and dot_part the shares of
+    // P_l = <D_l, W_down^l>, dot_n per layer, which are all that dlambda needs (see lambda_grad).
+    const float* coef; const float* dot_part; int dot_n;
     const float* lam_part; int lam_blocks;                   // null: the lambda gradients are already in grads
     const float *pooled_a, *dlogits, *loss_b;                // per-sample vectors the forward half left: mean_s a_L, dlogits, loss
     const float* hbar; const int* ids; long long N;          // token mean of the last cached layer, per cache sample; the batch's ids
@@ -642,6 +645,52 @@ __device__ __forceinline__ unsigned ld_acquire_gpu(const unsigned* p) {
     return v;
 }
 
+// dlambda_l = sum dz_l (u_l - a_{l-1}) without u or a.  With dz_l = cprod_l open_l daL and u_l = h_l W_l the first half is cprod_l P_l,
+// P_l = <D_l, W_l>; and where gates l .. L are open, a_{l-1} = sum over i < l with gates i .. l-1 open of
+// lambda_i prod_{i < l' < l} (1 - lambda_l') u_i, so the second half is sum_{i<l} lambda_i (prod_{l' > i, l' != l} (1 - lambda_l')) P_i.
+__device__ __forceinline__ float lambda_grad(const float* lam, const float* P, int L, int l) {
+    float e = 1.f;
+    for (int k = L - 1; k > l; --k) e *= 1.f - lam[k];
+    float g = e * P[l];
+    for (int i = l - 1; i >= 0; --i) {
+        g -= lam[i] * e * P[i];
+        e *= 1.f - lam[i];
+    }
+    return g;
+}
+// The gradients of W_down (four elements per thread) and lambda (last block) from the second pass's partial sums where no
+// finalisation kernel follows (L <= 128).
+__global__ void __launch_bounds__(256) gated_grads_kernel(const float* __restrict__ part, int splits, long long n, int dr, int L, const float* __restrict__ lam,
+                                                          const float* __restrict__ coef, const float* __restrict__ dot_part, int dot_n,
+                                                          float* __restrict__ gW, float* __restrict__ glam) {
+    if (blockIdx.x + 1 == gridDim.x) {
+        __shared__ float lam_s[128], dot_s[128];
+        for (int l = threadIdx.x; l < L; l += 256) {
+            lam_s[l] = lam[l];
+            float acc = 0.f;
+            for (int k = 0; k < dot_n; ++k) acc += dot_part[(long long)l * dot_n + k];
+            dot_s[l] = acc;
+        }
+        __syncthreads();
+        for (int l = threadIdx.x; l < L; l += 256) glam[l] = lambda_grad(lam_s, dot_s, L, l);
+        return;
+    }
+    const long long i = ((long long)blockIdx.x * 256 + threadIdx.x) * 4;
+    if (i >= n) return;
+    float4 a = *reinterpret_cast<const float4*>(part + i);
+    for (int s = 1; s < splits; ++s) {
+        const float4 v = *reinterpret_cast<const float4*>(part + s * n + i);
+        a.x += v.x; a.y += v.y; a.z += v.z; a.w += v.w;
+    }
+    const float c = coef[i / dr];
+    *reinterpret_cast<float4*>(gW + i) = make_float4(a.x * c, a.y * c, a.z * c, a.w * c);
+}
+__device__ __forceinline__ void lambda_update(const FinalizeParams& f, int l, float g) {
+    const long long i = f.lay.lam + l;
+    f.grads[i] = g;
+    if (f.adam) adamw_element(f.params, f.m, f.v, i, g * f.grad_scale, f.lay, f.hp, f.bc1, f.bc2, f.wdT, f.d, f.r);
+}
+
 // (five blocks per SM: 48 registers, no spills; T5-Base step 51.0 -> 50.3 us against the 63 registers of an open bound)
 __global__ void __launch_bounds__(256, 5) finalize_cls_kernel(FinalizeParams f) {
     pdl_trigger();
@@ -661,32 +710,15 @@ __global__ void __launch_bounds__(256, 5) finalize_cls_kernel(FinalizeParams f) 
         m4 = *reinterpret_cast<const float4*>(f.m + i_wd);
         v4 = *reinterpret_cast<const float4*>(f.v + i_wd);
     }
-    // Block 0 (dlambda and the mean loss) needs only what the forward half left behind, which is
-    // complete whenever this kernel runs (see above): it does not wait for the second pass at all, so a loss
-    // that goes straight to host memory is on its way long before the step ends.
+    // Block 0: the mean loss needs only what the forward half left behind, which is complete whenever this kernel runs
+    // (see above), so a loss that goes straight to host memory is on its way long before the step ends; dlambda comes last.
     // Set by a wait that ran out in this step's forward half or in any earlier step since the last
     // pac_sync (the forward half has completed whenever this kernel runs); a wait that runs out in this
     // step's second pass is seen by the W_down blocks behind their own wait below.
     const bool dead = status_timed_out(f.status);
     if (blk < 0) {
-        // dlambda_l (one warp per layer, lanes over the per-block partials, fixed
-        // shuffle order) and the mean loss
         const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
         if (dead && f.adam && threadIdx.x == 0) atomicAdd(&f.status[ST_SKIPPED_STEPS], 1u);
-        for (int l = warp; l < f.L && !dead; l += nw) {
-            const long long i = lay.lam + l;
-            float acc = 0.f;
-            if (f.lam_part) {
-                for (int k = lane; k < f.lam_blocks; k += 32) acc += f.lam_part[(long long)l * f.lam_blocks + k];
-                acc = warp_sum(acc);
-            } else {
-                acc = f.grads[i];
-            }
-            if (lane == 0) {
-                f.grads[i] = acc;
-                if (f.adam) adamw_element(f.params, f.m, f.v, i, acc * f.grad_scale, f.lay, f.hp, f.bc1, f.bc2, f.wdT, f.d, f.r);
-            }
-        }
         if (warp == nw - 1) {
             float acc = 0.f;
             for (int b = lane; b < f.B; b += 32) acc += f.loss_b[b];
@@ -706,6 +738,28 @@ __global__ void __launch_bounds__(256, 5) finalize_cls_kernel(FinalizeParams f) 
                     atomicExch(f.next_dev_tag, f.next_seq);
                 }
             }
+        }
+        // dlambda: warp per layer, lanes over its partial sums, fixed shuffle order
+        __shared__ float lam_s[MID_MAX_L], dot_s[MID_MAX_L];
+        const bool dots = f.dot_part != nullptr;
+        if (dots && threadIdx.x < f.L) lam_s[threadIdx.x] = f.params_in[lay.lam + threadIdx.x];
+        if (dots) pdl_wait();                            // the partial sums of P_l come from the second pass
+        const float* parts = dots ? f.dot_part : f.lam_part;
+        const int np = dots ? f.dot_n : f.lam_blocks;
+        for (int l = warp; l < f.L; l += nw) {
+            float acc = 0.f;
+            if (parts) {
+                for (int k = lane; k < np; k += 32) acc += parts[(long long)l * np + k];
+                acc = warp_sum(acc);
+            } else {
+                acc = f.grads[lay.lam + l];
+            }
+            if (lane == 0 && dots) dot_s[l] = acc;
+            if (lane == 0 && !dots && !dead) lambda_update(f, l, acc);
+        }
+        if (dots) {
+            __syncthreads();
+            if (threadIdx.x < f.L && !status_timed_out(f.status)) lambda_update(f, threadIdx.x, lambda_grad(lam_s, dot_s, f.L, threadIdx.x));
         }
         return;
     }
@@ -779,11 +833,15 @@ __global__ void __launch_bounds__(256, 5) finalize_cls_kernel(FinalizeParams f) 
         const long long i = i_wd;
         if (i >= lay.lam || status_timed_out(f.status)) return;
         float4 g4;
-        if (f.splits > 1) {
+        if (f.splits >= 1) {
             g4 = *reinterpret_cast<const float4*>(f.dw_part + i);
             for (int j = 1; j < f.splits; ++j) {                 // split order
                 const float4 q = *reinterpret_cast<const float4*>(f.dw_part + (long long)j * f.dw_elems + i);
                 g4.x += q.x; g4.y += q.y; g4.z += q.z; g4.w += q.w;
+            }
+            if (f.coef) {
+                const float c = f.coef[(int)(i / ((long long)f.d * f.r))];
+                g4.x *= c; g4.y *= c; g4.z *= c; g4.w *= c;
             }
             *reinterpret_cast<float4*>(f.grads + i) = g4;
         } else {
