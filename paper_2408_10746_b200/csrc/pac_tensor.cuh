@@ -116,6 +116,12 @@ __device__ __forceinline__ bool mbar_wait_uniform(uint32_t bar, uint32_t parity,
     const bool ok = mbar_wait(bar, parity, abort_flag, status);
     return __all_sync(0xffffffffu, ok) != 0;
 }
+// Bytes of x by selector; a selector nibble of 8 + k gives eight copies of byte k's top bit.
+__device__ __forceinline__ uint32_t spread_sign(uint32_t x, uint32_t sel) {
+    uint32_t d;
+    asm("prmt.b32 %0, %1, %1, %2;" : "=r"(d) : "r"(x), "r"(sel));
+    return d;
+}
 // True in exactly one lane of a converged warp.
 __device__ __forceinline__ bool elect_one() {
     uint32_t pred;
@@ -296,6 +302,7 @@ __host__ __device__ constexpr uint32_t instr_desc_bf16(int M, int N, int a_mn_ma
 
 constexpr int TC_THREADS = 192;            // warp 0: TMA producer, warp 1: MMA issuer, warps 2-5: epilogue
 constexpr int DW_THREADS = 320;            // dW_down: two epilogue warps per TMEM lane quadrant (warps 2-9)
+constexpr int DW_GEN_WARPS = 8;            // the same warps while they build du tiles
 constexpr int KC = 64;                     // bf16 elements per 128-byte swizzled row
 constexpr int FWD_ROWS = 128;              // token rows per forward tile (MMA M)
 constexpr int BWD_KR = 64;                 // token rows per backward stage (MMA K extent per stage)
@@ -503,7 +510,14 @@ struct BwdParams {
     int stages;
     int tmem_cols;
     int early_ids;                         // 1: no kernel ahead of this one in the stream writes the ids
-    float* out;                            // splits == 1: dW_down [L][d][r]; else partials [J][L][d][r]
+    // gen: du_l is not read but built in shared memory from one byte per element (see MidParams in pac_mid.cuh) and da_L, one vector per
+    // sample or token, in one or two bf16 terms: B = open_l ? da : 0, out = h_l^T B without the layer's factor.
+    int gen;
+    const uint8_t* tc;                     // [max_rows][r]
+    const bf16* da; long long da_term, da_sample; int da_token;      // strides in elements
+    const float* w;                        // fp32 W_down [L][d][r] for
+    float* dot_part;                       // [L][d_groups][J]: this CTA's share of <out, W_down^l>
+    float* out;                            // splits == 1 and not gen: dW_down [L][d][r]; else partials [J][L][d][r]
     unsigned* status;
     unsigned long long* stamp;             // optional stream-phase timestamps (see stamp_begin)
 };
@@ -513,15 +527,24 @@ struct BwdParams {
 // it streams 64-token tiles of h_l (MN-major A: the 128 output rows are h's columns) and of
 // du_l (MN-major B: N = r), accumulates [128 x r] blocks in TMEM over all its rows and writes
 // them once.  With splits > 1 the partial sums are added afterwards in split order.
+// Generated du: warps 2 - 9, idle until the accumulators are complete, fill the B part of every stage.  That takes the
+// L * M * r * 2 bytes of du out of memory in both directions; the tile costs five integer instructions per four elements.
+// GQ: 16-column groups of a generated tile per thread (r = 64 GQ at most; 0: du comes through TMA), GT: its terms.  Registers are
+// bounded so that three finalisation blocks fit beside a CTA (r <= 64; with 155 instead of 88 the step took 58 us for 53).
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(DW_THREADS, 1)
+template <int GQ, int GT>
+__global__ void __launch_bounds__(DW_THREADS) __maxnreg__(GQ <= 1 ? 88 : 168)
 dw_down_tc_kernel(const __grid_constant__ CUtensorMap map_cache, const __grid_constant__ CUtensorMap map_du, BwdParams p) {
+    constexpr bool GEN = GQ > 0;
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     const int r_pad = (p.r + 15) & ~15;
     const uint32_t box_bytes = BWD_KR * 128;                       // one [64 tokens][64 columns] box
-    const uint32_t a_bytes = (uint32_t)p.chunks * 2 * box_bytes, b_bytes = (uint32_t)(p.r_blocks * p.terms) * box_bytes;
-    const uint32_t stage_bytes = a_bytes + b_bytes;
+    const uint32_t a_bytes = (uint32_t)p.chunks * 2 * box_bytes, b_bytes = (uint32_t)(p.r_blocks * (GEN ? GT : p.terms)) * box_bytes;
+    const uint32_t stage_bytes = a_bytes + b_bytes, tx_bytes = GEN ? a_bytes : stage_bytes;
+    constexpr bool side = GT == 2 && GQ <= 2;                      // the terms side by side along N, added up in the epilogue
+    const int n_cols = side ? 128 * p.r_blocks : r_pad;            // TMEM columns per accumulator
+    __shared__ float dot_s[DW_GEN_WARPS];
     __shared__ __align__(8) unsigned long long bars[2 * 16 + 2];
     __shared__ uint32_t tmem_base_sh;
     __shared__ int abort_sh;
@@ -538,11 +561,11 @@ dw_down_tc_kernel(const __grid_constant__ CUtensorMap map_cache, const __grid_co
 
     if (threadIdx.x == 0) {
         abort_sh = 0;
-        for (int s = 0; s < p.stages; ++s) { mbar_init(full0 + 8 * s, 1); mbar_init(empty0 + 8 * s, 1); }
+        for (int s = 0; s < p.stages; ++s) { mbar_init(full0 + 8 * s, GEN ? 1 + DW_GEN_WARPS : 1); mbar_init(empty0 + 8 * s, 1); }
         mbar_init(accf, 1);
         fence_mbar_init();
         tma_prefetch_desc(&map_cache);
-        tma_prefetch_desc(&map_du);
+        if (!GEN) tma_prefetch_desc(&map_du);
     }
     if (warp == 1) { tmem_alloc(smem_u32(&tmem_base_sh), (uint32_t)p.tmem_cols); tmem_relinquish(); }
     tc_fence_before();
@@ -561,7 +584,7 @@ dw_down_tc_kernel(const __grid_constant__ CUtensorMap map_cache, const __grid_co
                 const int rt = rt0 + (int)i, sc = rt % p.s_chunks, b = rt / p.s_chunks;
                 const int id = (int)safe_id(p.ids, b, p.N, nullptr);
                 const uint32_t dst = smem_u32(smem + (size_t)i * stage_bytes);
-                mbar_expect_tx(full0 + 8 * i, stage_bytes);
+                mbar_expect_tx(full0 + 8 * i, tx_bytes);
                 for (int q = 0; q < 2 * p.chunks; ++q)
                     tma_load_4d_hint(dst + q * box_bytes, &map_cache, full0 + 8 * i, col0 + q * 64, sc * BWD_KR, l, id, pol);
             }
@@ -587,16 +610,16 @@ dw_down_tc_kernel(const __grid_constant__ CUtensorMap map_cache, const __grid_co
             if (pre > 0) {
                 // first ring: the h tiles are already on their way
                 --pre;
-                if (elect_one())
+                if (!GEN && elect_one())
                     for (int q = 0; q < p.r_blocks * p.terms; ++q)
                         tma_load_3d(dst + a_bytes + q * box_bytes, &map_du, full, (q % p.r_blocks) * 64, b * p.S + sc * BWD_KR, l * p.terms + q / p.r_blocks);
             } else {
                 if (!mbar_wait_uniform(empty0 + 8 * s, eph, abort_flag, p.status)) break;
                 if (elect_one()) {
-                    mbar_expect_tx(full, stage_bytes);
+                    mbar_expect_tx(full, tx_bytes);
                     for (int q = 0; q < 2 * p.chunks; ++q)
                         tma_load_4d_hint(dst + q * box_bytes, &map_cache, full, col0 + q * 64, sc * BWD_KR, l, id, pol);
-                    for (int q = 0; q < p.r_blocks * p.terms; ++q)
+                    for (int q = 0; q < p.r_blocks * p.terms && !GEN; ++q)
                         tma_load_3d(dst + a_bytes + q * box_bytes, &map_du, full, (q % p.r_blocks) * 64, b * p.S + sc * BWD_KR, l * p.terms + q / p.r_blocks);
                 }
             }
@@ -609,7 +632,8 @@ dw_down_tc_kernel(const __grid_constant__ CUtensorMap map_cache, const __grid_co
             }
         }
     } else if (warp == 1) {
-        const uint32_t idesc = instr_desc_bf16(128, r_pad, 1, 1);
+        const uint32_t idesc = instr_desc_bf16(128, n_cols, 1, 1);
+        const int passes = side ? 1 : GEN ? GT : p.terms;          // products per K step and column block
         // descriptors of a stage's first K step (start-address field in 16-byte units)
         const uint32_t ring0 = smem_u32(smem);
         const uint64_t a_desc0 = smem_desc_sw128(ring0, box_bytes, 1024), b_desc0 = smem_desc_sw128(ring0 + a_bytes, box_bytes, 1024);
@@ -626,9 +650,9 @@ dw_down_tc_kernel(const __grid_constant__ CUtensorMap map_cache, const __grid_co
                 // the result of the one before it would have to wait for that one to finish
 #pragma unroll
                 for (int k = 0; k < BWD_KR / 16; ++k)          // 16 tokens = 2048 B further along K in both operands
-                    for (int t = 0; t < p.terms; ++t)
+                    for (int t = 0; t < passes; ++t)
                         for (int c = 0; c < p.chunks; ++c)
-                            umma_bf16(tmem_base + (uint32_t)(c * r_pad), ad0 + (uint64_t)c * a_chunk + (uint64_t)(k * 128),
+                            umma_bf16(tmem_base + (uint32_t)(c * n_cols), ad0 + (uint64_t)c * a_chunk + (uint64_t)(k * 128),
                                       bd0 + (uint64_t)t * term_step + (uint64_t)(k * 128), idesc, (first | (uint32_t)k | (uint32_t)t) ? 1u : 0u);
                 umma_commit(empty0 + 8 * s);
             }
@@ -643,36 +667,136 @@ dw_down_tc_kernel(const __grid_constant__ CUtensorMap map_cache, const __grid_co
         }
     } else {
         const int q = warp & 3;                                   // TMEM lane quadrant this warp may read
-        const int ne = ((int)(blockDim.x >> 5) - 2) >> 2, e16 = ((warp - 2) >> 2) * 16;      // warps per quadrant; this warp's first 16 columns
-        if (rt1 > rt0) {
-            if (mbar_wait_warp(accf, 0, abort_flag, p.status)) {
-                tc_fence_after();
-                if (threadIdx.x == 64) stamp_end(p.stamp);
-                for (int c = 0; c < p.chunks; ++c) {
-                    const int k = col0 + c * 128 + q * 32 + lane;             // column of h = row of dW_down
-                    float* dst = p.out + (((long long)j * p.L + l) * p.d + k) * p.r;
-                    const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(c * r_pad);
-                    for (int c0 = e16; c0 < p.r; c0 += 16 * ne) {              // the quadrant's warps share its columns
-                        float v[16];
-                        tmem_ld16(taddr + c0, v);
-                        tmem_ld_wait();
-                        if (k < p.d) {
-                            // (16-byte stores: with 32-byte ones here the step measured 0.4 us slower)
+        const int e16 = ((warp - 2) >> 2) * 16;                   // this warp's first 16 columns of every 32; the quadrant's two warps share them
+        const uint32_t tq = tmem_base + ((uint32_t)(q * 32) << 16);
+        bool ok = true;
+        // ---- generated tiles: group g of a stage = 16 columns of one token; this thread's groups lie 256 apart ----
+        if constexpr (GEN) {
+            constexpr int AHEAD = GQ < 4 ? 2 : 1;                 // stages whose gates and da are in registers ahead of use
+            int row[GQ], cg[GQ], f_rt = rt0, f_sc = rt0 % p.s_chunks, f_b = rt0 / p.s_chunks;
+            uint32_t off[GQ], gs = 0, geph = 1, gdst = smem_u32(smem) + a_bytes;
+            const uint32_t open_bias = (uint32_t)(l | 0x80) * 0x01010101u;
+            uint4 t4[AHEAD][GQ], d4[AHEAD][GQ][2 * GT];
+            auto fetch = [&](uint4 (&t)[GQ], uint4 (&dd)[GQ][2 * GT]) {
+                if (f_rt >= rt1) return;
 #pragma unroll
-                            for (int cc = 0; cc < 16; cc += 4)
-                                *reinterpret_cast<float4*>(dst + c0 + cc) = make_float4(v[cc], v[cc + 1], v[cc + 2], v[cc + 3]);
-                        }
+                for (int i = 0; i < GQ; ++i) {
+                    if (row[i] < 0) continue;
+                    const int tok = f_sc * BWD_KR + row[i];
+                    t[i] = make_uint4(0x7f7f7f7fu, 0x7f7f7f7fu, 0x7f7f7f7fu, 0x7f7f7f7fu);      // closed
+                    if (tok < p.S) t[i] = __ldcg(reinterpret_cast<const uint4*>(p.tc + ((long long)f_b * p.S + tok) * p.r + cg[i]));
+                    const uint4* d = reinterpret_cast<const uint4*>(p.da + f_b * p.da_sample + (long long)min(tok, p.S - 1) * p.da_token + cg[i]);
+#pragma unroll
+                    for (int k = 0; k < GT; ++k) {
+                        dd[i][2 * k] = d[0]; dd[i][2 * k + 1] = d[1];
+                        d = reinterpret_cast<const uint4*>(reinterpret_cast<const bf16*>(d) + p.da_term);
                     }
                 }
-            }
-        } else {
-            // no rows in this split: the partial is zero
-            for (int c = 0; c < p.chunks; ++c) {
-                const int k = col0 + c * 128 + q * 32 + lane;
-                if (k < p.d && e16 == 0) {
-                    float* dst = p.out + (((long long)j * p.L + l) * p.d + k) * p.r;
-                    for (int c0 = 0; c0 < p.r; ++c0) dst[c0] = 0.f;
+                ++f_rt;
+                if (++f_sc == p.s_chunks) { f_sc = 0; ++f_b; }
+            };
+            // Builds the next stage's tile and requests the gates of the stage AHEAD further on.
+            auto build = [&](uint4 (&t)[GQ], uint4 (&dd)[GQ][2 * GT]) -> bool {
+                if (!mbar_wait_uniform(empty0 + 8 * gs, geph, abort_flag, p.status)) return false;
+#pragma unroll
+                for (int i = 0; i < GQ; ++i) {
+                    if (row[i] < 0) continue;
+                    // open where l + 1 > tc: bit 7 of (l + 128) - tc, byte by byte, spread over the element's two bytes
+                    const uint32_t y[4] = {open_bias - t[i].x, open_bias - t[i].y, open_bias - t[i].z, open_bias - t[i].w};
+                    uint32_t m[8];
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) { m[2 * e] = spread_sign(y[e], 0x9988u); m[2 * e + 1] = spread_sign(y[e], 0xbbaau); }
+#pragma unroll
+                    for (int k = 0; k < GT; ++k) {
+                        const uint4 x = dd[i][2 * k], z = dd[i][2 * k + 1];
+                        const uint32_t a0 = gdst + (uint32_t)k * ((uint32_t)p.r_blocks * box_bytes) + off[i];
+                        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(a0), "r"(x.x & m[0]), "r"(x.y & m[1]), "r"(x.z & m[2]), "r"(x.w & m[3]) : "memory");
+                        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(a0 ^ 16u), "r"(z.x & m[4]), "r"(z.y & m[5]), "r"(z.z & m[6]), "r"(z.w & m[7]) : "memory");
+                    }
                 }
+                fence_proxy_async();                              // the tile is read by the tensor core
+                __syncwarp();
+                if (lane == 0) mbar_arrive(full0 + 8 * gs);
+                fetch(t, dd);
+                gdst += stage_bytes;
+                if (++gs == (uint32_t)p.stages) { gs = 0; geph ^= 1u; gdst = smem_u32(smem) + a_bytes; }
+                return true;
+            };
+            const int g16 = p.r >> 4, total = BWD_KR * g16;
+#pragma unroll
+            for (int i = 0; i < GQ; ++i) {
+                const int gi = (int)threadIdx.x - 64 + 256 * i;
+                row[i] = gi / g16; cg[i] = (gi - row[i] * g16) * 16;
+                // box of 64 columns, rows of 128 bytes, 16-byte chunks swizzled with the row
+                off[i] = (uint32_t)(cg[i] >> 6) * box_bytes + (uint32_t)row[i] * 128u + (uint32_t)((((cg[i] & 63) >> 3) ^ (row[i] & 7)) << 4);
+                if (gi >= total) row[i] = -1;
+            }
+#pragma unroll
+            for (int k = 0; k < AHEAD; ++k) fetch(t4[k], d4[k]);
+            for (int rt = rt0; rt < rt1 && ok; rt += AHEAD)
+#pragma unroll
+                for (int k = 0; k < AHEAD; ++k)
+                    if (ok && rt + k < rt1) ok = build(t4[k], d4[k]);
+        }
+        // ---- out (zeros for a split without rows), and its share of <out, W_down>: (column block, 16 columns) units, W_down requested two
+        // units ahead, the first two before the accumulators are complete ----
+        const int steps = (p.r - e16 + 31) >> 5, units = p.chunks * steps;
+        float dot = 0.f;
+        float4 w[2][4];
+        auto load_w = [&](int u, float4 (&x)[4]) {
+            const int c = u / steps, k = col0 + c * 128 + q * 32 + lane;
+            const float4* src = reinterpret_cast<const float4*>(p.w + ((long long)l * p.d + k) * p.r + e16 + 32 * (u - c * steps));
+#pragma unroll
+            for (int e = 0; e < 4; ++e) x[e] = GEN && u < units && k < p.d ? __ldcg(src + e) : make_float4(0.f, 0.f, 0.f, 0.f);
+        };
+        auto finish = [&](int u, const float4 (&x)[4]) {
+            const int c = u / steps, c0 = e16 + 32 * (u - c * steps), k = col0 + c * 128 + q * 32 + lane;     // column of h = row of dW_down
+            float v[16] = {};
+            if (rt0 < rt1) {
+                const uint32_t taddr = tq + (uint32_t)(c * n_cols + c0);
+                tmem_ld16(taddr, v);
+                if (side) {
+                    float v2[16];
+                    tmem_ld16(taddr + (uint32_t)(64 * p.r_blocks), v2);
+                    tmem_ld_wait();
+#pragma unroll
+                    for (int e = 0; e < 16; ++e) v[e] += v2[e];
+                } else {
+                    tmem_ld_wait();
+                }
+            }
+            if (k >= p.d) return;
+            float* dst = p.out + (((long long)j * p.L + l) * p.d + k) * p.r + c0;
+            // (16-byte stores: with 32-byte ones here the step measured 0.4 us slower)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                *reinterpret_cast<float4*>(dst + 4 * e) = make_float4(v[4 * e], v[4 * e + 1], v[4 * e + 2], v[4 * e + 3]);
+                if (GEN) dot = fmaf(v[4 * e], x[e].x, fmaf(v[4 * e + 1], x[e].y, fmaf(v[4 * e + 2], x[e].z, fmaf(v[4 * e + 3], x[e].w, dot))));
+            }
+        };
+        if (steps > 0) { load_w(0, w[0]); load_w(1, w[1]); }
+        if (rt0 < rt1) {
+            ok = ok && mbar_wait_warp(accf, 0, abort_flag, p.status);
+            tc_fence_after();
+            if (threadIdx.x == 64 && ok) stamp_end(p.stamp);
+        }
+        if (ok && steps > 0)
+            for (int u = 0; u < units; u += 2) {
+                finish(u, w[0]);
+                load_w(u + 2, w[0]);
+                if (u + 1 < units) finish(u + 1, w[1]);
+                load_w(u + 3, w[1]);
+            }
+        if (GEN) {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
+            if (lane == 0) dot_s[warp - 2] = dot;
+            asm volatile("bar.sync 1, %0;" ::"n"(32 * DW_GEN_WARPS) : "memory");
+            if (threadIdx.x == 64) {
+                float t = 0.f;
+#pragma unroll
+                for (int i = 0; i < DW_GEN_WARPS; ++i) t += dot_s[i];
+                p.dot_part[((long long)l * p.d_groups + g) * p.splits + j] = t;
             }
         }
     }
@@ -725,7 +849,7 @@ inline void pdl_launch_config(cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr
 }
 
 inline bool tensor_shape_supported(const Dims& dm) {
-    return dm.d % 8 == 0 && dm.d >= 64 && dm.r % 16 == 0 && dm.r >= 16 && dm.r <= 256;
+    return dm.d % 8 == 0 && dm.d >= 64 && dm.r % 16 == 0 && dm.r >= 16 && dm.r <= 256 && dm.L <= 127;      // (gate bytes hold a layer number)
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
@@ -768,7 +892,8 @@ inline int pow2_at_least(int x) { int p = 32; while (p < x) p <<= 1; return p; }
 // [L][3][max_rows][r]), whose sum is the fp32 value, so the products are those of fp32 operands.  *part_floats receives the
 // size of the split-partial buffer dW needs (0 when no split is used).
 inline pac_status tensor_plan_create(TensorPlan& tp, int device, const bf16* cache, const Dims& dm, int max_batch,
-                                     const bf16* wdT, const bf16* du16, long long* part_floats, bool exact = false) {
+                                     const bf16* wdT, const bf16* du16, long long* part_floats, bool exact = false, bool per_token = false) {
+    const bool gen = !exact;                                 // du is generated (pointwise bodies)
     tp.ready = false;
     tp.dm = dm;
     tp.max_batch = max_batch;
@@ -779,7 +904,11 @@ inline pac_status tensor_plan_create(TensorPlan& tp, int device, const bf16* cac
     const int max_smem = (int)prop.sharedMemPerBlockOptin;
     const long long max_rows = (long long)max_batch * dm.S;
     const int r_pad = (dm.r + 15) & ~15;
-    const int wt = exact ? 3 : 2, dt = exact ? 3 : 1;        // bf16 terms of W_down and du
+    const int wt = exact ? 3 : 2;                            // bf16 terms of W_down
+    // of du: the fp32 value exactly, or generated: two terms of da, as precise as W_down, where the second one's products cost nothing beside the
+    // stream (with one, dlambda of a small batch is off by a percent); one for wide adapters with da per sample, where they cost power
+    // and du entered in one term before
+    const int dt = exact ? 3 : dm.r <= 64 || per_token ? 2 : 1;
 
     // ---- tensor maps ----
     {
@@ -795,7 +924,8 @@ inline pac_status tensor_plan_create(TensorPlan& tp, int device, const bf16* cac
         cuuint32_t box[4] = {64, KC, (cuuint32_t)wt, 1};
         if (!make_map(&tp.map_w, wdT, 4, dims, str, box)) return PAC_ERR_UNSUPPORTED;
     }
-    {
+    tp.map_du = tp.map_w;                                    // unused when du is generated
+    if (!gen) {
         cuuint64_t dims[3] = {(cuuint64_t)dm.r, (cuuint64_t)max_rows, (cuuint64_t)dm.L * dt};
         cuuint64_t str[2] = {(cuuint64_t)dm.r * 2, (cuuint64_t)max_rows * dm.r * 2};
         cuuint32_t box[3] = {KC, BWD_KR, 1};
@@ -826,10 +956,11 @@ inline pac_status tensor_plan_create(TensorPlan& tp, int device, const bf16* cac
     b.N = dm.N; b.L = dm.L; b.S = dm.S; b.d = dm.d; b.r = dm.r;
     b.s_chunks = (dm.S + BWD_KR - 1) / BWD_KR;
     b.r_blocks = (dm.r + 63) / 64;
-    b.terms = dt;
-    b.chunks = (dm.d >= 256 && 2 * r_pad <= 512) ? 2 : 1;
+    b.terms = dt; b.gen = gen ? 1 : 0;
+    const int n_cols = gen && dt == 2 && dm.r <= 128 ? 128 * b.r_blocks : r_pad;
+    b.chunks = (dm.d >= 256 && 2 * n_cols <= 512) ? 2 : 1;
     b.d_groups = (dm.d + 128 * b.chunks - 1) / (128 * b.chunks);
-    b.tmem_cols = pow2_at_least(b.chunks * r_pad);
+    b.tmem_cols = pow2_at_least(b.chunks * n_cols);
     {
         const int stage = (b.chunks * 2 + b.r_blocks * dt) * BWD_KR * 128;
         int st = (max_smem - 2048) / stage;
@@ -852,10 +983,9 @@ inline pac_status tensor_plan_create(TensorPlan& tp, int device, const bf16* cac
         b.splits = best;
     }
     tp.dw_elems = (long long)dm.L * dm.d * dm.r;
-    *part_floats = b.splits > 1 ? tp.dw_elems * b.splits : 0;
+    *part_floats = gen || b.splits > 1 ? tp.dw_elems * b.splits : 0;
 
-    if (smem_opt_in((const void*)down_fwd_tc_kernel, tp.smem_fwd) != cudaSuccess ||
-        smem_opt_in((const void*)dw_down_tc_kernel, tp.smem_bwd) != cudaSuccess) {
+    if (smem_opt_in((const void*)down_fwd_tc_kernel, tp.smem_fwd) != cudaSuccess) {
         tensor_err() = "cudaFuncSetAttribute(MaxDynamicSharedMemorySize) failed";
         cudaGetLastError();
         return PAC_ERR_CUDA;
@@ -888,24 +1018,33 @@ inline int tensor_splits(const TensorPlan& tp, int B) {
     return J;
 }
 
-// With reduce_splits == false and more than one split the partial sums stay in `part`
+// What the second pass builds du from (BwdParams).
+struct DuGen { const uint8_t* tc; const bf16* da; long long da_term, da_sample; int da_token; const float* w; float* dot_part; };
+
+// With reduce_splits == false and more than one split, and always when du is generated, the partial sums stay in `part`
 // ([J][L][d][r]) for the caller's own reduction.
 inline pac_status tensor_dw_down(TensorPlan& tp, cudaStream_t stream, const int* d_ids, int B, const bf16* /*du16*/,
                                  float* dW, float* part, bool reduce_splits, unsigned* status, long long* launches,
-                                 unsigned long long* stamp = nullptr, bool early_ids = false) {
+                                 unsigned long long* stamp = nullptr, bool early_ids = false, const DuGen* gen = nullptr) {
     BwdParams p = tp.bp;
+    if (p.gen) { p.tc = gen->tc; p.da = gen->da; p.da_term = gen->da_term; p.da_sample = gen->da_sample; p.da_token = gen->da_token; p.w = gen->w; p.dot_part = gen->dot_part; }
     p.ids = d_ids; p.B = B; p.status = status; p.stamp = stamp; p.early_ids = early_ids ? 1 : 0;
     const int J = tensor_splits(tp, B);
     p.splits = J;
-    p.out = J > 1 ? part : dW;
+    p.out = p.gen || J > 1 ? part : dW;
     const int grid = p.L * p.d_groups * J;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[1];
     pdl_launch_config(&cfg, attr, dim3((unsigned)grid), dim3(DW_THREADS), tp.smem_bwd, stream);
-    cudaError_t e = cudaLaunchKernelEx(&cfg, dw_down_tc_kernel, tp.map_cache_bwd, tp.map_du, p);
+    const auto kernel = !p.gen ? dw_down_tc_kernel<0, 1> : p.r <= 64 ? dw_down_tc_kernel<1, 2>
+                      : p.r <= 128 ? (p.terms == 2 ? dw_down_tc_kernel<2, 2> : dw_down_tc_kernel<2, 1>)
+                                   : (p.terms == 2 ? dw_down_tc_kernel<4, 2> : dw_down_tc_kernel<4, 1>);
+    cudaError_t e = smem_opt_in((const void*)kernel, tp.smem_bwd);
+    if (e != cudaSuccess) { tensor_err() = cudaGetErrorString(e); return PAC_ERR_CUDA; }
+    e = cudaLaunchKernelEx(&cfg, kernel, tp.map_cache_bwd, tp.map_du, p);
     (*launches)++;
     if (e != cudaSuccess) { tensor_err() = cudaGetErrorString(e); return PAC_ERR_CUDA; }
-    if (J > 1 && reduce_splits) {
+    if (!p.gen && J > 1 && reduce_splits) {
         reduce_splits_kernel<<<(unsigned)((tp.dw_elems / 4 + 255) / 256), 256, 0, stream>>>(part, J, tp.dw_elems, dW);
         (*launches)++;
         e = cudaGetLastError();
