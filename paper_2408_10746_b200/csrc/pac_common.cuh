@@ -57,14 +57,32 @@ inline cudaError_t smem_opt_in(const void* kernel, size_t bytes) {
 // term 0), ...; two terms carry about 16 mantissa bits, three the fp32 value exactly.
 struct WdShadow {
     bf16* p; int terms;
-    __device__ __forceinline__ void put(long long l, long long dr, long long rem, float x) const {
-        for (int t = 0; t < terms; ++t) {
-            const bf16 v = __float2bfloat16(x);
-            p[(l * terms + t) * dr + rem] = v;
-            x -= __bfloat162float(v);
+    // x into the terms of one element, `dr` apart.
+    __device__ __forceinline__ void put(long long at, long long dr, float x) const {
+        const bf16 a = __float2bfloat16(x);
+        x -= __bfloat162float(a);
+        const bf16 b = __float2bfloat16(x);
+        p[at] = a; p[at + dr] = b;
+        if (terms == 3) p[at + 2 * dr] = __float2bfloat16(x - __bfloat162float(b));
+    }
+    __device__ __forceinline__ void put4(long long at, long long dr, const float (&x)[4]) const {
+        bf16 v[3][4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            v[0][e] = __float2bfloat16(x[e]);
+            const float y = x[e] - __bfloat162float(v[0][e]);
+            v[1][e] = __float2bfloat16(y);
+            v[2][e] = __float2bfloat16(y - __bfloat162float(v[1][e]));
         }
+        *reinterpret_cast<uint2*>(p + at) = *reinterpret_cast<const uint2*>(v[0]);
+        *reinterpret_cast<uint2*>(p + at + dr) = *reinterpret_cast<const uint2*>(v[1]);
+        if (terms == 3) *reinterpret_cast<uint2*>(p + at + 2 * dr) = *reinterpret_cast<const uint2*>(v[2]);
     }
 };
+// Layer of element i of the W_down block (dr = d r elements each): a 32-bit division where the block's size allows it.
+__device__ __forceinline__ int wd_layer(long long i, long long lam, unsigned dr) {
+    return lam <= 0x7fffffffLL ? (int)((unsigned)i / dr) : (int)(i / dr);
+}
 
 struct Dims {
     long long N;   // samples in the cache

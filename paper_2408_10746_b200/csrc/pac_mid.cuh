@@ -705,6 +705,7 @@ __global__ void __launch_bounds__(256, 5) finalize_cls_kernel(FinalizeParams f) 
     const long long i_wd = ((long long)(blk - f.rest_blocks) * blockDim.x + threadIdx.x) * 4;
     const bool wd_thread = blk >= f.rest_blocks && i_wd < lay.lam;
     float4 p4 = make_float4(0.f, 0.f, 0.f, 0.f), m4 = p4, v4 = p4;
+    const int l_wd = wd_thread ? wd_layer(i_wd, lay.lam, (unsigned)(f.d * f.r)) : 0;
     if (wd_thread && f.adam) {
         p4 = *reinterpret_cast<const float4*>(f.params + i_wd);
         m4 = *reinterpret_cast<const float4*>(f.m + i_wd);
@@ -840,7 +841,7 @@ __global__ void __launch_bounds__(256, 5) finalize_cls_kernel(FinalizeParams f) 
                 g4.x += q.x; g4.y += q.y; g4.z += q.z; g4.w += q.w;
             }
             if (f.coef) {
-                const float c = f.coef[(int)(i / ((long long)f.d * f.r))];
+                const float c = f.coef[l_wd];
                 g4.x *= c; g4.y *= c; g4.z *= c; g4.w *= c;
             }
             *reinterpret_cast<float4*>(f.grads + i) = g4;
@@ -849,7 +850,7 @@ __global__ void __launch_bounds__(256, 5) finalize_cls_kernel(FinalizeParams f) 
         }
         if (f.adam) {
             g4.x *= f.grad_scale; g4.y *= f.grad_scale; g4.z *= f.grad_scale; g4.w *= f.grad_scale;
-            adamw_w_down4_loaded(f.params, f.m, f.v, i, p4, m4, v4, g4, f.hp, f.bc1, f.bc2, f.wdT, f.d, f.r);
+            adamw_w_down4_loaded(f.params, f.m, f.v, i, l_wd, p4, m4, v4, g4, f.hp, f.bc1, f.bc2, f.wdT, f.d, f.r);
         }
         return;
     }

@@ -530,25 +530,16 @@ __device__ __forceinline__ void adamw_element(float* __restrict__ p, float* __re
     v[i] = vi;
     p[i] = th;
     if (wdT.p && i < lay.lam) {
-        const long long dr = (long long)d * r, l = i / dr;
-        wdT.put(l, dr, i - l * dr, th);
+        const long long dr = (long long)d * r, l = wd_layer(i, lay.lam, (unsigned)dr);
+        wdT.put(i + l * (wdT.terms - 1) * dr, dr, th);
     }
 }
 
 // Four consecutive elements of the W_down block (i a multiple of 4; d*r is a multiple of 4, so
 // the four share a layer): vector loads and stores, the same arithmetic per element.
-// The same with the old parameter and moments already in registers (a caller may fetch them early).
+// The old parameter and moments are already in registers (a caller may fetch them early), and so is the layer.
 __device__ __forceinline__ void adamw_w_down4_loaded(float* __restrict__ p, float* __restrict__ m, float* __restrict__ v,
-                                                     long long i, float4 p4, float4 m4, float4 v4, float4 g4, const pac_adamw& hp,
-                                                     float bc1, float bc2, WdShadow wdT, int d, int r);
-__device__ __forceinline__ void adamw_w_down4(float* __restrict__ p, float* __restrict__ m, float* __restrict__ v,
-                                              long long i, float4 g4, const pac_adamw& hp, float bc1, float bc2,
-                                              WdShadow wdT, int d, int r) {
-    const float4 p4 = *reinterpret_cast<float4*>(p + i), m4 = *reinterpret_cast<float4*>(m + i), v4 = *reinterpret_cast<float4*>(v + i);
-    adamw_w_down4_loaded(p, m, v, i, p4, m4, v4, g4, hp, bc1, bc2, wdT, d, r);
-}
-__device__ __forceinline__ void adamw_w_down4_loaded(float* __restrict__ p, float* __restrict__ m, float* __restrict__ v,
-                                                     long long i, float4 p4, float4 m4, float4 v4, float4 g4, const pac_adamw& hp,
+                                                     long long i, int l, float4 p4, float4 m4, float4 v4, float4 g4, const pac_adamw& hp,
                                                      float bc1, float bc2, WdShadow wdT, int d, int r) {
     p4.x = adamw_math(p4.x, m4.x, v4.x, g4.x, true, hp, bc1, bc2);
     p4.y = adamw_math(p4.y, m4.y, v4.y, g4.y, true, hp, bc1, bc2);
@@ -558,17 +549,9 @@ __device__ __forceinline__ void adamw_w_down4_loaded(float* __restrict__ p, floa
     *reinterpret_cast<float4*>(m + i) = m4;
     *reinterpret_cast<float4*>(v + i) = v4;
     if (wdT.p) {
-        const long long dr = (long long)d * r, l = i / dr, rem = i - l * dr;
-        float th[4] = {p4.x, p4.y, p4.z, p4.w};
-        for (int t = 0; t < wdT.terms; ++t) {
-            bf16 v[4];
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                v[e] = __float2bfloat16(th[e]);
-                th[e] -= __bfloat162float(v[e]);
-            }
-            *reinterpret_cast<uint2*>(wdT.p + (l * wdT.terms + t) * dr + rem) = *reinterpret_cast<const uint2*>(v);
-        }
+        const long long dr = (long long)d * r;
+        const float th[4] = {p4.x, p4.y, p4.z, p4.w};
+        wdT.put4(i + l * (wdT.terms - 1) * dr, dr, th);
     }
 }
 
@@ -590,7 +573,8 @@ __global__ void adamw_kernel(float* __restrict__ p, const float* __restrict__ g,
         if (i < lay.lam) {
             float4 g4 = *reinterpret_cast<const float4*>(g + i);
             g4.x *= grad_scale; g4.y *= grad_scale; g4.z *= grad_scale; g4.w *= grad_scale;
-            adamw_w_down4(p, m, v, i, g4, hp, bc1, bc2, wdT, d, r);
+            adamw_w_down4_loaded(p, m, v, i, wd_layer(i, lay.lam, (unsigned)(d * r)), *reinterpret_cast<float4*>(p + i), *reinterpret_cast<float4*>(m + i),
+                                 *reinterpret_cast<float4*>(v + i), g4, hp, bc1, bc2, wdT, d, r);
         }
         return;
     }
@@ -604,7 +588,7 @@ __global__ void shadow_wdown_kernel(const float* __restrict__ w, WdShadow wdT, i
     long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= (long long)L * d * r) return;
     const long long dr = (long long)d * r, l = i / dr;
-    wdT.put(l, dr, i - l * dr, w[i]);
+    wdT.put(i + l * (wdT.terms - 1) * dr, dr, w[i]);
 }
 
 }  // namespace pac
