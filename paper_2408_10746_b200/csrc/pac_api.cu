@@ -67,7 +67,8 @@ struct Scratch {
     uint8_t* tc = nullptr;         // [M][r] 1 + highest closed layer
     bf16* da16 = nullptr;          // [2][max_batch][r] (classifier) or [2][M][r] (LM): da_L in two terms
     float* coef = nullptr;         // [L] lambda_l prod_{l' > l} (1 - lambda_l')
-    float* dot_part = nullptr;     // [L][d groups][splits] shares of <D_l, W_down^l>
+    float* dot_part = nullptr;     // [L][blocks per layer] shares of <D_l, W_down^l>, and the count of blocks done
+    unsigned* dot_done = nullptr;
     float* pool_part = nullptr;    // [B][s_chunks * 4][r] token sums of a_L per 32-token group (chain-in-epilogue forward)
     float* prodW = nullptr;        // [r][C] W_up W_head of the current parameters (stand-alone head kernels)
 };
@@ -420,7 +421,7 @@ pac_status adam_body_enqueue(pac_ctx* c, const pac_adamw* hp);
 // move four elements at a time; otherwise the kernels that form the d-wide vectors.
 bool plain_head_ok(const pac_ctx* c, int B) {
     const Dims& dm = c->dm;
-    return c->cfg.head == PAC_HEAD_MEANPOOL_CLS && dm.C <= MID_MAX_C && (!use_tensor(c) || dm.L <= MID_MAX_L) && 9 * dm.r + dm.C + 32 <= 12000 && ((long long)dm.L * dm.d * dm.r) % 4 == 0 &&
+    return c->cfg.head == PAC_HEAD_MEANPOOL_CLS && dm.C <= MID_MAX_C && (!use_tensor(c) || dm.L <= MID_MAX_L) && 9 * dm.r + dm.C + 32 <= 12000 && ((long long)dm.L * dm.d * dm.r) % 4 == 0 && (long long)dm.L * dm.d * dm.r <= 0x7fffffffLL &&
            (2LL * B + dm.r + dm.C) * FIN_KB * 4 <= 48 * 1024;
 }
 pac_status plain_head(pac_ctx* c, const int* d_ids, int B, bool train, const float* aL, float* d_logits_out) {
@@ -649,9 +650,9 @@ pac_status backward(pac_ctx* c, const int* d_ids, int B, float* d_loss, const pa
             return finalize_enqueue(c, d_ids, B, d_loss, hp);
         }
         const long long ne = (long long)dm.L * dm.d * dm.r;
-        const int J = tensor_splits(c->tplan, B);
-        gated_grads_kernel<<<cdiv(ne / 4, 256) + 1, 256, 0, c->stream>>>(sc.dw_part, J, ne, dm.d * dm.r, dm.L, c->params + c->lay.lam, sc.coef, sc.dot_part,
-                                                                       c->tplan.bp.d_groups * J, c->grads + c->lay.w_down, c->grads + c->lay.lam);
+        const int per_layer = (int)cdiv((long long)dm.d * dm.r, 1024);
+        gated_grads_kernel<<<dm.L * per_layer, 256, 0, c->stream>>>(sc.dw_part, tensor_splits(c->tplan, B), ne, dm.d * dm.r, per_layer, dm.L, c->params + c->lay.w_down,
+                                                                  c->params + c->lay.lam, sc.coef, sc.dot_part, sc.dot_done, c->grads + c->lay.w_down, c->grads + c->lay.lam);
         LAUNCH_CHECK(c);
         return PAC_OK;
     }
@@ -934,7 +935,6 @@ pac_status dw_down(pac_ctx* c, const int* d_ids, int B, bool reduce_splits) {
         const bool lm = c->cfg.head == PAC_HEAD_FROZEN_LM;
         gen.tc = c->sc.tc; gen.da = c->sc.da16; gen.da_term = (long long)(lm ? c->max_rows : c->cfg.max_batch) * dm.r;
         gen.da_sample = lm ? (long long)dm.S * dm.r : dm.r; gen.da_token = lm ? dm.r : 0;
-        gen.w = c->params + c->lay.w_down; gen.dot_part = c->sc.dot_part;
         st = tensor_dw_down(c->tplan, c->stream, d_ids, B, c->sc.du16, c->grads + c->lay.w_down, c->sc.dw_part,
                             reduce_splits, c->status, &c->launches, next_stamp(c, 1),
                             c->step_early_ids && !c->step_host_ids, &gen);       // ids no kernel in flight writes
@@ -1074,7 +1074,7 @@ pac_status finalize_enqueue(pac_ctx* c, const int* d_ids, int B, float* d_loss, 
     const bool tens = use_tensor(c) || c->exact_ok;
     f.dw_part = tens ? sc.dw_part : sc.dw_spart;
     f.splits = tens ? tensor_splits(c->tplan, B) : dw_simt_slices(c, B);
-    if (use_tensor(c)) { f.coef = sc.coef; f.dot_part = sc.dot_part; f.dot_n = c->tplan.bp.d_groups * f.splits; }
+    if (use_tensor(c)) { f.coef = sc.coef; f.dot_part = sc.dot_part; f.done = sc.dot_done; }
     else if (f.splits <= 1) f.splits = 0;                // already in the gradient buffer
     f.dw_elems = (long long)dm.L * dm.d * dm.r;
     // per-CTA partial sums of dlambda: the fused head kernels', or the plain reverse chain's; transformer bodies: done
@@ -1091,7 +1091,11 @@ pac_status finalize_enqueue(pac_ctx* c, const int* d_ids, int B, float* d_loss, 
         f.wdT = wd_shadow(c);
         f.grad_scale = c->grad_scale;
     }
-    f.wd_blocks = (int)cdiv(c->lay.lam / 4, 256);
+    // (a layer of the plain path may not be a multiple of four elements: all layers as one then)
+    const bool by_layer = ((long long)dm.d * dm.r) % 4 == 0;
+    f.wd_layer_elems = by_layer ? dm.d * dm.r : (int)c->lay.lam;
+    f.wd_per_layer = (int)cdiv(f.wd_layer_elems / 4, 256);
+    f.wd_blocks = f.wd_per_layer * (by_layer ? dm.L : 1);
     if (c->step_host_ids) {
         // the step after this one will look for its ids under sequence number zc_count + 2 in the next ring slot
         const unsigned next_seq = (unsigned)(c->zc_count + 2);
@@ -1183,7 +1187,7 @@ void free_all(pac_ctx* c) {
     Scratch& s = c->sc;
     if (c->hc.on) s.hbar = nullptr;            // points into a staging slot, freed below
     void* ptrs[] = {s.ids, s.u, s.a, s.du, s.du16, s.lam_part, s.loss, s.hbar, s.pooled_a, s.pooled_y, s.logits,
-                    s.dlogits, s.loss_b, s.gvec, s.daL, s.y, s.lm_logits, s.dy, s.y16, s.dlog16, s.aL16, s.wup16, s.dy16, s.wdT, s.lm_part, s.dw_part, s.dw_spart, s.tc, s.da16, s.coef, s.dot_part, s.pool_part, s.prodW, c->tb.buf, c->params, c->grads,
+                    s.dlogits, s.loss_b, s.gvec, s.daL, s.y, s.lm_logits, s.dy, s.y16, s.dlog16, s.aL16, s.wup16, s.dy16, s.wdT, s.lm_part, s.dw_part, s.dw_spart, s.tc, s.da16, s.coef, s.dot_part, s.dot_done, s.pool_part, s.prodW, c->tb.buf, c->params, c->grads,
                     c->m, c->v, c->status, c->d_perm, c->d_losses, c->d_stamps};
     for (void* p : ptrs)
         if (p) cudaFree(p);
@@ -1479,7 +1483,9 @@ pac_status pac_adapter_init(pac_ctx* c, const pac_adapter_cfg* cfg, unsigned lon
             }
             if (ts == PAC_OK) {
                 A(dmalloc(c, &s.dw_part, part_floats));
-                A(dmalloc(c, &s.dot_part, (long long)dm.L * c->tplan.bp.d_groups * c->tplan.bp.splits));
+                A(dmalloc(c, &s.dot_part, (long long)dm.L * cdiv((long long)dm.d * dm.r, 1024)));
+                A(dmalloc(c, &s.dot_done, 1));
+                if (st == PAC_OK) CU_OK(c, cudaMemsetAsync(s.dot_done, 0, sizeof(unsigned), c->stream));
                 c->chain_ok = false;
                 if (st == PAC_OK && cls && c->mplan.ok && chain_fwd_supported(dm) && c->tplan.fp.wide_n) {
                     c->pplan = mid_plan_pooled(dm);

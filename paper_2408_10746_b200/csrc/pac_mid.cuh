@@ -607,15 +607,16 @@ struct FinalizeParams {
     ParamLayout lay;
     int B, d, r, C, L;
     const float* dw_part; int splits; long long dw_elems;     // splits < 1: W_down gradient already in grads
-    // Tensor-core path: dw_part holds D_l = h_l^T (open_l daL) (see MidParams), dW_down^l = coef[l] D_l, and dot_part the shares of
-    // P_l = <D_l, W_down^l>, dot_n per layer, which are all that dlambda needs (see lambda_grad).
-    const float* coef; const float* dot_part; int dot_n;
+    // Tensor-core path: dw_part holds D_l = h_l^T (open_l daL) (see MidParams), dW_down^l = coef[l] D_l, and P_l = <D_l, W_down^l>
+    // is all that dlambda needs (see lambda_grad): every W_down block leaves its share in dot_part [L][wd_per_layer], the last one to
+    // finish (counted in `done`, which it puts back to zero) updates lambda.
+    const float* coef; float* dot_part; unsigned* done;
     const float* lam_part; int lam_blocks;                   // null: the lambda gradients are already in grads
     const float *pooled_a, *dlogits, *loss_b;                // per-sample vectors the forward half left: mean_s a_L, dlogits, loss
     const float* hbar; const int* ids; long long N;          // token mean of the last cached layer, per cache sample; the batch's ids
     const float* params_in;                                  // the parameters the forward half used (W_up, W_head are read)
     float* grads; float* loss_out;
-    int wd_blocks;                                           // blocks that handle W_down, 4 elements per thread
+    int wd_blocks, wd_per_layer, wd_layer_elems;             // blocks that handle W_down, 4 elements per thread, within one layer each
     int rest_blocks;                                         // blocks that handle the head side: FIN_KB columns of the hidden width each
     // AdamW
     int adam;
@@ -658,32 +659,62 @@ __device__ __forceinline__ float lambda_grad(const float* lam, const float* P, i
     }
     return g;
 }
-// The gradients of W_down (four elements per thread) and lambda (last block) from the second pass's partial sums where no
-// finalisation kernel follows (L <= 128).
-__global__ void __launch_bounds__(256) gated_grads_kernel(const float* __restrict__ part, int splits, long long n, int dr, int L, const float* __restrict__ lam,
-                                                          const float* __restrict__ coef, const float* __restrict__ dot_part, int dot_n,
-                                                          float* __restrict__ gW, float* __restrict__ glam) {
-    if (blockIdx.x + 1 == gridDim.x) {
-        __shared__ float lam_s[128], dot_s[128];
-        for (int l = threadIdx.x; l < L; l += 256) {
-            lam_s[l] = lam[l];
-            float acc = 0.f;
-            for (int k = 0; k < dot_n; ++k) acc += dot_part[(long long)l * dot_n + k];
-            dot_s[l] = acc;
+// Blocks of 256 threads: the block's sum of `dot` goes to dot_part[blk]; true in the block that finishes last of n (the shares of all are
+// then visible to it), which puts the counter back.
+__device__ __forceinline__ bool last_with_dots(float dot, float* __restrict__ dot_part, int blk, int n, unsigned* done) {
+    __shared__ float red[8];
+    __shared__ unsigned last;
+    dot = warp_sum(dot);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = dot;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        float t = 0.f;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) t += red[w];
+        dot_part[blk] = t;
+        __threadfence();
+        last = atomicAdd(done, 1u) == (unsigned)(n - 1);
+        if (last) { *done = 0u; __threadfence(); }
+    }
+    __syncthreads();
+    return last != 0u;
+}
+// P_l from the blocks' shares, warp per layer, and lambda, into shared memory.
+__device__ __forceinline__ void sum_dots(const float* lam, const float* dot_part, int per_layer, int L, float* lam_s, float* dot_s) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    for (int l = threadIdx.x; l < L; l += 256) lam_s[l] = lam[l];
+    for (int l = warp; l < L; l += 8) {
+        float acc = 0.f;
+        for (int k = lane; k < per_layer; k += 32) acc += __ldcg(dot_part + (long long)l * per_layer + k);
+        acc = warp_sum(acc);
+        if (lane == 0) dot_s[l] = acc;
+    }
+    __syncthreads();
+}
+// The gradients of W_down (four elements per thread, blocks within one layer each) and lambda (the block that finishes last) from
+// the second pass's partial sums where no finalisation kernel follows (L <= 128).
+__global__ void __launch_bounds__(256) gated_grads_kernel(const float* __restrict__ part, int splits, long long n, int dr, int per_layer, int L,
+                                                          const float* __restrict__ w, const float* __restrict__ lam, const float* __restrict__ coef,
+                                                          float* __restrict__ dot_part, unsigned* done, float* __restrict__ gW, float* __restrict__ glam) {
+    const int l = blockIdx.x / per_layer, o = ((blockIdx.x - l * per_layer) * 256 + threadIdx.x) * 4;
+    float dot = 0.f;
+    if (o < dr) {
+        const long long i = (long long)l * dr + o;
+        const float4 p = *reinterpret_cast<const float4*>(w + i);
+        float4 a = *reinterpret_cast<const float4*>(part + i);
+        for (int s = 1; s < splits; ++s) {
+            const float4 v = *reinterpret_cast<const float4*>(part + s * n + i);
+            a.x += v.x; a.y += v.y; a.z += v.z; a.w += v.w;
         }
-        __syncthreads();
-        for (int l = threadIdx.x; l < L; l += 256) glam[l] = lambda_grad(lam_s, dot_s, L, l);
-        return;
+        dot = fmaf(a.x, p.x, fmaf(a.y, p.y, fmaf(a.z, p.z, a.w * p.w)));
+        const float c = coef[l];
+        *reinterpret_cast<float4*>(gW + i) = make_float4(a.x * c, a.y * c, a.z * c, a.w * c);
     }
-    const long long i = ((long long)blockIdx.x * 256 + threadIdx.x) * 4;
-    if (i >= n) return;
-    float4 a = *reinterpret_cast<const float4*>(part + i);
-    for (int s = 1; s < splits; ++s) {
-        const float4 v = *reinterpret_cast<const float4*>(part + s * n + i);
-        a.x += v.x; a.y += v.y; a.z += v.z; a.w += v.w;
+    __shared__ float lam_s[128], dot_s[128];
+    if (last_with_dots(dot, dot_part, blockIdx.x, gridDim.x, done)) {
+        sum_dots(lam, dot_part, per_layer, L, lam_s, dot_s);
+        for (int k = threadIdx.x; k < L; k += 256) glam[k] = lambda_grad(lam_s, dot_s, L, k);
     }
-    const float c = coef[i / dr];
-    *reinterpret_cast<float4*>(gW + i) = make_float4(a.x * c, a.y * c, a.z * c, a.w * c);
 }
 __device__ __forceinline__ void lambda_update(const FinalizeParams& f, int l, float g) {
     const long long i = f.lay.lam + l;
@@ -702,17 +733,19 @@ __global__ void __launch_bounds__(256, 5) finalize_cls_kernel(FinalizeParams f) 
     // block 0 takes dlambda and the loss (scheduled first, so it runs at once), the next rest_blocks blocks the
     // head parameters, the remaining wd_blocks blocks W_down
     const int blk = (int)blockIdx.x - 1;
-    const long long i_wd = ((long long)(blk - f.rest_blocks) * blockDim.x + threadIdx.x) * 4;
-    const bool wd_thread = blk >= f.rest_blocks && i_wd < lay.lam;
+    const int l_wd = blk >= f.rest_blocks ? (blk - f.rest_blocks) / f.wd_per_layer : 0;
+    const int o_wd = ((blk - f.rest_blocks - l_wd * f.wd_per_layer) * (int)blockDim.x + (int)threadIdx.x) * 4;      // inside the layer
+    const long long i_wd = (long long)l_wd * f.wd_layer_elems + o_wd;
+    const bool wd_thread = blk >= f.rest_blocks && o_wd < f.wd_layer_elems;
     float4 p4 = make_float4(0.f, 0.f, 0.f, 0.f), m4 = p4, v4 = p4;
-    const int l_wd = wd_thread ? wd_layer(i_wd, lay.lam, (unsigned)(f.d * f.r)) : 0;
+    if (wd_thread && f.coef && !f.adam) p4 = *reinterpret_cast<const float4*>(f.params_in + i_wd);
     if (wd_thread && f.adam) {
         p4 = *reinterpret_cast<const float4*>(f.params + i_wd);
         m4 = *reinterpret_cast<const float4*>(f.m + i_wd);
         v4 = *reinterpret_cast<const float4*>(f.v + i_wd);
     }
     // Block 0: the mean loss needs only what the forward half left behind, which is complete whenever this kernel runs
-    // (see above), so a loss that goes straight to host memory is on its way long before the step ends; dlambda comes last.
+    // (see above), so a loss that goes straight to host memory is on its way long before the step ends.
     // Set by a wait that ran out in this step's forward half or in any earlier step since the last
     // pac_sync (the forward half has completed whenever this kernel runs); a wait that runs out in this
     // step's second pass is seen by the W_down blocks behind their own wait below.
@@ -740,27 +773,16 @@ __global__ void __launch_bounds__(256, 5) finalize_cls_kernel(FinalizeParams f) 
                 }
             }
         }
-        // dlambda: warp per layer, lanes over its partial sums, fixed shuffle order
-        __shared__ float lam_s[MID_MAX_L], dot_s[MID_MAX_L];
-        const bool dots = f.dot_part != nullptr;
-        if (dots && threadIdx.x < f.L) lam_s[threadIdx.x] = f.params_in[lay.lam + threadIdx.x];
-        if (dots) pdl_wait();                            // the partial sums of P_l come from the second pass
-        const float* parts = dots ? f.dot_part : f.lam_part;
-        const int np = dots ? f.dot_n : f.lam_blocks;
-        for (int l = warp; l < f.L; l += nw) {
+        // dlambda where it does not come from the W_down blocks: warp per layer, lanes over its partial sums, fixed shuffle order
+        for (int l = warp; l < f.L && !f.coef && !dead; l += nw) {
             float acc = 0.f;
-            if (parts) {
-                for (int k = lane; k < np; k += 32) acc += parts[(long long)l * np + k];
+            if (f.lam_part) {
+                for (int k = lane; k < f.lam_blocks; k += 32) acc += f.lam_part[(long long)l * f.lam_blocks + k];
                 acc = warp_sum(acc);
             } else {
                 acc = f.grads[lay.lam + l];
             }
-            if (lane == 0 && dots) dot_s[l] = acc;
-            if (lane == 0 && !dots && !dead) lambda_update(f, l, acc);
-        }
-        if (dots) {
-            __syncthreads();
-            if (threadIdx.x < f.L && !status_timed_out(f.status)) lambda_update(f, threadIdx.x, lambda_grad(lam_s, dot_s, f.L, threadIdx.x));
+            if (lane == 0) lambda_update(f, l, acc);
         }
         return;
     }
@@ -832,25 +854,36 @@ __global__ void __launch_bounds__(256, 5) finalize_cls_kernel(FinalizeParams f) 
     {
         // W_down block, four consecutive elements per thread
         const long long i = i_wd;
-        if (i >= lay.lam || status_timed_out(f.status)) return;
-        float4 g4;
-        if (f.splits >= 1) {
-            g4 = *reinterpret_cast<const float4*>(f.dw_part + i);
-            for (int j = 1; j < f.splits; ++j) {                 // split order
-                const float4 q = *reinterpret_cast<const float4*>(f.dw_part + (long long)j * f.dw_elems + i);
-                g4.x += q.x; g4.y += q.y; g4.z += q.z; g4.w += q.w;
+        if (status_timed_out(f.status)) return;
+        float dot = 0.f;
+        if (wd_thread) {
+            float4 g4;
+            if (f.splits >= 1) {
+                g4 = *reinterpret_cast<const float4*>(f.dw_part + i);
+                for (int j = 1; j < f.splits; ++j) {                 // split order
+                    const float4 q = *reinterpret_cast<const float4*>(f.dw_part + (long long)j * f.dw_elems + i);
+                    g4.x += q.x; g4.y += q.y; g4.z += q.z; g4.w += q.w;
+                }
+                if (f.coef) {
+                    dot = fmaf(g4.x, p4.x, fmaf(g4.y, p4.y, fmaf(g4.z, p4.z, g4.w * p4.w)));
+                    const float c = f.coef[l_wd];
+                    g4.x *= c; g4.y *= c; g4.z *= c; g4.w *= c;
+                }
+                *reinterpret_cast<float4*>(f.grads + i) = g4;
+            } else {
+                g4 = *reinterpret_cast<const float4*>(f.grads + i);
             }
-            if (f.coef) {
-                const float c = f.coef[l_wd];
-                g4.x *= c; g4.y *= c; g4.z *= c; g4.w *= c;
+            if (f.adam) {
+                g4.x *= f.grad_scale; g4.y *= f.grad_scale; g4.z *= f.grad_scale; g4.w *= f.grad_scale;
+                adamw_w_down4_loaded(f.params, f.m, f.v, i, l_wd, p4, m4, v4, g4, f.hp, f.bc1, f.bc2, f.wdT, f.d, f.r);
             }
-            *reinterpret_cast<float4*>(f.grads + i) = g4;
-        } else {
-            g4 = *reinterpret_cast<const float4*>(f.grads + i);
         }
-        if (f.adam) {
-            g4.x *= f.grad_scale; g4.y *= f.grad_scale; g4.z *= f.grad_scale; g4.w *= f.grad_scale;
-            adamw_w_down4_loaded(f.params, f.m, f.v, i, l_wd, p4, m4, v4, g4, f.hp, f.bc1, f.bc2, f.wdT, f.d, f.r);
+        if (f.coef) {
+            __shared__ float lam_s[MID_MAX_L], dot_s[MID_MAX_L];
+            if (last_with_dots(dot, f.dot_part, blk - f.rest_blocks, f.wd_blocks, f.done)) {
+                sum_dots(f.params_in + lay.lam, f.dot_part, f.wd_per_layer, f.L, lam_s, dot_s);
+                if (threadIdx.x < f.L) lambda_update(f, threadIdx.x, lambda_grad(lam_s, dot_s, f.L, threadIdx.x));
+            }
         }
         return;
     }

@@ -515,8 +515,6 @@ struct BwdParams {
     int gen;
     const uint8_t* tc;                     // [max_rows][r]
     const bf16* da; long long da_term, da_sample; int da_token;      // strides in elements
-    const float* w;                        // fp32 W_down [L][d][r] for
-    float* dot_part;                       // [L][d_groups][J]: this CTA's share of <out, W_down^l>
     float* out;                            // splits == 1 and not gen: dW_down [L][d][r]; else partials [J][L][d][r]
     unsigned* status;
     unsigned long long* stamp;             // optional stream-phase timestamps (see stamp_begin)
@@ -544,7 +542,6 @@ dw_down_tc_kernel(const __grid_constant__ CUtensorMap map_cache, const __grid_co
     const uint32_t stage_bytes = a_bytes + b_bytes, tx_bytes = GEN ? a_bytes : stage_bytes;
     constexpr bool side = GT == 2 && GQ <= 2;                      // the terms side by side along N, added up in the epilogue
     const int n_cols = side ? 128 * p.r_blocks : r_pad;            // TMEM columns per accumulator
-    __shared__ float dot_s[DW_GEN_WARPS];
     __shared__ __align__(8) unsigned long long bars[2 * 16 + 2];
     __shared__ uint32_t tmem_base_sh;
     __shared__ int abort_sh;
@@ -738,67 +735,37 @@ dw_down_tc_kernel(const __grid_constant__ CUtensorMap map_cache, const __grid_co
                 for (int k = 0; k < AHEAD; ++k)
                     if (ok && rt + k < rt1) ok = build(t4[k], d4[k]);
         }
-        // ---- out (zeros for a split without rows), and its share of <out, W_down>: (column block, 16 columns) units, W_down requested two
-        // units ahead, the first two before the accumulators are complete ----
-        const int steps = (p.r - e16 + 31) >> 5, units = p.chunks * steps;
-        float dot = 0.f;
-        float4 w[2][4];
-        auto load_w = [&](int u, float4 (&x)[4]) {
-            const int c = u / steps, k = col0 + c * 128 + q * 32 + lane;
-            const float4* src = reinterpret_cast<const float4*>(p.w + ((long long)l * p.d + k) * p.r + e16 + 32 * (u - c * steps));
-#pragma unroll
-            for (int e = 0; e < 4; ++e) x[e] = GEN && u < units && k < p.d ? __ldcg(src + e) : make_float4(0.f, 0.f, 0.f, 0.f);
-        };
-        auto finish = [&](int u, const float4 (&x)[4]) {
-            const int c = u / steps, c0 = e16 + 32 * (u - c * steps), k = col0 + c * 128 + q * 32 + lane;     // column of h = row of dW_down
-            float v[16] = {};
-            if (rt0 < rt1) {
-                const uint32_t taddr = tq + (uint32_t)(c * n_cols + c0);
-                tmem_ld16(taddr, v);
-                if (side) {
-                    float v2[16];
-                    tmem_ld16(taddr + (uint32_t)(64 * p.r_blocks), v2);
-                    tmem_ld_wait();
-#pragma unroll
-                    for (int e = 0; e < 16; ++e) v[e] += v2[e];
-                } else {
-                    tmem_ld_wait();
-                }
-            }
-            if (k >= p.d) return;
-            float* dst = p.out + (((long long)j * p.L + l) * p.d + k) * p.r + c0;
-            // (16-byte stores: with 32-byte ones here the step measured 0.4 us slower)
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                *reinterpret_cast<float4*>(dst + 4 * e) = make_float4(v[4 * e], v[4 * e + 1], v[4 * e + 2], v[4 * e + 3]);
-                if (GEN) dot = fmaf(v[4 * e], x[e].x, fmaf(v[4 * e + 1], x[e].y, fmaf(v[4 * e + 2], x[e].z, fmaf(v[4 * e + 3], x[e].w, dot))));
-            }
-        };
-        if (steps > 0) { load_w(0, w[0]); load_w(1, w[1]); }
+        // ---- out (zeros for a split without rows) ----
         if (rt0 < rt1) {
             ok = ok && mbar_wait_warp(accf, 0, abort_flag, p.status);
             tc_fence_after();
             if (threadIdx.x == 64 && ok) stamp_end(p.stamp);
         }
-        if (ok && steps > 0)
-            for (int u = 0; u < units; u += 2) {
-                finish(u, w[0]);
-                load_w(u + 2, w[0]);
-                if (u + 1 < units) finish(u + 1, w[1]);
-                load_w(u + 3, w[1]);
-            }
-        if (GEN) {
+        if (ok)
+            for (int c = 0; c < p.chunks; ++c) {
+                const int k = col0 + c * 128 + q * 32 + lane;     // column of h = row of dW_down
+                for (int c0 = e16; c0 < p.r; c0 += 32) {
+                    float v[16] = {};
+                    if (rt0 < rt1) {
+                        const uint32_t taddr = tq + (uint32_t)(c * n_cols + c0);
+                        tmem_ld16(taddr, v);
+                        if (side) {
+                            float v2[16];
+                            tmem_ld16(taddr + (uint32_t)(64 * p.r_blocks), v2);
+                            tmem_ld_wait();
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
-            if (lane == 0) dot_s[warp - 2] = dot;
-            asm volatile("bar.sync 1, %0;" ::"n"(32 * DW_GEN_WARPS) : "memory");
-            if (threadIdx.x == 64) {
-                float t = 0.f;
+                            for (int e = 0; e < 16; ++e) v[e] += v2[e];
+                        } else {
+                            tmem_ld_wait();
+                        }
+                    }
+                    if (k >= p.d) continue;
+                    float* dst = p.out + (((long long)j * p.L + l) * p.d + k) * p.r + c0;
+                    // (16-byte stores: with 32-byte ones here the step measured 0.4 us slower)
 #pragma unroll
-                for (int i = 0; i < DW_GEN_WARPS; ++i) t += dot_s[i];
-                p.dot_part[((long long)l * p.d_groups + g) * p.splits + j] = t;
+                    for (int e = 0; e < 16; e += 4) *reinterpret_cast<float4*>(dst + e) = make_float4(v[e], v[e + 1], v[e + 2], v[e + 3]);
+                }
             }
-        }
     }
     tc_fence_before();
     __syncthreads();
@@ -1019,7 +986,7 @@ inline int tensor_splits(const TensorPlan& tp, int B) {
 }
 
 // What the second pass builds du from (BwdParams).
-struct DuGen { const uint8_t* tc; const bf16* da; long long da_term, da_sample; int da_token; const float* w; float* dot_part; };
+struct DuGen { const uint8_t* tc; const bf16* da; long long da_term, da_sample; int da_token; };
 
 // With reduce_splits == false and more than one split, and always when du is generated, the partial sums stay in `part`
 // ([J][L][d][r]) for the caller's own reduction.
@@ -1027,7 +994,7 @@ inline pac_status tensor_dw_down(TensorPlan& tp, cudaStream_t stream, const int*
                                  float* dW, float* part, bool reduce_splits, unsigned* status, long long* launches,
                                  unsigned long long* stamp = nullptr, bool early_ids = false, const DuGen* gen = nullptr) {
     BwdParams p = tp.bp;
-    if (p.gen) { p.tc = gen->tc; p.da = gen->da; p.da_term = gen->da_term; p.da_sample = gen->da_sample; p.da_token = gen->da_token; p.w = gen->w; p.dot_part = gen->dot_part; }
+    if (p.gen) { p.tc = gen->tc; p.da = gen->da; p.da_term = gen->da_term; p.da_sample = gen->da_sample; p.da_token = gen->da_token; }
     p.ids = d_ids; p.B = B; p.status = status; p.stamp = stamp; p.early_ids = early_ids ? 1 : 0;
     const int J = tensor_splits(tp, B);
     p.splits = J;
