@@ -14,7 +14,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 LIB = os.path.join(HERE, "libpac_b200.so")
 SOURCES = [os.path.join(HERE, "csrc", "pac_api.cu")]
-HEADERS = [os.path.join(HERE, "csrc", f) for f in ("pac_common.cuh", "pac_simt.cuh", "pac_tensor.cuh", "pac_mid.cuh", "pac_fused_fwd.cuh", "pac_gemm.cuh", "pac_quant.cuh", "pac_chain_fwd.cuh", "pac_tbody.cuh", "pac_sgemm.cuh", "pac_tbody_fused.cuh")] + \
+HEADERS = [os.path.join(HERE, "csrc", f) for f in ("pac_common.cuh", "pac_simt.cuh", "pac_tensor.cuh", "pac_mid.cuh", "pac_fused_fwd.cuh", "pac_gemm.cuh", "pac_quant.cuh", "pac_chain_fwd.cuh", "pac_tbody.cuh", "pac_xgemm.cuh", "pac_tbody_fused.cuh")] + \
           [os.path.join(ROOT, "include", "pac.h")]
 
 

@@ -20,7 +20,7 @@
 #include "pac_gemm.cuh"
 #include "pac_quant.cuh"
 #include "pac_tbody.cuh"
-#include "pac_sgemm.cuh"
+#include "pac_xgemm.cuh"
 #include "pac_tbody_fused.cuh"
 
 using namespace pac;
@@ -367,49 +367,39 @@ pac_status stage_ids(pac_ctx* c, const int* ids, int B, const char* who) {
 // ---------------------------------------------------------------------------
 // Forward: u_l for every layer, the chain, and the head.  ids are on the device.
 // ---------------------------------------------------------------------------
-// out[z] = rows(z) W[z] in fp32.  Tile widths follow N (a 64-wide tile of N = 16 would multiply 48 columns of zeros);
-// few 64-row tiles: 32-row tiles, so that the same work spreads over twice the CTAs.
+// out[z] = rows(z) W[z] at fp32 precision.
 template <class AL>
-pac_status sgemm_rows(pac_ctx* c, int M, int N, int K, int Z, const AL& A, const SgRows& W, float* out, long long zstride) {
-    auto grid = [&](int bm, int bn) { return dim3(cdiv(N, bn), cdiv(M, bm), (unsigned)Z); };
-    cudaStream_t st = c->stream;
-    if (N <= 16) sgemm_rows_kernel<32, 16, 2, 2><<<grid(32, 16), 128, 0, st>>>(M, N, K, A, W, out, zstride);
-    else if (N <= 32 || (N > 64 && N <= 96)) sgemm_rows_kernel<64, 32, 4, 4><<<grid(64, 32), 128, 0, st>>>(M, N, K, A, W, out, zstride);
-    else if ((long long)cdiv(N, 64) * cdiv(M, 64) * Z < c->sms) sgemm_rows_kernel<32, 64, 4, 4><<<grid(32, 64), 128, 0, st>>>(M, N, K, A, W, out, zstride);
-    else sgemm_rows_kernel<64, 64, 8, 4><<<grid(64, 64), 128, 0, st>>>(M, N, K, A, W, out, zstride);
-    LAUNCH_CHECK(c);
+pac_status xgemm_rows(pac_ctx* c, int M, int N, int K, int Z, const AL& A, const XgRows& W, float* out, long long zstride) {
+    XgJobs<AL> J;
+    J.tile_j = xg_tile_j(N);
+    J.add(A, M, W, N, 0);
+    cudaError_t e = xgemm_launch<false>(J, K, Z, 1, out, zstride, 0, c->status, c->stream);
+    c->launches++;
+    if (e != cudaSuccess) return fail(c, PAC_ERR_CUDA, "product kernel launch failed: %s", cudaGetErrorString(e));
+    return PAC_OK;
+}
+// The jobs' A^T B over M rows for all Z layers, `slices` row slices (partial sums part_stride apart when more than one).
+template <class AL>
+pac_status xgemm_tn(pac_ctx* c, const XgJobs<AL>& J, int M, int Z, int slices, float* out, long long zstride, long long part_stride) {
+    cudaError_t e = xgemm_launch<true>(J, M, Z, slices, out, zstride, part_stride, c->status, c->stream);
+    c->launches++;
+    if (e != cudaSuccess) return fail(c, PAC_ERR_CUDA, "product kernel launch failed: %s", cudaGetErrorString(e));
     return PAC_OK;
 }
 
-// Tile of the A^T B products whose output is N wide.
-void tn_tile(int N, int* bi, int* bj) { *bi = 64; *bj = N <= 16 ? 16 : (N <= 32 || (N > 64 && N <= 96)) ? 32 : 64; }
-
-// The jobs' products over M rows for all Z layers, `slices` row slices (partial sums part_stride apart when more than one).
-template <class AL>
-pac_status sgemm_tn(pac_ctx* c, const TnJobs<AL>& J, int M, int Z, int slices, float* out, long long zstride, long long part_stride) {
-    const int m_slice = (int)cdiv(cdiv(M, slices), TN_KR) * TN_KR;
-    dim3 grid((unsigned)J.first[J.n], (unsigned)Z, (unsigned)slices);
-    cudaStream_t st = c->stream;
-    if (J.tile_j == 16) sgemm_tn_kernel<64, 16, 4, 2><<<grid, 128, 0, st>>>(J, M, m_slice, out, zstride, part_stride);
-    else if (J.tile_j == 32) sgemm_tn_kernel<64, 32, 4, 4><<<grid, 128, 0, st>>>(J, M, m_slice, out, zstride, part_stride);
-    else sgemm_tn_kernel<64, 64, 8, 4><<<grid, 128, 0, st>>>(J, M, m_slice, out, zstride, part_stride);
-    LAUNCH_CHECK(c);
-    return PAC_OK;
-}
-
-SgRows sg_rows(const float* base, long long zstride, int ld) {
-    return SgRows{base, zstride, ld, ((uintptr_t)base & 15) == 0 && zstride % 4 == 0 && ld % 4 == 0};
+XgRows xg_rows(const float* base, long long zstride, int ld) {
+    return XgRows{base, zstride, ld, ((uintptr_t)base & 15) == 0 && zstride % 4 == 0 && ld % 4 == 0};
 }
 template <typename T>
-SgCacheRows<T> sg_cache_rows(const pac_ctx* c, const int* d_ids) {
+XgCacheRows<T> xg_cache_rows(const pac_ctx* c, const int* d_ids) {
     const Dims& dm = c->dm;
-    return SgCacheRows<T>{(const T*)c->cache, d_ids, dm.N, dm.L, dm.S, dm.d, dm.d % 4 == 0};
+    return XgCacheRows<T>{(const T*)c->cache, d_ids, dm.N, dm.L, dm.S, dm.d, (dm.d * (int)sizeof(T)) % 16 == 0};
 }
 
 template <typename T>
 pac_status down_projection_simt(pac_ctx* c, const int* d_ids, int B) {
     const Dims& dm = c->dm;
-    return sgemm_rows(c, B * dm.S, dm.r, dm.d, dm.L, sg_cache_rows<T>(c, d_ids), sg_rows(c->params + c->lay.w_down, (long long)dm.d * dm.r, dm.r),
+    return xgemm_rows(c, B * dm.S, dm.r, dm.d, dm.L, xg_cache_rows<T>(c, d_ids), xg_rows(c->params + c->lay.w_down, (long long)dm.d * dm.r, dm.r),
                       c->sc.u, (long long)c->max_rows * dm.r);
 }
 
@@ -532,23 +522,21 @@ pac_status forward(pac_ctx* c, const int* d_ids, int B, bool train, float* d_log
     return PAC_OK;
 }
 
-// Row slices of the plain path's dW_down (partial sums in sc.dw_spart when more than one).
+// Tiles of the plain path's dW_down, and its row slices (partial sums in sc.dw_spart when more than one).
+long long dw_simt_tiles(const Dims& dm) { return (long long)dm.L * cdiv(dm.d, XG_TILE) * cdiv(dm.r, xg_tile_j(dm.r)); }
 int dw_simt_slices(const pac_ctx* c, int B) {
-    const Dims& dm = c->dm;
-    int bi, bj;
-    tn_tile(dm.r, &bi, &bj);
-    return c->sc.dw_spart ? tn_slices((long long)dm.L * cdiv(dm.d, bi) * cdiv(dm.r, bj), B * dm.S, c->sms, c->dw_simt_max) : 1;
+    return c->sc.dw_spart ? xg_slices(dw_simt_tiles(c->dm), B * c->dm.S, c->sms, c->dw_simt_max) : 1;
 }
 
 template <typename T>
 pac_status dw_down_simt(pac_ctx* c, const int* d_ids, int B, bool reduce_splits) {
     const Dims& dm = c->dm;
-    TnJobs<SgCacheRows<T>> J;
-    tn_tile(dm.r, &J.tile_i, &J.tile_j);
-    J.add(sg_cache_rows<T>(c, d_ids), dm.d, sg_rows(c->sc.du, (long long)c->max_rows * dm.r, dm.r), dm.r, 0);
+    XgJobs<XgCacheRows<T>> J;
+    J.tile_j = xg_tile_j(dm.r);
+    J.add(xg_cache_rows<T>(c, d_ids), dm.d, xg_rows(c->sc.du, (long long)c->max_rows * dm.r, dm.r), dm.r, 0);
     const int slices = dw_simt_slices(c, B);
     const long long ne = (long long)dm.L * dm.d * dm.r;
-    pac_status st = sgemm_tn(c, J, B * dm.S, dm.L, slices, slices > 1 ? c->sc.dw_spart : c->grads + c->lay.w_down, (long long)dm.d * dm.r, ne);
+    pac_status st = xgemm_tn(c, J, B * dm.S, dm.L, slices, slices > 1 ? c->sc.dw_spart : c->grads + c->lay.w_down, (long long)dm.d * dm.r, ne);
     if (st != PAC_OK || slices == 1 || !reduce_splits) return st;
     reduce_splits_kernel<<<cdiv(ne / 4, 256), 256, 0, c->stream>>>(c->sc.dw_spart, slices, ne, c->grads + c->lay.w_down);
     LAUNCH_CHECK(c);
@@ -599,12 +587,12 @@ pac_status backward(pac_ctx* c, const int* d_ids, int B, float* d_loss, const pa
         };
         // dW_up = a_L^T dy
         {
-            TnJobs<SgRows> J;
-            tn_tile(dm.d, &J.tile_i, &J.tile_j);
-            J.add(sg_rows(aL, 0, dm.r), dm.r, sg_rows(sc.dy, 0, dm.d), dm.d, 0);
+            XgJobs<XgRows> J;                      // (dy^T a_L, stored transposed: 128 columns of d to a tile)
+            J.tile_j = xg_tile_j(dm.r); J.trans = 1;
+            J.add(xg_rows(sc.dy, 0, dm.d), dm.d, xg_rows(aL, 0, dm.r), dm.r, 0);
             const long long ne = (long long)dm.r * dm.d;
-            const int sl = sc.lm_part && ne % 4 == 0 ? tn_slices(J.first[1], M, c->sms, LM_MAX_K_SLICES) : 1;
-            pac_status ts = sgemm_tn(c, J, M, 1, sl, sl > 1 ? sc.lm_part : c->grads + c->lay.w_up, 0, ne);
+            const int sl = sc.lm_part && ne % 4 == 0 ? xg_slices(J.first[1], M, c->sms, LM_MAX_K_SLICES) : 1;
+            pac_status ts = xgemm_tn(c, J, M, 1, sl, sl > 1 ? sc.lm_part : c->grads + c->lay.w_up, 0, ne);
             if (ts != PAC_OK) return ts;
             if (sl > 1) {
                 sum_slices_kernel<<<cdiv(ne / 4, 256), 256, 0, c->stream>>>(sc.lm_part, sl, ne, c->grads + c->lay.w_up);
@@ -752,14 +740,14 @@ pac_status tb_fused_backward(pac_ctx* c, int B) {
     LAUNCH_CHECK(c);
     // dW = A^T B over all rows, all six products of all layers at once
     const long long rr = (long long)r * r, rf = (long long)r * f, per = 4 * rr + 2 * rf;
-    TnJobs<SgRows> J;
-    tn_tile(r, &J.tile_i, &J.tile_j);
-    for (int k = 0; k < 3; ++k) J.add(sg_rows(s.n1, s.sMr, r), r, sg_rows(s.dqkv + k * s.sMr, 3 * s.sMr, r), r, k * rr);
-    J.add(sg_rows(s.o, s.sMr, r), r, sg_rows(s.dx1, s.sMr, r), r, 3 * rr);
-    J.add(sg_rows(s.n2, s.sMr, r), r, sg_rows(s.dpre, s.sMf, f), f, 4 * rr);
-    J.add(sg_rows(s.hid, s.sMf, f), f, sg_rows(s.da, s.sMr, r), r, 4 * rr + rf);
-    const int slices = tn_slices((long long)J.first[J.n] * L, M, c->sms, t.wg_slices);
-    pac_status st = sgemm_tn(c, J, M, L, slices, t.wg_part, per, per * L);
+    XgJobs<XgRows> J;
+    J.tile_j = xg_tile_j(r);
+    for (int k = 0; k < 3; ++k) J.add(xg_rows(s.n1, s.sMr, r), r, xg_rows(s.dqkv + k * s.sMr, 3 * s.sMr, r), r, k * rr);
+    J.add(xg_rows(s.o, s.sMr, r), r, xg_rows(s.dx1, s.sMr, r), r, 3 * rr);
+    J.add(xg_rows(s.n2, s.sMr, r), r, xg_rows(s.dpre, s.sMf, f), f, 4 * rr);
+    J.add(xg_rows(s.hid, s.sMf, f), f, xg_rows(s.da, s.sMr, r), r, 4 * rr + rf);
+    const int slices = xg_slices((long long)J.first[J.n] * L, M, c->sms, t.wg_slices);
+    pac_status st = xgemm_tn(c, J, M, L, slices, t.wg_part, per, per * L);
     if (st != PAC_OK) return st;
     tb_reduce_slices_kernel<<<dim3(cdiv(per, 256), (unsigned)L), 256, 0, c->stream>>>(t.wg_part, slices, per * L, per, bl, gbody);
     LAUNCH_CHECK(c);
@@ -1528,9 +1516,9 @@ pac_status pac_adapter_init(pac_ctx* c, const pac_adapter_cfg* cfg, unsigned lon
     if (st == PAC_OK && !use_tensor(c)) {
         A(dmalloc(c, &s.du, Mr * dm.L));    // the plain path keeps du in fp32
         const long long ne = (long long)dm.L * dm.d * dm.r;
-        int bi, bj;
-        tn_tile(dm.r, &bi, &bj);
-        c->dw_simt_max = ne % 4 == 0 ? tn_slices((long long)dm.L * cdiv(dm.d, bi) * cdiv(dm.r, bj), c->max_rows, c->sms, 8) : 1;
+        // (a smaller batch may take more slices than the largest one)
+        c->dw_simt_max = 1;
+        for (int b = 1; b <= cfg->max_batch && ne % 4 == 0; ++b) c->dw_simt_max = std::max(c->dw_simt_max, xg_slices(dw_simt_tiles(dm), b * dm.S, c->sms, 8));
         if (c->dw_simt_max > 1) A(dmalloc(c, &s.dw_spart, ne * c->dw_simt_max));
     }
     if (st == PAC_OK && c->tb.on) {

@@ -53,6 +53,20 @@ inline cudaError_t smem_opt_in(const void* kernel, size_t bytes) {
     return e;
 }
 
+__device__ __forceinline__ uint32_t bf16_pair(float lo, float hi) {
+    uint32_t d;
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(hi), "f"(lo));
+    return d;
+}
+// (x, y) = h + m + l exactly, each term a bf16 pair.
+__device__ __forceinline__ void split3_pair(float x, float y, uint32_t& h, uint32_t& m, uint32_t& l) {
+    h = bf16_pair(x, y);
+    x -= __uint_as_float(h << 16); y -= __uint_as_float(h & 0xffff0000u);
+    m = bf16_pair(x, y);
+    x -= __uint_as_float(m << 16); y -= __uint_as_float(m & 0xffff0000u);
+    l = bf16_pair(x, y);
+}
+
 // bf16 terms of W_down for the tensor-core products, [L][terms][d][r] in the master's order: term 0 = bf16(W), term 1 = bf16(W -
 // term 0), ...; two terms carry about 16 mantissa bits, three the fp32 value exactly.
 struct WdShadow {

@@ -5,7 +5,7 @@
 // q, k, v of layer i; launch l of the backward pass runs dk, dv, LayerNorm 1 and the merge of layer l + 1 and
 // then feed-forward, LayerNorm 2, do and dq of layer l.  A CTA owns 16 tokens of one sample from end to end;
 // what it needs of the sample's other tokens (k, v; in reverse q, do, P, dS) was written by the launch before.
-// The weight gradients A^T B over all rows follow in one launch for all layers (sgemm_tn_kernel).
+// The weight gradients A^T B over all rows follow in one launch for all layers (xgemm_kernel).
 //
 // Products at fp32 precision on the warp-level tensor instructions: 16 tokens are one m16 tile, far below the 128
 // rows of a tcgen05 tile, and a CTA's products are short and serial.  Every fp32 operand is the exact sum of three bf16 terms
@@ -106,19 +106,6 @@ struct TbLayerParams {
 // ---------------------------------------------------------------------------
 // Three-term operands
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ uint32_t tb_pack2(float lo, float hi) {
-    uint32_t d;
-    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(hi), "f"(lo));
-    return d;
-}
-// (x, y) = h + m + l, each term a bf16 pair.
-__device__ __forceinline__ void tb_split2(float x, float y, uint32_t& h, uint32_t& m, uint32_t& l) {
-    h = tb_pack2(x, y);
-    x -= __uint_as_float(h << 16); y -= __uint_as_float(h & 0xffff0000u);
-    m = tb_pack2(x, y);
-    x -= __uint_as_float(m << 16); y -= __uint_as_float(m & 0xffff0000u);
-    l = tb_pack2(x, y);
-}
 __device__ __forceinline__ void tb_mma(float (&c)[4], const uint32_t (&a)[4], const uint32_t (&b)[2]) {
     asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
                  : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
@@ -132,17 +119,17 @@ __device__ __forceinline__ void tb_mma6(float (&c)[4], const TbA& a, const TbB& 
     tb_mma(c, a.h, b.m); tb_mma(c, a.m, b.h); tb_mma(c, a.h, b.h);
 }
 __device__ __forceinline__ void tb_split_b(TbB& b, float k0, float k1, float k8, float k9) {
-    tb_split2(k0, k1, b.h[0], b.m[0], b.l[0]);
-    tb_split2(k8, k9, b.h[1], b.m[1], b.l[1]);
+    split3_pair(k0, k1, b.h[0], b.m[0], b.l[0]);
+    split3_pair(k8, k9, b.h[1], b.m[1], b.l[1]);
 }
 // A tile from fp32 rows in shared memory: p points at (row lane / 4, column 2 (lane % 4)) of the tile.
 __device__ __forceinline__ void tb_split_a(TbA& a, const float* p, int stride) {
     const float2 v0 = *reinterpret_cast<const float2*>(p), v1 = *reinterpret_cast<const float2*>(p + 8 * stride);
     const float2 v2 = *reinterpret_cast<const float2*>(p + 8), v3 = *reinterpret_cast<const float2*>(p + 8 * stride + 8);
-    tb_split2(v0.x, v0.y, a.h[0], a.m[0], a.l[0]);
-    tb_split2(v1.x, v1.y, a.h[1], a.m[1], a.l[1]);
-    tb_split2(v2.x, v2.y, a.h[2], a.m[2], a.l[2]);
-    tb_split2(v3.x, v3.y, a.h[3], a.m[3], a.l[3]);
+    split3_pair(v0.x, v0.y, a.h[0], a.m[0], a.l[0]);
+    split3_pair(v1.x, v1.y, a.h[1], a.m[1], a.l[1]);
+    split3_pair(v2.x, v2.y, a.h[2], a.m[2], a.l[2]);
+    split3_pair(v3.x, v3.y, a.h[3], a.m[3], a.l[3]);
 }
 __device__ __forceinline__ void tb_ldmatrix4(uint32_t (&r)[4], uint32_t addr) {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
@@ -151,13 +138,13 @@ __device__ __forceinline__ void tb_ldmatrix4(uint32_t (&r)[4], uint32_t addr) {
 // into different banks).
 __device__ __forceinline__ void tb_put2(bf16* pl, int stride, int t, int c, float x, float y) {      // columns c, c + 1 (c even)
     uint32_t h, m, l;
-    tb_split2(x, y, h, m, l);
+    split3_pair(x, y, h, m, l);
     uint32_t* q = reinterpret_cast<uint32_t*>(pl + t * stride + c);
     q[0] = h; q[8 * stride] = m; q[16 * stride] = l;
 }
 __device__ __forceinline__ void tb_put1(bf16* pl, int stride, int t, int c, float x) {
     uint32_t h, m, l;
-    tb_split2(x, 0.f, h, m, l);
+    split3_pair(x, 0.f, h, m, l);
     uint16_t* q = reinterpret_cast<uint16_t*>(pl + t * stride + c);
     q[0] = (uint16_t)h; q[16 * stride] = (uint16_t)m; q[32 * stride] = (uint16_t)l;
 }
@@ -321,7 +308,7 @@ __device__ __forceinline__ void tb_scores(const float* __restrict__ X, int r, co
                     v[i] = c < dh ? act[(q + ((i >> 1) & 1) * 8) * rs + col + c] : 0.f;
                 }
 #pragma unroll
-                for (int i = 0; i < 4; ++i) tb_split2(v[2 * i], v[2 * i + 1], a.h[i], a.m[i], a.l[i]);
+                for (int i = 0; i < 4; ++i) split3_pair(v[2 * i], v[2 * i + 1], a.h[i], a.m[i], a.l[i]);
             }
 #pragma unroll
             for (int n = 0; n < 4; ++n) {
@@ -747,7 +734,7 @@ __global__ void __launch_bounds__(TBF_THREADS) tb_bwd_kernel(const __grid_consta
                         const float duv = lm * y;
                         if (p.du3) {
                             uint32_t h, m, lo;
-                            tb_split2(duv, 0.f, h, m, lo);
+                            split3_pair(duv, 0.f, h, m, lo);
                             uint16_t* w = reinterpret_cast<uint16_t*>(p.du3) + 3 * l * p.u_stride + m0 * r + e;
                             w[0] = (uint16_t)h; w[p.u_stride] = (uint16_t)m; w[2 * p.u_stride] = (uint16_t)lo;
                         } else {

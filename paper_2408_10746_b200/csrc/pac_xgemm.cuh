@@ -1,0 +1,306 @@
+// Products at fp32 precision on tcgen05, operands converted on the way into shared memory.
+//
+//   rows   out[z][m][j] = sum_k A(z; m, k) B[z][k][j]        (u_l = h_l W_down^l)
+//   tn     out[i][j]    = sum_m A(z; m, i) B[z][m][j]        (dW = A^T B over all token rows)
+//
+// An fp32 operand enters as the exact sum of three bf16 terms (8 + 8 + 8 mantissa bits), a bf16 one as it is.  Of the products of terms those
+// of relative size 2^-16 and above are formed, six or three; the dropped ones, below 2^-25, are smaller than the rounding of one fp32
+// multiplication.  Sums are fp32.  That is 1365 products per clock and SM against 128 on the FP32 pipe, so the kernel is bound
+// by bringing the operands in: A comes straight from the activation cache (the gather is the address; any row length and alignment),
+// 16 producer warps fetch it into registers, split it and store the swizzled tiles, one warp issues the MMAs.  The producers work in two
+// teams, each filling one of two stages: a team's loads are in flight while the other converts.
+// The FP32-pipe tiles before it (8 x 4 outputs per thread) took 77 us for u and 84 us for dW_down at 2048 rows, 12 layers, d = 768, r = 64.
+// Every output is summed in a fixed order.
+#pragma once
+#include "pac_common.cuh"
+#include "pac_tensor.cuh"
+
+namespace pac {
+
+// Row m of the minibatch at layer z, straight from the cache.
+template <typename T>
+struct XgCacheRows {
+    typedef T elem;
+    const T* cache; const int* ids; long long N; int L, S, d;
+    bool vec;                                   // rows start on 16-byte boundaries
+    __device__ const T* row(int z, int m) const {
+        const int b = m / S, s = m - b * S;
+        return cache + ((safe_id(ids, b, N, nullptr) * L + z) * S + s) * (long long)d;
+    }
+};
+// Row m of a row-major fp32 stack.
+struct XgRows {
+    typedef float elem;
+    const float* base; long long zstride; int ld;
+    bool vec;                                   // rows start on 16-byte boundaries
+    __device__ const float* row(int z, int m) const { return base + z * zstride + (long long)m * ld; }
+};
+
+constexpr int XG_PRODUCERS = 16, XG_THREADS = 32 * (XG_PRODUCERS + 1), XG_TILE = 128, XG_K = 64, XG_MAX_JOBS = 6, XG_TMEM = 128;
+constexpr uint32_t XG_TERM_A = XG_TILE * XG_K * 2, XG_BOX = 64 * 128;
+
+// Products of one launch: several per layer (tn), all layers.
+template <class AL>
+struct XgJobs {
+    AL A[XG_MAX_JOBS];
+    XgRows B[XG_MAX_JOBS];
+    int mi[XG_MAX_JOBS], nj[XG_MAX_JOBS];       // output extent
+    int tiles_j[XG_MAX_JOBS], first[XG_MAX_JOBS + 1];
+    long long out_off[XG_MAX_JOBS];
+    int n = 0;
+    int tile_j = 16;                            // columns per tile, a multiple of 16 up to 128
+    int trans = 0;                              // 1: out[j][i]
+    void add(const AL& a, int mi_, const XgRows& b, int nj_, long long off) {
+        A[n] = a; B[n] = b; mi[n] = mi_; nj[n] = nj_; out_off[n] = off;
+        tiles_j[n] = (nj_ + tile_j - 1) / tile_j;
+        if (n == 0) first[0] = 0;
+        first[n + 1] = first[n] + tiles_j[n] * ((mi_ + XG_TILE - 1) / XG_TILE);
+        ++n;
+    }
+};
+
+// Eight consecutive columns of a row, zeros from n on.
+struct XgF8 { float v[8]; };
+__device__ __forceinline__ void xg_load(const float* __restrict__ row, int c, int n, bool vec, XgF8& o) {
+    if (vec && c + 8 <= n) {
+        const float4 a = __ldg(reinterpret_cast<const float4*>(row + c)), b = __ldg(reinterpret_cast<const float4*>(row + c) + 1);
+        o.v[0] = a.x; o.v[1] = a.y; o.v[2] = a.z; o.v[3] = a.w; o.v[4] = b.x; o.v[5] = b.y; o.v[6] = b.z; o.v[7] = b.w;
+    } else {
+#pragma unroll
+        for (int e = 0; e < 8; ++e) o.v[e] = c + e < n ? __ldg(row + c + e) : 0.f;
+    }
+}
+__device__ __forceinline__ void xg_load(const bf16* __restrict__ row, int c, int n, bool vec, uint4& o) {
+    if (vec && c + 8 <= n) {
+        o = __ldg(reinterpret_cast<const uint4*>(row + c));
+    } else {
+        uint32_t w[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const uint32_t lo = c + 2 * e < n ? __ldg(reinterpret_cast<const unsigned short*>(row) + c + 2 * e) : 0;
+            const uint32_t hi = c + 2 * e + 1 < n ? __ldg(reinterpret_cast<const unsigned short*>(row) + c + 2 * e + 1) : 0;
+            w[e] = lo | (hi << 16);
+        }
+        o = make_uint4(w[0], w[1], w[2], w[3]);
+    }
+}
+__device__ __forceinline__ void xg_st(uint32_t a, uint32_t x, uint32_t y, uint32_t z, uint32_t w) {
+    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(a), "r"(x), "r"(y), "r"(z), "r"(w) : "memory");
+}
+__device__ __forceinline__ void xg_store(uint32_t a, uint32_t term, const uint4& v) { xg_st(a, v.x, v.y, v.z, v.w); (void)term; }
+__device__ __forceinline__ void xg_store(uint32_t a, uint32_t term, const XgF8& x) {
+    uint32_t h[4], m[4], l[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) split3_pair(x.v[2 * e], x.v[2 * e + 1], h[e], m[e], l[e]);
+    xg_st(a, h[0], h[1], h[2], h[3]);
+    xg_st(a + term, m[0], m[1], m[2], m[3]);
+    xg_st(a + 2 * term, l[0], l[1], l[2], l[3]);
+}
+template <typename T> struct XgTerms { static constexpr int n = 3; typedef XgF8 reg; };
+template <> struct XgTerms<bf16> { static constexpr int n = 1; typedef uint4 reg; };
+
+__host__ __device__ inline uint32_t xg_term_b(int tile_j) { return (uint32_t)((tile_j + 63) / 64) * XG_BOX; }
+template <class AL>
+inline size_t xg_smem(int tile_j) { return 2 * ((size_t)XgTerms<typename AL::elem>::n * XG_TERM_A + 3 * xg_term_b(tile_j)) + 1024; }
+
+// Grid: (tiles of all jobs, layers, slices of the reduction).  With more than one slice the partial sums of slice s go to
+// out + s * part_stride and are added up in slice order by whoever reads them.  GB: 8-column groups of B per thread (tile_j = 32 GB at most).
+template <bool TN, int GB, class AL>
+__global__ void __launch_bounds__(XG_THREADS, 1)
+xgemm_kernel(const __grid_constant__ XgJobs<AL> J, int K, int k_slice, float* __restrict__ out, long long zstride, long long part_stride, unsigned* status) {
+    typedef typename AL::elem T;
+    constexpr int TA = XgTerms<T>::n;
+    extern __shared__ unsigned char smem_raw[];
+    const uint32_t ring = (smem_u32(smem_raw) + 1023u) & ~1023u;
+    const int nj_tile = J.tile_j;
+    const uint32_t term_b = xg_term_b(nj_tile), stage = TA * XG_TERM_A + 3 * term_b;
+    __shared__ __align__(8) unsigned long long bars[5];
+    __shared__ uint32_t tmem_base_sh;
+    __shared__ int abort_sh;
+    const uint32_t full0 = smem_u32(&bars[0]), empty0 = smem_u32(&bars[2]), accf = smem_u32(&bars[4]);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, z = blockIdx.y;
+    int jb = 0;
+    while (jb + 1 < J.n && (int)blockIdx.x >= J.first[jb + 1]) ++jb;
+    const int tile = blockIdx.x - J.first[jb];
+    const int i0 = tile / J.tiles_j[jb] * XG_TILE, j0 = tile % J.tiles_j[jb] * nj_tile;
+    const int Mi = J.mi[jb], Nj = J.nj[jb];
+    const int kb = blockIdx.z * k_slice, ke = min(K, kb + k_slice), stages = ke > kb ? (ke - kb + XG_K - 1) / XG_K : 0;
+    if (threadIdx.x == 0) {
+        abort_sh = 0;
+        for (int s = 0; s < 2; ++s) { mbar_init(full0 + 8 * s, XG_PRODUCERS / 2); mbar_init(empty0 + 8 * s, 1); }
+        mbar_init(accf, 1);
+        fence_mbar_init();
+    }
+    if (warp == XG_PRODUCERS) { tmem_alloc(smem_u32(&tmem_base_sh), XG_TMEM); tmem_relinquish(); }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_base = tmem_base_sh;
+    volatile int* abort_flag = &abort_sh;
+    pdl_wait();
+    pdl_trigger();      // (not before: a successor may rely on everything ahead of this kernel being complete when it starts)
+    if (warp == XG_PRODUCERS) {
+        const uint32_t idesc = instr_desc_bf16(XG_TILE, nj_tile, TN ? 1 : 0, 1);
+        // (term of A, term of B), small products first
+        constexpr int NP = TA == 3 ? 6 : 3;
+        constexpr int pa[6] = {1, 0, 2, 0, 1, 0}, pb[6] = {1, 2, 0, 1, 0, 0};
+        bool ok = true;
+        for (int it = 0; it < stages && ok; ++it) {
+            const uint32_t s = it & 1u;
+            if (!mbar_wait_uniform(full0 + 8 * s, (it >> 1) & 1u, abort_flag, status)) { ok = false; break; }
+            tc_fence_after();
+            if (elect_one()) {
+                const uint32_t a = ring + s * stage, b = a + TA * XG_TERM_A;
+                const uint64_t ad = TN ? smem_desc_sw128(a, XG_BOX, 1024) : smem_desc_sw128(a, 16, 1024), bd = smem_desc_sw128(b, XG_BOX, 1024);
+#pragma unroll
+                for (int k = 0; k < XG_K / 16; ++k)
+#pragma unroll
+                    for (int p = 0; p < NP; ++p) {
+                        const int ta = TA == 3 ? pa[p] : 0, tb = TA == 3 ? pb[p] : 2 - p;
+                        umma_bf16(tmem_base, ad + (uint64_t)((ta * XG_TERM_A) >> 4) + (uint64_t)(k * (TN ? 128 : 2)),
+                                  bd + (uint64_t)((tb * term_b) >> 4) + (uint64_t)(k * 128), idesc, (it | k | p) ? 1u : 0u);
+                    }
+                umma_commit(empty0 + 8 * s);
+                if (it + 1 == stages) umma_commit(accf);
+            }
+            __syncwarp();
+        }
+    } else {
+        const int team = warp >> 3, t = threadIdx.x & 255;
+        const AL A = J.A[jb];
+        const XgRows B = J.B[jb];
+        typename XgTerms<T>::reg ra[4];
+        XgF8 rb[GB];
+        uint32_t offa[4], offb[GB];
+        int rowa[4], cola[4], rowb[GB], colb[GB];
+        const T* pa[4];
+        const int nb8 = nj_tile >> 3;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int g = t + 256 * i;
+            rowa[i] = TN ? g >> 4 : g >> 3;
+            const int c8 = TN ? g & 15 : g & 7;
+            cola[i] = c8 * 8;
+            offa[i] = (uint32_t)(c8 >> 3) * XG_BOX + (uint32_t)rowa[i] * 128u + (uint32_t)(((c8 & 7) ^ (rowa[i] & 7)) << 4);
+            if (!TN) pa[i] = A.row(z, min(i0 + rowa[i], Mi - 1));
+        }
+#pragma unroll
+        for (int i = 0; i < GB; ++i) {
+            const int g = t + 256 * i;
+            rowb[i] = g / nb8;
+            const int c8 = g - rowb[i] * nb8;
+            colb[i] = j0 + c8 * 8;
+            offb[i] = (uint32_t)(c8 >> 3) * XG_BOX + (uint32_t)rowb[i] * 128u + (uint32_t)(((c8 & 7) ^ (rowb[i] & 7)) << 4);
+            if (rowb[i] >= XG_K) rowb[i] = -1;
+        }
+        auto fetch = [&](int k0) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                // rows beyond the output or the slice read nothing and enter as zeros
+                if (TN) {
+                    const int m = k0 + rowa[i];
+                    xg_load(A.row(z, min(m, ke - 1)), i0 + cola[i], m < ke ? Mi : 0, A.vec, ra[i]);
+                } else {
+                    xg_load(pa[i], k0 + cola[i], i0 + rowa[i] < Mi ? ke : 0, A.vec, ra[i]);
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < GB; ++i)
+                if (rowb[i] >= 0) {
+                    const int k = k0 + rowb[i];
+                    xg_load(B.row(z, min(k, ke - 1)), colb[i], k < ke ? Nj : 0, B.vec, rb[i]);
+                }
+        };
+        bool ok = true;
+        if (team < stages) fetch(kb + team * XG_K);
+        for (int it = team; it < stages; it += 2) {
+            if (!mbar_wait_uniform(empty0 + 8 * team, ((it >> 1) & 1u) ^ 1u, abort_flag, status)) { ok = false; break; }
+            const uint32_t a = ring + team * stage, b = a + TA * XG_TERM_A;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) xg_store(a + offa[i], XG_TERM_A, ra[i]);
+#pragma unroll
+            for (int i = 0; i < GB; ++i)
+                if (rowb[i] >= 0) xg_store(b + offb[i], term_b, rb[i]);
+            fence_proxy_async();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(full0 + 8 * team);
+            if (it + 2 < stages) fetch(kb + (it + 2) * XG_K);
+        }
+        if (stages > 0) {
+            ok = ok && mbar_wait_warp(accf, 0, abort_flag, status);
+            tc_fence_after();
+        }
+        if (ok) {
+            const int q = warp & 3, i = i0 + q * 32 + lane;
+            float* o = out + blockIdx.z * part_stride + z * zstride + J.out_off[jb];
+            const bool vec = !J.trans && (Nj & 3) == 0 && ((uintptr_t)o & 15) == 0;
+            for (int c0 = (warp >> 2) * 16; c0 < nj_tile; c0 += 64) {
+                float v[16] = {};
+                if (stages > 0) { tmem_ld16(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)c0, v); tmem_ld_wait(); }
+                if (i >= Mi) continue;
+#pragma unroll
+                for (int e = 0; e < 16; e += 4) {
+                    const int j = j0 + c0 + e;
+                    if (vec && j < Nj) {
+                        *reinterpret_cast<float4*>(o + (long long)i * Nj + j) = make_float4(v[e], v[e + 1], v[e + 2], v[e + 3]);
+                    } else {
+#pragma unroll
+                        for (int x = 0; x < 4; ++x)
+                            if (j + x < Nj) o[J.trans ? (long long)(j + x) * Mi + i : (long long)i * Nj + j + x] = v[e + x];
+                    }
+                }
+            }
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    drain_after_abort(abort_flag);
+    if (warp == XG_PRODUCERS) tmem_dealloc(tmem_base, XG_TMEM);
+}
+
+template <bool TN, class AL>
+inline cudaError_t xgemm_launch(const XgJobs<AL>& J, int K, int Z, int slices, float* out, long long zstride, long long part_stride, unsigned* status, cudaStream_t stream) {
+    const int k_slice = ((K + slices - 1) / slices + XG_K - 1) / XG_K * XG_K;
+    const auto kernel = J.tile_j <= 64 ? xgemm_kernel<TN, 2, AL> : xgemm_kernel<TN, 4, AL>;
+    const size_t smem = xg_smem<AL>(J.tile_j);
+    cudaError_t e = smem_opt_in((const void*)kernel, smem);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    pdl_launch_config(&cfg, attr, dim3((unsigned)J.first[J.n], (unsigned)Z, (unsigned)slices), dim3(XG_THREADS), smem, stream);
+    return cudaLaunchKernelEx(&cfg, kernel, J, K, k_slice, out, zstride, part_stride, status);
+}
+
+// Columns per tile for an output N wide, tiles of equal width.
+inline int xg_tile_j(int N) {
+    const int tiles = (N + 127) / 128;
+    return ((N + tiles - 1) / tiles + 15) / 16 * 16;
+}
+
+// out[i] = sum_s part[s][i] in slice order (n a multiple of 4).  The gradient blocks behind lambda[L] in the flat vector start
+// on a 16-byte boundary only when L % 4 == 0: vector loads, scalar stores.
+__global__ void __launch_bounds__(256) sum_slices_kernel(const float* __restrict__ part, int slices, long long n, float* __restrict__ out) {
+    const long long i = ((long long)blockIdx.x * blockDim.x + threadIdx.x) * 4;
+    if (i >= n) return;
+    float4 a = *reinterpret_cast<const float4*>(part + i);
+    for (int s = 1; s < slices; ++s) {
+        const float4 v = *reinterpret_cast<const float4*>(part + s * n + i);
+        a.x += v.x; a.y += v.y; a.z += v.z; a.w += v.w;
+    }
+    out[i] = a.x; out[i + 1] = a.y; out[i + 2] = a.z; out[i + 3] = a.w;
+}
+
+// Slices of a reduction over K rows: whole waves of CTAs, each about 2 us plus 0.6 us per stage (measured), and the slices' own traffic.
+inline int xg_slices(long long tiles, int K, int sms, int most) {
+    const int stages = (K + XG_K - 1) / XG_K;
+    int best = 1;
+    double best_cost = 1e30;
+    for (int s = 1; s <= most && s <= stages; ++s) {
+        const double waves = (double)((tiles * s + sms - 1) / sms);
+        const double cost = waves * (2.0 + 0.6 * ((stages + s - 1) / s)) + 0.3 * (s - 1);
+        if (cost < best_cost) { best_cost = cost; best = s; }
+    }
+    return best;
+}
+
+}  // namespace pac
