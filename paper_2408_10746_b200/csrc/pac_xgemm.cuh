@@ -9,7 +9,9 @@
 // by bringing the operands in: A comes straight from the activation cache (the gather is the address; any row length and alignment),
 // 16 producer warps fetch it into registers, split it and store the swizzled tiles, one warp issues the MMAs.  The producers work in two
 // teams, each filling one of two stages: a team's loads are in flight while the other converts.
-// The FP32-pipe tiles before it (8 x 4 outputs per thread) took 77 us for u and 84 us for dW_down at 2048 rows, 12 layers, d = 768, r = 64.
+// At 2048 rows, 12 layers, d = 768, r = 64: u 41 us, dW_down 30 us (the FP32-pipe tiles before it, 8 x 4 outputs per thread: 77 and 84 us).
+// Loads are what it waits for (a third of the issue slots are used); row addresses are therefore formed once per stage (tn) or once per kernel
+// (rows).  Prefetching the stage after next into L2 made the step 8 % slower.
 // Every output is summed in a fixed order.
 #pragma once
 #include "pac_common.cuh"
@@ -172,18 +174,21 @@ xgemm_kernel(const __grid_constant__ XgJobs<AL> J, int K, int k_slice, float* __
         typename XgTerms<T>::reg ra[4];
         XgF8 rb[GB];
         uint32_t offa[4], offb[GB];
-        int rowa[4], cola[4], rowb[GB], colb[GB];
+        int cola[4], rowa = 0, rowb[GB], colb[GB];
         const T* pa[4];
+        const float* pb[GB];
         const int nb8 = nj_tile >> 3;
+        // tn: four threads share a row, so that the row's address is formed once per stage; odd rows take their column groups in another
+        // order, which spreads a quarter-warp's stores over all banks.  rows: four fixed rows.
+        if (TN) rowa = t >> 2;
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            const int g = t + 256 * i;
-            rowa[i] = TN ? g >> 4 : g >> 3;
-            const int c8 = TN ? g & 15 : g & 7;
+            const int row = TN ? rowa : (t + 256 * i) >> 3, c8 = TN ? (t & 3) + 4 * (i ^ (row & 1)) : t & 7;
             cola[i] = c8 * 8;
-            offa[i] = (uint32_t)(c8 >> 3) * XG_BOX + (uint32_t)rowa[i] * 128u + (uint32_t)(((c8 & 7) ^ (rowa[i] & 7)) << 4);
-            if (!TN) pa[i] = A.row(z, min(i0 + rowa[i], Mi - 1));
+            offa[i] = (uint32_t)(c8 >> 3) * XG_BOX + (uint32_t)row * 128u + (uint32_t)(((c8 & 7) ^ (row & 7)) << 4);
+            if (!TN) pa[i] = i0 + row < Mi ? A.row(z, i0 + row) : nullptr;
         }
+        const long long step_b = 2LL * XG_K * B.ld;
 #pragma unroll
         for (int i = 0; i < GB; ++i) {
             const int g = t + 256 * i;
@@ -191,24 +196,25 @@ xgemm_kernel(const __grid_constant__ XgJobs<AL> J, int K, int k_slice, float* __
             const int c8 = g - rowb[i] * nb8;
             colb[i] = j0 + c8 * 8;
             offb[i] = (uint32_t)(c8 >> 3) * XG_BOX + (uint32_t)rowb[i] * 128u + (uint32_t)(((c8 & 7) ^ (rowb[i] & 7)) << 4);
+            pb[i] = B.row(z, kb + team * XG_K + rowb[i]);
             if (rowb[i] >= XG_K) rowb[i] = -1;
         }
+        // rows beyond the output or the slice are not read and enter as zeros
         auto fetch = [&](int k0) {
+            if (TN) {
+                const int m = k0 + rowa;
+                const T* row = A.row(z, min(m, ke - 1));
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                // rows beyond the output or the slice read nothing and enter as zeros
-                if (TN) {
-                    const int m = k0 + rowa[i];
-                    xg_load(A.row(z, min(m, ke - 1)), i0 + cola[i], m < ke ? Mi : 0, A.vec, ra[i]);
-                } else {
-                    xg_load(pa[i], k0 + cola[i], i0 + rowa[i] < Mi ? ke : 0, A.vec, ra[i]);
-                }
+                for (int i = 0; i < 4; ++i) xg_load(row, i0 + cola[i], m < ke ? Mi : 0, A.vec, ra[i]);
+            } else {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) xg_load(pa[i], k0 + cola[i], pa[i] ? ke : 0, A.vec, ra[i]);
             }
 #pragma unroll
             for (int i = 0; i < GB; ++i)
                 if (rowb[i] >= 0) {
-                    const int k = k0 + rowb[i];
-                    xg_load(B.row(z, min(k, ke - 1)), colb[i], k < ke ? Nj : 0, B.vec, rb[i]);
+                    xg_load(pb[i], colb[i], k0 + rowb[i] < ke ? Nj : 0, B.vec, rb[i]);
+                    pb[i] += step_b;
                 }
         };
         bool ok = true;
