@@ -595,7 +595,7 @@ pac_status backward(pac_ctx* c, const int* d_ids, int B, float* d_loss, const pa
             pac_status ts = xgemm_tn(c, J, M, 1, sl, sl > 1 ? sc.lm_part : c->grads + c->lay.w_up, 0, ne);
             if (ts != PAC_OK) return ts;
             if (sl > 1) {
-                sum_slices_kernel<<<cdiv(ne / 4, 256), 256, 0, c->stream>>>(sc.lm_part, sl, ne, c->grads + c->lay.w_up);
+                reduce_splits_kernel<<<cdiv(ne / 4, 256), 256, 0, c->stream>>>(sc.lm_part, sl, ne, c->grads + c->lay.w_up);
                 LAUNCH_CHECK(c);
             }
         }
@@ -647,7 +647,7 @@ pac_status backward(pac_ctx* c, const int* d_ids, int B, float* d_loss, const pa
     const float* lam = c->params + c->lay.lam;
     const unsigned blocks = cdiv(n, 256);
 #define CHAIN_BWD(ACT)                                                                                        \
-    chain_bwd_kernel<ACT, float><<<blocks, 256, 0, c->stream>>>(sc.u, sc.a, lam, sc.daL, per_sample, dm.S, dm.r, \
+    chain_bwd_kernel<ACT><<<blocks, 256, 0, c->stream>>>(sc.u, sc.a, lam, sc.daL, per_sample, dm.S, dm.r, \
                                                                 dm.L, n, stride, sc.du, sc.lam_part)
     if (c->cfg.act == PAC_ACT_RELU) CHAIN_BWD(PAC_ACT_RELU); else CHAIN_BWD(PAC_ACT_IDENTITY);
 #undef CHAIN_BWD
@@ -923,7 +923,7 @@ pac_status dw_down(pac_ctx* c, const int* d_ids, int B, bool reduce_splits) {
         const bool lm = c->cfg.head == PAC_HEAD_FROZEN_LM;
         gen.tc = c->sc.tc; gen.da = c->sc.da16; gen.da_term = (long long)(lm ? c->max_rows : c->cfg.max_batch) * dm.r;
         gen.da_sample = lm ? (long long)dm.S * dm.r : dm.r; gen.da_token = lm ? dm.r : 0;
-        st = tensor_dw_down(c->tplan, c->stream, d_ids, B, c->sc.du16, c->grads + c->lay.w_down, c->sc.dw_part,
+        st = tensor_dw_down(c->tplan, c->stream, d_ids, B, c->grads + c->lay.w_down, c->sc.dw_part,
                             reduce_splits, c->status, &c->launches, next_stamp(c, 1),
                             c->step_early_ids && !c->step_host_ids, &gen);       // ids no kernel in flight writes
         if (st != PAC_OK) return fail(c, st, "tensor-core dW_down launch failed: %s", tensor_last_error());

@@ -9,13 +9,13 @@
 //      layer go to the u buffer in global memory and are released to the peers with the arrival at a
 //      cluster barrier, long before the stream ends.  A CTA's last layer (together the cluster's top
 //      min(G, L) layers) is complete only when the stream is over: its rows go straight into the
-//      shared memory of the CTA that owns the token (st.async), which counts the bytes on an mbarrier
+//      shared memory of the CTA that owns the token (bulk copies), which counts the bytes on an mbarrier
 //      of its own: no store has to be acknowledged and no barrier crossed behind the stream,
 //   2. the wait at that cluster barrier (long satisfied), behind which every CTA fetches the u rows of
 //      its tokens for the lower layers (L2 hits) into the shared memory the pipeline no longer needs,
 //   3. everything the stand-alone fused kernel does afterwards (mid_body): merge/activation chain
 //      (the handed-over top layers are awaited only where the chain reaches them), pooling, head,
-//      loss, reverse chain -> du_l and dlambda partials.
+//      loss, and the gates and da_L that the second pass builds du_l from.
 #pragma once
 #include "pac_mid.cuh"
 #include "pac_tensor.cuh"

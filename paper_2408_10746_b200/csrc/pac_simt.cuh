@@ -124,16 +124,6 @@ struct CacheRows {            // A(z=l; i=row, k) = h_l[row][k]
         return to_f32(cache[(((id * L) + (layer0 + z)) * S + s) * (long long)d + k]);
     }
 };
-template <typename T>
-struct CacheRowsT {           // A(z=l; i=k_d, k=row) = h_l[row][k_d]   (for dW_down = h^T du)
-    static constexpr bool k_contiguous = false;
-    const T* cache; const int* ids; long long N; int L, S, d;
-    __device__ float operator()(int z, int i, int k) const {
-        int b = k / S, s = k - b * S;
-        long long id = safe_id(ids, b, N, nullptr);
-        return to_f32(cache[(((id * L) + z) * S + s) * (long long)d + i]);
-    }
-};
 struct RowMajor {             // X(z; p, q) = base[z*zstride + p*ld + q]; q contiguous
     const float* base; long long zstride; int ld;
 };
@@ -409,15 +399,14 @@ __global__ void cls_grads_kernel(const float* __restrict__ pooled_a, const float
 // token, daL[b][j]) or per row (LM head: daL[m][j]).  For l = L..1:
 //   dz = da * phi'(z_l)   (ReLU: z_l > 0 <=> a_l > 0),  dlambda_l += dz (u_l - a_{l-1}),
 //   du_l = lambda_l dz,  da = (1 - lambda_l) dz.
-// du is stored in DU (float or bf16).  dlambda: per-block partials, reduced afterwards
-// in block order.  blockDim = 256.
+// dlambda: per-block partials, reduced afterwards in block order.  blockDim = 256.
 // ---------------------------------------------------------------------------
-template <int ACT, typename DU>
+template <int ACT>
 __global__ void __launch_bounds__(256) chain_bwd_kernel(const float* __restrict__ u, const float* __restrict__ a,
                                                         const float* __restrict__ lam,
                                                         const float* __restrict__ daL, int per_sample, int S,
                                                         int r, int L, long long n, long long stride,
-                                                        DU* __restrict__ du, float* __restrict__ lam_part) {
+                                                        float* __restrict__ du, float* __restrict__ lam_part) {
     __shared__ float red[32];
     long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const bool live = e < n;
@@ -438,9 +427,7 @@ __global__ void __launch_bounds__(256) chain_bwd_kernel(const float* __restrict_
         float dz = (ACT == PAC_ACT_RELU) ? (a_l > 0.f ? da : 0.f) : da;
         float part = live ? dz * (u[(long long)l * stride + e] - a_prev) : 0.f;
         if (live) {
-            float v = lm * dz;
-            if constexpr (sizeof(DU) == 2) du[(long long)l * stride + e] = __float2bfloat16(v);
-            else du[(long long)l * stride + e] = v;
+            du[(long long)l * stride + e] = lm * dz;
         }
         da = (1.f - lm) * dz;
         a_l = a_prev;

@@ -13,7 +13,7 @@
 // dropped ones (below 2^-25) are smaller than the rounding of one fp32 multiplication, and sums are fp32.
 // Per SM that is 170 products per clock against 128 on the FP32 pipe, with a tenth of the instructions:
 // the same kernels on FMA tiles (8 tokens x 4 columns per thread, weights through a shared-memory ring) took 60 us
-// per launch instead of 8 at B = 16, S = 128, r = 64, waiting for instructions and shared memory, not for the pipe.
+// per forward launch instead of 30 at B = 16, S = 128, r = 64, waiting for instructions and shared memory, not for the pipe.
 // Weights arrive from L2 in the order of the tile fragments (tb_pack_kernel: a warp reads 512 contiguous bytes per
 // 16 x 8 tile) and are split in registers; activations are split once by whoever produces them.
 #pragma once

@@ -773,7 +773,8 @@ dw_down_tc_kernel(const __grid_constant__ CUtensorMap map_cache, const __grid_co
     if (warp == 1) tmem_dealloc(tmem_base, (uint32_t)p.tmem_cols);
 }
 
-// out[i] = sum_j part[j][i] in split order (deterministic).
+// out[i] = sum_j part[j][i] in split order (deterministic), n a multiple of 4.  The gradient blocks behind lambda[L] in the flat vector
+// start on a 16-byte boundary only when L % 4 == 0.
 __global__ void reduce_splits_kernel(const float* __restrict__ part, int splits, long long n, float* __restrict__ out) {
     long long i = ((long long)blockIdx.x * blockDim.x + threadIdx.x) * 4;
     if (i >= n) return;
@@ -782,7 +783,8 @@ __global__ void reduce_splits_kernel(const float* __restrict__ part, int splits,
         float4 v = *reinterpret_cast<const float4*>(part + (long long)j * n + i);
         acc.x += v.x; acc.y += v.y; acc.z += v.z; acc.w += v.w;
     }
-    *reinterpret_cast<float4*>(out + i) = acc;
+    if (((uintptr_t)out & 15) == 0) *reinterpret_cast<float4*>(out + i) = acc;
+    else { out[i] = acc.x; out[i + 1] = acc.y; out[i + 2] = acc.z; out[i + 3] = acc.w; }
 }
 
 // ---------------------------------------------------------------------------
@@ -990,7 +992,7 @@ struct DuGen { const uint8_t* tc; const bf16* da; long long da_term, da_sample; 
 
 // With reduce_splits == false and more than one split, and always when du is generated, the partial sums stay in `part`
 // ([J][L][d][r]) for the caller's own reduction.
-inline pac_status tensor_dw_down(TensorPlan& tp, cudaStream_t stream, const int* d_ids, int B, const bf16* /*du16*/,
+inline pac_status tensor_dw_down(TensorPlan& tp, cudaStream_t stream, const int* d_ids, int B,
                                  float* dW, float* part, bool reduce_splits, unsigned* status, long long* launches,
                                  unsigned long long* stamp = nullptr, bool early_ids = false, const DuGen* gen = nullptr) {
     BwdParams p = tp.bp;

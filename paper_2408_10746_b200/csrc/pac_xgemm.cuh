@@ -283,19 +283,6 @@ inline int xg_tile_j(int N) {
     return ((N + tiles - 1) / tiles + 15) / 16 * 16;
 }
 
-// out[i] = sum_s part[s][i] in slice order (n a multiple of 4).  The gradient blocks behind lambda[L] in the flat vector start
-// on a 16-byte boundary only when L % 4 == 0: vector loads, scalar stores.
-__global__ void __launch_bounds__(256) sum_slices_kernel(const float* __restrict__ part, int slices, long long n, float* __restrict__ out) {
-    const long long i = ((long long)blockIdx.x * blockDim.x + threadIdx.x) * 4;
-    if (i >= n) return;
-    float4 a = *reinterpret_cast<const float4*>(part + i);
-    for (int s = 1; s < slices; ++s) {
-        const float4 v = *reinterpret_cast<const float4*>(part + s * n + i);
-        a.x += v.x; a.y += v.y; a.z += v.z; a.w += v.w;
-    }
-    out[i] = a.x; out[i + 1] = a.y; out[i + 2] = a.z; out[i + 3] = a.w;
-}
-
 // Slices of a reduction over K rows: whole waves of CTAs, each about 2 us plus 0.6 us per stage (measured), and the slices' own traffic.
 inline int xg_slices(long long tiles, int K, int sms, int most) {
     const int stages = (K + XG_K - 1) / XG_K;

@@ -23,8 +23,10 @@ SPECS = [
     spec("r_16", r=16, S=33),
     spec("r_17", r=17, d=130, dtype="bf16"),                        # first width of the next tile
     spec("r_65", r=65, S=65, d=100),
-    spec("r_96", r=96, d=68, S=31),                                 # three 32-wide tiles
-    spec("r_97", r=97, d=192, dtype="bf16"),                        # two 64-wide tiles, the second nearly empty
+    spec("r_96", r=96, d=68, S=31),
+    spec("r_97", r=97, d=192, dtype="bf16"),
+    spec("r_129", r=129, d=72, S=34),                               # first width of two tiles
+    spec("r_256", r=256, d=136, S=20, L=2),                         # two full tiles
     spec("one_row", r=20, S=1, B=1, d=64),
     spec("row_slices", r=16, S=160, B=6, d=80, L=2),                # the reduction over rows cut into slices
     spec("row_slices_odd", r=24, S=171, B=6, d=132, L=2, dtype="bf16"),
