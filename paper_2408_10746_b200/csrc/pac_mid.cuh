@@ -656,11 +656,25 @@ __device__ __forceinline__ float lambda_grad(const float* lam, const float* P, i
     }
     return g;
 }
-// Blocks of 256 threads: the block's sum of `dot` goes to dot_part[blk]; true in the block that finishes last of n (the shares of all are
-// then visible to it), which puts the counter back.
-__device__ __forceinline__ bool last_with_dots(float dot, float* __restrict__ dot_part, int blk, int n, unsigned* done) {
+// Four consecutive elements of sum_j part[j], j in order, requested three splits at a time.
+__device__ __forceinline__ float4 sum_parts4(const float* __restrict__ part, int splits, long long stride) {
+    float4 a = *reinterpret_cast<const float4*>(part);
+    for (int j = 1; j < splits; j += 3) {
+        float4 q[3];
+#pragma unroll
+        for (int k = 0; k < 3; ++k)
+            if (j + k < splits) q[k] = *reinterpret_cast<const float4*>(part + (j + k) * stride);
+#pragma unroll
+        for (int k = 0; k < 3; ++k)
+            if (j + k < splits) { a.x += q[k].x; a.y += q[k].y; a.z += q[k].z; a.w += q[k].w; }
+    }
+    return a;
+}
+// Blocks of 256 threads: the block's sum of `dot` goes to dot_part[blk]; *last (valid behind the caller's next barrier) says that this block
+// is the last of n to get here: the shares of all are then visible to it.  Called before the block's stores, so that the fence has nothing
+// but the share to wait for.
+__device__ __forceinline__ void publish_dot(float dot, float* __restrict__ dot_part, int blk, int n, unsigned* done, unsigned* last) {
     __shared__ float red[8];
-    __shared__ unsigned last;
     dot = warp_sum(dot);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = dot;
     __syncthreads();
@@ -670,11 +684,9 @@ __device__ __forceinline__ bool last_with_dots(float dot, float* __restrict__ do
         for (int w = 0; w < 8; ++w) t += red[w];
         dot_part[blk] = t;
         __threadfence();
-        last = atomicAdd(done, 1u) == (unsigned)(n - 1);
-        if (last) { *done = 0u; __threadfence(); }
+        *last = atomicAdd(done, 1u) == (unsigned)(n - 1);
+        if (*last) { *done = 0u; __threadfence(); }
     }
-    __syncthreads();
-    return last != 0u;
 }
 // P_l from the blocks' shares, warp per layer, and lambda, into shared memory.
 __device__ __forceinline__ void sum_dots(const float* lam, const float* dot_part, int per_layer, int L, float* lam_s, float* dot_s) {
@@ -682,6 +694,7 @@ __device__ __forceinline__ void sum_dots(const float* lam, const float* dot_part
     for (int l = threadIdx.x; l < L; l += 256) lam_s[l] = lam[l];
     for (int l = warp; l < L; l += 8) {
         float acc = 0.f;
+#pragma unroll 4
         for (int k = lane; k < per_layer; k += 32) acc += __ldcg(dot_part + (long long)l * per_layer + k);
         acc = warp_sum(acc);
         if (lane == 0) dot_s[l] = acc;
@@ -694,29 +707,38 @@ __global__ void __launch_bounds__(256) gated_grads_kernel(const float* __restric
                                                           const float* __restrict__ w, const float* __restrict__ lam, const float* __restrict__ coef,
                                                           float* __restrict__ dot_part, unsigned* done, float* __restrict__ gW, float* __restrict__ glam) {
     const int l = blockIdx.x / per_layer, o = ((blockIdx.x - l * per_layer) * 256 + threadIdx.x) * 4;
-    float dot = 0.f;
+    const long long i = (long long)l * dr + o;
+    float4 a = make_float4(0.f, 0.f, 0.f, 0.f), p = a;
     if (o < dr) {
-        const long long i = (long long)l * dr + o;
-        const float4 p = *reinterpret_cast<const float4*>(w + i);
-        float4 a = *reinterpret_cast<const float4*>(part + i);
-        for (int s = 1; s < splits; ++s) {
-            const float4 v = *reinterpret_cast<const float4*>(part + s * n + i);
-            a.x += v.x; a.y += v.y; a.z += v.z; a.w += v.w;
-        }
-        dot = fmaf(a.x, p.x, fmaf(a.y, p.y, fmaf(a.z, p.z, a.w * p.w)));
+        p = *reinterpret_cast<const float4*>(w + i);
+        a = sum_parts4(part + i, splits, n);
+    }
+    __shared__ float lam_s[128], dot_s[128];
+    __shared__ unsigned last;
+    publish_dot(fmaf(a.x, p.x, fmaf(a.y, p.y, fmaf(a.z, p.z, a.w * p.w))), dot_part, blockIdx.x, gridDim.x, done, &last);
+    if (o < dr) {
         const float c = coef[l];
         *reinterpret_cast<float4*>(gW + i) = make_float4(a.x * c, a.y * c, a.z * c, a.w * c);
     }
-    __shared__ float lam_s[128], dot_s[128];
-    if (last_with_dots(dot, dot_part, blockIdx.x, gridDim.x, done)) {
+    __syncthreads();
+    if (last) {
         sum_dots(lam, dot_part, per_layer, L, lam_s, dot_s);
         for (int k = threadIdx.x; k < L; k += 256) glam[k] = lambda_grad(lam_s, dot_s, L, k);
     }
 }
-__device__ __forceinline__ void lambda_update(const FinalizeParams& f, int l, float g) {
+// lambda_l with its moments, requested before its gradient is known.
+struct LambdaState { float p, m, v; };
+__device__ __forceinline__ LambdaState lambda_load(const FinalizeParams& f, int l) {
+    const long long i = f.lay.lam + l;
+    return f.adam ? LambdaState{f.params[i], f.m[i], f.v[i]} : LambdaState{0.f, 0.f, 0.f};
+}
+__device__ __forceinline__ void lambda_update(const FinalizeParams& f, int l, float g, LambdaState s) {
     const long long i = f.lay.lam + l;
     f.grads[i] = g;
-    if (f.adam) adamw_element(f.params, f.m, f.v, i, g * f.grad_scale, f.lay, f.hp, f.bc1, f.bc2, f.wdT, f.d, f.r);
+    if (!f.adam) return;
+    f.params[i] = adamw_math(s.p, s.m, s.v, g * f.grad_scale, false, f.hp, f.bc1, f.bc2);
+    f.m[i] = s.m;
+    f.v[i] = s.v;
 }
 
 // (five blocks per SM: 48 registers, no spills; T5-Base step 51.0 -> 50.3 us against the 63 registers of an open bound)
@@ -773,13 +795,15 @@ __global__ void __launch_bounds__(256, 5) finalize_cls_kernel(FinalizeParams f) 
         // dlambda where it does not come from the W_down blocks: warp per layer, lanes over its partial sums, fixed shuffle order
         for (int l = warp; l < f.L && !f.coef && !dead; l += nw) {
             float acc = 0.f;
+            const LambdaState old = lambda_load(f, l);
             if (f.lam_part) {
+#pragma unroll 4
                 for (int k = lane; k < f.lam_blocks; k += 32) acc += f.lam_part[(long long)l * f.lam_blocks + k];
                 acc = warp_sum(acc);
             } else {
                 acc = f.grads[lay.lam + l];
             }
-            if (lane == 0) lambda_update(f, l, acc);
+            if (lane == 0) lambda_update(f, l, acc, old);
         }
         return;
     }
@@ -847,42 +871,33 @@ __global__ void __launch_bounds__(256, 5) finalize_cls_kernel(FinalizeParams f) 
         }
         return;
     }
+    const float cf = f.coef ? f.coef[l_wd] : 1.f;
     pdl_wait();
-    {
-        // W_down block, four consecutive elements per thread
-        const long long i = i_wd;
-        if (status_timed_out(f.status)) return;
-        float dot = 0.f;
-        if (wd_thread) {
-            float4 g4;
-            if (f.splits >= 1) {
-                g4 = *reinterpret_cast<const float4*>(f.dw_part + i);
-                for (int j = 1; j < f.splits; ++j) {                 // split order
-                    const float4 q = *reinterpret_cast<const float4*>(f.dw_part + (long long)j * f.dw_elems + i);
-                    g4.x += q.x; g4.y += q.y; g4.z += q.z; g4.w += q.w;
-                }
-                if (f.coef) {
-                    dot = fmaf(g4.x, p4.x, fmaf(g4.y, p4.y, fmaf(g4.z, p4.z, g4.w * p4.w)));
-                    const float c = f.coef[l_wd];
-                    g4.x *= c; g4.y *= c; g4.z *= c; g4.w *= c;
-                }
-                *reinterpret_cast<float4*>(f.grads + i) = g4;
-            } else {
-                g4 = *reinterpret_cast<const float4*>(f.grads + i);
-            }
-            if (f.adam) {
-                g4.x *= f.grad_scale; g4.y *= f.grad_scale; g4.z *= f.grad_scale; g4.w *= f.grad_scale;
-                adamw_w_down4_loaded(f.params, f.m, f.v, i, l_wd, p4, m4, v4, g4, f.hp, f.bc1, f.bc2, f.wdT, f.d, f.r);
-            }
+    // W_down block, four consecutive elements per thread
+    const long long i = i_wd;
+    const unsigned late = f.status ? *reinterpret_cast<const volatile unsigned*>(f.status + ST_TIMEOUT) : 0u;     // (on its way beside the sums)
+    float4 g4 = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (wd_thread) g4 = f.splits >= 1 ? sum_parts4(f.dw_part + i, f.splits, f.dw_elems) : *reinterpret_cast<const float4*>(f.grads + i);
+    if (late) return;
+    __shared__ unsigned last;
+    if (f.coef) publish_dot(fmaf(g4.x, p4.x, fmaf(g4.y, p4.y, fmaf(g4.z, p4.z, g4.w * p4.w))), f.dot_part, blk - f.rest_blocks, f.wd_blocks, f.done, &last);
+    if (wd_thread) {
+        if (f.splits >= 1) {
+            g4.x *= cf; g4.y *= cf; g4.z *= cf; g4.w *= cf;
+            *reinterpret_cast<float4*>(f.grads + i) = g4;
         }
-        if (f.coef) {
-            __shared__ float lam_s[MID_MAX_L], dot_s[MID_MAX_L];
-            if (last_with_dots(dot, f.dot_part, blk - f.rest_blocks, f.wd_blocks, f.done)) {
-                sum_dots(f.params_in + lay.lam, f.dot_part, f.wd_per_layer, f.L, lam_s, dot_s);
-                if (threadIdx.x < f.L) lambda_update(f, threadIdx.x, lambda_grad(lam_s, dot_s, f.L, threadIdx.x));
-            }
+        if (f.adam) {
+            g4.x *= f.grad_scale; g4.y *= f.grad_scale; g4.z *= f.grad_scale; g4.w *= f.grad_scale;
+            adamw_w_down4_loaded(f.params, f.m, f.v, i, l_wd, p4, m4, v4, g4, f.hp, f.bc1, f.bc2, f.wdT, f.d, f.r);
         }
-        return;
+    }
+    if (!f.coef) return;
+    __syncthreads();
+    if (last) {
+        __shared__ float lam_s[MID_MAX_L], dot_s[MID_MAX_L];
+        const LambdaState old = lambda_load(f, min((int)threadIdx.x, f.L - 1));
+        sum_dots(f.params_in + lay.lam, f.dot_part, f.wd_per_layer, f.L, lam_s, dot_s);
+        if (threadIdx.x < f.L) lambda_update(f, threadIdx.x, lambda_grad(lam_s, dot_s, f.L, threadIdx.x), old);
     }
 }
 
