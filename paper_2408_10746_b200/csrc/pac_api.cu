@@ -67,8 +67,7 @@ struct Scratch {
     uint8_t* tc = nullptr;         // [M][r] 1 + highest closed layer
     bf16* da16 = nullptr;          // [2][max_batch][r] (classifier) or [2][M][r] (LM): da_L in two terms
     float* coef = nullptr;         // [L] lambda_l prod_{l' > l} (1 - lambda_l')
-    float* dot_part = nullptr;     // [L][blocks per layer] shares of <D_l, W_down^l>, and the count of blocks done
-    unsigned* dot_done = nullptr;
+    unsigned long long* dot_part = nullptr;     // [L][blocks per layer] shares of <D_l, W_down^l> (publish_dot)
     float* pool_part = nullptr;    // [B][s_chunks * 4][r] token sums of a_L per 32-token group (chain-in-epilogue forward)
     float* prodW = nullptr;        // [r][C] W_up W_head of the current parameters (stand-alone head kernels)
 };
@@ -639,8 +638,8 @@ pac_status backward(pac_ctx* c, const int* d_ids, int B, float* d_loss, const pa
         }
         const long long ne = (long long)dm.L * dm.d * dm.r;
         const int per_layer = (int)cdiv((long long)dm.d * dm.r, 1024);
-        gated_grads_kernel<<<dm.L * per_layer, 256, 0, c->stream>>>(sc.dw_part, tensor_splits(c->tplan, B), ne, dm.d * dm.r, per_layer, dm.L, c->params + c->lay.w_down,
-                                                                  c->params + c->lay.lam, sc.coef, sc.dot_part, sc.dot_done, c->grads + c->lay.w_down, c->grads + c->lay.lam);
+        gated_grads_kernel<<<1 + dm.L * per_layer, 256, 0, c->stream>>>(sc.dw_part, tensor_splits(c->tplan, B), ne, dm.d * dm.r, per_layer, dm.L, c->params + c->lay.w_down,
+                                                                  c->params + c->lay.lam, sc.coef, sc.dot_part, c->grads + c->lay.w_down, c->grads + c->lay.lam, c->status);
         LAUNCH_CHECK(c);
         return PAC_OK;
     }
@@ -1062,7 +1061,7 @@ pac_status finalize_enqueue(pac_ctx* c, const int* d_ids, int B, float* d_loss, 
     const bool tens = use_tensor(c) || c->exact_ok;
     f.dw_part = tens ? sc.dw_part : sc.dw_spart;
     f.splits = tens ? tensor_splits(c->tplan, B) : dw_simt_slices(c, B);
-    if (use_tensor(c)) { f.coef = sc.coef; f.dot_part = sc.dot_part; f.done = sc.dot_done; }
+    if (use_tensor(c)) { f.coef = sc.coef; f.dot_part = sc.dot_part; }
     else if (f.splits <= 1) f.splits = 0;                // already in the gradient buffer
     f.dw_elems = (long long)dm.L * dm.d * dm.r;
     // per-CTA partial sums of dlambda: the fused head kernels', or the plain reverse chain's; transformer bodies: done
@@ -1175,7 +1174,7 @@ void free_all(pac_ctx* c) {
     Scratch& s = c->sc;
     if (c->hc.on) s.hbar = nullptr;            // points into a staging slot, freed below
     void* ptrs[] = {s.ids, s.u, s.a, s.du, s.du16, s.lam_part, s.loss, s.hbar, s.pooled_a, s.pooled_y, s.logits,
-                    s.dlogits, s.loss_b, s.gvec, s.daL, s.y, s.lm_logits, s.dy, s.y16, s.dlog16, s.aL16, s.wup16, s.dy16, s.wdT, s.lm_part, s.dw_part, s.dw_spart, s.tc, s.da16, s.coef, s.dot_part, s.dot_done, s.pool_part, s.prodW, c->tb.buf, c->params, c->grads,
+                    s.dlogits, s.loss_b, s.gvec, s.daL, s.y, s.lm_logits, s.dy, s.y16, s.dlog16, s.aL16, s.wup16, s.dy16, s.wdT, s.lm_part, s.dw_part, s.dw_spart, s.tc, s.da16, s.coef, s.dot_part, s.pool_part, s.prodW, c->tb.buf, c->params, c->grads,
                     c->m, c->v, c->status, c->d_perm, c->d_losses, c->d_stamps};
     for (void* p : ptrs)
         if (p) cudaFree(p);
@@ -1471,9 +1470,9 @@ pac_status pac_adapter_init(pac_ctx* c, const pac_adapter_cfg* cfg, unsigned lon
             }
             if (ts == PAC_OK) {
                 A(dmalloc(c, &s.dw_part, part_floats));
-                A(dmalloc(c, &s.dot_part, (long long)dm.L * cdiv((long long)dm.d * dm.r, 1024)));
-                A(dmalloc(c, &s.dot_done, 1));
-                if (st == PAC_OK) CU_OK(c, cudaMemsetAsync(s.dot_done, 0, sizeof(unsigned), c->stream));
+                const long long shares = (long long)dm.L * cdiv((long long)dm.d * dm.r, 1024);
+                A(dmalloc(c, &s.dot_part, shares));
+                if (st == PAC_OK) CU_OK(c, cudaMemsetAsync(s.dot_part, 0, sizeof(*s.dot_part) * shares, c->stream));
                 c->chain_ok = false;
                 if (st == PAC_OK && cls && c->mplan.ok && chain_fwd_supported(dm) && c->tplan.fp.wide_n) {
                     c->pplan = mid_plan_pooled(dm);
@@ -2002,6 +2001,8 @@ pac_status pac_sync(pac_ctx* c) {
     // optimizer updates that found the timeout flag set were left out: they do not count as steps
     const long long skipped = (long long)c->h_status[ST_SKIPPED_STEPS];
     c->step = c->step > skipped ? c->step - skipped : 0;
+    if (c->h_status[ST_TIMEOUT] && c->sc.dot_part)          // shares that nobody collected
+        CU_OK(c, cudaMemsetAsync(c->sc.dot_part, 0, sizeof(*c->sc.dot_part) * c->dm.L * cdiv((long long)c->dm.d * c->dm.r, 1024), c->stream));
     if (c->h_status[ST_TIMEOUT])
         return fail(c, PAC_ERR_TIMEOUT, "a bounded device-side wait ran out (%u); %lld later optimizer updates were skipped",
                     c->h_status[ST_TIMEOUT], skipped);

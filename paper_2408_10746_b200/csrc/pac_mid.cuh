@@ -605,9 +605,9 @@ struct FinalizeParams {
     int B, d, r, C, L;
     const float* dw_part; int splits; long long dw_elems;     // splits < 1: W_down gradient already in grads
     // Tensor-core path: dw_part holds D_l = h_l^T (open_l daL) (see MidParams), dW_down^l = coef[l] D_l, and P_l = <D_l, W_down^l>
-    // is all that dlambda needs (see lambda_grad): every W_down block leaves its share in dot_part [L][wd_per_layer], the last one to
-    // finish (counted in `done`, which it puts back to zero) updates lambda.
-    const float* coef; float* dot_part; unsigned* done;
+    // is all that dlambda needs (see lambda_grad): every W_down block leaves its share in dot_part [L][wd_per_layer], block 0 waits for
+    // them and updates lambda.
+    const float* coef; unsigned long long* dot_part;
     const float* lam_part; int lam_blocks;                   // null: the lambda gradients are already in grads
     const float *pooled_a, *dlogits, *loss_b;                // per-sample vectors the forward half left: mean_s a_L, dlogits, loss
     const float* hbar; const int* ids; long long N;          // token mean of the last cached layer, per cache sample; the batch's ids
@@ -670,10 +670,10 @@ __device__ __forceinline__ float4 sum_parts4(const float* __restrict__ part, int
     }
     return a;
 }
-// Blocks of 256 threads: the block's sum of `dot` goes to dot_part[blk]; *last (valid behind the caller's next barrier) says that this block
-// is the last of n to get here: the shares of all are then visible to it.  Called before the block's stores, so that the fence has nothing
-// but the share to wait for.
-__device__ __forceinline__ void publish_dot(float dot, float* __restrict__ dot_part, int blk, int n, unsigned* done, unsigned* last) {
+// Shares of P_l travel as (value, 1) in one 64-bit word, so that a block leaves its share with a plain store: no fence, no counter, and the
+// block's slot is free a memory round trip earlier.  The collecting block puts the words back to zero.
+// Blocks of 256 threads: the block's sum of `dot` goes to dot_part[blk].
+__device__ __forceinline__ void publish_dot(float dot, unsigned long long* __restrict__ dot_part, int blk) {
     __shared__ float red[8];
     dot = warp_sum(dot);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = dot;
@@ -682,48 +682,61 @@ __device__ __forceinline__ void publish_dot(float dot, float* __restrict__ dot_p
         float t = 0.f;
 #pragma unroll
         for (int w = 0; w < 8; ++w) t += red[w];
-        dot_part[blk] = t;
-        __threadfence();
-        *last = atomicAdd(done, 1u) == (unsigned)(n - 1);
-        if (*last) { *done = 0u; __threadfence(); }
+        const unsigned long long word = 1ull << 32 | __float_as_uint(t);
+        asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(dot_part + blk), "l"(word) : "memory");
     }
 }
-// P_l from the blocks' shares, warp per layer, and lambda, into shared memory.
-__device__ __forceinline__ void sum_dots(const float* lam, const float* dot_part, int per_layer, int L, float* lam_s, float* dot_s) {
+constexpr int DOT_POLLS = 1 << 24;      // bound on a wait for one share, about ten seconds: another stream's kernel may hold the other blocks back
+// P_l from the blocks' shares, warp per layer, and lambda, into shared memory: one block of 256 threads that runs beside those that publish
+// (it holds one slot, so they all get to run).  False if a share did not arrive; *ok_sh is shared memory.
+__device__ __forceinline__ bool collect_dots(const float* lam, unsigned long long* dot_part, int per_layer, int L, float* lam_s, float* dot_s,
+                                             int* ok_sh, unsigned* status) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (threadIdx.x == 0) *ok_sh = 1;
     for (int l = threadIdx.x; l < L; l += 256) lam_s[l] = lam[l];
+    __syncthreads();
     for (int l = warp; l < L; l += 8) {
         float acc = 0.f;
-#pragma unroll 4
-        for (int k = lane; k < per_layer; k += 32) acc += __ldcg(dot_part + (long long)l * per_layer + k);
+        for (int k = lane; k < per_layer; k += 32) {
+            unsigned long long* at = dot_part + (long long)l * per_layer + k;
+            unsigned long long word = 0;
+            for (int n = 0; n < DOT_POLLS; ++n) {
+                asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(word) : "l"(at) : "memory");
+                if (word != 0ull || *reinterpret_cast<volatile int*>(ok_sh) == 0) break;
+            }
+            if (word == 0ull && atomicExch(ok_sh, 0) && status) atomicAdd(&status[ST_TIMEOUT], 1u);
+            *at = 0ull;
+            acc += __uint_as_float((unsigned)word);
+        }
         acc = warp_sum(acc);
         if (lane == 0) dot_s[l] = acc;
     }
     __syncthreads();
+    return *ok_sh != 0;
 }
-// The gradients of W_down (four elements per thread, blocks within one layer each) and lambda (the block that finishes last) from
-// the second pass's partial sums where no finalisation kernel follows (L <= 128).
+// The gradients of W_down (four elements per thread, blocks within one layer each) and lambda (the first block) from the second pass's
+// partial sums where no finalisation kernel follows (L <= 128).
 __global__ void __launch_bounds__(256) gated_grads_kernel(const float* __restrict__ part, int splits, long long n, int dr, int per_layer, int L,
                                                           const float* __restrict__ w, const float* __restrict__ lam, const float* __restrict__ coef,
-                                                          float* __restrict__ dot_part, unsigned* done, float* __restrict__ gW, float* __restrict__ glam) {
-    const int l = blockIdx.x / per_layer, o = ((blockIdx.x - l * per_layer) * 256 + threadIdx.x) * 4;
+                                                          unsigned long long* __restrict__ dot_part, float* __restrict__ gW, float* __restrict__ glam, unsigned* status) {
+    if (blockIdx.x == 0) {
+        __shared__ float lam_s[128], dot_s[128];
+        __shared__ int ok;
+        if (collect_dots(lam, dot_part, per_layer, L, lam_s, dot_s, &ok, status))
+            for (int k = threadIdx.x; k < L; k += 256) glam[k] = lambda_grad(lam_s, dot_s, L, k);
+        return;
+    }
+    const int blk = blockIdx.x - 1, l = blk / per_layer, o = ((blk - l * per_layer) * 256 + threadIdx.x) * 4;
     const long long i = (long long)l * dr + o;
     float4 a = make_float4(0.f, 0.f, 0.f, 0.f), p = a;
     if (o < dr) {
         p = *reinterpret_cast<const float4*>(w + i);
         a = sum_parts4(part + i, splits, n);
     }
-    __shared__ float lam_s[128], dot_s[128];
-    __shared__ unsigned last;
-    publish_dot(fmaf(a.x, p.x, fmaf(a.y, p.y, fmaf(a.z, p.z, a.w * p.w))), dot_part, blockIdx.x, gridDim.x, done, &last);
+    publish_dot(fmaf(a.x, p.x, fmaf(a.y, p.y, fmaf(a.z, p.z, a.w * p.w))), dot_part, blk);
     if (o < dr) {
         const float c = coef[l];
         *reinterpret_cast<float4*>(gW + i) = make_float4(a.x * c, a.y * c, a.z * c, a.w * c);
-    }
-    __syncthreads();
-    if (last) {
-        sum_dots(lam, dot_part, per_layer, L, lam_s, dot_s);
-        for (int k = threadIdx.x; k < L; k += 256) glam[k] = lambda_grad(lam_s, dot_s, L, k);
     }
 }
 // lambda_l with its moments, requested before its gradient is known.
@@ -805,6 +818,14 @@ __global__ void __launch_bounds__(256, 5) finalize_cls_kernel(FinalizeParams f) 
             }
             if (lane == 0) lambda_update(f, l, acc, old);
         }
+        if (!f.coef) return;
+        const LambdaState old = lambda_load(f, min((int)threadIdx.x, f.L - 1));
+        pdl_wait();
+        if (status_timed_out(f.status)) return;          // (as in the W_down blocks: final behind the wait)
+        __shared__ float lam_s[MID_MAX_L], dot_s[MID_MAX_L];
+        __shared__ int ok;
+        if (collect_dots(f.params_in + lay.lam, f.dot_part, f.wd_per_layer, f.L, lam_s, dot_s, &ok, f.status) && threadIdx.x < f.L)
+            lambda_update(f, threadIdx.x, lambda_grad(lam_s, dot_s, f.L, threadIdx.x), old);
         return;
     }
     if (blk < f.rest_blocks) {
@@ -879,8 +900,7 @@ __global__ void __launch_bounds__(256, 5) finalize_cls_kernel(FinalizeParams f) 
     float4 g4 = make_float4(0.f, 0.f, 0.f, 0.f);
     if (wd_thread) g4 = f.splits >= 1 ? sum_parts4(f.dw_part + i, f.splits, f.dw_elems) : *reinterpret_cast<const float4*>(f.grads + i);
     if (late) return;
-    __shared__ unsigned last;
-    if (f.coef) publish_dot(fmaf(g4.x, p4.x, fmaf(g4.y, p4.y, fmaf(g4.z, p4.z, g4.w * p4.w))), f.dot_part, blk - f.rest_blocks, f.wd_blocks, f.done, &last);
+    if (f.coef) publish_dot(fmaf(g4.x, p4.x, fmaf(g4.y, p4.y, fmaf(g4.z, p4.z, g4.w * p4.w))), f.dot_part, blk - f.rest_blocks);
     if (wd_thread) {
         if (f.splits >= 1) {
             g4.x *= cf; g4.y *= cf; g4.z *= cf; g4.w *= cf;
@@ -890,14 +910,6 @@ __global__ void __launch_bounds__(256, 5) finalize_cls_kernel(FinalizeParams f) 
             g4.x *= f.grad_scale; g4.y *= f.grad_scale; g4.z *= f.grad_scale; g4.w *= f.grad_scale;
             adamw_w_down4_loaded(f.params, f.m, f.v, i, l_wd, p4, m4, v4, g4, f.hp, f.bc1, f.bc2, f.wdT, f.d, f.r);
         }
-    }
-    if (!f.coef) return;
-    __syncthreads();
-    if (last) {
-        __shared__ float lam_s[MID_MAX_L], dot_s[MID_MAX_L];
-        const LambdaState old = lambda_load(f, min((int)threadIdx.x, f.L - 1));
-        sum_dots(f.params_in + lay.lam, f.dot_part, f.wd_per_layer, f.L, lam_s, dot_s);
-        if (threadIdx.x < f.L) lambda_update(f, threadIdx.x, lambda_grad(lam_s, dot_s, f.L, threadIdx.x), old);
     }
 }
 
