@@ -284,11 +284,6 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
 constexpr int CE_THREADS = 512, CE_V4_PER_THREAD = 16, CE_MAX_V = CE_THREADS * CE_V4_PER_THREAD * 4;
 constexpr uint32_t CE_COPY_BYTES = 32768;                 // size of one bulk copy
 
-__device__ __forceinline__ void bulk_load_1d(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                 ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
-}
-
 __global__ void __launch_bounds__(CE_THREADS, 1)
 lm_ce_stream_kernel(const float* __restrict__ logits, const int* __restrict__ ids, long long N, const int* __restrict__ targets,
                     int S, int V, int M, float* __restrict__ loss_row, bf16* __restrict__ dlog16, unsigned* status) {

@@ -63,6 +63,11 @@ __device__ __forceinline__ void dsmem_bulk_copy(uint32_t dst_cluster, uint32_t s
     asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                  ::"r"(dst_cluster), "r"(src_cta), "r"(bytes), "r"(bar_cluster) : "memory");
 }
+// Copy of consecutive global memory into this CTA; addresses and size multiples of 16 bytes.
+__device__ __forceinline__ void bulk_load_1d(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                 ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
+}
 // One arrival at an mbarrier of a CTA of this cluster (address from mapa_shared).
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar_cluster) {
     asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar_cluster) : "memory");
@@ -527,25 +532,29 @@ struct BwdParams {
 // them once.  With splits > 1 the partial sums are added afterwards in split order.
 // Generated du: warps 2 - 9, idle until the accumulators are complete, fill the B part of every stage.  That takes the
 // L * M * r * 2 bytes of du out of memory in both directions; the tile costs five integer instructions per four elements.
+// Gate bytes: a builder that loads them itself runs at two stages per memory latency (1.1 us a stage).  At two and more groups per thread, whose
+// registers allow no deeper look-ahead, they therefore come through the stage ring with the h tile (S = 256, B = 64, L = 24, d = 1024, r = 128:
+// 187 -> 154 us, the rate of the memory).  With one group the ring was slower by 0.7 us: short loops, and one more hop before the first product.
 // GQ: 16-column groups of a generated tile per thread (r = 64 GQ at most; 0: du comes through TMA), GT: its terms.  Registers are
 // bounded so that three finalisation blocks fit beside a CTA (r <= 64; with 155 instead of 88 the step took 58 us for 53).
 // ---------------------------------------------------------------------------
 template <int GQ, int GT>
 __global__ void __launch_bounds__(DW_THREADS) __maxnreg__(GQ <= 1 ? 88 : 168)
 dw_down_tc_kernel(const __grid_constant__ CUtensorMap map_cache, const __grid_constant__ CUtensorMap map_du, BwdParams p) {
-    constexpr bool GEN = GQ > 0;
+    constexpr bool GEN = GQ > 0, RING = GQ > 1;                   // RING: gate bytes through the stage ring, else straight into registers
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     const int r_pad = (p.r + 15) & ~15;
     const uint32_t box_bytes = BWD_KR * 128;                       // one [64 tokens][64 columns] box
     const uint32_t a_bytes = (uint32_t)p.chunks * 2 * box_bytes, b_bytes = (uint32_t)(p.r_blocks * (GEN ? GT : p.terms)) * box_bytes;
-    const uint32_t stage_bytes = a_bytes + b_bytes, tx_bytes = GEN ? a_bytes : stage_bytes;
+    const uint32_t tx_bytes = GEN ? a_bytes : a_bytes + b_bytes, g_off = a_bytes + b_bytes;      // a stage: h tile, du tile, gate bytes
+    const uint32_t stage_bytes = g_off + (RING ? (uint32_t)(BWD_KR * p.r) : 0u);
     constexpr bool side = GT == 2 && GQ <= 2;                      // the terms side by side along N, added up in the epilogue
     const int n_cols = side ? 128 * p.r_blocks : r_pad;            // TMEM columns per accumulator
-    __shared__ __align__(8) unsigned long long bars[2 * 16 + 2];
+    __shared__ __align__(8) unsigned long long bars[3 * 16 + 1];
     __shared__ uint32_t tmem_base_sh;
     __shared__ int abort_sh;
-    const uint32_t full0 = smem_u32(&bars[0]), empty0 = smem_u32(&bars[16]), accf = smem_u32(&bars[32]);
+    const uint32_t full0 = smem_u32(&bars[0]), empty0 = smem_u32(&bars[16]), gate0 = smem_u32(&bars[32]), accf = smem_u32(&bars[48]);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
     int item = blockIdx.x;
@@ -558,7 +567,7 @@ dw_down_tc_kernel(const __grid_constant__ CUtensorMap map_cache, const __grid_co
 
     if (threadIdx.x == 0) {
         abort_sh = 0;
-        for (int s = 0; s < p.stages; ++s) { mbar_init(full0 + 8 * s, GEN ? 1 + DW_GEN_WARPS : 1); mbar_init(empty0 + 8 * s, 1); }
+        for (int s = 0; s < p.stages; ++s) { mbar_init(full0 + 8 * s, GEN ? 1 + DW_GEN_WARPS : 1); mbar_init(empty0 + 8 * s, 1); mbar_init(gate0 + 8 * s, 1); }
         mbar_init(accf, 1);
         fence_mbar_init();
         tma_prefetch_desc(&map_cache);
@@ -602,17 +611,25 @@ dw_down_tc_kernel(const __grid_constant__ CUtensorMap map_cache, const __grid_co
         uint32_t dst = ring0;
         int sc = rt0 % p.s_chunks, b = rt0 / p.s_chunks;
         int id = rt1 > rt0 ? (int)safe_id(p.ids, b, p.N, nullptr) : 0;
+        // the gate bytes of a stage's tokens: consecutive rows of r bytes (those beyond the sample are not read)
+        auto load_gates = [&] {
+            const uint32_t bytes = (uint32_t)(min(BWD_KR, p.S - sc * BWD_KR) * p.r);
+            mbar_expect_tx(gate0 + 8 * s, bytes);
+            bulk_load_1d(dst + g_off, p.tc + ((long long)b * p.S + sc * BWD_KR) * p.r, bytes, gate0 + 8 * s);
+        };
         for (int rt = rt0; rt < rt1; ++rt) {
             const uint32_t full = full0 + 8 * s;
             if (pre > 0) {
                 // first ring: the h tiles are already on their way
                 --pre;
+                if (RING && elect_one()) load_gates();
                 if (!GEN && elect_one())
                     for (int q = 0; q < p.r_blocks * p.terms; ++q)
                         tma_load_3d(dst + a_bytes + q * box_bytes, &map_du, full, (q % p.r_blocks) * 64, b * p.S + sc * BWD_KR, l * p.terms + q / p.r_blocks);
             } else {
                 if (!mbar_wait_uniform(empty0 + 8 * s, eph, abort_flag, p.status)) break;
                 if (elect_one()) {
+                    if (RING) load_gates();
                     mbar_expect_tx(full, tx_bytes);
                     for (int q = 0; q < 2 * p.chunks; ++q)
                         tma_load_4d_hint(dst + q * box_bytes, &map_cache, full, col0 + q * 64, sc * BWD_KR, l, id, pol);
@@ -669,19 +686,19 @@ dw_down_tc_kernel(const __grid_constant__ CUtensorMap map_cache, const __grid_co
         bool ok = true;
         // ---- generated tiles: group g of a stage = 16 columns of one token; this thread's groups lie 256 apart ----
         if constexpr (GEN) {
-            constexpr int AHEAD = GQ < 4 ? 2 : 1;                 // stages whose gates and da are in registers ahead of use
-            int row[GQ], cg[GQ], f_rt = rt0, f_sc = rt0 % p.s_chunks, f_b = rt0 / p.s_chunks;
-            uint32_t off[GQ], gs = 0, geph = 1, gdst = smem_u32(smem) + a_bytes;
+            constexpr int AHEAD = GQ < 4 ? 2 : 1;                 // stages whose da (and gates) are in registers ahead of use
+            int row[GQ], cg[GQ], f_rt = rt0, f_sc = rt0 % p.s_chunks, f_b = rt0 / p.s_chunks, left = p.S - f_sc * BWD_KR;      // left: tokens from the stage's first on
+            uint32_t off[GQ], gs = 0, gph = 0, gdst = smem_u32(smem);
             const uint32_t open_bias = (uint32_t)(l | 0x80) * 0x01010101u;
-            uint4 t4[AHEAD][GQ], d4[AHEAD][GQ][2 * GT];
-            auto fetch = [&](uint4 (&t)[GQ], uint4 (&dd)[GQ][2 * GT]) {
+            uint4 t4[AHEAD], d4[AHEAD][GQ][2 * GT];
+            const uint4 closed = make_uint4(0x7f7f7f7fu, 0x7f7f7f7fu, 0x7f7f7f7fu, 0x7f7f7f7fu);
+            auto fetch = [&](uint4& gates, uint4 (&dd)[GQ][2 * GT]) {
                 if (f_rt >= rt1) return;
 #pragma unroll
                 for (int i = 0; i < GQ; ++i) {
                     if (row[i] < 0) continue;
                     const int tok = f_sc * BWD_KR + row[i];
-                    t[i] = make_uint4(0x7f7f7f7fu, 0x7f7f7f7fu, 0x7f7f7f7fu, 0x7f7f7f7fu);      // closed
-                    if (tok < p.S) t[i] = __ldcg(reinterpret_cast<const uint4*>(p.tc + ((long long)f_b * p.S + tok) * p.r + cg[i]));
+                    if constexpr (!RING) gates = tok < p.S ? __ldcg(reinterpret_cast<const uint4*>(p.tc + ((long long)f_b * p.S + tok) * p.r + cg[i])) : closed;
                     const uint4* d = reinterpret_cast<const uint4*>(p.da + f_b * p.da_sample + (long long)min(tok, p.S - 1) * p.da_token + cg[i]);
 #pragma unroll
                     for (int k = 0; k < GT; ++k) {
@@ -692,14 +709,18 @@ dw_down_tc_kernel(const __grid_constant__ CUtensorMap map_cache, const __grid_co
                 ++f_rt;
                 if (++f_sc == p.s_chunks) { f_sc = 0; ++f_b; }
             };
-            // Builds the next stage's tile and requests the gates of the stage AHEAD further on.
-            auto build = [&](uint4 (&t)[GQ], uint4 (&dd)[GQ][2 * GT]) -> bool {
-                if (!mbar_wait_uniform(empty0 + 8 * gs, geph, abort_flag, p.status)) return false;
+            // Builds the next stage's tile and requests da of the stage AHEAD further on.
+            auto build = [&](uint4& gates, uint4 (&dd)[GQ][2 * GT]) -> bool {
+                // (a stage is free before its gates are requested)
+                if (!mbar_wait_uniform((RING ? gate0 : empty0) + 8 * gs, RING ? gph : gph ^ 1u, abort_flag, p.status)) return false;
 #pragma unroll
                 for (int i = 0; i < GQ; ++i) {
                     if (row[i] < 0) continue;
+                    uint4 t = RING ? closed : gates;
+                    if (RING && row[i] < left)
+                        asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(t.x), "=r"(t.y), "=r"(t.z), "=r"(t.w) : "r"(gdst + g_off + (threadIdx.x - 64 + 256 * i) * 16) : "memory");
                     // open where l + 1 > tc: bit 7 of (l + 128) - tc, byte by byte, spread over the element's two bytes
-                    const uint32_t y[4] = {open_bias - t[i].x, open_bias - t[i].y, open_bias - t[i].z, open_bias - t[i].w};
+                    const uint32_t y[4] = {open_bias - t.x, open_bias - t.y, open_bias - t.z, open_bias - t.w};
                     uint32_t m[8];
 #pragma unroll
                     for (int e = 0; e < 4; ++e) { m[2 * e] = spread_sign(y[e], 0x9988u); m[2 * e + 1] = spread_sign(y[e], 0xbbaau); }
@@ -714,9 +735,11 @@ dw_down_tc_kernel(const __grid_constant__ CUtensorMap map_cache, const __grid_co
                 fence_proxy_async();                              // the tile is read by the tensor core
                 __syncwarp();
                 if (lane == 0) mbar_arrive(full0 + 8 * gs);
-                fetch(t, dd);
+                fetch(gates, dd);
+                left -= BWD_KR;
+                if (left <= 0) left = p.S;
                 gdst += stage_bytes;
-                if (++gs == (uint32_t)p.stages) { gs = 0; geph ^= 1u; gdst = smem_u32(smem) + a_bytes; }
+                if (++gs == (uint32_t)p.stages) { gs = 0; gph ^= 1u; gdst = smem_u32(smem); }
                 return true;
             };
             const int g16 = p.r >> 4, total = BWD_KR * g16;
@@ -725,7 +748,7 @@ dw_down_tc_kernel(const __grid_constant__ CUtensorMap map_cache, const __grid_co
                 const int gi = (int)threadIdx.x - 64 + 256 * i;
                 row[i] = gi / g16; cg[i] = (gi - row[i] * g16) * 16;
                 // box of 64 columns, rows of 128 bytes, 16-byte chunks swizzled with the row
-                off[i] = (uint32_t)(cg[i] >> 6) * box_bytes + (uint32_t)row[i] * 128u + (uint32_t)((((cg[i] & 63) >> 3) ^ (row[i] & 7)) << 4);
+                off[i] = a_bytes + (uint32_t)(cg[i] >> 6) * box_bytes + (uint32_t)row[i] * 128u + (uint32_t)((((cg[i] & 63) >> 3) ^ (row[i] & 7)) << 4);
                 if (gi >= total) row[i] = -1;
             }
 #pragma unroll
@@ -931,7 +954,7 @@ inline pac_status tensor_plan_create(TensorPlan& tp, int device, const bf16* cac
     b.d_groups = (dm.d + 128 * b.chunks - 1) / (128 * b.chunks);
     b.tmem_cols = pow2_at_least(b.chunks * n_cols);
     {
-        const int stage = (b.chunks * 2 + b.r_blocks * dt) * BWD_KR * 128;
+        const int stage = (b.chunks * 2 + b.r_blocks * dt) * BWD_KR * 128 + (gen && dm.r > 64 ? BWD_KR * dm.r : 0);
         int st = (max_smem - 2048) / stage;
         if (st > 16) st = 16;
         if (st < 2) { tensor_err() = "not enough shared memory for the backward pipeline"; return PAC_ERR_UNSUPPORTED; }
