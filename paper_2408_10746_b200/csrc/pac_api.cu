@@ -1171,9 +1171,12 @@ pac_status adam_enqueue(pac_ctx* c, const pac_adamw* hp) {
     const int wd_blocks = (c->lay.lam % 4 == 0) ? (int)cdiv(c->lay.lam / 4, 256) : 0;
     const long long total = c->tb.on ? c->lay.body : c->lay.total;
     const unsigned rest = cdiv(total - (wd_blocks ? c->lay.lam : 0), 256);
-    adamw_kernel<<<wd_blocks + rest, 256, 0, c->stream>>>(c->params, c->grads, c->m, c->v, total, c->lay, *hp, bc1, bc2,
-                                                          wd_shadow(c), c->dm.d, c->dm.r, wd_blocks, c->status, c->grad_scale);
-    LAUNCH_CHECK(c);
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    pdl_launch_config(&cfg, attr, dim3(wd_blocks + rest), dim3(256), 0, c->stream);
+    CU_OK(c, cudaLaunchKernelEx(&cfg, adamw_kernel, c->params, (const float*)c->grads, c->m, c->v, total, c->lay, *hp, bc1, bc2, wd_shadow(c), c->dm.d, c->dm.r,
+                                wd_blocks, c->status, c->grad_scale));
+    c->launches++;
     return c->tb.on ? adam_body_enqueue(c, hp) : PAC_OK;
 }
 

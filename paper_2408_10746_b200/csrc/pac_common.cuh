@@ -25,6 +25,13 @@ __device__ __forceinline__ bool status_timed_out(const unsigned* status) {
     return status && *reinterpret_cast<const volatile unsigned*>(status + ST_TIMEOUT) != 0u;
 }
 
+// Programmatic dependent launch: a kernel launched with the programmatic-serialization
+// attribute may start while its predecessor in the stream is still running; pdl_wait() blocks
+// until the predecessor grid has completed and its writes are visible, pdl_trigger() lets the
+// successor start launching.  Without the attribute both are no-ops.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // Sample id of batch row b, clamped into [0, N) so that no kernel can read outside
 // the cache even if a device-resident id is bad; clamps are counted.
 __device__ __forceinline__ long long safe_id(const int* __restrict__ ids, int b, long long N, unsigned* status) {

@@ -165,7 +165,8 @@ __global__ void __launch_bounds__(256) head_matrix_kernel(const float* __restric
     if (e >= r * C) return;
     const int j = e / C, c = e - j * C;
     float acc = 0.f;
-    for (int k = lane; k < d; k += 32) acc = fmaf(W_up[(long long)j * d + k], W_head[(long long)k * C + c], acc);
+#pragma unroll 8
+    for (int k = lane; k < d; k += 32) acc = fmaf(__ldg(W_up + (long long)j * d + k), __ldg(W_head + (long long)k * C + c), acc);
     acc = warp_sum(acc);
     if (lane == 0) prodW[e] = acc;
 }

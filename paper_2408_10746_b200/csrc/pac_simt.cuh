@@ -550,6 +550,8 @@ __global__ void adamw_kernel(float* __restrict__ p, const float* __restrict__ g,
                              float* __restrict__ v, long long n, ParamLayout lay, pac_adamw hp, float bc1,
                              float bc2, WdShadow wdT, int d, int r, int wd_blocks, unsigned* status,
                              float grad_scale) {
+    pdl_wait();
+    pdl_trigger();
     // gradients computed after a bounded wait ran out are not trustworthy: leave the state alone
     if (status_timed_out(status)) {
         if (blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(&status[ST_SKIPPED_STEPS], 1u);

@@ -29,12 +29,6 @@ __device__ __forceinline__ void st_global_32(void* p, uint4 a, uint4 b) {
     asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
                  ::"l"(p), "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b.x), "r"(b.y), "r"(b.z), "r"(b.w) : "memory");
 }
-// Programmatic dependent launch: a kernel launched with the programmatic-serialization
-// attribute may start while its predecessor in the stream is still running; pdl_wait() blocks
-// until the predecessor grid has completed and its writes are visible, pdl_trigger() lets the
-// successor start launching.  Without the attribute both are no-ops.
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
