@@ -62,6 +62,8 @@ struct Scratch {
     bf16* wdT = nullptr;           // bf16 terms of W_down, [L][2 or 3][d][r]
     float* lm_part = nullptr;      // [slices][...] partial sums of the LM path's two skinny products (dW_up, da_L)
     float* dw_part = nullptr;      // split partials of dW_down
+    float* xg_ws = nullptr;        // sums of the tiles that several CTAs share, and their counts (plain path)
+    unsigned* xg_cnt = nullptr;
     float* dw_spart = nullptr;     // row-slice partials of dW_down on the plain path
     // what the second pass over the cache builds du from (tensor-core path, see MidParams)
     uint8_t* tc = nullptr;         // [M][r] 1 + highest closed layer
@@ -395,7 +397,7 @@ pac_status xgemm_rows(pac_ctx* c, int M, int N, int K, int Z, const AL& A, const
     XgJobs<AL> J;
     J.tile_j = xg_tile_j(N);
     J.add(A, M, W, N, 0);
-    cudaError_t e = xgemm_launch<false>(J, K, Z, 1, out, zstride, 0, c->status, c->stream);
+    cudaError_t e = xgemm_launch_rows(J, K, Z, c->sms, out, zstride, c->sc.xg_ws, c->sc.xg_cnt, c->status, c->stream);
     c->launches++;
     if (e != cudaSuccess) return fail(c, PAC_ERR_CUDA, "product kernel launch failed: %s", cudaGetErrorString(e));
     return PAC_OK;
@@ -403,7 +405,7 @@ pac_status xgemm_rows(pac_ctx* c, int M, int N, int K, int Z, const AL& A, const
 // The jobs' A^T B over M rows for all Z layers, `slices` row slices (partial sums part_stride apart when more than one).
 template <class AL>
 pac_status xgemm_tn(pac_ctx* c, const XgJobs<AL>& J, int M, int Z, int slices, float* out, long long zstride, long long part_stride) {
-    cudaError_t e = xgemm_launch<true>(J, M, Z, slices, out, zstride, part_stride, c->status, c->stream);
+    cudaError_t e = xgemm_launch_tn(J, M, Z, slices, out, zstride, part_stride, c->status, c->stream);
     c->launches++;
     if (e != cudaSuccess) return fail(c, PAC_ERR_CUDA, "product kernel launch failed: %s", cudaGetErrorString(e));
     return PAC_OK;
@@ -1200,7 +1202,7 @@ void free_all(pac_ctx* c) {
     Scratch& s = c->sc;
     if (c->hc.on) s.hbar = nullptr;            // points into a staging slot, freed below
     void* ptrs[] = {s.ids, s.u, s.a, s.du, s.du16, s.lam_part, s.loss, s.hbar, s.pooled_a, s.pooled_y, s.logits,
-                    s.dlogits, s.loss_b, s.gvec, s.daL, s.y, s.lm_logits, s.dy, s.y16, s.dlog16, s.aL16, s.wup16, s.dy16, s.wdT, s.lm_part, s.dw_part, s.dw_spart, s.tc, s.da16, s.coef, s.dot_part, s.pool_part, s.prodW, c->tb.buf, c->params, c->grads,
+                    s.dlogits, s.loss_b, s.gvec, s.daL, s.y, s.lm_logits, s.dy, s.y16, s.dlog16, s.aL16, s.wup16, s.dy16, s.wdT, s.lm_part, s.dw_part, s.dw_spart, s.xg_ws, s.xg_cnt, s.tc, s.da16, s.coef, s.dot_part, s.pool_part, s.prodW, c->tb.buf, c->params, c->grads,
                     c->m, c->v, c->status, c->d_perm, c->d_stamps};
     for (void* p : ptrs)
         if (p) cudaFree(p);
@@ -1546,6 +1548,9 @@ pac_status pac_adapter_init(pac_ctx* c, const pac_adapter_cfg* cfg, unsigned lon
         c->dw_simt_max = 1;
         for (int b = 1; b <= cfg->max_batch && ne % 4 == 0; ++b) c->dw_simt_max = std::max(c->dw_simt_max, xg_slices(dw_simt_tiles(dm), b * dm.S, c->sms, 8));
         if (c->dw_simt_max > 1) A(dmalloc(c, &s.dw_spart, ne * c->dw_simt_max));
+        A(dmalloc(c, &s.xg_ws, (long long)c->sms * XG_TILE * xg_tile_j(dm.r)));
+        A(dmalloc(c, &s.xg_cnt, c->sms));
+        if (st == PAC_OK) CU_OK(c, cudaMemsetAsync(s.xg_cnt, 0, sizeof(unsigned) * c->sms, c->stream));
     }
     if (st == PAC_OK && c->tb.on) {
         TBody& t = c->tb;

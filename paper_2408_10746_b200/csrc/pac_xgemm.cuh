@@ -105,11 +105,17 @@ __host__ __device__ inline uint32_t xg_term_b(int tile_j) { return (uint32_t)((t
 template <class AL>
 inline size_t xg_smem(int tile_j) { return 2 * ((size_t)XgTerms<typename AL::elem>::n * XG_TERM_A + 3 * xg_term_b(tile_j)) + 1024; }
 
-// Grid: (tiles of all jobs, layers, slices of the reduction).  With more than one slice the partial sums of slice s go to
+// The tiles of an incomplete last wave (rows): `whole` tiles are computed by one CTA each, every later one by `parts` CTAs that take k_slice
+// of the reduction each, leave their sums in ws and are added up, in order, by the one that finishes last (counted in cnt, which it puts back
+// to zero).  At 192 tiles of 12 stages on 148 SMs
+// the fp32 step went from 93.8 to 92.0 us (a CTA's start and end, not its stages, are the larger part of what the last wave costs).
+struct XgTail { int whole, parts; float* ws; unsigned* cnt; };
+// tn: grid (tiles of all jobs, layers, slices of the reduction); rows: (whole + parts * the other tiles).
+// tn with more than one slice: the partial sums of slice s go to
 // out + s * part_stride and are added up in slice order by whoever reads them.  GB: 8-column groups of B per thread (tile_j = 32 GB at most).
 template <bool TN, int GB, class AL>
 __global__ void __launch_bounds__(XG_THREADS, 1)
-xgemm_kernel(const __grid_constant__ XgJobs<AL> J, int K, int k_slice, float* __restrict__ out, long long zstride, long long part_stride, unsigned* status) {
+xgemm_kernel(const __grid_constant__ XgJobs<AL> J, int K, int k_slice, float* __restrict__ out, long long zstride, long long part_stride, XgTail tail, unsigned* status) {
     typedef typename AL::elem T;
     constexpr int TA = XgTerms<T>::n;
     extern __shared__ unsigned char smem_raw[];
@@ -120,13 +126,25 @@ xgemm_kernel(const __grid_constant__ XgJobs<AL> J, int K, int k_slice, float* __
     __shared__ uint32_t tmem_base_sh;
     __shared__ int abort_sh;
     const uint32_t full0 = smem_u32(&bars[0]), empty0 = smem_u32(&bars[2]), accf = smem_u32(&bars[4]);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, z = blockIdx.y;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    int z = blockIdx.y, at = blockIdx.x, split = TN ? (int)blockIdx.z : 0, shared_tile = -1;
+    if (!TN) {
+        if (at >= tail.whole) {
+            const int q = at - tail.whole;
+            shared_tile = q / tail.parts;
+            split = q - shared_tile * tail.parts;
+            at = tail.whole + shared_tile;
+        }
+        const int tiles = J.first[J.n];
+        z = at / tiles;
+        at -= z * tiles;
+    }
     int jb = 0;
-    while (jb + 1 < J.n && (int)blockIdx.x >= J.first[jb + 1]) ++jb;
-    const int tile = blockIdx.x - J.first[jb];
+    while (jb + 1 < J.n && at >= J.first[jb + 1]) ++jb;
+    const int tile = at - J.first[jb];
     const int i0 = tile / J.tiles_j[jb] * XG_TILE, j0 = tile % J.tiles_j[jb] * nj_tile;
     const int Mi = J.mi[jb], Nj = J.nj[jb];
-    const int kb = blockIdx.z * k_slice, ke = min(K, kb + k_slice), stages = ke > kb ? (ke - kb + XG_K - 1) / XG_K : 0;
+    const int kb = split * k_slice, ke = !TN && shared_tile < 0 ? K : min(K, kb + k_slice), stages = ke > kb ? (ke - kb + XG_K - 1) / XG_K : 0;
     if (threadIdx.x == 0) {
         abort_sh = 0;
         for (int s = 0; s < 2; ++s) { mbar_init(full0 + 8 * s, XG_PRODUCERS / 2); mbar_init(empty0 + 8 * s, 1); }
@@ -238,11 +256,17 @@ xgemm_kernel(const __grid_constant__ XgJobs<AL> J, int K, int k_slice, float* __
         }
         if (ok) {
             const int q = warp & 3, i = i0 + q * 32 + lane;
-            float* o = out + blockIdx.z * part_stride + z * zstride + J.out_off[jb];
+            float* o = out + split * part_stride + z * zstride + J.out_off[jb];
+            float* ws = tail.ws + ((long long)(shared_tile * tail.parts + split) * XG_TILE + q * 32 + lane) * nj_tile;
             const bool vec = !J.trans && (Nj & 3) == 0 && ((uintptr_t)o & 15) == 0;
             for (int c0 = (warp >> 2) * 16; c0 < nj_tile; c0 += 64) {
                 float v[16] = {};
                 if (stages > 0) { tmem_ld16(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)c0, v); tmem_ld_wait(); }
+                if (!TN && shared_tile >= 0) {
+#pragma unroll
+                    for (int e = 0; e < 16; e += 4) *reinterpret_cast<float4*>(ws + c0 + e) = make_float4(v[e], v[e + 1], v[e + 2], v[e + 3]);
+                    continue;
+                }
                 if (i >= Mi) continue;
 #pragma unroll
                 for (int e = 0; e < 16; e += 4) {
@@ -258,6 +282,32 @@ xgemm_kernel(const __grid_constant__ XgJobs<AL> J, int K, int k_slice, float* __
             }
         }
     }
+    if (!TN && shared_tile >= 0) {
+        __shared__ int last;
+        __threadfence();
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            last = atomicAdd(tail.cnt + shared_tile, 1u) == (unsigned)(tail.parts - 1);
+            if (last) tail.cnt[shared_tile] = 0u;
+            __threadfence();
+        }
+        __syncthreads();
+        if (last) {
+            const float* ws = tail.ws + (long long)shared_tile * tail.parts * XG_TILE * nj_tile;
+            float* o = out + z * zstride + J.out_off[jb];
+            for (int e = threadIdx.x * 4; e < XG_TILE * nj_tile; e += XG_THREADS * 4) {
+                float4 a = __ldcg(reinterpret_cast<const float4*>(ws + e));
+                for (int k = 1; k < tail.parts; ++k) {
+                    const float4 b = __ldcg(reinterpret_cast<const float4*>(ws + (long long)k * XG_TILE * nj_tile + e));
+                    a.x += b.x; a.y += b.y; a.z += b.z; a.w += b.w;
+                }
+                const int i = i0 + e / nj_tile, j = j0 + e % nj_tile;
+                const float v[4] = {a.x, a.y, a.z, a.w};
+                for (int x = 0; x < 4 && i < Mi; ++x)
+                    if (j + x < Nj) o[(long long)i * Nj + j + x] = v[x];
+            }
+        }
+    }
     tc_fence_before();
     __syncthreads();
     drain_after_abort(abort_flag);
@@ -265,16 +315,33 @@ xgemm_kernel(const __grid_constant__ XgJobs<AL> J, int K, int k_slice, float* __
 }
 
 template <bool TN, class AL>
-inline cudaError_t xgemm_launch(const XgJobs<AL>& J, int K, int Z, int slices, float* out, long long zstride, long long part_stride, unsigned* status, cudaStream_t stream) {
-    const int k_slice = ((K + slices - 1) / slices + XG_K - 1) / XG_K * XG_K;
+inline cudaError_t xgemm_launch(const XgJobs<AL>& J, int K, dim3 grid, int k_slice, float* out, long long zstride, long long part_stride, const XgTail& tail, unsigned* status, cudaStream_t stream) {
     const auto kernel = J.tile_j <= 64 ? xgemm_kernel<TN, 2, AL> : xgemm_kernel<TN, 4, AL>;
     const size_t smem = xg_smem<AL>(J.tile_j);
     cudaError_t e = smem_opt_in((const void*)kernel, smem);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[1];
-    pdl_launch_config(&cfg, attr, dim3((unsigned)J.first[J.n], (unsigned)Z, (unsigned)slices), dim3(XG_THREADS), smem, stream);
-    return cudaLaunchKernelEx(&cfg, kernel, J, K, k_slice, out, zstride, part_stride, status);
+    pdl_launch_config(&cfg, attr, grid, dim3(XG_THREADS), smem, stream);
+    return cudaLaunchKernelEx(&cfg, kernel, J, K, k_slice, out, zstride, part_stride, tail, status);
+}
+template <class AL>
+inline cudaError_t xgemm_launch_tn(const XgJobs<AL>& J, int K, int Z, int slices, float* out, long long zstride, long long part_stride, unsigned* status, cudaStream_t stream) {
+    const int k_slice = ((K + slices - 1) / slices + XG_K - 1) / XG_K * XG_K;
+    return xgemm_launch<true>(J, K, dim3((unsigned)J.first[J.n], (unsigned)Z, (unsigned)slices), k_slice, out, zstride, part_stride, XgTail{}, status, stream);
+}
+// ws: sms tiles of 128 x tile_j floats, cnt: sms words of zero.  A tile of the last wave is shared when that takes four or more stages off its CTA
+// (the exchange costs about as much as three).
+template <class AL>
+inline cudaError_t xgemm_launch_rows(const XgJobs<AL>& J, int K, int Z, int sms, float* out, long long zstride, float* ws, unsigned* cnt, unsigned* status, cudaStream_t stream) {
+    const int total = J.first[J.n] * Z, stages = (K + XG_K - 1) / XG_K, rest = total % sms;
+    XgTail tail{total, 1, ws, cnt};
+    int per = stages;
+    if (rest > 0) {
+        per = (stages + sms / rest - 1) / (sms / rest);
+        if (stages - per >= 4) { tail.whole = total - rest; tail.parts = (stages + per - 1) / per; }
+    }
+    return xgemm_launch<false>(J, K, dim3((unsigned)(tail.whole + (total - tail.whole) * tail.parts)), per * XG_K, out, zstride, 0, tail, status, stream);
 }
 
 // Columns per tile for an output N wide, tiles of equal width.
