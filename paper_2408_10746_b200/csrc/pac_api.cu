@@ -106,6 +106,8 @@ struct HostCache {
     const int* host_labels = nullptr;       // [N][labels_per_sample], host memory
     long long N = 0;                        // samples in the host cache
     long long sample_bytes = 0;             // L * S * d * element size
+    long long pair_pitch = 0;               // largest pitch of a two-sample copy (0: pageable memory, one copy per sample)
+    std::vector<char> paired;               // per row of the batch: already copied with an earlier one
     int cur = 0;                            // slot the next step uses
     unsigned char* stage[2] = {nullptr, nullptr};   // device [max_batch][L][S][d]
     int* lab_stage[2] = {nullptr, nullptr};         // device [max_batch][labels_per_sample]
@@ -1311,6 +1313,11 @@ pac_status pac_cache_register_host(pac_ctx* c, const void* host_cache, int dtype
     if (st != PAC_OK) return st;
     c->hc.on = true;
     c->hc.host = (const unsigned char*)host_cache;
+    cudaPointerAttributes pa;
+    if (cudaPointerGetAttributes(&pa, host_cache) != cudaSuccess) { cudaGetLastError(); pa.type = cudaMemoryTypeUnregistered; }
+    int pitch = 0;
+    if (pa.type == cudaMemoryTypeHost) CU_OK(c, cudaDeviceGetAttribute(&pitch, cudaDevAttrMaxPitch, c->device));
+    c->hc.pair_pitch = pitch;
     c->hc.host_labels = host_labels;
     c->hc.N = N;
     c->hc.sample_bytes = (long long)L * S * d * (dtype == PAC_F32 ? 4 : 2);
@@ -1659,9 +1666,23 @@ pac_status host_cache_stage(pac_ctx* c, const int* ids, int B, const char* who, 
     // its step must have finished before the slabs are overwritten
     CU_OK(c, cudaEventSynchronize(h.ready[k]));
     CU_OK(c, cudaStreamWaitEvent(h.copy_stream, h.freed[k], 0));
+    // Two samples in ascending order, wherever they lie, are the two rows of one pitched copy: a copy costs the engine about 5 us on top of
+    // its bytes (2.4 MB samples: 49.6 GB/s one by one, 52.7 in pairs, 55.4 in one piece; reads by a kernel reach 51).
+    h.paired.assign(B, 0);
     for (int b = 0; b < B; ++b) {
-        CU_OK(c, cudaMemcpyAsync(h.stage[k] + (size_t)b * h.sample_bytes, h.host + (size_t)ids[b] * h.sample_bytes,
-                                 (size_t)h.sample_bytes, cudaMemcpyHostToDevice, h.copy_stream));
+        if (!h.paired[b]) {
+            const long long n = h.sample_bytes, most = h.pair_pitch / n;
+            int j = most > 0 ? b + 1 : B;
+            while (j < B && (h.paired[j] || ids[j] <= ids[b] || ids[j] - ids[b] > most || j - b > most)) ++j;
+            unsigned char* dst = h.stage[k] + b * n;
+            const unsigned char* src = h.host + ids[b] * n;
+            if (j < B && cudaMemcpy2DAsync(dst, (size_t)((j - b) * n), src, (size_t)((ids[j] - ids[b]) * n), (size_t)n, 2, cudaMemcpyHostToDevice, h.copy_stream) == cudaSuccess) {
+                h.paired[j] = 1;
+            } else {
+                if (j < B) { cudaGetLastError(); h.pair_pitch = 0; }       // (host memory locked in pieces)
+                CU_OK(c, cudaMemcpyAsync(dst, src, (size_t)n, cudaMemcpyHostToDevice, h.copy_stream));
+            }
+        }
         std::memcpy(h.h_lab[k] + (size_t)b * lps, h.host_labels + (size_t)ids[b] * lps, sizeof(int) * lps);
     }
     CU_OK(c, cudaMemcpyAsync(h.lab_stage[k], h.h_lab[k], sizeof(int) * (size_t)B * lps, cudaMemcpyHostToDevice, h.copy_stream));

@@ -43,3 +43,20 @@ def test_epoch_equals_epoch_with_device_ids(case, n, B):
     assert np.array_equal(host.get_params(), dev.get_params())
     assert host.train_step(perm[:B]) == dev.train_step(perm[:B])
     host.close(); dev.close()
+
+
+@pytest.mark.parametrize("pinned", [True, False], ids=["pinned", "pageable"])
+@pytest.mark.parametrize("ids", [[5], [3, 9], [9, 3], [4, 4, 4], [599, 0, 598, 1, 2, 2, 300], list(range(20)), list(range(20, 0, -1))], ids=str)
+def test_samples_from_host_memory_land_in_their_rows(case, ids, pinned):
+    """Two samples of a batch may travel as the rows of one copy: ascending, descending, repeated and odd ones."""
+    cache, labels = case.cache.cpu(), case.labels.cpu()
+    if pinned:
+        cache, labels = cache.pin_memory(), labels.pin_memory()
+    ctx = pac.PacContext(0)
+    ctx.cache_register_host(cache, labels)
+    ctx.adapter_init(r=SPEC.r, n_out=SPEC.n_out, max_batch=20, seed=1)
+    out = torch.empty((SPEC.L, len(ids), SPEC.S, SPEC.d), dtype=torch.bfloat16, device="cuda")
+    ctx.gather(ids, out)
+    ctx.sync()
+    assert torch.equal(out, case.cache[torch.tensor(ids, device="cuda")].transpose(0, 1))
+    ctx.close()
