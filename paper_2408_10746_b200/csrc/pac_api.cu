@@ -1497,12 +1497,12 @@ pac_status pac_adapter_init(pac_ctx* c, const pac_adapter_cfg* cfg, unsigned lon
         long long part_floats = 0;
         if (st == PAC_OK) {
             pac_status ts = tensor_plan_create(c->tplan, c->device, (const bf16*)c->cache, dm, cfg->max_batch, s.wdT,
-                                               nullptr, &part_floats, false, !cls);
+                                               nullptr, &part_floats);
             if (ts == PAC_OK && c->hc.on) {
                 // one set of tensor maps per staging slot
                 c->hc.tplan[0] = c->tplan;
                 long long pf2 = 0;
-                ts = tensor_plan_create(c->hc.tplan[1], c->device, (const bf16*)c->hc.stage[1], dm, cfg->max_batch, s.wdT, nullptr, &pf2, false, !cls);
+                ts = tensor_plan_create(c->hc.tplan[1], c->device, (const bf16*)c->hc.stage[1], dm, cfg->max_batch, s.wdT, nullptr, &pf2);
             }
             if (ts == PAC_OK) {
                 A(dmalloc(c, &s.dw_part, part_floats));

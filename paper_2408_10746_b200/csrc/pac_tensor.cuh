@@ -510,7 +510,7 @@ struct BwdParams {
     int tmem_cols;
     int early_ids;                         // 1: no kernel ahead of this one in the stream writes the ids
     // gen: du_l is not read but built in shared memory from one byte per element (see MidParams in pac_mid.cuh) and da_L, one vector per
-    // sample or token, in one or two bf16 terms: B = open_l ? da : 0, out = h_l^T B without the layer's factor.
+    // sample or token, in two bf16 terms: B = open_l ? da : 0, out = h_l^T B without the layer's factor.
     int gen;
     const uint8_t* tc;                     // [max_rows][r]
     const bf16* da; long long da_term, da_sample; int da_token;      // strides in elements
@@ -529,13 +529,14 @@ struct BwdParams {
 // Gate bytes: a builder that loads them itself runs at two stages per memory latency (1.1 us a stage).  At two and more groups per thread, whose
 // registers allow no deeper look-ahead, they therefore come through the stage ring with the h tile (S = 256, B = 64, L = 24, d = 1024, r = 128:
 // 187 -> 154 us, the rate of the memory).  With one group the ring was slower by 0.7 us: short loops, and one more hop before the first product.
-// GQ: 16-column groups of a generated tile per thread (r = 64 GQ at most; 0: du comes through TMA), GT: its terms.  Registers are
+// GQ: 16-column groups of a generated tile per thread (r = 64 GQ at most; 0: du comes through TMA).  Registers are
 // bounded so that three finalisation blocks fit beside a CTA (r <= 64; with 155 instead of 88 the step took 58 us for 53).
 // ---------------------------------------------------------------------------
-template <int GQ, int GT>
+template <int GQ>
 __global__ void __launch_bounds__(DW_THREADS) __maxnreg__(GQ <= 1 ? 88 : 168)
 dw_down_tc_kernel(const __grid_constant__ CUtensorMap map_cache, const __grid_constant__ CUtensorMap map_du, BwdParams p) {
     constexpr bool GEN = GQ > 0, RING = GQ > 1;                   // RING: gate bytes through the stage ring, else straight into registers
+    constexpr int GT = 2;                                         // terms of a generated tile
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     const int r_pad = (p.r + 15) & ~15;
@@ -543,7 +544,7 @@ dw_down_tc_kernel(const __grid_constant__ CUtensorMap map_cache, const __grid_co
     const uint32_t a_bytes = (uint32_t)p.chunks * 2 * box_bytes, b_bytes = (uint32_t)(p.r_blocks * (GEN ? GT : p.terms)) * box_bytes;
     const uint32_t tx_bytes = GEN ? a_bytes : a_bytes + b_bytes, g_off = a_bytes + b_bytes;      // a stage: h tile, du tile, gate bytes
     const uint32_t stage_bytes = g_off + (RING ? (uint32_t)(BWD_KR * p.r) : 0u);
-    constexpr bool side = GT == 2 && GQ <= 2;                      // the terms side by side along N, added up in the epilogue
+    constexpr bool side = GEN && GQ <= 2;                          // the terms side by side along N, added up in the epilogue
     const int n_cols = side ? 128 * p.r_blocks : r_pad;            // TMEM columns per accumulator
     __shared__ __align__(8) unsigned long long bars[3 * 16 + 1];
     __shared__ uint32_t tmem_base_sh;
@@ -878,7 +879,7 @@ inline int pow2_at_least(int x) { int p = 32; while (p < x) p <<= 1; return p; }
 // [L][3][max_rows][r]), whose sum is the fp32 value, so the products are those of fp32 operands.  *part_floats receives the
 // size of the split-partial buffer dW needs (0 when no split is used).
 inline pac_status tensor_plan_create(TensorPlan& tp, int device, const bf16* cache, const Dims& dm, int max_batch,
-                                     const bf16* wdT, const bf16* du16, long long* part_floats, bool exact = false, bool per_token = false) {
+                                     const bf16* wdT, const bf16* du16, long long* part_floats, bool exact = false) {
     const bool gen = !exact;                                 // du is generated (pointwise bodies)
     tp.ready = false;
     tp.dm = dm;
@@ -891,10 +892,10 @@ inline pac_status tensor_plan_create(TensorPlan& tp, int device, const bf16* cac
     const long long max_rows = (long long)max_batch * dm.S;
     const int r_pad = (dm.r + 15) & ~15;
     const int wt = exact ? 3 : 2;                            // bf16 terms of W_down
-    // of du: the fp32 value exactly, or generated: two terms of da, as precise as W_down, where the second one's products cost nothing beside the
-    // stream (with one, dlambda of a small batch is off by a percent); one for wide adapters with da per sample, where they cost power
-    // and du entered in one term before
-    const int dt = exact ? 3 : dm.r <= 64 || per_token ? 2 : 1;
+    // of du: the fp32 value exactly, or generated: two terms of da, as dlambda, which comes from the same product, needs them: against 64 bits it is
+    // off by 1e-3 to 8e-3 with one and by 2e-6 to 2e-5 with two.  Up to r = 64 the second term's products cost nothing beside the stream; at
+    // B = 64, S = 256, L = 24, d = 1024, r = 128 the step takes 465 us for 430.
+    const int dt = exact ? 3 : 2;
 
     // ---- tensor maps ----
     {
@@ -943,7 +944,7 @@ inline pac_status tensor_plan_create(TensorPlan& tp, int device, const bf16* cac
     b.s_chunks = (dm.S + BWD_KR - 1) / BWD_KR;
     b.r_blocks = (dm.r + 63) / 64;
     b.terms = dt; b.gen = gen ? 1 : 0;
-    const int n_cols = gen && dt == 2 && dm.r <= 128 ? 128 * b.r_blocks : r_pad;
+    const int n_cols = gen && dm.r <= 128 ? 128 * b.r_blocks : r_pad;
     b.chunks = (dm.d >= 256 && 2 * n_cols <= 512) ? 2 : 1;
     b.d_groups = (dm.d + 128 * b.chunks - 1) / (128 * b.chunks);
     b.tmem_cols = pow2_at_least(b.chunks * n_cols);
@@ -1022,9 +1023,7 @@ inline pac_status tensor_dw_down(TensorPlan& tp, cudaStream_t stream, const int*
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[1];
     pdl_launch_config(&cfg, attr, dim3((unsigned)grid), dim3(DW_THREADS), tp.smem_bwd, stream);
-    const auto kernel = !p.gen ? dw_down_tc_kernel<0, 1> : p.r <= 64 ? dw_down_tc_kernel<1, 2>
-                      : p.r <= 128 ? (p.terms == 2 ? dw_down_tc_kernel<2, 2> : dw_down_tc_kernel<2, 1>)
-                                   : (p.terms == 2 ? dw_down_tc_kernel<4, 2> : dw_down_tc_kernel<4, 1>);
+    const auto kernel = !p.gen ? dw_down_tc_kernel<0> : p.r <= 64 ? dw_down_tc_kernel<1> : p.r <= 128 ? dw_down_tc_kernel<2> : dw_down_tc_kernel<4>;
     cudaError_t e = smem_opt_in((const void*)kernel, tp.smem_bwd);
     if (e != cudaSuccess) { tensor_err() = cudaGetErrorString(e); return PAC_ERR_CUDA; }
     e = cudaLaunchKernelEx(&cfg, kernel, tp.map_cache_bwd, tp.map_du, p);

@@ -1,0 +1,46 @@
+"""Gradients against the oracle in 64 bits, at sizes where a shortened operand or a drifting accumulation shows.
+
+bf16 caches (identity bodies, so that no gate flips): da_L and W_down enter the tensor-core products as two bf16 terms each, 2^-17 of a value at
+worst and 2^-18 on average; dlambda is a sum of B S r products of either sign, a few times smaller than its terms: 1e-4.  One term is 2^-9.
+fp32 caches: sums of at most 1024 products rounded to 24 bits one by one differ by about 1024^0.5 * 2^-25 = 1e-6; a chain of
+288 additions cut instead of rounded is off by 3e-6 to 5e-6."""
+import numpy as np
+import pytest
+
+import pac_inputs as pi
+from oracle import pac_oracle as po
+from tests.common import Case, block_slices, rel_l2
+
+pytestmark = pytest.mark.gpu
+
+
+def errors(sp, act, force_simt=False, seeds=(3, 4, 5)):
+    case = Case(sp)
+    ctx = case.context(act=act, force_simt=force_simt)
+    worst = {}
+    for seed in seeds:
+        flat = pi.random_params(sp, seed)
+        ctx.set_params(flat)
+        ids = [(3 * i + seed) % sp.N for i in range(sp.B)]
+        ctx.train_step(ids)
+        g = ctx.get_grads()
+        ref = po.flatten(case.oracle_loss_grads(flat, ids, act, dtype=np.float64)[1])
+        for name, sl in block_slices(sp).items():
+            worst[name] = max(worst.get(name, 0.0), rel_l2(g[sl], ref[sl]))
+    path = ctx.kernel_path()
+    ctx.close()
+    return worst, path
+
+
+def bf16(name, **kw):
+    return pi.CacheSpec(name, **{**dict(N=16, L=4, S=64, d=256, dtype="bf16", r=64, n_out=3, B=4), **kw})
+
+
+@pytest.mark.parametrize("sp", [
+    bf16("r_64"), bf16("r_80_one_sample", r=80, B=1, S=40, d=128), bf16("r_96_short", r=96, S=30), bf16("r_128", r=128), bf16("r_128_many", r=128, B=16),
+    bf16("r_128_chain", r=128, S=256, B=8, L=3), bf16("r_192", r=192), bf16("r_256_one_sample", r=256, B=1, S=32),
+], ids=lambda s: s.name)
+def test_tensor_path_keeps_the_bits_of_da(sp):
+    worst, path = errors(sp, act=1)
+    assert path.startswith("tensor")
+    assert worst["lam"] < 1e-4 and worst["W_down"] < 2e-5, worst
