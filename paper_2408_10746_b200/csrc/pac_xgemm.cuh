@@ -5,7 +5,7 @@
 //
 // An fp32 operand enters as the exact sum of three bf16 terms (8 + 8 + 8 mantissa bits), a bf16 one as it is.  Of the products of terms those
 // of relative size 2^-16 and above are formed, six or three; the dropped ones, below 2^-25, are smaller than the rounding of one fp32
-// multiplication.  Sums are fp32.  That is 1365 products per clock and SM against 128 on the FP32 pipe, so the kernel is bound
+// multiplication.  Sums are fp32, in several accumulators (xg_accs).  That is 1365 products per clock and SM against 128 on the FP32 pipe, so the kernel is bound
 // by bringing the operands in: A comes straight from the activation cache (the gather is the address; any row length and alignment),
 // 16 producer warps fetch it into registers, split it and store the swizzled tiles, one warp issues the MMAs.  The producers work in two
 // teams, each filling one of two stages: a team's loads are in flight while the other converts.
@@ -38,7 +38,7 @@ struct XgRows {
     __device__ const float* row(int z, int m) const { return base + z * zstride + (long long)m * ld; }
 };
 
-constexpr int XG_PRODUCERS = 16, XG_THREADS = 32 * (XG_PRODUCERS + 1), XG_TILE = 128, XG_K = 64, XG_MAX_JOBS = 6, XG_TMEM = 128;
+constexpr int XG_PRODUCERS = 16, XG_THREADS = 32 * (XG_PRODUCERS + 1), XG_TILE = 128, XG_K = 64, XG_MAX_JOBS = 6;
 constexpr uint32_t XG_TERM_A = XG_TILE * XG_K * 2, XG_BOX = 64 * 128;
 
 // Products of one launch: several per layer (tn), all layers.
@@ -101,6 +101,15 @@ __device__ __forceinline__ void xg_store(uint32_t a, uint32_t term, const XgF8& 
 template <typename T> struct XgTerms { static constexpr int n = 3; typedef XgF8 reg; };
 template <> struct XgTerms<bf16> { static constexpr int n = 1; typedef uint4 reg; };
 
+// Accumulators of a tile.  The tensor core cuts every partial sum to the accumulator's 24 bits instead of rounding it, an error that grows with the
+// number of additions and not with its root.  The products of first terms therefore take turns, 16 of the reduction at a time, in accumulators of at most 24
+// additions where tensor memory has the columns, and all smaller products have one of their own.  (One for all: against 64 bits u and dW_down were off by
+// 3e-6 to 6e-6 at d = 768 and 1024 to 2048 rows; so by 2e-7 to 3e-7, the FP32 pipe by 6e-7.)
+constexpr int XG_ACC_STEPS = 24;
+inline int xg_accs(int tile_j, int k_steps) {      // beside that of the smaller products
+    const int want = (k_steps + XG_ACC_STEPS - 1) / XG_ACC_STEPS, room = 512 / tile_j - 1;
+    return want < 1 ? 1 : want < room ? want : room;
+}
 __host__ __device__ inline uint32_t xg_term_b(int tile_j) { return (uint32_t)((tile_j + 63) / 64) * XG_BOX; }
 template <class AL>
 inline size_t xg_smem(int tile_j) { return 2 * ((size_t)XgTerms<typename AL::elem>::n * XG_TERM_A + 3 * xg_term_b(tile_j)) + 1024; }
@@ -115,7 +124,7 @@ struct XgTail { int whole, parts; float* ws; unsigned* cnt; };
 // out + s * part_stride and are added up in slice order by whoever reads them.  GB: 8-column groups of B per thread (tile_j = 32 GB at most).
 template <bool TN, int GB, class AL>
 __global__ void __launch_bounds__(XG_THREADS, 1)
-xgemm_kernel(const __grid_constant__ XgJobs<AL> J, int K, int k_slice, float* __restrict__ out, long long zstride, long long part_stride, XgTail tail, unsigned* status) {
+xgemm_kernel(const __grid_constant__ XgJobs<AL> J, int K, int k_slice, int accs_most, float* __restrict__ out, long long zstride, long long part_stride, XgTail tail, unsigned* status) {
     typedef typename AL::elem T;
     constexpr int TA = XgTerms<T>::n;
     extern __shared__ unsigned char smem_raw[];
@@ -151,7 +160,10 @@ xgemm_kernel(const __grid_constant__ XgJobs<AL> J, int K, int k_slice, float* __
         mbar_init(accf, 1);
         fence_mbar_init();
     }
-    if (warp == XG_PRODUCERS) { tmem_alloc(smem_u32(&tmem_base_sh), XG_TMEM); tmem_relinquish(); }
+    const int accs = min(accs_most, max(1, stages * (XG_K / 16)));      // (a short last slice)
+    uint32_t tmem_cols = 32;
+    while (tmem_cols < (uint32_t)((accs + 1) * nj_tile)) tmem_cols *= 2;
+    if (warp == XG_PRODUCERS) { tmem_alloc(smem_u32(&tmem_base_sh), tmem_cols); tmem_relinquish(); }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -161,10 +173,11 @@ xgemm_kernel(const __grid_constant__ XgJobs<AL> J, int K, int k_slice, float* __
     pdl_trigger();      // (not before: a successor may rely on everything ahead of this kernel being complete when it starts)
     if (warp == XG_PRODUCERS) {
         const uint32_t idesc = instr_desc_bf16(XG_TILE, nj_tile, TN ? 1 : 0, 1);
-        // (term of A, term of B), small products first
+        // (term of A, term of B), the product of the first terms last
         constexpr int NP = TA == 3 ? 6 : 3;
         constexpr int pa[6] = {1, 0, 2, 0, 1, 0}, pb[6] = {1, 2, 0, 1, 0, 0};
         bool ok = true;
+        int turn = 0;                               // accumulator of the stage's first product of first terms
         for (int it = 0; it < stages && ok; ++it) {
             const uint32_t s = it & 1u;
             if (!mbar_wait_uniform(full0 + 8 * s, (it >> 1) & 1u, abort_flag, status)) { ok = false; break; }
@@ -172,18 +185,22 @@ xgemm_kernel(const __grid_constant__ XgJobs<AL> J, int K, int k_slice, float* __
             if (elect_one()) {
                 const uint32_t a = ring + s * stage, b = a + TA * XG_TERM_A;
                 const uint64_t ad = TN ? smem_desc_sw128(a, XG_BOX, 1024) : smem_desc_sw128(a, 16, 1024), bd = smem_desc_sw128(b, XG_BOX, 1024);
-#pragma unroll
-                for (int k = 0; k < XG_K / 16; ++k)
+#pragma unroll 1
+                for (int k = 0, at = turn; k < XG_K / 16; ++k) {       // (rolled: a CTA has few stages, its code is fetched from memory)
 #pragma unroll
                     for (int p = 0; p < NP; ++p) {
                         const int ta = TA == 3 ? pa[p] : 0, tb = TA == 3 ? pb[p] : 2 - p;
-                        umma_bf16(tmem_base, ad + (uint64_t)((ta * XG_TERM_A) >> 4) + (uint64_t)(k * (TN ? 128 : 2)),
-                                  bd + (uint64_t)((tb * term_b) >> 4) + (uint64_t)(k * 128), idesc, (it | k | p) ? 1u : 0u);
+                        const bool first = p == NP - 1;
+                        umma_bf16(tmem_base + (uint32_t)((first ? 1 + at : 0) * nj_tile), ad + (uint64_t)((ta * XG_TERM_A) >> 4) + (uint64_t)(k * (TN ? 128 : 2)),
+                                  bd + (uint64_t)((tb * term_b) >> 4) + (uint64_t)(k * 128), idesc, (first ? it * (XG_K / 16) + k >= accs : (it | k | p) != 0) ? 1u : 0u);
                     }
+                    if (++at == accs) at = 0;
+                }
                 umma_commit(empty0 + 8 * s);
                 if (it + 1 == stages) umma_commit(accf);
             }
             __syncwarp();
+            for (turn += XG_K / 16; turn >= accs;) turn -= accs;
         }
     } else {
         const int team = warp >> 3, t = threadIdx.x & 255;
@@ -261,7 +278,22 @@ xgemm_kernel(const __grid_constant__ XgJobs<AL> J, int K, int k_slice, float* __
             const bool vec = !J.trans && (Nj & 3) == 0 && ((uintptr_t)o & 15) == 0;
             for (int c0 = (warp >> 2) * 16; c0 < nj_tile; c0 += 64) {
                 float v[16] = {};
-                if (stages > 0) { tmem_ld16(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)c0, v); tmem_ld_wait(); }
+                if (stages > 0) {
+                    const uint32_t at = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)c0;
+                    float w[16];
+                    tmem_ld16(at, v);                    // the smaller products
+                    tmem_ld16(at + (uint32_t)(accs * nj_tile), w);
+                    tmem_ld_wait();
+#pragma unroll
+                    for (int e = 0; e < 16; ++e) v[e] += w[e];
+#pragma unroll 1
+                    for (int a = accs - 1; a > 0; --a) {
+                        tmem_ld16(at + (uint32_t)(a * nj_tile), w);
+                        tmem_ld_wait();
+#pragma unroll
+                        for (int e = 0; e < 16; ++e) v[e] += w[e];
+                    }
+                }
                 if (!TN && shared_tile >= 0) {
 #pragma unroll
                     for (int e = 0; e < 16; e += 4) *reinterpret_cast<float4*>(ws + c0 + e) = make_float4(v[e], v[e + 1], v[e + 2], v[e + 3]);
@@ -311,7 +343,7 @@ xgemm_kernel(const __grid_constant__ XgJobs<AL> J, int K, int k_slice, float* __
     tc_fence_before();
     __syncthreads();
     drain_after_abort(abort_flag);
-    if (warp == XG_PRODUCERS) tmem_dealloc(tmem_base, XG_TMEM);
+    if (warp == XG_PRODUCERS) tmem_dealloc(tmem_base, tmem_cols);
 }
 
 template <bool TN, class AL>
@@ -323,7 +355,9 @@ inline cudaError_t xgemm_launch(const XgJobs<AL>& J, int K, dim3 grid, int k_sli
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[1];
     pdl_launch_config(&cfg, attr, grid, dim3(XG_THREADS), smem, stream);
-    return cudaLaunchKernelEx(&cfg, kernel, J, K, k_slice, out, zstride, part_stride, tail, status);
+    const int longest = !TN && tail.whole > 0 ? K : K < k_slice ? K : k_slice;      // a CTA's share of the reduction
+    const int accs = xg_accs(J.tile_j, (longest + XG_K - 1) / XG_K * (XG_K / 16));
+    return cudaLaunchKernelEx(&cfg, kernel, J, K, k_slice, accs, out, zstride, part_stride, tail, status);
 }
 template <class AL>
 inline cudaError_t xgemm_launch_tn(const XgJobs<AL>& J, int K, int Z, int slices, float* out, long long zstride, long long part_stride, unsigned* status, cudaStream_t stream) {

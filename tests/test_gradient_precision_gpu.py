@@ -44,3 +44,17 @@ def test_tensor_path_keeps_the_bits_of_da(sp):
     worst, path = errors(sp, act=1)
     assert path.startswith("tensor")
     assert worst["lam"] < 1e-4 and worst["W_down"] < 2e-5, worst
+
+
+def f32(name, **kw):
+    return bf16(name, **{**dict(dtype="f32", L=4, S=128, d=768, B=8, N=12), **kw})
+
+
+@pytest.mark.parametrize("sp", [
+    f32("d_768"), f32("r_128_wide", d=1024, r=128), f32("r_16", r=16, d=512, S=64), f32("two_tiles_d_2048", d=2048, r=144, S=64, B=4, L=2),
+    f32("bf16_cache", dtype="bf16", r=24),
+], ids=lambda s: s.name)
+def test_plain_products_round_like_fp32(sp):
+    worst, _ = errors(sp, act=1, force_simt=True)
+    for name in ("W_down", "W_up", "lam"):
+        assert worst[name] < (1e-6 if name != "lam" else 4e-6), worst            # (lam: a sum of both signs, see above)
