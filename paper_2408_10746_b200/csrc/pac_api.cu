@@ -37,7 +37,6 @@ struct Scratch {
     float* u = nullptr;            // [L][M][r] down-projections
     float* a = nullptr;            // [L][M][r] adapter states
     float* du = nullptr;           // [L][M][r] fp32 (plain path)
-    bf16* du16 = nullptr;          // three terms of du, [L][3][M][r] (transformer bodies on a bf16 cache)
     float* lam_part = nullptr;     // [L][blocks]
     float* loss = nullptr;         // [1]
     // classifier head
@@ -59,7 +58,7 @@ struct Scratch {
     bf16* wup16 = nullptr;
     bf16* dy16 = nullptr;
     // tensor path
-    bf16* wdT = nullptr;           // bf16 terms of W_down, [L][2 or 3][d][r]
+    bf16* wdT = nullptr;           // bf16 terms of W_down, [L][2][d][r]
     float* lm_part = nullptr;      // [slices][...] partial sums of the LM path's two skinny products (dW_up, da_L)
     float* dw_part = nullptr;      // split partials of dW_down
     float* xg_ws = nullptr;        // sums of the tiles that several CTAs share, and their counts (plain path)
@@ -197,7 +196,6 @@ struct pac_ctx {
     unsigned long long* d_stamps = nullptr;
     size_t stamps_used[2] = {0, 0};
     bool tensor_ok = false;
-    bool exact_ok = false;         // the two cache passes run on the tensor cores at fp32 precision (three bf16 terms per fp32 operand)
     long long launches = 0;
     TensorPlan tplan{};
     MidPlan mplan{};               // fused classifier-head kernel (when the shape allows)
@@ -268,7 +266,7 @@ pac_status dmalloc(pac_ctx* c, T** p, long long n) {
 }
 
 bool use_tensor(const pac_ctx* c) { return c->tensor_ok && !c->force_simt; }
-WdShadow wd_shadow(const pac_ctx* c) { return WdShadow{c->sc.wdT, c->exact_ok ? 3 : 2}; }
+WdShadow wd_shadow(const pac_ctx* c) { return WdShadow{c->sc.wdT}; }
 pac_status adam_enqueue(pac_ctx* c, const pac_adamw* hp);
 pac_status down_projection(pac_ctx* c, const int* d_ids, int B);
 pac_status dw_down(pac_ctx* c, const int* d_ids, int B, bool reduce_splits);
@@ -709,7 +707,7 @@ TbLayerParams tb_params(pac_ctx* c, int B, bool train) {
     TbLayerParams p{};
     p.B = B; p.S = c->dm.S; p.r = c->dm.r; p.f = t.f; p.H = t.H; p.train = train ? 1 : 0;
     p.s = t.st;
-    p.u = c->sc.u; p.u_stride = (long long)c->max_rows * c->dm.r; p.du = c->sc.du; p.du3 = c->exact_ok ? c->sc.du16 : nullptr;
+    p.u = c->sc.u; p.u_stride = (long long)c->max_rows * c->dm.r; p.du = c->sc.du;
     p.lam = c->params + c->lay.lam; p.daL = c->sc.daL;
     return p;
 }
@@ -929,7 +927,7 @@ int cls_cluster_size(const pac_ctx* c, int B) {
 pac_status down_projection(pac_ctx* c, const int* d_ids, int B) {
     pac_status st;
     time_mark(c, 0, false);
-    if (use_tensor(c) || c->exact_ok) {
+    if (use_tensor(c)) {
         st = tensor_down_projection(c->tplan, c->stream, d_ids, B, c->sc.u, c->status, &c->launches, next_stamp(c, 0));
         if (st != PAC_OK) return fail(c, st, "tensor-core down-projection launch failed: %s", tensor_last_error());
     } else {
@@ -943,15 +941,14 @@ pac_status down_projection(pac_ctx* c, const int* d_ids, int B) {
 pac_status dw_down(pac_ctx* c, const int* d_ids, int B, bool reduce_splits) {
     pac_status st;
     time_mark(c, 2, false);
-    if (use_tensor(c) || c->exact_ok) {
+    if (use_tensor(c)) {
         const Dims& dm = c->dm;
         DuGen gen{};
         const bool lm = c->cfg.head == PAC_HEAD_FROZEN_LM;
         gen.tc = c->sc.tc; gen.da = c->sc.da16; gen.da_term = (long long)(lm ? c->max_rows : c->cfg.max_batch) * dm.r;
         gen.da_sample = lm ? (long long)dm.S * dm.r : dm.r; gen.da_token = lm ? dm.r : 0;
-        st = tensor_dw_down(c->tplan, c->stream, d_ids, B, c->grads + c->lay.w_down, c->sc.dw_part,
-                            reduce_splits, c->status, &c->launches, next_stamp(c, 1),
-                            c->step_early_ids && !c->step_host_ids, &gen);       // ids no kernel in flight writes
+        st = tensor_dw_down(c->tplan, c->stream, d_ids, B, gen, c->sc.dw_part, c->status, &c->launches, next_stamp(c, 1),
+                            c->step_early_ids && !c->step_host_ids);       // ids no kernel in flight writes
         if (st != PAC_OK) return fail(c, st, "tensor-core dW_down launch failed: %s", tensor_last_error());
     } else {
         st = c->dtype == PAC_F32 ? dw_down_simt<float>(c, d_ids, B, reduce_splits) : dw_down_simt<bf16>(c, d_ids, B, reduce_splits);
@@ -1085,10 +1082,10 @@ pac_status finalize_enqueue(pac_ctx* c, const int* d_ids, int B, float* d_loss, 
     Scratch& sc = c->sc;
     FinalizeParams f{};
     f.lay = c->lay; f.B = B; f.d = dm.d; f.r = dm.r; f.C = dm.C; f.L = dm.L;
-    const bool tens = use_tensor(c) || c->exact_ok;
+    const bool tens = use_tensor(c);
     f.dw_part = tens ? sc.dw_part : sc.dw_spart;
     f.splits = tens ? tensor_splits(c->tplan, B) : dw_simt_slices(c, B);
-    if (use_tensor(c)) { f.coef = sc.coef; f.dot_part = sc.dot_part; }
+    if (tens) { f.coef = sc.coef; f.dot_part = sc.dot_part; }
     else if (f.splits <= 1) f.splits = 0;                // already in the gradient buffer
     f.dw_elems = (long long)dm.L * dm.d * dm.r;
     // per-CTA partial sums of dlambda: the fused head kernels', or the plain reverse chain's; transformer bodies: done
@@ -1203,7 +1200,7 @@ pac_status refresh_shadow(pac_ctx* c) {
 void free_all(pac_ctx* c) {
     Scratch& s = c->sc;
     if (c->hc.on) s.hbar = nullptr;            // points into a staging slot, freed below
-    void* ptrs[] = {s.ids, s.u, s.a, s.du, s.du16, s.lam_part, s.loss, s.hbar, s.pooled_a, s.pooled_y, s.logits,
+    void* ptrs[] = {s.ids, s.u, s.a, s.du, s.lam_part, s.loss, s.hbar, s.pooled_a, s.pooled_y, s.logits,
                     s.dlogits, s.loss_b, s.gvec, s.daL, s.y, s.lm_logits, s.dy, s.y16, s.dlog16, s.aL16, s.wup16, s.dy16, s.wdT, s.lm_part, s.dw_part, s.dw_spart, s.xg_ws, s.xg_cnt, s.tc, s.da16, s.coef, s.dot_part, s.pool_part, s.prodW, c->tb.buf, c->params, c->grads,
                     c->m, c->v, c->status, c->d_perm, c->d_stamps};
     for (void* p : ptrs)
@@ -1496,13 +1493,12 @@ pac_status pac_adapter_init(pac_ctx* c, const pac_adapter_cfg* cfg, unsigned lon
         A(dmalloc(c, &s.da16, 2LL * (cls ? (long long)cfg->max_batch * dm.r : Mr)));
         long long part_floats = 0;
         if (st == PAC_OK) {
-            pac_status ts = tensor_plan_create(c->tplan, c->device, (const bf16*)c->cache, dm, cfg->max_batch, s.wdT,
-                                               nullptr, &part_floats);
+            pac_status ts = tensor_plan_create(c->tplan, c->device, (const bf16*)c->cache, dm, cfg->max_batch, s.wdT, &part_floats);
             if (ts == PAC_OK && c->hc.on) {
                 // one set of tensor maps per staging slot
                 c->hc.tplan[0] = c->tplan;
                 long long pf2 = 0;
-                ts = tensor_plan_create(c->hc.tplan[1], c->device, (const bf16*)c->hc.stage[1], dm, cfg->max_batch, s.wdT, nullptr, &pf2);
+                ts = tensor_plan_create(c->hc.tplan[1], c->device, (const bf16*)c->hc.stage[1], dm, cfg->max_batch, s.wdT, &pf2);
             }
             if (ts == PAC_OK) {
                 A(dmalloc(c, &s.dw_part, part_floats));
@@ -1603,27 +1599,10 @@ pac_status pac_adapter_init(pac_ctx* c, const pac_adapter_cfg* cfg, unsigned lon
         }
         }
     }
-    // transformer bodies on a bf16 cache: the cache passes alone, at the precision of the fp32 kernels around them
-    c->exact_ok = false;
-    if (st == PAC_OK && c->dtype == PAC_BF16 && tensor_shape_supported(dm) && c->tb.plan.ok && !c->force_simt) {
-        A(dmalloc(c, &s.wdT, (long long)dm.L * 3 * dm.r * dm.d));
-        A(dmalloc(c, &s.du16, 3 * Mr * dm.L));
-        long long part_floats = 0;
-        if (st == PAC_OK) {
-            pac_status ts = tensor_plan_create(c->tplan, c->device, (const bf16*)c->cache, dm, cfg->max_batch, s.wdT, s.du16, &part_floats, true);
-            if (ts == PAC_OK) {
-                A(dmalloc(c, &s.dw_part, part_floats));
-                c->exact_ok = st == PAC_OK;
-            } else if (ts != PAC_ERR_UNSUPPORTED) {
-                st = fail(c, ts, "tensor path set-up failed: %s", tensor_last_error());
-            }
-        }
-    }
     if (st != PAC_OK) return st;
     CU_OK(c, cudaMemsetAsync(s.u, 0, sizeof(float) * Mr * dm.L, c->stream));
     CU_OK(c, cudaMemsetAsync(s.a, 0, sizeof(float) * Mr * dm.L, c->stream));
     if (s.du) CU_OK(c, cudaMemsetAsync(s.du, 0, sizeof(float) * Mr * dm.L, c->stream));
-    if (s.du16) CU_OK(c, cudaMemsetAsync(s.du16, 0, sizeof(bf16) * Mr * dm.L * (c->exact_ok ? 3 : 1), c->stream));
     CU_OK(c, cudaMemsetAsync(c->grads, 0, sizeof(float) * c->lay.total, c->stream));
     CU_OK(c, cudaMemsetAsync(c->m, 0, sizeof(float) * c->lay.total, c->stream));
     CU_OK(c, cudaMemsetAsync(c->v, 0, sizeof(float) * c->lay.total, c->stream));

@@ -74,30 +74,24 @@ __device__ __forceinline__ void split3_pair(float x, float y, uint32_t& h, uint3
     l = bf16_pair(x, y);
 }
 
-// bf16 terms of W_down for the tensor-core products, [L][terms][d][r] in the master's order: term 0 = bf16(W), term 1 = bf16(W -
-// term 0), ...; two terms carry about 16 mantissa bits, three the fp32 value exactly.
+// bf16 terms of W_down for the tensor-core products, [L][2][d][r] in the master's order: hi = bf16(W), lo = bf16(W - hi), together about 16
+// mantissa bits.
 struct WdShadow {
-    bf16* p; int terms;
+    bf16* p;
     // x into the terms of one element, `dr` apart.
     __device__ __forceinline__ void put(long long at, long long dr, float x) const {
         const bf16 a = __float2bfloat16(x);
-        x -= __bfloat162float(a);
-        const bf16 b = __float2bfloat16(x);
-        p[at] = a; p[at + dr] = b;
-        if (terms == 3) p[at + 2 * dr] = __float2bfloat16(x - __bfloat162float(b));
+        p[at] = a; p[at + dr] = __float2bfloat16(x - __bfloat162float(a));
     }
     __device__ __forceinline__ void put4(long long at, long long dr, const float (&x)[4]) const {
-        bf16 v[3][4];
+        bf16 v[2][4];
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
             v[0][e] = __float2bfloat16(x[e]);
-            const float y = x[e] - __bfloat162float(v[0][e]);
-            v[1][e] = __float2bfloat16(y);
-            v[2][e] = __float2bfloat16(y - __bfloat162float(v[1][e]));
+            v[1][e] = __float2bfloat16(x[e] - __bfloat162float(v[0][e]));
         }
         *reinterpret_cast<uint2*>(p + at) = *reinterpret_cast<const uint2*>(v[0]);
         *reinterpret_cast<uint2*>(p + at + dr) = *reinterpret_cast<const uint2*>(v[1]);
-        if (terms == 3) *reinterpret_cast<uint2*>(p + at + 2 * dr) = *reinterpret_cast<const uint2*>(v[2]);
     }
 };
 // Layer of element i of the W_down block (dr = d r elements each): a 32-bit division where the block's size allows it.

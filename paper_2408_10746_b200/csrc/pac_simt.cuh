@@ -518,7 +518,7 @@ __device__ __forceinline__ void adamw_element(float* __restrict__ p, float* __re
     p[i] = th;
     if (wdT.p && i < lay.lam) {
         const long long dr = (long long)d * r, l = wd_layer(i, lay.lam, (unsigned)dr);
-        wdT.put(i + l * (wdT.terms - 1) * dr, dr, th);
+        wdT.put(i + l * dr, dr, th);
     }
 }
 
@@ -538,7 +538,7 @@ __device__ __forceinline__ void adamw_w_down4_loaded(float* __restrict__ p, floa
     if (wdT.p) {
         const long long dr = (long long)d * r;
         const float th[4] = {p4.x, p4.y, p4.z, p4.w};
-        wdT.put4(i + l * (wdT.terms - 1) * dr, dr, th);
+        wdT.put4(i + l * dr, dr, th);
     }
 }
 
@@ -577,7 +577,7 @@ __global__ void shadow_wdown_kernel(const float* __restrict__ w, WdShadow wdT, i
     long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= (long long)L * d * r) return;
     const long long dr = (long long)d * r, l = i / dr;
-    wdT.put(i + l * (wdT.terms - 1) * dr, dr, w[i]);
+    wdT.put(i + l * dr, dr, w[i]);
 }
 
 }  // namespace pac

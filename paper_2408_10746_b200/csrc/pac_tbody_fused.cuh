@@ -97,7 +97,7 @@ struct TbLayerParams {
     int ka, kb, rs, ss;                // row strides in shared memory: wide and narrow operand terms (bf16), fp32 rows, score rows
     TbStacks s;
     const float* u; long long u_stride;
-    float* du; bf16* du3;              // backward: fp32 [L][M][r], u_stride apart, or its three bf16 terms [L][3][M][r]
+    float* du;                         // backward: [L][M][r], u_stride apart
     const float* lam;
     const float *g1, *b1, *g2, *b2, *c1, *c2;      // parameter vectors: forward g1, b1 of `head`, the rest of `tail`; backward g1 of `tail`, g2 of `head`
     const float* daL;                  // [B][r]
@@ -731,15 +731,7 @@ __global__ void __launch_bounds__(TBF_THREADS) tb_bwd_kernel(const __grid_consta
                     if (ph) s.dx1[o + e] = y;
                     else {
                         acc = fmaf(y, __ldg(u + e) - (ap ? __ldg(ap + e) : 0.f), acc);
-                        const float duv = lm * y;
-                        if (p.du3) {
-                            uint32_t h, m, lo;
-                            split3_pair(duv, 0.f, h, m, lo);
-                            uint16_t* w = reinterpret_cast<uint16_t*>(p.du3) + 3 * l * p.u_stride + m0 * r + e;
-                            w[0] = (uint16_t)h; w[p.u_stride] = (uint16_t)m; w[2 * p.u_stride] = (uint16_t)lo;
-                        } else {
-                            p.du[l * p.u_stride + m0 * r + e] = duv;
-                        }
+                        p.du[l * p.u_stride + m0 * r + e] = lm * y;
                         y *= 1.f - lm;
                         if (p.head >= 0) s.da[p.head * s.sMr + m0 * r + e] = y;
                     }

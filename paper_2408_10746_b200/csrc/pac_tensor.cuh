@@ -314,8 +314,7 @@ struct FwdParams {
     int stages;
     int tmem_cols;                         // power of two >= 2 * r_pad
     int acc_stride;                        // column offset of the second accumulator
-    int terms;                             // bf16 terms of W_down: 2 (hi + lo), or 3 (the fp32 value exactly)
-    int wide_n;                            // 1: the terms' blocks form one N = 64 * terms * r_blocks MMA, summed in the epilogue
+    int wide_n;                            // 1: hi and lo blocks form one N = 128*r_blocks MMA, summed in the epilogue
     float* u; long long layer_stride;      // u[l][m][j], layer_stride = max_rows * r
     unsigned* status;
     unsigned long long* stamp;             // optional stream-phase timestamps (see stamp_begin)
@@ -326,7 +325,7 @@ struct FwdParams {
 // straight from the cache.  B tile: 64 rows of W_down^l in its natural [d][r] order (an
 // MN-major operand), split into two bf16 terms (hi = bf16(W), lo = bf16(W - hi); shadow
 // [L][2][d][r]); both products accumulate into the same fp32 accumulator, so the weights
-// enter with about 16 mantissa bits, or with a third term exactly.  (With bf16-rounded weights alone the ReLU masks of about one element in a
+// enter with about 16 mantissa bits.  (With bf16-rounded weights alone the ReLU masks of about one element in a
 // thousand flip, which alone costs ~3% relative error in dW_down and dlambda.)
 // Persistent CTAs walk tiles (layer, sample, token chunk); accumulators are double-buffered
 // in TMEM so the epilogue of one tile overlaps the loads and MMAs of the next.
@@ -338,7 +337,7 @@ down_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_cache, const __grid_c
     const int r_pad = (p.r + 7) & ~7;
     const int r_blocks = (p.r + 63) >> 6;
     const uint32_t a_bytes = FWD_ROWS * KC * 2, b_box = KC * 128;            // one [64 k][64 columns of r] box
-    const uint32_t rb_bytes = (uint32_t)p.terms * b_box, b_bytes = (uint32_t)r_blocks * rb_bytes;      // [r block][term][64 k][128 B]
+    const uint32_t b_bytes = (uint32_t)r_blocks * 2 * b_box;                 // [r block][hi|lo][64 k][128 B]
     const uint32_t b_off = a_bytes, stage_bytes = a_bytes + b_bytes;
     __shared__ __align__(8) unsigned long long bars[2 * 16 + 4];
     __shared__ uint32_t tmem_base_sh;
@@ -388,7 +387,7 @@ down_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_cache, const __grid_c
                     mbar_expect_tx(full, a_bytes + b_bytes);
                     tma_load_4d_hint(dst, &map_cache, full, kc * KC, sc * FWD_ROWS, l, id, pol);
                     for (int rb = 0; rb < r_blocks; ++rb)
-                        tma_load_4d(dst + b_off + rb * rb_bytes, &map_w, full, rb * 64, kc * KC, 0, l);
+                        tma_load_4d(dst + b_off + rb * 2 * b_box, &map_w, full, rb * 64, kc * KC, 0, l);
                 }
                 __syncwarp();
                 dst += stage_bytes;
@@ -396,14 +395,14 @@ down_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_cache, const __grid_c
             }
         }
     } else if (warp == 1) {
-        // wide_n: the terms' blocks lie next to each other along N ([r block][term] in 64-column
-        // blocks), so one MMA of N = 64 * terms * r_blocks yields the terms' sums side by side in TMEM
-        const uint32_t idesc = p.wide_n ? instr_desc_bf16(FWD_ROWS, 64 * p.terms * r_blocks, 0, 1) : instr_desc_bf16(FWD_ROWS, r_pad, 0, 1);
+        // wide_n: the hi and lo blocks lie next to each other along N ([r block][hi|lo] in 64-column
+        // blocks), so one MMA of N = 128 * r_blocks yields u_hi | u_lo side by side in TMEM
+        const uint32_t idesc = p.wide_n ? instr_desc_bf16(FWD_ROWS, 128 * r_blocks, 0, 1) : instr_desc_bf16(FWD_ROWS, r_pad, 0, 1);
         // descriptors of a stage's first 16-wide K step (start-address field in 16-byte units); later steps
         // only move the start address: +32 B per step in the K-major A tile, +2048 B (16 rows) in B
         const uint32_t ring0 = smem_u32(smem);
         const uint64_t a_desc0 = smem_desc_sw128(ring0, 16, 1024), bw_desc0 = smem_desc_sw128(ring0 + b_off, b_box, 1024);
-        const uint64_t bh_desc0 = smem_desc_sw128(ring0 + b_off, rb_bytes, 1024), term_step = (uint64_t)(b_box >> 4);
+        const uint64_t bh_desc0 = smem_desc_sw128(ring0 + b_off, 2 * b_box, 1024), term_step = (uint64_t)(b_box >> 4);
         const uint64_t desc_step = (uint64_t)(stage_bytes >> 4);
         uint64_t doff = 0;
         uint32_t s = 0, ph = 0, tile_n = 0;
@@ -429,7 +428,6 @@ down_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_cache, const __grid_c
                         for (int k = 0; k < KC / 16; ++k) {
                             umma_bf16(d_tmem, ad0 + (uint64_t)(k * 2), bh0 + (uint64_t)(k * 128), idesc, (kc | k) ? 1u : 0u);
                             umma_bf16(d_tmem, ad0 + (uint64_t)(k * 2), bh0 + term_step + (uint64_t)(k * 128), idesc, 1u);
-                            if (p.terms == 3) umma_bf16(d_tmem, ad0 + (uint64_t)(k * 2), bh0 + 2 * term_step + (uint64_t)(k * 128), idesc, 1u);
                         }
                     }
                     umma_commit(empty0 + 8 * s);          // frees the smem slot once these MMAs are done
@@ -459,19 +457,12 @@ down_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_cache, const __grid_c
             for (int c0 = 0; c0 < p.r; c0 += 16) {
                 float v[16];
                 if (p.wide_n) {
-                    // column c of u: first term at TMEM column (c/64)*64*terms + c%64, the next 64 columns further
+                    // column c of u: hi part at TMEM column (c/64)*128 + c%64, lo part 64 columns further
                     float w[16];
-                    const uint32_t col = (uint32_t)((c0 >> 6) * 64 * p.terms + (c0 & 63));
+                    const uint32_t col = (uint32_t)((c0 >> 6) * 128 + (c0 & 63));
                     tmem_ld16(taddr + col, v);
                     tmem_ld16(taddr + col + 64, w);
                     tmem_ld_wait();
-                    if (p.terms == 3) {
-                        float x[16];
-                        tmem_ld16(taddr + col + 128, x);
-                        tmem_ld_wait();
-#pragma unroll
-                        for (int c = 0; c < 16; ++c) w[c] += x[c];
-                    }
 #pragma unroll
                     for (int c = 0; c < 16; ++c) v[c] += w[c];
                 } else {
@@ -505,16 +496,14 @@ struct BwdParams {
     int chunks;                            // 128-column blocks of h per CTA (accumulators in TMEM)
     int splits;                            // row splits J: partial sums per output
     int r_blocks;                          // ceil(r / 64)
-    int terms;                             // bf16 terms of du: 1, or 3 (the fp32 value exactly); term t of layer l at l * terms + t of the du map
     int stages;
     int tmem_cols;
     int early_ids;                         // 1: no kernel ahead of this one in the stream writes the ids
-    // gen: du_l is not read but built in shared memory from one byte per element (see MidParams in pac_mid.cuh) and da_L, one vector per
+    // du_l is not read but built in shared memory from one byte per element (see MidParams in pac_mid.cuh) and da_L, one vector per
     // sample or token, in two bf16 terms: B = open_l ? da : 0, out = h_l^T B without the layer's factor.
-    int gen;
     const uint8_t* tc;                     // [max_rows][r]
     const bf16* da; long long da_term, da_sample; int da_token;      // strides in elements
-    float* out;                            // splits == 1 and not gen: dW_down [L][d][r]; else partials [J][L][d][r]
+    float* out;                            // [J][L][d][r], a sum per row split
     unsigned* status;
     unsigned long long* stamp;             // optional stream-phase timestamps (see stamp_begin)
 };
@@ -524,27 +513,27 @@ struct BwdParams {
 // it streams 64-token tiles of h_l (MN-major A: the 128 output rows are h's columns) and of
 // du_l (MN-major B: N = r), accumulates [128 x r] blocks in TMEM over all its rows and writes
 // them once.  With splits > 1 the partial sums are added afterwards in split order.
-// Generated du: warps 2 - 9, idle until the accumulators are complete, fill the B part of every stage.  That takes the
+// du tiles: warps 2 - 9, idle until the accumulators are complete, fill the B part of every stage.  That takes the
 // L * M * r * 2 bytes of du out of memory in both directions; the tile costs five integer instructions per four elements.
 // Gate bytes: a builder that loads them itself runs at two stages per memory latency (1.1 us a stage).  At two and more groups per thread, whose
 // registers allow no deeper look-ahead, they therefore come through the stage ring with the h tile (S = 256, B = 64, L = 24, d = 1024, r = 128:
 // 187 -> 154 us, the rate of the memory).  With one group the ring was slower by 0.7 us: short loops, and one more hop before the first product.
-// GQ: 16-column groups of a generated tile per thread (r = 64 GQ at most; 0: du comes through TMA).  Registers are
+// GQ: 16-column groups of a du tile per thread (r = 64 GQ at most).  Registers are
 // bounded so that three finalisation blocks fit beside a CTA (r <= 64; with 155 instead of 88 the step took 58 us for 53).
 // ---------------------------------------------------------------------------
 template <int GQ>
 __global__ void __launch_bounds__(DW_THREADS) __maxnreg__(GQ <= 1 ? 88 : 168)
-dw_down_tc_kernel(const __grid_constant__ CUtensorMap map_cache, const __grid_constant__ CUtensorMap map_du, BwdParams p) {
-    constexpr bool GEN = GQ > 0, RING = GQ > 1;                   // RING: gate bytes through the stage ring, else straight into registers
-    constexpr int GT = 2;                                         // terms of a generated tile
+dw_down_tc_kernel(const __grid_constant__ CUtensorMap map_cache, BwdParams p) {
+    constexpr bool RING = GQ > 1;                                 // gate bytes through the stage ring, else straight into registers
+    constexpr int GT = 2;                                         // terms of a du tile
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     const int r_pad = (p.r + 15) & ~15;
     const uint32_t box_bytes = BWD_KR * 128;                       // one [64 tokens][64 columns] box
-    const uint32_t a_bytes = (uint32_t)p.chunks * 2 * box_bytes, b_bytes = (uint32_t)(p.r_blocks * (GEN ? GT : p.terms)) * box_bytes;
-    const uint32_t tx_bytes = GEN ? a_bytes : a_bytes + b_bytes, g_off = a_bytes + b_bytes;      // a stage: h tile, du tile, gate bytes
+    const uint32_t a_bytes = (uint32_t)p.chunks * 2 * box_bytes, b_bytes = (uint32_t)(p.r_blocks * GT) * box_bytes;
+    const uint32_t g_off = a_bytes + b_bytes;                      // a stage: h tile, du tile, gate bytes
     const uint32_t stage_bytes = g_off + (RING ? (uint32_t)(BWD_KR * p.r) : 0u);
-    constexpr bool side = GEN && GQ <= 2;                          // the terms side by side along N, added up in the epilogue
+    constexpr bool side = GQ <= 2;                                 // the terms side by side along N, added up in the epilogue
     const int n_cols = side ? 128 * p.r_blocks : r_pad;            // TMEM columns per accumulator
     __shared__ __align__(8) unsigned long long bars[3 * 16 + 1];
     __shared__ uint32_t tmem_base_sh;
@@ -562,11 +551,10 @@ dw_down_tc_kernel(const __grid_constant__ CUtensorMap map_cache, const __grid_co
 
     if (threadIdx.x == 0) {
         abort_sh = 0;
-        for (int s = 0; s < p.stages; ++s) { mbar_init(full0 + 8 * s, GEN ? 1 + DW_GEN_WARPS : 1); mbar_init(empty0 + 8 * s, 1); mbar_init(gate0 + 8 * s, 1); }
+        for (int s = 0; s < p.stages; ++s) { mbar_init(full0 + 8 * s, 1 + DW_GEN_WARPS); mbar_init(empty0 + 8 * s, 1); mbar_init(gate0 + 8 * s, 1); }
         mbar_init(accf, 1);
         fence_mbar_init();
         tma_prefetch_desc(&map_cache);
-        if (!GEN) tma_prefetch_desc(&map_du);
     }
     if (warp == 1) { tmem_alloc(smem_u32(&tmem_base_sh), (uint32_t)p.tmem_cols); tmem_relinquish(); }
     tc_fence_before();
@@ -585,7 +573,7 @@ dw_down_tc_kernel(const __grid_constant__ CUtensorMap map_cache, const __grid_co
                 const int rt = rt0 + (int)i, sc = rt % p.s_chunks, b = rt / p.s_chunks;
                 const int id = (int)safe_id(p.ids, b, p.N, nullptr);
                 const uint32_t dst = smem_u32(smem + (size_t)i * stage_bytes);
-                mbar_expect_tx(full0 + 8 * i, tx_bytes);
+                mbar_expect_tx(full0 + 8 * i, a_bytes);
                 for (int q = 0; q < 2 * p.chunks; ++q)
                     tma_load_4d_hint(dst + q * box_bytes, &map_cache, full0 + 8 * i, col0 + q * 64, sc * BWD_KR, l, id, pol);
             }
@@ -618,18 +606,13 @@ dw_down_tc_kernel(const __grid_constant__ CUtensorMap map_cache, const __grid_co
                 // first ring: the h tiles are already on their way
                 --pre;
                 if (RING && elect_one()) load_gates();
-                if (!GEN && elect_one())
-                    for (int q = 0; q < p.r_blocks * p.terms; ++q)
-                        tma_load_3d(dst + a_bytes + q * box_bytes, &map_du, full, (q % p.r_blocks) * 64, b * p.S + sc * BWD_KR, l * p.terms + q / p.r_blocks);
             } else {
                 if (!mbar_wait_uniform(empty0 + 8 * s, eph, abort_flag, p.status)) break;
                 if (elect_one()) {
                     if (RING) load_gates();
-                    mbar_expect_tx(full, tx_bytes);
+                    mbar_expect_tx(full, a_bytes);
                     for (int q = 0; q < 2 * p.chunks; ++q)
                         tma_load_4d_hint(dst + q * box_bytes, &map_cache, full, col0 + q * 64, sc * BWD_KR, l, id, pol);
-                    for (int q = 0; q < p.r_blocks * p.terms && !GEN; ++q)
-                        tma_load_3d(dst + a_bytes + q * box_bytes, &map_du, full, (q % p.r_blocks) * 64, b * p.S + sc * BWD_KR, l * p.terms + q / p.r_blocks);
                 }
             }
             __syncwarp();
@@ -642,7 +625,7 @@ dw_down_tc_kernel(const __grid_constant__ CUtensorMap map_cache, const __grid_co
         }
     } else if (warp == 1) {
         const uint32_t idesc = instr_desc_bf16(128, n_cols, 1, 1);
-        const int passes = side ? 1 : GEN ? GT : p.terms;          // products per K step and column block
+        constexpr int passes = side ? 1 : GT;                      // products per K step and column block
         // descriptors of a stage's first K step (start-address field in 16-byte units)
         const uint32_t ring0 = smem_u32(smem);
         const uint64_t a_desc0 = smem_desc_sw128(ring0, box_bytes, 1024), b_desc0 = smem_desc_sw128(ring0 + a_bytes, box_bytes, 1024);
@@ -679,8 +662,8 @@ dw_down_tc_kernel(const __grid_constant__ CUtensorMap map_cache, const __grid_co
         const int e16 = ((warp - 2) >> 2) * 16;                   // this warp's first 16 columns of every 32; the quadrant's two warps share them
         const uint32_t tq = tmem_base + ((uint32_t)(q * 32) << 16);
         bool ok = true;
-        // ---- generated tiles: group g of a stage = 16 columns of one token; this thread's groups lie 256 apart ----
-        if constexpr (GEN) {
+        // ---- du tiles: group g of a stage = 16 columns of one token; this thread's groups lie 256 apart ----
+        {
             constexpr int AHEAD = GQ < 4 ? 2 : 1;                 // stages whose da (and gates) are in registers ahead of use
             int row[GQ], cg[GQ], f_rt = rt0, f_sc = rt0 % p.s_chunks, f_b = rt0 / p.s_chunks, left = p.S - f_sc * BWD_KR;      // left: tokens from the stage's first on
             uint32_t off[GQ], gs = 0, gph = 0, gdst = smem_u32(smem);
@@ -812,7 +795,7 @@ struct TensorPlan {
     bool ready = false;
     Dims dm{};
     int max_batch = 0, sms = 0;
-    CUtensorMap map_cache_fwd, map_cache_bwd, map_w, map_du;
+    CUtensorMap map_cache_fwd, map_cache_bwd, map_w;
     FwdParams fp{};
     BwdParams bp{};
     size_t smem_fwd = 0, smem_bwd = 0;
@@ -875,12 +858,10 @@ inline bool make_map(CUtensorMap* map, const void* base, int rank, const cuuint6
 
 inline int pow2_at_least(int x) { int p = 32; while (p < x) p <<= 1; return p; }
 
-// wdT: [L][2][d][r] bf16 hi/lo shadow of W_down; du16: [L][max_rows][r] bf16; exact: three terms of either ([L][3][d][r],
-// [L][3][max_rows][r]), whose sum is the fp32 value, so the products are those of fp32 operands.  *part_floats receives the
+// wdT: [L][2][d][r] bf16 hi/lo shadow of W_down.  *part_floats receives the
 // size of the split-partial buffer dW needs (0 when no split is used).
 inline pac_status tensor_plan_create(TensorPlan& tp, int device, const bf16* cache, const Dims& dm, int max_batch,
-                                     const bf16* wdT, const bf16* du16, long long* part_floats, bool exact = false) {
-    const bool gen = !exact;                                 // du is generated (pointwise bodies)
+                                     const bf16* wdT, long long* part_floats) {
     tp.ready = false;
     tp.dm = dm;
     tp.max_batch = max_batch;
@@ -891,11 +872,10 @@ inline pac_status tensor_plan_create(TensorPlan& tp, int device, const bf16* cac
     const int max_smem = (int)prop.sharedMemPerBlockOptin;
     const long long max_rows = (long long)max_batch * dm.S;
     const int r_pad = (dm.r + 15) & ~15;
-    const int wt = exact ? 3 : 2;                            // bf16 terms of W_down
-    // of du: the fp32 value exactly, or generated: two terms of da, as dlambda, which comes from the same product, needs them: against 64 bits it is
+    // Terms of da: dlambda, which comes from the same product as dW_down, needs two: against 64 bits it is
     // off by 1e-3 to 8e-3 with one and by 2e-6 to 2e-5 with two.  Up to r = 64 the second term's products cost nothing beside the stream; at
     // B = 64, S = 256, L = 24, d = 1024, r = 128 the step takes 465 us for 430.
-    const int dt = exact ? 3 : 2;
+    constexpr int dt = 2;
 
     // ---- tensor maps ----
     {
@@ -906,17 +886,10 @@ inline pac_status tensor_plan_create(TensorPlan& tp, int device, const bf16* cac
         if (!make_map(&tp.map_cache_bwd, cache, 4, dims, str, box_b)) return PAC_ERR_UNSUPPORTED;
     }
     {
-        cuuint64_t dims[4] = {(cuuint64_t)dm.r, (cuuint64_t)dm.d, (cuuint64_t)wt, (cuuint64_t)dm.L};
-        cuuint64_t str[3] = {(cuuint64_t)dm.r * 2, (cuuint64_t)dm.r * dm.d * 2, (cuuint64_t)wt * dm.r * dm.d * 2};
-        cuuint32_t box[4] = {64, KC, (cuuint32_t)wt, 1};
+        cuuint64_t dims[4] = {(cuuint64_t)dm.r, (cuuint64_t)dm.d, 2, (cuuint64_t)dm.L};
+        cuuint64_t str[3] = {(cuuint64_t)dm.r * 2, (cuuint64_t)dm.r * dm.d * 2, (cuuint64_t)2 * dm.r * dm.d * 2};
+        cuuint32_t box[4] = {64, KC, 2, 1};
         if (!make_map(&tp.map_w, wdT, 4, dims, str, box)) return PAC_ERR_UNSUPPORTED;
-    }
-    tp.map_du = tp.map_w;                                    // unused when du is generated
-    if (!gen) {
-        cuuint64_t dims[3] = {(cuuint64_t)dm.r, (cuuint64_t)max_rows, (cuuint64_t)dm.L * dt};
-        cuuint64_t str[2] = {(cuuint64_t)dm.r * 2, (cuuint64_t)max_rows * dm.r * 2};
-        cuuint32_t box[3] = {KC, BWD_KR, 1};
-        if (!make_map(&tp.map_du, du16, 3, dims, str, box)) return PAC_ERR_UNSUPPORTED;
     }
 
     // ---- forward plan ----
@@ -924,12 +897,11 @@ inline pac_status tensor_plan_create(TensorPlan& tp, int device, const bf16* cac
     f.N = dm.N; f.L = dm.L; f.S = dm.S; f.d = dm.d; f.r = dm.r;
     f.s_chunks = (dm.S + FWD_ROWS - 1) / FWD_ROWS;
     f.k_chunks = (dm.d + KC - 1) / KC;
-    f.terms = wt;
-    f.wide_n = 64 * wt * ((dm.r + 63) / 64) <= 256 ? 1 : 0;
-    f.tmem_cols = pow2_at_least(2 * (f.wide_n ? 64 * wt * ((dm.r + 63) / 64) : r_pad));
+    f.wide_n = dm.r <= 128 ? 1 : 0;          // N = 128 * r_blocks must stay within 256
+    f.tmem_cols = pow2_at_least(2 * (f.wide_n ? 128 * ((dm.r + 63) / 64) : r_pad));
     f.acc_stride = f.tmem_cols / 2;
     {
-        const int stage = FWD_ROWS * KC * 2 + ((dm.r + 63) / 64) * wt * KC * 128;
+        const int stage = FWD_ROWS * KC * 2 + ((dm.r + 63) / 64) * 2 * KC * 128;
         int st = (max_smem - 2048) / stage;
         if (st > 16) st = 16;
         if (st < 2) { tensor_err() = "not enough shared memory for the forward pipeline"; return PAC_ERR_UNSUPPORTED; }
@@ -943,13 +915,12 @@ inline pac_status tensor_plan_create(TensorPlan& tp, int device, const bf16* cac
     b.N = dm.N; b.L = dm.L; b.S = dm.S; b.d = dm.d; b.r = dm.r;
     b.s_chunks = (dm.S + BWD_KR - 1) / BWD_KR;
     b.r_blocks = (dm.r + 63) / 64;
-    b.terms = dt; b.gen = gen ? 1 : 0;
-    const int n_cols = gen && dm.r <= 128 ? 128 * b.r_blocks : r_pad;
+    const int n_cols = dm.r <= 128 ? 128 * b.r_blocks : r_pad;
     b.chunks = (dm.d >= 256 && 2 * n_cols <= 512) ? 2 : 1;
     b.d_groups = (dm.d + 128 * b.chunks - 1) / (128 * b.chunks);
     b.tmem_cols = pow2_at_least(b.chunks * n_cols);
     {
-        const int stage = (b.chunks * 2 + b.r_blocks * dt) * BWD_KR * 128 + (gen && dm.r > 64 ? BWD_KR * dm.r : 0);
+        const int stage = (b.chunks * 2 + b.r_blocks * dt) * BWD_KR * 128 + (dm.r > 64 ? BWD_KR * dm.r : 0);
         int st = (max_smem - 2048) / stage;
         if (st > 16) st = 16;
         if (st < 2) { tensor_err() = "not enough shared memory for the backward pipeline"; return PAC_ERR_UNSUPPORTED; }
@@ -970,7 +941,7 @@ inline pac_status tensor_plan_create(TensorPlan& tp, int device, const bf16* cac
         b.splits = best;
     }
     tp.dw_elems = (long long)dm.L * dm.d * dm.r;
-    *part_floats = gen || b.splits > 1 ? tp.dw_elems * b.splits : 0;
+    *part_floats = tp.dw_elems * b.splits;
 
     if (smem_opt_in((const void*)down_fwd_tc_kernel, tp.smem_fwd) != cudaSuccess) {
         tensor_err() = "cudaFuncSetAttribute(MaxDynamicSharedMemorySize) failed";
@@ -1008,33 +979,25 @@ inline int tensor_splits(const TensorPlan& tp, int B) {
 // What the second pass builds du from (BwdParams).
 struct DuGen { const uint8_t* tc; const bf16* da; long long da_term, da_sample; int da_token; };
 
-// With reduce_splits == false and more than one split, and always when du is generated, the partial sums stay in `part`
-// ([J][L][d][r]) for the caller's own reduction.
-inline pac_status tensor_dw_down(TensorPlan& tp, cudaStream_t stream, const int* d_ids, int B,
-                                 float* dW, float* part, bool reduce_splits, unsigned* status, long long* launches,
-                                 unsigned long long* stamp = nullptr, bool early_ids = false, const DuGen* gen = nullptr) {
+// The sums of the row splits stay in `part` ([J][L][d][r]) for the caller's own reduction.
+inline pac_status tensor_dw_down(TensorPlan& tp, cudaStream_t stream, const int* d_ids, int B, const DuGen& gen, float* part, unsigned* status,
+                                 long long* launches, unsigned long long* stamp = nullptr, bool early_ids = false) {
     BwdParams p = tp.bp;
-    if (p.gen) { p.tc = gen->tc; p.da = gen->da; p.da_term = gen->da_term; p.da_sample = gen->da_sample; p.da_token = gen->da_token; }
+    p.tc = gen.tc; p.da = gen.da; p.da_term = gen.da_term; p.da_sample = gen.da_sample; p.da_token = gen.da_token;
     p.ids = d_ids; p.B = B; p.status = status; p.stamp = stamp; p.early_ids = early_ids ? 1 : 0;
     const int J = tensor_splits(tp, B);
     p.splits = J;
-    p.out = p.gen || J > 1 ? part : dW;
+    p.out = part;
     const int grid = p.L * p.d_groups * J;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[1];
     pdl_launch_config(&cfg, attr, dim3((unsigned)grid), dim3(DW_THREADS), tp.smem_bwd, stream);
-    const auto kernel = !p.gen ? dw_down_tc_kernel<0> : p.r <= 64 ? dw_down_tc_kernel<1> : p.r <= 128 ? dw_down_tc_kernel<2> : dw_down_tc_kernel<4>;
+    const auto kernel = p.r <= 64 ? dw_down_tc_kernel<1> : p.r <= 128 ? dw_down_tc_kernel<2> : dw_down_tc_kernel<4>;
     cudaError_t e = smem_opt_in((const void*)kernel, tp.smem_bwd);
     if (e != cudaSuccess) { tensor_err() = cudaGetErrorString(e); return PAC_ERR_CUDA; }
-    e = cudaLaunchKernelEx(&cfg, kernel, tp.map_cache_bwd, tp.map_du, p);
+    e = cudaLaunchKernelEx(&cfg, kernel, tp.map_cache_bwd, p);
     (*launches)++;
     if (e != cudaSuccess) { tensor_err() = cudaGetErrorString(e); return PAC_ERR_CUDA; }
-    if (!p.gen && J > 1 && reduce_splits) {
-        reduce_splits_kernel<<<(unsigned)((tp.dw_elems / 4 + 255) / 256), 256, 0, stream>>>(part, J, tp.dw_elems, dW);
-        (*launches)++;
-        e = cudaGetLastError();
-        if (e != cudaSuccess) { tensor_err() = cudaGetErrorString(e); return PAC_ERR_CUDA; }
-    }
     return PAC_OK;
 }
 

@@ -9,7 +9,9 @@ import pytest
 
 import pac_inputs as pi
 from oracle import pac_oracle as po
+from oracle import tbody_oracle as tb
 from tests.common import Case, block_slices, rel_l2
+from tests.test_tbody_gpu import make_ctx, random_flat
 
 pytestmark = pytest.mark.gpu
 
@@ -58,3 +60,25 @@ def test_plain_products_round_like_fp32(sp):
     worst, _ = errors(sp, act=1, force_simt=True)
     for name in ("W_down", "W_up", "lam"):
         assert worst[name] < (1e-6 if name != "lam" else 4e-6), worst            # (lam: a sum of both signs, see above)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_transformer_body_rounds_like_fp32(dtype):
+    """1024 rows and d = 1024: long reductions in both passes over the cache (those of the layers between them are shorter)."""
+    sp, heads, f = bf16("tb", dtype=dtype, L=2, S=256, d=1024, r=16, B=4, N=6), 2, 32
+    ctx = make_ctx(sp, heads, f)
+    ids = [5, 0, 3, 3]
+    H = pi.cache_samples(sp, 0, ids, "cpu").double().numpy()
+    lab = pi.labels(sp, 0, "cpu").numpy().astype(np.int64)[ids]
+    for seed in (3, 4):
+        flat = random_flat(sp, f, seed)
+        ctx.set_params(flat)
+        ctx.train_step(ids)
+        g = ctx.get_grads()
+        P, T = tb.unflatten(flat.astype(np.float64), sp.L, sp.d, sp.r, sp.n_out, f)
+        ref = tb.flatten(*tb.loss_and_grads_cls(P, T, H, lab, heads)[1])
+        body = sum(s.stop - s.start for s in block_slices(sp).values())
+        assert rel_l2(g[body:], ref[body:]) < 1.5e-6
+        for name, sl in block_slices(sp).items():
+            assert rel_l2(g[sl], ref[sl]) < (4e-6 if name == "lam" else 1.5e-6), (name, seed, rel_l2(g[sl], ref[sl]))
+    ctx.close()
