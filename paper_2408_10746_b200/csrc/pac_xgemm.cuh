@@ -114,6 +114,26 @@ __host__ __device__ inline uint32_t xg_term_b(int tile_j) { return (uint32_t)((t
 template <class AL>
 inline size_t xg_smem(int tile_j) { return 2 * ((size_t)XgTerms<typename AL::elem>::n * XG_TERM_A + 3 * xg_term_b(tile_j)) + 1024; }
 
+// Outputs (i, j0 + c) for a warp's columns c of a tile, recomputed in fp32 where the sum of split products is not finite: an infinite operand,
+// or a finite one beyond the largest bf16, has a first term of infinity and no second one, and a partial sum may overflow on the way.
+// dst: the thread's row of sums, `step` apart.
+template <bool TN, class AL>
+__device__ __noinline__ void xg_redo(const AL& A, const XgRows& B, int z, int i, int j0, int c0, int nj_tile, int Nj, int kb, int ke, float* dst, long long step) {
+#pragma unroll 1
+    for (; c0 < nj_tile; c0 += 64)
+#pragma unroll 1
+        for (int c = c0; c < c0 + 16 && j0 + c < Nj; ++c) {
+            if (fabsf(dst[c * step]) <= 3.402823466e38f) continue;
+            float acc = 0.f;
+#pragma unroll 4
+            for (int k = kb; k < ke; ++k) {
+                acc = fmaf(TN ? to_f32(A.row(z, k)[i]) : to_f32(A.row(z, i)[k]), B.row(z, k)[j0 + c], acc);
+                if (acc != acc) break;
+            }
+            dst[c * step] = acc;
+        }
+}
+
 // The tiles of an incomplete last wave (rows): `whole` tiles are computed by one CTA each, every later one by `parts` CTAs that take k_slice
 // of the reduction each, leave their sums in ws and are added up, in order, by the one that finishes last (counted in cnt, which it puts back
 // to zero).  At 192 tiles of 12 stages on 148 SMs
@@ -276,6 +296,7 @@ xgemm_kernel(const __grid_constant__ XgJobs<AL> J, int K, int k_slice, int accs_
             float* o = out + split * part_stride + z * zstride + J.out_off[jb];
             float* ws = tail.ws + ((long long)(shared_tile * tail.parts + split) * XG_TILE + q * 32 + lane) * nj_tile;
             const bool vec = !J.trans && (Nj & 3) == 0 && ((uintptr_t)o & 15) == 0;
+            float odd = 0.f;                             // not zero once an element is not finite
             for (int c0 = (warp >> 2) * 16; c0 < nj_tile; c0 += 64) {
                 float v[16] = {};
                 if (stages > 0) {
@@ -294,6 +315,8 @@ xgemm_kernel(const __grid_constant__ XgJobs<AL> J, int K, int k_slice, int accs_
                         for (int e = 0; e < 16; ++e) v[e] += w[e];
                     }
                 }
+#pragma unroll
+                for (int e = 0; e < 16; ++e) odd = fmaf(v[e], 0.f, odd);
                 if (!TN && shared_tile >= 0) {
 #pragma unroll
                     for (int e = 0; e < 16; e += 4) *reinterpret_cast<float4*>(ws + c0 + e) = make_float4(v[e], v[e + 1], v[e + 2], v[e + 3]);
@@ -311,6 +334,10 @@ xgemm_kernel(const __grid_constant__ XgJobs<AL> J, int K, int k_slice, int accs_
                             if (j + x < Nj) o[J.trans ? (long long)(j + x) * Mi + i : (long long)i * Nj + j + x] = v[e + x];
                     }
                 }
+            }
+            if (!(odd == 0.f) && i < Mi) {
+                const bool part = !TN && shared_tile >= 0;
+                xg_redo<TN>(J.A[jb], J.B[jb], z, i, j0, (warp >> 2) * 16, nj_tile, Nj, kb, ke, part ? ws : J.trans ? o + (long long)j0 * Mi + i : o + (long long)i * Nj + j0, J.trans ? Mi : 1);
             }
         }
     }
