@@ -716,12 +716,12 @@ __device__ __forceinline__ bool collect_dots(const float* lam, unsigned long lon
     return *ok_sh != 0;
 }
 // The gradients of W_down (four elements per thread, blocks within one layer each) and lambda (the first block) from the second pass's
-// partial sums where no finalisation kernel follows (L <= 128).
+// partial sums where no finalisation kernel follows (L <= 256).
 __global__ void __launch_bounds__(256) gated_grads_kernel(const float* __restrict__ part, int splits, long long n, int dr, int per_layer, int L,
                                                           const float* __restrict__ w, const float* __restrict__ lam, const float* __restrict__ coef,
                                                           unsigned long long* __restrict__ dot_part, float* __restrict__ gW, float* __restrict__ glam, unsigned* status) {
     if (blockIdx.x == 0) {
-        __shared__ float lam_s[128], dot_s[128];
+        __shared__ float lam_s[256], dot_s[256];
         __shared__ int ok;
         if (collect_dots(lam, dot_part, per_layer, L, lam_s, dot_s, &ok, status))
             for (int k = threadIdx.x; k < L; k += 256) glam[k] = lambda_grad(lam_s, dot_s, L, k);

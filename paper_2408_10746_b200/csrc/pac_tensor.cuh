@@ -121,6 +121,11 @@ __device__ __forceinline__ uint32_t spread_sign(uint32_t x, uint32_t sel) {
     asm("prmt.b32 %0, %1, %1, %2;" : "=r"(d) : "r"(x), "r"(sel));
     return d;
 }
+// Bit 7 of every byte: l >= that byte of t.
+__device__ __forceinline__ uint32_t bytes_ge(int l, uint32_t t) {
+    const uint32_t x = (uint32_t)l * 0x01010101u, low = (x | 0x80808080u) - (t & 0x7f7f7f7fu);
+    return (x & ~t) | (~(x ^ t) & low);
+}
 // True in exactly one lane of a converged warp.
 __device__ __forceinline__ bool elect_one() {
     uint32_t pred;
@@ -669,7 +674,9 @@ dw_down_tc_kernel(const __grid_constant__ CUtensorMap map_cache, BwdParams p) {
             uint32_t off[GQ], gs = 0, gph = 0, gdst = smem_u32(smem);
             const uint32_t open_bias = (uint32_t)(l | 0x80) * 0x01010101u;
             uint4 t4[AHEAD], d4[AHEAD][GQ][2 * GT];
-            const uint4 closed = make_uint4(0x7f7f7f7fu, 0x7f7f7f7fu, 0x7f7f7f7fu, 0x7f7f7f7fu);
+            const bool deep = p.L > 127;                          // layer numbers of eight bits
+            const uint32_t shut = deep ? 0xffffffffu : 0x7f7f7f7fu;
+            const uint4 closed = make_uint4(shut, shut, shut, shut);
             auto fetch = [&](uint4& gates, uint4 (&dd)[GQ][2 * GT]) {
                 if (f_rt >= rt1) return;
 #pragma unroll
@@ -698,7 +705,8 @@ dw_down_tc_kernel(const __grid_constant__ CUtensorMap map_cache, BwdParams p) {
                     if (RING && row[i] < left)
                         asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(t.x), "=r"(t.y), "=r"(t.z), "=r"(t.w) : "r"(gdst + g_off + (threadIdx.x - 64 + 256 * i) * 16) : "memory");
                     // open where l + 1 > tc: bit 7 of (l + 128) - tc, byte by byte, spread over the element's two bytes
-                    const uint32_t y[4] = {open_bias - t.x, open_bias - t.y, open_bias - t.z, open_bias - t.w};
+                    uint32_t y[4] = {open_bias - t.x, open_bias - t.y, open_bias - t.z, open_bias - t.w};
+                    if (deep) { y[0] = bytes_ge(l, t.x); y[1] = bytes_ge(l, t.y); y[2] = bytes_ge(l, t.z); y[3] = bytes_ge(l, t.w); }
                     uint32_t m[8];
 #pragma unroll
                     for (int e = 0; e < 4; ++e) { m[2 * e] = spread_sign(y[e], 0x9988u); m[2 * e + 1] = spread_sign(y[e], 0xbbaau); }
@@ -819,7 +827,7 @@ inline void pdl_launch_config(cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr
 }
 
 inline bool tensor_shape_supported(const Dims& dm) {
-    return dm.d % 8 == 0 && dm.d >= 64 && dm.r % 16 == 0 && dm.r >= 16 && dm.r <= 256 && dm.L <= 127;      // (gate bytes hold a layer number)
+    return dm.d % 8 == 0 && dm.d >= 64 && dm.r % 16 == 0 && dm.r >= 16 && dm.r <= 256 && dm.L <= 255;      // (gate bytes hold a layer number)
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
