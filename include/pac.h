@@ -290,13 +290,15 @@ pac_status pac_sync(pac_ctx* ctx);
  * optimizer update (fused or pac_adam_step) finds the flag and leaves parameters, moments and gradients
  * untouched; pac_sync reports PAC_ERR_TIMEOUT once, clears the flag and takes the skipped updates off the
  * step counter.  Only the step in which the wait ran out can be half applied (when it was the second
- * pass that gave up, the head-side parameters of that step are already updated): restore the last
+ * pass that gave up, the head-side parameters of that step are already updated; when it was the update's own wait
+ * for the parts of lambda's gradient, whose limit is about ten seconds, all but lambda may be): restore the last
  * checkpoint (pac_set_params / pac_set_opt_state) after a PAC_ERR_TIMEOUT unless the timed-out call was
  * pac_selftest_wait_expiry.
  *
  * pac_selftest_wait_expiry exercises that path without breaking anything: one CTA allocates tensor
  * memory, waits limit_ns nanoseconds (1e3 .. 1e8) on a barrier nobody arrives at, and leaves the way the
- * pipeline kernels do after an abort.  The call waits for the stream; it returns PAC_OK when the wait
+ * pipeline kernels do after an abort; another collects parts of lambda's gradient of which one never comes, with a limit of
+ * 64 looks.  The call waits for the stream; it returns PAC_OK when both waits
  * reported expiry, and the status word it set is then reported by the next pac_sync like any other
  * timeout.  The paper describes no failure handling for this path; this is the library's own contract. */
 pac_status pac_selftest_wait_expiry(pac_ctx* ctx, unsigned long long limit_ns);

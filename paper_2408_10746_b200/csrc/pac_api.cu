@@ -2045,21 +2045,30 @@ pac_status pac_selftest_wait_expiry(pac_ctx* c, unsigned long long limit_ns) {
     if (limit_ns < 1000ull || limit_ns > 100000000ull)
         return fail(c, PAC_ERR_INVALID_ARG, "pac_selftest_wait_expiry: limit_ns must lie in [1e3, 1e8]");
     CU_OK(c, cudaSetDevice(c->device));
-    unsigned* d_res = nullptr;
-    CU_OK(c, cudaMalloc((void**)&d_res, 2 * sizeof(unsigned)));
-    unsigned h_res[2] = {0u, 0u};
-    cudaError_t e = cudaMemsetAsync(d_res, 0, 2 * sizeof(unsigned), c->stream);
+    // the results of both tests (one word per half), two lambdas, and a table of shares in which one is missing
+    const unsigned long long share = 1ull << 32 | 0x3f800000u;
+    unsigned long long h[8] = {0, 0, share, share, 0, share, share, share};
+    unsigned long long* d = nullptr;
+    CU_OK(c, cudaMalloc((void**)&d, sizeof h));
+    unsigned* res = (unsigned*)d;
+    cudaError_t e = cudaMemcpyAsync(d, h, sizeof h, cudaMemcpyHostToDevice, c->stream);
     if (e == cudaSuccess) {
-        selftest_wait_expiry_kernel<<<1, 64, 0, c->stream>>>(c->status, limit_ns, d_res);
-        c->launches++;
+        selftest_wait_expiry_kernel<<<1, 64, 0, c->stream>>>(c->status, limit_ns, res);
+        selftest_collect_kernel<<<1, 256, 0, c->stream>>>((const float*)(d + 1), d + 2, c->status, res + 2);
+        c->launches += 2;
         e = cudaGetLastError();
     }
-    if (e == cudaSuccess) e = cudaMemcpyAsync(h_res, d_res, sizeof h_res, cudaMemcpyDeviceToHost, c->stream);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(h, d, sizeof h, cudaMemcpyDeviceToHost, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-    cudaFree(d_res);
+    cudaFree(d);
     if (e != cudaSuccess) return fail(c, PAC_ERR_CUDA, "pac_selftest_wait_expiry: %s", cudaGetErrorString(e));
-    if (h_res[0] != 1u || h_res[1] != 1u)
-        return fail(c, PAC_ERR_BAD_STATE, "pac_selftest_wait_expiry: the wait did not report expiry (expired=%u abort=%u)", h_res[0], h_res[1]);
+    unsigned r[3];
+    std::memcpy(r, h, 2 * sizeof(unsigned));
+    r[2] = (unsigned)h[1];
+    unsigned long long left = 0;
+    for (int k = 2; k < 8; ++k) left |= h[k];
+    if (r[0] != 1u || r[1] != 1u || r[2] != 1u || left != 0)
+        return fail(c, PAC_ERR_BAD_STATE, "pac_selftest_wait_expiry: a wait did not report expiry (expired=%u abort=%u shares=%u left=%llx)", r[0], r[1], r[2], left);
     return PAC_OK;
 }
 

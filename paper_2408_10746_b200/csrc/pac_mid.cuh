@@ -626,8 +626,10 @@ struct FinalizeParams {
     // ring (tag == next_seq), block 0 copies them to device memory, off every kernel's critical path.
     const int* next_host_ids; const unsigned* next_host_tag; unsigned next_seq; int next_n;
     int* next_dev_ids; unsigned* next_dev_tag;
-    // Device status words: when a bounded wait of this or an earlier step has run out, the gradients
-    // are not trustworthy, so nothing is written to the gradients, parameters or moments.
+    // Device status words: when a bounded wait of this step's passes or of an earlier step has run out, the gradients
+    // are not trustworthy, so nothing is written to the gradients, parameters or moments.  The wait for the shares of P_l in this
+    // kernel itself is different: should it run out, lambda stays as it is while blocks that had left their share have
+    // updated what they own, and the caller goes back to a checkpoint.
     unsigned* status;
 };
 
@@ -691,7 +693,7 @@ constexpr int DOT_POLLS = 1 << 24;      // bound on a wait for one share, about 
 // P_l from the blocks' shares, warp per layer, and lambda, into shared memory: one block of 256 threads that runs beside those that publish
 // (it holds one slot, so they all get to run).  False if a share did not arrive; *ok_sh is shared memory.
 __device__ __forceinline__ bool collect_dots(const float* lam, unsigned long long* dot_part, int per_layer, int L, float* lam_s, float* dot_s,
-                                             int* ok_sh, unsigned* status) {
+                                             int* ok_sh, unsigned* status, int polls = DOT_POLLS) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) *ok_sh = 1;
     for (int l = threadIdx.x; l < L; l += 256) lam_s[l] = lam[l];
@@ -701,7 +703,7 @@ __device__ __forceinline__ bool collect_dots(const float* lam, unsigned long lon
         for (int k = lane; k < per_layer; k += 32) {
             unsigned long long* at = dot_part + (long long)l * per_layer + k;
             unsigned long long word = 0;
-            for (int n = 0; n < DOT_POLLS; ++n) {
+            for (int n = 0; n < polls; ++n) {
                 asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(word) : "l"(at) : "memory");
                 if (word != 0ull || *reinterpret_cast<volatile int*>(ok_sh) == 0) break;
             }
@@ -714,6 +716,14 @@ __device__ __forceinline__ bool collect_dots(const float* lam, unsigned long lon
     }
     __syncthreads();
     return *ok_sh != 0;
+}
+// Self-test: collects two layers of three shares with a short limit; the caller has left one share out.  result[0] = 1 if the wait was reported
+// as run out.
+__global__ void __launch_bounds__(256) selftest_collect_kernel(const float* lam, unsigned long long* dot_part, unsigned* status, unsigned* result) {
+    __shared__ float lam_s[2], dot_s[2];
+    __shared__ int ok;
+    const bool all = collect_dots(lam, dot_part, 3, 2, lam_s, dot_s, &ok, status, 64);
+    if (threadIdx.x == 0) result[0] = all ? 0u : 1u;
 }
 // The gradients of W_down (four elements per thread, blocks within one layer each) and lambda (the first block) from the second pass's
 // partial sums where no finalisation kernel follows (L <= 256).
