@@ -652,7 +652,7 @@ pac_status backward(pac_ctx* c, const int* d_ids, int B, float* d_loss, const pa
     }
     if (use_tensor(c)) {
         // the second pass builds du from the gates and da_L: per sample (classifier) or per token (LM)
-        const int nd = (per_sample ? B : M) * dm.r;
+        const long long nd = (long long)(per_sample ? B : M) * dm.r;
         split_terms_kernel<<<cdiv(nd, 256), 256, 0, c->stream>>>(sc.daL, nd, (long long)(per_sample ? c->cfg.max_batch : c->max_rows) * dm.r, sc.da16);
         LAUNCH_CHECK(c);
         pac_status ds = dw_down(c, d_ids, B, false);

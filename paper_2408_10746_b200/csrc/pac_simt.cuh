@@ -225,8 +225,8 @@ __global__ void __launch_bounds__(256) chain_gate_kernel(const float* __restrict
 }
 
 // Two bf16 terms of x, `stride` apart.
-__global__ void __launch_bounds__(256) split_terms_kernel(const float* __restrict__ x, int n, long long stride, bf16* __restrict__ out) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+__global__ void __launch_bounds__(256) split_terms_kernel(const float* __restrict__ x, long long n, long long stride, bf16* __restrict__ out) {
+    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const bf16 h = __float2bfloat16(x[i]);
     out[i] = h;
