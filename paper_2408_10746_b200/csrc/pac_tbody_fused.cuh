@@ -238,8 +238,8 @@ __device__ __forceinline__ void tb_tiles(TbStream& st, int from, int to, uint32_
                 for (int i = 0; i < N; ++i) {
                     TbB b;
                     tb_split_b(b, w[k * N + i].x, w[k * N + i].y, w[k * N + i].z, w[k * N + i].w);
-                    tb_mma(acc[i][0], a.m, b.m); tb_mma(acc[i][1], a.h, b.m); tb_mma(acc[i][2], a.h, b.h);
-                    tb_mma(acc[i][0], a.h, b.l); tb_mma(acc[i][1], a.m, b.h); tb_mma(acc[i][0], a.l, b.h);
+                    tb_mma(acc[i][0], a.m, b.m); tb_mma(acc[i][1 + (k & 1)], a.h, b.h); tb_mma(acc[i][0], a.h, b.l);
+                    tb_mma(acc[i][0], a.l, b.h); tb_mma(acc[i][0], a.h, b.m); tb_mma(acc[i][0], a.m, b.h);
                 }
             }
         }
@@ -247,7 +247,7 @@ __device__ __forceinline__ void tb_tiles(TbStream& st, int from, int to, uint32_
 #pragma unroll
     for (int i = 0; i < N; ++i)
 #pragma unroll
-        for (int e = 0; e < 4; ++e) v[i][e] = acc[i][2][e] + (acc[i][1][e] + acc[i][0][e]);
+        for (int e = 0; e < 4; ++e) v[i][e] = (acc[i][2][e] + acc[i][1][e]) + acc[i][0][e];
 }
 
 // Partial results of warps 8 - 15 to warps 0 - 7, lane by lane (every thread of the CTA takes part).
