@@ -395,7 +395,7 @@ def main():
     ap.add_argument("--impl", default="ours", choices=["ours", "reference"])
     ap.add_argument("--cpu-budget", type=float, default=12.0, help="seconds of oracle time for cpu_baseline")
     ap.add_argument("--no-cpu-baseline", action="store_true")
-    ap.add_argument("--force-simt", action="store_true", help="use the plain fp32-FMA kernels")
+    ap.add_argument("--force-simt", action="store_true", help="use the plain path (fp32 precision)")
     ap.add_argument("--forward", choices=["auto", "split", "one-kernel"], default="auto",
                     help="tensor-core path: down-projections and head phase as one kernel or two (default: library's choice)")
     ap.add_argument("--parallelism", default="replicas", choices=["replicas", "dp"],

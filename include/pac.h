@@ -65,7 +65,8 @@ typedef enum { PAC_HEAD_MEANPOOL_CLS = 0, PAC_HEAD_FROZEN_LM = 1 } pac_head;
  *     x' = x + concat_h(softmax(q_h k_h^T / sqrt(r/H)) v_h) Wo;  n2 = LayerNorm(x')
  *     a_l = x' + relu(n2 W1 + c1) W2 + c2
  * (pre-norm, bidirectional attention over the S tokens of a sample, LayerNorm eps 1e-5 with gain and
- * bias, no dropout).  Classifier head only; it runs on the plain fp32 kernels. */
+ * bias, no dropout).  Classifier head only; fp32 precision throughout, also on bf16
+ * caches. */
 typedef enum { PAC_BODY_POINTWISE = 0, PAC_BODY_TRANSFORMER = 1 } pac_body;
 
 typedef struct {
@@ -92,7 +93,7 @@ typedef enum {
                                      tiles to fill the device (2 * B * ceil(S/128) >= SMs, r a multiple of 32 up
                                      to 128) the merge / activation chain runs in the epilogue of the
                                      down-projection kernel instead; otherwise two plain launches,
-                                 1 = force the plain fp32-FMA kernels,
+                                 1 = force the plain path (fp32 precision; pac_kernel_path() says "simt"),
                                  2 = tensor-core path, forward half always as two plain launches,
                                  3 = tensor-core path, one-launch forward whenever the shape allows it,
                                  4 = tensor-core path, chain-in-epilogue forward whenever the shape allows it (with

@@ -214,7 +214,7 @@ struct pac_ctx {
     int dw_simt_max = 1;           // row slices sc.dw_spart has room for on the plain path
     bool lm_ce_stream = false;     // LM cross-entropy as a register-resident stream over the logits (V <= 32768, V % 4 == 0)
     HostCache hc;                  // out-of-core mode (pac_cache_register_host)
-    TBody tb;                      // transformer-body adapters (plain fp32 kernels)
+    TBody tb;                      // transformer-body adapters (fp32 precision throughout)
     // pac_train_step_async without copy nodes in the stream: a ring of id slots in page-locked host memory that
     // the forward kernel reads directly (two halves, an event per half orders the reuse)
     int* zc_ids = nullptr;         // [ZC_SLOTS][max_batch]
@@ -623,9 +623,8 @@ pac_status backward(pac_ctx* c, const int* d_ids, int B, float* d_loss, const pa
                 LAUNCH_CHECK(c);
             }
         }
-        // da_L = dy W_up^T: on the tensor cores when the bf16 copy of dy exists (da_L only feeds du, which is
-        // rounded to bf16 anyway).  dW_up above stays in fp32 FMA: with a_L and dy rounded to bf16 its error,
-        // amplified by Adam, took the parameters after ten steps past the 1e-2 bound (1.1e-2 measured).
+        // da_L = dy W_up^T: from the bf16 copy of dy where it exists.  dW_up above is formed at fp32 precision: with a_L and dy
+        // rounded to bf16 its error, amplified by Adam, took the parameters after ten steps past the 1e-2 bound (1.1e-2 measured).
         if (c->lm_tensor && c->lm_skinny_tensor) {
             pac_status gs = gemm_launch(c->g_daL, c->stream, M, sc.daL, dm.r, c->status, &c->launches);
             if (gs != PAC_OK) return fail(c, gs, "tensor-core da_L GEMM launch failed: %s", tensor_last_error());
@@ -690,7 +689,8 @@ pac_status backward(pac_ctx* c, const int* d_ids, int B, float* d_loss, const pa
 }
 
 // ---------------------------------------------------------------------------
-// Transformer-body adapters (plain fp32 kernels; see pac_tbody.cuh).  ids are on the device.
+// Transformer-body adapters: a launch per layer boundary (pac_tbody_fused.cuh) where the widths allow it, else a kernel per operation
+// (pac_tbody.cuh).  ids are on the device.
 // ---------------------------------------------------------------------------
 template <class AF, class BF, class EF>
 pac_status tb_gemm(pac_ctx* c, int M, int N, int K, int Z, const AF& A, const BF& Bm, const EF& E) {
@@ -1054,7 +1054,8 @@ pac_status chain_fwd_enqueue(pac_ctx* c, const int* d_ids, int B, bool train, fl
     return PAC_OK;
 }
 
-// Forward half of a classifier-head step (everything up to du and the per-sample head vectors).
+// Forward half of a classifier-head step: everything up to the per-sample head vectors and what the second pass builds du from (gates and da_L;
+// du itself on the plain path).
 pac_status cls_forward_enqueue(pac_ctx* c, const int* d_ids, int B, bool train, float* d_logits_out) {
     pac_status st;
     if (use_chain_fwd(c, B)) return chain_fwd_enqueue(c, d_ids, B, train, d_logits_out);
@@ -1645,8 +1646,9 @@ pac_status host_cache_stage(pac_ctx* c, const int* ids, int B, const char* who, 
     // its step must have finished before the slabs are overwritten
     CU_OK(c, cudaEventSynchronize(h.ready[k]));
     CU_OK(c, cudaStreamWaitEvent(h.copy_stream, h.freed[k], 0));
-    // Two samples in ascending order, wherever they lie, are the two rows of one pitched copy: a copy costs the engine about 5 us on top of
-    // its bytes (2.4 MB samples: 49.6 GB/s one by one, 52.7 in pairs, 55.4 in one piece; reads by a kernel reach 51).
+    // Two samples in ascending order are the two rows of one pitched copy if they lie within the largest pitch (2 GB: 910 samples of 2.4 MB, 170 of
+    // 12.6 MB): a copy costs the engine about 5 us on top of its bytes (2.4 MB samples: 49.6 GB/s one by one, 52.7 in pairs, 55.4 in one piece;
+    // reads by a kernel reach 51).  In a cache of many times that size most samples of a shuffled batch find no partner and travel one by one.
     h.paired.assign(B, 0);
     for (int b = 0; b < B; ++b) {
         if (!h.paired[b]) {

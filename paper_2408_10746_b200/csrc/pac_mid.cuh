@@ -595,9 +595,9 @@ __global__ void __launch_bounds__(512, STATE == STATE_SMEM ? 1 : 2) mid_cls_kern
 }
 
 // ---------------------------------------------------------------------------
-// Gradient finalisation for the classifier head, one thread per flat parameter index:
-//   W_down : sum of the row-split partials of h^T du (split order), or already final
-//   lambda : sum of per-block partials (block order)
+// Gradient finalisation for the classifier head:
+//   W_down : sum of the second pass's row splits (split order), on the tensor-core path times the layer's factor; or already final
+//   lambda : from <D_l, W_down^l> (lambda_grad), on the plain path the sum of per-block partials (block order); or already final
 //   W_up   : pooled_a^T g        W_head : pooled_y^T dlogits        b_head : sum_b dlogits
 // plus the mean loss.  With adam != 0 the AdamW update of the same element follows at once.
 // ---------------------------------------------------------------------------

@@ -1,6 +1,5 @@
-// Plain fp32-FMA kernels: every step of the path for any shape and both cache
-// dtypes.  They serve the fp32 configuration (whose 1e-4 tolerance rules out
-// reduced-precision tensor-core operands) and shapes the tensor-core path does not
+// The plain path's kernels besides its products over the cache (pac_xgemm.cuh): every step for any shape and both cache
+// dtypes.  They serve fp32 caches and shapes the tensor-core path does not
 // take; the small per-sample head/chain kernels here are shared by both paths.
 //
 // Notation follows Section IV-A of the paper: h_l cached state of layer l,

@@ -3,7 +3,8 @@
 //   rows   out[z][m][j] = sum_k A(z; m, k) B[z][k][j]        (u_l = h_l W_down^l)
 //   tn     out[i][j]    = sum_m A(z; m, i) B[z][m][j]        (dW = A^T B over all token rows)
 //
-// An fp32 operand enters as the exact sum of three bf16 terms (8 + 8 + 8 mantissa bits), a bf16 one as it is.  Of the products of terms those
+// An fp32 operand enters as the exact sum of three bf16 terms (8 + 8 + 8 mantissa bits; exact for magnitudes from about 2^-110, where the third
+// term starts to underflow, to the largest bf16, and see xg_redo for what lies beyond), a bf16 one as it is.  Of the products of terms those
 // of relative size 2^-16 and above are formed, six or three; the dropped ones, below 2^-25, are smaller than the rounding of one fp32
 // multiplication.  Sums are fp32, in several accumulators (xg_accs).  That is 1365 products per clock and SM against 128 on the FP32 pipe, so the kernel is bound
 // by bringing the operands in: A comes straight from the activation cache (the gather is the address; any row length and alignment),

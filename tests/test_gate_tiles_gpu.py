@@ -1,7 +1,8 @@
 """The second pass on the tensor path builds du from gate bytes and da_L, and lambda's gradient comes from <D, W_down>: at the edges of
 its tiles, term counts, row splits and of both finalisations, against the oracle.
 
-Tolerance 2e-2 per gradient block as for the other bf16 tests: da enters in one or two bf16 terms, 2^-9 per element at worst."""
+Tolerance 2e-2 per gradient block as for the other bf16 tests; what two bf16 terms of da give without flipped gates is bounded in
+test_gradient_precision_gpu.py."""
 import numpy as np
 import pytest
 
@@ -20,7 +21,7 @@ def spec(name, **kw):
 SPECS = [
     spec("one_token", S=1, r=16, d=64, B=3),
     spec("r_64_two_terms", r=64, S=65, d=264),              # widest adapter of the two-term tiles, two chunks of d and a remainder
-    spec("r_80_one_term", r=80, S=129, d=136),
+    spec("r_80", r=80, S=129, d=136),
     spec("r_128", r=128, S=63, d=256),
     spec("r_144_wide", r=144, S=64, d=128),                 # four column blocks, the third partly filled, the fourth empty
     spec("r_256", r=256, S=33, d=128, L=2),

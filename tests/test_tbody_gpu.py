@@ -1,6 +1,6 @@
 """Transformer-body adapters (paper Section IV-A: the side network as a lightweight version of the
-backbone transformer; Section VI-A: all widths 1/rho of the backbone's) on the plain fp32 CUDA
-kernels against the oracle: loss, every gradient block, evaluation, and a 10-step AdamW trajectory."""
+backbone transformer; Section VI-A: all widths 1/rho of the backbone's) at fp32
+precision against the oracle: loss, every gradient block, evaluation, and a 10-step AdamW trajectory."""
 import numpy as np
 import pytest
 import torch
