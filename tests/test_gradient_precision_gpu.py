@@ -82,3 +82,22 @@ def test_transformer_body_rounds_like_fp32(dtype):
         for name, sl in block_slices(sp).items():
             assert rel_l2(g[sl], ref[sl]) < (4e-6 if name == "lam" else 1.5e-6), (name, seed, rel_l2(g[sl], ref[sl]))
     ctx.close()
+
+
+def test_wide_transformer_body_forward_rounds_like_fp32():
+    """r = 128 on a bf16 cache: W_up's gradient is a_L^T dy, with nothing of the reverse pass in it (a gate that flips there moves other
+    blocks by single elements)."""
+    sp, heads, f = bf16("tb_wide", L=3, S=128, d=1024, r=128, B=4, N=6), 8, 256
+    ctx = make_ctx(sp, heads, f)
+    ids = [5, 0, 3, 1]
+    H = pi.cache_samples(sp, 0, ids, "cpu").double().numpy()
+    lab = pi.labels(sp, 0, "cpu").numpy().astype(np.int64)[ids]
+    flat = random_flat(sp, f, 3)
+    ctx.set_params(flat)
+    ctx.train_step(ids)
+    g = ctx.get_grads()
+    P, T = tb.unflatten(flat.astype(np.float64), sp.L, sp.d, sp.r, sp.n_out, f)
+    ref = tb.flatten(*tb.loss_and_grads_cls(P, T, H, lab, heads)[1])
+    sl = block_slices(sp)["W_up"]
+    assert rel_l2(g[sl], ref[sl]) < 1e-6, rel_l2(g[sl], ref[sl])
+    ctx.close()
