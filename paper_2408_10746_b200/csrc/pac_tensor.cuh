@@ -522,7 +522,8 @@ struct BwdParams {
 // L * M * r * 2 bytes of du out of memory in both directions; the tile costs five integer instructions per four elements.
 // Gate bytes: a builder that loads them itself runs at two stages per memory latency (1.1 us a stage).  At two and more groups per thread, whose
 // registers allow no deeper look-ahead, they therefore come through the stage ring with the h tile (S = 256, B = 64, L = 24, d = 1024, r = 128:
-// 187 -> 154 us, the rate of the memory).  With one group the ring was slower by 0.7 us: short loops, and one more hop before the first product.
+// 187 -> 154 us, the rate of the memory, with da in one term; 196 with two, where the products and not the loads pace a stage: a deeper ring for h with
+// the du tiles apart, or da held in registers over a sample, changed nothing).  With one group the ring was slower by 0.7 us: short loops, and one more hop before the first product.
 // GQ: 16-column groups of a du tile per thread (r = 64 GQ at most).  Registers are
 // bounded so that three finalisation blocks fit beside a CTA (r <= 64; with 155 instead of 88 the step took 58 us for 53).
 // ---------------------------------------------------------------------------
