@@ -127,7 +127,7 @@ pac_status pac_cache_register(pac_ctx* ctx, const void* dev_cache, int dtype, lo
  * then waits for the host.  pac_adapter_init allocates two device staging slots of max_batch
  * samples each (2 * max_batch * L*S*d elements).  Every call that takes host sample ids
  * (pac_train_step, pac_train_step_async, pac_train_epoch, pac_eval_logits, pac_gather) first copies
- * the slabs and labels of its ids into a slot, one contiguous copy per sample on a copy stream of
+ * the slabs and labels of its ids into a slot, in copies of one sample or (page-locked memory) two on a copy stream of
  * the context's own, and runs the same kernels on the slot; the copies of a step overlap the
  * kernels of the step before it, and the host runs at most two steps ahead of the copies.  Results
  * are bit-identical to those on a device-resident cache.  pac_train_epoch_dev (ids on the device)
