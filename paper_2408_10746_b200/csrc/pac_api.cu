@@ -90,7 +90,7 @@ struct TBody {
     TbPlan plan{};
     TbPack pk{};
     TbStacks st{};
-    float *packed = nullptr, *wg_part = nullptr;     // weights laid out for the ring [L][..]; row slices of the weight products
+    float *packed = nullptr, *wg_part = nullptr;     // weights split and laid out in stream order [L][..]; row slices of the weight products
     int wg_slices = 1;
 };
 
@@ -712,22 +712,28 @@ TbLayerParams tb_params(pac_ctx* c, int B, bool train) {
     return p;
 }
 
+// The packed weights of layer l, as one launch reads them: stream s and where the warps' shares of it begin.
+void tb_weights(const TBody& t, int l, int s, const unsigned char** w, int (&off)[TBF_WARPS + 1]) {
+    *w = reinterpret_cast<const unsigned char*>(t.packed) + l * t.pk.layer_bytes() + (size_t)t.pk.base[s] * TB_UNIT;
+    std::memcpy(off, t.pk.off[s], sizeof(off));
+}
+
 pac_status tb_fused_forward(pac_ctx* c, int B, bool train) {
     TBody& t = c->tb;
-    const TbPack& pk = t.pk;
     const BodyLayout& bl = t.bl;
     const int L = c->dm.L;
     for (int i = 0; i <= L; ++i) {
         TbLayerParams p = tb_params(c, B, train);
         p.tail = i - 1; p.head = i < L ? i : -1;
+        for (int m = 0; m < 4; ++m) p.mats[m] = t.pk.mat(m);
         if (p.tail >= 0) {
-            const float *w = t.packed + p.tail * pk.per_layer, *v = c->params + c->lay.body + p.tail * bl.per_layer;
-            for (int m = 0; m < 3; ++m) p.mats[m] = pk.mat(w, m);
+            const float* v = c->params + c->lay.body + p.tail * bl.per_layer;
+            tb_weights(t, p.tail, 0, &p.w0, p.off0);
             p.g2 = v + bl.g2; p.b2 = v + bl.b2; p.c1 = v + bl.c1; p.c2 = v + bl.c2;
         }
         if (p.head >= 0) {
             const float* v = c->params + c->lay.body + p.head * bl.per_layer;
-            p.mats[3] = pk.mat(t.packed + p.head * pk.per_layer, 3);
+            tb_weights(t, p.head, 1, &p.w1, p.off1);
             p.g1 = v + bl.g1; p.b1 = v + bl.b1;
         }
         cudaError_t e = tb_layer_launch(t.plan, p, false, c->stream);
@@ -739,20 +745,19 @@ pac_status tb_fused_forward(pac_ctx* c, int B, bool train) {
 
 pac_status tb_fused_backward(pac_ctx* c, int B) {
     TBody& t = c->tb;
-    const TbPack& pk = t.pk;
     const BodyLayout& bl = t.bl;
     const TbStacks& s = t.st;
     const int L = c->dm.L, r = c->dm.r, f = t.f, M = B * c->dm.S;
     for (int l = L - 1; l >= -1; --l) {
         TbLayerParams p = tb_params(c, B, true);
         p.tail = l + 1 < L ? l + 1 : -1; p.head = l;
+        for (int m = 0; m < 4; ++m) p.mats[m] = t.pk.mat(4 + m);
         if (p.tail >= 0) {
-            p.mats[0] = pk.mat(t.packed + p.tail * pk.per_layer, 4);
+            tb_weights(t, p.tail, 2, &p.w0, p.off0);
             p.g1 = c->params + c->lay.body + p.tail * bl.per_layer + bl.g1;
         }
         if (p.head >= 0) {
-            const float* w = t.packed + p.head * pk.per_layer;
-            for (int m = 1; m < 4; ++m) p.mats[m] = pk.mat(w, 4 + m);
+            tb_weights(t, p.head, 3, &p.w1, p.off1);
             p.g2 = c->params + c->lay.body + p.head * bl.per_layer + bl.g2;
         }
         cudaError_t e = tb_layer_launch(t.plan, p, true, c->stream);
@@ -787,7 +792,7 @@ pac_status tb_forward(pac_ctx* c, const int* d_ids, int B, bool train, float* d_
     const long long n = (long long)M * r, stride = (long long)c->max_rows * r;
     cudaStream_t st = c->stream;
     if (t.plan.ok) {
-        tb_pack_kernel<<<dim3(cdiv(t.pk.per_layer, 1024), (unsigned)dm.L), 256, 0, st>>>(c->params + c->lay.body, bl.per_layer, bl, t.pk, t.packed);
+        tb_pack_kernel<<<dim3(cdiv(t.pk.tiles(), 8), (unsigned)dm.L), 256, 0, st>>>(c->params + c->lay.body, bl.per_layer, bl, t.pk, reinterpret_cast<unsigned char*>(t.packed));
         LAUNCH_CHECK(c);
     }
     if (plain_head_ok(c, B)) TB_OK(head_matrix_enqueue(c));
@@ -1576,7 +1581,7 @@ pac_status pac_adapter_init(pac_ctx* c, const pac_adapter_cfg* cfg, unsigned lon
             const long long parts[] = {
                 k.sMr * dm.L, k.sMr * dm.L, k.sMr * dm.L, 3 * k.sMr * dm.L, k.sMr * dm.L, k.sMr * dm.L, k.sMr * dm.L,
                 k.sMf * dm.L, k.sP * dm.L, k.sM * dm.L, k.sM * dm.L, k.sMr * dm.L, k.sMr * dm.L, 3 * k.sMr * dm.L, k.sMf * dm.L,
-                k.sMr, k.sMr, k.sP, k.sP, ctas * k.part_w * dm.L, t.pk.per_layer * dm.L, per * dm.L * t.wg_slices};
+                k.sMr, k.sMr, k.sP, k.sP, ctas * k.part_w * dm.L, (long long)(t.pk.layer_bytes() / sizeof(float)) * dm.L, per * dm.L * t.wg_slices};
             float** const where[] = {&k.x, &k.xhat1, &k.n1, &k.qkv, &k.o, &k.xhat2, &k.n2, &k.hid, &k.P, &k.rstd1, &k.rstd2, &k.da,
                                      &k.dx1, &k.dqkv, &k.dpre, &k.dob[0], &k.dob[1], &k.dS[0], &k.dS[1], &k.part, &t.packed, &t.wg_part};
             long long total = 0;

@@ -11,11 +11,14 @@
 // rows of a tcgen05 tile, and a CTA's products are short and serial.  Every fp32 operand is the exact sum of three bf16 terms
 // (8 + 8 + 8 mantissa bits); of the nine products the six of relative size 2^-16 and above are formed, so the
 // dropped ones (below 2^-25) are smaller than the rounding of one fp32 multiplication, and sums are fp32.
-// Per SM that is 170 products per clock against 128 on the FP32 pipe, with a tenth of the instructions:
-// the same kernels on FMA tiles (8 tokens x 4 columns per thread, weights through a shared-memory ring) took 60 us
-// per forward launch instead of 30 at B = 16, S = 128, r = 64, waiting for instructions and shared memory, not for the pipe.
-// Weights arrive from L2 in the order of the tile fragments (tb_pack_kernel: a warp reads 512 contiguous bytes per
-// 16 x 8 tile) and are split in registers; activations are split once by whoever produces them.
+//
+// A launch is one chain of about ten dependent phases on 16 warps, so latency bounds it, not a rate: everything that is final before the
+// phase that needs it is requested ahead (weights through a ring of asynchronous copies that runs across phases, q, k, v and the residual rows
+// before the attention, gate bits before the product ahead of them), scores, softmax and its reverse stay in the registers of
+// the tensor instructions' fragments, a token's residual row stays in the registers of the warp that owns it, and halves of sums along K meet in
+// the row phase that reads them instead of in a phase of their own.  Weights arrive split and in the order in which a warp consumes them
+// (tb_pack_kernel).  Against scores, weights and rows in shared memory and weights split by their readers the step at B = 16, S = 128, r = 64, 12 layers went
+// from 953 to 769 us.  Loads of the second attention's operands ahead of the product before them cost 64 us in spilled registers.
 #pragma once
 #include "pac_tbody.cuh"
 #include "pac_tensor.cuh"
@@ -24,57 +27,109 @@ namespace pac {
 
 constexpr int TBF_THREADS = 512, TBF_WARPS = TBF_THREADS / 32, TBF_T = 16, TBF_MAX_R = 192;
 
-// One packed weight matrix: K x N in 16 x 8 tiles, tile (ks, j) at (ks * nt + j) * 128 floats, zero-padded; lane l of a
-// tile holds rows 2 (l % 4) + {0, 1, 8, 9} of column l / 4.
-struct TbMat { const float* w; int ks, nt; };
 __host__ __device__ inline int tb_up16(int x) { return (x + 15) & ~15; }
 __host__ __device__ inline int tb_up8(int x) { return (x + 7) & ~7; }
 
-// Offsets (floats) of the packed weights of one layer.
-struct TbPack {
-    int r, f;
-    long long off[8], per_layer;       // Wo, W1, W2, Wqkv | Wqkv^T, W2^T, W1^T, Wo^T
-    __host__ __device__ int rows(int m) const { return m == 2 || m == 6 ? f : m == 4 ? 3 * r : r; }                  // K
-    __host__ __device__ int cols(int m) const { return m == 1 || m == 5 ? tb_up8(f) : m == 3 ? 3 * tb_up8(r) : tb_up8(r); }
-    __host__ __device__ static TbPack make(int r, int f) {
-        TbPack p;
-        p.r = r; p.f = f;
-        long long o = 0;
-        for (int m = 0; m < 8; ++m) { p.off[m] = o; o += (long long)tb_up16(p.rows(m)) * p.cols(m); }
-        p.per_layer = o;
-        return p;
+// One weight matrix: K x N in 16 x 8 tiles, ks along K, nt along N.  A product whose output is r wide and has up to eight tiles along N is cut in half along K
+// between warps 0 - 7 and 8 - 15, every other one has its tiles dealt to the warps in turn.  A warp takes its tiles in pairs 16 apart, k step by k step, or
+// one tile two k steps at a time: two tiles either way, one unit of its stream.
+struct TbMat {
+    int ks, nt;
+    bool cut;
+    __host__ __device__ int from(int warp) const { return cut && warp >= TBF_WARPS / 2 ? (ks + 1) / 2 : 0; }
+    __host__ __device__ int to(int warp) const { return cut && warp < TBF_WARPS / 2 ? (ks + 1) / 2 : ks; }
+    __host__ __device__ int first(int warp) const { return cut ? warp & (TBF_WARPS / 2 - 1) : warp; }
+    __host__ __device__ int tiles(int warp) const {            // of this warp
+        const int j = first(warp);
+        return j >= nt ? 0 : cut ? 1 : (nt - j + TBF_WARPS - 1) / TBF_WARPS;
     }
-    TbMat mat(const float* base, int m) const { return TbMat{base + off[m], tb_up16(rows(m)) / 16, cols(m) / 8}; }
+    __host__ __device__ int units(int warp) const {
+        const int n = tiles(warp);
+        return (n >> 1) * ks + (n & 1) * ((to(warp) - from(warp) + 1) >> 1);
+    }
 };
 
-// Lays the weights of every layer out in tile order: grid (blocks, L).
-__global__ void __launch_bounds__(256) tb_pack_kernel(const float* __restrict__ body, long long body_per, BodyLayout bl,
-                                                      const __grid_constant__ TbPack p, float* __restrict__ packed) {
-    const float* w = body + blockIdx.y * body_per;
-    float* dst = packed + blockIdx.y * p.per_layer;
-    const int r = p.r, f = p.f, r8 = tb_up8(r);
-    for (int e = (blockIdx.x * blockDim.x + threadIdx.x) * 4; e < (int)p.per_layer; e += gridDim.x * blockDim.x * 4) {
-        int m = 0;
-        while (m < 7 && e >= p.off[m + 1]) ++m;
-        const int q = e - (int)p.off[m], lane = (q >> 2) & 31, tile = q >> 7, nt = p.cols(m) >> 3;
-        const int k0 = (tile / nt) * 16 + 2 * (lane & 3), n = (tile % nt) * 8 + (lane >> 2), K = p.rows(m);
-        float v[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int k = k0 + (i & 1) + (i >> 1) * 8;
-            v[i] = 0.f;
-            if (k >= K) continue;
-            if (m == 0) { if (n < r) v[i] = w[bl.wo + k * r + n]; }
-            else if (m == 1) { if (n < f) v[i] = w[bl.w1 + k * f + n]; }
-            else if (m == 2) { if (n < r) v[i] = w[bl.w2 + k * r + n]; }
-            else if (m == 3) { const int s = n / r8, c = n - s * r8; if (c < r) v[i] = w[bl.wq + (s * r + k) * r + c]; }
-            else if (m == 4) { const int s = k / r, j = k - s * r; if (n < r) v[i] = w[bl.wq + (s * r + n) * r + j]; }
-            else if (m == 5) { if (n < f) v[i] = w[bl.w2 + n * r + k]; }
-            else if (m == 6) { if (n < r) v[i] = w[bl.w1 + n * f + k]; }
-            else if (n < r) v[i] = w[bl.wo + n * r + k];
-        }
-        *reinterpret_cast<float4*>(dst + e) = make_float4(v[0], v[1], v[2], v[3]);
+// A unit: two tiles in three bf16 terms.  512 bytes each of first and second terms (lane l of a tile holds, of column l / 4, rows 2 (l % 4) + {0, 1} and
+// {8, 9}: two words per term), then 256 bytes each of third terms.
+constexpr int TB_UNIT = 1536;
+
+// The packed weights of one layer: four streams (Wo W1 W2 | Wqkv | Wqkv^T | W2^T W1^T Wo^T: what one launch reads of a layer), a warp's units consecutive in each.
+struct TbPack {
+    int r, f;
+    int off[4][TBF_WARPS + 1];         // first unit of a warp in a stream; total
+    int base[5];                       // first unit of a stream; per layer
+    static __host__ __device__ int stream(int m) { return m < 3 ? 0 : m - 2 < 3 ? m - 2 : 3; }
+    __host__ __device__ TbMat mat(int m) const {
+        const int K = m == 2 || m == 6 ? f : m == 4 ? 3 * r : r, n8 = m == 1 || m == 5 ? tb_up8(f) : m == 3 ? 3 * tb_up8(r) : tb_up8(r);
+        return TbMat{tb_up16(K) / 16, n8 / 8, m != 1 && m != 3 && m != 5 && n8 / 8 <= TBF_WARPS / 2};
     }
+    static TbPack make(int r, int f) {
+        TbPack p;
+        p.r = r; p.f = f;
+        int at = 0;
+        for (int s = 0; s < 4; ++s) {
+            int o = 0;
+            for (int w = 0; w < TBF_WARPS; ++w) {
+                p.off[s][w] = o;
+                for (int m = 0; m < 8; ++m) if (stream(m) == s) o += p.mat(m).units(w);
+            }
+            p.off[s][TBF_WARPS] = o;
+            p.base[s] = at;
+            at += o;
+        }
+        p.base[4] = at;
+        return p;
+    }
+    size_t layer_bytes() const { return (size_t)base[4] * TB_UNIT; }
+    int tiles() const { int t = 0; for (int m = 0; m < 8; ++m) t += mat(m).ks * mat(m).nt; return t; }
+};
+
+__device__ __forceinline__ void tb_split_b(uint32_t (&h)[2], uint32_t (&m)[2], uint32_t (&l)[2], float k0, float k1, float k8, float k9) {
+    split3_pair(k0, k1, h[0], m[0], l[0]);
+    split3_pair(k8, k9, h[1], m[1], l[1]);
+}
+
+// Splits the weights of every layer and lays them out in stream order, a tile per warp: grid (tiles / 8, L).
+__global__ void __launch_bounds__(256) tb_pack_kernel(const float* __restrict__ body, long long body_per, BodyLayout bl,
+                                                      const __grid_constant__ TbPack p, unsigned char* __restrict__ packed) {
+    const float* w = body + blockIdx.y * body_per;
+    const int r = p.r, f = p.f, r8 = tb_up8(r), lane = threadIdx.x & 31;
+    int tile = blockIdx.x * 8 + (threadIdx.x >> 5), m = 0;
+    TbMat mt = p.mat(0);
+    while (tile >= mt.ks * mt.nt) {
+        tile -= mt.ks * mt.nt;
+        if (++m == 8) return;
+        mt = p.mat(m);
+    }
+    const int ks = tile / mt.nt, j = tile - ks * mt.nt, K = m == 2 || m == 6 ? f : m == 4 ? 3 * r : r;
+    const int k0 = ks * 16 + 2 * (lane & 3), n = j * 8 + (lane >> 2);
+    float v[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int k = k0 + (i & 1) + (i >> 1) * 8;
+        v[i] = 0.f;
+        if (k >= K) continue;
+        if (m == 0) { if (n < r) v[i] = w[bl.wo + k * r + n]; }
+        else if (m == 1) { if (n < f) v[i] = w[bl.w1 + k * f + n]; }
+        else if (m == 2) { if (n < r) v[i] = w[bl.w2 + k * r + n]; }
+        else if (m == 3) { const int s = n / r8, c = n - s * r8; if (c < r) v[i] = w[bl.wq + (s * r + k) * r + c]; }
+        else if (m == 4) { const int s = k / r, c = k - s * r; if (n < r) v[i] = w[bl.wq + (s * r + n) * r + c]; }
+        else if (m == 5) { if (n < f) v[i] = w[bl.w2 + n * r + k]; }
+        else if (m == 6) { if (n < r) v[i] = w[bl.w1 + n * f + k]; }
+        else if (n < r) v[i] = w[bl.wo + n * r + k];
+    }
+    const int half = mt.cut && ks >= (mt.ks + 1) / 2 ? TBF_WARPS / 2 : 0, warp = mt.cut ? j + half : j & (TBF_WARPS - 1), step = ks - mt.from(warp);
+    const int i = mt.cut ? 0 : j / TBF_WARPS, pairs = i >> 1;
+    const bool pair = (i | 1) < mt.tiles(warp);
+    const int s = TbPack::stream(m);
+    int unit = p.base[s] + p.off[s][warp] + pairs * mt.ks + (pair ? step : step >> 1);
+    for (int q = 0; q < m; ++q) if (TbPack::stream(q) == s) unit += p.mat(q).units(warp);
+    const int sub = pair ? i & 1 : step & 1;
+    uint32_t h[2], mm[2], l[2];
+    tb_split_b(h, mm, l, v[0], v[1], v[2], v[3]);
+    unsigned char* dst = packed + (blockIdx.y * (long long)p.base[4] + unit) * TB_UNIT;
+    *reinterpret_cast<uint4*>(dst + sub * 512 + lane * 16) = make_uint4(h[0], h[1], mm[0], mm[1]);
+    *reinterpret_cast<uint2*>(dst + 1024 + sub * 256 + lane * 8) = make_uint2(l[0], l[1]);
 }
 
 // Saved activations and reverse-pass stacks, all fp32, layer l at l * stride.
@@ -89,12 +144,15 @@ struct TbStacks {
 
 struct TbLayerParams {
     TbMat mats[4];                     // of phases 0 .. 3 (see the kernels)
+    const unsigned char *w0, *w1;      // packed streams: of `tail`'s phases, then of `head`'s
+    int off0[TBF_WARPS + 1], off1[TBF_WARPS + 1];
     int tail, head;                    // forward: layer whose attention + feed-forward half runs / layer whose q, k, v are formed (-1: none);
                                        // backward: layer whose dk, dv + merge run / layer whose feed-forward + dq run
-    int B, S, r, f, H, hg;             // hg: heads whose score rows are in shared memory at a time
+    int B, S, r, f, H;
+    int nc, hg;                        // warps per head (32 keys each and round), heads at a time
     int tiles;                         // CTAs per sample
     int train;
-    int ka, kb, rs, ss;                // row strides in shared memory: wide and narrow operand terms (bf16), fp32 rows, score rows
+    int ka, kb, rs;                    // row strides in shared memory: wide and narrow operand terms (bf16), fp32 rows
     TbStacks s;
     const float* u; long long u_stride;
     float* du;                         // backward: [L][M][r], u_stride apart
@@ -113,26 +171,17 @@ __device__ __forceinline__ void tb_mma(float (&c)[4], const uint32_t (&a)[4], co
 }
 struct TbA { uint32_t h[4], m[4], l[4]; };     // 16 x 16 tile, three terms
 struct TbB { uint32_t h[2], m[2], l[2]; };     // 16 x 8 tile
-// c += A B, small products first.
-__device__ __forceinline__ void tb_mma6(float (&c)[4], const TbA& a, const TbB& b) {
-    tb_mma(c, a.m, b.m); tb_mma(c, a.h, b.l); tb_mma(c, a.l, b.h);
-    tb_mma(c, a.h, b.m); tb_mma(c, a.m, b.h); tb_mma(c, a.h, b.h);
+__device__ __forceinline__ void tb_split_a(TbA& a, const float (&v)[8]) {      // pairs (row q, q + 8) x (columns c2, c2 + 8)
+#pragma unroll
+    for (int i = 0; i < 4; ++i) split3_pair(v[2 * i], v[2 * i + 1], a.h[i], a.m[i], a.l[i]);
 }
-__device__ __forceinline__ void tb_split_b(TbB& b, float k0, float k1, float k8, float k9) {
-    split3_pair(k0, k1, b.h[0], b.m[0], b.l[0]);
-    split3_pair(k8, k9, b.h[1], b.m[1], b.l[1]);
-}
-// A tile from fp32 rows in shared memory: p points at (row lane / 4, column 2 (lane % 4)) of the tile.
-__device__ __forceinline__ void tb_split_a(TbA& a, const float* p, int stride) {
-    const float2 v0 = *reinterpret_cast<const float2*>(p), v1 = *reinterpret_cast<const float2*>(p + 8 * stride);
-    const float2 v2 = *reinterpret_cast<const float2*>(p + 8), v3 = *reinterpret_cast<const float2*>(p + 8 * stride + 8);
-    split3_pair(v0.x, v0.y, a.h[0], a.m[0], a.l[0]);
-    split3_pair(v1.x, v1.y, a.h[1], a.m[1], a.l[1]);
-    split3_pair(v2.x, v2.y, a.h[2], a.m[2], a.l[2]);
-    split3_pair(v3.x, v3.y, a.h[3], a.m[3], a.l[3]);
+// The products in two accumulators: first terms, and the smaller ones.
+__device__ __forceinline__ void tb_mma6(float (&big)[4], float (&small)[4], const TbA& a, const TbB& b) {
+    tb_mma(small, a.m, b.m); tb_mma(big, a.h, b.h); tb_mma(small, a.h, b.l);
+    tb_mma(small, a.l, b.h); tb_mma(small, a.h, b.m); tb_mma(small, a.m, b.h);
 }
 __device__ __forceinline__ void tb_ldmatrix4(uint32_t (&r)[4], uint32_t addr) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
 }
 // Operand terms in shared memory: [term][16 tokens][stride] bf16, stride = K rounded to 16, + 8 (eight rows of 16 bytes fall
 // into different banks).
@@ -152,134 +201,97 @@ __device__ __forceinline__ void tb_put1(bf16* pl, int stride, int t, int c, floa
 // ---------------------------------------------------------------------------
 // Building blocks (a CTA of sixteen warps and 16 tokens)
 // ---------------------------------------------------------------------------
-// A matrix of up to eight tiles along N is cut in half along K between warps 0 - 7 and 8 - 15 (every other product has a tile for
-// each warp): the k steps [from, to) of `half`.
-__device__ __forceinline__ bool tb_cut(int nt) { return nt <= TBF_WARPS / 2; }
-// A warp's own stream of weight tiles: phase after phase, pairs of tiles (columns 128 apart), k step by k step.
-// Every lane copies and later reads its own 16 bytes of a tile, so the stream needs no barrier: it runs TBF_AHEAD tiles
-// ahead of the products, across phases, and starts before the wait for the predecessor launch.
-constexpr int TBF_SLOTS = 16, TBF_AHEAD = 12, TBF_BATCH = 4;
+// A warp's own stream of weight units, U of them in flight: it runs ahead of the products, across phases, and starts before the wait for the
+// predecessor launch.  Copies are per lane and read by the whole warp, so the ring needs no barrier beyond the warp.
+template <int U>
 struct TbStream {
-    const TbMat* mats;
-    int ph, last;                      // phase being fetched, one past the last
-    int j0, n, i, ks, to, nt;          // first tile of the pair, its tiles, tile, k step and its end; the matrix' tiles along N
-    int from;
-    const float *base, *src;           // lane's address of the matrix' first tile / of the next tile
-    uint32_t ring;                     // lane's address of slot 0
-    int put = 0, get = 0;
-    __device__ TbStream(const TbMat* m, int first, int last_, unsigned char* mem) : mats(m), ph(first), last(last_) {
-        ring = smem_u32(mem) + (threadIdx.x >> 5) * (TBF_SLOTS * 512) + (threadIdx.x & 31) * 16;
-        open();
+    const unsigned char *src, *next_src;
+    int left, next_left;
+    uint32_t ring;                     // of the warp
+    uint32_t put = 0, get = 0;         // byte offsets in it
+    __device__ __forceinline__ TbStream(const TbLayerParams& p, unsigned char* mem) {
+        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+        ring = smem_u32(mem) + warp * (U * TB_UNIT);
+        src = p.w0 + (long long)p.off0[warp] * TB_UNIT + lane * 16;
+        left = p.tail >= 0 ? p.off0[warp + 1] - p.off0[warp] : 0;
+        next_src = p.w1 + (long long)p.off1[warp] * TB_UNIT + lane * 16;
+        next_left = p.head >= 0 ? p.off1[warp + 1] - p.off1[warp] : 0;
     }
-    __device__ void aim() { n = j0 + TBF_WARPS < nt ? 2 : 1; ks = from; src = base + (long long)(from * nt + j0) * 128; i = 0; }
-    __device__ void open() {           // first tile of phase `ph` (phases in which this warp has no tile are passed over)
-        const int warp = threadIdx.x >> 5;
-        for (; ph < last; ++ph) {
-            nt = mats[ph].nt;
-            const int n_ks = mats[ph].ks;
-            const bool cut = tb_cut(nt), half = cut && warp >= TBF_WARPS / 2;
-            from = half ? (n_ks + 1) / 2 : 0;
-            to = cut && !half ? (n_ks + 1) / 2 : n_ks;
-            base = mats[ph].w + (threadIdx.x & 31) * 4;
-            j0 = half ? warp - TBF_WARPS / 2 : warp;
-            if (j0 < nt && (!cut || j0 < TBF_WARPS / 2) && from < to) { aim(); return; }
+    __device__ __forceinline__ void issue() {
+        if (left == 0) { src = next_src; left = next_left; next_left = 0; }
+        if (left > 0) {
+            const uint32_t d = ring + put + (threadIdx.x & 31) * 16;
+#pragma unroll
+            for (int i = 0; i < 3; ++i) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d + i * 512), "l"(src + i * 512) : "memory");
+            src += TB_UNIT;
+            --left;
         }
-    }
-    __device__ void issue() {
-        if (ph < last) {
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(ring + put * 512), "l"(src) : "memory");
-            put = (put + 1) & (TBF_SLOTS - 1);
-            src += TBF_WARPS * 128;
-            if (++i == n) {
-                i = 0;
-                src += (nt - n * TBF_WARPS) * 128;
-                if (++ks == to) {
-                    j0 += 2 * TBF_WARPS;
-                    if (j0 < nt && !tb_cut(nt)) aim();
-                    else { ++ph; open(); }
-                }
-            }
-        }
+        put = put + TB_UNIT == U * TB_UNIT ? 0 : put + TB_UNIT;
         asm volatile("cp.async.commit_group;" ::: "memory");
     }
-    // The next `count` <= TBF_BATCH tiles, and as many sent for.
-    __device__ void next(float4 (&v)[TBF_BATCH], int count) {
-        asm volatile("cp.async.wait_group %0;" ::"n"(TBF_AHEAD - TBF_BATCH) : "memory");
+    // The next unit's tiles, and another unit sent for.
+    __device__ __forceinline__ void next(TbB (&b)[2]) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(U - 1) : "memory");
+        __syncwarp();
+        const uint32_t a = ring + get, lane = threadIdx.x & 31;
 #pragma unroll
-        for (int e = 0; e < TBF_BATCH; ++e)
-            if (e < count) {
-                asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v[e].x), "=f"(v[e].y), "=f"(v[e].z), "=f"(v[e].w)
-                             : "r"(ring + ((get + e) & (TBF_SLOTS - 1)) * 512) : "memory");
-            }
-        get += count;
-#pragma unroll 1
-        for (int e = 0; e < count; ++e) issue();
+        for (int i = 0; i < 2; ++i) {
+            asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(b[i].h[0]), "=r"(b[i].h[1]), "=r"(b[i].m[0]), "=r"(b[i].m[1]) : "r"(a + i * 512 + lane * 16) : "memory");
+            asm volatile("ld.shared.v2.b32 {%0, %1}, [%2];" : "=r"(b[i].l[0]), "=r"(b[i].l[1]) : "r"(a + 1024 + i * 256 + lane * 8) : "memory");
+        }
+        get = get + TB_UNIT == U * TB_UNIT ? 0 : get + TB_UNIT;
+        __syncwarp();
+        issue();
     }
 };
 
-// acc += the k steps [from, to) of N tiles: batches of TBF_BATCH tiles are in registers before the first is split.
-// Three accumulators per tile shorten the dependent chain of a k step to three.
-template <int N>
-__device__ __forceinline__ void tb_tiles(TbStream& st, int from, int to, uint32_t a0, uint32_t term, float (&v)[2][4]) {
-    constexpr int KU = TBF_BATCH / N;
-    float acc[N][3][4] = {};
+// out = act W for the 16 tokens: act's terms at pl, W the stream's next matrix.  ep(half, i, n, v): columns n, n + 1 of rows lane / 4 (v[0], v[1])
+// and lane / 4 + 8 (v[2], v[3]), the half's share of the sum where the matrix is cut; i counts the warp's tiles; called by whole warps.
+// First terms are added up in two accumulators per tile, the smaller products in a third.
+template <int U, class EP>
+__device__ __forceinline__ void tb_product(TbStream<U>& st, const TbMat& m, const bf16* pl, int stride, EP ep) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, half = m.cut ? warp >> 3 : 0;
+    const uint32_t a00 = smem_u32(pl) + (((lane & 15) * stride) + (lane >> 4) * 8) * 2, term = 32 * stride;
+    const int tiles = m.tiles(warp), from = m.from(warp), steps = m.to(warp) - from, j = m.first(warp);
 #pragma unroll 1
-    for (int ks = from; ks < to; ks += KU) {
-        const int steps = min(KU, to - ks);
-        float4 w[TBF_BATCH];
-        st.next(w, steps * N);
+    for (int i = 0; i < tiles; i += 2) {
+        const bool pair = i + 1 < tiles;
+        const int units = pair ? steps : (steps + 1) >> 1;
+        const uint32_t to_second = pair ? 0 : 32, step = pair ? 32 : 64;
+        uint32_t ad = a00 + from * 32;
+        float acc[2][3][4] = {};
+#pragma unroll 1
+        for (int u = 0; u < units; u += 2) {
 #pragma unroll
-        for (int k = 0; k < KU; ++k) {
-            if (k < steps) {
+            for (int e = 0; e < 2; ++e) {
+                if (u + e >= units) break;
+                TbB b[2];
                 TbA a;
-                const uint32_t ad = a0 + (ks + k) * 32;
                 tb_ldmatrix4(a.h, ad); tb_ldmatrix4(a.m, ad + term); tb_ldmatrix4(a.l, ad + 2 * term);
-#pragma unroll
-                for (int i = 0; i < N; ++i) {
-                    TbB b;
-                    tb_split_b(b, w[k * N + i].x, w[k * N + i].y, w[k * N + i].z, w[k * N + i].w);
-                    tb_mma(acc[i][0], a.m, b.m); tb_mma(acc[i][1 + (k & 1)], a.h, b.h); tb_mma(acc[i][0], a.h, b.l);
-                    tb_mma(acc[i][0], a.l, b.h); tb_mma(acc[i][0], a.h, b.m); tb_mma(acc[i][0], a.m, b.h);
+                st.next(b);
+                tb_mma6(acc[0][1 + e], acc[0][0], a, b[0]);
+                if (pair || 2 * (u + e) + 1 < steps) {
+                    if (!pair) { tb_ldmatrix4(a.h, ad + to_second); tb_ldmatrix4(a.m, ad + to_second + term); tb_ldmatrix4(a.l, ad + to_second + 2 * term); }
+                    tb_mma6(acc[1][1 + e], acc[1][0], a, b[1]);
                 }
+                ad += step;
             }
         }
-    }
+        float v[2][4];
 #pragma unroll
-    for (int i = 0; i < N; ++i)
+        for (int k = 0; k < 2; ++k)
 #pragma unroll
-        for (int e = 0; e < 4; ++e) v[i][e] = (acc[i][2][e] + acc[i][1][e]) + acc[i][0][e];
-}
-
-// Partial results of warps 8 - 15 to warps 0 - 7, lane by lane (every thread of the CTA takes part).
-__device__ __forceinline__ void tb_combine(float4* red, float (&v)[4]) {
-    const int t = threadIdx.x, h = TBF_THREADS / 2;
-    if (t >= h) red[t - h] = make_float4(v[0], v[1], v[2], v[3]);
-    __syncthreads();
-    if (t < h) { const float4 o = red[t]; v[0] += o.x; v[1] += o.y; v[2] += o.z; v[3] += o.w; }
-}
-
-// out = act W for the 16 tokens: act's terms at pl, W the stream's next matrix.  ep(n, v): columns n, n + 1 of rows lane / 4 (v[0], v[1])
-// and lane / 4 + 8 (v[2], v[3]); called by whole warps.
-template <class EP>
-__device__ __forceinline__ void tb_product(TbStream& st, const TbMat& m, const bf16* pl, int stride, float4* red, EP ep) {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint32_t a0 = smem_u32(pl) + (((lane & 15) * stride) + (lane >> 4) * 8) * 2, term = 32 * stride;
-    const int nt = m.nt, n_ks = m.ks;
-    const bool cut = tb_cut(nt), half = cut && warp >= TBF_WARPS / 2;
-    const int from = half ? (n_ks + 1) / 2 : 0, to = cut && !half ? (n_ks + 1) / 2 : n_ks;
-    int j0 = half ? warp - TBF_WARPS / 2 : warp;
-    do {
-        const bool mine = j0 < nt, two = !cut && j0 + TBF_WARPS < nt;
-        float v[2][4] = {};
-        if (two) tb_tiles<2>(st, from, to, a0, term, v);
-        else if (mine) tb_tiles<1>(st, from, to, a0, term, v);
-        if (cut) tb_combine(red, v[0]);
-        if (mine && !half) {
-            ep(j0 * 8 + 2 * (lane & 3), v[0]);
-            if (two) ep((j0 + TBF_WARPS) * 8 + 2 * (lane & 3), v[1]);
+            for (int e = 0; e < 4; ++e) v[k][e] = (acc[k][2][e] + acc[k][1][e]) + acc[k][0][e];
+        const int n = (j + i * TBF_WARPS) * 8 + 2 * (lane & 3);
+        if (pair) {
+            ep(half, i, n, v[0]);
+            ep(half, i + 1, n + TBF_WARPS * 8, v[1]);
+        } else {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) v[0][e] += v[1][e];
+            ep(half, i, n, v[0]);
         }
-        j0 += 2 * TBF_WARPS;
-    } while (!cut && j0 < nt);
+    }
 }
 
 // Two consecutive floats of a row (zeros past n); `even`: the row starts on an 8-byte boundary.
@@ -287,87 +299,84 @@ __device__ __forceinline__ float2 tb_ld2(const float* __restrict__ p, int c, int
     if (even && c + 1 < n) return __ldg(reinterpret_cast<const float2*>(p + c));
     return make_float2(c < n ? __ldg(p + c) : 0.f, c + 1 < n ? __ldg(p + c + 1) : 0.f);
 }
-
-// sc[(h * 16 + t) * ss + j] = sum_i act[t][(h0 + h) dh + i] X[j][(h0 + h) dh + i]: scores of the 16 tokens against all S tokens of
-// the sample.  act: fp32 rows in shared memory, X: [S][r] in global memory.  A warp takes 32 keys of one head.
-__device__ __forceinline__ void tb_scores(const float* __restrict__ X, int r, const float* act, int rs, int S, int dh, int h0, int hg, float* sc, int ss) {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, q = lane >> 2, c2 = 2 * (lane & 3);
-    const int chunks = (S + 31) >> 5;
-    const bool even = ((dh | r) & 1) == 0;
-    for (int w = warp; w < hg * chunks; w += TBF_WARPS) {
-        const int h = w / chunks, n0 = (w - h * chunks) * 32, col = (h0 + h) * dh;
-        float acc[4][4] = {};
-        for (int k = 0; k < dh; k += 16) {
-            // columns past the head's are zeros on the X side; what act holds there is finite
-            TbA a;
-            {
-                float v[8];
-#pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    const int c = k + c2 + (i & 1) + (i >> 2) * 8;
-                    v[i] = c < dh ? act[(q + ((i >> 1) & 1) * 8) * rs + col + c] : 0.f;
-                }
-#pragma unroll
-                for (int i = 0; i < 4; ++i) split3_pair(v[2 * i], v[2 * i + 1], a.h[i], a.m[i], a.l[i]);
-            }
-#pragma unroll
-            for (int n = 0; n < 4; ++n) {
-                if (n0 + n * 8 < S) {
-                    const float* x = X + (long long)min(n0 + n * 8 + q, S - 1) * r + col + k;
-                    const float2 v0 = tb_ld2(x, c2, dh - k, even), v1 = tb_ld2(x, c2 + 8, dh - k, even);
-                    TbB b;
-                    tb_split_b(b, v0.x, v0.y, v1.x, v1.y);
-                    tb_mma6(acc[n], a, b);
-                }
-            }
-        }
-        float* o = sc + (h * 16 + q) * ss + n0 + c2;
-#pragma unroll
-        for (int n = 0; n < 4; ++n)
-            if (n0 + n * 8 < S) {
-                *reinterpret_cast<float2*>(o + n * 8) = make_float2(acc[n][0], acc[n][1]);
-                *reinterpret_cast<float2*>(o + 8 * ss + n * 8) = make_float2(acc[n][2], acc[n][3]);
-            }
-    }
+__device__ __forceinline__ void tb_st2(float* p, float x, float y, bool two, bool even) {
+    if (even && two) *reinterpret_cast<float2*>(p) = make_float2(x, y);
+    else { p[0] = x; if (two) p[1] = y; }
 }
 
-// ep(c, two, v) with v = rows (lane / 4, + 8) x columns (c, c + 1) of  sum_j sc[h][t][j] X[j][c],  c from h0 * dh to (h0 + hg) * dh: mixes the
-// rows of all S tokens with the weights in shared memory (zero from S to the next multiple of 16).  c may be odd and c + 1 may lie
-// past the head: `two` says whether it counts.  A warp takes eight columns of one head; up to eight such tasks: half of the rows each.
-template <class EP>
-__device__ __forceinline__ void tb_mix(const float* __restrict__ X, int r, const float* sc, int ss, int S, int dh, int h0, int hg, float4* red, EP ep) {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, q = lane >> 2, c2 = 2 * (lane & 3);
-    const int tiles = (dh + 7) >> 3, tasks = hg * tiles;
-    const bool cut = tb_cut(tasks), half = cut && warp >= TBF_WARPS / 2;
-    const int mid = ((S + 31) >> 5) * 16, from = half ? mid : 0, to = cut && !half ? min(mid, S) : S;
-    int w = half ? warp - TBF_WARPS / 2 : warp;
-    do {
-        const bool mine = w < tasks;
-        const int h = w / tiles, n0 = (w - h * tiles) * 8;
-        float v[4] = {};
-        if (mine) {
-            const float* x = X + (h0 + h) * dh + min(n0 + q, dh - 1);
-            const float* a_row = sc + (h * 16 + q) * ss + c2;
-            float acc[2][4] = {};
-#pragma unroll 4
-            for (int k = from; k < to; k += 16) {
-                const int j = k + c2;
-                TbA a;
-                TbB b;
-                const float x0 = __ldg(x + (long long)min(j, S - 1) * r), x1 = __ldg(x + (long long)min(j + 1, S - 1) * r);
-                const float x8 = __ldg(x + (long long)min(j + 8, S - 1) * r), x9 = __ldg(x + (long long)min(j + 9, S - 1) * r);
-                tb_split_a(a, a_row + k, ss);
-                tb_split_b(b, x0, x1, x8, x9);
-                tb_mma(acc[0], a.m, b.m); tb_mma(acc[1], a.h, b.m); tb_mma(acc[0], a.h, b.l);
-                tb_mma(acc[1], a.m, b.h); tb_mma(acc[0], a.l, b.h); tb_mma(acc[1], a.h, b.h);
-            }
+// 32 rows (keys) x 16 columns of a head, as the B operand of scores: pair (c2, c2 + 1) and (c2 + 8, + 9) of row 8 n + lane / 4.  X: the head's first column
+// of the sample's rows; columns from `cols` on are zeros, rows from S on repeat the last one.
+struct TbKeys { float2 x[4][2]; };
+__device__ __forceinline__ void tb_load_keys(TbKeys& o, const float* __restrict__ X, int r, int key0, int S, int k, int cols, bool even) {
+    const int lane = threadIdx.x & 31, q = lane >> 2, c2 = 2 * (lane & 3);
 #pragma unroll
-            for (int e = 0; e < 4; ++e) v[e] = acc[1][e] + acc[0][e];
+    for (int n = 0; n < 4; ++n) {
+        const float* x = X + (long long)min(key0 + n * 8 + q, S - 1) * r;
+        o.x[n][0] = tb_ld2(x, k + c2, cols, even); o.x[n][1] = tb_ld2(x, k + c2 + 8, cols, even);
+    }
+}
+// acc[n] += act (16 tokens x 16 columns) keys^T: scores of 32 keys.
+__device__ __forceinline__ void tb_scores(float (&acc)[4][4], const TbA& a, const TbKeys& k) {
+#pragma unroll
+    for (int n = 0; n < 4; ++n) {
+        TbB b;
+        tb_split_b(b.h, b.m, b.l, k.x[n][0].x, k.x[n][0].y, k.x[n][1].x, k.x[n][1].y);
+        float small[4] = {};
+        tb_mma6(acc[n], small, a, b);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) acc[n][e] += small[e];
+    }
+}
+// 32 rows x 16 columns of a head, as the B operand of a mix over rows.
+struct TbVals { float v[2][2][4]; };
+__device__ __forceinline__ void tb_load_vals(TbVals& o, const float* __restrict__ X, int r, int key0, int S, int n0, int dh) {
+    const int lane = threadIdx.x & 31, q = lane >> 2, c2 = 2 * (lane & 3);
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const float* x = X + (long long)min(key0 + 16 * k + c2 + (i & 1) + (i >> 1) * 8, S - 1) * r;
+#pragma unroll
+            for (int n = 0; n < 2; ++n) o.v[k][n][i] = __ldg(x + min(n0 + n * 8 + q, dh - 1));
         }
-        if (cut) tb_combine(red, v);
-        if (mine && !half && n0 + c2 < dh) ep((h0 + h) * dh + n0 + c2, n0 + c2 + 1 < dh, v);
-        w += TBF_WARPS;
-    } while (!cut && w < tasks);
+}
+// acc[n] += weights (16 tokens x 16 rows, zero past the last row) vals, k the k step of the 32 rows.
+__device__ __forceinline__ void tb_mix(float (&big)[2][4], float (&small)[2][4], const TbA& a, const TbVals& x, int k) {
+#pragma unroll
+    for (int n = 0; n < 2; ++n) {
+        TbB b;
+        tb_split_b(b.h, b.m, b.l, x.v[k][n][0], x.v[k][n][1], x.v[k][n][2], x.v[k][n][3]);
+        tb_mma6(big[n], small[n], a, b);
+    }
+}
+// Score fragments (tiles 2 k, 2 k + 1) as the A operand of k step k.
+__device__ __forceinline__ void tb_frag_a(TbA& a, const float (&sc)[4][4], int k) {
+    const float v[8] = {sc[2 * k][0], sc[2 * k][1], sc[2 * k][2], sc[2 * k][3], sc[2 * k + 1][0], sc[2 * k + 1][1], sc[2 * k + 1][2], sc[2 * k + 1][3]};
+    tb_split_a(a, v);
+}
+
+// Shares of a mix: 16 tokens x 16 columns per warp; columns of every other row pair are swapped by eights, which spreads the fragments' rows over the banks.
+constexpr int TB_SHARE = TBF_T * 16;
+__device__ __forceinline__ void tb_share_put(float* part, const float (&big)[2][4], const float (&small)[2][4]) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, q = lane >> 2, c2 = 2 * (lane & 3), sw = ((q >> 1) & 1) * 8;
+    float* o = part + warp * TB_SHARE + q * 16;
+#pragma unroll
+    for (int n = 0; n < 2; ++n) {
+        *reinterpret_cast<float2*>(o + ((n * 8 + c2) ^ sw)) = make_float2(big[n][0] + small[n][0], big[n][1] + small[n][1]);
+        *reinterpret_cast<float2*>(o + 8 * 16 + ((n * 8 + c2) ^ sw)) = make_float2(big[n][2] + small[n][2], big[n][3] + small[n][3]);
+    }
+}
+// Sums of the nc shares of each of n heads, in order: ep(head, column, value) for token `warp`, columns n0 .. n0 + 15 of a head dh wide.
+template <class EP>
+__device__ __forceinline__ void tb_share_sum(const float* part, int nc, int n, int n0, int dh, EP ep) {
+    const int t = threadIdx.x >> 5, lane = threadIdx.x & 31, sw = ((t >> 1) & 1) * 8, cc = lane & 15;
+    for (int h = lane >> 4; h < n; h += 2) {
+        if (n0 + cc >= dh) continue;
+        const float* s = part + h * nc * TB_SHARE + t * 16 + (cc ^ sw);
+        float v = s[0];
+        for (int i = 1; i < nc; ++i) v += s[i * TB_SHARE];
+        ep(h, n0 + cc, v);
+    }
 }
 
 // Sum over the 16 tokens of a column pair: v of tb_product's epilogue, the result in every lane of the column.
@@ -378,414 +387,628 @@ __device__ __forceinline__ float tb_col_sum(float top, float bottom) {
     s += __shfl_xor_sync(0xffffffffu, s, 16);
     return s;
 }
+// Column sums of 16 rows in shared memory: a warp four columns at a time, eight lanes each.
+__device__ __forceinline__ void tb_col_sums(const float* rows, int rs, int r, float* __restrict__ out) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, t = lane & 7;
+    for (int c0 = warp * 4; c0 < r; c0 += TBF_WARPS * 4) {
+        const int c = c0 + (lane >> 3), cc = min(c, r - 1);
+        float s = rows[t * rs + cc] + rows[(t + 8) * rs + cc];
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (t == 0 && c < r) out[c] = s;
+    }
+}
+__device__ __forceinline__ float tb_quad_max(float v) {
+    v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, 1));
+    return fmaxf(v, __shfl_xor_sync(0xffffffffu, v, 2));
+}
+__device__ __forceinline__ float tb_quad_sum(float v) {
+    v += __shfl_xor_sync(0xffffffffu, v, 1);
+    return v + __shfl_xor_sync(0xffffffffu, v, 2);
+}
 
-// Shared memory: tile ring | halves of sums | operand terms wide, narrow | fp32 rows xb, qf | score rows.
-struct TbSmem { unsigned char* ring; float4* red; bf16 *wide, *narrow; float *xb, *qf, *sc; };
-constexpr size_t TBF_FIXED = TBF_SLOTS * TBF_WARPS * 512 + TBF_THREADS / 2 * 16;
+// e / d, rounded correctly for a correctly rounded inverse (Markstein, IBM J. Res. Dev. 34, 1990).
+__device__ __forceinline__ float tb_quotient(float e, float d, float inverse) {
+    const float x = e * inverse;
+    return fmaf(fmaf(-x, d, e), inverse, x);
+}
+
+// Shared memory: weight ring | operand terms wide, narrow | fp32 rows (four products' worth) | parameter vectors | row statistics | shares of mixes, two rounds.
+struct TbSmem { unsigned char* ring; bf16 *wide, *narrow; float *rows, *vec, *stat0, *stat1, *share; };
 __host__ __device__ inline size_t tb_smem_terms(int stride) { return (size_t)3 * TBF_T * stride * 2; }
-__device__ __forceinline__ TbSmem tb_carve(unsigned char* base, const TbLayerParams& p) {
+__host__ __device__ inline int tb_vec_floats(int r, int f) { return tb_up8(5 * r + f); }
+__host__ __device__ inline size_t tb_smem_fixed(int ka, int kb, int rs, int r, int f) {
+    return tb_smem_terms(ka) + tb_smem_terms(kb) + sizeof(float) * (4 * TBF_T * rs + tb_vec_floats(r, f) + 2 * TBF_WARPS * TBF_T + 2 * TBF_WARPS * TB_SHARE);
+}
+__device__ __forceinline__ TbSmem tb_carve(unsigned char* base, size_t ring, const TbLayerParams& p) {
     TbSmem s;
     s.ring = base;
-    s.red = reinterpret_cast<float4*>(base + TBF_SLOTS * TBF_WARPS * 512);
-    s.wide = reinterpret_cast<bf16*>(base + TBF_FIXED);
+    s.wide = reinterpret_cast<bf16*>(base + ring);
     s.narrow = s.wide + 3 * TBF_T * p.ka;
-    s.xb = reinterpret_cast<float*>(s.narrow + 3 * TBF_T * p.kb);
-    s.qf = s.xb + TBF_T * p.rs;
-    s.sc = s.qf + TBF_T * p.rs;
+    s.rows = reinterpret_cast<float*>(s.narrow + 3 * TBF_T * p.kb);
+    s.vec = s.rows + 4 * TBF_T * p.rs;
+    s.stat0 = s.vec + tb_vec_floats(p.r, p.f);
+    s.stat1 = s.stat0 + TBF_WARPS * TBF_T;
+    s.share = s.stat1 + TBF_WARPS * TBF_T;
     // the padding of the terms is multiplied with zero weights: it has to be finite
-    uint32_t* z = reinterpret_cast<uint32_t*>(s.wide);
-    for (int i = threadIdx.x; i < 3 * TBF_T * (p.ka + p.kb) / 2; i += TBF_THREADS) z[i] = 0u;
+    uint4* z = reinterpret_cast<uint4*>(s.wide);
+    for (int i = threadIdx.x; i < 3 * TBF_T * (p.ka + p.kb) / 8; i += TBF_THREADS) z[i] = make_uint4(0u, 0u, 0u, 0u);
     return s;
+}
+__device__ __forceinline__ void tb_vec_in(float* dst, const float* __restrict__ src, int n) {
+    for (int i = threadIdx.x; i < n; i += TBF_THREADS) dst[i] = __ldg(src + i);
+}
+// A row's columns lane, lane + 32, ... (zeros past n or where the row is not live).
+template <int NR>
+__device__ __forceinline__ void tb_row_in(float (&v)[NR], const float* __restrict__ row, int n, bool live) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int i = 0; i < NR; ++i) v[i] = live && lane + 32 * i < n ? __ldg(row + lane + 32 * i) : 0.f;
 }
 
 // Phases: 0 x1 = x + o Wo, 1 hid = relu(LN2(x1) W1 + c1), 2 a = x1 + hid W2 + c2 (of `tail`), 3 q, k, v = LN1(x) [Wq Wk Wv] (of `head`).
 // They run through ONE copy of the code: a phase is executed once per launch, so instructions it does not share are fetched
-// from memory.
+// from memory.  NR: columns per lane of a row, U: weight units in flight, CW: rounds of 32 keys per warp.
+template <int NR, int U, int CW>
 __global__ void __launch_bounds__(TBF_THREADS) tb_fwd_kernel(const __grid_constant__ TbLayerParams p) {
     extern __shared__ __align__(128) unsigned char tb_sm[];
     const int b = blockIdx.x / p.tiles, t0 = (blockIdx.x - b * p.tiles) * TBF_T;
-    const int S = p.S, r = p.r, f = p.f, H = p.H, dh = r / H, nt = min(TBF_T, S - t0), rs = p.rs, ss = p.ss;
+    const int S = p.S, r = p.r, f = p.f, H = p.H, dh = r / H, nt = min(TBF_T, S - t0), rs = p.rs;
     const long long m0 = (long long)b * S + t0;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, q = lane >> 2;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, q = lane >> 2, c2 = 2 * (lane & 3);
     const int first = p.tail >= 0 ? 0 : 3, last = p.head >= 0 ? 4 : 3;
-    TbStream st(p.mats, first, last, tb_sm);
-    for (int i = 0; i < TBF_AHEAD; ++i) st.issue();             // the packed weights were final before the predecessor started
-    const TbSmem sm = tb_carve(tb_sm, p);
+    TbStream<U> st(p, tb_sm);
+#pragma unroll 1
+    for (int i = 0; i < U; ++i) st.issue();                     // the packed weights were final before the predecessor started
+    const TbSmem sm = tb_carve(tb_sm, (size_t)TBF_WARPS * U * TB_UNIT, p);
+    if (p.head >= 0) { tb_vec_in(sm.vec, p.g1, r); tb_vec_in(sm.vec + r, p.b1, r); }
+    if (p.tail >= 0) {
+        tb_vec_in(sm.vec + 2 * r, p.g2, r); tb_vec_in(sm.vec + 3 * r, p.b2, r); tb_vec_in(sm.vec + 4 * r, p.c2, r);
+        tb_vec_in(sm.vec + 5 * r, p.c1, f);
+    }
+    const float lm = p.head >= 0 ? __ldg(p.lam + p.head) : 0.f;
     pdl_wait();
     pdl_trigger();
-    __syncthreads();
     const TbStacks& s = p.s;
-    const bool even = (r & 1) == 0;
-    const bool live0 = q < nt, live1 = q + 8 < nt;
+    const bool live = warp < nt;                                // token `warp` is this warp's row
+    float res[NR], un[NR];                                      // residual row of `tail`, u row of `head`
+    if (p.tail >= 0) tb_row_in(res, s.x + p.tail * s.sMr + (m0 + warp) * r, r, live);
+    if (p.head >= 0) tb_row_in(un, p.u + p.head * p.u_stride + (m0 + warp) * r, r, live);
+    __syncthreads();
     if (p.tail >= 0) {
-        const int l = p.tail;
-        const float* qkv = s.qkv + 3 * l * s.sMr;
-        for (int c = lane; c < r; c += 32) sm.qf[warp * rs + c] = warp < nt ? __ldg(qkv + (m0 + warp) * r + c) : 0.f;
-        __syncthreads();
+        const float* qkv = s.qkv + 3 * p.tail * s.sMr + (long long)b * S * r;
         const float scale = 1.f / sqrtf((float)dh);
-        const int S16 = tb_up16(S);
+        const bool even = ((dh | r) & 1) == 0, evenS = (S & 1) == 0;
+        const int hl = warp / p.nc, key0 = (warp - hl * p.nc) * 32, key_step = p.nc * 32;
+        int buf = 0;
 #pragma unroll 1
         for (int h0 = 0; h0 < H; h0 += p.hg) {
-            const int hg = min(p.hg, H - h0);
-            tb_scores(qkv + s.sMr + (long long)b * S * r, r, sm.qf, rs, S, dh, h0, hg, sm.sc, ss);
-            __syncthreads();
-            // softmax over the keys: a warp takes four rows at a time, so that four dependent chains overlap
-            for (int w = warp * 4; w < hg * TBF_T; w += TBF_WARPS * 4) {
-                float* row = sm.sc + w * ss;
-                const int t = w & (TBF_T - 1), h = h0 + (w >> 4);
-                float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY}, se[4] = {};
-#pragma unroll 2
-                for (int j = lane; j < S; j += 32)
+            const int hg = min(p.hg, H - h0), col = (h0 + hl) * dh;
+            const bool mine = hl < hg;
+            float sc[CW][4][4] = {};
+            TbVals vals[CW];
+            float mx[2] = {-INFINITY, -INFINITY};
+            if (mine) {
+#pragma unroll 1
+                for (int k = 0; k < dh; k += 16) {
+                    TbKeys keys[CW];
+                    float2 qa[2][2];
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) mx[i] = fmaxf(mx[i], row[i * ss + j] * scale);
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) mx[i] = fmaxf(mx[i], __shfl_xor_sync(0xffffffffu, mx[i], o));
-#pragma unroll 2
-                for (int j = lane; j < S; j += 32)
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) { const float e = expf(row[i * ss + j] * scale - mx[i]); row[i * ss + j] = e; se[i] += e; }
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) se[i] += __shfl_xor_sync(0xffffffffu, se[i], o);
-                float* P = s.P + l * s.sP + (((long long)b * H + h) * S + t0 + t) * S;
-#pragma unroll 2
-                for (int j = lane; j < S16; j += 32)
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const float e = j < S ? row[i * ss + j] / se[i] : 0.f;
-                        row[i * ss + j] = e;
-                        if (p.train && t + i < nt && j < S) P[i * S + j] = e;
+                    for (int i = 0; i < 2; ++i) {
+                        const float* row = qkv + (long long)min(t0 + q + 8 * i, S - 1) * r + col;
+                        qa[i][0] = tb_ld2(row, k + c2, dh, even); qa[i][1] = tb_ld2(row, k + c2 + 8, dh, even);
                     }
+#pragma unroll
+                    for (int w = 0; w < CW; ++w) tb_load_keys(keys[w], qkv + s.sMr + col, r, key0 + w * key_step, S, k, dh, even);
+                    if (k == 0)
+#pragma unroll
+                        for (int w = 0; w < CW; ++w) tb_load_vals(vals[w], qkv + 2 * s.sMr + col, r, key0 + w * key_step, S, 0, dh);
+                    TbA a;
+                    const float v[8] = {qa[0][0].x, qa[0][0].y, qa[1][0].x, qa[1][0].y, qa[0][1].x, qa[0][1].y, qa[1][1].x, qa[1][1].y};
+                    tb_split_a(a, v);
+#pragma unroll
+                    for (int w = 0; w < CW; ++w) tb_scores(sc[w], a, keys[w]);
+                }
+                // softmax over the keys: fragments of rows q and q + 8, keys from S on weigh nothing
+#pragma unroll
+                for (int w = 0; w < CW; ++w)
+#pragma unroll
+                    for (int n = 0; n < 4; ++n)
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) {
+                            const bool in = key0 + w * key_step + n * 8 + c2 + (e & 1) < S;
+                            sc[w][n][e] = in ? sc[w][n][e] * scale : -INFINITY;
+                            mx[e >> 1] = fmaxf(mx[e >> 1], sc[w][n][e]);
+                        }
+            }
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                mx[i] = tb_quad_max(mx[i]);
+                if ((lane & 3) == 0) sm.stat0[warp * TBF_T + q + 8 * i] = mx[i];
             }
             __syncthreads();
-            tb_mix(qkv + 2 * s.sMr + (long long)b * S * r, r, sm.sc, ss, S, dh, h0, hg, sm.red, [&](int c, bool two, const float (&v)[4]) {
-                tb_put1(sm.narrow, p.kb, q, c, v[0]); tb_put1(sm.narrow, p.kb, q + 8, c, v[2]);
-                if (two) { tb_put1(sm.narrow, p.kb, q, c + 1, v[1]); tb_put1(sm.narrow, p.kb, q + 8, c + 1, v[3]); }
-                if (p.train) {
-                    float* o = s.o + l * s.sMr + (m0 + q) * r + c;
-                    if (live0) { o[0] = v[0]; if (two) o[1] = v[1]; }
-                    if (live1) { o[8LL * r] = v[2]; if (two) o[8LL * r + 1] = v[3]; }
+            float sum[2] = {};
+            if (mine) {
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    mx[i] = -INFINITY;
+                    for (int c = 0; c < p.nc; ++c) mx[i] = fmaxf(mx[i], sm.stat0[(hl * p.nc + c) * TBF_T + q + 8 * i]);
                 }
-            });
+#pragma unroll
+                for (int w = 0; w < CW; ++w)
+#pragma unroll
+                    for (int n = 0; n < 4; ++n)
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) {
+                            const bool in = key0 + w * key_step + n * 8 + c2 + (e & 1) < S;
+                            sc[w][n][e] = in ? expf(sc[w][n][e] - mx[e >> 1]) : 0.f;
+                            sum[e >> 1] += sc[w][n][e];
+                        }
+            }
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                sum[i] = tb_quad_sum(sum[i]);
+                if ((lane & 3) == 0) sm.stat1[warp * TBF_T + q + 8 * i] = sum[i];
+            }
             __syncthreads();
+            if (mine) {
+                float* P = s.P + p.tail * s.sP + (((long long)b * H + h0 + hl) * S + t0 + q) * S;
+                float inv[2];
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    sum[i] = 0.f;
+                    for (int c = 0; c < p.nc; ++c) sum[i] += sm.stat1[(hl * p.nc + c) * TBF_T + q + 8 * i];
+                    inv[i] = __frcp_rn(sum[i]);
+                }
+#pragma unroll
+                for (int w = 0; w < CW; ++w)
+#pragma unroll
+                    for (int n = 0; n < 4; ++n) {
+                        const int key = key0 + w * key_step + n * 8 + c2;
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) sc[w][n][e] = tb_quotient(sc[w][n][e], sum[e >> 1], inv[e >> 1]);
+                        if (p.train && key < S) {
+                            if (q < nt) tb_st2(P + key, sc[w][n][0], sc[w][n][1], key + 1 < S, evenS);
+                            if (q + 8 < nt) tb_st2(P + 8LL * S + key, sc[w][n][2], sc[w][n][3], key + 1 < S, evenS);
+                        }
+                    }
+            }
+#pragma unroll 1
+            for (int n0 = 0; n0 < dh; n0 += 16, buf ^= 1) {
+                float* share = sm.share + buf * TBF_WARPS * TB_SHARE;
+                if (mine) {
+                    if (n0 > 0)
+#pragma unroll
+                        for (int w = 0; w < CW; ++w) tb_load_vals(vals[w], qkv + 2 * s.sMr + col, r, key0 + w * key_step, S, n0, dh);
+                    float big[2][4] = {}, small[2][4] = {};
+#pragma unroll
+                    for (int w = 0; w < CW; ++w)
+#pragma unroll
+                        for (int k = 0; k < 2; ++k) {
+                            TbA a;
+                            tb_frag_a(a, sc[w], k);
+                            tb_mix(big, small, a, vals[w], k);
+                        }
+                    tb_share_put(share, big, small);
+                }
+                __syncthreads();
+                float* o = s.o + p.tail * s.sMr + (m0 + warp) * r + h0 * dh;
+                tb_share_sum(share, p.nc, hg, n0, dh, [&](int h, int c, float v) {
+                    tb_put1(sm.narrow, p.kb, warp, (h0 + h) * dh + c, v);
+                    if (p.train && live) o[h * dh + c] = v;
+                });
+            }
         }
+        __syncthreads();
     }
 #pragma unroll 1
     for (int ph = first; ph < last; ++ph) {
         if (ph & 1) {
-            // LayerNorm 2 of `tail`, or merge and LayerNorm 1 of `head`; a row per warp, lanes over the columns
+            // LayerNorm 2 of `tail`, or merge and LayerNorm 1 of `head`
             const bool one = ph == 3;
             const int l = one ? p.head : p.tail;
-            const long long o = l * s.sMr + m0 * r;
-            const float *g = one ? p.g1 : p.g2, *be = one ? p.b1 : p.b2;
-            float *xh_out = (one ? s.xhat1 : s.xhat2) + o, *n_out = (one ? s.n1 : s.n2) + o, *x_out = s.x + o;
-            const float* u = p.u + l * p.u_stride + m0 * r;
-            const float lm = one ? __ldg(p.lam + l) : 0.f;
-            for (int t = warp; t < TBF_T; t += TBF_WARPS) {
-                float v[TBF_MAX_R / 32], sum = 0.f, var = 0.f;
+            const long long o = l * s.sMr + (m0 + warp) * r;
+            const float *g = sm.vec + (one ? 0 : 2 * r), *be = g + r;
+            float *xh_out = (one ? s.xhat1 : s.xhat2) + o, *n_out = (one ? s.n1 : s.n2) + o;
+            float v[NR], sum = 0.f, var = 0.f;
 #pragma unroll
-                for (int i = 0; i < TBF_MAX_R / 32; ++i) {
-                    const int c = lane + 32 * i;
-                    v[i] = 0.f;
-                    if (c < r) {
-                        v[i] = one && p.tail < 0 ? 0.f : sm.xb[t * rs + c];
-                        if (one) {
-                            v[i] = lm * (t < nt ? __ldg(u + t * r + c) : 0.f) + (1.f - lm) * v[i];
-                            if (t < nt) x_out[t * r + c] = v[i];
-                        }
-                        sum += v[i];
+            for (int i = 0; i < NR; ++i) {
+                const int c = lane + 32 * i;
+                v[i] = 0.f;
+                if (c < r) {
+                    if (p.tail >= 0) {
+                        const float* y = sm.rows + warp * rs + c;
+                        v[i] = res[i];
+                        if (one) v[i] += sm.vec[4 * r + c];
+                        v[i] = (p.mats[0].cut ? y[0] + y[TBF_T * rs] : y[0]) + v[i];       // (phases 0 and 2 are r wide: cut alike)
+                        if (one && live) s.a[p.tail * p.u_stride + (m0 + warp) * r + c] = v[i];
                     }
-                }
-                const float mu = warp_sum(sum) / (float)r;
-#pragma unroll
-                for (int i = 0; i < TBF_MAX_R / 32; ++i)
-                    if (lane + 32 * i < r) { const float d = v[i] - mu; var = fmaf(d, d, var); }
-                const float rstd = 1.f / sqrtf(warp_sum(var) / (float)r + TB_LN_EPS);
-#pragma unroll
-                for (int i = 0; i < TBF_MAX_R / 32; ++i) {
-                    const int c = lane + 32 * i;
-                    if (c < r) {
-                        const float xh = (v[i] - mu) * rstd, n = xh * __ldg(g + c) + __ldg(be + c);
-                        tb_put1(sm.narrow, p.kb, t, c, n);
-                        if (p.train && t < nt) { xh_out[t * r + c] = xh; n_out[t * r + c] = n; }
+                    if (one) {
+                        v[i] = lm * un[i] + (1.f - lm) * v[i];
+                        if (live) s.x[o + c] = v[i];
+                    } else {
+                        res[i] = v[i];
                     }
+                    sum += v[i];
                 }
-                if (lane == 0 && t < nt) (one ? s.rstd1 : s.rstd2)[l * s.sM + m0 + t] = rstd;
             }
+            const float mu = warp_sum(sum) / (float)r;
+#pragma unroll
+            for (int i = 0; i < NR; ++i)
+                if (lane + 32 * i < r) { const float d = v[i] - mu; var = fmaf(d, d, var); }
+            const float rstd = 1.f / sqrtf(warp_sum(var) / (float)r + TB_LN_EPS);
+#pragma unroll
+            for (int i = 0; i < NR; ++i) {
+                const int c = lane + 32 * i;
+                if (c < r) {
+                    const float xh = (v[i] - mu) * rstd, n = xh * g[c] + be[c];
+                    tb_put1(sm.narrow, p.kb, warp, c, n);
+                    if (p.train && live) { xh_out[c] = xh; n_out[c] = n; }
+                }
+            }
+            if (lane == 0 && live) (one ? s.rstd1 : s.rstd2)[l * s.sM + m0 + warp] = rstd;
             __syncthreads();
         }
         const bool wide_in = ph == 2;
-        const long long o_tail = p.tail * s.sMr + m0 * r, o_hid = p.tail * s.sMf + m0 * f, o_a = p.tail * p.u_stride + m0 * r;
         const int r8 = tb_up8(r);
-        tb_product(st, p.mats[ph], wide_in ? sm.wide : sm.narrow, wide_in ? p.ka : p.kb, sm.red, [&](int n, const float (&v)[4]) {
+        tb_product(st, p.mats[ph], wide_in ? sm.wide : sm.narrow, wide_in ? p.ka : p.kb, [&](int half, int, int n, const float (&v)[4]) {
             if (ph == 1) {
-                const float2 c = tb_ld2(p.c1, n, f, false);
-                float h[4] = {fmaxf(v[0] + c.x, 0.f), fmaxf(v[1] + c.y, 0.f), fmaxf(v[2] + c.x, 0.f), fmaxf(v[3] + c.y, 0.f)};
-                if (n + 1 >= f) { h[1] = 0.f; h[3] = 0.f; }
                 if (n < f) {
+                    const bool two = n + 1 < f;
+                    const float x = sm.vec[5 * r + n], y = two ? sm.vec[5 * r + n + 1] : 0.f;
+                    const float h[4] = {fmaxf(v[0] + x, 0.f), two ? fmaxf(v[1] + y, 0.f) : 0.f, fmaxf(v[2] + x, 0.f), two ? fmaxf(v[3] + y, 0.f) : 0.f};
                     tb_put2(sm.wide, p.ka, q, n, h[0], h[1]); tb_put2(sm.wide, p.ka, q + 8, n, h[2], h[3]);
                     if (p.train) {
-                        float* out = s.hid + o_hid + (long long)q * f + n;
-                        if (live0) { out[0] = h[0]; if (n + 1 < f) out[1] = h[1]; }
-                        if (live1) { out[8LL * f] = h[2]; if (n + 1 < f) out[8LL * f + 1] = h[3]; }
+                        float* out = s.hid + p.tail * s.sMf + (m0 + q) * f + n;
+                        const bool even = (f & 1) == 0;
+                        if (q < nt) tb_st2(out, h[0], h[1], two, even);
+                        if (q + 8 < nt) tb_st2(out + 8LL * f, h[2], h[3], two, even);
                     }
                 }
             } else if (ph < 3) {
                 if (n < r) {
-                    const bool two = n + 1 < r;
-                    float* x = sm.xb + q * rs + n;
-                    const float2 z = make_float2(0.f, 0.f);
-                    float2 a0, a1;
-                    if (ph == 0) {
-                        const float* xg = s.x + o_tail + (long long)q * r;
-                        a0 = live0 ? tb_ld2(xg, n, r, even) : z; a1 = live1 ? tb_ld2(xg + 8LL * r, n, r, even) : z;
-                    } else {
-                        const float2 c = tb_ld2(p.c2, n, r, false);
-                        a0 = make_float2(x[0] + c.x, x[1] + c.y); a1 = make_float2(x[8 * rs] + c.x, x[8 * rs + 1] + c.y);
-                    }
-                    const float y0 = v[0] + a0.x, y1 = v[1] + a0.y, y2 = v[2] + a1.x, y3 = v[3] + a1.y;
-                    *reinterpret_cast<float2*>(x) = make_float2(y0, y1);
-                    *reinterpret_cast<float2*>(x + 8 * rs) = make_float2(y2, y3);
-                    if (ph == 2) {
-                        float* out = s.a + o_a + (long long)q * r + n;
-                        if (live0) { out[0] = y0; if (two) out[1] = y1; }
-                        if (live1) { out[8LL * r] = y2; if (two) out[8LL * r + 1] = y3; }
-                    }
+                    float* x = sm.rows + (half * TBF_T + q) * rs + n;
+                    *reinterpret_cast<float2*>(x) = make_float2(v[0], v[1]);
+                    *reinterpret_cast<float2*>(x + 8 * rs) = make_float2(v[2], v[3]);
                 }
             } else {
-                const int k = n / r8, c = n - k * r8;
+                const int k = n >= 2 * r8 ? 2 : n >= r8 ? 1 : 0, c = n - k * r8;
                 if (c < r) {
                     float* out = s.qkv + (3 * p.head + k) * s.sMr + (m0 + q) * r + c;
-                    if (live0) { out[0] = v[0]; if (c + 1 < r) out[1] = v[1]; }
-                    if (live1) { out[8LL * r] = v[2]; if (c + 1 < r) out[8LL * r + 1] = v[3]; }
+                    const bool even = (r & 1) == 0, two = c + 1 < r;
+                    if (q < nt) tb_st2(out, v[0], v[1], two, even);
+                    if (q + 8 < nt) tb_st2(out + 8LL * r, v[2], v[3], two, even);
                 }
             }
         });
-        __syncthreads();
+        if (ph < 3) __syncthreads();
+    }
+    if (p.tail >= 0 && p.head < 0) {
+        // the last layer's a, which nothing in this launch reads
+#pragma unroll
+        for (int i = 0; i < NR; ++i) {
+            const int c = lane + 32 * i;
+            const float* y = sm.rows + warp * rs + c;
+            if (c < r && live)
+                s.a[p.tail * p.u_stride + (m0 + warp) * r + c] = (p.mats[0].cut ? y[0] + y[TBF_T * rs] : y[0]) + (res[i] + sm.vec[4 * r + c]);
+        }
     }
 }
 
 // Phases: 0 dn1 = [dq | dk | dv] [Wq | Wk | Wv]^T (of `tail`); 1 dhid = da W2^T, 2 dn2 = dpre W1^T, 3 do = dx1 Wo^T (of `head`).
+template <int NR, int U, int CW>
 __global__ void __launch_bounds__(TBF_THREADS) tb_bwd_kernel(const __grid_constant__ TbLayerParams p) {
     extern __shared__ __align__(128) unsigned char tb_sm[];
-    __shared__ float lam_red[32];
     const int b = blockIdx.x / p.tiles, t0 = (blockIdx.x - b * p.tiles) * TBF_T;
-    const int S = p.S, r = p.r, f = p.f, H = p.H, dh = r / H, nt = min(TBF_T, S - t0), rs = p.rs, ss = p.ss, S16 = tb_up16(S);
+    const int S = p.S, r = p.r, f = p.f, H = p.H, dh = r / H, nt = min(TBF_T, S - t0), rs = p.rs;
     const long long m0 = (long long)b * S + t0;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, q = lane >> 2;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, q = lane >> 2, c2 = 2 * (lane & 3);
     const float scale = 1.f / sqrtf((float)dh);
     const int first = p.tail >= 0 ? 0 : 1, last = p.head >= 0 ? 4 : 1;
-    TbStream st(p.mats, first, last, tb_sm);
-    for (int i = 0; i < TBF_AHEAD; ++i) st.issue();
-    const TbSmem sm = tb_carve(tb_sm, p);
-    pdl_wait();
-    pdl_trigger();
-    __syncthreads();
+    const int hl = warp / p.nc, key0 = (warp - hl * p.nc) * 32, key_step = p.nc * 32;
+    const bool live = warp < nt;                                // token `warp` is this warp's row
     const TbStacks& s = p.s;
-    const bool even = (r & 1) == 0, live0 = q < nt, live1 = q + 8 < nt;
+    TbStream<U> st(p, tb_sm);
+#pragma unroll 1
+    for (int i = 0; i < U; ++i) st.issue();
+    const TbSmem sm = tb_carve(tb_sm, (size_t)TBF_WARPS * U * TB_UNIT, p);
+    // What the forward pass left was final before the predecessor started, except for the first launch, whose predecessor triggers nothing.
+    float xh[NR], up[NR], rstd = 0.f;                           // normalised row; u - a_prev
+    float lm = 0.f;
     if (p.tail >= 0) {
         const int l = p.tail;
-        float* dqkv = s.dqkv + 3 * l * s.sMr + m0 * r;
-        const bool vec = (S & 3) == 0;
-        // dk[t] = scale sum_s dS[s][t] q[s],  dv[t] = sum_s P[s][t] do[s]   (own tokens t, all tokens s)
-#pragma unroll 1
-        for (int hk = 0, hg; hk < 2 * H; hk += hg) {
-            const int k = hk >= H, h0 = k ? hk - H : hk;
-            hg = min(p.hg, H - h0);
-            const float* src = (k ? s.P + l * s.sP : s.dS[l & 1]) + ((long long)b * H + h0) * S * S + t0;
-            // columns t0 .. t0 + 15 of the S x S matrices, transposed into score rows: a thread moves four tokens of one row
-            for (int e = threadIdx.x; e < hg * 4 * S16; e += TBF_THREADS) {
-                const int hq = e / S16, j = e - hq * S16, t = (hq & 3) * 4;
-                float v[4] = {0.f, 0.f, 0.f, 0.f};
-                if (j < S) {
-                    const float* g = src + ((long long)(hq >> 2) * S + j) * S + t;
-                    if (vec && t < nt) { const float4 x = __ldg(reinterpret_cast<const float4*>(g)); v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w; }
-                    else
+        float ap[NR];
+        tb_vec_in(sm.vec, p.g1, r);
+        tb_row_in(xh, s.xhat1 + l * s.sMr + (m0 + warp) * r, r, live);
+        tb_row_in(up, p.u + l * p.u_stride + (m0 + warp) * r, r, live);
+        tb_row_in(ap, s.a + (l - 1) * p.u_stride + (m0 + warp) * r, r, live && l > 0);
 #pragma unroll
-                        for (int i = 0; i < 4; ++i) if (t + i < nt) v[i] = __ldg(g + i);
-                }
-                float* o = sm.sc + ((hq >> 2) * TBF_T + t) * ss + j;
-#pragma unroll
-                for (int i = 0; i < 4; ++i) o[i * ss] = v[i];
-            }
-            __syncthreads();
-            const float* X = (k ? s.dob[l & 1] : s.qkv + 3 * l * s.sMr) + (long long)b * S * r;
-            const float sc = k ? 1.f : scale;
-            tb_mix(X, r, sm.sc, ss, S, dh, h0, hg, sm.red, [&](int c, bool two, const float (&v)[4]) {
-                const float y0 = v[0] * sc, y1 = v[1] * sc, y2 = v[2] * sc, y3 = v[3] * sc;
-                const int w = (k + 1) * r + c;
-                tb_put1(sm.wide, p.ka, q, w, y0); tb_put1(sm.wide, p.ka, q + 8, w, y2);
-                if (two) { tb_put1(sm.wide, p.ka, q, w + 1, y1); tb_put1(sm.wide, p.ka, q + 8, w + 1, y3); }
-                float* o = dqkv + (k + 1) * s.sMr + (long long)q * r + c;
-                if (live0) { o[0] = y0; if (two) o[1] = y1; }
-                if (live1) { o[8LL * r] = y2; if (two) o[8LL * r + 1] = y3; }
-            });
-            __syncthreads();
+        for (int i = 0; i < NR; ++i) up[i] -= ap[i];
+        rstd = live ? __ldg(s.rstd1 + l * s.sM + m0 + warp) : 0.f;
+        lm = __ldg(p.lam + l);
+    }
+    if (p.head >= 0) tb_vec_in(sm.vec + r, p.g2, r);
+    pdl_wait();
+    pdl_trigger();
+    float res[NR];                                              // gradient past the norm: dx1 of `tail`, then da of `head`
+    unsigned open = 0;                                          // hidden units of this warp's first eight tiles
+    if (p.head >= 0) {
+        const float* hid = s.hid + p.head * s.sMf + (m0 + q) * f;
+        const int tiles = p.mats[1].tiles(warp);
+        const bool even = (f & 1) == 0;
+#pragma unroll 2
+        for (int i = 0; i < min(8, tiles); ++i) {
+            const int n = (warp + i * TBF_WARPS) * 8 + c2;
+            const float2 h0 = q < nt ? tb_ld2(hid, n, f, even) : make_float2(0.f, 0.f), h1 = q + 8 < nt ? tb_ld2(hid + 8LL * f, n, f, even) : make_float2(0.f, 0.f);
+            open |= (unsigned)((h0.x > 0.f ? 1 : 0) | (h0.y > 0.f ? 2 : 0) | (h1.x > 0.f ? 4 : 0) | (h1.y > 0.f ? 8 : 0)) << (4 * i);
         }
-        for (int c = lane; c < r; c += 32) tb_put1(sm.wide, p.ka, warp, c, warp < nt ? __ldg(dqkv + warp * r + c) : 0.f);
+    }
+    __syncthreads();
+    if (p.tail >= 0) {
+        const int l = p.tail;
+        float* dqkv = s.dqkv + 3 * l * s.sMr + (m0 + warp) * r;
+        float dq[NR];
+        tb_row_in(dq, dqkv, r, live);
+        tb_row_in(res, s.dx1 + l * s.sMr + (m0 + warp) * r, r, live);
+        // dk[t] = scale sum_s dS[s][t] q[s],  dv[t] = sum_s P[s][t] do[s]   (own tokens t, all tokens s): 2 H heads of one mix
+        int buf = 0;
+#pragma unroll 1
+        for (int hk0 = 0; hk0 < 2 * H; hk0 += p.hg) {
+            const int hg = min(p.hg, 2 * H - hk0);
+            const bool mine = hl < hg;
+            const int hk = hk0 + hl, k = hk >= H, h = hk - k * H;
+            const float* W = (k ? s.P + l * s.sP : s.dS[l & 1]) + ((long long)b * H + h) * S * S + t0;
+            const float* X = (k ? s.dob[l & 1] : s.qkv + 3 * l * s.sMr) + (long long)b * S * r + h * dh;
+#pragma unroll 1
+            for (int n0 = 0; n0 < dh; n0 += 16, buf ^= 1) {
+                float* share = sm.share + buf * TBF_WARPS * TB_SHARE;
+                if (mine) {
+                    float big[2][4] = {}, small[2][4] = {};
+#pragma unroll
+                    for (int w = 0; w < CW; ++w) {
+                        const int s0 = key0 + w * key_step;
+                        float wt[2][8];
+                        TbVals x;
+#pragma unroll
+                        for (int j = 0; j < 2; ++j)
+#pragma unroll
+                            for (int i = 0; i < 8; ++i) {      // pairs (row q, q + 8) x (k c2, c2 + 8)
+                                const int k_ = s0 + 16 * j + c2 + (i & 1) + (i >> 2) * 8, t = q + ((i >> 1) & 1) * 8;
+                                wt[j][i] = k_ < S && t < nt ? __ldg(W + (long long)k_ * S + t) : 0.f;
+                            }
+                        tb_load_vals(x, X, r, s0, S, n0, dh);
+#pragma unroll
+                        for (int j = 0; j < 2; ++j) {
+                            TbA a;
+                            tb_split_a(a, wt[j]);
+                            tb_mix(big, small, a, x, j);
+                        }
+                    }
+                    tb_share_put(share, big, small);
+                }
+                __syncthreads();
+                tb_share_sum(share, p.nc, hg, n0, dh, [&](int i, int c, float v) {
+                    const int k1 = hk0 + i >= H ? 2 : 1, at = (hk0 + i - (k1 - 1) * H) * dh + c;
+                    if (k1 == 1) v *= scale;
+                    tb_put1(sm.wide, p.ka, warp, k1 * r + at, v);
+                    if (live) dqkv[k1 * s.sMr + at] = v;
+                });
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < NR; ++i)
+            if (lane + 32 * i < r) tb_put1(sm.wide, p.ka, warp, lane + 32 * i, dq[i]);
     } else {
         // da_L: the same vector for every token of the sample
-        const int t = warp;
-        for (int c = lane; c < r; c += 32) {
-            const int e = t * r + c;
-            const float v = t < nt ? __ldg(p.daL + (long long)b * r + c) : 0.f;
-            sm.xb[t * rs + c] = v;
-            tb_put1(sm.narrow, p.kb, t, c, v);
-            if (t < nt) s.da[p.head * s.sMr + m0 * r + e] = v;
+        tb_row_in(res, p.daL + (long long)b * r, r, live);
+#pragma unroll
+        for (int i = 0; i < NR; ++i) {
+            const int c = lane + 32 * i;
+            if (c >= r) continue;
+            sm.rows[(2 * TBF_T + warp) * rs + c] = res[i];
+            tb_put1(sm.narrow, p.kb, warp, c, res[i]);
+            if (live) s.da[p.head * s.sMr + (m0 + warp) * r + c] = res[i];
         }
     }
     __syncthreads();
 #pragma unroll 1
     for (int ph = first; ph < last; ++ph) {
         const int l = ph ? p.head : p.tail;
-        const long long o = l * s.sMr + m0 * r, o_hid = l * s.sMf + m0 * f;
-        float* part = s.part + ((long long)l * gridDim.x + blockIdx.x) * s.part_w;
-        const float* xhat = (ph ? s.xhat2 : s.xhat1) + o;
-        if (ph == 1)                                   // dc2: column sums of da
-            for (int c = threadIdx.x; c < r; c += TBF_THREADS) {
-                float a = 0.f;
-#pragma unroll
-                for (int t = 0; t < TBF_T; ++t) a += sm.xb[t * rs + c];
-                part[4 * r + c] = a;
-            }
+        const long long o = l * s.sMr + (m0 + warp) * r;
+        float* part = s.part + ((long long)l * gridDim.x + blockIdx.x) * p.s.part_w;
+        if (ph == 1) {
+            tb_col_sums(sm.rows + 2 * TBF_T * rs, rs, r, part + 4 * r);               // dc2: column sums of da
+            tb_row_in(xh, s.xhat2 + o, r, live);
+            rstd = live ? __ldg(s.rstd2 + l * s.sM + m0 + warp) : 0.f;
+        }
         const bool wide_in = !(ph & 1);
-        tb_product(st, p.mats[ph], wide_in ? sm.wide : sm.narrow, wide_in ? p.ka : p.kb, sm.red, [&](int n, const float (&v)[4]) {
+        tb_product(st, p.mats[ph], wide_in ? sm.wide : sm.narrow, wide_in ? p.ka : p.kb, [&](int half, int i, int n, const float (&v)[4]) {
             if (ph == 1) {                             // dpre = dhid where the unit is open; dc1
-                const float2 z = make_float2(0.f, 0.f);
-                const float* hid = s.hid + o_hid + (long long)q * f;
-                const bool ev = (f & 1) == 0;
-                const float2 h0 = live0 ? tb_ld2(hid, n, f, ev) : z, h1 = live1 ? tb_ld2(hid + 8LL * f, n, f, ev) : z;
-                const float y0 = h0.x > 0.f ? v[0] : 0.f, y1 = h0.y > 0.f ? v[1] : 0.f, y2 = h1.x > 0.f ? v[2] : 0.f, y3 = h1.y > 0.f ? v[3] : 0.f;
-                const float c0 = tb_col_sum(y0, y2), c1 = tb_col_sum(y1, y3);
+                unsigned on = open >> (4 * i);
+                if (i >= 8) {
+                    const float* hid = s.hid + l * s.sMf + (m0 + q) * f;
+                    const float2 z = make_float2(0.f, 0.f), h0 = q < nt ? tb_ld2(hid, n, f, false) : z, h1 = q + 8 < nt ? tb_ld2(hid + 8LL * f, n, f, false) : z;
+                    on = (h0.x > 0.f ? 1 : 0) | (h0.y > 0.f ? 2 : 0) | (h1.x > 0.f ? 4 : 0) | (h1.y > 0.f ? 8 : 0);
+                }
+                const float y0 = on & 1 ? v[0] : 0.f, y1 = on & 2 ? v[1] : 0.f, y2 = on & 4 ? v[2] : 0.f, y3 = on & 8 ? v[3] : 0.f;
+                const float s0 = tb_col_sum(y0, y2), s1 = tb_col_sum(y1, y3);
                 if (n < f) {
-                    const bool two = n + 1 < f;
+                    const bool two = n + 1 < f, ev = (f & 1) == 0;
                     tb_put2(sm.wide, p.ka, q, n, y0, y1); tb_put2(sm.wide, p.ka, q + 8, n, y2, y3);
-                    float* out = s.dpre + o_hid + (long long)q * f + n;
-                    if (live0) { out[0] = y0; if (two) out[1] = y1; }
-                    if (live1) { out[8LL * f] = y2; if (two) out[8LL * f + 1] = y3; }
-                    if (q == 0) { part[5 * r + n] = c0; if (two) part[5 * r + n + 1] = c1; }
+                    float* out = s.dpre + l * s.sMf + (m0 + q) * f + n;
+                    if (q < nt) tb_st2(out, y0, y1, two, ev);
+                    if (q + 8 < nt) tb_st2(out + 8LL * f, y2, y3, two, ev);
+                    if (q == 0) { part[5 * r + n] = s0; if (two) part[5 * r + n + 1] = s1; }
                 }
-            } else {
-                const bool norm = ph < 3, two = n + 1 < r;
-                float gx = 0.f, gy = 0.f, bx = 0.f, by = 0.f;
-                if (norm) {                            // dg = sum dn xhat, db = sum dn
-                    const float2 z = make_float2(0.f, 0.f);
-                    const float2 x0 = live0 ? tb_ld2(xhat + (long long)q * r, n, r, even) : z, x1 = live1 ? tb_ld2(xhat + (long long)(q + 8) * r, n, r, even) : z;
-                    gx = tb_col_sum(v[0] * x0.x, v[2] * x1.x); gy = tb_col_sum(v[1] * x0.y, v[3] * x1.y);
-                    bx = tb_col_sum(v[0], v[2]); by = tb_col_sum(v[1], v[3]);
-                }
-                if (n < r) {
-                    float* d = sm.qf + q * rs + n;
-                    *reinterpret_cast<float2*>(d) = make_float2(v[0], v[1]);
-                    *reinterpret_cast<float2*>(d + 8 * rs) = make_float2(v[2], v[3]);
-                    if (norm && q == 0) {
-                        float* w = part + (ph ? 2 * r : 0) + n;
-                        w[0] = gx; w[r] = bx;
-                        if (two) { w[1] = gy; w[r + 1] = by; }
-                    }
-                    if (!norm) {
-                        float* out = s.dob[l & 1] + (m0 + q) * r + n;
-                        if (live0) { out[0] = v[0]; if (two) out[1] = v[1]; }
-                        if (live1) { out[8LL * r] = v[2]; if (two) out[8LL * r + 1] = v[3]; }
-                    }
-                }
+            } else if (n < r) {
+                float* d = sm.rows + (((ph == 3 ? 2 : 0) + half) * TBF_T + q) * rs + n;
+                *reinterpret_cast<float2*>(d) = make_float2(v[0], v[1]);
+                *reinterpret_cast<float2*>(d + 8 * rs) = make_float2(v[2], v[3]);
             }
         });
         __syncthreads();
         if (ph & 1) continue;
-        // LayerNorm backward, a row per warp: dx = (gradient past the norm) + (dxhat - mean(dxhat) - xhat mean(dxhat xhat)) rstd;
-        // then dx1 of `head`, or the merge x = lambda u + (1 - lambda) a_prev of `tail`, whose da goes on to the layer below
-        const float* g = ph ? p.g2 : p.g1;
-        const float* rstd = (ph ? s.rstd2 : s.rstd1) + l * s.sM + m0;
-        const float* dx1 = s.dx1 + o;
-        const float lm = __ldg(p.lam + l);
-        const float *u = p.u + l * p.u_stride + m0 * r, *ap = l > 0 ? s.a + (l - 1) * p.u_stride + m0 * r : nullptr;
-        float acc = 0.f;
-        for (int t = warp; t < TBF_T; t += TBF_WARPS) {
-            float dxh[TBF_MAX_R / 32], xh[TBF_MAX_R / 32], s1 = 0.f, s2 = 0.f;
-            const bool live = t < nt;
+        // LayerNorm backward: dx = (gradient past the norm) + (dxhat - mean(dxhat) - xhat mean(dxhat xhat)) rstd;
+        // then dx1 of `head`, or the merge x = lambda u + (1 - lambda) a_prev of `tail`, whose da goes on to the layer below.
+        // dn and dn xhat go where the products' halves were (a row is read and written by its own warp): their column sums are db and dg.
+        const float* g = sm.vec + (ph ? r : 0);
+        float* row = sm.rows + warp * rs;
+        float dn[NR], s1 = 0.f, s2 = 0.f, acc = 0.f;
 #pragma unroll
-            for (int i = 0; i < TBF_MAX_R / 32; ++i) {
-                const int c = lane + 32 * i;
-                dxh[i] = xh[i] = 0.f;
-                if (c < r && live) {
-                    dxh[i] = sm.qf[t * rs + c] * __ldg(g + c);
-                    xh[i] = __ldg(xhat + t * r + c);
-                    s1 += dxh[i];
-                    s2 = fmaf(dxh[i], xh[i], s2);
+        for (int i = 0; i < NR; ++i) {
+            const int c = lane + 32 * i;
+            dn[i] = 0.f;
+            if (c < r) {
+                if (live) dn[i] = p.mats[ph].cut ? row[c] + row[TBF_T * rs + c] : row[c];
+                const float dxh = dn[i] * g[c];
+                s1 += dxh;
+                s2 = fmaf(dxh, xh[i], s2);
+            }
+        }
+        s1 = warp_sum(s1) / (float)r;
+        s2 = warp_sum(s2) / (float)r;
+#pragma unroll
+        for (int i = 0; i < NR; ++i) {
+            const int c = lane + 32 * i;
+            if (c >= r) continue;
+            float y = 0.f;
+            if (live) {
+                y = res[i] + (dn[i] * g[c] - s1 - xh[i] * s2) * rstd;
+                if (ph) s.dx1[o + c] = y;
+                else {
+                    acc = fmaf(y, up[i], acc);
+                    p.du[l * p.u_stride + (m0 + warp) * r + c] = lm * y;
+                    y *= 1.f - lm;
+                    if (p.head >= 0) s.da[p.head * s.sMr + (m0 + warp) * r + c] = y;
                 }
             }
-            s1 = warp_sum(s1) / (float)r;
-            s2 = warp_sum(s2) / (float)r;
-            const float rsd = live ? __ldg(rstd + t) : 0.f;
-#pragma unroll
-            for (int i = 0; i < TBF_MAX_R / 32; ++i) {
-                const int c = lane + 32 * i, e = t * r + c;
-                if (c >= r) continue;
-                float y = 0.f;
-                if (live) {
-                    y = (ph ? sm.xb[t * rs + c] : __ldg(dx1 + e)) + (dxh[i] - s1 - xh[i] * s2) * rsd;
-                    if (ph) s.dx1[o + e] = y;
-                    else {
-                        acc = fmaf(y, __ldg(u + e) - (ap ? __ldg(ap + e) : 0.f), acc);
-                        p.du[l * p.u_stride + m0 * r + e] = lm * y;
-                        y *= 1.f - lm;
-                        if (p.head >= 0) s.da[p.head * s.sMr + m0 * r + e] = y;
-                    }
-                }
-                sm.xb[t * rs + c] = y;
-                tb_put1(sm.narrow, p.kb, t, c, y);
-            }
+            row[c] = dn[i];
+            row[TBF_T * rs + c] = dn[i] * xh[i];
+            if (!ph) { row[2 * TBF_T * rs + c] = y; res[i] = y; }
+            tb_put1(sm.narrow, p.kb, warp, c, y);
         }
         if (ph == 0) {
-            const float tot = block_sum(acc, lam_red);
-            if (threadIdx.x == 0) part[5 * r + f] = tot;
+            acc = warp_sum(acc);
+            if (lane == 0) sm.stat0[warp] = acc;
         }
         __syncthreads();
+        tb_col_sums(sm.rows, rs, r, part + (ph ? 3 * r : r));
+        tb_col_sums(sm.rows + TBF_T * rs, rs, r, part + (ph ? 2 * r : 0));
+        if (ph == 0 && threadIdx.x == 0) {
+            float tot = 0.f;
+            for (int i = 0; i < TBF_WARPS; ++i) tot += sm.stat0[i];
+            part[5 * r + f] = tot;
+        }
     }
     if (p.head < 0) return;
     const int l = p.head;
-    // own queries: dP = do v^T, dS = P (dP - sum dP P), dq = scale dS k
+    TbKeys keys[CW];                   // v of the first 16 columns of a head, k as a mix operand, and P: operands of the second attention
+    TbVals vals[CW];
+    float P[CW][4][4];
+    const bool even = ((dh | r) & 1) == 0, evenS = (S & 1) == 0;
+    const float* qkv = s.qkv + 3 * l * s.sMr + (long long)b * S * r;
+    const auto operands = [&](int h) {
+        const float* Pg = s.P + l * s.sP + (((long long)b * H + h) * S + t0 + q) * S;
+#pragma unroll
+        for (int w = 0; w < CW; ++w) {
+            const int k0 = key0 + w * key_step;
+            tb_load_keys(keys[w], qkv + 2 * s.sMr + h * dh, r, k0, S, 0, dh, even);
+            tb_load_vals(vals[w], qkv + s.sMr + h * dh, r, k0, S, 0, dh);
+#pragma unroll
+            for (int n = 0; n < 4; ++n) {
+                const int key = k0 + n * 8 + c2;
+                const float2 x = q < nt ? tb_ld2(Pg, key, S, evenS) : make_float2(0.f, 0.f), y = q + 8 < nt ? tb_ld2(Pg + 8LL * S, key, S, evenS) : make_float2(0.f, 0.f);
+                P[w][n][0] = x.x; P[w][n][1] = x.y; P[w][n][2] = y.x; P[w][n][3] = y.y;
+            }
+        }
+    };
+    // own queries: dP = do v^T, dS = P (dP - sum dP P), dq = scale dS k; do stands in two halves
+    const float *do0 = sm.rows + 2 * TBF_T * rs, *do1 = do0 + TBF_T * rs;
+    const bool halves = p.mats[3].cut;
+    if (live)
+        for (int c = lane; c < r; c += 32) s.dob[l & 1][(m0 + warp) * r + c] = halves ? do0[warp * rs + c] + do1[warp * rs + c] : do0[warp * rs + c];
+    int buf = 0;
 #pragma unroll 1
     for (int h0 = 0; h0 < H; h0 += p.hg) {
-        const int hg = min(p.hg, H - h0);
-        tb_scores(s.qkv + (3 * l + 2) * s.sMr + (long long)b * S * r, r, sm.qf, rs, S, dh, h0, hg, sm.sc, ss);
-        __syncthreads();
-        for (int w = warp * 4; w < hg * TBF_T; w += TBF_WARPS * 4) {
-            float* row = sm.sc + w * ss;
-            const int t = w & (TBF_T - 1), h = h0 + (w >> 4);
-            const long long po = (((long long)b * H + h) * S + t0 + t) * S;
-            const float* P = s.P + l * s.sP + po;
-            float* dS = s.dS[l & 1] + po;
-            float dot[4] = {};
-#pragma unroll 4
-            for (int j = lane; j < S; j += 32)
+        const int hg = min(p.hg, H - h0), h = h0 + hl;
+        const bool mine = hl < hg;
+        float sc[CW][4][4] = {}, dot[2] = {};
+        if (mine) {
+            operands(h);
+#pragma unroll 1
+            for (int k = 0; k < dh; k += 16) {
+                if (k > 0)
 #pragma unroll
-                for (int i = 0; i < 4; ++i) dot[i] = fmaf(row[i * ss + j], t + i < nt ? __ldg(P + i * S + j) : 0.f, dot[i]);
+                    for (int w = 0; w < CW; ++w) tb_load_keys(keys[w], qkv + 2 * s.sMr + h * dh, r, key0 + w * key_step, S, k, dh, even);
+                // columns past the head's are zeros on the v side; what do holds there is finite
+                float v[8];
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-                for (int i = 0; i < 4; ++i) dot[i] += __shfl_xor_sync(0xffffffffu, dot[i], o);
-#pragma unroll 4
-            for (int j = lane; j < S16; j += 32)
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const bool live = t + i < nt && j < S;
-                    const float v = live ? __ldg(P + i * S + j) * (row[i * ss + j] - dot[i]) : 0.f;
-                    row[i * ss + j] = v;
-                    if (live) dS[i * S + j] = v;
+                for (int i = 0; i < 8; ++i) {
+                    const int c = k + c2 + (i & 1) + (i >> 2) * 8, at = (q + ((i >> 1) & 1) * 8) * rs + h * dh + c;
+                    v[i] = c < dh ? (halves ? do0[at] + do1[at] : do0[at]) : 0.f;
                 }
+                TbA a;
+                tb_split_a(a, v);
+#pragma unroll
+                for (int w = 0; w < CW; ++w) tb_scores(sc[w], a, keys[w]);
+            }
+#pragma unroll
+            for (int w = 0; w < CW; ++w)
+#pragma unroll
+                for (int n = 0; n < 4; ++n)
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) dot[e >> 1] = fmaf(sc[w][n][e], P[w][n][e], dot[e >> 1]);
+        }
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            dot[i] = tb_quad_sum(dot[i]);
+            if ((lane & 3) == 0) sm.stat0[warp * TBF_T + q + 8 * i] = dot[i];
         }
         __syncthreads();
-        tb_mix(s.qkv + (3 * l + 1) * s.sMr + (long long)b * S * r, r, sm.sc, ss, S, dh, h0, hg, sm.red, [&](int c, bool two, const float (&v)[4]) {
-            float* o = s.dqkv + 3 * l * s.sMr + (m0 + q) * r + c;
-            if (live0) { o[0] = v[0] * scale; if (two) o[1] = v[1] * scale; }
-            if (live1) { o[8LL * r] = v[2] * scale; if (two) o[8LL * r + 1] = v[3] * scale; }
-        });
-        __syncthreads();
+        if (mine) {
+            float* dS = s.dS[l & 1] + (((long long)b * H + h) * S + t0 + q) * S;
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                dot[i] = 0.f;
+                for (int c = 0; c < p.nc; ++c) dot[i] += sm.stat0[(hl * p.nc + c) * TBF_T + q + 8 * i];
+            }
+#pragma unroll
+            for (int w = 0; w < CW; ++w)
+#pragma unroll
+                for (int n = 0; n < 4; ++n) {
+                    const int key = key0 + w * key_step + n * 8 + c2;
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) sc[w][n][e] = key + (e & 1) < S ? P[w][n][e] * (sc[w][n][e] - dot[e >> 1]) : 0.f;
+                    if (key < S) {
+                        if (q < nt) tb_st2(dS + key, sc[w][n][0], sc[w][n][1], key + 1 < S, evenS);
+                        if (q + 8 < nt) tb_st2(dS + 8LL * S + key, sc[w][n][2], sc[w][n][3], key + 1 < S, evenS);
+                    }
+                }
+        }
+#pragma unroll 1
+        for (int n0 = 0; n0 < dh; n0 += 16, buf ^= 1) {
+            float* share = sm.share + buf * TBF_WARPS * TB_SHARE;
+            if (mine) {
+                if (n0 > 0)
+#pragma unroll
+                    for (int w = 0; w < CW; ++w) tb_load_vals(vals[w], qkv + s.sMr + h * dh, r, key0 + w * key_step, S, n0, dh);
+                float big[2][4] = {}, small[2][4] = {};
+#pragma unroll
+                for (int w = 0; w < CW; ++w)
+#pragma unroll
+                    for (int k = 0; k < 2; ++k) {
+                        TbA a;
+                        tb_frag_a(a, sc[w], k);
+                        tb_mix(big, small, a, vals[w], k);
+                    }
+                tb_share_put(share, big, small);
+            }
+            __syncthreads();
+            if (live) {
+                float* dq = s.dqkv + 3 * l * s.sMr + (m0 + warp) * r + h0 * dh;
+                tb_share_sum(share, p.nc, hg, n0, dh, [&](int i, int c, float v) { dq[i * dh + c] = v * scale; });
+            }
+        }
     }
 }
 
@@ -824,11 +1047,21 @@ __global__ void __launch_bounds__(256) tb_reduce_slices_kernel(const float* __re
     g[e < rr4 ? bl.wq + e : e < rr4 + rf ? bl.w1 + e - rr4 : bl.w2 + e - rr4 - rf] = v;
 }
 
+// Variant of the kernels for a shape: NR by the width, as many units in flight as shared memory leaves room for, and three rounds of keys per warp for
+// sequences beyond 16 warps of 32.
 struct TbPlan {
     bool ok = false;
-    int hg = 0, ka = 0, kb = 0, rs = 0, ss = 0;
+    int variant = 0, ka = 0, kb = 0, rs = 0, nc = 0, hg = 0;
     size_t smem = 0;
 };
+struct TbVariant { int nr, u, cw; const void *fwd, *bwd; };
+#define TB_VARIANT(NR, U, CW) {NR, U, CW, (const void*)tb_fwd_kernel<NR, U, CW>, (const void*)tb_bwd_kernel<NR, U, CW>}
+inline const TbVariant* tb_variants(int* n) {
+    static const TbVariant v[] = {TB_VARIANT(2, 5, 1), TB_VARIANT(2, 3, 1), TB_VARIANT(3, 4, 1), TB_VARIANT(6, 3, 1), TB_VARIANT(6, 2, 1), TB_VARIANT(6, 2, 3)};
+    *n = (int)(sizeof(v) / sizeof(v[0]));
+    return v;
+}
+#undef TB_VARIANT
 
 inline TbPlan tb_plan(int S, int r, int f, int H, int max_smem) {
     TbPlan pl;
@@ -836,20 +1069,20 @@ inline TbPlan tb_plan(int S, int r, int f, int H, int max_smem) {
     pl.ka = tb_up16(f > 3 * r ? f : 3 * r) + 8;
     pl.kb = tb_up16(r) + 8;
     pl.rs = (r + 31) / 32 * 32 + 8;            // = 8 mod 32: the fragments' pairs of four rows fall into different banks
-    pl.ss = (tb_up16(S) + 31) / 32 * 32 + 8;
-    const size_t fixed = TBF_FIXED + tb_smem_terms(pl.ka) + tb_smem_terms(pl.kb) + sizeof(float) * 2 * TBF_T * pl.rs;
-    const size_t per_head = sizeof(float) * TBF_T * pl.ss;
-    const size_t most = (size_t)max_smem - 1024;
-    if (fixed + per_head > most) return pl;
-    const int fit = (int)((most - fixed) / per_head);
-    const int groups = (H + fit - 1) / fit;
-    pl.hg = (H + groups - 1) / groups;         // heads in even groups
-    pl.smem = fixed + pl.hg * per_head;
-    if (smem_opt_in((const void*)tb_fwd_kernel, pl.smem) != cudaSuccess || smem_opt_in((const void*)tb_bwd_kernel, pl.smem) != cudaSuccess) {
-        cudaGetLastError();
+    const int chunks = (S + 31) / 32;
+    pl.nc = chunks < TBF_WARPS ? chunks : TBF_WARPS;
+    pl.hg = TBF_WARPS / pl.nc;
+    int n;
+    const TbVariant* v = tb_variants(&n);
+    for (int i = 0; i < n; ++i) {
+        if (r > 32 * v[i].nr || chunks > pl.nc * v[i].cw) continue;
+        pl.smem = (size_t)TBF_WARPS * v[i].u * TB_UNIT + tb_smem_fixed(pl.ka, pl.kb, pl.rs, r, f);
+        if (pl.smem + 1024 > (size_t)max_smem) continue;
+        if (smem_opt_in(v[i].fwd, pl.smem) != cudaSuccess || smem_opt_in(v[i].bwd, pl.smem) != cudaSuccess) { cudaGetLastError(); continue; }
+        pl.variant = i;
+        pl.ok = true;
         return pl;
     }
-    pl.ok = true;
     return pl;
 }
 
@@ -857,11 +1090,14 @@ inline int tb_ctas(int B, int S) { return B * ((S + TBF_T - 1) / TBF_T); }
 
 inline cudaError_t tb_layer_launch(const TbPlan& pl, TbLayerParams p, bool backward, cudaStream_t stream) {
     p.tiles = (p.S + TBF_T - 1) / TBF_T;
-    p.hg = pl.hg; p.ka = pl.ka; p.kb = pl.kb; p.rs = pl.rs; p.ss = pl.ss;
+    p.nc = pl.nc; p.hg = pl.hg; p.ka = pl.ka; p.kb = pl.kb; p.rs = pl.rs;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[1];
     pdl_launch_config(&cfg, attr, dim3((unsigned)tb_ctas(p.B, p.S)), dim3(TBF_THREADS), pl.smem, stream);
-    return backward ? cudaLaunchKernelEx(&cfg, tb_bwd_kernel, p) : cudaLaunchKernelEx(&cfg, tb_fwd_kernel, p);
+    int n;
+    const TbVariant& v = tb_variants(&n)[pl.variant];
+    void* args[] = {&p};
+    return cudaLaunchKernelExC(&cfg, backward ? v.bwd : v.fwd, args);
 }
 
 }  // namespace pac
