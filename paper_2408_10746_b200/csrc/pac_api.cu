@@ -29,7 +29,6 @@ namespace {
 
 constexpr int STAGE_SLOTS = 8;
 constexpr int LM_MAX_K_SLICES = 8;
-constexpr int ZC_SLOTS = 64;
 
 struct Scratch {
     // per-step state, sized for max_batch
@@ -215,15 +214,7 @@ struct pac_ctx {
     bool lm_ce_stream = false;     // LM cross-entropy as a register-resident stream over the logits (V <= 32768, V % 4 == 0)
     HostCache hc;                  // out-of-core mode (pac_cache_register_host)
     TBody tb;                      // transformer-body adapters (fp32 precision throughout)
-    // pac_train_step_async without copy nodes in the stream: a ring of id slots in page-locked host memory that
-    // the forward kernel reads directly (two halves, an event per half orders the reuse)
-    int* zc_ids = nullptr;         // [ZC_SLOTS][max_batch]
-    unsigned* zc_tags = nullptr;   // [ZC_SLOTS] page-locked: sequence number of the step whose ids the slot holds (written last)
-    int* zc_dev_ids = nullptr;     // [2][max_batch] device: ids a finalisation kernel fetched for the step after it
-    unsigned* zc_dev_tag = nullptr;// [2] device: sequence number those ids belong to
-    cudaEvent_t zc_ev[2] = {nullptr, nullptr};
-    unsigned long long zc_count = 0;
-    bool step_host_ids = false;    // the step being enqueued reads its ids from the ring
+    const int* step_arg_ids = nullptr;   // host ids of the step being enqueued, which travel as arguments of its kernels (arg_ids_ok)
     bool step_early_ids = false;   // the step's device ids were final before any kernel still in flight was launched
     std::string err;
 };
@@ -348,7 +339,8 @@ void time_mark(pac_ctx* c, int which, bool stop) {
 }
 
 // ---- staging of host ids ----
-// Ids of an ordinary minibatch (or short epoch) travel as a kernel argument: a copy from page-locked memory is another engine's work,
+// Ids of the one-launch forward are arguments of the kernels themselves (step_arg_ids).  Elsewhere the ids of an ordinary minibatch (or short epoch) travel as the
+// argument of a kernel that stores them: a copy from page-locked memory is another engine's work,
 // with a hand-over before and after it (blocking fp32 step on the smallest configuration 58.6 -> 47.6 us,
 // with the loss written straight to host memory; evaluation of 27 samples 26.8 -> 23.7 us).
 // Above PUT_IDS (2 KB of arguments) the copy engine's rate counts.
@@ -370,13 +362,17 @@ pac_status put_ids(pac_ctx* c, const int* ids, int n, int* out) {
     if (e != cudaSuccess) return fail(c, PAC_ERR_CUDA, "id kernel launch failed: %s", cudaGetErrorString(e));
     return PAC_OK;
 }
-pac_status stage_ids(pac_ctx* c, const int* ids, int B, const char* who) {
+pac_status check_ids(pac_ctx* c, const int* ids, int B, const char* who) {
     if (!ids) return fail(c, PAC_ERR_INVALID_ARG, "%s: sample_ids is NULL", who);
     if (B < 1 || B > c->cfg.max_batch)
         return fail(c, PAC_ERR_INVALID_ARG, "%s: B=%d outside [1, max_batch=%d]", who, B, c->cfg.max_batch);
     for (int b = 0; b < B; ++b)
         if (ids[b] < 0 || ids[b] >= c->dm.N)
             return fail(c, PAC_ERR_SAMPLE_ID_RANGE, "%s: sample_ids[%d]=%d outside [0, %lld)", who, b, ids[b], c->dm.N);
+    return PAC_OK;
+}
+// (after check_ids)
+pac_status stage_ids(pac_ctx* c, const int* ids, int B) {
     if (B <= PUT_IDS) return put_ids(c, ids, B, c->sc.ids);
     int s = c->slot;
     c->slot = (c->slot + 1) % STAGE_SLOTS;
@@ -943,6 +939,17 @@ pac_status down_projection(pac_ctx* c, const int* d_ids, int B) {
     return PAC_OK;
 }
 
+// Whether a step's host ids can be arguments of its kernels: the one-launch forward and the second pass then request their first cache tiles ahead of
+// everything before them in the stream, and no kernel has to store the ids first (T5-Base: evaluation of 27 samples
+// 23.6 -> 22.1 us, a step of 32 with its own update launch 62.0 -> 58.0, with the fused one, whose ids the forward read from host memory before, 55.8 -> 55.0).
+bool arg_ids_ok(const pac_ctx* c, int B) { return !c->hc.on && !c->tb.on && B <= ARG_IDS && use_fused_fwd(c, B); }
+ArgIds arg_ids(const pac_ctx* c, int B) {
+    ArgIds a;
+    a.n = c->step_arg_ids ? B : 0;
+    if (a.n) std::memcpy(a.v, c->step_arg_ids, sizeof(int) * B);
+    return a;
+}
+
 pac_status dw_down(pac_ctx* c, const int* d_ids, int B, bool reduce_splits) {
     pac_status st;
     time_mark(c, 2, false);
@@ -952,8 +959,7 @@ pac_status dw_down(pac_ctx* c, const int* d_ids, int B, bool reduce_splits) {
         const bool lm = c->cfg.head == PAC_HEAD_FROZEN_LM;
         gen.tc = c->sc.tc; gen.da = c->sc.da16; gen.da_term = (long long)(lm ? c->max_rows : c->cfg.max_batch) * dm.r;
         gen.da_sample = lm ? (long long)dm.S * dm.r : dm.r; gen.da_token = lm ? dm.r : 0;
-        st = tensor_dw_down(c->tplan, c->stream, d_ids, B, gen, c->sc.dw_part, c->status, &c->launches, next_stamp(c, 1),
-                            c->step_early_ids && !c->step_host_ids);       // ids no kernel in flight writes
+        st = tensor_dw_down(c->tplan, c->stream, d_ids, B, gen, c->sc.dw_part, c->status, &c->launches, next_stamp(c, 1), c->step_early_ids, arg_ids(c, B));
         if (st != PAC_OK) return fail(c, st, "tensor-core dW_down launch failed: %s", tensor_last_error());
     } else {
         st = c->dtype == PAC_F32 ? dw_down_simt<float>(c, d_ids, B, reduce_splits) : dw_down_simt<bf16>(c, d_ids, B, reduce_splits);
@@ -1012,17 +1018,11 @@ pac_status fused_fwd_enqueue(pac_ctx* c, const int* d_ids, int B, bool train, fl
     FusedFwdParams fp{};
     fp.mid = mid_params(c, pl.mp, d_ids, B, train, d_logits_out);
     fp.mid.layers_per_cta = pl.layers_per_cta;
-    if (c->step_host_ids) {
-        fp.mid.host_ids = 1; fp.mid.ids_copy = c->sc.ids;
-        const unsigned seq = (unsigned)(c->zc_count + 1);
-        fp.mid.pref_ids = c->zc_dev_ids + (size_t)(seq & 1u) * c->cfg.max_batch;
-        fp.mid.pref_tag = c->zc_dev_tag + (seq & 1u);
-        fp.mid.pref_seq = seq;
-    }
+    if (c->step_arg_ids && train) fp.mid.ids_copy = c->sc.ids;
     fp.mid.early_ids = c->step_early_ids ? 1 : 0;
     fp.k_chunks = pl.k_chunks; fp.stages = pl.stages; fp.mid_offset = pl.mid_offset; fp.state_offset = pl.state_offset; fp.n_land = pl.n_land; fp.wide_n = pl.wide_n;
     fp.stamp = next_stamp(c, 0);
-    cudaError_t e = fused_fwd_launch(pl, c->tplan.map_cache_fwd, c->tplan.map_w, fp, c->cfg.act, c->stream);
+    cudaError_t e = fused_fwd_launch(pl, c->tplan.map_cache_fwd, c->tplan.map_w, fp, arg_ids(c, B), c->cfg.act, c->stream);
     c->launches++;
     if (e != cudaSuccess) return fail(c, PAC_ERR_CUDA, "fused forward kernel launch failed: %s", cudaGetErrorString(e));
     return PAC_OK;
@@ -1113,16 +1113,6 @@ pac_status finalize_enqueue(pac_ctx* c, const int* d_ids, int B, float* d_loss, 
     f.wd_layer_elems = by_layer ? dm.d * dm.r : (int)c->lay.lam;
     f.wd_per_layer = (int)cdiv(f.wd_layer_elems / 4, 256);
     f.wd_blocks = f.wd_per_layer * (by_layer ? dm.L : 1);
-    if (c->step_host_ids) {
-        // the step after this one will look for its ids under sequence number zc_count + 2 in the next ring slot
-        const unsigned next_seq = (unsigned)(c->zc_count + 2);
-        const int next_slot = (int)((c->zc_count + 1) % ZC_SLOTS);
-        f.next_host_ids = c->zc_ids + (size_t)next_slot * c->cfg.max_batch;
-        f.next_host_tag = c->zc_tags + next_slot;
-        f.next_seq = next_seq; f.next_n = c->cfg.max_batch;
-        f.next_dev_ids = c->zc_dev_ids + (size_t)(next_seq & 1u) * c->cfg.max_batch;
-        f.next_dev_tag = c->zc_dev_tag + (next_seq & 1u);
-    }
     f.status = c->status;
     const unsigned rest_blocks = cdiv(dm.d, FIN_KB);
     f.rest_blocks = (int)rest_blocks;
@@ -1146,7 +1136,6 @@ pac_status train_enqueue(pac_ctx* c, const int* d_ids, int B, float* d_loss, con
     }
     if (use_fused_cls(c)) {
         if ((st = cls_forward_enqueue(c, d_ids, B, true, nullptr)) != PAC_OK) return st;
-        if (c->step_host_ids) d_ids = c->sc.ids;          // the forward kernel left a device copy for the later kernels
         if ((st = dw_down(c, d_ids, B, false)) != PAC_OK) return st;
         time_mark(c, 3, false);
         st = finalize_enqueue(c, d_ids, B, d_loss, hp);
@@ -1222,12 +1211,6 @@ void free_all(pac_ctx* c) {
     if (c->hc.iota) cudaFree(c->hc.iota);
     if (c->hc.copy_stream) cudaStreamDestroy(c->hc.copy_stream);
     if (c->hc.map_base) munmap(c->hc.map_base, c->hc.map_bytes);
-    if (c->zc_ids) cudaFreeHost(c->zc_ids);
-    if (c->zc_tags) cudaFreeHost(c->zc_tags);
-    if (c->zc_dev_ids) cudaFree(c->zc_dev_ids);
-    if (c->zc_dev_tag) cudaFree(c->zc_dev_tag);
-    for (auto& e : c->zc_ev)
-        if (e) cudaEventDestroy(e);
     if (c->h_ids) cudaFreeHost(c->h_ids);
     if (c->h_loss) cudaFreeHost(c->h_loss);
     if (c->h_losses) cudaFreeHost(c->h_losses);
@@ -1475,22 +1458,6 @@ pac_status pac_adapter_init(pac_ctx* c, const pac_adapter_cfg* cfg, unsigned lon
     }
     if (st == PAC_OK && cudaMallocHost((void**)&c->h_ids, sizeof(int) * STAGE_SLOTS * cfg->max_batch) != cudaSuccess)
         st = fail(c, PAC_ERR_NOMEM, "pinned id staging allocation failed");
-    if (st == PAC_OK && fused_shape) {
-        // id ring of pac_train_step_async (only the one-launch forward reads ids from host memory)
-        if (cudaMallocHost((void**)&c->zc_ids, sizeof(int) * ZC_SLOTS * cfg->max_batch) != cudaSuccess ||
-            cudaMallocHost((void**)&c->zc_tags, sizeof(unsigned) * ZC_SLOTS) != cudaSuccess ||
-            cudaMalloc((void**)&c->zc_dev_ids, sizeof(int) * 2 * cfg->max_batch) != cudaSuccess ||
-            cudaMalloc((void**)&c->zc_dev_tag, sizeof(unsigned) * 2) != cudaSuccess ||
-            cudaMemset(c->zc_dev_tag, 0, sizeof(unsigned) * 2) != cudaSuccess ||
-            cudaEventCreateWithFlags(&c->zc_ev[0], cudaEventDisableTiming) != cudaSuccess ||
-            cudaEventCreateWithFlags(&c->zc_ev[1], cudaEventDisableTiming) != cudaSuccess)
-            st = fail(c, PAC_ERR_NOMEM, "pinned id ring allocation failed");
-        else
-        {
-            std::memset(c->zc_tags, 0, sizeof(unsigned) * ZC_SLOTS);      // sequence numbers start at 1
-            std::memset(c->zc_ids, 0, sizeof(int) * ZC_SLOTS * cfg->max_batch);
-        }
-    }
     // tensor-core path: bf16 cache with TMA/UMMA-compatible sizes
     c->tensor_ok = false;
     if (st == PAC_OK && c->dtype == PAC_BF16 && tensor_shape_supported(dm) && !c->tb.on) {
@@ -1700,23 +1667,31 @@ pac_status host_cache_release(pac_ctx* c) {
 }
 
 // Ids of a step, wherever the cache lives: device ids the kernels index the (staged) cache with.
-pac_status prepare_ids(pac_ctx* c, const int* sample_ids, int B, const char* who, const int** d_ids) {
+// In the caller's kernels as arguments where `args` says that they take them so.
+pac_status prepare_ids(pac_ctx* c, const int* sample_ids, int B, const char* who, const int** d_ids, bool args) {
     if (c->hc.on) return host_cache_stage(c, sample_ids, B, who, d_ids);
     *d_ids = c->sc.ids;
-    return stage_ids(c, sample_ids, B, who);
+    pac_status st = check_ids(c, sample_ids, B, who);
+    if (st != PAC_OK) return st;
+    if (args) { c->step_arg_ids = sample_ids; return PAC_OK; }
+    return stage_ids(c, sample_ids, B);
 }
-pac_status finish_ids(pac_ctx* c) { return c->hc.on ? host_cache_release(c) : PAC_OK; }
+// After the step's kernels have been enqueued, with what came of that.
+pac_status finish_ids(pac_ctx* c, pac_status st) {
+    c->step_arg_ids = nullptr;
+    return st == PAC_OK && c->hc.on ? host_cache_release(c) : st;
+}
 
 }  // namespace
 
 pac_status pac_train_step(pac_ctx* c, const int* sample_ids, int B, float* loss_out) {
     NEED_INIT(c, "pac_train_step");
     const int* d_ids = nullptr;
-    pac_status st = prepare_ids(c, sample_ids, B, "pac_train_step", &d_ids);
+    pac_status st = prepare_ids(c, sample_ids, B, "pac_train_step", &d_ids, arg_ids_ok(c, B));
     if (st != PAC_OK) return st;
     // a loss somebody waits for goes straight to page-locked host memory
-    if ((st = train_enqueue(c, d_ids, B, loss_out ? c->h_loss : c->sc.loss, nullptr)) != PAC_OK) return st;
-    if ((st = finish_ids(c)) != PAC_OK) return st;
+    st = train_enqueue(c, d_ids, B, loss_out ? c->h_loss : c->sc.loss, nullptr);
+    if ((st = finish_ids(c, st)) != PAC_OK) return st;
     if (loss_out) {
         CU_OK(c, cudaStreamSynchronize(c->stream));
         *loss_out = *c->h_loss;
@@ -1727,10 +1702,9 @@ pac_status pac_train_step(pac_ctx* c, const int* sample_ids, int B, float* loss_
 pac_status pac_train_step_dev_loss(pac_ctx* c, const int* sample_ids, int B, float* dev_loss) {
     NEED_INIT(c, "pac_train_step_dev_loss");
     const int* d_ids = nullptr;
-    pac_status st = prepare_ids(c, sample_ids, B, "pac_train_step_dev_loss", &d_ids);
+    pac_status st = prepare_ids(c, sample_ids, B, "pac_train_step_dev_loss", &d_ids, arg_ids_ok(c, B));
     if (st != PAC_OK) return st;
-    if ((st = train_enqueue(c, d_ids, B, dev_loss ? dev_loss : c->sc.loss, nullptr)) != PAC_OK) return st;
-    return finish_ids(c);
+    return finish_ids(c, train_enqueue(c, d_ids, B, dev_loss ? dev_loss : c->sc.loss, nullptr));
 }
 
 pac_status pac_set_grad_scale(pac_ctx* c, float scale) {
@@ -1757,32 +1731,9 @@ pac_status pac_train_step_async(pac_ctx* c, const int* sample_ids, int B, const 
         }
     }
     const int* d_ids = nullptr;
-    if (!c->hc.on && c->zc_ids && c->timing == 0 && use_fused_fwd(c, B)) {
-        // one-launch forward: it reads the ids straight from a page-locked ring slot, so the step is three
-        // kernels back to back with nothing between them and the steps overlap as in pac_train_epoch_dev
-        if (!sample_ids) return fail(c, PAC_ERR_INVALID_ARG, "pac_train_step_async: sample_ids is NULL");
-        if (B < 1 || B > c->cfg.max_batch)
-            return fail(c, PAC_ERR_INVALID_ARG, "pac_train_step_async: B=%d outside [1, max_batch=%d]", B, c->cfg.max_batch);
-        for (int b = 0; b < B; ++b)
-            if (sample_ids[b] < 0 || sample_ids[b] >= c->dm.N)
-                return fail(c, PAC_ERR_SAMPLE_ID_RANGE, "pac_train_step_async: sample_ids[%d]=%d outside [0, %lld)", b, sample_ids[b], c->dm.N);
-        const int slot = (int)(c->zc_count % ZC_SLOTS), half = slot / (ZC_SLOTS / 2);
-        if (slot % (ZC_SLOTS / 2) == 0) CU_OK(c, cudaEventSynchronize(c->zc_ev[half]));     // the half's previous steps have run
-        int* h = c->zc_ids + (size_t)slot * c->cfg.max_batch;
-        std::memcpy(h, sample_ids, sizeof(int) * B);
-        // publish: ids first, then the step's sequence number (the kernel of the step before may be looking)
-        __atomic_store_n(&c->zc_tags[slot], (unsigned)(c->zc_count + 1), __ATOMIC_RELEASE);
-        c->step_host_ids = true;
-        st = train_enqueue(c, h, B, d_loss, hp);
-        c->step_host_ids = false;
-        if (st != PAC_OK) return st;
-        c->zc_count++;
-        if (slot % (ZC_SLOTS / 2) == ZC_SLOTS / 2 - 1) CU_OK(c, cudaEventRecord(c->zc_ev[half], c->stream));
-    } else {
-        if ((st = prepare_ids(c, sample_ids, B, "pac_train_step_async", &d_ids)) != PAC_OK) return st;
-        if ((st = train_enqueue(c, d_ids, B, d_loss, hp)) != PAC_OK) return st;
-        if ((st = finish_ids(c)) != PAC_OK) return st;
-    }
+    if ((st = prepare_ids(c, sample_ids, B, "pac_train_step_async", &d_ids, arg_ids_ok(c, B))) != PAC_OK) return st;
+    st = train_enqueue(c, d_ids, B, d_loss, hp);
+    if ((st = finish_ids(c, st)) != PAC_OK) return st;
     if (copy_loss) CU_OK(c, cudaMemcpyAsync(loss_out, d_loss, sizeof(float), cudaMemcpyDeviceToHost, c->stream));
     return PAC_OK;
 }
@@ -1798,29 +1749,30 @@ pac_status pac_eval_logits(pac_ctx* c, const int* sample_ids, int B, float* dev_
     NEED_INIT(c, "pac_eval_logits");
     if (!dev_out) return fail(c, PAC_ERR_INVALID_ARG, "pac_eval_logits: dev_out is NULL");
     const int* d_ids = nullptr;
-    pac_status st = prepare_ids(c, sample_ids, B, "pac_eval_logits", &d_ids);
+    pac_status st = prepare_ids(c, sample_ids, B, "pac_eval_logits", &d_ids, arg_ids_ok(c, B));
     if (st != PAC_OK) return st;
     st = c->tb.on ? tb_forward(c, d_ids, B, false, dev_out)
        : use_fused_cls(c) ? cls_forward_enqueue(c, d_ids, B, false, dev_out) : forward(c, d_ids, B, false, dev_out);
-    if (st != PAC_OK) return st;
-    return finish_ids(c);
+    return finish_ids(c, st);
 }
 
 pac_status pac_gather(pac_ctx* c, const int* sample_ids, int B, void* dev_out) {
     NEED_INIT(c, "pac_gather");
     if (!dev_out) return fail(c, PAC_ERR_INVALID_ARG, "pac_gather: dev_out is NULL");
     const int* d_ids = nullptr;
-    pac_status st = prepare_ids(c, sample_ids, B, "pac_gather", &d_ids);
+    pac_status st = prepare_ids(c, sample_ids, B, "pac_gather", &d_ids, !c->hc.on && B <= ARG_IDS);
     if (st != PAC_OK) return st;
     const Dims& dm = c->dm;
     const long long slab = (long long)dm.S * dm.d * (c->dtype == PAC_F32 ? 4 : 2);
     const int vec16 = (slab % 16 == 0) && (((uintptr_t)dev_out & 15) == 0);
     unsigned chunks = (unsigned)std::min<long long>(64, std::max<long long>(1, slab / (16 * 256 * 4)));
+    const ArgIds arg = arg_ids(c, B);
+    c->step_arg_ids = nullptr;
     dim3 grid((unsigned)(B * dm.L), chunks, 1);
     gather_kernel<<<grid, 256, 0, c->stream>>>((const unsigned char*)c->cache, d_ids, dm.N, dm.L, B, slab,
-                                               (unsigned char*)dev_out, vec16, c->status);
+                                               (unsigned char*)dev_out, vec16, c->status, arg);
     LAUNCH_CHECK(c);
-    return finish_ids(c);
+    return finish_ids(c, PAC_OK);
 }
 
 static pac_status epoch_common(pac_ctx* c, const int* d_perm, long long n, int B, const pac_adamw* hp, float* d_losses) {
@@ -1860,6 +1812,16 @@ pac_status pac_train_epoch(pac_ctx* c, const int* perm, long long n, int B, cons
             if ((st = host_cache_stage(c, perm + s * B, B, "pac_train_epoch", &d_ids)) != PAC_OK) return st;
             if ((st = train_enqueue(c, d_ids, B, c->h_losses + s, hp)) != PAC_OK) return st;
             if ((st = host_cache_release(c)) != PAC_OK) return st;
+        }
+        CU_OK(c, cudaStreamSynchronize(c->stream));
+        if (losses_out) std::memcpy(losses_out, c->h_losses, sizeof(float) * (n / B));
+        return PAC_OK;
+    }
+    if (arg_ids_ok(c, B)) {
+        for (long long s = 0; s < n / B; ++s) {
+            c->step_arg_ids = perm + s * B;
+            st = finish_ids(c, train_enqueue(c, c->sc.ids, B, c->h_losses + s, hp));
+            if (st != PAC_OK) return st;
         }
         CU_OK(c, cudaStreamSynchronize(c->stream));
         if (losses_out) std::memcpy(losses_out, c->h_losses, sizeof(float) * (n / B));

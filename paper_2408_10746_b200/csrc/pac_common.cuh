@@ -43,6 +43,11 @@ __device__ __forceinline__ long long safe_id(const int* __restrict__ ids, int b,
     return id;
 }
 
+// A minibatch's ids as a kernel argument (validated on the host): known before anything ahead in the stream has finished, at the price of one
+// constant load.  160: the one-launch forward takes a sample per cluster and 148 SMs hold fewer clusters than that.
+constexpr int ARG_IDS = 160;
+struct ArgIds { int n, v[ARG_IDS]; };       // n == 0: ids in memory
+
 // Dynamic shared memory above 48 KB needs an opt-in per kernel, and the attribute belongs to the
 // device the call is made on.  Several contexts (other shapes, other devices) share the kernels, so
 // the largest size granted so far is kept per (device, kernel) and never lowered.

@@ -39,7 +39,7 @@ constexpr int FUSED_DRAIN_WARP0 = 4;   // warps 4 .. 15 drain accumulators; warp
 
 template <int ACT>
 __global__ void __launch_bounds__(512, 1)
-fwd_cluster_kernel(const __grid_constant__ CUtensorMap map_cache, const __grid_constant__ CUtensorMap map_w, FusedFwdParams fp) {
+fwd_cluster_kernel(const __grid_constant__ CUtensorMap map_cache, const __grid_constant__ CUtensorMap map_w, FusedFwdParams fp, const __grid_constant__ ArgIds arg) {
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     cg::cluster_group cluster = cg::this_cluster();
@@ -74,15 +74,11 @@ fwd_cluster_kernel(const __grid_constant__ CUtensorMap map_cache, const __grid_c
     }
     if (warp == 1) { tmem_alloc(smem_u32(&tmem_base_sh), 512u); tmem_relinquish(); }
     pdl_trigger();
-    // Ids that were final before this launch (written by the host, or device ids no kernel ahead of this one
-    // touches) are read while the predecessor still drains, and so are the first cache tiles: the cache never
-    // changes, only the weights (updated by the predecessor) have to wait.  One thread fetches the id for the
-    // whole CTA: with ids in host memory every reading warp would be a transaction on the host link.
-    const bool early = p.host_ids || p.early_ids;
-    if (early && threadIdx.x == 64) {
-        const bool pref = p.host_ids && p.pref_tag && ld_acquire_gpu(p.pref_tag) == p.pref_seq;
-        id_sh = safe_id(pref ? p.pref_ids : p.ids, b, p.N, q == 0 ? p.status : nullptr);
-    }
+    // Ids that were final before this launch (arguments, or device ids no kernel ahead of this one
+    // touches) are known while the predecessor still drains, and so are the first cache tiles: the cache never
+    // changes, only the weights (updated by the predecessor) have to wait.
+    const bool early = arg.n > 0 || p.early_ids;
+    if (p.early_ids && threadIdx.x == 64) id_sh = safe_id(p.ids, b, p.N, q == 0 ? p.status : nullptr);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -92,7 +88,7 @@ fwd_cluster_kernel(const __grid_constant__ CUtensorMap map_cache, const __grid_c
     cluster.barrier_arrive();
     const uint32_t tmem_base = tmem_base_sh;
     volatile int* abort_flag = &abort_sh;
-    long long id = early ? id_sh : -1;
+    long long id = arg.n > 0 ? arg.v[b] : p.early_ids ? id_sh : -1;
     const uint64_t pol = l2_policy_evict_first();
     uint32_t pre = 0;                                            // stages whose cache tile is already on its way
     if (early && warp == 0 && n_layers > 0) {
@@ -383,7 +379,7 @@ inline int fused_fwd_max_clusters(const FusedFwdPlan& pl, int act) {
 
 template <int ACT>
 inline cudaError_t fused_fwd_launch_act(const FusedFwdPlan& pl, const CUtensorMap& map_cache, const CUtensorMap& map_w,
-                                        const FusedFwdParams& fp, cudaStream_t stream) {
+                                        const FusedFwdParams& fp, const ArgIds& arg, cudaStream_t stream) {
     {
         cudaError_t e = smem_opt_in((const void*)fwd_cluster_kernel<ACT>, pl.smem);
         if (e != cudaSuccess) return e;
@@ -402,13 +398,13 @@ inline cudaError_t fused_fwd_launch_act(const FusedFwdPlan& pl, const CUtensorMa
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, fwd_cluster_kernel<ACT>, map_cache, map_w, fp);
+    return cudaLaunchKernelEx(&cfg, fwd_cluster_kernel<ACT>, map_cache, map_w, fp, arg);
 }
 
 inline cudaError_t fused_fwd_launch(const FusedFwdPlan& pl, const CUtensorMap& map_cache, const CUtensorMap& map_w,
-                                    const FusedFwdParams& fp, int act, cudaStream_t stream) {
-    return act == PAC_ACT_RELU ? fused_fwd_launch_act<PAC_ACT_RELU>(pl, map_cache, map_w, fp, stream)
-                               : fused_fwd_launch_act<PAC_ACT_IDENTITY>(pl, map_cache, map_w, fp, stream);
+                                    const FusedFwdParams& fp, const ArgIds& arg, int act, cudaStream_t stream) {
+    return act == PAC_ACT_RELU ? fused_fwd_launch_act<PAC_ACT_RELU>(pl, map_cache, map_w, fp, arg, stream)
+                               : fused_fwd_launch_act<PAC_ACT_IDENTITY>(pl, map_cache, map_w, fp, arg, stream);
 }
 
 }  // namespace pac

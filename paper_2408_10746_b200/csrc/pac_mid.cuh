@@ -31,13 +31,8 @@ struct MidParams {
     int scratch;                // floats of block-local reduction scratch
     int aL_floats;              // floats of the a_L tile in shared memory (Sg * r; 0 when the chain ran elsewhere)
     int layers_per_cta;         // one-kernel forward: layers whose down-projections each CTA of the cluster computes
-    int host_ids;               // 1: ids points at host memory the device can read (written before the launch, so
-                                // it may be read ahead of the predecessor's completion); read once per CTA
     int early_ids;              // 1: no kernel ahead of this one in the stream writes the ids (device memory)
-    // host_ids only: where the previous step's finalisation may already have left this step's ids in device
-    // memory (valid when *pref_tag == pref_seq); otherwise the ids are fetched across the host link
-    const int* pref_ids; const unsigned* pref_tag; unsigned pref_seq;
-    int* ids_copy;              // one-kernel forward: device copy of the batch's (clamped) ids for the later kernels, or null
+    int* ids_copy;              // one-kernel forward: device copy of the batch's ids for the finalisation, or null
     // STATE_POOLED: what the down-projection kernel's epilogue left behind
     const float* pool_part;     // [B][n_pool_parts][r] token sums of a_L per token group
     int n_pool_parts;
@@ -622,10 +617,6 @@ struct FinalizeParams {
     pac_adamw hp; float bc1, bc2;
     float grad_scale;                                        // factor on every gradient entering the fused update
     WdShadow wdT;                                            // bf16 terms of W_down (p may be null)
-    // Ids of the NEXT step (pac_train_step_async): if the host has already published them in its page-locked
-    // ring (tag == next_seq), block 0 copies them to device memory, off every kernel's critical path.
-    const int* next_host_ids; const unsigned* next_host_tag; unsigned next_seq; int next_n;
-    int* next_dev_ids; unsigned* next_dev_tag;
     // Device status words: when a bounded wait of this step's passes or of an earlier step has run out, the gradients
     // are not trustworthy, so nothing is written to the gradients, parameters or moments.  The wait for the shares of P_l in this
     // kernel itself is different: should it run out, lambda stays as it is while blocks that had left their share have
@@ -634,17 +625,6 @@ struct FinalizeParams {
 };
 
 constexpr int FIN_KB = 4;       // hidden-width columns per head-side block of the finalisation kernel
-
-__device__ __forceinline__ unsigned ld_acquire_sys(const unsigned* p) {
-    unsigned v;
-    asm volatile("ld.acquire.sys.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-__device__ __forceinline__ unsigned ld_acquire_gpu(const unsigned* p) {
-    unsigned v;
-    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
 
 // dlambda_l = sum dz_l (u_l - a_{l-1}) without u or a.  With dz_l = cprod_l open_l daL and u_l = h_l W_l the first half is cprod_l P_l,
 // P_l = <D_l, W_l>; and where gates l .. L are open, a_{l-1} = sum over i < l with gates i .. l-1 open of
@@ -801,20 +781,6 @@ __global__ void __launch_bounds__(256, 5) finalize_cls_kernel(FinalizeParams f) 
             for (int b = lane; b < f.B; b += 32) acc += f.loss_b[b];
             acc = warp_sum(acc);
             if (lane == 0) *f.loss_out = acc / (float)f.B;
-        }
-        if (warp == 0 && f.next_host_tag) {
-            // the host writes a slot's ids first and its tag last; tag read first here, ids after it
-            const unsigned tag = ld_acquire_sys(f.next_host_tag);
-            if (tag == f.next_seq) {
-                for (int b = lane; b < f.next_n; b += 32) f.next_dev_ids[b] = *reinterpret_cast<const volatile int*>(f.next_host_ids + b);
-                // publish: the warp barrier orders every lane's id stores before lane 0, whose fence then
-                // comes between them and the tag
-                __syncwarp();
-                if (lane == 0) {
-                    __threadfence();
-                    atomicExch(f.next_dev_tag, f.next_seq);
-                }
-            }
         }
         // dlambda where it does not come from the W_down blocks: warp per layer, lanes over its partial sums, fixed shuffle order
         for (int l = warp; l < f.L && !f.coef && !dead; l += nw) {

@@ -16,9 +16,9 @@ namespace pac {
 // ---------------------------------------------------------------------------
 __global__ void gather_kernel(const unsigned char* __restrict__ cache, const int* __restrict__ ids, long long N,
                               int L, int B, long long slab_bytes, unsigned char* __restrict__ out, int vec16,
-                              unsigned* status) {
+                              unsigned* status, const __grid_constant__ ArgIds arg) {
     int l = blockIdx.x % L, b = blockIdx.x / L;
-    long long id = safe_id(ids, b, N, threadIdx.x == 0 && blockIdx.y == 0 ? status : nullptr);
+    long long id = arg.n > 0 ? arg.v[b] : safe_id(ids, b, N, threadIdx.x == 0 && blockIdx.y == 0 ? status : nullptr);
     const unsigned char* src = cache + (id * L + l) * slab_bytes;
     unsigned char* dst = out + ((long long)l * B + b) * slab_bytes;
     long long t = (long long)blockIdx.y * blockDim.x + threadIdx.x, step = (long long)gridDim.y * blockDim.x;

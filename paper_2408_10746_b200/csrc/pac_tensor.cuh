@@ -498,7 +498,7 @@ struct BwdParams {
     int r_blocks;                          // ceil(r / 64)
     int stages;
     int tmem_cols;
-    int early_ids;                         // 1: no kernel ahead of this one in the stream writes the ids
+    int early_ids;                         // 1: no kernel ahead of this one in the stream writes the ids (arguments, or in memory)
     // du_l is not read but built in shared memory from one byte per element (see MidParams in pac_mid.cuh) and da_L, one vector per
     // sample or token, in two bf16 terms: B = open_l ? da : 0, out = h_l^T B without the layer's factor.
     const uint8_t* tc;                     // [max_rows][r]
@@ -524,7 +524,7 @@ struct BwdParams {
 // ---------------------------------------------------------------------------
 template <int GQ>
 __global__ void __launch_bounds__(DW_THREADS) __maxnreg__(GQ <= 1 ? 88 : 168)
-dw_down_tc_kernel(const __grid_constant__ CUtensorMap map_cache, BwdParams p) {
+dw_down_tc_kernel(const __grid_constant__ CUtensorMap map_cache, BwdParams p, const __grid_constant__ ArgIds arg) {
     constexpr bool RING = GQ > 1;                                 // gate bytes through the stage ring, else straight into registers
     constexpr int GT = 2;                                         // terms of a du tile
     extern __shared__ unsigned char smem_raw[];
@@ -565,6 +565,7 @@ dw_down_tc_kernel(const __grid_constant__ CUtensorMap map_cache, BwdParams p) {
     volatile int* abort_flag = &abort_sh;
     // The cache never changes: with ids that were final before this launch the h tiles of the first ring are
     // requested while the predecessor still runs; only du (its result) has to wait.
+    const auto sample = [&](int b) { return arg.n > 0 ? arg.v[b] : (int)safe_id(p.ids, b, p.N, nullptr); };
     uint32_t pre = 0;
     if (p.early_ids && warp == 0 && rt1 > rt0) {
         pre = (uint32_t)min(rt1 - rt0, p.stages);
@@ -572,7 +573,7 @@ dw_down_tc_kernel(const __grid_constant__ CUtensorMap map_cache, BwdParams p) {
             const uint64_t pol = l2_policy_evict_first();
             for (uint32_t i = 0; i < pre; ++i) {
                 const int rt = rt0 + (int)i, sc = rt % p.s_chunks, b = rt / p.s_chunks;
-                const int id = (int)safe_id(p.ids, b, p.N, nullptr);
+                const int id = sample(b);
                 const uint32_t dst = smem_u32(smem + (size_t)i * stage_bytes);
                 mbar_expect_tx(full0 + 8 * i, a_bytes);
                 for (int q = 0; q < 2 * p.chunks; ++q)
@@ -594,7 +595,7 @@ dw_down_tc_kernel(const __grid_constant__ CUtensorMap map_cache, BwdParams p) {
         const uint32_t ring0 = smem_u32(smem);
         uint32_t dst = ring0;
         int sc = rt0 % p.s_chunks, b = rt0 / p.s_chunks;
-        int id = rt1 > rt0 ? (int)safe_id(p.ids, b, p.N, nullptr) : 0;
+        int id = rt1 > rt0 ? sample(b) : 0;
         // the gate bytes of a stage's tokens: consecutive rows of r bytes (those beyond the sample are not read)
         auto load_gates = [&] {
             const uint32_t bytes = (uint32_t)(min(BWD_KR, p.S - sc * BWD_KR) * p.r);
@@ -621,7 +622,7 @@ dw_down_tc_kernel(const __grid_constant__ CUtensorMap map_cache, BwdParams p) {
             if (++s == (uint32_t)p.stages) { s = 0; eph ^= 1u; dst = ring0; }
             if (++sc == p.s_chunks) {
                 sc = 0; ++b;
-                if (rt + 1 < rt1) id = (int)safe_id(p.ids, b, p.N, nullptr);
+                if (rt + 1 < rt1) id = sample(b);
             }
         }
     } else if (warp == 1) {
@@ -985,10 +986,10 @@ struct DuGen { const uint8_t* tc; const bf16* da; long long da_term, da_sample; 
 
 // The sums of the row splits stay in `part` ([J][L][d][r]) for the caller's own reduction.
 inline pac_status tensor_dw_down(TensorPlan& tp, cudaStream_t stream, const int* d_ids, int B, const DuGen& gen, float* part, unsigned* status,
-                                 long long* launches, unsigned long long* stamp = nullptr, bool early_ids = false) {
+                                 long long* launches, unsigned long long* stamp, bool early_ids, const ArgIds& arg) {
     BwdParams p = tp.bp;
     p.tc = gen.tc; p.da = gen.da; p.da_term = gen.da_term; p.da_sample = gen.da_sample; p.da_token = gen.da_token;
-    p.ids = d_ids; p.B = B; p.status = status; p.stamp = stamp; p.early_ids = early_ids ? 1 : 0;
+    p.ids = d_ids; p.B = B; p.status = status; p.stamp = stamp; p.early_ids = early_ids || arg.n > 0 ? 1 : 0;
     const int J = tensor_splits(tp, B);
     p.splits = J;
     p.out = part;
@@ -999,7 +1000,7 @@ inline pac_status tensor_dw_down(TensorPlan& tp, cudaStream_t stream, const int*
     const auto kernel = p.r <= 64 ? dw_down_tc_kernel<1> : p.r <= 128 ? dw_down_tc_kernel<2> : dw_down_tc_kernel<4>;
     cudaError_t e = smem_opt_in((const void*)kernel, tp.smem_bwd);
     if (e != cudaSuccess) { tensor_err() = cudaGetErrorString(e); return PAC_ERR_CUDA; }
-    e = cudaLaunchKernelEx(&cfg, kernel, tp.map_cache_bwd, p);
+    e = cudaLaunchKernelEx(&cfg, kernel, tp.map_cache_bwd, p, arg);
     (*launches)++;
     if (e != cudaSuccess) { tensor_err() = cudaGetErrorString(e); return PAC_ERR_CUDA; }
     return PAC_OK;
