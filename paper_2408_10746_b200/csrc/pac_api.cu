@@ -1525,9 +1525,9 @@ pac_status pac_adapter_init(pac_ctx* c, const pac_adapter_cfg* cfg, unsigned lon
         for (int b = 1; b <= cfg->max_batch && ne % 4 == 0; ++b) c->dw_simt_max = std::max(c->dw_simt_max, xg_slices(dw_simt_tiles(dm), b * dm.S, c->sms, 8));
         if (c->dw_simt_max > 1) A(dmalloc(c, &s.dw_spart, ne * c->dw_simt_max));
         if (dm.d > 4 * XG_K) {              // (fewer stages are never shared)
-            A(dmalloc(c, &s.xg_ws, (long long)c->sms * XG_TILE * xg_tile_j(dm.r)));
-            A(dmalloc(c, &s.xg_cnt, c->sms));
-            if (st == PAC_OK) CU_OK(c, cudaMemsetAsync(s.xg_cnt, 0, sizeof(unsigned) * c->sms, c->stream));
+            A(dmalloc(c, &s.xg_ws, 2LL * c->sms * XG_TILE * xg_tile_j(dm.r)));
+            A(dmalloc(c, &s.xg_cnt, 2 * c->sms));
+            if (st == PAC_OK) CU_OK(c, cudaMemsetAsync(s.xg_cnt, 0, sizeof(unsigned) * 2 * c->sms, c->stream));
         }
     }
     if (st == PAC_OK && c->tb.on) {

@@ -8,9 +8,10 @@
 // of relative size 2^-16 and above are formed, six or three; the dropped ones, below 2^-25, are smaller than the rounding of one fp32
 // multiplication.  Sums are fp32, in several accumulators (xg_accs).  That is 1365 products per clock and SM against 128 on the FP32 pipe, so the kernel is bound
 // by bringing the operands in: A comes straight from the activation cache (the gather is the address; any row length and alignment),
-// 16 producer warps fetch it into registers, split it and store the swizzled tiles, one warp issues the MMAs.  The producers work in two
-// teams, each filling one of two stages: a team's loads are in flight while the other converts.
-// At 2048 rows, 12 layers, d = 768, r = 64: u 41 us, dW_down 30 us (the FP32-pipe tiles before it, 8 x 4 outputs per thread: 77 and 84 us).
+// producer warps fetch it into registers, split it and store the swizzled tiles, one warp issues the MMAs.  Two teams of eight producers take turns, each with
+// a stage of its own, so that a team's loads are in flight while the other converts: in one CTA, or in two CTAs of one team each on an SM, whose starts
+// and ends then fall under each other's stages (rows of more than one wave: 2048 x 768 x 64 x 12 layers, 192 tiles: 38 -> 35 us, on a bf16 cache 34 -> 27).
+// At 2048 rows, 12 layers, d = 768, r = 64: u 35 us, dW_down 30 us (the FP32-pipe tiles before it, 8 x 4 outputs per thread: 77 and 84 us).
 // Loads are what it waits for (a third of the issue slots are used); row addresses are therefore formed once per stage (tn) or once per kernel
 // (rows).  Prefetching the stage after next into L2 made the step 8 % slower.
 // Every output is summed in a fixed order.
@@ -39,7 +40,8 @@ struct XgRows {
     __device__ const float* row(int z, int m) const { return base + z * zstride + (long long)m * ld; }
 };
 
-constexpr int XG_PRODUCERS = 16, XG_THREADS = 32 * (XG_PRODUCERS + 1), XG_TILE = 128, XG_K = 64, XG_MAX_JOBS = 6;
+constexpr int XG_TEAM = 8, XG_TILE = 128, XG_K = 64, XG_MAX_JOBS = 6;
+__host__ __device__ constexpr int xg_threads(int teams) { return 32 * (teams * XG_TEAM + 1); }
 constexpr uint32_t XG_TERM_A = XG_TILE * XG_K * 2, XG_BOX = 64 * 128;
 
 // Products of one launch: several per layer (tn), all layers.
@@ -113,15 +115,15 @@ inline int xg_accs(int tile_j, int k_steps) {      // beside that of the smaller
 }
 __host__ __device__ inline uint32_t xg_term_b(int tile_j) { return (uint32_t)((tile_j + 63) / 64) * XG_BOX; }
 template <class AL>
-inline size_t xg_smem(int tile_j) { return 2 * ((size_t)XgTerms<typename AL::elem>::n * XG_TERM_A + 3 * xg_term_b(tile_j)) + 1024; }
+inline size_t xg_smem(int tile_j, int teams) { return teams * ((size_t)XgTerms<typename AL::elem>::n * XG_TERM_A + 3 * xg_term_b(tile_j)) + 1024; }
 
 // Outputs (i, j0 + c) for a warp's columns c of a tile, recomputed in fp32 where the sum of split products is not finite: an infinite operand,
 // or a finite one beyond the largest bf16, has a first term of infinity and no second one, and a partial sum may overflow on the way.
 // dst: the thread's row of sums, `step` apart.
 template <bool TN, class AL>
-__device__ __noinline__ void xg_redo(const AL& A, const XgRows& B, int z, int i, int j0, int c0, int nj_tile, int Nj, int kb, int ke, float* dst, long long step) {
+__device__ __noinline__ void xg_redo(const AL& A, const XgRows& B, int z, int i, int j0, int c0, int c_step, int nj_tile, int Nj, int kb, int ke, float* dst, long long step) {
 #pragma unroll 1
-    for (; c0 < nj_tile; c0 += 64)
+    for (; c0 < nj_tile; c0 += c_step)
 #pragma unroll 1
         for (int c = c0; c < c0 + 16 && j0 + c < Nj; ++c) {
             if (fabsf(dst[c * step]) <= 3.402823466e38f) continue;
@@ -143,11 +145,11 @@ struct XgTail { int whole, parts; float* ws; unsigned* cnt; };
 // tn: grid (tiles of all jobs, layers, slices of the reduction); rows: (whole + parts * the other tiles).
 // tn with more than one slice: the partial sums of slice s go to
 // out + s * part_stride and are added up in slice order by whoever reads them.  GB: 8-column groups of B per thread (tile_j = 32 GB at most).
-template <bool TN, int GB, class AL>
-__global__ void __launch_bounds__(XG_THREADS, 1)
+template <bool TN, int GB, int TEAMS, class AL>
+__global__ void __launch_bounds__(xg_threads(TEAMS), TEAMS == 1 ? 2 : 1)
 xgemm_kernel(const __grid_constant__ XgJobs<AL> J, int K, int k_slice, int accs_most, float* __restrict__ out, long long zstride, long long part_stride, XgTail tail, unsigned* status) {
     typedef typename AL::elem T;
-    constexpr int TA = XgTerms<T>::n;
+    constexpr int TA = XgTerms<T>::n, PRODUCERS = TEAMS * XG_TEAM, THREADS = xg_threads(TEAMS);
     extern __shared__ unsigned char smem_raw[];
     const uint32_t ring = (smem_u32(smem_raw) + 1023u) & ~1023u;
     const int nj_tile = J.tile_j;
@@ -177,14 +179,14 @@ xgemm_kernel(const __grid_constant__ XgJobs<AL> J, int K, int k_slice, int accs_
     const int kb = split * k_slice, ke = !TN && shared_tile < 0 ? K : min(K, kb + k_slice), stages = ke > kb ? (ke - kb + XG_K - 1) / XG_K : 0;
     if (threadIdx.x == 0) {
         abort_sh = 0;
-        for (int s = 0; s < 2; ++s) { mbar_init(full0 + 8 * s, XG_PRODUCERS / 2); mbar_init(empty0 + 8 * s, 1); }
+        for (int s = 0; s < TEAMS; ++s) { mbar_init(full0 + 8 * s, XG_TEAM); mbar_init(empty0 + 8 * s, 1); }
         mbar_init(accf, 1);
         fence_mbar_init();
     }
     const int accs = min(accs_most, max(1, stages * (XG_K / 16)));      // (a short last slice)
     uint32_t tmem_cols = 32;
     while (tmem_cols < (uint32_t)((accs + 1) * nj_tile)) tmem_cols *= 2;
-    if (warp == XG_PRODUCERS) { tmem_alloc(smem_u32(&tmem_base_sh), tmem_cols); tmem_relinquish(); }
+    if (warp == PRODUCERS) { tmem_alloc(smem_u32(&tmem_base_sh), tmem_cols); tmem_relinquish(); }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -192,7 +194,7 @@ xgemm_kernel(const __grid_constant__ XgJobs<AL> J, int K, int k_slice, int accs_
     volatile int* abort_flag = &abort_sh;
     pdl_wait();
     pdl_trigger();      // (not before: a successor may rely on everything ahead of this kernel being complete when it starts)
-    if (warp == XG_PRODUCERS) {
+    if (warp == PRODUCERS) {
         const uint32_t idesc = instr_desc_bf16(XG_TILE, nj_tile, TN ? 1 : 0, 1);
         // (term of A, term of B), the product of the first terms last
         constexpr int NP = TA == 3 ? 6 : 3;
@@ -200,8 +202,8 @@ xgemm_kernel(const __grid_constant__ XgJobs<AL> J, int K, int k_slice, int accs_
         bool ok = true;
         int turn = 0;                               // accumulator of the stage's first product of first terms
         for (int it = 0; it < stages && ok; ++it) {
-            const uint32_t s = it & 1u;
-            if (!mbar_wait_uniform(full0 + 8 * s, (it >> 1) & 1u, abort_flag, status)) { ok = false; break; }
+            const uint32_t s = TEAMS == 1 ? 0u : it & 1u;
+            if (!mbar_wait_uniform(full0 + 8 * s, (TEAMS == 1 ? it : it >> 1) & 1u, abort_flag, status)) { ok = false; break; }
             tc_fence_after();
             if (elect_one()) {
                 const uint32_t a = ring + s * stage, b = a + TA * XG_TERM_A;
@@ -224,7 +226,7 @@ xgemm_kernel(const __grid_constant__ XgJobs<AL> J, int K, int k_slice, int accs_
             for (turn += XG_K / 16; turn >= accs;) turn -= accs;
         }
     } else {
-        const int team = warp >> 3, t = threadIdx.x & 255;
+        const int team = TEAMS == 1 ? 0 : warp >> 3, t = threadIdx.x & 255;
         const AL A = J.A[jb];
         const XgRows B = J.B[jb];
         typename XgTerms<T>::reg ra[4];
@@ -244,7 +246,7 @@ xgemm_kernel(const __grid_constant__ XgJobs<AL> J, int K, int k_slice, int accs_
             offa[i] = (uint32_t)(c8 >> 3) * XG_BOX + (uint32_t)row * 128u + (uint32_t)(((c8 & 7) ^ (row & 7)) << 4);
             if (!TN) pa[i] = i0 + row < Mi ? A.row(z, i0 + row) : nullptr;
         }
-        const long long step_b = 2LL * XG_K * B.ld;
+        const long long step_b = (long long)TEAMS * XG_K * B.ld;
 #pragma unroll
         for (int i = 0; i < GB; ++i) {
             const int g = t + 256 * i;
@@ -275,8 +277,8 @@ xgemm_kernel(const __grid_constant__ XgJobs<AL> J, int K, int k_slice, int accs_
         };
         bool ok = true;
         if (team < stages) fetch(kb + team * XG_K);
-        for (int it = team; it < stages; it += 2) {
-            if (!mbar_wait_uniform(empty0 + 8 * team, ((it >> 1) & 1u) ^ 1u, abort_flag, status)) { ok = false; break; }
+        for (int it = team; it < stages; it += TEAMS) {
+            if (!mbar_wait_uniform(empty0 + 8 * team, ((TEAMS == 1 ? it : it >> 1) & 1u) ^ 1u, abort_flag, status)) { ok = false; break; }
             const uint32_t a = ring + team * stage, b = a + TA * XG_TERM_A;
 #pragma unroll
             for (int i = 0; i < 4; ++i) xg_store(a + offa[i], XG_TERM_A, ra[i]);
@@ -286,7 +288,7 @@ xgemm_kernel(const __grid_constant__ XgJobs<AL> J, int K, int k_slice, int accs_
             fence_proxy_async();
             __syncwarp();
             if (lane == 0) mbar_arrive(full0 + 8 * team);
-            if (it + 2 < stages) fetch(kb + (it + 2) * XG_K);
+            if (it + TEAMS < stages) fetch(kb + (it + TEAMS) * XG_K);
         }
         if (stages > 0) {
             ok = ok && mbar_wait_warp(accf, 0, abort_flag, status);
@@ -298,7 +300,7 @@ xgemm_kernel(const __grid_constant__ XgJobs<AL> J, int K, int k_slice, int accs_
             float* ws = tail.ws + ((long long)(shared_tile * tail.parts + split) * XG_TILE + q * 32 + lane) * nj_tile;
             const bool vec = !J.trans && (Nj & 3) == 0 && ((uintptr_t)o & 15) == 0;
             float odd = 0.f;                             // not zero once an element is not finite
-            for (int c0 = (warp >> 2) * 16; c0 < nj_tile; c0 += 64) {
+            for (int c0 = (warp >> 2) * 16; c0 < nj_tile; c0 += 32 * TEAMS) {
                 float v[16] = {};
                 if (stages > 0) {
                     const uint32_t at = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)c0;
@@ -338,7 +340,7 @@ xgemm_kernel(const __grid_constant__ XgJobs<AL> J, int K, int k_slice, int accs_
             }
             if (!(odd == 0.f) && i < Mi) {
                 const bool part = !TN && shared_tile >= 0;
-                xg_redo<TN>(J.A[jb], J.B[jb], z, i, j0, (warp >> 2) * 16, nj_tile, Nj, kb, ke, part ? ws : J.trans ? o + (long long)j0 * Mi + i : o + (long long)i * Nj + j0, J.trans ? Mi : 1);
+                xg_redo<TN>(J.A[jb], J.B[jb], z, i, j0, (warp >> 2) * 16, 32 * TEAMS, nj_tile, Nj, kb, ke, part ? ws : J.trans ? o + (long long)j0 * Mi + i : o + (long long)i * Nj + j0, J.trans ? Mi : 1);
             }
         }
     }
@@ -355,7 +357,7 @@ xgemm_kernel(const __grid_constant__ XgJobs<AL> J, int K, int k_slice, int accs_
         if (last) {
             const float* ws = tail.ws + (long long)shared_tile * tail.parts * XG_TILE * nj_tile;
             float* o = out + z * zstride + J.out_off[jb];
-            for (int e = threadIdx.x * 4; e < XG_TILE * nj_tile; e += XG_THREADS * 4) {
+            for (int e = threadIdx.x * 4; e < XG_TILE * nj_tile; e += THREADS * 4) {
                 float4 a = __ldcg(reinterpret_cast<const float4*>(ws + e));
                 for (int k = 1; k < tail.parts; ++k) {
                     const float4 b = __ldcg(reinterpret_cast<const float4*>(ws + (long long)k * XG_TILE * nj_tile + e));
@@ -371,18 +373,18 @@ xgemm_kernel(const __grid_constant__ XgJobs<AL> J, int K, int k_slice, int accs_
     tc_fence_before();
     __syncthreads();
     drain_after_abort(abort_flag);
-    if (warp == XG_PRODUCERS) tmem_dealloc(tmem_base, tmem_cols);
+    if (warp == PRODUCERS) tmem_dealloc(tmem_base, tmem_cols);
 }
 
-template <bool TN, class AL>
+template <bool TN, int TEAMS, class AL>
 inline cudaError_t xgemm_launch(const XgJobs<AL>& J, int K, dim3 grid, int k_slice, float* out, long long zstride, long long part_stride, const XgTail& tail, unsigned* status, cudaStream_t stream) {
-    const auto kernel = J.tile_j <= 64 ? xgemm_kernel<TN, 2, AL> : xgemm_kernel<TN, 4, AL>;
-    const size_t smem = xg_smem<AL>(J.tile_j);
+    const auto kernel = J.tile_j <= 64 ? xgemm_kernel<TN, 2, TEAMS, AL> : xgemm_kernel<TN, 4, TEAMS, AL>;
+    const size_t smem = xg_smem<AL>(J.tile_j, TEAMS);
     cudaError_t e = smem_opt_in((const void*)kernel, smem);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[1];
-    pdl_launch_config(&cfg, attr, grid, dim3(XG_THREADS), smem, stream);
+    pdl_launch_config(&cfg, attr, grid, dim3(xg_threads(TEAMS)), smem, stream);
     const int longest = !TN && tail.whole > 0 ? K : K < k_slice ? K : k_slice;      // a CTA's share of the reduction
     const int accs = xg_accs(J.tile_j, (longest + XG_K - 1) / XG_K * (XG_K / 16));
     return cudaLaunchKernelEx(&cfg, kernel, J, K, k_slice, accs, out, zstride, part_stride, tail, status);
@@ -390,20 +392,24 @@ inline cudaError_t xgemm_launch(const XgJobs<AL>& J, int K, dim3 grid, int k_sli
 template <class AL>
 inline cudaError_t xgemm_launch_tn(const XgJobs<AL>& J, int K, int Z, int slices, float* out, long long zstride, long long part_stride, unsigned* status, cudaStream_t stream) {
     const int k_slice = ((K + slices - 1) / slices + XG_K - 1) / XG_K * XG_K;
-    return xgemm_launch<true>(J, K, dim3((unsigned)J.first[J.n], (unsigned)Z, (unsigned)slices), k_slice, out, zstride, part_stride, XgTail{}, status, stream);
+    return xgemm_launch<true, 2>(J, K, dim3((unsigned)J.first[J.n], (unsigned)Z, (unsigned)slices), k_slice, out, zstride, part_stride, XgTail{}, status, stream);
 }
-// ws: sms tiles of 128 x tile_j floats, cnt: sms words of zero.  A tile of the last wave is shared when that takes four or more stages off its CTA
+// ws: 2 sms tiles of 128 x tile_j floats, cnt: 2 sms words of zero.  A tile of the last wave is shared when that takes four or more stages off its CTA
 // (the exchange costs about as much as three).
 template <class AL>
 inline cudaError_t xgemm_launch_rows(const XgJobs<AL>& J, int K, int Z, int sms, float* out, long long zstride, float* ws, unsigned* cnt, unsigned* status, cudaStream_t stream) {
-    const int total = J.first[J.n] * Z, stages = (K + XG_K - 1) / XG_K, rest = total % sms;
+    const int total = J.first[J.n] * Z, stages = (K + XG_K - 1) / XG_K;
+    const bool one = total > sms && xg_accs(J.tile_j, stages * (XG_K / 16)) * J.tile_j + J.tile_j <= 256;
+    if (one) sms *= 2;                              // CTAs at a time (their accumulators have to fit beside each other)
+    const int rest = total % sms;
     XgTail tail{total, 1, ws, cnt};
     int per = stages;
     if (rest > 0) {
         per = (stages + sms / rest - 1) / (sms / rest);
         if (stages - per >= 4) { tail.whole = total - rest; tail.parts = (stages + per - 1) / per; }
     }
-    return xgemm_launch<false>(J, K, dim3((unsigned)(tail.whole + (total - tail.whole) * tail.parts)), per * XG_K, out, zstride, 0, tail, status, stream);
+    const dim3 grid((unsigned)(tail.whole + (total - tail.whole) * tail.parts));
+    return one ? xgemm_launch<false, 1>(J, K, grid, per * XG_K, out, zstride, 0, tail, status, stream) : xgemm_launch<false, 2>(J, K, grid, per * XG_K, out, zstride, 0, tail, status, stream);
 }
 
 // Columns per tile for an output N wide, tiles of equal width.
