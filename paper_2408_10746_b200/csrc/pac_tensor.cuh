@@ -14,6 +14,7 @@
 // ST_TIMEOUT in the context's status words, stops issuing work, releases its TMEM and
 // returns, so a broken pipeline shows up as PAC_ERR_TIMEOUT instead of a hang.
 #pragma once
+#include <algorithm>
 #include <cuda.h>
 #include <cmath>
 
@@ -517,8 +518,8 @@ struct BwdParams {
 // L * M * r * 2 bytes of du out of memory in both directions; the tile costs five integer instructions per four elements.
 // Gate bytes: a builder that loads them itself runs at two stages per memory latency (1.1 us a stage).  At two and more groups per thread, whose
 // registers allow no deeper look-ahead, they therefore come through the stage ring with the h tile (S = 256, B = 64, L = 24, d = 1024, r = 128:
-// 187 -> 154 us, the rate of the memory, with da in one term; 196 with two, where the products and not the loads pace a stage: a deeper ring for h with
-// the du tiles apart, or da held in registers over a sample, changed nothing).  With one group the ring was slower by 0.7 us: short loops, and one more hop before the first product.
+// 187 -> 154 us, the rate of the memory, with da in one term; 196 with two, where the products and not the loads pace a stage; dw_down_gates_kernel needs
+// no second term).  With one group the ring was slower by 0.7 us: short loops, and one more hop before the first product.
 // GQ: 16-column groups of a du tile per thread (r = 64 GQ at most).  Registers are
 // bounded so that three finalisation blocks fit beside a CTA (r <= 64; with 155 instead of 88 the step took 58 us for 53).
 // ---------------------------------------------------------------------------
@@ -779,6 +780,201 @@ dw_down_tc_kernel(const __grid_constant__ CUtensorMap map_cache, BwdParams p, co
     if (warp == 1) tmem_dealloc(tmem_base, (uint32_t)p.tmem_cols);
 }
 
+// The same for classifier heads and 64 < r <= 128, where da_L is one vector per sample: the product is formed with the gates alone, as ones and zeros, one sample at
+// a time, and a sample's sums are multiplied with its da_L in fp32 and added up in registers.  One term instead of two: half the products
+// (at r = 128 two terms are 206 GFLOP per step of S = 256, B = 64, L = 24, d = 1024 and paced the kernel), and operands without rounding.
+// Sixteen worker warps build the gate tiles (16 elements per thread and stage) and own 32 rows x 64 columns of the sums each.  Order of a worker: the tiles of
+// sample i, then the sums of sample i - 1, whose products run meanwhile; products of sample i + 1 go where those of i - 1 were, and their tiles
+// are announced only by workers that have read these, so the full barriers say that, too.
+constexpr int DG_WORKERS = 16, DG_THREADS = 32 * (2 + DG_WORKERS);
+__global__ void __launch_bounds__(DG_THREADS, 1)
+dw_down_gates_kernel(const __grid_constant__ CUtensorMap map_cache, BwdParams p) {
+    extern __shared__ unsigned char smem_raw[];
+    unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    const uint32_t box_bytes = BWD_KR * 128, a_bytes = (uint32_t)p.chunks * 2 * box_bytes, g_off = a_bytes + 2 * box_bytes;      // a stage: h tile, gate tile, gate bytes
+    const uint32_t stage_bytes = g_off + (uint32_t)(BWD_KR * p.r);
+    __shared__ __align__(8) unsigned long long bars[3 * 16 + 2];
+    __shared__ __align__(16) float da_sh[DG_WORKERS][64];
+    __shared__ uint32_t tmem_base_sh;
+    __shared__ int abort_sh;
+    const uint32_t full0 = smem_u32(&bars[0]), empty0 = smem_u32(&bars[16]), gate0 = smem_u32(&bars[32]), accf0 = smem_u32(&bars[48]);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    int item = blockIdx.x;
+    const int j = item % p.splits; item /= p.splits;
+    const int g = item % p.d_groups, l = p.L - 1 - item / p.d_groups;
+    const int row_tiles = p.B * p.s_chunks;
+    const int rt0 = (int)((long long)row_tiles * j / p.splits), rt1 = (int)((long long)row_tiles * (j + 1) / p.splits);
+    const int col0 = g * p.chunks * 128, b0 = rt0 / p.s_chunks;
+    if (threadIdx.x == 0) {
+        abort_sh = 0;
+        for (int s = 0; s < p.stages; ++s) { mbar_init(full0 + 8 * s, 1 + DG_WORKERS); mbar_init(empty0 + 8 * s, 1); mbar_init(gate0 + 8 * s, 1); }
+        mbar_init(accf0, 1); mbar_init(accf0 + 8, 1);
+        fence_mbar_init();
+        tma_prefetch_desc(&map_cache);
+    }
+    if (warp == 1) { tmem_alloc(smem_u32(&tmem_base_sh), 512u); tmem_relinquish(); }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_base = tmem_base_sh;
+    volatile int* abort_flag = &abort_sh;
+    const uint64_t pol = l2_policy_evict_first();
+    const auto load_h = [&](uint32_t dst, uint32_t full, int sc, int id) {
+        mbar_expect_tx(full, a_bytes);
+        for (int q = 0; q < 2 * p.chunks; ++q)
+            tma_load_4d_hint(dst + q * box_bytes, &map_cache, full, col0 + q * 64, sc * BWD_KR, l, id, pol);
+    };
+    // the first ring of h tiles ahead of the wait, as in dw_down_tc_kernel
+    uint32_t pre = 0;
+    if (p.early_ids && warp == 0 && rt1 > rt0) {
+        pre = (uint32_t)min(rt1 - rt0, p.stages);
+        if (elect_one())
+            for (uint32_t i = 0; i < pre; ++i) {
+                const int rt = rt0 + (int)i, b = rt / p.s_chunks;
+                load_h(smem_u32(smem) + i * stage_bytes, full0 + 8 * i, rt - b * p.s_chunks, (int)safe_id(p.ids, b, p.N, nullptr));
+            }
+        __syncwarp();
+    }
+    pdl_wait();
+    pdl_trigger();
+    if (warp == 0) {
+        if (lane == 0 && rt1 > rt0) stamp_begin(p.stamp);
+        uint32_t s = 0, eph = 1;
+        const uint32_t ring0 = smem_u32(smem);
+        uint32_t dst = ring0;
+        int b = b0, sc = rt0 - b0 * p.s_chunks;
+        int id = rt1 > rt0 ? (int)safe_id(p.ids, b, p.N, nullptr) : 0;
+        for (int rt = rt0; rt < rt1; ++rt) {
+            if (pre == 0 && !mbar_wait_uniform(empty0 + 8 * s, eph, abort_flag, p.status)) break;
+            if (elect_one()) {
+                const uint32_t bytes = (uint32_t)(min(BWD_KR, p.S - sc * BWD_KR) * p.r);
+                mbar_expect_tx(gate0 + 8 * s, bytes);
+                bulk_load_1d(dst + g_off, p.tc + ((long long)b * p.S + sc * BWD_KR) * p.r, bytes, gate0 + 8 * s);
+                if (pre == 0) load_h(dst, full0 + 8 * s, sc, id);
+            }
+            if (pre > 0) --pre;
+            __syncwarp();
+            dst += stage_bytes;
+            if (++s == (uint32_t)p.stages) { s = 0; eph ^= 1u; dst = ring0; }
+            if (++sc == p.s_chunks) {
+                sc = 0; ++b;
+                if (rt + 1 < rt1) id = (int)safe_id(p.ids, b, p.N, nullptr);
+            }
+        }
+    } else if (warp == 1) {
+        const uint32_t idesc = instr_desc_bf16(128, p.r, 1, 1);
+        const uint32_t ring0 = smem_u32(smem);
+        const uint64_t a_desc0 = smem_desc_sw128(ring0, box_bytes, 1024), b_desc0 = smem_desc_sw128(ring0 + a_bytes, box_bytes, 1024);
+        const uint64_t desc_step = (uint64_t)(stage_bytes >> 4), a_chunk = (uint64_t)((2 * box_bytes) >> 4);
+        uint64_t doff = 0;
+        uint32_t s = 0, ph = 0, buf = 0, first = 0;
+        int sc = rt0 - b0 * p.s_chunks;
+        for (int rt = rt0; rt < rt1; ++rt) {
+            if (!mbar_wait_uniform(full0 + 8 * s, ph, abort_flag, p.status)) break;
+            tc_fence_after();
+            const bool ends = ++sc == p.s_chunks || rt + 1 == rt1;       // of a sample
+            if (elect_one()) {
+#pragma unroll
+                for (int k = 0; k < BWD_KR / 16; ++k)
+                    for (int c = 0; c < p.chunks; ++c)
+                        umma_bf16(tmem_base + buf * 256u + (uint32_t)c * 128u, a_desc0 + doff + (uint64_t)c * a_chunk + (uint64_t)(k * 128),
+                                  b_desc0 + doff + (uint64_t)(k * 128), idesc, (first | (uint32_t)k) ? 1u : 0u);
+                umma_commit(empty0 + 8 * s);
+                if (ends) umma_commit(accf0 + 8 * buf);
+            }
+            __syncwarp();
+            first = 1;
+            if (ends) { sc = 0; first = 0; buf ^= 1u; }
+            doff += desc_step;
+            if (++s == (uint32_t)p.stages) { s = 0; ph ^= 1u; doff = 0; }
+        }
+    } else {
+        const int q = warp & 3, w = (warp - 2) >> 2, c = w >> 1, n0 = (w & 1) * 64, nc = c < p.chunks ? min(64, p.r - n0) : 0;      // rows and columns of this warp's sums
+        const int g16 = p.r >> 4, t = threadIdx.x - 64, row = t / g16, cg = (t - row * g16) * 16;
+        const bool builds = t < BWD_KR * g16;
+        const uint32_t off = a_bytes + (uint32_t)(cg >> 6) * box_bytes + (uint32_t)row * 128u + (uint32_t)((((cg & 63) >> 3) ^ (row & 7)) << 4);
+        const bool deep = p.L > 127;
+        const uint32_t shut = deep ? 0xffffffffu : 0x7f7f7f7fu, open_bias = (uint32_t)(l | 0x80) * 0x01010101u;
+        float acc[64] = {}, mine[2] = {};                         // mine: da of columns n0 + lane, n0 + lane + 32, of the sample whose sums come next
+        bool ok = true;
+        // sums of the sample in accumulators `seg`, times its da
+        auto add = [&](uint32_t seg) {
+            float* d = da_sh[warp - 2];
+            __syncwarp();
+            d[lane] = mine[0]; d[lane + 32] = mine[1];
+            __syncwarp();
+            if (!mbar_wait_warp(accf0 + 8 * (seg & 1u), (seg >> 1) & 1u, abort_flag, p.status)) { ok = false; return; }
+            tc_fence_after();
+            const uint32_t at = tmem_base + ((uint32_t)(q * 32) << 16) + (seg & 1u) * 256u + (uint32_t)(c * 128 + n0);
+#pragma unroll
+            for (int x = 0; x < 64; x += 16) {
+                if (x < nc) {
+                    float v[16];
+                    tmem_ld16(at + (uint32_t)x, v);
+                    tmem_ld_wait();
+#pragma unroll
+                    for (int e = 0; e < 16; e += 4) {
+                        const float4 f = *reinterpret_cast<const float4*>(d + x + e);
+                        acc[x + e] = fmaf(v[e], f.x, acc[x + e]); acc[x + e + 1] = fmaf(v[e + 1], f.y, acc[x + e + 1]);
+                        acc[x + e + 2] = fmaf(v[e + 2], f.z, acc[x + e + 2]); acc[x + e + 3] = fmaf(v[e + 3], f.w, acc[x + e + 3]);
+                    }
+                }
+            }
+            tc_fence_before();
+        };
+        uint32_t gs = 0, gph = 0, gdst = smem_u32(smem);
+        const uint32_t segs = rt1 > rt0 ? (uint32_t)((rt1 - 1) / p.s_chunks - b0 + 1) : 0u;
+        int rt = rt0, sc = rt0 - b0 * p.s_chunks;
+#pragma unroll 1
+        for (uint32_t seg = 0; seg <= segs && ok; ++seg) {
+            const bf16* da = p.da + (long long)min(b0 + (int)seg, p.B - 1) * p.da_sample + n0;
+            float next[2];
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                const int x = lane + 32 * i;
+                next[i] = n0 + x < p.r ? __bfloat162float(da[x]) + __bfloat162float(da[p.da_term + x]) : 0.f;
+            }
+            for (; sc < p.s_chunks && rt < rt1; ++sc, ++rt) {
+                // (a stage is free before its gates are requested)
+                if (!mbar_wait_uniform(gate0 + 8 * gs, gph, abort_flag, p.status)) { ok = false; break; }
+                if (builds) {
+                    uint4 x = make_uint4(shut, shut, shut, shut);
+                    if (row < p.S - sc * BWD_KR)
+                        asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(x.x), "=r"(x.y), "=r"(x.z), "=r"(x.w) : "r"(gdst + g_off + t * 16) : "memory");
+                    // open where l + 1 > tc: bit 7 of (l + 128) - tc, byte by byte, spread over the element's two bytes
+                    uint32_t y[4] = {open_bias - x.x, open_bias - x.y, open_bias - x.z, open_bias - x.w};
+                    if (deep) { y[0] = bytes_ge(l, x.x); y[1] = bytes_ge(l, x.y); y[2] = bytes_ge(l, x.z); y[3] = bytes_ge(l, x.w); }
+                    const uint32_t one = 0x3f803f80u, a0 = gdst + off;
+                    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(a0), "r"(spread_sign(y[0], 0x9988u) & one), "r"(spread_sign(y[0], 0xbbaau) & one),
+                                 "r"(spread_sign(y[1], 0x9988u) & one), "r"(spread_sign(y[1], 0xbbaau) & one) : "memory");
+                    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(a0 ^ 16u), "r"(spread_sign(y[2], 0x9988u) & one), "r"(spread_sign(y[2], 0xbbaau) & one),
+                                 "r"(spread_sign(y[3], 0x9988u) & one), "r"(spread_sign(y[3], 0xbbaau) & one) : "memory");
+                }
+                fence_proxy_async();                              // the tile is read by the tensor core
+                __syncwarp();
+                if (lane == 0) mbar_arrive(full0 + 8 * gs);
+                gdst += stage_bytes;
+                if (++gs == (uint32_t)p.stages) { gs = 0; gph ^= 1u; gdst = smem_u32(smem); }
+            }
+            sc = 0;
+            if (seg > 0 && ok) add(seg - 1);
+            mine[0] = next[0]; mine[1] = next[1];
+        }
+        if (threadIdx.x == 64 && ok && rt0 < rt1) stamp_end(p.stamp);
+        const int k = col0 + c * 128 + q * 32 + lane;             // column of h = row of dW_down
+        if (ok && k < p.d) {
+            float* dst = p.out + (((long long)j * p.L + l) * p.d + k) * p.r + n0;
+#pragma unroll
+            for (int x = 0; x < 64; x += 4)
+                if (x < nc) *reinterpret_cast<float4*>(dst + x) = make_float4(acc[x], acc[x + 1], acc[x + 2], acc[x + 3]);
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    drain_after_abort(abort_flag);
+    if (warp == 1) tmem_dealloc(tmem_base, 512u);
+}
+
 // out[i] = sum_j part[j][i] in split order (deterministic), n a multiple of 4.  The gradient blocks behind lambda[L] in the flat vector
 // start on a 16-byte boundary only when L % 4 == 0.
 __global__ void reduce_splits_kernel(const float* __restrict__ part, int splits, long long n, float* __restrict__ out) {
@@ -804,6 +1000,8 @@ struct TensorPlan {
     FwdParams fp{};
     BwdParams bp{};
     size_t smem_fwd = 0, smem_bwd = 0;
+    int max_smem = 0;
+    bool gates = false;            // dW_down by dw_down_gates_kernel where da_L is one vector per sample
     long long dw_elems = 0;
 };
 
@@ -875,11 +1073,14 @@ inline pac_status tensor_plan_create(TensorPlan& tp, int device, const bf16* cac
     if (prop.major != 10) { tensor_err() = "device is not sm_100"; return PAC_ERR_UNSUPPORTED; }
     tp.sms = prop.multiProcessorCount;
     const int max_smem = (int)prop.sharedMemPerBlockOptin;
+    tp.max_smem = max_smem;
     const long long max_rows = (long long)max_batch * dm.S;
     const int r_pad = (dm.r + 15) & ~15;
+    // Three and more 64-token tiles to a sample: the sums of shorter samples are read too often (step at B = 64, L = 24, d = 1024, r = 128, two terms / gates alone:
+    // S = 64 236 / 266 us, 128 325 / 334, 140 369 / 353, 192 393 / 382, 256 489 / 445).
+    tp.gates = dm.r > 64 && dm.r <= 128 && dm.S > 2 * BWD_KR;
     // Terms of da: dlambda, which comes from the same product as dW_down, needs two: against 64 bits it is
-    // off by 1e-3 to 8e-3 with one and by 2e-6 to 2e-5 with two.  Up to r = 64 the second term's products cost nothing beside the stream; at
-    // B = 64, S = 256, L = 24, d = 1024, r = 128 the step takes 465 us for 430.
+    // off by 1e-3 to 8e-3 with one and by 2e-6 to 2e-5 with two.  Up to r = 64 the second term's products cost nothing beside the stream.
     constexpr int dt = 2;
 
     // ---- tensor maps ----
@@ -997,6 +1198,17 @@ inline pac_status tensor_dw_down(TensorPlan& tp, cudaStream_t stream, const int*
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[1];
     pdl_launch_config(&cfg, attr, dim3((unsigned)grid), dim3(DW_THREADS), tp.smem_bwd, stream);
+    if (tp.gates && p.da_token == 0 && arg.n == 0) {
+        const int stage = (p.chunks + 1) * 2 * BWD_KR * 128 + BWD_KR * p.r;
+        p.stages = std::min(16, (tp.max_smem - 8192) / stage);
+        const size_t smem = (size_t)p.stages * stage + 1024;
+        pdl_launch_config(&cfg, attr, dim3((unsigned)grid), dim3(DG_THREADS), smem, stream);
+        cudaError_t e = smem_opt_in((const void*)dw_down_gates_kernel, smem);
+        if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, dw_down_gates_kernel, tp.map_cache_bwd, p);
+        (*launches)++;
+        if (e != cudaSuccess) { tensor_err() = cudaGetErrorString(e); return PAC_ERR_CUDA; }
+        return PAC_OK;
+    }
     const auto kernel = p.r <= 64 ? dw_down_tc_kernel<1> : p.r <= 128 ? dw_down_tc_kernel<2> : dw_down_tc_kernel<4>;
     cudaError_t e = smem_opt_in((const void*)kernel, tp.smem_bwd);
     if (e != cudaSuccess) { tensor_err() = cudaGetErrorString(e); return PAC_ERR_CUDA; }
