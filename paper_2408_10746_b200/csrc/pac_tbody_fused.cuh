@@ -309,9 +309,15 @@ __device__ __forceinline__ void tb_st2(float* p, float x, float y, bool two, boo
 struct TbKeys { float2 x[4][2]; };
 __device__ __forceinline__ void tb_load_keys(TbKeys& o, const float* __restrict__ X, int r, int key0, int S, int k, int cols, bool even) {
     const int lane = threadIdx.x & 31, q = lane >> 2, c2 = 2 * (lane & 3);
+    if (even && key0 + 32 <= S && k + 16 <= cols) {            // nothing to clamp
+        const float* x = X + (key0 + q) * r + k + c2;
+#pragma unroll
+        for (int n = 0; n < 4; ++n, x += 8 * r) { o.x[n][0] = __ldg(reinterpret_cast<const float2*>(x)); o.x[n][1] = __ldg(reinterpret_cast<const float2*>(x) + 4); }
+        return;
+    }
 #pragma unroll
     for (int n = 0; n < 4; ++n) {
-        const float* x = X + (long long)min(key0 + n * 8 + q, S - 1) * r;
+        const float* x = X + min(key0 + n * 8 + q, S - 1) * r;
         o.x[n][0] = tb_ld2(x, k + c2, cols, even); o.x[n][1] = tb_ld2(x, k + c2 + 8, cols, even);
     }
 }
@@ -331,13 +337,15 @@ __device__ __forceinline__ void tb_scores(float (&acc)[4][4], const TbA& a, cons
 struct TbVals { float v[2][2][4]; };
 __device__ __forceinline__ void tb_load_vals(TbVals& o, const float* __restrict__ X, int r, int key0, int S, int n0, int dh) {
     const int lane = threadIdx.x & 31, q = lane >> 2, c2 = 2 * (lane & 3);
+    const bool full = key0 + 32 <= S;
+    const float *x0 = X + min(n0 + q, dh - 1), *x1 = X + min(n0 + 8 + q, dh - 1);
 #pragma unroll
     for (int k = 0; k < 2; ++k)
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            const float* x = X + (long long)min(key0 + 16 * k + c2 + (i & 1) + (i >> 1) * 8, S - 1) * r;
-#pragma unroll
-            for (int n = 0; n < 2; ++n) o.v[k][n][i] = __ldg(x + min(n0 + n * 8 + q, dh - 1));
+            const int j = key0 + 16 * k + c2 + (i & 1) + (i >> 1) * 8, at = (full ? j : min(j, S - 1)) * r;
+            o.v[k][0][i] = __ldg(x0 + at);
+            o.v[k][1][i] = __ldg(x1 + at);
         }
 }
 // acc[n] += weights (16 tokens x 16 rows, zero past the last row) vals, k the k step of the 32 rows.
@@ -430,14 +438,19 @@ __device__ __forceinline__ TbSmem tb_carve(unsigned char* base, size_t ring, con
     s.stat0 = s.vec + tb_vec_floats(p.r, p.f);
     s.stat1 = s.stat0 + TBF_WARPS * TBF_T;
     s.share = s.stat1 + TBF_WARPS * TBF_T;
-    // the padding of the terms is multiplied with zero weights: it has to be finite
-    uint4* z = reinterpret_cast<uint4*>(s.wide);
-    for (int i = threadIdx.x; i < 3 * TBF_T * (p.ka + p.kb) / 8; i += TBF_THREADS) z[i] = make_uint4(0u, 0u, 0u, 0u);
     return s;
 }
-__device__ __forceinline__ void tb_vec_in(float* dst, const float* __restrict__ src, int n) {
-    for (int i = threadIdx.x; i < n; i += TBF_THREADS) dst[i] = __ldg(src + i);
+// The padding of the terms is multiplied with zero weights: it has to be finite.
+__device__ __forceinline__ void tb_zero_terms(const TbSmem& s, const TbLayerParams& p) {
+    uint4* z = reinterpret_cast<uint4*>(s.wide);
+    for (int i = threadIdx.x; i < 3 * TBF_T * (p.ka + p.kb) / 8; i += TBF_THREADS) z[i] = make_uint4(0u, 0u, 0u, 0u);
 }
+// Parameter vectors arrive as asynchronous copies, the oldest group of every thread's ring: tb_vec_wait and a barrier before their first use.
+__device__ __forceinline__ void tb_vec_in(float* dst, const float* __restrict__ src, int n) {
+    for (int i = threadIdx.x; i < n; i += TBF_THREADS) asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(dst + i)), "l"(src + i) : "memory");
+}
+template <int U>
+__device__ __forceinline__ void tb_vec_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(U) : "memory"); }
 // A row's columns lane, lane + 32, ... (zeros past n or where the row is not live).
 template <int NR>
 __device__ __forceinline__ void tb_row_in(float (&v)[NR], const float* __restrict__ row, int n, bool live) {
@@ -457,15 +470,18 @@ __global__ void __launch_bounds__(TBF_THREADS) tb_fwd_kernel(const __grid_consta
     const long long m0 = (long long)b * S + t0;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, q = lane >> 2, c2 = 2 * (lane & 3);
     const int first = p.tail >= 0 ? 0 : 3, last = p.head >= 0 ? 4 : 3;
-    TbStream<U> st(p, tb_sm);
-#pragma unroll 1
-    for (int i = 0; i < U; ++i) st.issue();                     // the packed weights were final before the predecessor started
     const TbSmem sm = tb_carve(tb_sm, (size_t)TBF_WARPS * U * TB_UNIT, p);
+    // (parameters and packed weights were final before the predecessor started)
     if (p.head >= 0) { tb_vec_in(sm.vec, p.g1, r); tb_vec_in(sm.vec + r, p.b1, r); }
     if (p.tail >= 0) {
         tb_vec_in(sm.vec + 2 * r, p.g2, r); tb_vec_in(sm.vec + 3 * r, p.b2, r); tb_vec_in(sm.vec + 4 * r, p.c2, r);
         tb_vec_in(sm.vec + 5 * r, p.c1, f);
     }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    TbStream<U> st(p, tb_sm);
+#pragma unroll 1
+    for (int i = 0; i < U; ++i) st.issue();
+    tb_zero_terms(sm, p);
     const float lm = p.head >= 0 ? __ldg(p.lam + p.head) : 0.f;
     pdl_wait();
     pdl_trigger();
@@ -474,6 +490,7 @@ __global__ void __launch_bounds__(TBF_THREADS) tb_fwd_kernel(const __grid_consta
     float res[NR], un[NR];                                      // residual row of `tail`, u row of `head`
     if (p.tail >= 0) tb_row_in(res, s.x + p.tail * s.sMr + (m0 + warp) * r, r, live);
     if (p.head >= 0) tb_row_in(un, p.u + p.head * p.u_stride + (m0 + warp) * r, r, live);
+    tb_vec_wait<U>();
     __syncthreads();
     if (p.tail >= 0) {
         const float* qkv = s.qkv + 3 * p.tail * s.sMr + (long long)b * S * r;
@@ -708,26 +725,25 @@ __global__ void __launch_bounds__(TBF_THREADS) tb_bwd_kernel(const __grid_consta
     const int hl = warp / p.nc, key0 = (warp - hl * p.nc) * 32, key_step = p.nc * 32;
     const bool live = warp < nt;                                // token `warp` is this warp's row
     const TbStacks& s = p.s;
+    const TbSmem sm = tb_carve(tb_sm, (size_t)TBF_WARPS * U * TB_UNIT, p);
+    if (p.tail >= 0) tb_vec_in(sm.vec, p.g1, r);
+    if (p.head >= 0) tb_vec_in(sm.vec + r, p.g2, r);
+    asm volatile("cp.async.commit_group;" ::: "memory");
     TbStream<U> st(p, tb_sm);
 #pragma unroll 1
     for (int i = 0; i < U; ++i) st.issue();
-    const TbSmem sm = tb_carve(tb_sm, (size_t)TBF_WARPS * U * TB_UNIT, p);
     // What the forward pass left was final before the predecessor started, except for the first launch, whose predecessor triggers nothing.
-    float xh[NR], up[NR], rstd = 0.f;                           // normalised row; u - a_prev
+    float xh[NR], up[NR], ap[NR], rstd = 0.f;                   // normalised row; u, a_prev
     float lm = 0.f;
     if (p.tail >= 0) {
         const int l = p.tail;
-        float ap[NR];
-        tb_vec_in(sm.vec, p.g1, r);
         tb_row_in(xh, s.xhat1 + l * s.sMr + (m0 + warp) * r, r, live);
         tb_row_in(up, p.u + l * p.u_stride + (m0 + warp) * r, r, live);
         tb_row_in(ap, s.a + (l - 1) * p.u_stride + (m0 + warp) * r, r, live && l > 0);
-#pragma unroll
-        for (int i = 0; i < NR; ++i) up[i] -= ap[i];
         rstd = live ? __ldg(s.rstd1 + l * s.sM + m0 + warp) : 0.f;
         lm = __ldg(p.lam + l);
     }
-    if (p.head >= 0) tb_vec_in(sm.vec + r, p.g2, r);
+    tb_zero_terms(sm, p);
     pdl_wait();
     pdl_trigger();
     float res[NR];                                              // gradient past the norm: dx1 of `tail`, then da of `head`
@@ -743,6 +759,7 @@ __global__ void __launch_bounds__(TBF_THREADS) tb_bwd_kernel(const __grid_consta
             open |= (unsigned)((h0.x > 0.f ? 1 : 0) | (h0.y > 0.f ? 2 : 0) | (h1.x > 0.f ? 4 : 0) | (h1.y > 0.f ? 8 : 0)) << (4 * i);
         }
     }
+    tb_vec_wait<U>();
     __syncthreads();
     if (p.tail >= 0) {
         const int l = p.tail;
@@ -769,6 +786,13 @@ __global__ void __launch_bounds__(TBF_THREADS) tb_bwd_kernel(const __grid_consta
                         const int s0 = key0 + w * key_step;
                         float wt[2][8];
                         TbVals x;
+                        if (s0 + 32 <= S && nt == TBF_T) {     // nothing to leave out
+                            const float* w0 = W + (s0 + c2) * S + q;
+#pragma unroll
+                            for (int j = 0; j < 2; ++j)
+#pragma unroll
+                                for (int i = 0; i < 8; ++i) wt[j][i] = __ldg(w0 + (16 * j + (i & 1) + (i >> 2) * 8) * S + ((i >> 1) & 1) * 8);
+                        } else
 #pragma unroll
                         for (int j = 0; j < 2; ++j)
 #pragma unroll
@@ -876,7 +900,7 @@ __global__ void __launch_bounds__(TBF_THREADS) tb_bwd_kernel(const __grid_consta
                 y = res[i] + (dn[i] * g[c] - s1 - xh[i] * s2) * rstd;
                 if (ph) s.dx1[o + c] = y;
                 else {
-                    acc = fmaf(y, up[i], acc);
+                    acc = fmaf(y, up[i] - ap[i], acc);
                     p.du[l * p.u_stride + (m0 + warp) * r + c] = lm * y;
                     y *= 1.f - lm;
                     if (p.head >= 0) s.da[p.head * s.sMr + (m0 + warp) * r + c] = y;
