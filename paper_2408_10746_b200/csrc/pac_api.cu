@@ -2209,16 +2209,17 @@ extern "C" pac_status pac_quantize_absmax(int device, void* cuda_stream, const f
         int lanes_log2 = 0;
         while ((16 << lanes_log2) < block) ++lanes_log2;
         quantize_absmax_subwarp_kernel<<<grid, 256, 0, st>>>(dev_x, n, lanes_log2, dev_q, dev_c);
-    } else if (al16 && block % 1024 == 0 && block <= 4096 && n_blocks <= 0x7fffffffLL) {
+    } else if (al16 && block % 1024 == 0 && block > 1024 && block <= 4096 && n_blocks <= 0x7fffffffLL) {      // (1024: 124 us a CTA per block, 105 a warp, at 2^26 values)
         switch (block / 1024) {
-            case 1: quantize_absmax_cta_reg_kernel<1><<<(unsigned)n_blocks, 256, 0, st>>>(dev_x, n, dev_q, dev_c); break;
             case 2: quantize_absmax_cta_reg_kernel<2><<<(unsigned)n_blocks, 256, 0, st>>>(dev_x, n, dev_q, dev_c); break;
             case 3: quantize_absmax_cta_reg_kernel<3><<<(unsigned)n_blocks, 256, 0, st>>>(dev_x, n, dev_q, dev_c); break;
             default: quantize_absmax_cta_reg_kernel<4><<<(unsigned)n_blocks, 256, 0, st>>>(dev_x, n, dev_q, dev_c); break;
         }
     } else if (al16 && block % 4 == 0 && block <= 1024) {
-        const long long warps = n_blocks < 148LL * 64 ? n_blocks : 148LL * 64;
-        quantize_absmax_warp4_kernel<<<(unsigned)((warps + 7) / 8), 256, 0, st>>>(dev_x, n, block, n_blocks, dev_q, dev_c);
+        const int per = block <= 128 ? 1 : block <= 256 ? 2 : block <= 512 ? 4 : 8;
+        const auto kernel = per == 1 ? quantize_absmax_warp4_kernel<1> : per == 2 ? quantize_absmax_warp4_kernel<2> : per == 4 ? quantize_absmax_warp4_kernel<4> : quantize_absmax_warp4_kernel<8>;
+        const long long want = (n_blocks + 8 / per - 1) / (8 / per), warps = want < 148LL * 64 ? want : 148LL * 64;
+        kernel<<<(unsigned)((warps + 7) / 8), 256, 0, st>>>(dev_x, n, block, n_blocks, dev_q, dev_c);
     } else if (block <= QUANT_WARP_MAX) {
         const long long warps = n_blocks < 148LL * 64 ? n_blocks : 148LL * 64;      // up to 8 CTAs of 8 warps per SM
         quantize_absmax_warp_kernel<<<(unsigned)((warps + 7) / 8), 256, 0, st>>>(dev_x, n, block, n_blocks, dev_q, dev_c);
@@ -2240,6 +2241,14 @@ extern "C" pac_status pac_dequantize_absmax(int device, void* cuda_stream, const
         const long long want = ((n + 15) / 16 + 255) / 256;
         const unsigned grid = (unsigned)(want < 148LL * 32 ? want : 148LL * 32);
         dequantize_absmax_16_kernel<<<grid, 256, 0, (cudaStream_t)cuda_stream>>>(dev_q, dev_c, n, b16, shift, dev_out);
+    } else if (block % 4 == 0 && block >= 16 && n < (1LL << 33) - 64 && ((uintptr_t)dev_q & 15) == 0 && ((uintptr_t)dev_out & 31) == 0) {
+        const uint32_t b4 = (uint32_t)block / 4;
+        int s = 0;
+        while ((1LL << s) < b4) ++s;
+        const uint32_t magic = (uint32_t)(((1ULL << (31 + s)) + b4 - 1) / b4);
+        const long long want = ((n + 15) / 16 + 255) / 256;
+        const unsigned grid = (unsigned)(want < 148LL * 32 ? want : 148LL * 32);
+        dequantize_absmax_16_any_kernel<<<grid, 256, 0, (cudaStream_t)cuda_stream>>>(dev_q, dev_c, n, (n + block - 1) / block, b4, magic, s - 1, dev_out);
     } else if (block % 4 == 0 && ((uintptr_t)dev_q & 3) == 0 && ((uintptr_t)dev_out & 15) == 0) {
         const long long want = (n / 4 + 1023) / 1024;
         const unsigned grid = (unsigned)(want < 148LL * 32 ? (want > 0 ? want : 1) : 148LL * 32);

@@ -70,14 +70,16 @@ __device__ __forceinline__ uint32_t quant_pack4(float a, float b, float c, float
 }
 // 32 bytes in one access (p 32-byte aligned).
 __device__ __forceinline__ void ld_global_32(const float* p, float (&v)[8]) {
-    asm volatile("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+    asm volatile("ld.global.nc.L1::no_allocate.L2::evict_first.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
                  : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7]) : "l"(p));
 }
 __device__ __forceinline__ void st_global_32f(float* p, const float (&v)[8]) {
-    asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
+    asm volatile("st.global.L1::no_allocate.L2::evict_first.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
                  ::"l"(p), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7]) : "memory");
 }
 
+// What is read or written once and larger (values) gives way in L2 to the codes, which the reader of both directions then finds there:
+// 4096 x 11008 values at block 64, both directions 78.6 -> 68.7 us.
 // Block = 16, 32, ... 512: a lane owns 16 consecutive values (two 32-byte loads, one 16-byte store), block / 16 lanes share a block
 // and one division.  Any n: the last group is handled value by value.  Bound by HBM; with one 16-byte load per thread in flight
 // and a division per four values the same blocks took 0.66 of the copy bandwidth.
@@ -115,46 +117,63 @@ __global__ void __launch_bounds__(256) quantize_absmax_subwarp_kernel(const floa
     }
 }
 
-// Block a multiple of 4 up to 1024 (any remainder of n): one warp per block, eight 16-byte loads per lane in flight.
+// Block a multiple of 4 up to 128 PER (any remainder of n): 8 / PER blocks per warp at a time, eight 16-byte loads per lane in flight.
+// (One block at a time left a lane one load for blocks of 100: both directions of 2^26 values 282 us; so 158 with the reader below.)
+template <int PER>
 __global__ void __launch_bounds__(256) quantize_absmax_warp4_kernel(const float* __restrict__ x, long long n, int block, long long n_blocks,
                                                                     signed char* __restrict__ q, float* __restrict__ c) {
+    constexpr int NB = 8 / PER;
     const int lane = threadIdx.x & 31;
     const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
-    for (long long j = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; j < n_blocks; j += nw) {
-        const long long i0 = j * block;
-        const int len = (int)((n - i0) < block ? (n - i0) : block);
-        float4 v[8];
-        float amax = 0.f;
+    for (long long j = (((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * NB; j < n_blocks; j += nw * NB) {
+        float4 v[NB][PER];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            const int e = (k * 32 + lane) * 4;
-            v[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (e + 4 <= len) v[k] = *reinterpret_cast<const float4*>(x + i0 + e);
-            else if (e < len) {
-                v[k].x = x[i0 + e];
-                if (e + 1 < len) v[k].y = x[i0 + e + 1];
-                if (e + 2 < len) v[k].z = x[i0 + e + 2];
+        for (int b = 0; b < NB; ++b) {
+            const long long i0 = (j + b) * block;
+            const int len = (int)(n - i0 < block ? (n - i0 > 0 ? n - i0 : 0) : block);
+#pragma unroll
+            for (int k = 0; k < PER; ++k) {
+                const int e = (k * 32 + lane) * 4;
+                v[b][k] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (e + 4 <= len) v[b][k] = __ldcs(reinterpret_cast<const float4*>(x + i0 + e));
+                else if (e < len) {
+                    v[b][k].x = x[i0 + e];
+                    if (e + 1 < len) v[b][k].y = x[i0 + e + 1];
+                    if (e + 2 < len) v[b][k].z = x[i0 + e + 2];
+                }
             }
         }
+        float amax[NB];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) amax = fmaxf(amax, absmax4(v[k]));
+        for (int b = 0; b < NB; ++b) {
+            amax[b] = 0.f;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
-        const float cj = amax > 0.f ? __fdiv_rn(127.f, amax) : 0.f;
-        if (lane == 0) c[j] = cj;
+            for (int k = 0; k < PER; ++k) amax[b] = fmaxf(amax[b], absmax4(v[b][k]));
+        }
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            const int e = (k * 32 + lane) * 4;
-            if (e >= len) continue;
-            const uint32_t w = quant_pack4(v[k].x, v[k].y, v[k].z, v[k].w, cj);
-            if (e + 4 <= len) *reinterpret_cast<uint32_t*>(q + i0 + e) = w;
-            else
-                for (int b = 0; e + b < len; ++b) q[i0 + e + b] = (signed char)(w >> (8 * b));
+        for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+            for (int b = 0; b < NB; ++b) amax[b] = fmaxf(amax[b], __shfl_xor_sync(0xffffffffu, amax[b], o));
+#pragma unroll
+        for (int b = 0; b < NB; ++b) {
+            const long long i0 = (j + b) * block;
+            const int len = (int)(n - i0 < block ? (n - i0 > 0 ? n - i0 : 0) : block);
+            const float cj = amax[b] > 0.f ? __fdiv_rn(127.f, amax[b]) : 0.f;
+            if (lane == 0 && len > 0) c[j + b] = cj;
+#pragma unroll
+            for (int k = 0; k < PER; ++k) {
+                const int e = (k * 32 + lane) * 4;
+                if (e >= len) continue;
+                const uint32_t w = quant_pack4(v[b][k].x, v[b][k].y, v[b][k].z, v[b][k].w, cj);
+                if (e + 4 <= len) *reinterpret_cast<uint32_t*>(q + i0 + e) = w;
+                else
+                    for (int t = 0; e + t < len; ++t) q[i0 + e + t] = (signed char)(w >> (8 * t));
+            }
         }
     }
 }
 
-// Single pass, one CTA of 256 threads per block, block = 1024 * K (K <= 4), any n.
+// Single pass, one CTA of 256 threads per block, block = 1024 * K (2 <= K <= 4), any n.
 template <int K>
 __global__ void __launch_bounds__(256) quantize_absmax_cta_reg_kernel(const float* __restrict__ x, long long n,
                                                                       signed char* __restrict__ q, float* __restrict__ c) {
@@ -167,7 +186,7 @@ __global__ void __launch_bounds__(256) quantize_absmax_cta_reg_kernel(const floa
     for (int k = 0; k < K; ++k) {
         const long long i = base + (k * 256 + threadIdx.x) * 4;
         v[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (i + 4 <= n) v[k] = *reinterpret_cast<const float4*>(x + i);
+        if (i + 4 <= n) v[k] = __ldcs(reinterpret_cast<const float4*>(x + i));
         else if (i < n) {
             v[k].x = x[i];
             if (i + 1 < n) v[k].y = x[i + 1];
@@ -246,6 +265,29 @@ __global__ void __launch_bounds__(256) dequantize_absmax_16_kernel(const signed 
     }
 }
 
+// The same where sixteen codes may lie in two blocks (block a multiple of 4 from 16 on, n < 2^33): each four codes in one, the first four's found by
+// a multiplication: group index (below 2^31) times ceil(2^(31 + s) / block4), 2^(s - 1) < block4 <= 2^s, shifted right by 31 + s (Granlund and Montgomery, PLDI 1994).
+__global__ void __launch_bounds__(256) dequantize_absmax_16_any_kernel(const signed char* __restrict__ q, const float* __restrict__ c, long long n, long long n_blocks,
+                                                                       uint32_t block4, uint32_t magic, int shift, float* __restrict__ out) {
+    const long long groups = (n + 15) >> 4, stride = (long long)gridDim.x * blockDim.x;
+    for (long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x; g < groups; g += stride) {
+        const long long i = g << 4;
+        const uint32_t i4 = (uint32_t)(g << 2), j = __umulhi(i4, magic) >> shift, edge = (j + 1) * block4;      // edge: first four codes of the next block
+        const float c0 = __ldg(c + j), c1 = i4 + 4 > edge && j + 1 < n_blocks ? __ldg(c + j + 1) : c0;
+        if (i + 16 <= n) {
+            const uint4 w = __ldg(reinterpret_cast<const uint4*>(q + i));
+            const DequantScale s0(c0), s1 = i4 + 4 > edge ? DequantScale(c1) : s0;
+            float a[8], b[8];
+            dequant4(w.x, s0, a);
+            dequant4(w.y, i4 + 1 < edge ? s0 : s1, a + 4); dequant4(w.z, i4 + 2 < edge ? s0 : s1, b); dequant4(w.w, i4 + 3 < edge ? s0 : s1, b + 4);
+            st_global_32f(out + i, a);
+            st_global_32f(out + i + 8, b);
+        } else {
+            for (int e = 0; i + e < n; ++e) out[i + e] = DequantScale(i4 + (e >> 2) < edge ? c0 : c1).slow((float)q[i + e]);
+        }
+    }
+}
+
 // Four codes per thread (block a multiple of 4), four independent groups in flight.  Any n.
 __global__ void __launch_bounds__(256) dequantize_absmax_vec_kernel(const signed char* __restrict__ q, const float* __restrict__ c,
                                                                     long long n, int block4, float* __restrict__ out) {
@@ -265,7 +307,7 @@ __global__ void __launch_bounds__(256) dequantize_absmax_vec_kernel(const signed
             if (i < n4) {
                 float o[4];
                 dequant4(b[k], DequantScale(cj[k]), o);
-                reinterpret_cast<float4*>(out)[i] = make_float4(o[0], o[1], o[2], o[3]);
+                __stcs(reinterpret_cast<float4*>(out) + i, make_float4(o[0], o[1], o[2], o[3]));
             }
         }
     }
