@@ -1125,26 +1125,25 @@ inline pac_status tensor_plan_create(TensorPlan& tp, int device, const bf16* cac
     b.chunks = (dm.d >= 256 && 2 * n_cols <= 512) ? 2 : 1;
     b.d_groups = (dm.d + 128 * b.chunks - 1) / (128 * b.chunks);
     b.tmem_cols = pow2_at_least(b.chunks * n_cols);
+    // Row splits: enough CTAs to fill the SMs in balanced waves, few enough partial sums.  Up to r = 64 a CTA may have an SM to itself or share it with another (half
+    // the stages each): of more than one wave the second then starts and ends under the first (L = 24, d = 1024, B = 32, S = 128: 288 CTAs, step 112.8 -> 109.8 us).
     {
         const int stage = (b.chunks * 2 + b.r_blocks * dt) * BWD_KR * 128 + (dm.r > 64 ? BWD_KR * dm.r : 0);
-        int st = (max_smem - 2048) / stage;
-        if (st > 16) st = 16;
-        if (st < 2) { tensor_err() = "not enough shared memory for the backward pipeline"; return PAC_ERR_UNSUPPORTED; }
-        b.stages = st;
-        tp.smem_bwd = (size_t)st * stage + 1024;
-    }
-    // row splits: enough CTAs to fill the SMs in balanced waves, few enough partial sums
-    {
         const int items = dm.L * b.d_groups;
         const int row_tiles_max = max_batch * b.s_chunks;
-        int best = 1;
         double best_cost = 1e30;
-        for (int J = 1; J <= 8 && J <= row_tiles_max; ++J) {
-            double waves = (double)items * J / tp.sms;
-            double cost = std::ceil(waves) / waves + 0.03 * (J - 1);
-            if (cost < best_cost - 1e-9) { best_cost = cost; best = J; }
+        for (int per_sm = 1; per_sm <= (dm.r <= 64 && b.tmem_cols <= 256 ? 2 : 1); ++per_sm) {
+            const int st = std::min(16, (max_smem / per_sm - 1024 - 1024 * per_sm) / stage);
+            if (st < 2) continue;
+            for (int J = 1; J <= 8 && J <= row_tiles_max; ++J) {
+                if (per_sm == 2 && row_tiles_max > 36 * J) continue;      // long streams gain more from depth (B = 48, 32 tiles: 160 -> 156 us; B = 64, 43 tiles: 193 -> 195)
+                const double waves = (double)items * J / (tp.sms * per_sm);
+                const double cost = std::ceil(waves) / waves + 0.03 * (J - 1) + 0.01 * (std::ceil(waves) - 1);
+                if (cost < best_cost - 1e-9) { best_cost = cost; b.splits = J; b.stages = st; }
+            }
         }
-        b.splits = best;
+        if (best_cost == 1e30) { tensor_err() = "not enough shared memory for the backward pipeline"; return PAC_ERR_UNSUPPORTED; }
+        tp.smem_bwd = (size_t)b.stages * stage + 1024;
     }
     tp.dw_elems = (long long)dm.L * dm.d * dm.r;
     *part_floats = tp.dw_elems * b.splits;
