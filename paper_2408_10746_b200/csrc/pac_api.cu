@@ -423,7 +423,7 @@ pac_status down_projection_simt(pac_ctx* c, const int* d_ids, int B) {
                       c->sc.u, (long long)c->max_rows * dm.r);
 }
 
-pac_status head_matrix_enqueue(pac_ctx* c);
+pac_status head_matrix_enqueue(pac_ctx* c, int B);
 pac_status finalize_enqueue(pac_ctx* c, const int* d_ids, int B, float* d_loss, const pac_adamw* hp);
 pac_status adam_body_enqueue(pac_ctx* c, const pac_adamw* hp);
 
@@ -470,7 +470,7 @@ pac_status forward(pac_ctx* c, const int* d_ids, int B, bool train, float* d_log
     const long long n = (long long)M * dm.r, stride = (long long)c->max_rows * dm.r;
     Scratch& sc = c->sc;
     pac_status st = PAC_OK;
-    if (plain_head_ok(c, B) && (st = head_matrix_enqueue(c)) != PAC_OK) return st;
+    if (plain_head_ok(c, B) && (st = head_matrix_enqueue(c, B)) != PAC_OK) return st;
     st = down_projection(c, d_ids, B);
     if (st != PAC_OK) return st;
     const float* lam = c->params + c->lay.lam;
@@ -791,7 +791,7 @@ pac_status tb_forward(pac_ctx* c, const int* d_ids, int B, bool train, float* d_
         tb_pack_kernel<<<dim3(cdiv(t.pk.tiles(), 8), (unsigned)dm.L), 256, 0, st>>>(c->params + c->lay.body, bl.per_layer, bl, t.pk, reinterpret_cast<unsigned char*>(t.packed));
         LAUNCH_CHECK(c);
     }
-    if (plain_head_ok(c, B)) TB_OK(head_matrix_enqueue(c));
+    if (plain_head_ok(c, B)) TB_OK(head_matrix_enqueue(c, B));
     TB_OK(down_projection(c, d_ids, B));
     const float* lam = c->params + c->lay.lam;
     const unsigned rows_grid = cdiv(M, 8), heads_grid = cdiv((long long)B * t.H * dm.S, 128);
@@ -942,7 +942,11 @@ pac_status down_projection(pac_ctx* c, const int* d_ids, int B) {
 // Whether a step's host ids can be arguments of its kernels: the one-launch forward and the second pass then request their first cache tiles ahead of
 // everything before them in the stream, and no kernel has to store the ids first (T5-Base: evaluation of 27 samples
 // 23.6 -> 22.1 us, a step of 32 with its own update launch 62.0 -> 58.0, with the fused one, whose ids the forward read from host memory before, 55.8 -> 55.0).
-bool arg_ids_ok(const pac_ctx* c, int B) { return !c->hc.on && !c->tb.on && B <= ARG_IDS && use_fused_fwd(c, B); }
+// Other classifier steps begin with head_matrix_kernel, which stores them for the kernels behind it.
+bool arg_ids_ok(const pac_ctx* c, int B) {
+    if (c->hc.on || B > ARG_IDS || c->cfg.head != PAC_HEAD_MEANPOOL_CLS) return false;
+    return c->tb.on || !use_fused_cls(c) ? plain_head_ok(c, B) : true;
+}
 ArgIds arg_ids(const pac_ctx* c, int B) {
     ArgIds a;
     a.n = c->step_arg_ids ? B : 0;
@@ -991,13 +995,13 @@ MidParams mid_params(pac_ctx* c, const MidPlan& mp, const int* d_ids, int B, boo
 
 // W_up W_head for the stand-alone head kernels, once per forward (launched ahead of the down-projections so that
 // it overlaps the tail of the previous step's optimizer update).
-pac_status head_matrix_enqueue(pac_ctx* c) {
+pac_status head_matrix_enqueue(pac_ctx* c, int B) {
     const Dims& dm = c->dm;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[1];
     pdl_launch_config(&cfg, attr, dim3(cdiv((long long)dm.r * dm.C, 8)), dim3(256), 0, c->stream);
     cudaError_t e = cudaLaunchKernelEx(&cfg, head_matrix_kernel, (const float*)(c->params + c->lay.w_up),
-                                       (const float*)(c->params + c->lay.w_head), dm.d, dm.r, dm.C, c->sc.prodW);
+                                       (const float*)(c->params + c->lay.w_head), dm.d, dm.r, dm.C, c->sc.prodW, arg_ids(c, B), c->sc.ids);
     c->launches++;
     if (e != cudaSuccess) return fail(c, PAC_ERR_CUDA, "head matrix kernel launch failed: %s", cudaGetErrorString(e));
     return PAC_OK;
@@ -1038,7 +1042,7 @@ pac_status chain_fwd_enqueue(pac_ctx* c, const int* d_ids, int B, bool train, fl
     cp.lam = c->params + c->lay.lam;
     cp.tc = c->sc.tc; cp.pool_part = c->sc.pool_part;
     cp.status = c->status; cp.stamp = next_stamp(c, 0);
-    pac_status hs = head_matrix_enqueue(c);
+    pac_status hs = head_matrix_enqueue(c, B);
     if (hs != PAC_OK) return hs;
     time_mark(c, 0, false);
     const bool pair = c->chain_pair_stages > 0 && c->forward_mode != 5 && ((B * cp.s_chunks) & 1) == 0;
@@ -1070,7 +1074,7 @@ pac_status cls_forward_enqueue(pac_ctx* c, const int* d_ids, int B, bool train, 
         time_mark(c, 0, true);
         return st;
     }
-    if ((st = head_matrix_enqueue(c)) != PAC_OK) return st;
+    if ((st = head_matrix_enqueue(c, B)) != PAC_OK) return st;
     if ((st = down_projection(c, d_ids, B)) != PAC_OK) return st;
     time_mark(c, 1, false);
     st = mid_enqueue(c, d_ids, B, train, d_logits_out);
@@ -1817,7 +1821,7 @@ pac_status pac_train_epoch(pac_ctx* c, const int* perm, long long n, int B, cons
         if (losses_out) std::memcpy(losses_out, c->h_losses, sizeof(float) * (n / B));
         return PAC_OK;
     }
-    if (arg_ids_ok(c, B)) {
+    if (arg_ids_ok(c, B)) {                        // (a launch less at the start of the epoch, and the second pass knows its ids early)
         for (long long s = 0; s < n / B; ++s) {
             c->step_arg_ids = perm + s * B;
             st = finish_ids(c, train_enqueue(c, c->sc.ids, B, c->h_losses + s, hp));

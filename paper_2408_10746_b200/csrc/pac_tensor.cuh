@@ -788,7 +788,7 @@ dw_down_tc_kernel(const __grid_constant__ CUtensorMap map_cache, BwdParams p, co
 // are announced only by workers that have read these, so the full barriers say that, too.
 constexpr int DG_WORKERS = 16, DG_THREADS = 32 * (2 + DG_WORKERS);
 __global__ void __launch_bounds__(DG_THREADS, 1)
-dw_down_gates_kernel(const __grid_constant__ CUtensorMap map_cache, BwdParams p) {
+dw_down_gates_kernel(const __grid_constant__ CUtensorMap map_cache, BwdParams p, const __grid_constant__ ArgIds arg) {
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     const uint32_t box_bytes = BWD_KR * 128, a_bytes = (uint32_t)p.chunks * 2 * box_bytes, g_off = a_bytes + 2 * box_bytes;      // a stage: h tile, gate tile, gate bytes
@@ -824,6 +824,7 @@ dw_down_gates_kernel(const __grid_constant__ CUtensorMap map_cache, BwdParams p)
         for (int q = 0; q < 2 * p.chunks; ++q)
             tma_load_4d_hint(dst + q * box_bytes, &map_cache, full, col0 + q * 64, sc * BWD_KR, l, id, pol);
     };
+    const auto sample = [&](int b) { return arg.n > 0 ? arg.v[b] : (int)safe_id(p.ids, b, p.N, nullptr); };
     // the first ring of h tiles ahead of the wait, as in dw_down_tc_kernel
     uint32_t pre = 0;
     if (p.early_ids && warp == 0 && rt1 > rt0) {
@@ -831,7 +832,7 @@ dw_down_gates_kernel(const __grid_constant__ CUtensorMap map_cache, BwdParams p)
         if (elect_one())
             for (uint32_t i = 0; i < pre; ++i) {
                 const int rt = rt0 + (int)i, b = rt / p.s_chunks;
-                load_h(smem_u32(smem) + i * stage_bytes, full0 + 8 * i, rt - b * p.s_chunks, (int)safe_id(p.ids, b, p.N, nullptr));
+                load_h(smem_u32(smem) + i * stage_bytes, full0 + 8 * i, rt - b * p.s_chunks, sample(b));
             }
         __syncwarp();
     }
@@ -843,7 +844,7 @@ dw_down_gates_kernel(const __grid_constant__ CUtensorMap map_cache, BwdParams p)
         const uint32_t ring0 = smem_u32(smem);
         uint32_t dst = ring0;
         int b = b0, sc = rt0 - b0 * p.s_chunks;
-        int id = rt1 > rt0 ? (int)safe_id(p.ids, b, p.N, nullptr) : 0;
+        int id = rt1 > rt0 ? sample(b) : 0;
         for (int rt = rt0; rt < rt1; ++rt) {
             if (pre == 0 && !mbar_wait_uniform(empty0 + 8 * s, eph, abort_flag, p.status)) break;
             if (elect_one()) {
@@ -858,7 +859,7 @@ dw_down_gates_kernel(const __grid_constant__ CUtensorMap map_cache, BwdParams p)
             if (++s == (uint32_t)p.stages) { s = 0; eph ^= 1u; dst = ring0; }
             if (++sc == p.s_chunks) {
                 sc = 0; ++b;
-                if (rt + 1 < rt1) id = (int)safe_id(p.ids, b, p.N, nullptr);
+                if (rt + 1 < rt1) id = sample(b);
             }
         }
     } else if (warp == 1) {
@@ -1197,13 +1198,13 @@ inline pac_status tensor_dw_down(TensorPlan& tp, cudaStream_t stream, const int*
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[1];
     pdl_launch_config(&cfg, attr, dim3((unsigned)grid), dim3(DW_THREADS), tp.smem_bwd, stream);
-    if (tp.gates && p.da_token == 0 && arg.n == 0) {
+    if (tp.gates && p.da_token == 0) {
         const int stage = (p.chunks + 1) * 2 * BWD_KR * 128 + BWD_KR * p.r;
         p.stages = std::min(16, (tp.max_smem - 8192) / stage);
         const size_t smem = (size_t)p.stages * stage + 1024;
         pdl_launch_config(&cfg, attr, dim3((unsigned)grid), dim3(DG_THREADS), smem, stream);
         cudaError_t e = smem_opt_in((const void*)dw_down_gates_kernel, smem);
-        if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, dw_down_gates_kernel, tp.map_cache_bwd, p);
+        if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, dw_down_gates_kernel, tp.map_cache_bwd, p, arg);
         (*launches)++;
         if (e != cudaSuccess) { tensor_err() = cudaGetErrorString(e); return PAC_ERR_CUDA; }
         return PAC_OK;
