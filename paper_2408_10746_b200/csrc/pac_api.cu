@@ -261,6 +261,7 @@ WdShadow wd_shadow(const pac_ctx* c) { return WdShadow{c->sc.wdT}; }
 pac_status adam_enqueue(pac_ctx* c, const pac_adamw* hp);
 pac_status down_projection(pac_ctx* c, const int* d_ids, int B);
 pac_status dw_down(pac_ctx* c, const int* d_ids, int B, bool reduce_splits);
+ArgIds arg_ids(const pac_ctx* c, int B);
 
 inline unsigned cdiv(long long a, long long b) { return (unsigned)((a + b - 1) / b); }
 
@@ -393,7 +394,7 @@ pac_status xgemm_rows(pac_ctx* c, int M, int N, int K, int Z, const AL& A, const
     XgJobs<AL> J;
     J.tile_j = xg_tile_j(N);
     J.add(A, M, W, N, 0);
-    cudaError_t e = xgemm_launch_rows(J, K, Z, c->sms, out, zstride, c->sc.xg_ws, c->sc.xg_cnt, c->status, c->stream);
+    cudaError_t e = xgemm_launch_rows(J, K, Z, c->sms, out, zstride, c->sc.xg_ws, c->sc.xg_cnt, c->status, c->stream, arg_ids(c, M / c->dm.S), c->sc.ids);
     c->launches++;
     if (e != cudaSuccess) return fail(c, PAC_ERR_CUDA, "product kernel launch failed: %s", cudaGetErrorString(e));
     return PAC_OK;
@@ -423,7 +424,7 @@ pac_status down_projection_simt(pac_ctx* c, const int* d_ids, int B) {
                       c->sc.u, (long long)c->max_rows * dm.r);
 }
 
-pac_status head_matrix_enqueue(pac_ctx* c, int B);
+pac_status head_matrix_enqueue(pac_ctx* c, int B, bool behind);
 pac_status finalize_enqueue(pac_ctx* c, const int* d_ids, int B, float* d_loss, const pac_adamw* hp);
 pac_status adam_body_enqueue(pac_ctx* c, const pac_adamw* hp);
 
@@ -470,9 +471,10 @@ pac_status forward(pac_ctx* c, const int* d_ids, int B, bool train, float* d_log
     const long long n = (long long)M * dm.r, stride = (long long)c->max_rows * dm.r;
     Scratch& sc = c->sc;
     pac_status st = PAC_OK;
-    if (plain_head_ok(c, B) && (st = head_matrix_enqueue(c, B)) != PAC_OK) return st;
+    if (use_tensor(c) && plain_head_ok(c, B) && (st = head_matrix_enqueue(c, B, false)) != PAC_OK) return st;
     st = down_projection(c, d_ids, B);
     if (st != PAC_OK) return st;
+    if (!use_tensor(c) && plain_head_ok(c, B) && (st = head_matrix_enqueue(c, B, true)) != PAC_OK) return st;
     const float* lam = c->params + c->lay.lam;
     float* aL = sc.a + (long long)(dm.L - 1) * stride;
     const bool relu = c->cfg.act == PAC_ACT_RELU;
@@ -791,8 +793,8 @@ pac_status tb_forward(pac_ctx* c, const int* d_ids, int B, bool train, float* d_
         tb_pack_kernel<<<dim3(cdiv(t.pk.tiles(), 8), (unsigned)dm.L), 256, 0, st>>>(c->params + c->lay.body, bl.per_layer, bl, t.pk, reinterpret_cast<unsigned char*>(t.packed));
         LAUNCH_CHECK(c);
     }
-    if (plain_head_ok(c, B)) TB_OK(head_matrix_enqueue(c, B));
     TB_OK(down_projection(c, d_ids, B));
+    if (plain_head_ok(c, B)) TB_OK(head_matrix_enqueue(c, B, true));
     const float* lam = c->params + c->lay.lam;
     const unsigned rows_grid = cdiv(M, 8), heads_grid = cdiv((long long)B * t.H * dm.S, 128);
     if (t.plan.ok) TB_OK(tb_fused_forward(c, B, train));
@@ -942,7 +944,7 @@ pac_status down_projection(pac_ctx* c, const int* d_ids, int B) {
 // Whether a step's host ids can be arguments of its kernels: the one-launch forward and the second pass then request their first cache tiles ahead of
 // everything before them in the stream, and no kernel has to store the ids first (T5-Base: evaluation of 27 samples
 // 23.6 -> 22.1 us, a step of 32 with its own update launch 62.0 -> 58.0, with the fused one, whose ids the forward read from host memory before, 55.8 -> 55.0).
-// Other classifier steps begin with head_matrix_kernel, which stores them for the kernels behind it.
+// In other classifier steps the first kernel that has them (the down-projection, or head_matrix_kernel ahead of it) stores them for the kernels behind it.
 bool arg_ids_ok(const pac_ctx* c, int B) {
     if (c->hc.on || B > ARG_IDS || c->cfg.head != PAC_HEAD_MEANPOOL_CLS) return false;
     return c->tb.on || !use_fused_cls(c) ? plain_head_ok(c, B) : true;
@@ -995,13 +997,13 @@ MidParams mid_params(pac_ctx* c, const MidPlan& mp, const int* d_ids, int B, boo
 
 // W_up W_head for the stand-alone head kernels, once per forward (launched ahead of the down-projections so that
 // it overlaps the tail of the previous step's optimizer update).
-pac_status head_matrix_enqueue(pac_ctx* c, int B) {
+pac_status head_matrix_enqueue(pac_ctx* c, int B, bool behind) {
     const Dims& dm = c->dm;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[1];
     pdl_launch_config(&cfg, attr, dim3(cdiv((long long)dm.r * dm.C, 8)), dim3(256), 0, c->stream);
     cudaError_t e = cudaLaunchKernelEx(&cfg, head_matrix_kernel, (const float*)(c->params + c->lay.w_up),
-                                       (const float*)(c->params + c->lay.w_head), dm.d, dm.r, dm.C, c->sc.prodW, arg_ids(c, B), c->sc.ids);
+                                       (const float*)(c->params + c->lay.w_head), dm.d, dm.r, dm.C, c->sc.prodW, behind ? 1 : 0, behind ? ArgIds{} : arg_ids(c, B), c->sc.ids);
     c->launches++;
     if (e != cudaSuccess) return fail(c, PAC_ERR_CUDA, "head matrix kernel launch failed: %s", cudaGetErrorString(e));
     return PAC_OK;
@@ -1042,16 +1044,17 @@ pac_status chain_fwd_enqueue(pac_ctx* c, const int* d_ids, int B, bool train, fl
     cp.lam = c->params + c->lay.lam;
     cp.tc = c->sc.tc; cp.pool_part = c->sc.pool_part;
     cp.status = c->status; cp.stamp = next_stamp(c, 0);
-    pac_status hs = head_matrix_enqueue(c, B);
-    if (hs != PAC_OK) return hs;
+    cp.ids_copy = c->sc.ids;
     time_mark(c, 0, false);
     const bool pair = c->chain_pair_stages > 0 && c->forward_mode != 5 && ((B * cp.s_chunks) & 1) == 0;
     if (pair) cp.stages = c->chain_pair_stages;
-    cudaError_t e = pair ? chain_pair_launch(c->tplan.map_cache_fwd, c->tplan.map_w, cp, chain_pair_smem(cp.stages), c->cfg.act, c->stream)
-                         : chain_fwd_launch(c->tplan.map_cache_fwd, c->tplan.map_w, cp, c->tplan.smem_fwd, c->cfg.act, c->stream);
+    cudaError_t e = pair ? chain_pair_launch(c->tplan.map_cache_fwd, c->tplan.map_w, cp, arg_ids(c, B), chain_pair_smem(cp.stages), c->cfg.act, c->stream)
+                         : chain_fwd_launch(c->tplan.map_cache_fwd, c->tplan.map_w, cp, arg_ids(c, B), c->tplan.smem_fwd, c->cfg.act, c->stream);
     c->launches++;
     time_mark(c, 0, true);
     if (e != cudaSuccess) return fail(c, PAC_ERR_CUDA, "chain-in-epilogue forward launch failed: %s", cudaGetErrorString(e));
+    pac_status hs = head_matrix_enqueue(c, B, true);
+    if (hs != PAC_OK) return hs;
     MidParams p = mid_params(c, c->pplan, d_ids, B, train, d_logits_out);
     p.pool_part = c->sc.pool_part; p.n_pool_parts = cp.s_chunks * CF_POOL_PARTS;
     p.prodW = c->sc.prodW;
@@ -1074,8 +1077,9 @@ pac_status cls_forward_enqueue(pac_ctx* c, const int* d_ids, int B, bool train, 
         time_mark(c, 0, true);
         return st;
     }
-    if ((st = head_matrix_enqueue(c, B)) != PAC_OK) return st;
+    if (use_tensor(c) && (st = head_matrix_enqueue(c, B, false)) != PAC_OK) return st;
     if ((st = down_projection(c, d_ids, B)) != PAC_OK) return st;
+    if (!use_tensor(c) && (st = head_matrix_enqueue(c, B, true)) != PAC_OK) return st;
     time_mark(c, 1, false);
     st = mid_enqueue(c, d_ids, B, train, d_logits_out);
     time_mark(c, 1, true);

@@ -28,6 +28,7 @@ struct ChainFwdParams {
     float* pool_part;                      // [B][s_chunks * CF_POOL_PARTS][r]: token sums of a_L per 32-token group
     unsigned* status;
     unsigned long long* stamp;
+    int* ids_copy;              // ids as an argument: their copy for the kernels behind this one
 };
 
 // The epilogue of one warp (see the kernel below).  acce0: "accumulator drained" barriers, in this CTA, or - acce_remote -
@@ -113,7 +114,7 @@ __device__ __forceinline__ void chain_epilogue(const ChainFwdParams& p, const fl
 // CH: 16-column chunks per epilogue warp (r = 32 * CH).
 template <int ACT, int CH>
 __global__ void __launch_bounds__(CF_THREADS, 1)
-down_chain_tc_kernel(const __grid_constant__ CUtensorMap map_cache, const __grid_constant__ CUtensorMap map_w, ChainFwdParams p) {
+down_chain_tc_kernel(const __grid_constant__ CUtensorMap map_cache, const __grid_constant__ CUtensorMap map_w, ChainFwdParams p, const __grid_constant__ ArgIds arg) {
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     const int r_blocks = (p.r + 63) >> 6;
@@ -138,19 +139,20 @@ down_chain_tc_kernel(const __grid_constant__ CUtensorMap map_cache, const __grid
         tma_prefetch_desc(&map_w);
     }
     if (warp == 1) { tmem_alloc(smem_u32(&tmem_base_sh), 512u); tmem_relinquish(); }
-    pdl_trigger();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = tmem_base_sh;
     volatile int* abort_flag = &abort_sh;
     pdl_wait();            // the weights (updated by the predecessor) and device ids are final from here on
+    pdl_trigger();         // (head_matrix_kernel behind this one reads parameters at once)
     if (warp >= 2) {
         // lambda of every layer for the epilogue warps (a barrier of their own: the pipeline warps never join it)
         if (warp == 2) lam_s[lane] = lane < p.L ? p.lam[lane] : 0.f;
         asm volatile("bar.sync 1, %0;" ::"r"(32 * CF_EPI_WARPS) : "memory");
     }
-    const int id = (int)safe_id(p.ids, b, p.N, (threadIdx.x == 0 && sc == 0) ? p.status : nullptr);
+    const int id = arg.n > 0 ? arg.v[b] : (int)safe_id(p.ids, b, p.N, (threadIdx.x == 0 && sc == 0) ? p.status : nullptr);
+    if (arg.n > 0 && threadIdx.x == 0 && sc == 0) p.ids_copy[b] = id;
 
     // Both pipeline loops carry ring positions, parities, addresses and descriptors from step to step: their own
     // instruction streams are on the critical path of a K step.
@@ -226,7 +228,7 @@ down_chain_tc_kernel(const __grid_constant__ CUtensorMap map_cache, const __grid
 // accumulators of both with multicast commits; the epilogue warps of both arrive at its "drained" barrier.
 template <int ACT, int CH>
 __global__ void __launch_bounds__(CF_THREADS, 1)
-down_chain_pair_kernel(const __grid_constant__ CUtensorMap map_cache, const __grid_constant__ CUtensorMap map_w, ChainFwdParams p) {
+down_chain_pair_kernel(const __grid_constant__ CUtensorMap map_cache, const __grid_constant__ CUtensorMap map_w, ChainFwdParams p, const __grid_constant__ ArgIds arg) {
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     namespace cg = cooperative_groups;
@@ -253,7 +255,6 @@ down_chain_pair_kernel(const __grid_constant__ CUtensorMap map_cache, const __gr
         tma_prefetch_desc(&map_w);
     }
     if (warp == 1) { tmem_alloc_pair(smem_u32(&tmem_base_sh), 512u); tmem_relinquish_pair(); }
-    pdl_trigger();
     tc_fence_before();
     __syncthreads();
     cluster.sync();                        // the peer's barriers exist before anything arrives at them
@@ -261,11 +262,13 @@ down_chain_pair_kernel(const __grid_constant__ CUtensorMap map_cache, const __gr
     const uint32_t tmem_base = tmem_base_sh;
     volatile int* abort_flag = &abort_sh;
     pdl_wait();
+    pdl_trigger();
     if (warp >= 2) {
         if (warp == 2) lam_s[lane] = lane < p.L ? p.lam[lane] : 0.f;
         asm volatile("bar.sync 1, %0;" ::"r"(32 * CF_EPI_WARPS) : "memory");
     }
-    const int id = (int)safe_id(p.ids, b, p.N, (threadIdx.x == 0 && sc == 0) ? p.status : nullptr);
+    const int id = arg.n > 0 ? arg.v[b] : (int)safe_id(p.ids, b, p.N, (threadIdx.x == 0 && sc == 0) ? p.status : nullptr);
+    if (arg.n > 0 && threadIdx.x == 0 && sc == 0) p.ids_copy[b] = id;
 
     if (warp == 0) {
         // both CTAs: own cache tile and weight block `rank`, counted on the barrier of CTA 0
@@ -336,7 +339,7 @@ down_chain_pair_kernel(const __grid_constant__ CUtensorMap map_cache, const __gr
 inline bool chain_fwd_supported(const Dims& dm) { return dm.r % 32 == 0 && dm.r >= 32 && dm.r <= 128 && dm.L <= 32 && dm.d % 8 == 0 && dm.d >= 64; }
 
 template <int ACT>
-inline cudaError_t chain_fwd_launch_act(const CUtensorMap& map_cache, const CUtensorMap& map_w, const ChainFwdParams& p, size_t smem,
+inline cudaError_t chain_fwd_launch_act(const CUtensorMap& map_cache, const CUtensorMap& map_w, const ChainFwdParams& p, const ArgIds& arg, size_t smem,
                                         cudaStream_t stream) {
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[1];
@@ -344,13 +347,13 @@ inline cudaError_t chain_fwd_launch_act(const CUtensorMap& map_cache, const CUte
     cudaError_t e;
     switch (p.r / 32) {
         case 1: if ((e = smem_opt_in((const void*)down_chain_tc_kernel<ACT, 1>, smem)) != cudaSuccess) return e;
-                return cudaLaunchKernelEx(&cfg, down_chain_tc_kernel<ACT, 1>, map_cache, map_w, p);
+                return cudaLaunchKernelEx(&cfg, down_chain_tc_kernel<ACT, 1>, map_cache, map_w, p, arg);
         case 2: if ((e = smem_opt_in((const void*)down_chain_tc_kernel<ACT, 2>, smem)) != cudaSuccess) return e;
-                return cudaLaunchKernelEx(&cfg, down_chain_tc_kernel<ACT, 2>, map_cache, map_w, p);
+                return cudaLaunchKernelEx(&cfg, down_chain_tc_kernel<ACT, 2>, map_cache, map_w, p, arg);
         case 3: if ((e = smem_opt_in((const void*)down_chain_tc_kernel<ACT, 3>, smem)) != cudaSuccess) return e;
-                return cudaLaunchKernelEx(&cfg, down_chain_tc_kernel<ACT, 3>, map_cache, map_w, p);
+                return cudaLaunchKernelEx(&cfg, down_chain_tc_kernel<ACT, 3>, map_cache, map_w, p, arg);
         default: if ((e = smem_opt_in((const void*)down_chain_tc_kernel<ACT, 4>, smem)) != cudaSuccess) return e;
-                 return cudaLaunchKernelEx(&cfg, down_chain_tc_kernel<ACT, 4>, map_cache, map_w, p);
+                 return cudaLaunchKernelEx(&cfg, down_chain_tc_kernel<ACT, 4>, map_cache, map_w, p, arg);
     }
 }
 
@@ -363,7 +366,7 @@ inline int chain_pair_stages(int max_smem) {
 inline size_t chain_pair_smem(int stages) { return (size_t)stages * (FWD_ROWS * KC * 2 + 2 * KC * 128) + 1024; }
 
 template <int ACT, int CH>
-inline cudaError_t chain_pair_launch_one(const CUtensorMap& map_cache, const CUtensorMap& map_w, const ChainFwdParams& p, size_t smem,
+inline cudaError_t chain_pair_launch_one(const CUtensorMap& map_cache, const CUtensorMap& map_w, const ChainFwdParams& p, const ArgIds& arg, size_t smem,
                                          cudaStream_t stream) {
     cudaError_t e = smem_opt_in((const void*)down_chain_pair_kernel<ACT, CH>, smem);
     if (e != cudaSuccess) return e;
@@ -381,23 +384,23 @@ inline cudaError_t chain_pair_launch_one(const CUtensorMap& map_cache, const CUt
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, down_chain_pair_kernel<ACT, CH>, map_cache, map_w, p);
+    return cudaLaunchKernelEx(&cfg, down_chain_pair_kernel<ACT, CH>, map_cache, map_w, p, arg);
 }
 // p.stages: stages of the pair kernel's ring; the grid (B * s_chunks) must be even.
-inline cudaError_t chain_pair_launch(const CUtensorMap& map_cache, const CUtensorMap& map_w, const ChainFwdParams& p, size_t smem, int act,
+inline cudaError_t chain_pair_launch(const CUtensorMap& map_cache, const CUtensorMap& map_w, const ChainFwdParams& p, const ArgIds& arg, size_t smem, int act,
                                      cudaStream_t stream) {
     const bool relu = act == PAC_ACT_RELU;
     if (p.r / 32 == 3)
-        return relu ? chain_pair_launch_one<PAC_ACT_RELU, 3>(map_cache, map_w, p, smem, stream)
-                    : chain_pair_launch_one<PAC_ACT_IDENTITY, 3>(map_cache, map_w, p, smem, stream);
-    return relu ? chain_pair_launch_one<PAC_ACT_RELU, 4>(map_cache, map_w, p, smem, stream)
-                : chain_pair_launch_one<PAC_ACT_IDENTITY, 4>(map_cache, map_w, p, smem, stream);
+        return relu ? chain_pair_launch_one<PAC_ACT_RELU, 3>(map_cache, map_w, p, arg, smem, stream)
+                    : chain_pair_launch_one<PAC_ACT_IDENTITY, 3>(map_cache, map_w, p, arg, smem, stream);
+    return relu ? chain_pair_launch_one<PAC_ACT_RELU, 4>(map_cache, map_w, p, arg, smem, stream)
+                : chain_pair_launch_one<PAC_ACT_IDENTITY, 4>(map_cache, map_w, p, arg, smem, stream);
 }
 
-inline cudaError_t chain_fwd_launch(const CUtensorMap& map_cache, const CUtensorMap& map_w, const ChainFwdParams& p, size_t smem, int act,
+inline cudaError_t chain_fwd_launch(const CUtensorMap& map_cache, const CUtensorMap& map_w, const ChainFwdParams& p, const ArgIds& arg, size_t smem, int act,
                                     cudaStream_t stream) {
-    return act == PAC_ACT_RELU ? chain_fwd_launch_act<PAC_ACT_RELU>(map_cache, map_w, p, smem, stream)
-                               : chain_fwd_launch_act<PAC_ACT_IDENTITY>(map_cache, map_w, p, smem, stream);
+    return act == PAC_ACT_RELU ? chain_fwd_launch_act<PAC_ACT_RELU>(map_cache, map_w, p, arg, smem, stream)
+                               : chain_fwd_launch_act<PAC_ACT_IDENTITY>(map_cache, map_w, p, arg, smem, stream);
 }
 
 }  // namespace pac

@@ -152,20 +152,24 @@ __device__ __forceinline__ void mid_head_products(const MidParams& p, const MidS
 // prodW[j][c] = sum_k W_up[j][k] W_head[k][c], one warp per entry, k in lane order then a fixed shuffle tree.  The
 // product does not depend on the sample: the stand-alone head kernels take it from here instead of forming
 // it again in every CTA (the one-launch forward forms it on warps that would otherwise idle under the stream).
-// The first block stores the step's ids where they travel as an argument: one launch less (blocking fp32 step on the smallest configuration 49.7 -> 47.3 us).
+// behind: the kernel ahead lets this one start only when everything ahead of itself is complete, so the parameters are final; it runs beside that kernel and ends after it, so
+// that whoever waits for this one finds both done (smallest blocking fp32 step 50.7 -> 48.4 us, fp32 step at T5-Base widths 91.6 -> 86.3, T5-Large step 436 -> 430).
+// Otherwise the first block stores the step's ids, where they travel as an argument (the kernel ahead does so then).
 __global__ void __launch_bounds__(256) head_matrix_kernel(const float* __restrict__ W_up, const float* __restrict__ W_head, int d, int r,
-                                                          int C, float* __restrict__ prodW, const __grid_constant__ ArgIds arg, int* __restrict__ ids) {
+                                                          int C, float* __restrict__ prodW, int behind, const __grid_constant__ ArgIds arg, int* __restrict__ ids) {
     pdl_trigger();
-    pdl_wait();                      // the parameters come from the optimizer update before this kernel, and the ids of the step before may be read until then
+    if (!behind) pdl_wait();         // the parameters come from the optimizer update before this kernel, and the ids of the step before may be read until then
     if (blockIdx.x == 0 && (int)threadIdx.x < arg.n) ids[threadIdx.x] = arg.v[threadIdx.x];
     const int e = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-    if (e >= r * C) return;
-    const int j = e / C, c = e - j * C;
-    float acc = 0.f;
+    if (e < r * C) {
+        const int j = e / C, c = e - j * C;
+        float acc = 0.f;
 #pragma unroll 8
-    for (int k = lane; k < d; k += 32) acc = fmaf(__ldg(W_up + (long long)j * d + k), __ldg(W_head + (long long)k * C + c), acc);
-    acc = warp_sum(acc);
-    if (lane == 0) prodW[e] = acc;
+        for (int k = lane; k < d; k += 32) acc = fmaf(__ldg(W_up + (long long)j * d + k), __ldg(W_head + (long long)k * C + c), acc);
+        acc = warp_sum(acc);
+        if (lane == 0) prodW[e] = acc;
+    }
+    if (behind) pdl_wait();
 }
 
 // Classifier head of the plain path, one CTA per sample: token mean of a_L, logits from the C-vectors (the head's matrix

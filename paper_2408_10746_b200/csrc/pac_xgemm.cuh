@@ -27,6 +27,7 @@ struct XgCacheRows {
     typedef T elem;
     const T* cache; const int* ids; long long N; int L, S, d;
     bool vec;                                   // rows start on 16-byte boundaries
+    __device__ void take_ids(const int* v) { ids = v; }
     __device__ const T* row(int z, int m) const {
         const int b = m / S, s = m - b * S;
         return cache + ((safe_id(ids, b, N, nullptr) * L + z) * S + s) * (long long)d;
@@ -37,6 +38,7 @@ struct XgRows {
     typedef float elem;
     const float* base; long long zstride; int ld;
     bool vec;                                   // rows start on 16-byte boundaries
+    __device__ void take_ids(const int*) {}
     __device__ const float* row(int z, int m) const { return base + z * zstride + (long long)m * ld; }
 };
 
@@ -121,7 +123,7 @@ inline size_t xg_smem(int tile_j, int teams) { return teams * ((size_t)XgTerms<t
 // or a finite one beyond the largest bf16, has a first term of infinity and no second one, and a partial sum may overflow on the way.
 // dst: the thread's row of sums, `step` apart.
 template <bool TN, class AL>
-__device__ __noinline__ void xg_redo(const AL& A, const XgRows& B, int z, int i, int j0, int c0, int c_step, int nj_tile, int Nj, int kb, int ke, float* dst, long long step) {
+__device__ __noinline__ void xg_redo(AL A, XgRows B, int z, int i, int j0, int c0, int c_step, int nj_tile, int Nj, int kb, int ke, float* dst, long long step) {
 #pragma unroll 1
     for (; c0 < nj_tile; c0 += c_step)
 #pragma unroll 1
@@ -147,7 +149,8 @@ struct XgTail { int whole, parts; float* ws; unsigned* cnt; };
 // out + s * part_stride and are added up in slice order by whoever reads them.  GB: 8-column groups of B per thread (tile_j = 32 GB at most).
 template <bool TN, int GB, int TEAMS, class AL>
 __global__ void __launch_bounds__(xg_threads(TEAMS), TEAMS == 1 ? 2 : 1)
-xgemm_kernel(const __grid_constant__ XgJobs<AL> J, int K, int k_slice, int accs_most, float* __restrict__ out, long long zstride, long long part_stride, XgTail tail, unsigned* status) {
+xgemm_kernel(const __grid_constant__ XgJobs<AL> J, int K, int k_slice, int accs_most, float* __restrict__ out, long long zstride, long long part_stride, XgTail tail, unsigned* status,
+             const __grid_constant__ ArgIds arg, int* __restrict__ ids_out) {
     typedef typename AL::elem T;
     constexpr int TA = XgTerms<T>::n, PRODUCERS = TEAMS * XG_TEAM, THREADS = xg_threads(TEAMS);
     extern __shared__ unsigned char smem_raw[];
@@ -194,6 +197,8 @@ xgemm_kernel(const __grid_constant__ XgJobs<AL> J, int K, int k_slice, int accs_
     volatile int* abort_flag = &abort_sh;
     pdl_wait();
     pdl_trigger();      // (not before: a successor may rely on everything ahead of this kernel being complete when it starts)
+    // the step's ids as an argument: this kernel reads them there and leaves a copy for the ones behind it
+    if (!TN && blockIdx.x == 0 && (int)threadIdx.x < arg.n) ids_out[threadIdx.x] = arg.v[threadIdx.x];
     if (warp == PRODUCERS) {
         const uint32_t idesc = instr_desc_bf16(XG_TILE, nj_tile, TN ? 1 : 0, 1);
         // (term of A, term of B), the product of the first terms last
@@ -227,7 +232,8 @@ xgemm_kernel(const __grid_constant__ XgJobs<AL> J, int K, int k_slice, int accs_
         }
     } else {
         const int team = TEAMS == 1 ? 0 : warp >> 3, t = threadIdx.x & 255;
-        const AL A = J.A[jb];
+        AL A = J.A[jb];
+        if (!TN && arg.n > 0) A.take_ids(arg.v);
         const XgRows B = J.B[jb];
         typename XgTerms<T>::reg ra[4];
         XgF8 rb[GB];
@@ -340,7 +346,7 @@ xgemm_kernel(const __grid_constant__ XgJobs<AL> J, int K, int k_slice, int accs_
             }
             if (!(odd == 0.f) && i < Mi) {
                 const bool part = !TN && shared_tile >= 0;
-                xg_redo<TN>(J.A[jb], J.B[jb], z, i, j0, (warp >> 2) * 16, 32 * TEAMS, nj_tile, Nj, kb, ke, part ? ws : J.trans ? o + (long long)j0 * Mi + i : o + (long long)i * Nj + j0, J.trans ? Mi : 1);
+                xg_redo<TN>(A, B, z, i, j0, (warp >> 2) * 16, 32 * TEAMS, nj_tile, Nj, kb, ke, part ? ws : J.trans ? o + (long long)j0 * Mi + i : o + (long long)i * Nj + j0, J.trans ? Mi : 1);
             }
         }
     }
@@ -377,7 +383,7 @@ xgemm_kernel(const __grid_constant__ XgJobs<AL> J, int K, int k_slice, int accs_
 }
 
 template <bool TN, int TEAMS, class AL>
-inline cudaError_t xgemm_launch(const XgJobs<AL>& J, int K, dim3 grid, int k_slice, float* out, long long zstride, long long part_stride, const XgTail& tail, unsigned* status, cudaStream_t stream) {
+inline cudaError_t xgemm_launch(const XgJobs<AL>& J, int K, dim3 grid, int k_slice, float* out, long long zstride, long long part_stride, const XgTail& tail, unsigned* status, cudaStream_t stream, const ArgIds& arg, int* ids_out) {
     const auto kernel = J.tile_j <= 64 ? xgemm_kernel<TN, 2, TEAMS, AL> : xgemm_kernel<TN, 4, TEAMS, AL>;
     const size_t smem = xg_smem<AL>(J.tile_j, TEAMS);
     cudaError_t e = smem_opt_in((const void*)kernel, smem);
@@ -387,17 +393,17 @@ inline cudaError_t xgemm_launch(const XgJobs<AL>& J, int K, dim3 grid, int k_sli
     pdl_launch_config(&cfg, attr, grid, dim3(xg_threads(TEAMS)), smem, stream);
     const int longest = !TN && tail.whole > 0 ? K : K < k_slice ? K : k_slice;      // a CTA's share of the reduction
     const int accs = xg_accs(J.tile_j, (longest + XG_K - 1) / XG_K * (XG_K / 16));
-    return cudaLaunchKernelEx(&cfg, kernel, J, K, k_slice, accs, out, zstride, part_stride, tail, status);
+    return cudaLaunchKernelEx(&cfg, kernel, J, K, k_slice, accs, out, zstride, part_stride, tail, status, arg, ids_out);
 }
 template <class AL>
 inline cudaError_t xgemm_launch_tn(const XgJobs<AL>& J, int K, int Z, int slices, float* out, long long zstride, long long part_stride, unsigned* status, cudaStream_t stream) {
     const int k_slice = ((K + slices - 1) / slices + XG_K - 1) / XG_K * XG_K;
-    return xgemm_launch<true, 2>(J, K, dim3((unsigned)J.first[J.n], (unsigned)Z, (unsigned)slices), k_slice, out, zstride, part_stride, XgTail{}, status, stream);
+    return xgemm_launch<true, 2>(J, K, dim3((unsigned)J.first[J.n], (unsigned)Z, (unsigned)slices), k_slice, out, zstride, part_stride, XgTail{}, status, stream, ArgIds{}, nullptr);
 }
 // ws: 2 sms tiles of 128 x tile_j floats, cnt: 2 sms words of zero.  A tile of the last wave is shared when that takes four or more stages off its CTA
 // (the exchange costs about as much as three).
 template <class AL>
-inline cudaError_t xgemm_launch_rows(const XgJobs<AL>& J, int K, int Z, int sms, float* out, long long zstride, float* ws, unsigned* cnt, unsigned* status, cudaStream_t stream) {
+inline cudaError_t xgemm_launch_rows(const XgJobs<AL>& J, int K, int Z, int sms, float* out, long long zstride, float* ws, unsigned* cnt, unsigned* status, cudaStream_t stream, const ArgIds& arg, int* ids_out) {
     const int total = J.first[J.n] * Z, stages = (K + XG_K - 1) / XG_K;
     const bool one = total > sms && xg_accs(J.tile_j, stages * (XG_K / 16)) * J.tile_j + J.tile_j <= 256;
     if (one) sms *= 2;                              // CTAs at a time (their accumulators have to fit beside each other)
@@ -409,7 +415,7 @@ inline cudaError_t xgemm_launch_rows(const XgJobs<AL>& J, int K, int Z, int sms,
         if (stages - per >= 4) { tail.whole = total - rest; tail.parts = (stages + per - 1) / per; }
     }
     const dim3 grid((unsigned)(tail.whole + (total - tail.whole) * tail.parts));
-    return one ? xgemm_launch<false, 1>(J, K, grid, per * XG_K, out, zstride, 0, tail, status, stream) : xgemm_launch<false, 2>(J, K, grid, per * XG_K, out, zstride, 0, tail, status, stream);
+    return one ? xgemm_launch<false, 1>(J, K, grid, per * XG_K, out, zstride, 0, tail, status, stream, arg, ids_out) : xgemm_launch<false, 2>(J, K, grid, per * XG_K, out, zstride, 0, tail, status, stream, arg, ids_out);
 }
 
 // Columns per tile for an output N wide, tiles of equal width.
