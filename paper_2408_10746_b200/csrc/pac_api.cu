@@ -547,7 +547,7 @@ pac_status forward(pac_ctx* c, const int* d_ids, int B, bool train, float* d_log
 // Tiles of the plain path's dW_down, and its row slices (partial sums in sc.dw_spart when more than one).
 long long dw_simt_tiles(const Dims& dm) { return (long long)dm.L * cdiv(dm.d, XG_TILE) * cdiv(dm.r, xg_tile_j(dm.r)); }
 int dw_simt_slices(const pac_ctx* c, int B) {
-    return c->sc.dw_spart ? xg_slices(dw_simt_tiles(c->dm), B * c->dm.S, c->sms, c->dw_simt_max) : 1;
+    return c->sc.dw_spart ? xg_slices(dw_simt_tiles(c->dm), B * c->dm.S, c->sms, c->dw_simt_max, xg_tile_j(c->dm.r)) : 1;
 }
 
 template <typename T>
@@ -613,7 +613,7 @@ pac_status backward(pac_ctx* c, const int* d_ids, int B, float* d_loss, const pa
             J.tile_j = xg_tile_j(dm.r); J.trans = 1;
             J.add(xg_rows(sc.dy, 0, dm.d), dm.d, xg_rows(aL, 0, dm.r), dm.r, 0);
             const long long ne = (long long)dm.r * dm.d;
-            const int sl = sc.lm_part && ne % 4 == 0 ? xg_slices(J.first[1], M, c->sms, LM_MAX_K_SLICES) : 1;
+            const int sl = sc.lm_part && ne % 4 == 0 ? xg_slices(J.first[1], M, c->sms, LM_MAX_K_SLICES, 0) : 1;
             pac_status ts = xgemm_tn(c, J, M, 1, sl, sl > 1 ? sc.lm_part : c->grads + c->lay.w_up, 0, ne);
             if (ts != PAC_OK) return ts;
             if (sl > 1) {
@@ -773,7 +773,7 @@ pac_status tb_fused_backward(pac_ctx* c, int B) {
     J.add(xg_rows(s.o, s.sMr, r), r, xg_rows(s.dx1, s.sMr, r), r, 3 * rr);
     J.add(xg_rows(s.n2, s.sMr, r), r, xg_rows(s.dpre, s.sMf, f), f, 4 * rr);
     J.add(xg_rows(s.hid, s.sMf, f), f, xg_rows(s.da, s.sMr, r), r, 4 * rr + rf);
-    const int slices = xg_slices((long long)J.first[J.n] * L, M, c->sms, t.wg_slices);
+    const int slices = xg_slices((long long)J.first[J.n] * L, M, c->sms, t.wg_slices, 0);
     pac_status st = xgemm_tn(c, J, M, L, slices, t.wg_part, per, per * L);
     if (st != PAC_OK) return st;
     tb_reduce_slices_kernel<<<dim3(cdiv(per, 256), (unsigned)L), 256, 0, c->stream>>>(t.wg_part, slices, per * L, per, bl, gbody);
@@ -1530,7 +1530,7 @@ pac_status pac_adapter_init(pac_ctx* c, const pac_adapter_cfg* cfg, unsigned lon
         const long long ne = (long long)dm.L * dm.d * dm.r;
         // (a smaller batch may take more slices than the largest one)
         c->dw_simt_max = 1;
-        for (int b = 1; b <= cfg->max_batch && ne % 4 == 0; ++b) c->dw_simt_max = std::max(c->dw_simt_max, xg_slices(dw_simt_tiles(dm), b * dm.S, c->sms, 8));
+        for (int b = 1; b <= cfg->max_batch && ne % 4 == 0; ++b) c->dw_simt_max = std::max(c->dw_simt_max, xg_slices(dw_simt_tiles(dm), b * dm.S, c->sms, 8, xg_tile_j(dm.r)));
         if (c->dw_simt_max > 1) A(dmalloc(c, &s.dw_spart, ne * c->dw_simt_max));
         if (dm.d > 4 * XG_K) {              // (fewer stages are never shared)
             A(dmalloc(c, &s.xg_ws, 2LL * c->sms * XG_TILE * xg_tile_j(dm.r)));

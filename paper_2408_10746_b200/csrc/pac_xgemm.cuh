@@ -25,6 +25,7 @@ namespace pac {
 template <typename T>
 struct XgCacheRows {
     typedef T elem;
+    static constexpr bool cache_rows = true;
     const T* cache; const int* ids; long long N; int L, S, d;
     bool vec;                                   // rows start on 16-byte boundaries
     __device__ void take_ids(const int* v) { ids = v; }
@@ -36,6 +37,7 @@ struct XgCacheRows {
 // Row m of a row-major fp32 stack.
 struct XgRows {
     typedef float elem;
+    static constexpr bool cache_rows = false;
     const float* base; long long zstride; int ld;
     bool vec;                                   // rows start on 16-byte boundaries
     __device__ void take_ids(const int*) {}
@@ -395,18 +397,23 @@ inline cudaError_t xgemm_launch(const XgJobs<AL>& J, int K, dim3 grid, int k_sli
     const int accs = xg_accs(J.tile_j, (longest + XG_K - 1) / XG_K * (XG_K / 16));
     return cudaLaunchKernelEx(&cfg, kernel, J, K, k_slice, accs, out, zstride, part_stride, tail, status, arg, ids_out);
 }
+// Whether the accumulators of two CTAs fit beside each other.
+inline bool xg_one_team(int tile_j, int stages) { return (xg_accs(tile_j, stages * (XG_K / 16)) + 1) * tile_j <= 256; }
 template <class AL>
 inline cudaError_t xgemm_launch_tn(const XgJobs<AL>& J, int K, int Z, int slices, float* out, long long zstride, long long part_stride, unsigned* status, cudaStream_t stream) {
-    const int k_slice = ((K + slices - 1) / slices + XG_K - 1) / XG_K * XG_K;
-    return xgemm_launch<true, 2>(J, K, dim3((unsigned)J.first[J.n], (unsigned)Z, (unsigned)slices), k_slice, out, zstride, part_stride, XgTail{}, status, stream, ArgIds{}, nullptr);
+    const int k_slice = ((K + slices - 1) / slices + XG_K - 1) / XG_K * XG_K, longest = K < k_slice ? K : k_slice;
+    const dim3 grid((unsigned)J.first[J.n], (unsigned)Z, (unsigned)slices);
+    if (AL::cache_rows && J.tile_j <= 64 && xg_one_team(J.tile_j, (longest + XG_K - 1) / XG_K))
+        return xgemm_launch<true, 1>(J, K, grid, k_slice, out, zstride, part_stride, XgTail{}, status, stream, ArgIds{}, nullptr);
+    return xgemm_launch<true, 2>(J, K, grid, k_slice, out, zstride, part_stride, XgTail{}, status, stream, ArgIds{}, nullptr);
 }
 // ws: 2 sms tiles of 128 x tile_j floats, cnt: 2 sms words of zero.  A tile of the last wave is shared when that takes four or more stages off its CTA
 // (the exchange costs about as much as three).
 template <class AL>
 inline cudaError_t xgemm_launch_rows(const XgJobs<AL>& J, int K, int Z, int sms, float* out, long long zstride, float* ws, unsigned* cnt, unsigned* status, cudaStream_t stream, const ArgIds& arg, int* ids_out) {
     const int total = J.first[J.n] * Z, stages = (K + XG_K - 1) / XG_K;
-    const bool one = total > sms && xg_accs(J.tile_j, stages * (XG_K / 16)) * J.tile_j + J.tile_j <= 256;
-    if (one) sms *= 2;                              // CTAs at a time (their accumulators have to fit beside each other)
+    const bool one = total > sms && xg_one_team(J.tile_j, stages);
+    if (one) sms *= 2;                              // CTAs at a time
     const int rest = total % sms;
     XgTail tail{total, 1, ws, cnt};
     int per = stages;
@@ -424,14 +431,19 @@ inline int xg_tile_j(int N) {
     return ((N + tiles - 1) / tiles + 15) / 16 * 16;
 }
 
-// Slices of a reduction over K rows: whole waves of CTAs, each about 2 us plus 0.6 us per stage (measured), and the slices' own traffic.
-inline int xg_slices(long long tiles, int K, int sms, int most) {
+// Slices of a reduction over K rows: whole waves of CTAs, each about 2 us plus 0.6 us per stage, or 1 us where it has one team and shares its SM (measured), and the slices' own
+// traffic.  Over the rows of the cache a CTA per team (fp32 step at T5-Base widths 86.2 -> 84.4 us, smallest one 48.4 -> 47.6); the weight products of
+// transformer bodies, whose rows lie in L2, were slower so, and tiles beyond 64 columns not reliably faster (steps of r = 128 216 -> 200, r = 80 96 -> 105).
+inline int xg_slices(long long tiles, int K, int sms, int most, int tile_j) {      // tile_j: of products over the rows of the cache, else 0
     const int stages = (K + XG_K - 1) / XG_K;
     int best = 1;
     double best_cost = 1e30;
     for (int s = 1; s <= most && s <= stages; ++s) {
-        const double waves = (double)((tiles * s + sms - 1) / sms);
-        const double cost = waves * (2.0 + 0.6 * ((stages + s - 1) / s)) + 0.3 * (s - 1);
+        const int each = (stages + s - 1) / s;
+        const bool one = tile_j > 0 && tile_j <= 64 && xg_one_team(tile_j, each);
+        const int slots = one ? 2 * sms : sms;
+        const double waves = (double)((tiles * s + slots - 1) / slots);
+        const double cost = waves * (2.0 + (one ? 1.0 : 0.6) * each) + 0.3 * (s - 1);
         if (cost < best_cost) { best_cost = cost; best = s; }
     }
     return best;
