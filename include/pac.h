@@ -182,14 +182,12 @@ pac_status pac_train_step(pac_ctx* ctx, const int* sample_ids, int B, float* los
 
 /* One whole training step without waiting: pac_train_step on sample_ids (host, B ints) followed by
  * the AdamW update of pac_adam_step with `hp`, all enqueued on the context's stream; the call
- * returns as soon as that is done (it waits only when too many earlier steps' ids are still in
- * flight: 8, or 32 to 64 with the one-launch forward).  If loss_out is non-NULL the step's mean loss
+ * returns as soon as that is done (with more than 512 ids a step it waits when eight earlier steps' ids are still
+ * in flight); sample_ids may be reused then.  If loss_out is non-NULL the step's mean loss
  * arrives there once the step has run: loss_out is HOST memory that must stay valid until the next
  * pac_sync; read it after pac_sync.  Page-locked memory (cudaHostAlloc / cudaHostRegister) is written
- * by the last kernel of the step itself; other memory gets a copy behind the step.  With the one-launch
- * forward the ids are likewise taken by the kernels from a page-locked ring inside the library (the
- * step before fetches them into device memory when the host is already a call ahead, otherwise the
- * forward kernel reads them across the host link), so a step is three kernels back to back and
+ * by the last kernel of the step itself; other memory gets a copy behind the step.  With a classifier head
+ * up to 160 ids travel as arguments of the step's kernels, so a step of the one-launch forward is three kernels back to back and
  * consecutive steps overlap as in pac_train_epoch_dev.  Errors of the arguments are reported at once,
  * device-side errors by the next pac_sync.  The step a caller loops over when the minibatches
  * are chosen on the host one at a time (Section IV-B: from the second epoch on a step needs

@@ -18,7 +18,8 @@
 // the tensor instructions' fragments, a token's residual row stays in the registers of the warp that owns it, and halves of sums along K meet in
 // the row phase that reads them instead of in a phase of their own.  Weights arrive split and in the order in which a warp consumes them
 // (tb_pack_kernel).  Against scores, weights and rows in shared memory and weights split by their readers the step at B = 16, S = 128, r = 64, 12 layers went
-// from 953 to 769 us.  Loads of the second attention's operands ahead of the product before them cost 64 us in spilled registers.
+// from 953 to 769 us; parameter vectors as asynchronous copies and plain addresses where nothing needs clamping made it 748.  Twice the warps with half the registers
+// took 1028: what does not fit spills past an L1 that shared memory leaves no room.  Loads of the second attention's operands ahead of the product before them cost 64 us in spilled registers.
 #pragma once
 #include "pac_tbody.cuh"
 #include "pac_tensor.cuh"
