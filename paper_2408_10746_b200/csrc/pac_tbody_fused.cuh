@@ -305,6 +305,13 @@ __device__ __forceinline__ void tb_st2(float* p, float x, float y, bool two, boo
     else { p[0] = x; if (two) p[1] = y; }
 }
 
+// First key of a warp's round w.  With several rounds the compiler would form the addresses of all of them ahead of the loops and spill them; the value is therefore opaque.
+template <int CW>
+__device__ __forceinline__ int tb_round(int key0, int key_step, int w) {
+    int k = key0 + w * key_step;
+    if (CW > 1) asm volatile("" : "+r"(k));
+    return k;
+}
 // 32 rows (keys) x 16 columns of a head, as the B operand of scores: pair (c2, c2 + 1) and (c2 + 8, + 9) of row 8 n + lane / 4.  X: the head's first column
 // of the sample's rows; columns from `cols` on are zeros, rows from S on repeat the last one.
 struct TbKeys { float2 x[4][2]; };
@@ -488,9 +495,12 @@ __global__ void __launch_bounds__(TBF_THREADS) tb_fwd_kernel(const __grid_consta
     pdl_trigger();
     const TbStacks& s = p.s;
     const bool live = warp < nt;                                // token `warp` is this warp's row
-    float res[NR], un[NR];                                      // residual row of `tail`, u row of `head`
-    if (p.tail >= 0) tb_row_in(res, s.x + p.tail * s.sMr + (m0 + warp) * r, r, live);
-    if (p.head >= 0) tb_row_in(un, p.u + p.head * p.u_stride + (m0 + warp) * r, r, live);
+    float res[NR], un[NR];                                      // residual row of `tail`, u row of `head` (ahead of the attention where registers allow it)
+    const auto rows_in = [&] {
+        if (p.tail >= 0) tb_row_in(res, s.x + p.tail * s.sMr + (m0 + warp) * r, r, live);
+        if (p.head >= 0) tb_row_in(un, p.u + p.head * p.u_stride + (m0 + warp) * r, r, live);
+    };
+    if (CW == 1) rows_in();
     tb_vec_wait<U>();
     __syncthreads();
     if (p.tail >= 0) {
@@ -504,28 +514,34 @@ __global__ void __launch_bounds__(TBF_THREADS) tb_fwd_kernel(const __grid_consta
             const int hg = min(p.hg, H - h0), col = (h0 + hl) * dh;
             const bool mine = hl < hg;
             float sc[CW][4][4] = {};
-            TbVals vals[CW];
+            TbVals vals;
             float mx[2] = {-INFINITY, -INFINITY};
             if (mine) {
 #pragma unroll 1
                 for (int k = 0; k < dh; k += 16) {
-                    TbKeys keys[CW];
+                    TbKeys keys;
                     float2 qa[2][2];
 #pragma unroll
                     for (int i = 0; i < 2; ++i) {
                         const float* row = qkv + (long long)min(t0 + q + 8 * i, S - 1) * r + col;
                         qa[i][0] = tb_ld2(row, k + c2, dh, even); qa[i][1] = tb_ld2(row, k + c2 + 8, dh, even);
                     }
-#pragma unroll
-                    for (int w = 0; w < CW; ++w) tb_load_keys(keys[w], qkv + s.sMr + col, r, key0 + w * key_step, S, k, dh, even);
-                    if (k == 0)
-#pragma unroll
-                        for (int w = 0; w < CW; ++w) tb_load_vals(vals[w], qkv + 2 * s.sMr + col, r, key0 + w * key_step, S, 0, dh);
+                    if (CW == 1) {
+                        tb_load_keys(keys, qkv + s.sMr + col, r, key0, S, k, dh, even);
+                        if (k == 0) tb_load_vals(vals, qkv + 2 * s.sMr + col, r, key0, S, 0, dh);
+                    }
                     TbA a;
                     const float v[8] = {qa[0][0].x, qa[0][0].y, qa[1][0].x, qa[1][0].y, qa[0][1].x, qa[0][1].y, qa[1][1].x, qa[1][1].y};
                     tb_split_a(a, v);
 #pragma unroll
-                    for (int w = 0; w < CW; ++w) tb_scores(sc[w], a, keys[w]);
+                    for (int w = 0; w < CW; ++w) {
+                        if (CW > 1) {
+                            const int k0 = tb_round<CW>(key0, key_step, w);
+                            if (k0 >= S) break;
+                            tb_load_keys(keys, qkv + s.sMr + col, r, k0, S, k, dh, even);
+                        }
+                        tb_scores(sc[w], a, keys);
+                    }
                 }
                 // softmax over the keys: fragments of rows q and q + 8, keys from S on weigh nothing
 #pragma unroll
@@ -579,10 +595,12 @@ __global__ void __launch_bounds__(TBF_THREADS) tb_fwd_kernel(const __grid_consta
                     inv[i] = __frcp_rn(sum[i]);
                 }
 #pragma unroll
-                for (int w = 0; w < CW; ++w)
+                for (int w = 0; w < CW; ++w) {
+                    const int k0 = tb_round<CW>(key0, key_step, w);
+                    if (CW > 1 && k0 >= S) break;
 #pragma unroll
                     for (int n = 0; n < 4; ++n) {
-                        const int key = key0 + w * key_step + n * 8 + c2;
+                        const int key = k0 + n * 8 + c2;
 #pragma unroll
                         for (int e = 0; e < 4; ++e) sc[w][n][e] = tb_quotient(sc[w][n][e], sum[e >> 1], inv[e >> 1]);
                         if (p.train && key < S) {
@@ -590,23 +608,25 @@ __global__ void __launch_bounds__(TBF_THREADS) tb_fwd_kernel(const __grid_consta
                             if (q + 8 < nt) tb_st2(P + 8LL * S + key, sc[w][n][2], sc[w][n][3], key + 1 < S, evenS);
                         }
                     }
+                }
             }
 #pragma unroll 1
             for (int n0 = 0; n0 < dh; n0 += 16, buf ^= 1) {
                 float* share = sm.share + buf * TBF_WARPS * TB_SHARE;
                 if (mine) {
-                    if (n0 > 0)
-#pragma unroll
-                        for (int w = 0; w < CW; ++w) tb_load_vals(vals[w], qkv + 2 * s.sMr + col, r, key0 + w * key_step, S, n0, dh);
                     float big[2][4] = {}, small[2][4] = {};
 #pragma unroll
-                    for (int w = 0; w < CW; ++w)
+                    for (int w = 0; w < CW; ++w) {
+                        const int k0 = tb_round<CW>(key0, key_step, w);
+                        if (CW > 1 && k0 >= S) break;
+                        if (CW > 1 || n0 > 0) tb_load_vals(vals, qkv + 2 * s.sMr + col, r, k0, S, n0, dh);
 #pragma unroll
                         for (int k = 0; k < 2; ++k) {
                             TbA a;
                             tb_frag_a(a, sc[w], k);
-                            tb_mix(big, small, a, vals[w], k);
+                            tb_mix(big, small, a, vals, k);
                         }
+                    }
                     tb_share_put(share, big, small);
                 }
                 __syncthreads();
@@ -619,6 +639,7 @@ __global__ void __launch_bounds__(TBF_THREADS) tb_fwd_kernel(const __grid_consta
         }
         __syncthreads();
     }
+    if (CW > 1) rows_in();
 #pragma unroll 1
     for (int ph = first; ph < last; ++ph) {
         if (ph & 1) {
@@ -782,9 +803,10 @@ __global__ void __launch_bounds__(TBF_THREADS) tb_bwd_kernel(const __grid_consta
                 float* share = sm.share + buf * TBF_WARPS * TB_SHARE;
                 if (mine) {
                     float big[2][4] = {}, small[2][4] = {};
-#pragma unroll
+#pragma unroll 1
                     for (int w = 0; w < CW; ++w) {
                         const int s0 = key0 + w * key_step;
+                        if (CW > 1 && s0 >= S) break;
                         float wt[2][8];
                         TbVals x;
                         if (s0 + 32 <= S && nt == TBF_T) {     // nothing to leave out
@@ -927,24 +949,18 @@ __global__ void __launch_bounds__(TBF_THREADS) tb_bwd_kernel(const __grid_consta
     }
     if (p.head < 0) return;
     const int l = p.head;
-    TbKeys keys[CW];                   // v of the first 16 columns of a head, k as a mix operand, and P: operands of the second attention
-    TbVals vals[CW];
-    float P[CW][4][4];
+    TbKeys keys;                       // v of the first 16 columns of a head, k as a mix operand, and P: operands of the second attention
+    TbVals vals;
+    float P[4][4];
     const bool even = ((dh | r) & 1) == 0, evenS = (S & 1) == 0;
     const float* qkv = s.qkv + 3 * l * s.sMr + (long long)b * S * r;
-    const auto operands = [&](int h) {
+    const auto load_P = [&](int h, int k0) {
         const float* Pg = s.P + l * s.sP + (((long long)b * H + h) * S + t0 + q) * S;
 #pragma unroll
-        for (int w = 0; w < CW; ++w) {
-            const int k0 = key0 + w * key_step;
-            tb_load_keys(keys[w], qkv + 2 * s.sMr + h * dh, r, k0, S, 0, dh, even);
-            tb_load_vals(vals[w], qkv + s.sMr + h * dh, r, k0, S, 0, dh);
-#pragma unroll
-            for (int n = 0; n < 4; ++n) {
-                const int key = k0 + n * 8 + c2;
-                const float2 x = q < nt ? tb_ld2(Pg, key, S, evenS) : make_float2(0.f, 0.f), y = q + 8 < nt ? tb_ld2(Pg + 8LL * S, key, S, evenS) : make_float2(0.f, 0.f);
-                P[w][n][0] = x.x; P[w][n][1] = x.y; P[w][n][2] = y.x; P[w][n][3] = y.y;
-            }
+        for (int n = 0; n < 4; ++n) {
+            const int key = k0 + n * 8 + c2;
+            const float2 x = q < nt ? tb_ld2(Pg, key, S, evenS) : make_float2(0.f, 0.f), y = q + 8 < nt ? tb_ld2(Pg + 8LL * S, key, S, evenS) : make_float2(0.f, 0.f);
+            P[n][0] = x.x; P[n][1] = x.y; P[n][2] = y.x; P[n][3] = y.y;
         }
     };
     // own queries: dP = do v^T, dS = P (dP - sum dP P), dq = scale dS k; do stands in two halves
@@ -959,12 +975,14 @@ __global__ void __launch_bounds__(TBF_THREADS) tb_bwd_kernel(const __grid_consta
         const bool mine = hl < hg;
         float sc[CW][4][4] = {}, dot[2] = {};
         if (mine) {
-            operands(h);
+            if (CW == 1) {
+                tb_load_keys(keys, qkv + 2 * s.sMr + h * dh, r, key0, S, 0, dh, even);
+                tb_load_vals(vals, qkv + s.sMr + h * dh, r, key0, S, 0, dh);
+                load_P(h, key0);
+            }
 #pragma unroll 1
             for (int k = 0; k < dh; k += 16) {
-                if (k > 0)
-#pragma unroll
-                    for (int w = 0; w < CW; ++w) tb_load_keys(keys[w], qkv + 2 * s.sMr + h * dh, r, key0 + w * key_step, S, k, dh, even);
+                if (CW == 1 && k > 0) tb_load_keys(keys, qkv + 2 * s.sMr + h * dh, r, key0, S, k, dh, even);
                 // columns past the head's are zeros on the v side; what do holds there is finite
                 float v[8];
 #pragma unroll
@@ -975,14 +993,27 @@ __global__ void __launch_bounds__(TBF_THREADS) tb_bwd_kernel(const __grid_consta
                 TbA a;
                 tb_split_a(a, v);
 #pragma unroll
-                for (int w = 0; w < CW; ++w) tb_scores(sc[w], a, keys[w]);
+                for (int w = 0; w < CW; ++w) {
+                    if (CW > 1) {
+                        const int k0 = tb_round<CW>(key0, key_step, w);
+                        if (k0 >= S) break;
+                        tb_load_keys(keys, qkv + 2 * s.sMr + h * dh, r, k0, S, k, dh, even);
+                    }
+                    tb_scores(sc[w], a, keys);
+                }
             }
 #pragma unroll
-            for (int w = 0; w < CW; ++w)
+            for (int w = 0; w < CW; ++w) {
+                if (CW > 1) {
+                    const int k0 = tb_round<CW>(key0, key_step, w);
+                    if (k0 >= S) break;
+                    load_P(h, k0);
+                }
 #pragma unroll
                 for (int n = 0; n < 4; ++n)
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) dot[e >> 1] = fmaf(sc[w][n][e], P[w][n][e], dot[e >> 1]);
+                    for (int e = 0; e < 4; ++e) dot[e >> 1] = fmaf(sc[w][n][e], P[n][e], dot[e >> 1]);
+            }
         }
 #pragma unroll
         for (int i = 0; i < 2; ++i) {
@@ -998,34 +1029,41 @@ __global__ void __launch_bounds__(TBF_THREADS) tb_bwd_kernel(const __grid_consta
                 for (int c = 0; c < p.nc; ++c) dot[i] += sm.stat0[(hl * p.nc + c) * TBF_T + q + 8 * i];
             }
 #pragma unroll
-            for (int w = 0; w < CW; ++w)
+            for (int w = 0; w < CW; ++w) {
+                const int k0 = tb_round<CW>(key0, key_step, w);
+                if (CW > 1) {
+                    if (k0 >= S) break;
+                    load_P(h, k0);
+                }
 #pragma unroll
                 for (int n = 0; n < 4; ++n) {
-                    const int key = key0 + w * key_step + n * 8 + c2;
+                    const int key = k0 + n * 8 + c2;
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) sc[w][n][e] = key + (e & 1) < S ? P[w][n][e] * (sc[w][n][e] - dot[e >> 1]) : 0.f;
+                    for (int e = 0; e < 4; ++e) sc[w][n][e] = key + (e & 1) < S ? P[n][e] * (sc[w][n][e] - dot[e >> 1]) : 0.f;
                     if (key < S) {
                         if (q < nt) tb_st2(dS + key, sc[w][n][0], sc[w][n][1], key + 1 < S, evenS);
                         if (q + 8 < nt) tb_st2(dS + 8LL * S + key, sc[w][n][2], sc[w][n][3], key + 1 < S, evenS);
                     }
                 }
+            }
         }
 #pragma unroll 1
         for (int n0 = 0; n0 < dh; n0 += 16, buf ^= 1) {
             float* share = sm.share + buf * TBF_WARPS * TB_SHARE;
             if (mine) {
-                if (n0 > 0)
-#pragma unroll
-                    for (int w = 0; w < CW; ++w) tb_load_vals(vals[w], qkv + s.sMr + h * dh, r, key0 + w * key_step, S, n0, dh);
                 float big[2][4] = {}, small[2][4] = {};
 #pragma unroll
-                for (int w = 0; w < CW; ++w)
+                for (int w = 0; w < CW; ++w) {
+                    const int k0 = tb_round<CW>(key0, key_step, w);
+                    if (CW > 1 && k0 >= S) break;
+                    if (CW > 1 || n0 > 0) tb_load_vals(vals, qkv + s.sMr + h * dh, r, k0, S, n0, dh);
 #pragma unroll
                     for (int k = 0; k < 2; ++k) {
                         TbA a;
                         tb_frag_a(a, sc[w], k);
-                        tb_mix(big, small, a, vals[w], k);
+                        tb_mix(big, small, a, vals, k);
                     }
+                }
                 tb_share_put(share, big, small);
             }
             __syncthreads();
@@ -1073,7 +1111,9 @@ __global__ void __launch_bounds__(256) tb_reduce_slices_kernel(const float* __re
 }
 
 // Variant of the kernels for a shape: NR by the width, as many units in flight as shared memory leaves room for, and three rounds of keys per warp for
-// sequences beyond 16 warps of 32.
+// sequences beyond 16 warps of 32.  Up to 24 rounds two heads go at a time, three rounds to each of a head's warps; beyond, one.  In several rounds operands are fetched
+// round by round (those of all three at a time spilled 0.4 to 2 KB per thread) and rounds past the sequence are left out; step at B = 4, L = 3, r = 64, 4 heads, S = 513 / 600 / 820:
+// 1051 / 1886 / 1994 us with every round taken and all operands held, 503 / 830 / 1204 so (score rows in shared memory before: 858 / 1670 / 2122).
 struct TbPlan {
     bool ok = false;
     int variant = 0, ka = 0, kb = 0, rs = 0, nc = 0, hg = 0;
@@ -1082,7 +1122,7 @@ struct TbPlan {
 struct TbVariant { int nr, u, cw; const void *fwd, *bwd; };
 #define TB_VARIANT(NR, U, CW) {NR, U, CW, (const void*)tb_fwd_kernel<NR, U, CW>, (const void*)tb_bwd_kernel<NR, U, CW>}
 inline const TbVariant* tb_variants(int* n) {
-    static const TbVariant v[] = {TB_VARIANT(2, 5, 1), TB_VARIANT(2, 3, 1), TB_VARIANT(3, 4, 1), TB_VARIANT(6, 3, 1), TB_VARIANT(6, 2, 1), TB_VARIANT(6, 2, 3)};
+    static const TbVariant v[] = {TB_VARIANT(2, 5, 1), TB_VARIANT(2, 3, 1), TB_VARIANT(3, 4, 1), TB_VARIANT(6, 3, 1), TB_VARIANT(6, 2, 1), TB_VARIANT(2, 5, 3), TB_VARIANT(3, 4, 3), TB_VARIANT(6, 2, 3)};
     *n = (int)(sizeof(v) / sizeof(v[0]));
     return v;
 }
@@ -1095,7 +1135,7 @@ inline TbPlan tb_plan(int S, int r, int f, int H, int max_smem) {
     pl.kb = tb_up16(r) + 8;
     pl.rs = (r + 31) / 32 * 32 + 8;            // = 8 mod 32: the fragments' pairs of four rows fall into different banks
     const int chunks = (S + 31) / 32;
-    pl.nc = chunks < TBF_WARPS ? chunks : TBF_WARPS;
+    pl.nc = chunks <= TBF_WARPS ? chunks : chunks <= 3 * (TBF_WARPS / 2) ? (chunks + 2) / 3 : TBF_WARPS;
     pl.hg = TBF_WARPS / pl.nc;
     int n;
     const TbVariant* v = tb_variants(&n);

@@ -19,6 +19,12 @@ CASES = [
     (spec("sixteen_warps_of_keys", S=512, B=1, L=1), 2, 32),
     (spec("two_rounds", S=530, B=1, L=1), 2, 32),
     (spec("three_rounds", S=1100, B=1, L=1, N=2), 1, 32),
+    (spec("first_key_of_a_second_round", S=513, B=1, L=2, r=18), 3, 40),      # two heads at a time, the last one alone
+    (spec("last_two_heads_at_a_time", S=768, B=1, L=1, r=32), 4, 64),
+    (spec("first_one_head_at_a_time", S=769, B=1, L=1, r=12), 3, 24),
+    (spec("two_rounds_three_columns", S=521, B=1, L=2, r=70), 2, 140),
+    (spec("two_rounds_six_columns", S=600, B=1, L=1, r=98), 2, 98),
+    (spec("two_rounds_short_ring", S=530, B=1, L=1, r=8), 1, 1100),           # a wide feed-forward layer leaves room for fewer weight units
     (spec("r_64", r=64), 4, 256),                          # widest of two columns per lane
     (spec("r_66", r=66), 2, 130),                          # three columns per lane; more than eight tiles: sums not cut along K
     (spec("r_96_seven_heads_of_keys", r=96, S=70), 8, 384),
