@@ -301,6 +301,10 @@ pac_status pac_sync(pac_ctx* ctx);
  * reported expiry, and the status word it set is then reported by the next pac_sync like any other
  * timeout.  The paper describes no failure handling for this path; this is the library's own contract. */
 pac_status pac_selftest_wait_expiry(pac_ctx* ctx, unsigned long long limit_ns);
+/* How the fp32-precision products u = h W_down deal `tiles` tiles of 128 rows x min(r, 128) columns and d / 64 stages each to a device of `sms`
+ * multiprocessors (host arithmetic only; f32, aligned: type of the cache, whether its rows start on 16-byte boundaries): producer teams per CTA, tiles that one CTA computes,
+ * CTAs that share each of the others, and stages per share.  For tests, which need to know that their sizes reach the forms they are about. */
+pac_status pac_selftest_rows_plan(int tiles, int d, int r, int f32, int aligned, int sms, int* teams, int* whole, int* parts, int* per);
 const char* pac_last_error(const pac_ctx* ctx);
 /* Which kernels the next train step will use (valid after adapter_init): "simt", "tensor",
  * "tensor+fused_forward" when a batch of max_batch samples runs the down-projections

@@ -27,7 +27,7 @@ EXPORTS = ["pac_create", "pac_destroy", "pac_cache_register", "pac_cache_registe
            "pac_cache_writer_create", "pac_cache_writer_store", "pac_cache_writer_close", "pac_cache_file_info", "pac_adapter_init", "pac_train_step", "pac_train_step_dev_loss", "pac_set_grad_scale", "pac_train_step_async",
            "pac_adam_step", "pac_eval_logits", "pac_gather", "pac_train_epoch", "pac_train_epoch_dev",
            "pac_param_count", "pac_get_params", "pac_set_params", "pac_get_grads", "pac_get_opt_state",
-           "pac_set_opt_state", "pac_set_option", "pac_device_buffers", "pac_params_changed", "pac_kernel_times", "pac_stream_phase_times", "pac_launch_count", "pac_sync", "pac_selftest_wait_expiry", "pac_last_error",
+           "pac_set_opt_state", "pac_set_option", "pac_device_buffers", "pac_params_changed", "pac_kernel_times", "pac_stream_phase_times", "pac_launch_count", "pac_sync", "pac_selftest_wait_expiry", "pac_selftest_rows_plan", "pac_last_error",
            "pac_kernel_path", "pac_eval_logits_static", "pac_quantize_absmax", "pac_dequantize_absmax"]
 
 
@@ -96,6 +96,7 @@ def load_library() -> C.CDLL:
         "pac_stream_phase_times": [P, C.POINTER(C.c_double), C.POINTER(LL)],
         "pac_device_buffers": [P, C.POINTER(P), C.POINTER(P)], "pac_params_changed": [P],
         "pac_selftest_wait_expiry": [P, C.c_ulonglong],
+        "pac_selftest_rows_plan": [I] * 6 + [C.POINTER(I)] * 4,
         "pac_train_step_dev_loss": [P, P, I, P], "pac_set_grad_scale": [P, F],
         "pac_cache_register_file": [P, C.c_char_p],
         "pac_cache_writer_create": [C.POINTER(P), C.c_char_p, I, LL, I, I, I, I],
@@ -352,6 +353,15 @@ class PacContext:
 
 
 STATIC_SCRATCH_BYTES = 8 << 20
+
+
+def rows_plan(tiles: int, d: int, r: int, f32: bool, aligned: bool, sms: int):
+    """(teams per CTA, whole tiles, CTAs per shared tile, stages per share) of the fp32-precision u = h W_down; host arithmetic only."""
+    out = [C.c_int() for _ in range(4)]
+    st = load_library().pac_selftest_rows_plan(tiles, d, r, int(f32), int(aligned), sms, *[C.byref(o) for o in out])
+    if st != 0:
+        raise PacError(st, "pac_selftest_rows_plan: sizes must be positive")
+    return tuple(o.value for o in out)
 
 
 def cache_file_info(path: str):

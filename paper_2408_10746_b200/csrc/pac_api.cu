@@ -2017,6 +2017,13 @@ pac_status pac_sync(pac_ctx* c) {
     return PAC_OK;
 }
 
+pac_status pac_selftest_rows_plan(int tiles, int d, int r, int f32, int aligned, int sms, int* teams, int* whole, int* parts, int* per) {
+    if (tiles < 1 || d < 1 || r < 1 || sms < 1 || !teams || !whole || !parts || !per) return PAC_ERR_INVALID_ARG;
+    const XgRowsPlan p = xg_rows_plan(tiles, (d + XG_K - 1) / XG_K, xg_tile_j(r), f32 != 0, !f32 && !aligned, sms);
+    *teams = p.teams; *whole = p.whole; *parts = p.parts; *per = p.per;
+    return PAC_OK;
+}
+
 pac_status pac_selftest_wait_expiry(pac_ctx* c, unsigned long long limit_ns) {
     NEED_CTX(c);
     if (limit_ns < 1000ull || limit_ns > 100000000ull)

@@ -10,8 +10,8 @@
 // by bringing the operands in: A comes straight from the activation cache (the gather is the address; any row length and alignment),
 // producer warps fetch it into registers, split it and store the swizzled tiles, one warp issues the MMAs.  Two teams of eight producers take turns, each with
 // a stage of its own, so that a team's loads are in flight while the other converts: in one CTA, or in two CTAs of one team each on an SM, whose starts
-// and ends then fall under each other's stages (rows of more than one wave: 2048 x 768 x 64 x 12 layers, 192 tiles: 38 -> 35 us, on a bf16 cache 34 -> 27).
-// At 2048 rows, 12 layers, d = 768, r = 64: u 35 us, dW_down 30 us (the FP32-pipe tiles before it, 8 x 4 outputs per thread: 77 and 84 us).
+// and ends then fall under each other's stages (2048 x 768 x 64 x 12 layers, u 38 -> 35 us, on a bf16 cache 34 -> 27; which form a launch takes: xg_rows_plan, xg_slices).
+// At 2048 rows, 12 layers, d = 768, r = 64: u 35 us, dW_down 29 us (the FP32-pipe tiles before it, 8 x 4 outputs per thread: 77 and 84 us).
 // Loads are what it waits for (a third of the issue slots are used); row addresses are therefore formed once per stage (tn) or once per kernel
 // (rows).  Prefetching the stage after next into L2 made the step 8 % slower.
 // Every output is summed in a fixed order.
@@ -384,9 +384,9 @@ xgemm_kernel(const __grid_constant__ XgJobs<AL> J, int K, int k_slice, int accs_
     if (warp == PRODUCERS) tmem_dealloc(tmem_base, tmem_cols);
 }
 
-template <bool TN, int TEAMS, class AL>
+template <bool TN, int GB, int TEAMS, class AL>
 inline cudaError_t xgemm_launch(const XgJobs<AL>& J, int K, dim3 grid, int k_slice, float* out, long long zstride, long long part_stride, const XgTail& tail, unsigned* status, cudaStream_t stream, const ArgIds& arg, int* ids_out) {
-    const auto kernel = J.tile_j <= 64 ? xgemm_kernel<TN, 2, TEAMS, AL> : xgemm_kernel<TN, 4, TEAMS, AL>;
+    const auto kernel = xgemm_kernel<TN, GB, TEAMS, AL>;
     const size_t smem = xg_smem<AL>(J.tile_j, TEAMS);
     cudaError_t e = smem_opt_in((const void*)kernel, smem);
     if (e != cudaSuccess) return e;
@@ -403,26 +403,44 @@ template <class AL>
 inline cudaError_t xgemm_launch_tn(const XgJobs<AL>& J, int K, int Z, int slices, float* out, long long zstride, long long part_stride, unsigned* status, cudaStream_t stream) {
     const int k_slice = ((K + slices - 1) / slices + XG_K - 1) / XG_K * XG_K, longest = K < k_slice ? K : k_slice;
     const dim3 grid((unsigned)J.first[J.n], (unsigned)Z, (unsigned)slices);
-    if (AL::cache_rows && J.tile_j <= 64 && xg_one_team(J.tile_j, (longest + XG_K - 1) / XG_K))
-        return xgemm_launch<true, 1>(J, K, grid, k_slice, out, zstride, part_stride, XgTail{}, status, stream, ArgIds{}, nullptr);
-    return xgemm_launch<true, 2>(J, K, grid, k_slice, out, zstride, part_stride, XgTail{}, status, stream, ArgIds{}, nullptr);
+    if constexpr (AL::cache_rows)
+        if (J.tile_j <= 64 && xg_one_team(J.tile_j, (longest + XG_K - 1) / XG_K))
+            return xgemm_launch<true, 2, 1>(J, K, grid, k_slice, out, zstride, part_stride, XgTail{}, status, stream, ArgIds{}, nullptr);
+    return J.tile_j <= 64 ? xgemm_launch<true, 2, 2>(J, K, grid, k_slice, out, zstride, part_stride, XgTail{}, status, stream, ArgIds{}, nullptr)
+                          : xgemm_launch<true, 4, 2>(J, K, grid, k_slice, out, zstride, part_stride, XgTail{}, status, stream, ArgIds{}, nullptr);
 }
-// ws: 2 sms tiles of 128 x tile_j floats, cnt: 2 sms words of zero.  A tile of the last wave is shared when that takes four or more stages off its CTA
-// (the exchange costs about as much as three).
+// How `total` tiles of `stages` stages over the rows of the cache are dealt out (f32: rows of three terms; odd_bf16: bf16 rows that start off a 16-byte boundary, which producers
+// load value by value).  A CTA per team from one wave on, except where its stages outweigh what its starts and ends save: a team alone on an SM does not hide its
+// loads, so in the first quarter of a second wave two teams to a tile, and the few tiles beyond the first wave shared by all SMs, are faster when reductions are long, and for
+// rows loaded value by value from some length on always.  Evaluation at r = 64, one team / two (us), tiles x stages:
+//   fp32    160 x 8  32.6 / 38.7   192 x 8  33.1 / 39.9   160 x 12 41.4 / 44.0   160 x 16 51.1 / 48.7   192 x 16 51.7 / 51.9 (24 layers 53.8 / 60.1)   256 x 16 53.3 / 56.0   480 x 16 96.9 / 103.3
+//   fp32, r = 16, and off a boundary at r = 64:   160 x 16 45.4 / 40.3, 66.0 / 57.8   192 x 16 45.7 / 43.9, 66.9 / 62.8   256 x 16 47.8 / 49.9, 68.5 / 72.6
+//   bf16    160 x 16 37.6 / 43.6   256 x 16 41.4 / 48.8   320 x 16 61.3 / 64.6
+//   bf16 off a boundary   160 x 4 27.1 / 31.6   160 x 9 46.9 / 41.7   256 x 9 48.2 / 48.2   160 x 13 68.1 / 51.3   384 x 13 107 / 92   384 x 16 123 / 110
+// A tile of the last wave is shared when that takes four or more stages off its CTA (the exchange costs about as much as three).
+struct XgRowsPlan { int teams, whole, parts, per; };      // per: stages of a part
+inline XgRowsPlan xg_rows_plan(int total, int stages, int tile_j, bool f32, bool odd_bf16, int sms) {
+    const bool one = total > sms && xg_one_team(tile_j, stages) && !(odd_bf16 && stages >= 8) && !(f32 && stages > 12 && 4LL * total <= 5LL * sms);
+    const int slots = one ? 2 * sms : sms, rest = total % slots;
+    XgRowsPlan p{one ? 1 : 2, total, 1, stages};
+    if (rest > 0) {
+        const int per = (stages + slots / rest - 1) / (slots / rest);
+        if (stages - per >= 4) p = XgRowsPlan{p.teams, total - rest, (stages + per - 1) / per, per};
+    }
+    return p;
+}
+// ws: 2 sms tiles of 128 x tile_j floats, cnt: 2 sms words of zero.
 template <class AL>
 inline cudaError_t xgemm_launch_rows(const XgJobs<AL>& J, int K, int Z, int sms, float* out, long long zstride, float* ws, unsigned* cnt, unsigned* status, cudaStream_t stream, const ArgIds& arg, int* ids_out) {
     const int total = J.first[J.n] * Z, stages = (K + XG_K - 1) / XG_K;
-    const bool one = total > sms && xg_one_team(J.tile_j, stages);
-    if (one) sms *= 2;                              // CTAs at a time
-    const int rest = total % sms;
-    XgTail tail{total, 1, ws, cnt};
-    int per = stages;
-    if (rest > 0) {
-        per = (stages + sms / rest - 1) / (sms / rest);
-        if (stages - per >= 4) { tail.whole = total - rest; tail.parts = (stages + per - 1) / per; }
-    }
-    const dim3 grid((unsigned)(tail.whole + (total - tail.whole) * tail.parts));
-    return one ? xgemm_launch<false, 1>(J, K, grid, per * XG_K, out, zstride, 0, tail, status, stream, arg, ids_out) : xgemm_launch<false, 2>(J, K, grid, per * XG_K, out, zstride, 0, tail, status, stream, arg, ids_out);
+    const bool f32 = XgTerms<typename AL::elem>::n == 3;
+    const XgRowsPlan p = xg_rows_plan(total, stages, J.tile_j, f32, !f32 && !J.A[0].vec, sms);
+    const XgTail tail{p.whole, p.parts, ws, cnt};
+    const dim3 grid((unsigned)(p.whole + (total - p.whole) * p.parts));
+    const int k_slice = p.per * XG_K;
+    if (J.tile_j <= 64)
+        return p.teams == 1 ? xgemm_launch<false, 2, 1>(J, K, grid, k_slice, out, zstride, 0, tail, status, stream, arg, ids_out) : xgemm_launch<false, 2, 2>(J, K, grid, k_slice, out, zstride, 0, tail, status, stream, arg, ids_out);
+    return p.teams == 1 ? xgemm_launch<false, 4, 1>(J, K, grid, k_slice, out, zstride, 0, tail, status, stream, arg, ids_out) : xgemm_launch<false, 4, 2>(J, K, grid, k_slice, out, zstride, 0, tail, status, stream, arg, ids_out);
 }
 
 // Columns per tile for an output N wide, tiles of equal width.
