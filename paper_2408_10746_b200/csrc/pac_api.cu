@@ -259,9 +259,10 @@ pac_status dmalloc(pac_ctx* c, T** p, long long n) {
 bool use_tensor(const pac_ctx* c) { return c->tensor_ok && !c->force_simt; }
 WdShadow wd_shadow(const pac_ctx* c) { return WdShadow{c->sc.wdT}; }
 pac_status adam_enqueue(pac_ctx* c, const pac_adamw* hp);
-pac_status down_projection(pac_ctx* c, const int* d_ids, int B);
+pac_status down_projection(pac_ctx* c, const int* d_ids, int B, bool train);
 pac_status dw_down(pac_ctx* c, const int* d_ids, int B, bool reduce_splits);
 ArgIds arg_ids(const pac_ctx* c, int B);
+bool use_fused_cls(const pac_ctx* c);
 
 inline unsigned cdiv(long long a, long long b) { return (unsigned)((a + b - 1) / b); }
 
@@ -388,13 +389,21 @@ pac_status stage_ids(pac_ctx* c, const int* ids, int B) {
 // ---------------------------------------------------------------------------
 // Forward: u_l for every layer, the chain, and the head.  ids are on the device.
 // ---------------------------------------------------------------------------
+// Whether a product over the rows of the cache follows a head kernel (of this step or the one before) that filled the shared memory of many SMs (`apart` of xgemm_launch).
+// L1 and shared memory are split at 196 KB and 228 KB: 24 layers at r = 64, S = 128 take the latter, 22 the former, which costs nothing.  With the heads of 32 SMs (B = 8)
+// the overlap is still the better in an evaluation (53.7 us for 54.8), with those of 52 it is not (83.9 for 79.7); a step, where the head has two products behind it, gains from 32 on
+// (136.8 -> 118.9, d = 512 79.8 -> 75.5).  bf16 rows loaded value by value gain nothing (384 tiles of 9 stages: 75.9 us, apart 77.1).
+template <class AL>
+bool behind_large_head(const pac_ctx* c, int B, bool train, const AL& A) {
+    return use_fused_cls(c) && !c->tb.on && c->mplan.smem > 195 * 1024 && (train ? 5LL : 3LL) * B * c->mplan.G > c->sms && (sizeof(typename AL::elem) == 4 || A.vec);
+}
 // out[z] = rows(z) W[z] at fp32 precision.
 template <class AL>
-pac_status xgemm_rows(pac_ctx* c, int M, int N, int K, int Z, const AL& A, const XgRows& W, float* out, long long zstride) {
+pac_status xgemm_rows(pac_ctx* c, int M, int N, int K, int Z, const AL& A, const XgRows& W, float* out, long long zstride, bool train) {
     XgJobs<AL> J;
     J.tile_j = xg_tile_j(N);
     J.add(A, M, W, N, 0);
-    cudaError_t e = xgemm_launch_rows(J, K, Z, c->sms, out, zstride, c->sc.xg_ws, c->sc.xg_cnt, c->status, c->stream, arg_ids(c, M / c->dm.S), c->sc.ids);
+    cudaError_t e = xgemm_launch_rows(J, K, Z, c->sms, out, zstride, c->sc.xg_ws, c->sc.xg_cnt, c->status, c->stream, arg_ids(c, M / c->dm.S), c->sc.ids, behind_large_head(c, M / c->dm.S, train, A));
     c->launches++;
     if (e != cudaSuccess) return fail(c, PAC_ERR_CUDA, "product kernel launch failed: %s", cudaGetErrorString(e));
     return PAC_OK;
@@ -402,7 +411,7 @@ pac_status xgemm_rows(pac_ctx* c, int M, int N, int K, int Z, const AL& A, const
 // The jobs' A^T B over M rows for all Z layers, `slices` row slices (partial sums part_stride apart when more than one).
 template <class AL>
 pac_status xgemm_tn(pac_ctx* c, const XgJobs<AL>& J, int M, int Z, int slices, float* out, long long zstride, long long part_stride) {
-    cudaError_t e = xgemm_launch_tn(J, M, Z, slices, out, zstride, part_stride, c->status, c->stream);
+    cudaError_t e = xgemm_launch_tn(J, M, Z, slices, out, zstride, part_stride, c->status, c->stream, AL::cache_rows && behind_large_head(c, M / c->dm.S, true, J.A[0]));
     c->launches++;
     if (e != cudaSuccess) return fail(c, PAC_ERR_CUDA, "product kernel launch failed: %s", cudaGetErrorString(e));
     return PAC_OK;
@@ -418,10 +427,10 @@ XgCacheRows<T> xg_cache_rows(const pac_ctx* c, const int* d_ids) {
 }
 
 template <typename T>
-pac_status down_projection_simt(pac_ctx* c, const int* d_ids, int B) {
+pac_status down_projection_simt(pac_ctx* c, const int* d_ids, int B, bool train) {
     const Dims& dm = c->dm;
     return xgemm_rows(c, B * dm.S, dm.r, dm.d, dm.L, xg_cache_rows<T>(c, d_ids), xg_rows(c->params + c->lay.w_down, (long long)dm.d * dm.r, dm.r),
-                      c->sc.u, (long long)c->max_rows * dm.r);
+                      c->sc.u, (long long)c->max_rows * dm.r, train);
 }
 
 pac_status head_matrix_enqueue(pac_ctx* c, int B, bool behind);
@@ -472,7 +481,7 @@ pac_status forward(pac_ctx* c, const int* d_ids, int B, bool train, float* d_log
     Scratch& sc = c->sc;
     pac_status st = PAC_OK;
     if (use_tensor(c) && plain_head_ok(c, B) && (st = head_matrix_enqueue(c, B, false)) != PAC_OK) return st;
-    st = down_projection(c, d_ids, B);
+    st = down_projection(c, d_ids, B, train);
     if (st != PAC_OK) return st;
     if (!use_tensor(c) && plain_head_ok(c, B) && (st = head_matrix_enqueue(c, B, true)) != PAC_OK) return st;
     const float* lam = c->params + c->lay.lam;
@@ -793,7 +802,7 @@ pac_status tb_forward(pac_ctx* c, const int* d_ids, int B, bool train, float* d_
         tb_pack_kernel<<<dim3(cdiv(t.pk.tiles(), 8), (unsigned)dm.L), 256, 0, st>>>(c->params + c->lay.body, bl.per_layer, bl, t.pk, reinterpret_cast<unsigned char*>(t.packed));
         LAUNCH_CHECK(c);
     }
-    TB_OK(down_projection(c, d_ids, B));
+    TB_OK(down_projection(c, d_ids, B, train));
     if (plain_head_ok(c, B)) TB_OK(head_matrix_enqueue(c, B, true));
     const float* lam = c->params + c->lay.lam;
     const unsigned rows_grid = cdiv(M, 8), heads_grid = cdiv((long long)B * t.H * dm.S, 128);
@@ -927,14 +936,14 @@ int cls_cluster_size(const pac_ctx* c, int B) {
     return use_chain_fwd(c, B) ? c->pplan.G : use_fused_fwd(c, B) ? fused_plan(c, B)->mp.G : c->mplan.G;
 }
 
-pac_status down_projection(pac_ctx* c, const int* d_ids, int B) {
+pac_status down_projection(pac_ctx* c, const int* d_ids, int B, bool train) {
     pac_status st;
     time_mark(c, 0, false);
     if (use_tensor(c)) {
         st = tensor_down_projection(c->tplan, c->stream, d_ids, B, c->sc.u, c->status, &c->launches, next_stamp(c, 0));
         if (st != PAC_OK) return fail(c, st, "tensor-core down-projection launch failed: %s", tensor_last_error());
     } else {
-        st = c->dtype == PAC_F32 ? down_projection_simt<float>(c, d_ids, B) : down_projection_simt<bf16>(c, d_ids, B);
+        st = c->dtype == PAC_F32 ? down_projection_simt<float>(c, d_ids, B, train) : down_projection_simt<bf16>(c, d_ids, B, train);
         if (st != PAC_OK) return st;
     }
     time_mark(c, 0, true);
@@ -1078,7 +1087,7 @@ pac_status cls_forward_enqueue(pac_ctx* c, const int* d_ids, int B, bool train, 
         return st;
     }
     if (use_tensor(c) && (st = head_matrix_enqueue(c, B, false)) != PAC_OK) return st;
-    if ((st = down_projection(c, d_ids, B)) != PAC_OK) return st;
+    if ((st = down_projection(c, d_ids, B, train)) != PAC_OK) return st;
     if (!use_tensor(c) && (st = head_matrix_enqueue(c, B, true)) != PAC_OK) return st;
     time_mark(c, 1, false);
     st = mid_enqueue(c, d_ids, B, train, d_logits_out);

@@ -384,8 +384,11 @@ xgemm_kernel(const __grid_constant__ XgJobs<AL> J, int K, int k_slice, int accs_
     if (warp == PRODUCERS) tmem_dealloc(tmem_base, tmem_cols);
 }
 
+// apart: not launched programmatically.  An SM keeps its split of L1 and shared memory until it drains, and between programmatic launches it does not: behind a head kernel of nearly all
+// the shared memory a CTA of this kernel ran with 28 KB of L1 instead of 92 (37 -> 41 to 50 us each; 384 tiles of 16 stages at r = 64: evaluation 95.8 us, launched apart 83.1, step
+// 202.9 -> 174.2; 480 tiles: 114.4 -> 92.3, 238 -> 197).  Where the head kernel leaves more of it the overlap is worth 1 to 3 us.
 template <bool TN, int GB, int TEAMS, class AL>
-inline cudaError_t xgemm_launch(const XgJobs<AL>& J, int K, dim3 grid, int k_slice, float* out, long long zstride, long long part_stride, const XgTail& tail, unsigned* status, cudaStream_t stream, const ArgIds& arg, int* ids_out) {
+inline cudaError_t xgemm_launch(const XgJobs<AL>& J, int K, dim3 grid, int k_slice, float* out, long long zstride, long long part_stride, const XgTail& tail, unsigned* status, cudaStream_t stream, const ArgIds& arg, int* ids_out, bool apart) {
     const auto kernel = xgemm_kernel<TN, GB, TEAMS, AL>;
     const size_t smem = xg_smem<AL>(J.tile_j, TEAMS);
     cudaError_t e = smem_opt_in((const void*)kernel, smem);
@@ -393,6 +396,7 @@ inline cudaError_t xgemm_launch(const XgJobs<AL>& J, int K, dim3 grid, int k_sli
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[1];
     pdl_launch_config(&cfg, attr, grid, dim3(xg_threads(TEAMS)), smem, stream);
+    if (apart) cfg.numAttrs = 0;
     const int longest = !TN && tail.whole > 0 ? K : K < k_slice ? K : k_slice;      // a CTA's share of the reduction
     const int accs = xg_accs(J.tile_j, (longest + XG_K - 1) / XG_K * (XG_K / 16));
     return cudaLaunchKernelEx(&cfg, kernel, J, K, k_slice, accs, out, zstride, part_stride, tail, status, arg, ids_out);
@@ -400,14 +404,14 @@ inline cudaError_t xgemm_launch(const XgJobs<AL>& J, int K, dim3 grid, int k_sli
 // Whether the accumulators of two CTAs fit beside each other.
 inline bool xg_one_team(int tile_j, int stages) { return (xg_accs(tile_j, stages * (XG_K / 16)) + 1) * tile_j <= 256; }
 template <class AL>
-inline cudaError_t xgemm_launch_tn(const XgJobs<AL>& J, int K, int Z, int slices, float* out, long long zstride, long long part_stride, unsigned* status, cudaStream_t stream) {
+inline cudaError_t xgemm_launch_tn(const XgJobs<AL>& J, int K, int Z, int slices, float* out, long long zstride, long long part_stride, unsigned* status, cudaStream_t stream, bool apart) {
     const int k_slice = ((K + slices - 1) / slices + XG_K - 1) / XG_K * XG_K, longest = K < k_slice ? K : k_slice;
     const dim3 grid((unsigned)J.first[J.n], (unsigned)Z, (unsigned)slices);
     if constexpr (AL::cache_rows)
         if (J.tile_j <= 64 && xg_one_team(J.tile_j, (longest + XG_K - 1) / XG_K))
-            return xgemm_launch<true, 2, 1>(J, K, grid, k_slice, out, zstride, part_stride, XgTail{}, status, stream, ArgIds{}, nullptr);
-    return J.tile_j <= 64 ? xgemm_launch<true, 2, 2>(J, K, grid, k_slice, out, zstride, part_stride, XgTail{}, status, stream, ArgIds{}, nullptr)
-                          : xgemm_launch<true, 4, 2>(J, K, grid, k_slice, out, zstride, part_stride, XgTail{}, status, stream, ArgIds{}, nullptr);
+            return xgemm_launch<true, 2, 1>(J, K, grid, k_slice, out, zstride, part_stride, XgTail{}, status, stream, ArgIds{}, nullptr, apart);
+    return J.tile_j <= 64 ? xgemm_launch<true, 2, 2>(J, K, grid, k_slice, out, zstride, part_stride, XgTail{}, status, stream, ArgIds{}, nullptr, apart)
+                          : xgemm_launch<true, 4, 2>(J, K, grid, k_slice, out, zstride, part_stride, XgTail{}, status, stream, ArgIds{}, nullptr, apart);
 }
 // How `total` tiles of `stages` stages over the rows of the cache are dealt out (f32: rows of three terms; odd_bf16: bf16 rows that start off a 16-byte boundary, which producers
 // load value by value).  A CTA per team from one wave on, except where its stages outweigh what its starts and ends save: a team alone on an SM does not hide its
@@ -431,7 +435,7 @@ inline XgRowsPlan xg_rows_plan(int total, int stages, int tile_j, bool f32, bool
 }
 // ws: 2 sms tiles of 128 x tile_j floats, cnt: 2 sms words of zero.
 template <class AL>
-inline cudaError_t xgemm_launch_rows(const XgJobs<AL>& J, int K, int Z, int sms, float* out, long long zstride, float* ws, unsigned* cnt, unsigned* status, cudaStream_t stream, const ArgIds& arg, int* ids_out) {
+inline cudaError_t xgemm_launch_rows(const XgJobs<AL>& J, int K, int Z, int sms, float* out, long long zstride, float* ws, unsigned* cnt, unsigned* status, cudaStream_t stream, const ArgIds& arg, int* ids_out, bool apart) {
     const int total = J.first[J.n] * Z, stages = (K + XG_K - 1) / XG_K;
     const bool f32 = XgTerms<typename AL::elem>::n == 3;
     const XgRowsPlan p = xg_rows_plan(total, stages, J.tile_j, f32, !f32 && !J.A[0].vec, sms);
@@ -439,8 +443,8 @@ inline cudaError_t xgemm_launch_rows(const XgJobs<AL>& J, int K, int Z, int sms,
     const dim3 grid((unsigned)(p.whole + (total - p.whole) * p.parts));
     const int k_slice = p.per * XG_K;
     if (J.tile_j <= 64)
-        return p.teams == 1 ? xgemm_launch<false, 2, 1>(J, K, grid, k_slice, out, zstride, 0, tail, status, stream, arg, ids_out) : xgemm_launch<false, 2, 2>(J, K, grid, k_slice, out, zstride, 0, tail, status, stream, arg, ids_out);
-    return p.teams == 1 ? xgemm_launch<false, 4, 1>(J, K, grid, k_slice, out, zstride, 0, tail, status, stream, arg, ids_out) : xgemm_launch<false, 4, 2>(J, K, grid, k_slice, out, zstride, 0, tail, status, stream, arg, ids_out);
+        return p.teams == 1 ? xgemm_launch<false, 2, 1>(J, K, grid, k_slice, out, zstride, 0, tail, status, stream, arg, ids_out, apart) : xgemm_launch<false, 2, 2>(J, K, grid, k_slice, out, zstride, 0, tail, status, stream, arg, ids_out, apart);
+    return p.teams == 1 ? xgemm_launch<false, 4, 1>(J, K, grid, k_slice, out, zstride, 0, tail, status, stream, arg, ids_out, apart) : xgemm_launch<false, 4, 2>(J, K, grid, k_slice, out, zstride, 0, tail, status, stream, arg, ids_out, apart);
 }
 
 // Columns per tile for an output N wide, tiles of equal width.
