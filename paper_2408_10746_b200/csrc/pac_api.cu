@@ -410,7 +410,7 @@ pac_status xgemm_rows(pac_ctx* c, int M, int N, int K, int Z, const AL& A, const
 }
 // The jobs' A^T B over M rows for all Z layers, `slices` row slices (partial sums part_stride apart when more than one).
 template <class AL>
-pac_status xgemm_tn(pac_ctx* c, const XgJobs<AL>& J, int M, int Z, int slices, float* out, long long zstride, long long part_stride) {
+pac_status xgemm_tn(pac_ctx* c, const XgJobs<AL>& J, int M, int Z, const XgSlices& slices, float* out, long long zstride, long long part_stride) {
     cudaError_t e = xgemm_launch_tn(J, M, Z, slices, out, zstride, part_stride, c->status, c->stream, AL::cache_rows && behind_large_head(c, M / c->dm.S, true, J.A[0]));
     c->launches++;
     if (e != cudaSuccess) return fail(c, PAC_ERR_CUDA, "product kernel launch failed: %s", cudaGetErrorString(e));
@@ -555,8 +555,8 @@ pac_status forward(pac_ctx* c, const int* d_ids, int B, bool train, float* d_log
 
 // Tiles of the plain path's dW_down, and its row slices (partial sums in sc.dw_spart when more than one).
 long long dw_simt_tiles(const Dims& dm) { return (long long)dm.L * cdiv(dm.d, XG_TILE) * cdiv(dm.r, xg_tile_j(dm.r)); }
-int dw_simt_slices(const pac_ctx* c, int B) {
-    return c->sc.dw_spart ? xg_slices(dw_simt_tiles(c->dm), B * c->dm.S, c->sms, c->dw_simt_max, xg_tile_j(c->dm.r)) : 1;
+XgSlices dw_simt_slices(const pac_ctx* c, int B) {
+    return xg_slices(dw_simt_tiles(c->dm), B * c->dm.S, c->sms, c->sc.dw_spart ? c->dw_simt_max : 1, xg_tile_j(c->dm.r));
 }
 
 template <typename T>
@@ -565,11 +565,11 @@ pac_status dw_down_simt(pac_ctx* c, const int* d_ids, int B, bool reduce_splits)
     XgJobs<XgCacheRows<T>> J;
     J.tile_j = xg_tile_j(dm.r);
     J.add(xg_cache_rows<T>(c, d_ids), dm.d, xg_rows(c->sc.du, (long long)c->max_rows * dm.r, dm.r), dm.r, 0);
-    const int slices = dw_simt_slices(c, B);
+    const XgSlices slices = dw_simt_slices(c, B);
     const long long ne = (long long)dm.L * dm.d * dm.r;
-    pac_status st = xgemm_tn(c, J, B * dm.S, dm.L, slices, slices > 1 ? c->sc.dw_spart : c->grads + c->lay.w_down, (long long)dm.d * dm.r, ne);
-    if (st != PAC_OK || slices == 1 || !reduce_splits) return st;
-    reduce_splits_kernel<<<cdiv(ne / 4, 256), 256, 0, c->stream>>>(c->sc.dw_spart, slices, ne, c->grads + c->lay.w_down);
+    pac_status st = xgemm_tn(c, J, B * dm.S, dm.L, slices, slices.n > 1 ? c->sc.dw_spart : c->grads + c->lay.w_down, (long long)dm.d * dm.r, ne);
+    if (st != PAC_OK || slices.n == 1 || !reduce_splits) return st;
+    reduce_splits_kernel<<<cdiv(ne / 4, 256), 256, 0, c->stream>>>(c->sc.dw_spart, slices.n, ne, c->grads + c->lay.w_down);
     LAUNCH_CHECK(c);
     return PAC_OK;
 }
@@ -622,11 +622,11 @@ pac_status backward(pac_ctx* c, const int* d_ids, int B, float* d_loss, const pa
             J.tile_j = xg_tile_j(dm.r); J.trans = 1;
             J.add(xg_rows(sc.dy, 0, dm.d), dm.d, xg_rows(aL, 0, dm.r), dm.r, 0);
             const long long ne = (long long)dm.r * dm.d;
-            const int sl = sc.lm_part && ne % 4 == 0 ? xg_slices(J.first[1], M, c->sms, LM_MAX_K_SLICES, 0) : 1;
-            pac_status ts = xgemm_tn(c, J, M, 1, sl, sl > 1 ? sc.lm_part : c->grads + c->lay.w_up, 0, ne);
+            const XgSlices sl = xg_slices(J.first[1], M, c->sms, sc.lm_part && ne % 4 == 0 ? LM_MAX_K_SLICES : 1, 0);
+            pac_status ts = xgemm_tn(c, J, M, 1, sl, sl.n > 1 ? sc.lm_part : c->grads + c->lay.w_up, 0, ne);
             if (ts != PAC_OK) return ts;
-            if (sl > 1) {
-                reduce_splits_kernel<<<cdiv(ne / 4, 256), 256, 0, c->stream>>>(sc.lm_part, sl, ne, c->grads + c->lay.w_up);
+            if (sl.n > 1) {
+                reduce_splits_kernel<<<cdiv(ne / 4, 256), 256, 0, c->stream>>>(sc.lm_part, sl.n, ne, c->grads + c->lay.w_up);
                 LAUNCH_CHECK(c);
             }
         }
@@ -782,10 +782,10 @@ pac_status tb_fused_backward(pac_ctx* c, int B) {
     J.add(xg_rows(s.o, s.sMr, r), r, xg_rows(s.dx1, s.sMr, r), r, 3 * rr);
     J.add(xg_rows(s.n2, s.sMr, r), r, xg_rows(s.dpre, s.sMf, f), f, 4 * rr);
     J.add(xg_rows(s.hid, s.sMf, f), f, xg_rows(s.da, s.sMr, r), r, 4 * rr + rf);
-    const int slices = xg_slices((long long)J.first[J.n] * L, M, c->sms, t.wg_slices, 0);
+    const XgSlices slices = xg_slices((long long)J.first[J.n] * L, M, c->sms, t.wg_slices, 0);
     pac_status st = xgemm_tn(c, J, M, L, slices, t.wg_part, per, per * L);
     if (st != PAC_OK) return st;
-    tb_reduce_slices_kernel<<<dim3(cdiv(per, 256), (unsigned)L), 256, 0, c->stream>>>(t.wg_part, slices, per * L, per, bl, gbody);
+    tb_reduce_slices_kernel<<<dim3(cdiv(per, 256), (unsigned)L), 256, 0, c->stream>>>(t.wg_part, slices.n, per * L, per, bl, gbody);
     LAUNCH_CHECK(c);
     return PAC_OK;
 }
@@ -1107,7 +1107,7 @@ pac_status finalize_enqueue(pac_ctx* c, const int* d_ids, int B, float* d_loss, 
     f.lay = c->lay; f.B = B; f.d = dm.d; f.r = dm.r; f.C = dm.C; f.L = dm.L;
     const bool tens = use_tensor(c);
     f.dw_part = tens ? sc.dw_part : sc.dw_spart;
-    f.splits = tens ? tensor_splits(c->tplan, B) : dw_simt_slices(c, B);
+    f.splits = tens ? tensor_splits(c->tplan, B) : dw_simt_slices(c, B).n;
     if (tens) { f.coef = sc.coef; f.dot_part = sc.dot_part; }
     else if (f.splits <= 1) f.splits = 0;                // already in the gradient buffer
     f.dw_elems = (long long)dm.L * dm.d * dm.r;
@@ -1539,7 +1539,7 @@ pac_status pac_adapter_init(pac_ctx* c, const pac_adapter_cfg* cfg, unsigned lon
         const long long ne = (long long)dm.L * dm.d * dm.r;
         // (a smaller batch may take more slices than the largest one)
         c->dw_simt_max = 1;
-        for (int b = 1; b <= cfg->max_batch && ne % 4 == 0; ++b) c->dw_simt_max = std::max(c->dw_simt_max, xg_slices(dw_simt_tiles(dm), b * dm.S, c->sms, 8, xg_tile_j(dm.r)));
+        for (int b = 1; b <= cfg->max_batch && ne % 4 == 0; ++b) c->dw_simt_max = std::max(c->dw_simt_max, xg_slices(dw_simt_tiles(dm), b * dm.S, c->sms, 8, xg_tile_j(dm.r)).n);
         if (c->dw_simt_max > 1) A(dmalloc(c, &s.dw_spart, ne * c->dw_simt_max));
         if (dm.d > 4 * XG_K) {              // (fewer stages are never shared)
             A(dmalloc(c, &s.xg_ws, 2LL * c->sms * XG_TILE * xg_tile_j(dm.r)));

@@ -403,13 +403,31 @@ inline cudaError_t xgemm_launch(const XgJobs<AL>& J, int K, dim3 grid, int k_sli
 }
 // Whether the accumulators of two CTAs fit beside each other.
 inline bool xg_one_team(int tile_j, int stages) { return (xg_accs(tile_j, stages * (XG_K / 16)) + 1) * tile_j <= 256; }
+// Slices of a reduction over K rows and producer teams per CTA: whole waves of CTAs, each about 2 us plus 0.6 us per stage, or 1 us where it has one team and shares its SM (measured), and
+// the slices' own traffic.  One team only over the rows of the cache (fp32 step at T5-Base widths 86.2 -> 84.4 us, smallest one 48.4 -> 47.6) and where it is the cheaper by this count: with few
+// tiles (d = 256, L = 12, r = 64) two are, 48.1 us for 51.0 at 2048 rows, 45.5 for 49.5 at 1600, 40.2 for 41.8 at 1024.  The weight products of
+// transformer bodies, whose rows lie in L2, were slower with one team, and tiles beyond 64 columns not reliably faster (steps of r = 128 216 -> 200, r = 80 96 -> 105).
+struct XgSlices { int n, teams; };
+inline XgSlices xg_slices(long long tiles, int K, int sms, int most, int tile_j) {      // tile_j: of products over the rows of the cache, else 0
+    const int stages = (K + XG_K - 1) / XG_K;
+    XgSlices best{1, 2};
+    double best_cost = 1e30;
+    for (int teams = 2; teams >= 1; --teams)
+        for (int s = 1; s <= most && s <= stages; ++s) {
+            const int each = (stages + s - 1) / s, slots = teams == 1 ? 2 * sms : sms;
+            if (teams == 1 && !(tile_j > 0 && tile_j <= 64 && xg_one_team(tile_j, each))) continue;
+            const double waves = (double)((tiles * s + slots - 1) / slots);
+            const double cost = waves * (2.0 + (teams == 1 ? 1.0 : 0.6) * each) + 0.3 * (s - 1);
+            if (cost < best_cost) { best_cost = cost; best = XgSlices{s, teams}; }
+        }
+    return best;
+}
 template <class AL>
-inline cudaError_t xgemm_launch_tn(const XgJobs<AL>& J, int K, int Z, int slices, float* out, long long zstride, long long part_stride, unsigned* status, cudaStream_t stream, bool apart) {
-    const int k_slice = ((K + slices - 1) / slices + XG_K - 1) / XG_K * XG_K, longest = K < k_slice ? K : k_slice;
-    const dim3 grid((unsigned)J.first[J.n], (unsigned)Z, (unsigned)slices);
+inline cudaError_t xgemm_launch_tn(const XgJobs<AL>& J, int K, int Z, const XgSlices& sl, float* out, long long zstride, long long part_stride, unsigned* status, cudaStream_t stream, bool apart) {
+    const int k_slice = ((K + sl.n - 1) / sl.n + XG_K - 1) / XG_K * XG_K;
+    const dim3 grid((unsigned)J.first[J.n], (unsigned)Z, (unsigned)sl.n);
     if constexpr (AL::cache_rows)
-        if (J.tile_j <= 64 && xg_one_team(J.tile_j, (longest + XG_K - 1) / XG_K))
-            return xgemm_launch<true, 2, 1>(J, K, grid, k_slice, out, zstride, part_stride, XgTail{}, status, stream, ArgIds{}, nullptr, apart);
+        if (sl.teams == 1) return xgemm_launch<true, 2, 1>(J, K, grid, k_slice, out, zstride, part_stride, XgTail{}, status, stream, ArgIds{}, nullptr, apart);
     return J.tile_j <= 64 ? xgemm_launch<true, 2, 2>(J, K, grid, k_slice, out, zstride, part_stride, XgTail{}, status, stream, ArgIds{}, nullptr, apart)
                           : xgemm_launch<true, 4, 2>(J, K, grid, k_slice, out, zstride, part_stride, XgTail{}, status, stream, ArgIds{}, nullptr, apart);
 }
@@ -451,24 +469,6 @@ inline cudaError_t xgemm_launch_rows(const XgJobs<AL>& J, int K, int Z, int sms,
 inline int xg_tile_j(int N) {
     const int tiles = (N + 127) / 128;
     return ((N + tiles - 1) / tiles + 15) / 16 * 16;
-}
-
-// Slices of a reduction over K rows: whole waves of CTAs, each about 2 us plus 0.6 us per stage, or 1 us where it has one team and shares its SM (measured), and the slices' own
-// traffic.  Over the rows of the cache a CTA per team (fp32 step at T5-Base widths 86.2 -> 84.4 us, smallest one 48.4 -> 47.6); the weight products of
-// transformer bodies, whose rows lie in L2, were slower so, and tiles beyond 64 columns not reliably faster (steps of r = 128 216 -> 200, r = 80 96 -> 105).
-inline int xg_slices(long long tiles, int K, int sms, int most, int tile_j) {      // tile_j: of products over the rows of the cache, else 0
-    const int stages = (K + XG_K - 1) / XG_K;
-    int best = 1;
-    double best_cost = 1e30;
-    for (int s = 1; s <= most && s <= stages; ++s) {
-        const int each = (stages + s - 1) / s;
-        const bool one = tile_j > 0 && tile_j <= 64 && xg_one_team(tile_j, each);
-        const int slots = one ? 2 * sms : sms;
-        const double waves = (double)((tiles * s + slots - 1) / slots);
-        const double cost = waves * (2.0 + (one ? 1.0 : 0.6) * each) + 0.3 * (s - 1);
-        if (cost < best_cost) { best_cost = cost; best = s; }
-    }
-    return best;
 }
 
 }  // namespace pac
