@@ -305,6 +305,9 @@ pac_status pac_selftest_wait_expiry(pac_ctx* ctx, unsigned long long limit_ns);
  * multiprocessors (host arithmetic only; f32, aligned: type of the cache, whether its rows start on 16-byte boundaries): producer teams per CTA, tiles that one CTA computes,
  * CTAs that share each of the others, and stages per share.  For tests, which need to know that their sizes reach the forms they are about. */
 pac_status pac_selftest_rows_plan(int tiles, int d, int r, int f32, int aligned, int sms, int* teams, int* whole, int* parts, int* per);
+/* The same for the second pass of the tensor-core path, on a device whose CTAs may have max_smem bytes of shared memory: row splits for a batch of B, stages of the
+ * ring, and whether a classifier step forms dW_down from the gates alone. */
+pac_status pac_selftest_second_pass_plan(int L, int S, int d, int r, int max_batch, int B, int sms, int max_smem, int* splits, int* stages, int* gates);
 const char* pac_last_error(const pac_ctx* ctx);
 /* Which kernels the next train step will use (valid after adapter_init): "simt", "tensor",
  * "tensor+fused_forward" when a batch of max_batch samples runs the down-projections

@@ -27,7 +27,7 @@ EXPORTS = ["pac_create", "pac_destroy", "pac_cache_register", "pac_cache_registe
            "pac_cache_writer_create", "pac_cache_writer_store", "pac_cache_writer_close", "pac_cache_file_info", "pac_adapter_init", "pac_train_step", "pac_train_step_dev_loss", "pac_set_grad_scale", "pac_train_step_async",
            "pac_adam_step", "pac_eval_logits", "pac_gather", "pac_train_epoch", "pac_train_epoch_dev",
            "pac_param_count", "pac_get_params", "pac_set_params", "pac_get_grads", "pac_get_opt_state",
-           "pac_set_opt_state", "pac_set_option", "pac_device_buffers", "pac_params_changed", "pac_kernel_times", "pac_stream_phase_times", "pac_launch_count", "pac_sync", "pac_selftest_wait_expiry", "pac_selftest_rows_plan", "pac_last_error",
+           "pac_set_opt_state", "pac_set_option", "pac_device_buffers", "pac_params_changed", "pac_kernel_times", "pac_stream_phase_times", "pac_launch_count", "pac_sync", "pac_selftest_wait_expiry", "pac_selftest_rows_plan", "pac_selftest_second_pass_plan", "pac_last_error",
            "pac_kernel_path", "pac_eval_logits_static", "pac_quantize_absmax", "pac_dequantize_absmax"]
 
 
@@ -97,6 +97,7 @@ def load_library() -> C.CDLL:
         "pac_device_buffers": [P, C.POINTER(P), C.POINTER(P)], "pac_params_changed": [P],
         "pac_selftest_wait_expiry": [P, C.c_ulonglong],
         "pac_selftest_rows_plan": [I] * 6 + [C.POINTER(I)] * 4,
+        "pac_selftest_second_pass_plan": [I] * 8 + [C.POINTER(I)] * 3,
         "pac_train_step_dev_loss": [P, P, I, P], "pac_set_grad_scale": [P, F],
         "pac_cache_register_file": [P, C.c_char_p],
         "pac_cache_writer_create": [C.POINTER(P), C.c_char_p, I, LL, I, I, I, I],
@@ -362,6 +363,15 @@ def rows_plan(tiles: int, d: int, r: int, f32: bool, aligned: bool, sms: int):
     if st != 0:
         raise PacError(st, "pac_selftest_rows_plan: sizes must be positive")
     return tuple(o.value for o in out)
+
+
+def second_pass_plan(L: int, S: int, d: int, r: int, max_batch: int, B: int, sms: int, max_smem: int):
+    """(row splits, ring stages, gates alone) of the tensor-core path's second pass; host arithmetic only."""
+    out = [C.c_int() for _ in range(3)]
+    st = load_library().pac_selftest_second_pass_plan(L, S, d, r, max_batch, B, sms, max_smem, *[C.byref(o) for o in out])
+    if st != 0:
+        raise PacError(st, "pac_selftest_second_pass_plan")
+    return out[0].value, out[1].value, bool(out[2].value)
 
 
 def cache_file_info(path: str):

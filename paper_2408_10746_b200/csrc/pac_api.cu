@@ -2033,6 +2033,17 @@ pac_status pac_selftest_rows_plan(int tiles, int d, int r, int f32, int aligned,
     return PAC_OK;
 }
 
+pac_status pac_selftest_second_pass_plan(int L, int S, int d, int r, int max_batch, int B, int sms, int max_smem, int* splits, int* stages, int* gates) {
+    if (L < 1 || S < 1 || d < 1 || r < 1 || B < 1 || B > max_batch || sms < 1 || !splits || !stages || !gates) return PAC_ERR_INVALID_ARG;
+    Dims dm{};
+    dm.N = 1; dm.L = L; dm.S = S; dm.d = d; dm.r = r;
+    BwdParams b{};
+    size_t smem = 0;
+    if (!bwd_plan(b, dm, max_batch, sms, max_smem, &smem)) return PAC_ERR_UNSUPPORTED;
+    *splits = bwd_splits(b, B); *stages = b.stages; *gates = bwd_gates(b, B, sms) ? 1 : 0;
+    return PAC_OK;
+}
+
 pac_status pac_selftest_wait_expiry(pac_ctx* c, unsigned long long limit_ns) {
     NEED_CTX(c);
     if (limit_ns < 1000ull || limit_ns > 100000000ull)

@@ -990,6 +990,57 @@ __global__ void reduce_splits_kernel(const float* __restrict__ part, int splits,
     else { out[i] = acc.x; out[i + 1] = acc.y; out[i + 2] = acc.z; out[i + 3] = acc.w; }
 }
 
+inline int pow2_at_least(int x) { int p = 32; while (p < x) p <<= 1; return p; }
+// Terms of da: dlambda, which comes from the same product as dW_down, needs two: against 64 bits it is
+// off by 1e-3 to 8e-3 with one and by 2e-6 to 2e-5 with two.  Up to r = 64 the second term's products cost nothing beside the stream.
+constexpr int DU_TERMS = 2;
+// The second pass: tiles, row splits and ring for batches of up to max_batch.  False: not enough shared memory.
+inline bool bwd_plan(BwdParams& b, const Dims& dm, int max_batch, int sms, int max_smem, size_t* smem) {
+    b.N = dm.N; b.L = dm.L; b.S = dm.S; b.d = dm.d; b.r = dm.r;
+    b.s_chunks = (dm.S + BWD_KR - 1) / BWD_KR;
+    b.r_blocks = (dm.r + 63) / 64;
+    const int n_cols = dm.r <= 128 ? 128 * b.r_blocks : (dm.r + 15) & ~15;
+    b.chunks = (dm.d >= 256 && 2 * n_cols <= 512) ? 2 : 1;
+    b.d_groups = (dm.d + 128 * b.chunks - 1) / (128 * b.chunks);
+    b.tmem_cols = pow2_at_least(b.chunks * n_cols);
+    // Row splits: enough CTAs to fill the SMs in balanced waves, few enough partial sums.  Up to r = 64 a CTA may have an SM to itself or share it with another (half
+    // the stages each): of more than one wave the second then starts and ends under the first (L = 24, d = 1024, B = 32, S = 128: 288 CTAs, step 112.8 -> 109.8 us).
+    {
+        const int stage = (b.chunks * 2 + b.r_blocks * DU_TERMS) * BWD_KR * 128 + (dm.r > 64 ? BWD_KR * dm.r : 0);
+        const int items = dm.L * b.d_groups;
+        const int row_tiles_max = max_batch * b.s_chunks;
+        double best_cost = 1e30;
+        for (int per_sm = 1; per_sm <= (dm.r <= 64 && b.tmem_cols <= 256 ? 2 : 1); ++per_sm) {
+            const int st = std::min(16, (max_smem / per_sm - 1024 - 1024 * per_sm) / stage);
+            if (st < 2) continue;
+            for (int J = 1; J <= 8 && J <= row_tiles_max; ++J) {
+                // long streams gain more from depth (B = 48, 32 tiles: 160 -> 156 us; B = 64, 43 tiles: 193 -> 195).  Where the plan takes two, a CTA each / two (us): L = 24, d = 1024, S = 128,
+                // B = 8, r = 64 65.9 / 61.5, r = 32 52.5 / 48.1; S = 30, r = 16 48.9 / 43.9; S = 256, B = 20 146 / 143, B = 32 205 / 206; L = 20, d = 512, S = 128, B = 20 56.3 / 52.3,
+                // S = 30, r = 16, B = 32 52.7 / 46.8; L = 32, d = 1024, S = 128, r = 32, B = 32 120 / 117
+                if (per_sm == 2 && row_tiles_max > 36 * J) continue;
+                const double waves = (double)items * J / (sms * per_sm);
+                const double cost = std::ceil(waves) / waves + 0.03 * (J - 1) + 0.01 * (std::ceil(waves) - 1);
+                if (cost < best_cost - 1e-9) { best_cost = cost; b.splits = J; b.stages = st; }
+            }
+        }
+        if (best_cost == 1e30) return false;
+        *smem = (size_t)b.stages * stage + 1024;
+    }
+    return true;
+}
+inline int bwd_splits(const BwdParams& b, int B) { return std::min(b.splits, B * b.s_chunks); }
+// Whether dw_down_gates_kernel takes a batch of B samples with a da_L each.
+// Three and more 64-token tiles to a sample: the sums of shorter samples are read too often (step at B = 64, L = 24, d = 1024, r = 128, two terms / gates alone:
+// S = 64 236 / 266 us, 128 325 / 334; on another box, S = 129 332 / 335, 160 339 / 337, 192 360 / 350, 224 391 / 379, 256 406 / 396, 300 563 / 533;
+// r = 112: 409 / 406, 416 / 398, 435 / 428, 485 / 463, 493 / 481, 642 / 590; r = 96: S = 129 315 / 309, 192 336 / 321, 256 408 / 365; r = 80: 365 / 355, 419 / 388, 475 / 427).
+// The eighteen warps of the gates kernel and its sums per sample cost a start and an end that short streams do not earn back: not below three tiles to a CTA (three steps of an epoch at
+// B = 2, L = 7, d = 768, S = 160, one tile: r = 80 110 us for 115, r = 96 120 for 126, r = 128 132 for 140), nor in several waves of short CTAs where two terms are narrow (B = 8, L = 24,
+// d = 1024, 288 CTAs of 8 tiles, S = 160: r = 80 266 for 272, r = 96 294 for 302, but r = 128 359 for 354).
+inline bool bwd_gates(const BwdParams& b, int B, int sms) {
+    const int J = bwd_splits(b, B), ctas = b.L * b.d_groups * J;
+    return b.r > 64 && b.r <= 128 && b.S > 2 * BWD_KR && B * b.s_chunks >= J * (b.r <= 96 && ctas > sms ? 24 : 3);
+}
+
 // ---------------------------------------------------------------------------
 // Host side
 // ---------------------------------------------------------------------------
@@ -1002,7 +1053,6 @@ struct TensorPlan {
     BwdParams bp{};
     size_t smem_fwd = 0, smem_bwd = 0;
     int max_smem = 0;
-    bool gates = false;            // dW_down by dw_down_gates_kernel where da_L is one vector per sample
     long long dw_elems = 0;
 };
 
@@ -1060,7 +1110,6 @@ inline bool make_map(CUtensorMap* map, const void* base, int rank, const cuuint6
     return true;
 }
 
-inline int pow2_at_least(int x) { int p = 32; while (p < x) p <<= 1; return p; }
 
 // wdT: [L][2][d][r] bf16 hi/lo shadow of W_down.  *part_floats receives the
 // size of the split-partial buffer dW needs (0 when no split is used).
@@ -1077,13 +1126,6 @@ inline pac_status tensor_plan_create(TensorPlan& tp, int device, const bf16* cac
     tp.max_smem = max_smem;
     const long long max_rows = (long long)max_batch * dm.S;
     const int r_pad = (dm.r + 15) & ~15;
-    // Three and more 64-token tiles to a sample: the sums of shorter samples are read too often (step at B = 64, L = 24, d = 1024, r = 128, two terms / gates alone:
-    // S = 64 236 / 266 us, 128 325 / 334, 140 369 / 353, 192 393 / 382, 256 489 / 445).
-    tp.gates = dm.r > 64 && dm.r <= 128 && dm.S > 2 * BWD_KR;
-    // Terms of da: dlambda, which comes from the same product as dW_down, needs two: against 64 bits it is
-    // off by 1e-3 to 8e-3 with one and by 2e-6 to 2e-5 with two.  Up to r = 64 the second term's products cost nothing beside the stream.
-    constexpr int dt = 2;
-
     // ---- tensor maps ----
     {
         cuuint64_t dims[4] = {(cuuint64_t)dm.d, (cuuint64_t)dm.S, (cuuint64_t)dm.L, (cuuint64_t)dm.N};
@@ -1117,37 +1159,9 @@ inline pac_status tensor_plan_create(TensorPlan& tp, int device, const bf16* cac
     }
     f.layer_stride = max_rows * dm.r;
 
-    // ---- backward plan ----
-    BwdParams& b = tp.bp;
-    b.N = dm.N; b.L = dm.L; b.S = dm.S; b.d = dm.d; b.r = dm.r;
-    b.s_chunks = (dm.S + BWD_KR - 1) / BWD_KR;
-    b.r_blocks = (dm.r + 63) / 64;
-    const int n_cols = dm.r <= 128 ? 128 * b.r_blocks : r_pad;
-    b.chunks = (dm.d >= 256 && 2 * n_cols <= 512) ? 2 : 1;
-    b.d_groups = (dm.d + 128 * b.chunks - 1) / (128 * b.chunks);
-    b.tmem_cols = pow2_at_least(b.chunks * n_cols);
-    // Row splits: enough CTAs to fill the SMs in balanced waves, few enough partial sums.  Up to r = 64 a CTA may have an SM to itself or share it with another (half
-    // the stages each): of more than one wave the second then starts and ends under the first (L = 24, d = 1024, B = 32, S = 128: 288 CTAs, step 112.8 -> 109.8 us).
-    {
-        const int stage = (b.chunks * 2 + b.r_blocks * dt) * BWD_KR * 128 + (dm.r > 64 ? BWD_KR * dm.r : 0);
-        const int items = dm.L * b.d_groups;
-        const int row_tiles_max = max_batch * b.s_chunks;
-        double best_cost = 1e30;
-        for (int per_sm = 1; per_sm <= (dm.r <= 64 && b.tmem_cols <= 256 ? 2 : 1); ++per_sm) {
-            const int st = std::min(16, (max_smem / per_sm - 1024 - 1024 * per_sm) / stage);
-            if (st < 2) continue;
-            for (int J = 1; J <= 8 && J <= row_tiles_max; ++J) {
-                if (per_sm == 2 && row_tiles_max > 36 * J) continue;      // long streams gain more from depth (B = 48, 32 tiles: 160 -> 156 us; B = 64, 43 tiles: 193 -> 195)
-                const double waves = (double)items * J / (tp.sms * per_sm);
-                const double cost = std::ceil(waves) / waves + 0.03 * (J - 1) + 0.01 * (std::ceil(waves) - 1);
-                if (cost < best_cost - 1e-9) { best_cost = cost; b.splits = J; b.stages = st; }
-            }
-        }
-        if (best_cost == 1e30) { tensor_err() = "not enough shared memory for the backward pipeline"; return PAC_ERR_UNSUPPORTED; }
-        tp.smem_bwd = (size_t)b.stages * stage + 1024;
-    }
+    if (!bwd_plan(tp.bp, dm, max_batch, tp.sms, max_smem, &tp.smem_bwd)) { tensor_err() = "not enough shared memory for the backward pipeline"; return PAC_ERR_UNSUPPORTED; }
     tp.dw_elems = (long long)dm.L * dm.d * dm.r;
-    *part_floats = tp.dw_elems * b.splits;
+    *part_floats = tp.dw_elems * tp.bp.splits;
 
     if (smem_opt_in((const void*)down_fwd_tc_kernel, tp.smem_fwd) != cudaSuccess) {
         tensor_err() = "cudaFuncSetAttribute(MaxDynamicSharedMemorySize) failed";
@@ -1176,11 +1190,7 @@ inline pac_status tensor_down_projection(TensorPlan& tp, cudaStream_t stream, co
 }
 
 // Row splits used for a batch of B samples (the partial sums the caller has to add up).
-inline int tensor_splits(const TensorPlan& tp, int B) {
-    int J = tp.bp.splits;
-    if (J > B * tp.bp.s_chunks) J = B * tp.bp.s_chunks;
-    return J;
-}
+inline int tensor_splits(const TensorPlan& tp, int B) { return bwd_splits(tp.bp, B); }
 
 // What the second pass builds du from (BwdParams).
 struct DuGen { const uint8_t* tc; const bf16* da; long long da_term, da_sample; int da_token; };
@@ -1198,7 +1208,7 @@ inline pac_status tensor_dw_down(TensorPlan& tp, cudaStream_t stream, const int*
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[1];
     pdl_launch_config(&cfg, attr, dim3((unsigned)grid), dim3(DW_THREADS), tp.smem_bwd, stream);
-    if (tp.gates && p.da_token == 0) {
+    if (p.da_token == 0 && bwd_gates(tp.bp, B, tp.sms)) {
         const int stage = (p.chunks + 1) * 2 * BWD_KR * 128 + BWD_KR * p.r;
         p.stages = std::min(16, (tp.max_smem - 8192) / stage);
         const size_t smem = (size_t)p.stages * stage + 1024;

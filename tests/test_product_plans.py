@@ -1,8 +1,9 @@
-"""How the tiles of the fp32-precision u = h W_down are dealt to CTAs: every stage of every tile is taken exactly once and the workspace suffices, and the
-sizes of the numeric tests reach the forms that they are about."""
+"""How the tiles of the fp32-precision u = h W_down are dealt to CTAs: every stage of every tile is taken exactly once and the workspace suffices; and the sizes
+of the numeric tests of both cache passes reach the forms that they are about."""
 import pytest
 
-from paper_2408_10746_b200.binding import rows_plan
+from paper_2408_10746_b200.binding import rows_plan, second_pass_plan
+from tests.test_gate_products_gpu import LONG, gates_of
 from tests.test_plain_products_gpu import PLANS, plan_of
 
 SMS = 148
@@ -40,3 +41,12 @@ def test_plans_cover_every_stage_once(f32, aligned):
 def test_sizes_reach_their_forms(sp, teams, mixed):
     got, whole, parts, _ = plan_of(sp, SMS)
     assert got == teams and (whole > 0 and parts > 1) == mixed
+
+
+def test_gates_alone_only_where_streams_are_long():
+    assert all(gates_of(sp, SMS) for sp in LONG)
+    for r, S, B, L, d, want in [(128, 256, 64, 24, 1024, True), (64, 256, 64, 24, 1024, False), (144, 256, 64, 24, 1024, False), (128, 128, 64, 24, 1024, False),
+                                (96, 129, 2, 7, 768, False), (96, 160, 4, 12, 768, True), (96, 160, 8, 24, 1024, False), (112, 160, 8, 24, 1024, True), (80, 129, 23, 24, 1024, False)]:
+        assert second_pass_plan(L, S, d, r, B, B, SMS, 232448)[2] == want, (r, S, B, L, d)
+    # the plan is made for the largest batch, the form chosen for the one that runs
+    assert second_pass_plan(12, 160, 768, 96, 16, 16, SMS, 232448)[2] and not second_pass_plan(12, 160, 768, 96, 16, 1, SMS, 232448)[2]
