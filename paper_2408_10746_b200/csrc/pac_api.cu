@@ -1010,7 +1010,7 @@ pac_status head_matrix_enqueue(pac_ctx* c, int B, bool behind) {
     const Dims& dm = c->dm;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[1];
-    pdl_launch_config(&cfg, attr, dim3(cdiv((long long)dm.r * dm.C, 8)), dim3(256), 0, c->stream);
+    pdl_launch_config(&cfg, attr, dim3(cdiv((long long)dm.r * dm.C, HEAD_MATRIX_THREADS / 32)), dim3(HEAD_MATRIX_THREADS), 0, c->stream);
     cudaError_t e = cudaLaunchKernelEx(&cfg, head_matrix_kernel, (const float*)(c->params + c->lay.w_up),
                                        (const float*)(c->params + c->lay.w_head), dm.d, dm.r, dm.C, c->sc.prodW, behind ? 1 : 0, behind ? ArgIds{} : arg_ids(c, B), c->sc.ids);
     c->launches++;

@@ -155,7 +155,9 @@ __device__ __forceinline__ void mid_head_products(const MidParams& p, const MidS
 // behind: the kernel ahead lets this one start only when everything ahead of itself is complete, so the parameters are final; it runs beside that kernel and ends after it, so
 // that whoever waits for this one finds both done (smallest blocking fp32 step 50.7 -> 48.4 us, fp32 step at T5-Base widths 91.6 -> 86.3, T5-Large step 436 -> 430).
 // Otherwise the first block stores the step's ids, where they travel as an argument (the kernel ahead does so then).
-__global__ void __launch_bounds__(256) head_matrix_kernel(const float* __restrict__ W_up, const float* __restrict__ W_head, int d, int r,
+constexpr int HEAD_MATRIX_THREADS = 256;
+static_assert(ARG_IDS <= HEAD_MATRIX_THREADS, "the first block stores the ids, one per thread");
+__global__ void __launch_bounds__(HEAD_MATRIX_THREADS) head_matrix_kernel(const float* __restrict__ W_up, const float* __restrict__ W_head, int d, int r,
                                                           int C, float* __restrict__ prodW, int behind, const __grid_constant__ ArgIds arg, int* __restrict__ ids) {
     // not behind: the parameters come from the optimizer update before this kernel, and the ids of the step before may be read until then; the down-projections are let in after
     // the wait, too: their CTAs beside the kernels before this one, which still run then, cost more than their start hides (d = 768, S = 151, B = 2, L = 8: step 35.2 -> 33.8 us, three

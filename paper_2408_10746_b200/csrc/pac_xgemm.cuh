@@ -46,6 +46,7 @@ struct XgRows {
 
 constexpr int XG_TEAM = 8, XG_TILE = 128, XG_K = 64, XG_MAX_JOBS = 6;
 __host__ __device__ constexpr int xg_threads(int teams) { return 32 * (teams * XG_TEAM + 1); }
+static_assert(ARG_IDS <= xg_threads(1), "the first block stores the ids, one per thread");
 constexpr uint32_t XG_TERM_A = XG_TILE * XG_K * 2, XG_BOX = 64 * 128;
 
 // Products of one launch: several per layer (tn), all layers.
