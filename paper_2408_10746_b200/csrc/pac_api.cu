@@ -341,10 +341,9 @@ void time_mark(pac_ctx* c, int which, bool stop) {
 }
 
 // ---- staging of host ids ----
-// Ids of the one-launch forward are arguments of the kernels themselves (step_arg_ids).  Elsewhere the ids of an ordinary minibatch (or short epoch) travel as the
-// argument of a kernel that stores them: a copy from page-locked memory is another engine's work,
-// with a hand-over before and after it (blocking fp32 step on the smallest configuration 58.6 -> 47.6 us,
-// with the loss written straight to host memory; evaluation of 27 samples 26.8 -> 23.7 us).
+// Up to ARG_IDS ids of a gather or a classifier-head step are arguments of its own kernels (step_arg_ids, arg_ids_ok).  Those of other calls (LM head, larger minibatches, epochs whose steps
+// cannot take them) travel as the argument of a kernel that stores them: a copy from page-locked memory is another engine's work, with a hand-over before and after it (when every call took this
+// kernel: blocking fp32 step on the smallest configuration 58.6 -> 47.6 us, with the loss written straight to host memory).
 // Above PUT_IDS (2 KB of arguments) the copy engine's rate counts.
 constexpr int PUT_IDS = 512;
 struct IdBlock { int v[PUT_IDS]; };
@@ -1004,8 +1003,8 @@ MidParams mid_params(pac_ctx* c, const MidPlan& mp, const int* d_ids, int B, boo
     return p;
 }
 
-// W_up W_head for the stand-alone head kernels, once per forward (launched ahead of the down-projections so that
-// it overlaps the tail of the previous step's optimizer update).
+// W_up W_head for the stand-alone head kernels, once per forward: behind the down-projections' launch and beside their kernel where that kernel lets its successor in after its own
+// wait (fp32-precision products, chain-in-epilogue forward), ahead of them otherwise.
 pac_status head_matrix_enqueue(pac_ctx* c, int B, bool behind) {
     const Dims& dm = c->dm;
     cudaLaunchConfig_t cfg = {};

@@ -781,8 +781,8 @@ dw_down_tc_kernel(const __grid_constant__ CUtensorMap map_cache, BwdParams p, co
 }
 
 // The same for classifier heads and 64 < r <= 128, where da_L is one vector per sample: the product is formed with the gates alone, as ones and zeros, one sample at
-// a time, and a sample's sums are multiplied with its da_L in fp32 and added up in registers.  One term instead of two: half the products
-// (at r = 128 two terms are 206 GFLOP per step of S = 256, B = 64, L = 24, d = 1024 and paced the kernel), and operands without rounding.
+// a time, and a sample's sums are multiplied with its da_L (the sum of the two bf16 terms that the head kernel leaves: rounded to about 2^-17) and added up in fp32 registers.  One term
+// instead of two: half the products (at r = 128 two terms are 206 GFLOP per step of S = 256, B = 64, L = 24, d = 1024 and paced the kernel).
 // Sixteen worker warps build the gate tiles (16 elements per thread and stage) and own 32 rows x 64 columns of the sums each.  Order of a worker: the tiles of
 // sample i, then the sums of sample i - 1, whose products run meanwhile; products of sample i + 1 go where those of i - 1 were, and their tiles
 // are announced only by workers that have read these, so the full barriers say that, too.
