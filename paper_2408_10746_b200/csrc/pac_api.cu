@@ -389,12 +389,16 @@ pac_status stage_ids(pac_ctx* c, const int* ids, int B) {
 // Forward: u_l for every layer, the chain, and the head.  ids are on the device.
 // ---------------------------------------------------------------------------
 // Whether a product over the rows of the cache follows a head kernel (of this step or the one before) that filled the shared memory of many SMs (`apart` of xgemm_launch).
-// L1 and shared memory are split at 196 KB and 228 KB: 24 layers at r = 64, S = 128 take the latter, 22 the former, which costs nothing.  With the heads of 32 SMs (B = 8)
-// the overlap is still the better in an evaluation (53.7 us for 54.8), with those of 52 it is not (83.9 for 79.7); a step, where the head has two products behind it, gains from 32 on
-// (136.8 -> 118.9, d = 512 79.8 -> 75.5).  bf16 rows loaded value by value gain nothing (384 tiles of 9 stages: 75.9 us, apart 77.1).
+// L1 and shared memory are split at 196 KB and 228 KB: 24 layers at r = 64, S = 128 take the latter, 22 the former, which costs nothing.  How many SMs it takes to matter depends on how
+// long the CTAs behind it read.  Evaluations, launched apart / overlapped: 64 heads (B = 16) 39.1 / 40.1 us at d = 256, 83.1 / 95.8 at d = 1024; 52 heads 37.6 / 35.3, d = 512 55.6 / 55.0,
+// d = 1024 79.7 / 83.9; 32 heads 54.8 / 53.7.  Steps, where the head has two products behind it: 16 heads d = 768 69.8 / 73.8, d = 1024 85.9 / 82.6;
+// 24 heads d = 512 63.9 / 64.2, d = 768 77.5 / 82.1, d = 1024 97.6 / 105.5; 32 heads d = 512 75.8 / 79.4, d = 1024 119.0 / 135.9; 52 heads d = 256 73.2 / 72.0.
+// bf16 rows loaded value by value gain nothing (384 tiles of 9 stages: 77.1 / 75.9).
 template <class AL>
 bool behind_large_head(const pac_ctx* c, int B, bool train, const AL& A) {
-    return use_fused_cls(c) && !c->tb.on && c->mplan.smem > 195 * 1024 && (train ? 5LL : 3LL) * B * c->mplan.G > c->sms && (sizeof(typename AL::elem) == 4 || A.vec);
+    if (!use_fused_cls(c) || c->tb.on || c->mplan.smem <= 195 * 1024 || (sizeof(typename AL::elem) == 2 && !A.vec)) return false;
+    const long long heads = (long long)B * c->mplan.G;
+    return 5 * heads > 2LL * c->sms || (c->dm.d > (train ? 256 : 512) && (train ? 7 : 3) * heads > c->sms);
 }
 // out[z] = rows(z) W[z] at fp32 precision.
 template <class AL>

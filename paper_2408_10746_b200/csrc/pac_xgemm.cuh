@@ -405,23 +405,26 @@ inline cudaError_t xgemm_launch(const XgJobs<AL>& J, int K, dim3 grid, int k_sli
 // Whether the accumulators of two CTAs fit beside each other.
 inline bool xg_one_team(int tile_j, int stages) { return (xg_accs(tile_j, stages * (XG_K / 16)) + 1) * tile_j <= 256; }
 // Slices of a reduction over K rows and producer teams per CTA: whole waves of CTAs, each about 2 us plus 0.6 us per stage, or 1 us where it has one team and shares its SM (measured), and
-// the slices' own traffic.  One team only over the rows of the cache (fp32 step at T5-Base widths 86.2 -> 84.4 us, smallest one 48.4 -> 47.6) and where it is the cheaper by this count: with few
-// tiles (d = 256, L = 12, r = 64) two are, 48.1 us for 51.0 at 2048 rows, 45.5 for 49.5 at 1600, 40.2 for 41.8 at 1024.  The weight products of
-// transformer bodies, whose rows lie in L2, were slower with one team, and tiles beyond 64 columns not reliably faster (steps of r = 128 216 -> 200, r = 80 96 -> 105).
+// the slices' own traffic.  One team only over the rows of the cache (fp32 step at T5-Base widths 86.2 -> 84.4 us, smallest one 48.4 -> 47.6).  Where its CTAs fill most of the second slots
+// their starts and ends fall under each other's stages, which the count does not know: it is then taken up to a quarter above two teams (d = 512, L = 12, 2048 rows, 48 tiles 66.3 us, two
+// teams 68.4; d = 576, L = 7, 35 tiles: three steps 106.8, 108.9).  With fewer tiles the count decides (d = 256, L = 12, r = 64, 24 tiles: two teams 48.1 us, one 51.0 at 2048 rows,
+// 45.5 / 49.5 at 1600, 40.2 / 41.8 at 1024); of a single stage only one team has work, and its CTA is the lighter one (smallest blocking fp32 step 42.3, two teams 43.8).  The weight products of transformer bodies, whose rows lie in L2, were slower with one team, and tiles beyond 64 columns not reliably faster
+// (steps of r = 128 216 -> 200, r = 80 96 -> 105).
 struct XgSlices { int n, teams; };
 inline XgSlices xg_slices(long long tiles, int K, int sms, int most, int tile_j) {      // tile_j: of products over the rows of the cache, else 0
     const int stages = (K + XG_K - 1) / XG_K;
-    XgSlices best{1, 2};
-    double best_cost = 1e30;
+    int best[3] = {0, 1, 1};
+    double best_cost[3] = {0, 1e30, 1e30};
     for (int teams = 2; teams >= 1; --teams)
         for (int s = 1; s <= most && s <= stages; ++s) {
             const int each = (stages + s - 1) / s, slots = teams == 1 ? 2 * sms : sms;
             if (teams == 1 && !(tile_j > 0 && tile_j <= 64 && xg_one_team(tile_j, each))) continue;
             const double waves = (double)((tiles * s + slots - 1) / slots);
-            const double cost = waves * (2.0 + (teams == 1 ? 1.0 : 0.6) * each) + 0.3 * (s - 1);
-            if (cost < best_cost) { best_cost = cost; best = XgSlices{s, teams}; }
+            const double cost = waves * (2.0 + (teams == 2 ? 0.6 : each == 1 ? 0.5 : 1.0) * each) + 0.3 * (s - 1);
+            if (cost < best_cost[teams]) { best_cost[teams] = cost; best[teams] = s; }
         }
-    return best;
+    const bool one = best_cost[1] < best_cost[2] * (5 * tiles * best[1] >= 7LL * sms ? 1.25 : 1.0);
+    return one ? XgSlices{best[1], 1} : XgSlices{best[2], 2};
 }
 template <class AL>
 inline cudaError_t xgemm_launch_tn(const XgJobs<AL>& J, int K, int Z, const XgSlices& sl, float* out, long long zstride, long long part_stride, unsigned* status, cudaStream_t stream, bool apart) {
